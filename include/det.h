@@ -313,11 +313,18 @@ int det_adamw_step(const det_adamw_desc* h, int pdtype, void* p, const float* g,
 /* ---- tensor hash (Appendix B: per-step state hash, here on the device) --------------------------------
  * Level 1: SHA-256 of every 4 KiB chunk of the raw bytes (last chunk may be shorter).  While more than 128
  * digests remain, the concatenated digests are hashed again in 4 KiB blocks (128 digests each).  root = SHA-256(remaining digests
- * || u64le(nbytes)), finished on the host; every level below it runs on the device.  p device, 16-byte aligned;
- * ws device, 16-byte aligned, det_tensor_hash_ws_bytes(nbytes) bytes; out32_host receives 32 bytes.
- * Synchronises `stream`. */
+ * || u64le(nbytes)).  p device, 16-byte aligned; ws device, 16-byte aligned, det_tensor_hash_ws_bytes(nbytes) bytes.
+ * det_tensor_hash copies the root to out32_host and synchronises `stream`; det_tensor_hash_async leaves it in out32_dev
+ * (device, 16-byte aligned) in stream order. */
 size_t det_tensor_hash_ws_bytes(size_t nbytes);
+int det_tensor_hash_async(const void* p, size_t nbytes, uint8_t* out32_dev, void* ws, size_t ws_bytes, void* stream);
 int det_tensor_hash(const void* p, size_t nbytes, uint8_t* out32_host, void* ws, size_t ws_bytes, void* stream);
+/* The hashes of many tensors at once: the same roots, 32 bytes each at roots_dev + 32 t (device, 16-byte aligned), in stream
+ * order.  ptrs / nbytes are HOST arrays of ntensors device pointers (16-byte aligned) and byte counts.  A level of a
+ * hash is one sequential chain per 4 KiB, so the levels of all tensors run together. */
+size_t det_tensor_hash_batch_ws_bytes(const size_t* nbytes, int ntensors);
+int det_tensor_hash_batch(const void* const* ptrs, const size_t* nbytes, int ntensors, uint8_t* roots_dev, void* ws,
+                          size_t ws_bytes, void* stream);
 
 #ifdef __cplusplus
 }

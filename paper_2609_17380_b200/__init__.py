@@ -53,7 +53,7 @@ def load():
         for name in ("det_sum_ws_bytes", "det_grad_norm_ws_bytes", "det_lsq_weight_scale_ws_bytes",
                      "det_lsq_act_scale_init_ws_bytes", "det_lsq_quantize_weight_ws_bytes", "det_linear_bwd_ws_bytes",
                      "det_rmsnorm_bwd_ws_bytes", "det_xent_ws_bytes", "det_attn_bwd_ws_bytes", "det_attn_bwd_fixq_ws_bytes",
-                     "det_tensor_hash_ws_bytes", "det_lmhead_fwd_v2_ws_bytes", "det_lmhead_bwd_v2_ws_bytes",
+                     "det_tensor_hash_ws_bytes", "det_tensor_hash_batch_ws_bytes", "det_lmhead_fwd_v2_ws_bytes", "det_lmhead_bwd_v2_ws_bytes",
                      "det_attn_fwd_v2_ws_bytes"):
             getattr(_lib, name).restype = C.c_size_t
         _lib.det_launch_count.restype = C.c_ulonglong
@@ -383,3 +383,18 @@ def det_tensor_hash(p, nbytes, ws):
     out = (C.c_uint8 * 32)()
     _check("det_tensor_hash", load().det_tensor_hash(_ptr(p), C.c_size_t(nbytes), out, *_ws(ws), _stream()))
     return bytes(out).hex()
+
+
+def _byte_counts(tensors):
+    return (C.c_size_t * len(tensors))(*[t.numel() * t.element_size() for t in tensors])
+
+
+def det_tensor_hash_batch_ws_bytes(tensors):
+    return load().det_tensor_hash_batch_ws_bytes(_byte_counts(tensors), C.c_int(len(tensors)))
+
+
+def det_tensor_hash_batch(tensors, roots_dev, ws):
+    """Queues the hashes of all tensors together; root t lands at roots_dev[32 t : 32 t + 32] in stream order."""
+    ptrs = (C.c_void_p * len(tensors))(*[t.data_ptr() for t in tensors])
+    _check("det_tensor_hash_batch", load().det_tensor_hash_batch(ptrs, _byte_counts(tensors), C.c_int(len(tensors)),
+                                                                 _ptr(roots_dev), *_ws(ws), _stream()))

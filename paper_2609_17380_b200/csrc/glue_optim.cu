@@ -1,5 +1,5 @@
 // Elementwise glue (SwiGLU, residual, embedding), the gradient-reduction replay (Algorithm 1 and the
-// TreeFold of Algorithm 2), AdamW, and the chunked SHA-256 tensor hash.  All HBM-bound.
+// TreeFold of Algorithm 2) and AdamW.  All HBM-bound.
 #include "common.cuh"
 #include "internal.h"
 
@@ -258,127 +258,6 @@ __global__ void __launch_bounds__(256) k_adamw(AdamScalars h, void* __restrict__
   }
 }
 
-// ------------------------------------------------------------------------------------------------
-// SHA-256 of 4 KiB chunks (of the data at level 1, of the concatenated digests above it): one thread per chunk,
-// message words fetched with 128-bit loads.  A chunk is one sequential chain of 64 compressions (~0.1 ms), so the
-// small chunk both bounds the latency of the short upper levels and gives a multi-gigabyte tensor hundreds of
-// thousands of independent chains to fill the integer pipes.
-// ------------------------------------------------------------------------------------------------
-__constant__ uint32_t c_K[64] = {
-    0x428a2f98, 0x71374491, 0xb5c0fbcf, 0xe9b5dba5, 0x3956c25b, 0x59f111f1, 0x923f82a4, 0xab1c5ed5, 0xd807aa98,
-    0x12835b01, 0x243185be, 0x550c7dc3, 0x72be5d74, 0x80deb1fe, 0x9bdc06a7, 0xc19bf174, 0xe49b69c1, 0xefbe4786,
-    0x0fc19dc6, 0x240ca1cc, 0x2de92c6f, 0x4a7484aa, 0x5cb0a9dc, 0x76f988da, 0x983e5152, 0xa831c66d, 0xb00327c8,
-    0xbf597fc7, 0xc6e00bf3, 0xd5a79147, 0x06ca6351, 0x14292967, 0x27b70a85, 0x2e1b2138, 0x4d2c6dfc, 0x53380d13,
-    0x650a7354, 0x766a0abb, 0x81c2c92e, 0x92722c85, 0xa2bfe8a1, 0xa81a664b, 0xc24b8b70, 0xc76c51a3, 0xd192e819,
-    0xd6990624, 0xf40e3585, 0x106aa070, 0x19a4c116, 0x1e376c08, 0x2748774c, 0x34b0bcb5, 0x391c0cb3, 0x4ed8aa4a,
-    0x5b9cca4f, 0x682e6ff3, 0x748f82ee, 0x78a5636f, 0x84c87814, 0x8cc70208, 0x90befffa, 0xa4506ceb, 0xbef9a3f7,
-    0xc67178f2};
-__device__ __forceinline__ uint32_t rotr32(uint32_t x, int r) { return __funnelshift_r(x, x, r); }
-__device__ __forceinline__ uint32_t bswap(uint32_t x) { return __byte_perm(x, 0, 0x0123); }
-
-__device__ __forceinline__ void sha_rounds(uint32_t h[8], uint32_t w[16]) {
-  uint32_t a = h[0], b = h[1], c = h[2], d = h[3], e = h[4], f = h[5], g = h[6], hh = h[7];
-#pragma unroll
-  for (int i = 0; i < 64; ++i) {
-    if (i >= 16) {
-      uint32_t w15 = w[(i + 1) & 15], w2 = w[(i + 14) & 15];
-      uint32_t s0 = rotr32(w15, 7) ^ rotr32(w15, 18) ^ (w15 >> 3);
-      uint32_t s1 = rotr32(w2, 17) ^ rotr32(w2, 19) ^ (w2 >> 10);
-      w[i & 15] = w[i & 15] + s0 + w[(i + 9) & 15] + s1;
-    }
-    uint32_t t1 = hh + (rotr32(e, 6) ^ rotr32(e, 11) ^ rotr32(e, 25)) + ((e & f) ^ (~e & g)) + c_K[i] + w[i & 15];
-    uint32_t t2 = (rotr32(a, 2) ^ rotr32(a, 13) ^ rotr32(a, 22)) + ((a & b) ^ (a & c) ^ (b & c));
-    hh = g; g = f; f = e; e = d + t1; d = c; c = b; b = a; a = t1 + t2;
-  }
-  h[0] += a; h[1] += b; h[2] += c; h[3] += d; h[4] += e; h[5] += f; h[6] += g; h[7] += hh;
-}
-
-__global__ void __launch_bounds__(64) k_sha_chunks(const uint8_t* __restrict__ data, size_t nbytes, size_t nchunks,
-                                                   uint8_t* __restrict__ digests) {
-  size_t c = (size_t)blockIdx.x * 64 + threadIdx.x;
-  if (c >= nchunks) return;
-  const size_t CH = 4096;
-  const uint8_t* p = data + c * CH;
-  const size_t len = (c + 1) * CH <= nbytes ? CH : nbytes - c * CH;
-  uint32_t h[8] = {0x6a09e667, 0xbb67ae85, 0x3c6ef372, 0xa54ff53a, 0x510e527f, 0x9b05688c, 0x1f83d9ab, 0x5be0cd19};
-  uint32_t w[16];
-  const size_t full = len / 64;
-  // the next 64-byte block is fetched while the 64 rounds of the current one run
-  uint4 nx[4];
-  if (full) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) nx[k] = __ldg(reinterpret_cast<const uint4*>(p) + k);
-  }
-  for (size_t b = 0; b < full; ++b) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const uint4 u = nx[k];
-      w[4 * k] = bswap(u.x); w[4 * k + 1] = bswap(u.y); w[4 * k + 2] = bswap(u.z); w[4 * k + 3] = bswap(u.w);
-    }
-    if (b + 1 < full) {
-      const uint4* q = reinterpret_cast<const uint4*>(p + (b + 1) * 64);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) nx[k] = __ldg(q + k);
-    }
-    sha_rounds(h, w);
-  }
-  // tail with padding (one or two blocks)
-  const size_t rem = len - full * 64;
-  uint8_t tail[128];
-  for (int i = 0; i < 128; ++i) tail[i] = 0;
-  for (size_t i = 0; i < rem; ++i) tail[i] = p[full * 64 + i];
-  tail[rem] = 0x80;
-  const int tl = (rem + 9 <= 64) ? 64 : 128;
-  const unsigned long long bits = (unsigned long long)len * 8ull;
-  for (int i = 0; i < 8; ++i) tail[tl - 1 - i] = (uint8_t)(bits >> (8 * i));
-  for (int b = 0; b < tl / 64; ++b) {
-    for (int k = 0; k < 16; ++k)
-      w[k] = ((uint32_t)tail[b * 64 + 4 * k] << 24) | ((uint32_t)tail[b * 64 + 4 * k + 1] << 16) |
-             ((uint32_t)tail[b * 64 + 4 * k + 2] << 8) | (uint32_t)tail[b * 64 + 4 * k + 3];
-    sha_rounds(h, w);
-  }
-  uint4* o = reinterpret_cast<uint4*>(digests + c * 32);
-  o[0] = make_uint4(bswap(h[0]), bswap(h[1]), bswap(h[2]), bswap(h[3]));
-  o[1] = make_uint4(bswap(h[4]), bswap(h[5]), bswap(h[6]), bswap(h[7]));
-}
-
-// Root of the tree: SHA-256(the nd <= 128 remaining digests || u64le(nbytes)), one thread (at most 65 compressions).
-__global__ void k_sha_root(const uint8_t* __restrict__ digests, int nd, unsigned long long nbytes, uint8_t* __restrict__ out32) {
-  uint32_t h[8] = {0x6a09e667, 0xbb67ae85, 0x3c6ef372, 0xa54ff53a, 0x510e527f, 0x9b05688c, 0x1f83d9ab, 0x5be0cd19};
-  uint32_t w[16];
-  const uint4* d4 = reinterpret_cast<const uint4*>(digests);
-  for (int b = 0; b < nd / 2; ++b) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const uint4 u = d4[4 * b + k];
-      w[4 * k] = bswap(u.x); w[4 * k + 1] = bswap(u.y); w[4 * k + 2] = bswap(u.z); w[4 * k + 3] = bswap(u.w);
-    }
-    sha_rounds(h, w);
-  }
-  // last block: an odd digest (32 bytes), the length word (8 bytes, little endian), 0x80, zeros, the bit count
-#pragma unroll
-  for (int k = 0; k < 16; ++k) w[k] = 0;
-  int pos = 0;   // words filled
-  if (nd & 1) {
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const uint4 u = d4[2 * (nd - 1) + k];
-      w[4 * k] = bswap(u.x); w[4 * k + 1] = bswap(u.y); w[4 * k + 2] = bswap(u.z); w[4 * k + 3] = bswap(u.w);
-    }
-    pos = 8;
-  }
-  const uint32_t lo = (uint32_t)nbytes, hi = (uint32_t)(nbytes >> 32);
-  const uint32_t wl = bswap(lo), wh = bswap(hi), pad = 0x80000000u;
-  if (pos == 0) { w[0] = wl; w[1] = wh; w[2] = pad; } else { w[8] = wl; w[9] = wh; w[10] = pad; }
-  const unsigned long long bits = ((unsigned long long)nd * 32ull + 8ull) * 8ull;
-  w[14] = (uint32_t)(bits >> 32);
-  w[15] = (uint32_t)bits;
-  sha_rounds(h, w);
-  uint4* o = reinterpret_cast<uint4*>(out32);
-  o[0] = make_uint4(bswap(h[0]), bswap(h[1]), bswap(h[2]), bswap(h[3]));
-  o[1] = make_uint4(bswap(h[4]), bswap(h[5]), bswap(h[6]), bswap(h[7]));
-}
-
 static double ipow(double b, int e) {
   double r = 1.0;
   while (e > 0) { if (e & 1) r *= b; b *= b; e >>= 1; }
@@ -562,47 +441,5 @@ extern "C" int det_adamw_step(const det_adamw_desc* d, int pdtype, void* p, cons
   if (pdtype == DET_BF16) k_adamw<true><<<DET_L(grid), 256, 0, (cudaStream_t)stream>>>(h, p, g, m, v, n);
   else k_adamw<false><<<DET_L(grid), 256, 0, (cudaStream_t)stream>>>(h, p, g, m, v, n);
   DET_CHECK_LAUNCH();
-  return DET_OK;
-}
-
-// Workspace: two areas of level-1 size, ping-ponged by the levels, and 256 bytes for the root of the synchronising call.
-static inline size_t hash_l1_bytes(size_t nbytes) { return align_up(((nbytes + 4095) / 4096) * 32 + 32, 256); }
-extern "C" size_t det_tensor_hash_ws_bytes(size_t nbytes) {
-  return hash_l1_bytes(nbytes) + hash_l1_bytes(hash_l1_bytes(nbytes)) + 256;
-}
-
-extern "C" int det_tensor_hash_async(const void* p, size_t nbytes, uint8_t* out32_dev, void* ws, size_t ws_bytes,
-                                     void* stream) {
-  if ((nbytes && !p) || !out32_dev) return DET_ERR_ARG;
-  if ((nbytes && !aligned16(p)) || !aligned16(out32_dev)) return DET_ERR_ALIGN;
-  if (ws_bytes < det_tensor_hash_ws_bytes(nbytes) || !ws || !aligned16(ws)) return DET_ERR_WORKSPACE;
-  cudaStream_t st = (cudaStream_t)stream;
-  uint8_t* a = (uint8_t*)ws;
-  uint8_t* b = a + hash_l1_bytes(nbytes);
-  size_t nc = (nbytes + 4095) / 4096;
-  if (nc) k_sha_chunks<<<DET_L((unsigned)((nc + 63) / 64)), 64, 0, st>>>((const uint8_t*)p, nbytes, nc, a);
-  DET_CHECK_LAUNCH();
-  while (nc > 128) {
-    const size_t lb = nc * 32, m = (lb + 4095) / 4096;
-    k_sha_chunks<<<DET_L((unsigned)((m + 63) / 64)), 64, 0, st>>>(a, lb, m, b);
-    DET_CHECK_LAUNCH();
-    uint8_t* t = a; a = b; b = t;
-    nc = m;
-  }
-  k_sha_root<<<DET_L(1), 1, 0, st>>>(a, (int)nc, (unsigned long long)nbytes, out32_dev);
-  DET_CHECK_LAUNCH();
-  return DET_OK;
-}
-
-extern "C" int det_tensor_hash(const void* p, size_t nbytes, uint8_t* out32_host, void* ws, size_t ws_bytes,
-                               void* stream) {
-  if (!out32_host) return DET_ERR_ARG;
-  if (ws_bytes < det_tensor_hash_ws_bytes(nbytes) || !ws || !aligned16(ws)) return DET_ERR_WORKSPACE;
-  uint8_t* root = (uint8_t*)ws + det_tensor_hash_ws_bytes(nbytes) - 256;
-  int rc = det_tensor_hash_async(p, nbytes, root, ws, ws_bytes, stream);
-  if (rc != DET_OK) return rc;
-  cudaStream_t st = (cudaStream_t)stream;
-  if (cudaMemcpyAsync(out32_host, root, 32, cudaMemcpyDeviceToHost, st) != cudaSuccess) return DET_ERR_CUDA;
-  if (cudaStreamSynchronize(st) != cudaSuccess) return DET_ERR_CUDA;
   return DET_OK;
 }

@@ -1,0 +1,335 @@
+// Chunked SHA-256 tensor hash (Appendix B: per-step state hash), many tensors per launch.
+//
+// Level 1 hashes every 4 KiB chunk of every tensor, the levels above it the concatenated digests of the level below while
+// more than 128 remain, and the root is SHA-256(remaining digests || u64le(nbytes)).  A chunk is one sequential chain of
+// 64 + 1 compressions, so what a level costs is either the integer pipes (many chunks: k_sha_chunks, a thread per
+// chunk) or the latency of one chain (few chunks: k_sha_few, four lanes per chunk), and never its launch: the levels of
+// all tensors of a call run together.
+#include "common.cuh"
+#include "internal.h"
+
+namespace det {
+
+constexpr int HASH_JOBS = 256;   // tensors per launch
+constexpr size_t HASH_CHUNK = 4096;
+
+// Job j covers the bytes base[j] .. base[j] + nbytes[j]; its chunks have the numbers first[j] .. first[j + 1] - 1 of the
+// launch, and chunk i leaves its digest at out + 32 i.  total: the tensor's byte count, appended to the message of a root.
+struct HashJobs {
+  int n;
+  uint32_t first[HASH_JOBS + 1];
+  const uint8_t* base[HASH_JOBS];
+  unsigned long long nbytes[HASH_JOBS];
+  unsigned long long total[HASH_JOBS];
+};
+
+__device__ __forceinline__ uint32_t rotr32(uint32_t x, int r) { return __funnelshift_r(x, x, r); }
+__device__ __forceinline__ uint32_t bswap(uint32_t x) { return __byte_perm(x, 0, 0x0123); }
+
+#define SHA_K_LIST \
+    0x428a2f98, 0x71374491, 0xb5c0fbcf, 0xe9b5dba5, 0x3956c25b, 0x59f111f1, 0x923f82a4, 0xab1c5ed5, 0xd807aa98, \
+    0x12835b01, 0x243185be, 0x550c7dc3, 0x72be5d74, 0x80deb1fe, 0x9bdc06a7, 0xc19bf174, 0xe49b69c1, 0xefbe4786, \
+    0x0fc19dc6, 0x240ca1cc, 0x2de92c6f, 0x4a7484aa, 0x5cb0a9dc, 0x76f988da, 0x983e5152, 0xa831c66d, 0xb00327c8, \
+    0xbf597fc7, 0xc6e00bf3, 0xd5a79147, 0x06ca6351, 0x14292967, 0x27b70a85, 0x2e1b2138, 0x4d2c6dfc, 0x53380d13, \
+    0x650a7354, 0x766a0abb, 0x81c2c92e, 0x92722c85, 0xa2bfe8a1, 0xa81a664b, 0xc24b8b70, 0xc76c51a3, 0xd192e819, \
+    0xd6990624, 0xf40e3585, 0x106aa070, 0x19a4c116, 0x1e376c08, 0x2748774c, 0x34b0bcb5, 0x391c0cb3, 0x4ed8aa4a, \
+    0x5b9cca4f, 0x682e6ff3, 0x748f82ee, 0x78a5636f, 0x84c87814, 0x8cc70208, 0x90befffa, 0xa4506ceb, 0xbef9a3f7, \
+    0xc67178f2
+
+__device__ __forceinline__ uint32_t big_s1(uint32_t e) { return rotr32(e, 6) ^ rotr32(e, 11) ^ rotr32(e, 25); }
+__device__ __forceinline__ uint32_t big_s0(uint32_t a) { return rotr32(a, 2) ^ rotr32(a, 13) ^ rotr32(a, 22); }
+__device__ __forceinline__ uint32_t sha_ch(uint32_t e, uint32_t f, uint32_t g) { return (e & f) ^ (~e & g); }
+__device__ __forceinline__ uint32_t sha_maj(uint32_t a, uint32_t b, uint32_t c) { return (a & b) ^ (a & c) ^ (b & c); }
+__device__ __forceinline__ uint32_t small_s0(uint32_t w) { return rotr32(w, 7) ^ rotr32(w, 18) ^ (w >> 3); }
+__device__ __forceinline__ uint32_t small_s1(uint32_t w) { return rotr32(w, 17) ^ rotr32(w, 19) ^ (w >> 10); }
+
+// one compression: 64 rounds with the message schedule kept in a rolling window of 16 words
+__device__ __forceinline__ void sha_rounds(uint32_t (&h)[8], uint32_t (&w)[16]) {
+  constexpr uint32_t K[64] = {SHA_K_LIST};
+  uint32_t a = h[0], b = h[1], c = h[2], d = h[3], e = h[4], f = h[5], g = h[6], hh = h[7];
+#pragma unroll
+  for (int i = 0; i < 64; ++i) {
+    if (i >= 16) w[i & 15] += small_s0(w[(i + 1) & 15]) + w[(i + 9) & 15] + small_s1(w[(i + 14) & 15]);
+    const uint32_t t1 = hh + big_s1(e) + sha_ch(e, f, g) + K[i] + w[i & 15];
+    const uint32_t t2 = big_s0(a) + sha_maj(a, b, c);
+    hh = g; g = f; f = e; e = d + t1; d = c; c = b; b = a; a = t1 + t2;
+  }
+  h[0] += a; h[1] += b; h[2] += c; h[3] += d; h[4] += e; h[5] += f; h[6] += g; h[7] += hh;
+}
+
+__device__ __forceinline__ void sha_init(uint32_t (&h)[8]) {
+  h[0] = 0x6a09e667; h[1] = 0xbb67ae85; h[2] = 0x3c6ef372; h[3] = 0xa54ff53a;
+  h[4] = 0x510e527f; h[5] = 0x9b05688c; h[6] = 0x1f83d9ab; h[7] = 0x5be0cd19;
+}
+__device__ __forceinline__ void sha_store(uint8_t* out, const uint32_t (&h)[8]) {
+  uint4* o = reinterpret_cast<uint4*>(out);
+  o[0] = make_uint4(bswap(h[0]), bswap(h[1]), bswap(h[2]), bswap(h[3]));
+  o[1] = make_uint4(bswap(h[4]), bswap(h[5]), bswap(h[6]), bswap(h[7]));
+}
+// A message: `len` bytes at p (4-byte aligned), then for a root the 8 bytes of `total`, then the padding of SHA-256.
+struct ShaMsg {
+  const uint8_t* p;
+  uint32_t len, sfx;
+  unsigned long long total;
+  __device__ __forceinline__ uint32_t blocks() const { return (len + sfx + 9 + 63) / 64; }
+  // byte i of the padded message, i < 64 * blocks()
+  __device__ __forceinline__ uint32_t byte(uint32_t i) const {
+    if (i < len) return p[i];
+    if (i < len + sfx) return (uint32_t)(total >> (8 * (i - len))) & 0xffu;
+    if (i == len + sfx) return 0x80u;
+    const uint32_t end = 64 * blocks();
+    return i + 8 < end ? 0u : (uint32_t)(((unsigned long long)(len + sfx) * 8ull) >> (8 * (end - 1 - i))) & 0xffu;
+  }
+  // block b where it is not wholly message bytes
+  __device__ __noinline__ void ragged_block(uint32_t b, uint32_t* w) const {
+    for (int k = 0; k < 16; ++k) {
+      const uint32_t i = b * 64 + 4 * k;
+      w[k] = i + 4 <= len ? bswap(*reinterpret_cast<const uint32_t*>(p + i))
+                          : (byte(i) << 24) | (byte(i + 1) << 16) | (byte(i + 2) << 8) | byte(i + 3);
+    }
+  }
+};
+template <bool ROOT>
+__device__ __forceinline__ ShaMsg sha_msg(const HashJobs& jobs, uint32_t chunk) {
+  int lo = 0, hi = jobs.n - 1;         // the last job whose first chunk is <= chunk
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (jobs.first[mid] <= chunk) lo = mid; else hi = mid - 1;
+  }
+  const size_t off = (size_t)(chunk - jobs.first[lo]) * HASH_CHUNK;
+  const size_t left = jobs.nbytes[lo] - off;
+  ShaMsg m;
+  m.p = jobs.base[lo] + off;
+  m.len = (uint32_t)(left < HASH_CHUNK ? left : HASH_CHUNK);
+  m.sfx = ROOT ? 8 : 0;
+  m.total = ROOT ? jobs.total[lo] : 0;
+  return m;
+}
+
+// Many chunks: a thread per chunk.  Bound by the integer pipe: 22 logic, shift and add instructions a round at half an
+// instruction per cycle and scheduler make 0.87 TB/s the ceiling at 1.965 GHz, and 1 GiB is hashed at 0.84 TB/s (additions
+// written as integer multiply-adds, meant for another pipe, measured 0.81: they take the same issue slots).
+__global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJobs jobs, uint8_t* __restrict__ out) {
+  const uint32_t c = blockIdx.x * 64 + threadIdx.x;
+  if (c >= jobs.first[jobs.n]) return;
+  const ShaMsg msg = sha_msg<false>(jobs, c);
+  uint32_t h[8], w[16];
+  sha_init(h);
+  const uint32_t full = msg.len / 64, nb = msg.blocks();
+  // the next 64-byte block is fetched while the 64 rounds of the current one run
+  uint4 nx[4];
+  if (full) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) nx[k] = __ldg(reinterpret_cast<const uint4*>(msg.p) + k);
+  }
+  for (uint32_t b = 0; b < nb; ++b) {
+    if (b < full) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint4 u = nx[k];
+        w[4 * k] = bswap(u.x); w[4 * k + 1] = bswap(u.y); w[4 * k + 2] = bswap(u.z); w[4 * k + 3] = bswap(u.w);
+      }
+      if (b + 1 < full) {
+        const uint4* q = reinterpret_cast<const uint4*>(msg.p + (b + 1) * 64);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) nx[k] = __ldg(q + k);
+      }
+    } else {
+      uint32_t t[16];
+      msg.ragged_block(b, t);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) w[k] = t[k];
+    }
+    sha_rounds(h, w);
+  }
+  sha_store(out + (size_t)c * 32, h);
+}
+
+// Few chunks: eight chains per warp, four lanes each.  Only the 64 rounds of a block depend on the block before, so the
+// four lanes of a chain expand the schedules of its next four blocks side by side (schedule word + round constant through
+// shared memory) and the chain itself is rounds alone: 14 instructions a round instead of 22 on the pipe that sets the pace
+// of a single warp, 0.085 ms for 65 blocks instead of 0.137 ms.
+constexpr int SF_CH = 8, SF_PITCH = 68;
+template <bool ROOT>
+__global__ void __launch_bounds__(32) k_sha_few(const __grid_constant__ HashJobs jobs, uint8_t* __restrict__ out) {
+  __shared__ __align__(16) uint32_t ws[4 * SF_CH * SF_PITCH];
+  constexpr uint32_t K[64] = {SHA_K_LIST};
+  const int ch = threadIdx.x >> 2, sub = threadIdx.x & 3;
+  const uint32_t c = blockIdx.x * SF_CH + ch;
+  const bool have = c < jobs.first[jobs.n];
+  ShaMsg msg = {};
+  uint32_t nb = 0;
+  if (have) { msg = sha_msg<ROOT>(jobs, c); nb = msg.blocks(); }
+  const uint32_t full = have ? msg.len / 64 : 0, nbmax = __reduce_max_sync(0xffffffffu, nb);
+  uint32_t h[8];
+  sha_init(h);
+  uint4 nx[4];
+  if ((uint32_t)sub < full) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) nx[k] = __ldg(reinterpret_cast<const uint4*>(msg.p + sub * 64) + k);
+  }
+  for (uint32_t b0 = 0; b0 < nbmax; b0 += 4) {
+    const uint32_t mine = b0 + sub;
+    if (mine < nb) {
+      uint32_t w[16];
+      if (mine < full) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint4 u = nx[k];
+          w[4 * k] = bswap(u.x); w[4 * k + 1] = bswap(u.y); w[4 * k + 2] = bswap(u.z); w[4 * k + 3] = bswap(u.w);
+        }
+      } else {
+        uint32_t t[16];
+        msg.ragged_block(mine, t);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) w[k] = t[k];
+      }
+      if (mine + 4 < full) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) nx[k] = __ldg(reinterpret_cast<const uint4*>(msg.p + (mine + 4) * 64) + k);
+      }
+      uint32_t* row = ws + (sub * SF_CH + ch) * SF_PITCH;
+#pragma unroll
+      for (int i = 0; i < 64; i += 4) {
+        uint32_t t[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int j = i + k;
+          if (j >= 16) w[j & 15] += small_s0(w[(j + 1) & 15]) + w[(j + 9) & 15] + small_s1(w[(j + 14) & 15]);
+          t[k] = w[j & 15] + K[j];
+        }
+        *reinterpret_cast<uint4*>(row + i) = make_uint4(t[0], t[1], t[2], t[3]);
+      }
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int s = 0; s < 4; ++s) {
+      if (b0 + s < nb) {
+        const uint32_t* row = ws + (s * SF_CH + ch) * SF_PITCH;
+        uint32_t a = h[0], b = h[1], cc = h[2], d = h[3], e = h[4], f = h[5], g = h[6], hh = h[7];
+#pragma unroll
+        for (int i = 0; i < 64; i += 4) {
+          const uint4 u = *reinterpret_cast<const uint4*>(row + i);
+          const uint32_t wk[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const uint32_t dx = wk[k] + hh + d;
+            const uint32_t en = big_s1(e) + sha_ch(e, f, g) + dx;
+            const uint32_t q = big_s0(a) + sha_maj(a, b, cc) - d;
+            hh = g; g = f; f = e; e = en; d = cc; cc = b; b = a; a = q + en;
+          }
+        }
+        h[0] += a; h[1] += b; h[2] += cc; h[3] += d; h[4] += e; h[5] += f; h[6] += g; h[7] += hh;
+      }
+    }
+    __syncwarp();
+  }
+  if (have && sub == 0) sha_store(out + (size_t)c * 32, h);
+}
+
+// The rule: as long as four lanes per chain leave at most one warp on a scheduler, the chain's latency is what counts and
+// the few-chunk form is the faster one (1000 chunks: 0.085 against 0.140 ms); with two warps per scheduler both take
+// about the same time (9000 chunks: 0.157 and 0.141 ms), beyond that a thread per chunk wins.
+static int hash_level(const HashJobs& jobs, uint8_t* out, cudaStream_t st) {
+  const uint32_t n = jobs.first[jobs.n];
+  if (!n) return DET_OK;
+  const int sms = dev_sm_count();
+  if (sms <= 0) return DET_ERR_CUDA;
+  if (n <= (uint32_t)sms * 4 * SF_CH) k_sha_few<false><<<DET_L((n + SF_CH - 1) / SF_CH), 32, 0, st>>>(jobs, out);
+  else k_sha_chunks<<<DET_L((n + 63) / 64), 64, 0, st>>>(jobs, out);
+  DET_CHECK_LAUNCH();
+  return DET_OK;
+}
+
+static inline size_t chunks_of(size_t nbytes) { return (nbytes + HASH_CHUNK - 1) / HASH_CHUNK; }
+
+}  // namespace det
+
+using namespace det;
+
+// The digests of every level of every tensor of a group lie one after the other: 32 bytes per chunk.
+extern "C" size_t det_tensor_hash_batch_ws_bytes(const size_t* nbytes, int ntensors) {
+  size_t most = 0;
+  for (int t0 = 0; t0 < ntensors; t0 += HASH_JOBS) {
+    size_t need = 0;
+    for (int t = t0; t < ntensors && t < t0 + HASH_JOBS; ++t) {
+      size_t nc = chunks_of(nbytes[t]);
+      need += nc;
+      while (nc > 128) { nc = chunks_of(nc * 32); need += nc; }
+    }
+    most = need > most ? need : most;
+  }
+  return most * 32 + 256;
+}
+extern "C" int det_tensor_hash_batch(const void* const* ptrs, const size_t* nbytes, int ntensors, uint8_t* roots_dev, void* ws,
+                                     size_t ws_bytes, void* stream) {
+  if (ntensors < 0 || (ntensors && (!ptrs || !nbytes || !roots_dev))) return DET_ERR_ARG;
+  if (ntensors == 0) return DET_OK;
+  for (int t = 0; t < ntensors; ++t) {
+    if (nbytes[t] && !ptrs[t]) return DET_ERR_ARG;
+    if (nbytes[t] && !aligned16(ptrs[t])) return DET_ERR_ALIGN;
+  }
+  if (!aligned16(roots_dev)) return DET_ERR_ALIGN;
+  if (!ws || !aligned16(ws) || ws_bytes < det_tensor_hash_batch_ws_bytes(nbytes, ntensors)) return DET_ERR_WORKSPACE;
+  cudaStream_t st = (cudaStream_t)stream;
+  for (int t0 = 0; t0 < ntensors; t0 += HASH_JOBS) {
+    const int n = ntensors - t0 < HASH_JOBS ? ntensors - t0 : HASH_JOBS;
+    uint8_t* out = (uint8_t*)ws;
+    HashJobs root, lv;                // lv: the tensors that still have a level to go, with their current bytes
+    int who[HASH_JOBS];
+    root.n = n;
+    lv.n = n;
+    for (int t = 0; t < n; ++t) {
+      who[t] = t;
+      lv.base[t] = (const uint8_t*)ptrs[t0 + t];
+      lv.nbytes[t] = nbytes[t0 + t];
+      root.first[t] = (uint32_t)t;
+      root.total[t] = nbytes[t0 + t];
+    }
+    root.first[n] = (uint32_t)n;
+    while (lv.n) {
+      size_t c = 0;
+      for (int j = 0; j < lv.n; ++j) { lv.first[j] = (uint32_t)c; c += chunks_of(lv.nbytes[j]); }
+      if (c > 0xffffffffull) return DET_ERR_SHAPE;
+      lv.first[lv.n] = (uint32_t)c;
+      const int rc = hash_level(lv, out, st);
+      if (rc != DET_OK) return rc;
+      // a tensor with at most 128 digests goes to its root, the others to the next level
+      int m = 0;
+      for (int j = 0; j < lv.n; ++j) {
+        const size_t nc = chunks_of(lv.nbytes[j]);
+        const uint8_t* dig = out + (size_t)lv.first[j] * 32;
+        if (nc <= 128) { root.base[who[j]] = dig; root.nbytes[who[j]] = nc * 32; }
+        else { lv.base[m] = dig; lv.nbytes[m] = nc * 32; who[m] = who[j]; ++m; }
+      }
+      out += c * 32;
+      lv.n = m;
+    }
+    k_sha_few<true><<<DET_L((n + SF_CH - 1) / SF_CH), 32, 0, st>>>(root, roots_dev + (size_t)t0 * 32);
+    DET_CHECK_LAUNCH();
+  }
+  return DET_OK;
+}
+
+// One tensor: the batch of one, and 256 bytes for the root of the synchronising call.
+extern "C" size_t det_tensor_hash_ws_bytes(size_t nbytes) {
+  return align_up(det_tensor_hash_batch_ws_bytes(&nbytes, 1), 256) + 256;
+}
+extern "C" int det_tensor_hash_async(const void* p, size_t nbytes, uint8_t* out32_dev, void* ws, size_t ws_bytes,
+                                     void* stream) {
+  if ((nbytes && !p) || !out32_dev) return DET_ERR_ARG;
+  if (ws_bytes < det_tensor_hash_ws_bytes(nbytes) || !ws || !aligned16(ws)) return DET_ERR_WORKSPACE;
+  return det_tensor_hash_batch(&p, &nbytes, 1, out32_dev, ws, ws_bytes, stream);
+}
+extern "C" int det_tensor_hash(const void* p, size_t nbytes, uint8_t* out32_host, void* ws, size_t ws_bytes,
+                               void* stream) {
+  if (!out32_host) return DET_ERR_ARG;
+  if (ws_bytes < det_tensor_hash_ws_bytes(nbytes) || !ws || !aligned16(ws)) return DET_ERR_WORKSPACE;
+  uint8_t* root = (uint8_t*)ws + det_tensor_hash_ws_bytes(nbytes) - 256;
+  int rc = det_tensor_hash_async(p, nbytes, root, ws, ws_bytes, stream);
+  if (rc != DET_OK) return rc;
+  cudaStream_t st = (cudaStream_t)stream;
+  if (cudaMemcpyAsync(out32_host, root, 32, cudaMemcpyDeviceToHost, st) != cudaSuccess) return DET_ERR_CUDA;
+  if (cudaStreamSynchronize(st) != cudaSuccess) return DET_ERR_CUDA;
+  return DET_OK;
+}

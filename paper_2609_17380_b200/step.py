@@ -151,7 +151,8 @@ class Replay:
         wsb = max(det.det_attn_bwd_fixq_ws_bytes(B, H, S, Hkv) if cfg.dq_fixed else det.det_attn_bwd_ws_bytes(B, H, S, Hkv),
                   det.det_xent_ws_bytes(T, V), det.det_rmsnorm_bwd_ws_bytes(T, D),
                   det.det_lsq_weight_scale_ws_bytes(2 * Fh, D), det.det_lsq_act_scale_init_ws_bytes(T * max(Fh, D)),
-                  det.det_tensor_hash_ws_bytes(g * 4), det.det_sum_ws_bytes(g), 1 << 20,
+                  *[det.det_tensor_hash_batch_ws_bytes([t for _, t in self._hash_jobs(per)]) for per in (True, False)],
+                  det.det_sum_ws_bytes(g), 1 << 20,
                   (max(det.det_lmhead_fwd_v2_ws_bytes(T, V, D), det.det_lmhead_bwd_v2_ws_bytes(T, V, D)) if cfg.arith == 2 else 0),
                   *[det.det_linear_bwd_ws_bytes(T, N, K) for (N, K) in ((QW, D), (D, D), (2 * Fh, D), (D, Fh))])
         self.ws = e(wsb + 4096, torch.uint8)
@@ -409,24 +410,19 @@ class Replay:
             det.det_adamw_step(desc, det.DET_BF16 if kind == "bf16" else det.DET_F32, self.p(name), self.g(self.gout, name),
                                self.g(self.m, name), self.g(self.v, name), _numel(shape))
 
+    def _hash_jobs(self, per_tensor):
+        jobs = [(name, self.p(name)) for name, _, _ in self.specs] if per_tensor else [("params_bf16", self.pbf), ("steps_f32", self.sx)]
+        return jobs + [("grad", self.gout), ("adam_m", self.m), ("adam_v", self.v)]
+
     def hashes(self, per_tensor=True):
-        """State hashes of the step (Appendix B).  Every hash is queued on the stream with its root finished on the
+        """State hashes of the step (Appendix B).  All of them are queued as one batch with the roots finished on the
         device; the roots come back in ONE copy, so the whole set costs one synchronisation."""
-        jobs = []
-        if per_tensor:
-            for name, shape, kind in self.specs:
-                t = self.p(name)
-                jobs.append((name, t, t.numel() * t.element_size()))
-        else:
-            jobs.append(("params_bf16", self.pbf, self.pbf.numel() * 2))
-            jobs.append(("steps_f32", self.sx, self.sx.numel() * 4))
-        jobs += [("grad", self.gout, self.n_grad * 4), ("adam_m", self.m, self.n_grad * 4), ("adam_v", self.v, self.n_grad * 4)]
+        jobs = self._hash_jobs(per_tensor)
         if self.roots.numel() < 32 * len(jobs):
             self.roots = torch.empty(32 * len(jobs), dtype=torch.uint8, device=self.dev)
-        for i, (_, t, nbytes) in enumerate(jobs):
-            det.det_tensor_hash_async(t, nbytes, self.roots[32 * i:32 * i + 32], self.ws)
+        det.det_tensor_hash_batch([t for _, t in jobs], self.roots, self.ws)
         raw = self.roots[:32 * len(jobs)].cpu().numpy().tobytes()
-        return {name: raw[32 * i:32 * i + 32].hex() for i, (name, _, _) in enumerate(jobs)}
+        return {name: raw[32 * i:32 * i + 32].hex() for i, (name, _) in enumerate(jobs)}
 
     def calibrate(self, tokens_mb):
         """Untimed: set every activation step from the first micro-batch (LSQ initialisation rule)."""
