@@ -207,7 +207,7 @@ int det_attn_fwd_int8pv(const det_bf16* q, const det_bf16* k, const det_bf16* v,
 /* dq (H heads), dk, dv (Hkv heads) with leading dimension ld_d; every contraction is one sequential ascending sum
  * from +0; the gradient of a shared key/value head runs over its query heads in ascending order and, within a
  * head, over the queries in ascending order.  ws (16-byte aligned, det_attn_bwd_ws_bytes) holds bf16(P) and
- * bf16(dS), [B*H, S, S] each, Delta [B*H, S], and for Hkv < H the f32 accumulators carried between query heads. */
+ * bf16(dS), [B*H, S, S] each, and Delta [B*H, S]. */
 size_t det_attn_bwd_ws_bytes(int B, int H, int Hkv, int S);
 int det_attn_bwd(const det_bf16* dout, const det_bf16* q, const det_bf16* k, const det_bf16* v, const det_bf16* out,
                  const float* lse, int ld, int ld_out, int B, int H, int Hkv, int S, int window, det_bf16* dq,

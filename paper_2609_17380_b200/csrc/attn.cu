@@ -20,273 +20,49 @@ __device__ __forceinline__ void unpack8a(const uint4& u, float v[8]) {
   v[4] = bflo(u.z); v[5] = bfhi(u.z); v[6] = bflo(u.w); v[7] = bfhi(u.w);
 }
 
-// ---------------------------------------------------------------------------------------------
-// forward: CTA = 128 queries of one (batch, head); 512 threads (four warps per scheduler, so that the softmax and
-// staging phases, which are chains of dependent instructions, overlap across warps), thread = 4 queries x 8 keys /
-// 8 dims.  Shared memory (f32): Q [dim][query], one buffer that holds K [dim][key] during the logits and V [key][dim]
-// during P.V, and P~ [key][query].  Multiply-adds use the fused instruction whenever no factor of the tile is
-// below 2^-63 in magnitude (then the exact bf16 x bf16 product cannot be subnormal and fused = unfused bit for bit).
-// ---------------------------------------------------------------------------------------------
-constexpr int FQ = 128, FK = 128, FT = 512;
-constexpr int LQ = FQ + 4;
-constexpr size_t FWD_SMEM = (size_t)(3 * DH * LQ) * sizeof(float);
-
 // conservative test for 0 < |v| < 2^-63 (also true for subnormal v, which only selects the slower exact path)
 __device__ __forceinline__ bool tiny1(float v) { return (__float_as_uint(v) * 2u - 1u) < 0x3fffffffu; }
-__device__ __forceinline__ bool tiny8a(const float v[8]) {
-  bool t = false;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) t |= tiny1(v[i]);
-  return t;
-}
-
-// acc[i][j] += A[k][ty*4 + i] * B[k][{tx*4.., 64 + tx*4..}] for k ascending
-template <bool FUSED>
-__device__ __forceinline__ void mac_4x8(const float (*As)[LQ], const float (*Bs)[LQ], int n, int ty, int tx,
-                                        float2 (&acc)[4][4]) {
-#pragma unroll 8
-  for (int k = 0; k < n; ++k) {
-    const float4 a0 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-    const float4 b0 = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-    const float4 b1 = *reinterpret_cast<const float4*>(&Bs[k][64 + tx * 4]);
-    const float av[4] = {a0.x, a0.y, a0.z, a0.w};
-    const float2 b[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y), make_float2(b1.z, b1.w)};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 a = make_float2(av[i], av[i]);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (FUSED) {
-          acc[i][j] = __ffma2_rn(a, b[j], acc[i][j]);
-        } else {  // scalar on purpose: a packed multiply + add pair would be contracted by ptxas
-          acc[i][j].x = fadd(acc[i][j].x, fmul(av[i], b[j].x));
-          acc[i][j].y = fadd(acc[i][j].y, fmul(av[i], b[j].y));
-        }
-      }
-    }
-  }
-}
-
-// Hkv key/value heads serve H query heads (head h reads key/value head h / (H/Hkv)); W > 0 restricts row i to the keys
-// j in (i - W, i] (W a multiple of 128): the tile loop then starts at the tile of q0 - W, and a row skips a tile that
-// holds none of its keys (its statistics stay untouched: alpha = 1, all weights 0).
-template <bool WIN>
-__global__ void __launch_bounds__(FT, 1) k_attn_fwd(const uint16_t* __restrict__ q, const uint16_t* __restrict__ k,
-                                                    const uint16_t* __restrict__ v, int ld, int H, int Hkv, int S, int Warg,
-                                                    uint16_t* __restrict__ out, int ld_out, float* __restrict__ lse,
-                                                    const float* __restrict__ s_q, int8_t* __restrict__ qout) {
-  const int W = WIN ? Warg : 0;
-  extern __shared__ __align__(16) float sm[];
-  float(*Qs)[LQ] = reinterpret_cast<float(*)[LQ]>(sm);                 // [dim][query]
-  float(*KV)[LQ] = reinterpret_cast<float(*)[LQ]>(sm + DH * LQ);       // K: [dim][key]; V: [key][dim]
-  float(*Ps)[LQ] = reinterpret_cast<float(*)[LQ]>(sm + 2 * DH * LQ);   // [key][query]
-  // blocks are handed out in linear order: the query block is the slow index and runs from the longest rows to the
-  // shortest, so the blocks that are still running at the end are the short ones
-  const int qb = gridDim.y - 1 - blockIdx.y;
-  const int h = blockIdx.x % H, b = blockIdx.x / H;
-  const int q0 = qb * FQ;
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const size_t row0 = (size_t)b * S;
-  const uint16_t* qp = q + row0 * ld + (size_t)h * DH;
-  const int hk = h / (H / Hkv);
-  const uint16_t* kp = k + row0 * ld + (size_t)hk * DH;
-  const uint16_t* vp = v + row0 * ld + (size_t)hk * DH;
-
-  // one 128 x 128 bf16 tile in flight: 4 sixteen-byte words per thread
-  uint4 rw[4];
-  auto fetch_k = [&](int j0) {
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int idx = tid + FT * it, key = idx & 127, ch = idx >> 7;
-      rw[it] = (j0 + key < S) ? __ldg(reinterpret_cast<const uint4*>(kp + (size_t)(j0 + key) * ld + ch * 8))
-                              : make_uint4(0u, 0u, 0u, 0u);
-    }
-  };
-  const int jt0 = (WIN && q0 > W) ? (q0 - W) / FK : 0;
-  fetch_k(jt0 * FK);
-  bool tq = false;
-#pragma unroll
-  for (int it = 0; it < 4; ++it) {
-    const int idx = tid + FT * it, r = idx & 127, ch = idx >> 7;
-    float t[8];
-    if (q0 + r < S) unpack8a(__ldg(reinterpret_cast<const uint4*>(qp + (size_t)(q0 + r) * ld + ch * 8)), t);
-    else {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) t[e] = 0.0f;
-    }
-    tq |= tiny8a(t);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) Qs[ch * 8 + e][r] = t[e];
-  }
-  const int tiny_q = __syncthreads_or(tq);
-  float m[4], l[4];
-  float2 o[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    m[i] = __int_as_float(0xff800000);
-    l[i] = 0.0f;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) o[i][e] = make_float2(0.0f, 0.0f);
-  }
-  const int ntiles = q0 / FK + 1;
-  for (int jt = jt0; jt < ntiles; ++jt) {
-    const int j0 = jt * FK;
-    // ---- K tile (fetched during the previous tile's P.V), transposed ----
-    bool tk = false;
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int idx = tid + FT * it, key = idx & 127, ch = idx >> 7;
-      float t[8];
-      unpack8a(rw[it], t);
-      tk |= tiny8a(t);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) KV[ch * 8 + e][key] = t[e];
-    }
-    // V words of this tile travel while the logits are computed
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int idx = tid + FT * it, key = idx >> 4, ch = idx & 15;
-      rw[it] = (j0 + key < S) ? __ldg(reinterpret_cast<const uint4*>(vp + (size_t)(j0 + key) * ld + ch * 8))
-                              : make_uint4(0u, 0u, 0u, 0u);
-    }
-    const int tiny_k = __syncthreads_or(tk);
-    float2 s[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) s[i][e] = make_float2(0.0f, 0.0f);
-    if (tiny_q || tiny_k) mac_4x8<false>(Qs, KV, DH, ty, tx, s);
-    else mac_4x8<true>(Qs, KV, DH, ty, tx, s);
-    // ---- online softmax statistics per row; P~ to shared memory ----
-    float alpha[4];
-    bool tp = false;
-    const bool diag = (jt == ntiles - 1);  // only the last tile of a row block reaches past the diagonal
-    const bool edge = WIN && j0 <= q0 + FQ - 1 - W;  // some row's window starts inside or after this tile
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int rl = ty * 4 + i;
-      const int row = q0 + rl;
-      const bool rowvalid = !(edge && j0 + FK - 1 <= row - W);
-      float sv[8] = {s[i][0].x, s[i][0].y, s[i][1].x, s[i][1].y, s[i][2].x, s[i][2].y, s[i][3].x, s[i][3].y};
-      float mt = m[i];
-      bool valid[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int key = j0 + ((e < 4) ? (tx * 4 + e) : (64 + tx * 4 + e - 4));
-        valid[e] = (!diag || key <= row) && (!edge || key > row - W);
-        sv[e] = fmul(sv[e], ATT_SCALE);
-        if (valid[e]) mt = fmaxf(mt, sv[e]);
-      }
-#pragma unroll
-      for (int w = 1; w < 16; w <<= 1) mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, w));
-      const float al = det_exp_le0(fsub(m[i], mt));
-      alpha[i] = rowvalid ? al : 1.0f;
-      float p[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) p[e] = det_exp_le0(fsub(sv[e], mt));   // branch-free, so the eight chains interleave
-#pragma unroll
-      for (int e = 0; e < 8; ++e) p[e] = valid[e] ? p[e] : 0.0f;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int kl = (e < 4) ? (tx * 4 + e) : (64 + tx * 4 + e - 4);
-        const float pt = bf2f(f2bf(p[e]));
-        tp |= tiny1(pt);
-        Ps[kl][rl] = pt;
-      }
-      float h0 = fadd(fadd(p[0], p[1]), fadd(p[2], p[3]));
-      float h1 = fadd(fadd(p[4], p[5]), fadd(p[6], p[7]));
-#pragma unroll
-      for (int w = 1; w < 16; w <<= 1) {
-        h0 = fadd(h0, __shfl_xor_sync(0xffffffffu, h0, w));
-        h1 = fadd(h1, __shfl_xor_sync(0xffffffffu, h1, w));
-      }
-      l[i] = fadd(fmul(l[i], alpha[i]), fadd(h0, h1));
-      m[i] = mt;
-    }
-    __syncthreads();  // every thread is done with K; P~ is complete
-    // ---- V tile, natural layout, into the same buffer ----
-    bool tv = false;
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int idx = tid + FT * it, key = idx >> 4, ch = idx & 15;
-      float t[8];
-      unpack8a(rw[it], t);
-      tv |= tiny8a(t);
-      *reinterpret_cast<float4*>(&KV[key][ch * 8]) = make_float4(t[0], t[1], t[2], t[3]);
-      *reinterpret_cast<float4*>(&KV[key][ch * 8 + 4]) = make_float4(t[4], t[5], t[6], t[7]);
-    }
-    // K words of the next tile travel during P.V
-    if (jt + 1 < ntiles) fetch_k(j0 + FK);
-    const int tiny_pv = __syncthreads_or(tp || tv);
-    // ---- u = P~ . V over the tile's keys in ascending order, then o = o*alpha + u ----
-    float2 u[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) u[i][e] = make_float2(0.0f, 0.0f);
-    const int kmax = min(FK, q0 + FQ - j0);
-    if (tiny_pv) mac_4x8<false>(Ps, KV, kmax, ty, tx, u);
-    else mac_4x8<true>(Ps, KV, kmax, ty, tx, u);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {  // scalar: the product o*alpha is rounded before the add
-        o[i][e].x = fadd(fmul(o[i][e].x, alpha[i]), u[i][e].x);
-        o[i][e].y = fadd(fmul(o[i][e].y, alpha[i]), u[i][e].y);
-      }
-    }
-    __syncthreads();  // V and P~ may be overwritten by the next tile
-  }
-  const float inv_q = qout ? fdiv(1.0f, s_q[0]) : 0.0f;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int row = q0 + ty * 4 + i;
-    if (row >= S) continue;
-    const float il = fdiv(1.0f, l[i]);
-    uint16_t* op = out + (row0 + row) * ld_out + (size_t)h * DH;
-    uint2 w0, w1;
-    w0.x = pack_bf2(fmul(o[i][0].x, il), fmul(o[i][0].y, il)); w0.y = pack_bf2(fmul(o[i][1].x, il), fmul(o[i][1].y, il));
-    w1.x = pack_bf2(fmul(o[i][2].x, il), fmul(o[i][2].y, il)); w1.y = pack_bf2(fmul(o[i][3].x, il), fmul(o[i][3].y, il));
-    *reinterpret_cast<uint2*>(op + tx * 4) = w0;
-    *reinterpret_cast<uint2*>(op + 64 + tx * 4) = w1;
-    if (qout) {   // the output projection's quantiser, applied to the bf16 values just stored
-      const float f[8] = {bflo(w0.x), bfhi(w0.x), bflo(w0.y), bfhi(w0.y), bflo(w1.x), bfhi(w1.x), bflo(w1.y), bfhi(w1.y)};
-      const uint2 c = quant8(f, inv_q);
-      int8_t* qp8 = qout + (row0 + row) * ld_out + (size_t)h * DH;
-      *reinterpret_cast<uint32_t*>(qp8 + tx * 4) = c.x;
-      *reinterpret_cast<uint32_t*>(qp8 + 64 + tx * 4) = c.y;
-    }
-    if (tx == 0) lse[((size_t)b * H + h) * S + row] = fadd(m[i], det_log(l[i]));
-  }
-}
-
 // ---------------------------------------------------------------------------------------------
-// forward, warp-specialised (full causal attention; the windowed layers keep k_attn_fwd<true>).
+// forward, warp-specialised; CTA = FQ queries of one (batch, head).
 //
-// What bounds the kernel above is shared-memory bandwidth: a 16-byte load costs the port one cycle per 128 distinct
-// bytes of every half-warp, its 4 x 8 register tiles need three such loads (10 port cycles per warp) for 16 packed
-// multiply-adds, and its phases (logits, softmax, P.V) are block-wide, so the FP32 pipe idles during every softmax.
-// Here a consumer warp owns 16 whole query rows: a lane holds 16 rows x 4 adjacent columns (keys while the logits are
+// A consumer warp owns 8 whole query rows: a lane holds 8 rows x 4 adjacent columns (keys while the logits are
 // formed, head dimensions during P.V), so the row operand is one address for the whole warp (q^T [dim][query] and
-// P~ [key][query] in shared memory) and the column operand one 16-byte word per lane: five loads (12 port cycles) per 32
+// P~ [key][query] in shared memory) and the column operand one 16-byte word per lane: three loads per 16
 // packed multiply-adds.  A row's 128 logits of a key block sit in one warp, so its maximum and its row sum (the
 // adjacent pairwise tree: four slots in the lane, then lanes 1, 2, 4, 8, 16 apart) are warp shuffles, P~ of the warp's
 // rows is written and read by that warp alone, and the running maximum, sum and rescale factor of row i live in lane i.
 // K and V arrive through an mbarrier-guarded ring of 16-deep slabs filled by four producer warps (K: 16 head dimensions
 // x 128 keys, eight per block; V: 16 keys x 128 dimensions, eight per block), so no block-wide barrier is left in the
-// loop and consumer warps are not coupled to each other.  The softmax evaluates its 64 exponentials per lane as one
-// straight-line block of branch-free chains and reduces the 16 rows with 16 shuffles per reduction.
+// loop and consumer warps are not coupled to each other.  The softmax evaluates its 32 exponentials per lane as one
+// straight-line block of branch-free chains and reduces the 8 rows with 9 shuffles per reduction.
 // On the diagonal block a warp stops P.V after the last key any of its rows may see.
-// Arithmetic and order per output are exactly those of k_attn_fwd (and of the definition): bit-identical results.
+// WIN: row i sees the keys j in (i - W, i] (W a multiple of 128): the tile loop starts at the tile of q0 - W, and a row
+// skips a tile that holds none of its keys (its statistics stay untouched: alpha = 1, all weights 0).
+// Hkv key/value heads serve H query heads (head h reads key/value head h / (H/Hkv)).
 // ---------------------------------------------------------------------------------------------
-constexpr int AF_RW = 8;                      // query rows per consumer warp (8: sixteen consumer warps, 16: eight)
-constexpr int AF_SLOTS = 8, AF_PF = 4, AF_CONS = (FQ / AF_RW) * 32, AF_PROD = 128, AF_THREADS = AF_CONS + AF_PROD;
-constexpr size_t AFW_SMEM = (size_t)(DH * LQ + FK * FQ + AF_SLOTS * OK * (OT + 4)) * sizeof(float);
+constexpr int FK = 128;
+constexpr int AF_RW = 8;                      // query rows per consumer warp
+constexpr int AF_PROD = 128;
+// Rows per CTA, ring slots, slabs in flight in the producers' registers, CTAs per SM, registers per consumer and producer thread after the hand-over.
+// A CTA of 128 rows has the best rate (26.6 us per row block and key block on a full GPU, against 14.1 us for 64 rows and
+// 8.1 us for 32), but its chain of key blocks is the longest: alone on its SM 26.6, 18 and 14 us per key block.
+template <int FQ_, int SLOTS_, int PF_, int CPS_, int RC_, int RP_>
+struct AfTile {
+  static constexpr int FQ = FQ_, LQ = FQ_ + 4, SLOTS = SLOTS_, PF = PF_, CPS = CPS_, RC = RC_, RP = RP_;
+  static constexpr int CONS = (FQ / AF_RW) * 32, THREADS = CONS + AF_PROD;
+  static constexpr size_t SMEM = (size_t)(DH * LQ + FK * FQ + SLOTS * OK * (OT + 4)) * sizeof(float);
+  // setmaxnreg: the counts after the hand-over must fit into what the block was launched with, or the increase never returns
+  static_assert(CONS * RC + AF_PROD * RP <= (65536 / (CPS * THREADS) / 8 * 8) * THREADS, "register hand-over exceeds the block's allocation");
+};
+typedef AfTile<128, 8, 4, 1, 104, 64> AfTall;
+typedef AfTile<64, 5, 2, 2, 96, 48> AfHalf;
+typedef AfTile<32, 4, 3, 3, 104, 56> AfShort;
 
-// one 16-deep slab: (row i, column c) += A[k][row i of the warp] * B[k][4 lane + c], accumulators laid out as RP() says.  A chunk g (rows 4g..4g+3) of step k is at ap + k * a_ld + ((chunk0 + g) ^ (PSWZ ? swizzle of the key : 0)) * 4.
+// one 16-deep slab: (row i, column c) += A[k][row i of the warp] * B[k][4 lane + c], accumulators laid out as RP() says.
+// Chunk g (rows 4g .. 4g+3) of step k is at ap + k * a_ld + ((chunk0 + g) ^ (PSWZ ? swizzle of the key : 0)) * 4.
 template <bool FUSED, bool PSWZ>
-__device__ __forceinline__ void mac_16x4(const float* __restrict__ ap, int a_ld, int chunk0, int key0,
-                                         const float (*Bs)[OT + 4], int lane, float2 (&acc)[AF_RW / 2][4]) {
+__device__ __forceinline__ void mac_8x4(const float* __restrict__ ap, int a_ld, int chunk0, int key0,
+                                        const float (*Bs)[OT + 4], int lane, float2 (&acc)[AF_RW / 2][4]) {
 #pragma unroll
   for (int k = 0; k < OK; ++k) {
     const int sw = PSWZ ? (((key0 + k) >> 2) & 7) : 0;
@@ -317,51 +93,37 @@ __device__ __forceinline__ void mac_16x4(const float* __restrict__ ap, int a_ld,
 // operand's register pairs come straight out of its 16-byte loads and only the four column values are duplicated into
 // pairs); i is a compile-time constant wherever this is used
 #define RP(acc, i, c) (((i) & 1) ? (acc)[(i) >> 1][c].y : (acc)[(i) >> 1][c].x)
-// Reduction of 16 rows across the warp (x[i]: this lane's value for row i) with partners 1, 2, 4, 8, 16 lanes apart in that
-// order, which for sums is the adjacent pairwise tree over the lanes.  Instead of 16 butterflies of five shuffles every
-// stage halves the rows a lane carries (it sends its partner the half the partner keeps): 8 + 4 + 2 + 1 + 1 shuffles, and
-// lane L ends with the result of row ROW_OF_LANE(L); both operand orders of an addition or a maximum give the same bits.
-#define ROW_OF_LANE(L) (AF_RW == 16 ? ((((L) & 1) << 3) | (((L) & 2) << 1) | (((L) & 4) >> 1) | (((L) & 8) >> 3)) \
-                                    : ((((L) & 1) << 2) | ((L) & 2) | (((L) & 4) >> 2)))
+// Reduction of 8 rows across the warp (x[i]: this lane's value for row i) with partners 1, 2, 4, 8, 16 lanes apart in that
+// order, which for sums is the adjacent pairwise tree over the lanes.  Instead of 8 butterflies of five shuffles the first
+// three stages halve the rows a lane carries (it sends its partner the half the partner keeps): 4 + 2 + 1 + 1 + 1 shuffles,
+// and lane L ends with the result of row ROW_OF_LANE(L); both operand orders of an addition or a maximum give the same bits.
+#define ROW_OF_LANE(L) ((((L) & 1) << 2) | ((L) & 2) | (((L) & 4) >> 2))
 #define ROW_LANE(i) ROW_OF_LANE(i)   /* a lane that holds row i (the bit reversal is its own inverse) */
 template <bool SUM>
 __device__ __forceinline__ float rows_reduce(const float (&x)[AF_RW], int lane) {
   auto op = [](float a, float b) { return SUM ? fadd(a, b) : fmaxf(a, b); };
-  const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4, b3 = lane & 8;
-  float d;
-  if (AF_RW == 16) {
-    float a[8], b[4], c[2];
+  const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4;
+  float b[4], c[2];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) a[j] = op(b0 ? x[(8 + j) % AF_RW] : x[j], __shfl_xor_sync(0xffffffffu, b0 ? x[j] : x[(8 + j) % AF_RW], 1));
+  for (int j = 0; j < 4; ++j) b[j] = op(b0 ? x[4 + j] : x[j], __shfl_xor_sync(0xffffffffu, b0 ? x[j] : x[4 + j], 1));
 #pragma unroll
-    for (int j = 0; j < 4; ++j) b[j] = op(b1 ? a[4 + j] : a[j], __shfl_xor_sync(0xffffffffu, b1 ? a[j] : a[4 + j], 2));
-#pragma unroll
-    for (int j = 0; j < 2; ++j) c[j] = op(b2 ? b[2 + j] : b[j], __shfl_xor_sync(0xffffffffu, b2 ? b[j] : b[2 + j], 4));
-    d = op(b3 ? c[1] : c[0], __shfl_xor_sync(0xffffffffu, b3 ? c[0] : c[1], 8));
-  } else {
-    float b[4], c[2];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) b[j] = op(b0 ? x[4 + j] : x[j], __shfl_xor_sync(0xffffffffu, b0 ? x[j] : x[4 + j], 1));
-#pragma unroll
-    for (int j = 0; j < 2; ++j) c[j] = op(b1 ? b[2 + j] : b[j], __shfl_xor_sync(0xffffffffu, b1 ? b[j] : b[2 + j], 2));
-    d = op(b2 ? c[1] : c[0], __shfl_xor_sync(0xffffffffu, b2 ? c[0] : c[1], 4));
-    d = op(d, __shfl_xor_sync(0xffffffffu, d, 8));
-  }
+  for (int j = 0; j < 2; ++j) c[j] = op(b1 ? b[2 + j] : b[j], __shfl_xor_sync(0xffffffffu, b1 ? b[j] : b[2 + j], 2));
+  float d = op(b2 ? c[1] : c[0], __shfl_xor_sync(0xffffffffu, b2 ? c[0] : c[1], 4));
+  d = op(d, __shfl_xor_sync(0xffffffffu, d, 8));
   return op(d, __shfl_xor_sync(0xffffffffu, d, 16));
 }
-// Register hand-over between the roles (setmaxnreg): the counts after it must fit into what the block was launched with
-// (threads x the launch-time register count: 384 x 168 for 16 rows per warp, 640 x 96 for 8), or the increase never returns.
-static_assert(AF_RW == 16 ? (AF_CONS * 216 + AF_PROD * 72 <= AF_THREADS * 168) : (AF_CONS * 104 + AF_PROD * 64 <= AF_THREADS * 96),
-              "register hand-over exceeds the block's allocation");
-__global__ void __launch_bounds__(AF_THREADS, 1)
-    k_attn_fwd_ws(const uint16_t* __restrict__ q, const uint16_t* __restrict__ k, const uint16_t* __restrict__ v, int ld,
-                  int H, int Hkv, int S, uint16_t* __restrict__ out, int ld_out, float* __restrict__ lse,
-                  const float* __restrict__ s_q, int8_t* __restrict__ qout) {
+template <class T, bool WIN>
+__global__ void __launch_bounds__(T::THREADS, T::CPS)
+    k_attn_fwd(const uint16_t* __restrict__ q, const uint16_t* __restrict__ k, const uint16_t* __restrict__ v, int ld,
+               int H, int Hkv, int S, int Warg, uint16_t* __restrict__ out, int ld_out, float* __restrict__ lse,
+               const float* __restrict__ s_q, int8_t* __restrict__ qout) {
+  constexpr int FQ = T::FQ, LQ = T::LQ, AF_SLOTS = T::SLOTS, AF_PF = T::PF, AF_CONS = T::CONS, AF_THREADS = T::THREADS;
+  const int W = WIN ? Warg : 0;
   extern __shared__ __align__(16) float sm[];
   float(*Qs)[LQ] = reinterpret_cast<float(*)[LQ]>(sm);                         // [dim][query]
   float* Ps = sm + DH * LQ;                                                    // [key][query], 16-byte chunks swizzled
   float(*Ring)[OK][OT + 4] = reinterpret_cast<float(*)[OK][OT + 4]>(sm + DH * LQ + FK * FQ);
-  __shared__ int tiny_s[AF_SLOTS][AF_PROD / 32];
+  __shared__ __align__(16) int tiny_s[AF_SLOTS][AF_PROD / 32];
   __shared__ int tiny_q_s, abort_s;
   __shared__ __align__(8) uint64_t bar_full[AF_SLOTS], bar_empty[AF_SLOTS];
   volatile int* abort_flag = &abort_s;
@@ -373,7 +135,9 @@ __global__ void __launch_bounds__(AF_THREADS, 1)
   const uint16_t* qp = q + row0 * ld + (size_t)h * DH;
   const uint16_t* kp = k + row0 * ld + (size_t)hk * DH;
   const uint16_t* vp = v + row0 * ld + (size_t)hk * DH;
-  const int ntiles = q0 / FK + 1, nslab = ntiles * 16;
+  const int jt0 = (WIN && q0 > W) ? (q0 - W) / FK : 0, ntiles = q0 / FK + 1;
+  // the last block ends with the last slab of 16 value rows that the CTA's last query may see
+  const int nslab = (ntiles - jt0) * 16 - 7 + (q0 % FK + FQ - 1) / OK;
   if (tid == 0) {
     for (int s = 0; s < AF_SLOTS; ++s) { mbar_init(&bar_full[s], AF_PROD / 32); mbar_init(&bar_empty[s], AF_CONS / 32); }
     tiny_q_s = 0;
@@ -384,7 +148,7 @@ __global__ void __launch_bounds__(AF_THREADS, 1)
   {  // q^T of the query block, staged once by everybody
     bool tq = false;
     for (int idx = tid; idx < FQ * 16; idx += AF_THREADS) {
-      const int r = idx & 127, ch = idx >> 7;
+      const int r = idx % FQ, ch = idx / FQ;
       float t[8];
       if (q0 + r < S) unpack8a(__ldg(reinterpret_cast<const uint4*>(qp + (size_t)(q0 + r) * ld + ch * 8)), t);
       else {
@@ -399,7 +163,7 @@ __global__ void __launch_bounds__(AF_THREADS, 1)
   __syncthreads();
   if (tid >= AF_CONS) {
     // ------------------------------- producers -------------------------------
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(AF_RW == 16 ? 72 : 64));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(T::RP));
     const int pt = tid - AF_CONS, pw = pt >> 5;
     // Slab s of the block sequence: block s / 16; s % 16 < 8: K, head dimensions 16 (s % 16) .. (thread = key, two
     // 16-byte words); else V, keys 16 (s % 16 - 8) .. (thread = four dimensions of keys kk, kk + 4, kk + 8, kk + 12).
@@ -409,7 +173,7 @@ __global__ void __launch_bounds__(AF_THREADS, 1)
     const int vf = pt & 31, vk = pt >> 5;            // V: dimensions 4 vf .. 4 vf + 3 of keys vk, vk + 4, vk + 8, vk + 12
     auto fetch = [&](int sn, uint4 (&w)[2]) {
       if (sn >= nslab) return;
-      const int j0n = (sn >> 4) * FK, phn = sn & 15;
+      const int j0n = (jt0 + (sn >> 4)) * FK, phn = sn & 15;
       if (phn < 8) {
         const int key = j0n + pt;
         const uint4* src = reinterpret_cast<const uint4*>(kp + (size_t)key * ld + phn * OK);
@@ -430,86 +194,90 @@ __global__ void __launch_bounds__(AF_THREADS, 1)
     };
     // unpack, test for factors below 2^-63 and store: K as [dimension][key] (thread = key), V as [key][dimension]
     auto store = [&](int ph, float (*dst)[OT + 4], const uint4 (&w)[2]) -> bool {
-      bool tiny = false;
+      uint32_t tiny = 0;
+      const uint32_t words[8] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w};
+#pragma unroll
+      for (int i = 0; i < 8; ++i) word_tiny(words[i], tiny);
       if (ph < 8) {
 #pragma unroll
-        for (int x = 0; x < 2; ++x) {
-          float t[8];
-          unpack8a(w[x], t);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) { tiny |= tiny1(t[e]); dst[x * 8 + e][pt] = t[e]; }
-        }
+        for (int i = 0; i < 8; ++i) { dst[2 * i][pt] = word_lo(words[i]); dst[2 * i + 1][pt] = word_hi(words[i]); }
       } else {
-        const uint32_t words[8] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float4 t = make_float4(bflo(words[2 * i]), bfhi(words[2 * i]), bflo(words[2 * i + 1]), bfhi(words[2 * i + 1]));
-          tiny |= tiny1(t.x) | tiny1(t.y) | tiny1(t.z) | tiny1(t.w);
-          *reinterpret_cast<float4*>(&dst[vk + 4 * i][4 * vf]) = t;
-        }
+        for (int i = 0; i < 4; ++i)
+          *reinterpret_cast<float4*>(&dst[vk + 4 * i][4 * vf]) =
+              make_float4(word_lo(words[2 * i]), word_hi(words[2 * i]), word_lo(words[2 * i + 1]), word_hi(words[2 * i + 1]));
       }
-      return tiny;
+      return words_tiny(tiny);
     };
 #pragma unroll
     for (int d = 0; d < AF_PF; ++d) fetch(d, raw[d]);
+    int slot = 0;
+    uint32_t par = 1;
     for (int s0 = 0; s0 < nslab; s0 += AF_PF) {
 #pragma unroll
       for (int d = 0; d < AF_PF; ++d) {
-        const int s = s0 + d, slot = s % AF_SLOTS, ph = s & 15;
-        if (s >= AF_SLOTS && !mbar_wait(&bar_empty[slot], (uint32_t)((s / AF_SLOTS - 1) & 1), abort_flag, nullptr)) return;
-        const bool tiny = store(ph, Ring[slot], raw[d]);
+        const int s = s0 + d;
+        if (s >= nslab || !mbar_wait(&bar_empty[slot], par, abort_flag, nullptr)) return;
+        const bool tiny = store(s & 15, Ring[slot], raw[d]);
         fetch(s + AF_PF, raw[d]);
         const int any = __any_sync(0xffffffffu, tiny);
         if (lane == 0) tiny_s[slot][pw] = any;
         __syncwarp();
         if (lane == 0) mbar_arrive(&bar_full[slot]);
+        if (++slot == AF_SLOTS) { slot = 0; par ^= 1u; }
       }
     }
     return;
   }
   // --------------------------------- consumers ---------------------------------
-  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(AF_RW == 16 ? 216 : 104));
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(T::RC));
   const int tiny_q = tiny_q_s;
   const int wrow = warp * AF_RW;                      // first row of this warp inside the query block
-  float m_mine = __int_as_float(0xff800000), l_mine = 0.0f, alpha_mine = 0.0f;   // row (lane & 15) of the warp
+  float m_mine = __int_as_float(0xff800000), l_mine = 0.0f, alpha_mine = 0.0f;   // row ROW_OF_LANE(lane) of the warp
   float2 o[AF_RW / 2][4];                                   // rows (2a, 2a+1) x column c
 #pragma unroll
   for (int a = 0; a < AF_RW / 2; ++a)
 #pragma unroll
     for (int c = 0; c < 4; ++c) o[a][c] = make_float2(0.0f, 0.0f);
-  int s = 0;
   bool ok = true;
-  // slab s is waited for (and its below-2^-63 flags fetched) one slab ahead of its use
-  int tiny_cur = 0;
-  auto acquire = [&](int sn) -> bool {
-    if (sn >= nslab) return true;
-    const int slot = sn % AF_SLOTS;
-    if (!mbar_wait(&bar_full[slot], (uint32_t)((sn / AF_SLOTS) & 1), abort_flag, nullptr)) return false;
-    tiny_cur = tiny_s[slot][0] | tiny_s[slot][1] | tiny_s[slot][2] | tiny_s[slot][3];
+  // the next slab is waited for (and its below-2^-63 flags fetched) one slab ahead of its use
+  int tiny_cur = 0, slot = 0, nslot = 0, left = nslab;
+  uint32_t npar = 0;
+  auto acquire = [&]() -> bool {
+    if (left == 0) return true;
+    --left;
+    if (!mbar_wait(&bar_full[nslot], npar, abort_flag, nullptr)) return false;
+    const int4 t4 = *reinterpret_cast<const int4*>(tiny_s[nslot]);
+    tiny_cur = t4.x | t4.y | t4.z | t4.w;
+    if (++nslot == AF_SLOTS) { nslot = 0; npar ^= 1u; }
     return true;
   };
-  ok = acquire(0);
-  for (int jt = 0; jt < ntiles && ok; ++jt) {
+  auto release = [&]() {
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&bar_empty[slot]);
+    if (++slot == AF_SLOTS) slot = 0;
+  };
+  ok = acquire();
+  for (int jt = jt0; jt < ntiles && ok; ++jt) {
     const int j0 = jt * FK;
     const bool diag = (jt == ntiles - 1);           // only the last block of a row block reaches past the diagonal
+    const bool edge = WIN && j0 <= q0 + FQ - 1 - W;  // some row's window starts inside or after this block
     // ---- logits: acc[i] = sum over the 128 dimensions ascending of q[row i][d] k[key][d], keys 4 lane .. 4 lane + 3 ----
     float2 acc[AF_RW / 2][4];
 #pragma unroll
     for (int a = 0; a < AF_RW / 2; ++a)
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[a][c] = make_float2(0.0f, 0.0f);
-    for (int sl = 0; sl < 8; ++sl, ++s) {
-      const int slot = s % AF_SLOTS;
+    for (int sl = 0; sl < 8; ++sl) {
       const int tiny = tiny_q | tiny_cur;
-      if (!acquire(s + 1)) { ok = false; break; }     // the next slab's flags travel while this one is multiplied
+      if (!acquire()) { ok = false; break; }          // the next slab's flags travel while this one is multiplied
       const float* ap = &Qs[sl * OK][wrow];
-      if (tiny) mac_16x4<false, false>(ap, LQ, 0, 0, Ring[slot], lane, acc);
-      else mac_16x4<true, false>(ap, LQ, 0, 0, Ring[slot], lane, acc);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bar_empty[slot]);
+      if (tiny) mac_8x4<false, false>(ap, LQ, 0, 0, Ring[slot], lane, acc);
+      else mac_8x4<true, false>(ap, LQ, 0, 0, Ring[slot], lane, acc);
+      release();
     }
     if (!ok) break;
-    // ---- online softmax of the warp's 16 rows ----
+    // ---- online softmax of the warp's 8 rows ----
     float rm[AF_RW];
 #pragma unroll
     for (int i = 0; i < AF_RW; ++i) {
@@ -519,19 +287,21 @@ __global__ void __launch_bounds__(AF_THREADS, 1)
       for (int e = 0; e < 4; ++e) {
         const float sv = fmul(RP(acc, i, e), ATT_SCALE);
         RP(acc, i, e) = sv;
-        if (!diag || j0 + 4 * lane + e <= row) mt = fmaxf(mt, sv);
+        const int key = j0 + 4 * lane + e;
+        if ((!diag || key <= row) && (!edge || key > row - W)) mt = fmaxf(mt, sv);
       }
       rm[i] = mt;
     }
-    // the lane that owns row r (see rows16_reduce) updates its running maximum (every row sees at least key 0 of the
-    // first block, so the maximum of a block it visits is a number) and the rescale factor of what it has accumulated
+    // the lane that owns row r (see rows_reduce) updates its running maximum (a row sees at least one key of a block it
+    // visits, so the maximum is a number) and the rescale factor of what it has accumulated
     const float m_new = fmaxf(m_mine, rows_reduce<false>(rm, lane));
     alpha_mine = det_exp_le0(fsub(m_mine, m_new));
+    if (edge && j0 + FK - 1 <= q0 + wrow + ROW_OF_LANE(lane) - W) alpha_mine = 1.0f;
     m_mine = m_new;
 #pragma unroll
     for (int i = 0; i < AF_RW; ++i) rm[i] = __shfl_sync(0xffffffffu, m_new, ROW_LANE(i));
     bool tp = false;
-    // 64 independent exponentials in one straight-line block (no branch, no shuffle in between), so that their
+    // 32 independent exponentials in one straight-line block (no branch, no shuffle in between), so that their
     // dependent chains interleave; invisible pairs are zeroed afterwards (their arguments may be anything)
 #pragma unroll
     for (int i = 0; i < AF_RW; ++i)
@@ -543,6 +313,13 @@ __global__ void __launch_bounds__(AF_THREADS, 1)
 #pragma unroll
         for (int e = 0; e < 4; ++e)
           if (j0 + 4 * lane + e > q0 + wrow + i) RP(acc, i, e) = 0.0f;
+    }
+    if (edge) {
+#pragma unroll
+      for (int i = 0; i < AF_RW; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (j0 + 4 * lane + e <= q0 + wrow + i - W) RP(acc, i, e) = 0.0f;
     }
 #pragma unroll
     for (int i = 0; i < AF_RW; ++i) {
@@ -571,18 +348,17 @@ __global__ void __launch_bounds__(AF_THREADS, 1)
     for (int a = 0; a < AF_RW / 2; ++a)
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[a][c] = make_float2(0.0f, 0.0f);
-    const int last_slab = diag ? (wrow + AF_RW - 1) / OK : 7;          // on the diagonal the warp's rows see no key past 16 (warp + 1)
-    for (int sl = 0; sl < 8; ++sl, ++s) {
-      const int slot = s % AF_SLOTS;
+    // on the diagonal the warp's rows see no key beyond its last row, the CTA's none beyond its own last row
+    const int last_slab = diag ? (q0 - j0 + wrow + AF_RW - 1) / OK : 7, last_block = diag ? (q0 - j0 + FQ - 1) / OK : 7;
+    for (int sl = 0; sl <= last_block; ++sl) {
       const int tiny = tiny_p | tiny_cur;
-      if (!acquire(s + 1)) { ok = false; break; }
+      if (!acquire()) { ok = false; break; }
       if (sl <= last_slab) {
         const float* ap = Ps + (size_t)(sl * OK) * FQ;
-        if (tiny) mac_16x4<false, true>(ap, FQ, wrow >> 2, sl * OK, Ring[slot], lane, acc);
-        else mac_16x4<true, true>(ap, FQ, wrow >> 2, sl * OK, Ring[slot], lane, acc);
+        if (tiny) mac_8x4<false, true>(ap, FQ, wrow >> 2, sl * OK, Ring[slot], lane, acc);
+        else mac_8x4<true, true>(ap, FQ, wrow >> 2, sl * OK, Ring[slot], lane, acc);
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bar_empty[slot]);
+      release();
     }
     if (!ok) break;
 #pragma unroll
@@ -644,25 +420,38 @@ __global__ void __launch_bounds__(256) k_attn_delta(const uint16_t* __restrict__
 // P = exp(S*scale - L) and dS = (P (dP - Delta)) scale and store bf16(P) and bf16(dS).  The producers already fetch
 // the next key block while the consumers are in that epilogue, and consumer warps are not coupled to each other.
 // ---------------------------------------------------------------------------------------------
-constexpr size_t SDP_SMEM = (size_t)(2 * DH * (OT + 4) + 2 * WS_STAGES * OK * (OT + 4)) * sizeof(float);
+// Rows per CTA (TM), ring slots, CTAs per SM, registers per consumer and producer thread.  128 rows: 26.8 us per row
+// block and key block on a full GPU, 24 alone; 64 rows: 15.8 and 19 us, for grids bound by the longest chain (8 heads x
+// 1024: 0.214 ms with 128 rows, 0.169 with 64).
+template <int TM_, int SLOTS_, int CPS_, int RC_, int RP_>
+struct SdpTile {
+  static constexpr int TM = TM_, SLOTS = SLOTS_, CPS = CPS_, RC = RC_, RP = RP_;
+  static constexpr int CONS = TM * 2, THREADS = CONS + OG_PROD;
+  static constexpr size_t SMEM = (size_t)(2 * DH * (TM + 4) + 2 * SLOTS * OK * (OT + 4)) * sizeof(float);
+  static_assert(CONS * RC + OG_PROD * RP <= (65536 / (CPS * THREADS) / 8 * 8) * THREADS, "register hand-over exceeds the block's allocation");
+};
+typedef SdpTile<128, 3, 1, 216, 72> SdpTall;
+typedef SdpTile<64, 2, 2, 200, 56> SdpHalf;
 
-__global__ void __launch_bounds__(WS_THREADS, 1)
-    k_attn_sdp_ws(const uint16_t* __restrict__ dout, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k,
-                  const uint16_t* __restrict__ v, const float* __restrict__ lse, const float* __restrict__ delta, int ld,
-                  int ld_out, int H, int Hkv, int S, int W, uint16_t* __restrict__ Pb, uint16_t* __restrict__ dSt) {
+template <class T>
+__global__ void __launch_bounds__(T::THREADS, T::CPS)
+    k_attn_sdp(const uint16_t* __restrict__ dout, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k,
+               const uint16_t* __restrict__ v, const float* __restrict__ lse, const float* __restrict__ delta, int ld,
+               int ld_out, int H, int Hkv, int S, int W, uint16_t* __restrict__ Pb, uint16_t* __restrict__ dSt) {
+  constexpr int TM = T::TM, SDP_SLOTS = T::SLOTS, SDP_CONS = T::CONS, SDP_THREADS = T::THREADS;
   extern __shared__ __align__(16) unsigned char osm[];
-  typedef float(*Full)[OT + 4];
+  typedef float(*Full)[TM + 4];
   Full Qs = reinterpret_cast<Full>(osm);                                            // [dim][query]
-  Full Os = reinterpret_cast<Full>(osm + (size_t)DH * (OT + 4) * sizeof(float));    // [dim][query] of dO
-  float(*Ks)[OK][OT + 4] = reinterpret_cast<float(*)[OK][OT + 4]>(osm + (size_t)2 * DH * (OT + 4) * sizeof(float));
-  float(*Vs)[OK][OT + 4] = Ks + WS_STAGES;
-  __shared__ int tiny_s[WS_STAGES][WS_PROD / 32];
+  Full Os = reinterpret_cast<Full>(osm + (size_t)DH * (TM + 4) * sizeof(float));    // [dim][query] of dO
+  float(*Ks)[OK][OT + 4] = reinterpret_cast<float(*)[OK][OT + 4]>(osm + (size_t)2 * DH * (TM + 4) * sizeof(float));
+  float(*Vs)[OK][OT + 4] = Ks + SDP_SLOTS;
+  __shared__ __align__(16) int tiny_s[SDP_SLOTS][OG_PROD / 32];
   __shared__ int tiny_qo, abort_s;
-  __shared__ __align__(8) uint64_t bar_full[WS_STAGES], bar_empty[WS_STAGES];
+  __shared__ __align__(8) uint64_t bar_full[SDP_SLOTS], bar_empty[SDP_SLOTS];
   volatile int* abort_flag = &abort_s;
   const int it = gridDim.y - 1 - blockIdx.y;        // longest rows first
   const int h = blockIdx.x % H, b = blockIdx.x / H, hk = h / (H / Hkv);
-  const int i0 = it * OT;
+  const int i0 = it * TM, jt_hi = i0 / OT;
   const int tid = threadIdx.x, lane = tid & 31;
   const size_t row0 = (size_t)b * S;
   const uint16_t* qp = q + row0 * ld + (size_t)h * DH;
@@ -670,9 +459,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
   const uint16_t* kp = k + row0 * ld + (size_t)hk * DH;
   const uint16_t* vp = v + row0 * ld + (size_t)hk * DH;
   const int jt_lo = (W > 0 && i0 > W) ? (i0 - W) / OT : 0;
-  const int ntile = it - jt_lo + 1, nslab = ntile * (DH / OK);
+  const int nslab = (jt_hi - jt_lo + 1) * (DH / OK);
   if (tid == 0) {
-    for (int s = 0; s < WS_STAGES; ++s) { mbar_init(&bar_full[s], WS_PROD / 32); mbar_init(&bar_empty[s], WS_CONS / 32); }
+    for (int s = 0; s < SDP_SLOTS; ++s) { mbar_init(&bar_full[s], OG_PROD / 32); mbar_init(&bar_empty[s], SDP_CONS / 32); }
     tiny_qo = 0;
     abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -680,8 +469,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
   __syncthreads();
   {  // q^T and dO^T of the query block, staged once by everybody
     bool tq = false;
-    for (int idx = tid; idx < 2 * OT * 16; idx += WS_THREADS) {
-      const int which = idx >= OT * 16, e = idx - which * OT * 16, r = e & 127, ch = e >> 7;
+    for (int idx = tid; idx < 2 * TM * 16; idx += SDP_THREADS) {
+      const int which = idx >= TM * 16, e = idx - which * TM * 16, r = e % TM, ch = e / TM;
       const uint16_t* src = which ? op + (size_t)(i0 + r) * ld_out : qp + (size_t)(i0 + r) * ld;
       float t[8];
       if (i0 + r < S) unpack8a(__ldg(reinterpret_cast<const uint4*>(src + ch * 8)), t);
@@ -696,64 +485,68 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     if (__any_sync(0xffffffffu, tq) && lane == 0) atomicOr(&tiny_qo, 1);
   }
   __syncthreads();
-  if (tid >= WS_CONS) {
+  if (tid >= SDP_CONS) {
     // ------------------------------- producers -------------------------------
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
-    const int pt = tid - WS_CONS, pw = pt >> 5;
-    WsRaw<CONTIG, false, OT> rk, rv;
-    ws_fetch<CONTIG, false, OT>(kp, S, DH, ld, jt_lo * OT, 0, pt, rk);
-    ws_fetch<CONTIG, false, OT>(vp, S, DH, ld, jt_lo * OT, 0, pt, rv);
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(T::RP));
+    const int pt = tid - SDP_CONS, pw = pt >> 5;
+    OgRaw<CONTIG, false, OT> rk, rv;
+    og_fetch<CONTIG, false, OT>(kp, S, DH, ld, jt_lo * OT, 0, pt, rk);
+    og_fetch<CONTIG, false, OT>(vp, S, DH, ld, jt_lo * OT, 0, pt, rv);
+    int slot = 0;
+    uint32_t par = 1;
     for (int s = 0; s < nslab; ++s) {
-      const int slot = s % WS_STAGES;
-      if (s >= WS_STAGES && !mbar_wait(&bar_empty[slot], (uint32_t)((s / WS_STAGES - 1) & 1), abort_flag, nullptr)) break;
-      bool tiny = ws_store<CONTIG, false, OT>(Ks[slot], pt, rk);
-      tiny |= ws_store<CONTIG, false, OT>(Vs[slot], pt, rv);
+      if (!mbar_wait(&bar_empty[slot], par, abort_flag, nullptr)) break;
+      bool tiny = og_store<CONTIG, false, OT>(Ks[slot], pt, rk);
+      tiny |= og_store<CONTIG, false, OT>(Vs[slot], pt, rv);
       if (s + 1 < nslab) {
         const int j0n = (jt_lo + (s + 1) / (DH / OK)) * OT, c0n = ((s + 1) % (DH / OK)) * OK;
-        ws_fetch<CONTIG, false, OT>(kp, S, DH, ld, j0n, c0n, pt, rk);
-        ws_fetch<CONTIG, false, OT>(vp, S, DH, ld, j0n, c0n, pt, rv);
+        og_fetch<CONTIG, false, OT>(kp, S, DH, ld, j0n, c0n, pt, rk);
+        og_fetch<CONTIG, false, OT>(vp, S, DH, ld, j0n, c0n, pt, rv);
       }
       const int any = __any_sync(0xffffffffu, tiny);
       if (lane == 0) tiny_s[slot][pw] = any;
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar_full[slot]);
+      if (++slot == SDP_SLOTS) { slot = 0; par ^= 1u; }
     }
     return;
   }
   // --------------------------------- consumers ---------------------------------
-  asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
-  const int ty = tid >> 4, tx = tid & 15;
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(T::RC));
+  const int ty = (tid >> 5) * 2 + (tid & 1), tx = (lane >> 1);   // neighbouring lanes share their columns (see og_lane)
   const int tqo = tiny_qo;
   const size_t bh = (size_t)b * H + h;
   float Lr[8], Dr[8];
 #pragma unroll
   for (int a = 0; a < 8; ++a) {
-    const int i = i0 + (a >> 2) * 64 + ty * 4 + (a & 3);
+    const int i = i0 + (a >> 2) * (TM / 2) + ty * 4 + (a & 3);
     Lr[a] = i < S ? lse[bh * S + i] : 0.0f;
     Dr[a] = i < S ? delta[bh * S + i] : 0.0f;
   }
-  int s = 0;
+  int slot = 0;
+  uint32_t par = 0;
   bool ok = true;
-  for (int jt = jt_lo; jt <= it && ok; ++jt) {
+  for (int jt = jt_lo; jt <= jt_hi && ok; ++jt) {
     const int j0 = jt * OT;
     float2 sa[8][4], da[8][4];
 #pragma unroll
     for (int a = 0; a < 8; ++a)
 #pragma unroll
       for (int c = 0; c < 4; ++c) { sa[a][c] = make_float2(0.f, 0.f); da[a][c] = make_float2(0.f, 0.f); }
-    for (int sl = 0; sl < DH / OK; ++sl, ++s) {
-      const int slot = s % WS_STAGES;
-      if (!mbar_wait(&bar_full[slot], (uint32_t)((s / WS_STAGES) & 1), abort_flag, nullptr)) { ok = false; break; }
-      const int tiny = tqo | tiny_s[slot][0] | tiny_s[slot][1] | tiny_s[slot][2] | tiny_s[slot][3];
-      if (tiny) { slab_mac<false, OT>(Qs + sl * OK, Ks[slot], ty, tx, sa); slab_mac<false, OT>(Os + sl * OK, Vs[slot], ty, tx, da); }
-      else { slab_mac<true, OT>(Qs + sl * OK, Ks[slot], ty, tx, sa); slab_mac<true, OT>(Os + sl * OK, Vs[slot], ty, tx, da); }
+    for (int sl = 0; sl < DH / OK; ++sl) {
+      if (!mbar_wait(&bar_full[slot], par, abort_flag, nullptr)) { ok = false; break; }
+      const int4 t4 = *reinterpret_cast<const int4*>(tiny_s[slot]);
+      const int tiny = tqo | t4.x | t4.y | t4.z | t4.w;
+      if (tiny) { slab_mac<false, TM, OT, 8>(Qs + sl * OK, Ks[slot], ty, tx, sa); slab_mac<false, TM, OT, 8>(Os + sl * OK, Vs[slot], ty, tx, da); }
+      else { slab_mac<true, TM, OT, 8>(Qs + sl * OK, Ks[slot], ty, tx, sa); slab_mac<true, TM, OT, 8>(Os + sl * OK, Vs[slot], ty, tx, da); }
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar_empty[slot]);
+      if (++slot == SDP_SLOTS) { slot = 0; par ^= 1u; }
     }
     if (!ok) break;
 #pragma unroll
     for (int a = 0; a < 8; ++a) {
-      const int i = i0 + (a >> 2) * 64 + ty * 4 + (a & 3);
+      const int i = i0 + (a >> 2) * (TM / 2) + ty * 4 + (a & 3);
       if (i >= S) continue;
 #pragma unroll
       for (int g = 0; g < 2; ++g) {
@@ -786,19 +579,67 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
 
 using namespace det;
 
+template <class T, bool WIN>
+static int attn_fwd_go(const det_bf16* q, const det_bf16* k, const det_bf16* v, int ld, int B, int H, int Hkv, int S, int window,
+                       det_bf16* out, int ld_out, float* lse, const float* s_q, int8_t* qout, cudaStream_t st) {
+  static DevOnce once = {};
+  const auto kern = k_attn_fwd<T, WIN>;
+  if (dev_ensure_smem(once, (const void*)kern, T::SMEM) != DET_OK) return DET_ERR_CUDA;
+  const dim3 grid(H * B, (S + T::FQ - 1) / T::FQ);
+  kern<<<DET_L(grid), T::THREADS, T::SMEM, st>>>(q, k, v, ld, H, Hkv, S, window, out, ld_out, lse, s_q, qout);
+  return DET_OK;
+}
+template <class T>
+static int attn_fwd_run(const det_bf16* q, const det_bf16* k, const det_bf16* v, int ld, int B, int H, int Hkv, int S, int window,
+                        det_bf16* out, int ld_out, float* lse, const float* s_q, int8_t* qout, cudaStream_t st) {
+  return window ? attn_fwd_go<T, true>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, st)
+                : attn_fwd_go<T, false>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, st);
+}
+// Rows per CTA: the longest chain of key blocks runs on one SM whatever the others do, and all chains together share the
+// GPU; the figures are the microseconds per key block of a CTA alone on its SM and of one among many, and the row count
+// with the smallest of the larger bounds is taken (16 heads x 832: 0.187 ms with 128 rows, 0.136 with 64, 0.128 with 32;
+// 64 heads x 2048: 1.56, 1.65 and 1.92 ms).
+struct RowCost { int rows; double alone, full; };
+template <int N>
+static int pick_rows(const RowCost (&c)[N], int heads, int S, int window) {
+  const int sms = dev_sm_count() > 0 ? dev_sm_count() : 1;
+  int best = c[0].rows;
+  double best_t = 0.0;
+  for (int i = 0; i < N; ++i) {
+    double longest = 0.0, total = 0.0;
+    for (int q0 = 0; q0 < S; q0 += c[i].rows) {
+      const int lo = window && q0 > window ? (q0 - window) / FK : 0;
+      const double tiles = q0 / FK + 1 - lo;
+      total += tiles;
+      if (tiles > longest) longest = tiles;
+    }
+    const double a = longest * c[i].alone, b = total * heads * c[i].full / sms, t = a > b ? a : b;
+    if (i == 0 || t < 0.97 * best_t) { best = c[i].rows; best_t = t; }
+  }
+  return best;
+}
+static int attn_rows(int heads, int S, int window) {
+  const RowCost c[3] = {{128, 26.6, 26.6}, {64, 18.0, 14.1}, {32, 14.0, 8.1}};
+  return pick_rows(c, heads, S, window);
+}
+static int sdp_rows(int heads, int S, int window) {
+  const RowCost c[2] = {{128, 24.5, 26.8}, {64, 19.0, 15.8}};
+  return pick_rows(c, heads, S, window);
+}
+
 static int attn_fwd_impl(const det_bf16* q, const det_bf16* k, const det_bf16* v, int ld, int B, int H, int Hkv, int S,
                          int window, det_bf16* out, int ld_out, float* lse, const float* s_q, int8_t* qout, void* stream) {
   if (!q || !k || !v || !out || !lse || B <= 0 || H <= 0 || Hkv <= 0 || S <= 0 || window < 0) return DET_ERR_ARG;
   if (qout && (!s_q || (((uintptr_t)qout) & 3u))) return qout && !s_q ? DET_ERR_ARG : DET_ERR_ALIGN;
   if (S % 64 || ld % 8 || ld_out % 8 || ld < H * DH || ld_out < H * DH || H % Hkv || window % 128) return DET_ERR_SHAPE;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out)) return DET_ERR_ALIGN;
-  static DevOnce once_win = {};
-  if (dev_ensure_smem(once_win, (const void*)k_attn_fwd<true>, FWD_SMEM) != DET_OK) return DET_ERR_CUDA;
-  dim3 grid(H * B, (S + FQ - 1) / FQ);
-  static DevOnce once_ws = {};
-  if (dev_ensure_smem(once_ws, (const void*)k_attn_fwd_ws, AFW_SMEM) != DET_OK) return DET_ERR_CUDA;
-  if (window) k_attn_fwd<true><<<DET_L(grid), FT, FWD_SMEM, (cudaStream_t)stream>>>(q, k, v, ld, H, Hkv, S, window, out, ld_out, lse, s_q, qout);
-  else k_attn_fwd_ws<<<DET_L(grid), AF_THREADS, AFW_SMEM, (cudaStream_t)stream>>>(q, k, v, ld, H, Hkv, S, out, ld_out, lse, s_q, qout);
+  int rc;
+  switch (attn_rows(B * H, S, window)) {
+    case 128: rc = attn_fwd_run<AfTall>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, (cudaStream_t)stream); break;
+    case 64: rc = attn_fwd_run<AfHalf>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, (cudaStream_t)stream); break;
+    default: rc = attn_fwd_run<AfShort>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, (cudaStream_t)stream);
+  }
+  if (rc != DET_OK) return rc;
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
@@ -813,15 +654,25 @@ extern "C" int det_attn_fwd_q(const det_bf16* q, const det_bf16* k, const det_bf
   return attn_fwd_impl(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, stream);
 }
 
-// workspace: bf16(P) and bf16(dS), [B*H, S, S] each, Delta f32 [B*H, S], and with grouped queries the f32 accumulators
-// [B*Hkv, S, 128] that carry dK / dV from one query head of a group to the next
+// workspace: bf16(P) and bf16(dS), [B*H, S, S] each, and Delta f32 [B*H, S]
 extern "C" size_t det_attn_bwd_ws_bytes(int B, int H, int Hkv, int S) {
-  return 2 * align_up((size_t)B * H * S * S * 2, 256) +
-         align_up((size_t)B * H * S * 4, 256) + (Hkv < H ? align_up((size_t)B * Hkv * S * DH * 4, 256) : 0);
+  (void)Hkv;
+  return 2 * align_up((size_t)B * H * S * S * 2, 256) + align_up((size_t)B * H * S * 4, 256);
 }
 
 // the fixed-point variant keeps its 64-bit accumulators in registers: no extra scratch
 extern "C" size_t det_attn_bwd_fixq_ws_bytes(int B, int H, int Hkv, int S) { return det_attn_bwd_ws_bytes(B, H, Hkv, S); }
+
+template <class T>
+static int sdp_run(const det_bf16* dout, const det_bf16* q, const det_bf16* k, const det_bf16* v, const float* lse,
+                   const float* delta, int ld, int ld_out, int B, int H, int Hkv, int S, int window, uint16_t* Pb, uint16_t* dSt,
+                   cudaStream_t st) {
+  static DevOnce once = {};
+  if (dev_ensure_smem(once, (const void*)k_attn_sdp<T>, T::SMEM) != DET_OK) return DET_ERR_CUDA;
+  const dim3 grid(H * B, (S + T::TM - 1) / T::TM);
+  k_attn_sdp<T><<<DET_L(grid), T::THREADS, T::SMEM, st>>>(dout, q, k, v, lse, delta, ld, ld_out, H, Hkv, S, window, Pb, dSt);
+  return DET_OK;
+}
 
 static int attn_bwd_impl(const det_bf16* dout, const det_bf16* q, const det_bf16* k, const det_bf16* v,
                          const det_bf16* out, const float* lse, int ld, int ld_out, int B, int H, int Hkv, int S,
@@ -838,60 +689,43 @@ static int attn_bwd_impl(const det_bf16* dout, const det_bf16* q, const det_bf16
   cudaStream_t st = (cudaStream_t)stream;
   const int G = H / Hkv;
   const size_t matP = align_up((size_t)B * H * S * S * 2, 256), matS = matP;
-  const size_t dl = align_up((size_t)B * H * S * 4, 256);
   uint16_t* Pb = (uint16_t*)ws;
   uint16_t* dSt = (uint16_t*)((uint8_t*)ws + matP);
   float* delta = (float*)((uint8_t*)ws + matP + matS);
-  float* carry = (float*)((uint8_t*)ws + matP + matS + dl);
   const size_t nrows = (size_t)B * H * S;
   k_attn_delta<<<DET_L((unsigned)((nrows + 7) / 8)), 256, 0, st>>>(dout, out, ld_out, H, S, nrows, delta);
   DET_CHECK_LAUNCH();
   // P[i,j] = exp(scale * sum_d q[i,d] k[j,d] - L_i) for visible (i,j) (f32; tiles without a visible pair are never
   // touched) and dS[i,j] = bf16((P[i,j] * (sum_d dO[i,d] v[j,d] - Delta_i)) * scale); both sums ascend over the 128 dims
-  static DevOnce once_sdp = {};
-  if (dev_ensure_smem(once_sdp, (const void*)k_attn_sdp_ws, SDP_SMEM) != DET_OK) return DET_ERR_CUDA;
-  dim3 gsdp(H * B, (S + OT - 1) / OT);
-  k_attn_sdp_ws<<<DET_L(gsdp), WS_THREADS, SDP_SMEM, st>>>(dout, q, k, v, lse, delta, ld, ld_out, H, Hkv, S, window, Pb, dSt);
+  int rc = sdp_rows(B * H, S, window) == 128
+               ? sdp_run<SdpTall>(dout, q, k, v, lse, delta, ld, ld_out, B, H, Hkv, S, window, Pb, dSt, st)
+               : sdp_run<SdpHalf>(dout, q, k, v, lse, delta, ld, ld_out, B, H, Hkv, S, window, Pb, dSt, st);
+  if (rc != DET_OK) return rc;
   DET_CHECK_LAUNCH();
-  int rc = DET_OK;
   // dV[j,c] = sum over the query heads g of the group, then over queries i >= j ascending, of P~[i,j] dO[i,c];
-  // dK[j,c] likewise with dS~ and q.  One accumulator per output: with G > 1 it travels through `carry` in f32, and
-  // the two chains then share that scratch and run one after the other.  dV, dK (for G == 1) and dQ are independent of
-  // each other and run side by side on auxiliary streams, so that the short blocks at the end of one grid overlap
-  // with the long blocks at the start of the next.
+  // dK[j,c] likewise with dS~ and q; dQ[i,c] = sum over visible keys j ascending of dS~[i,j] k[j,c].  The three are
+  // independent of each other and run side by side on auxiliary streams, so that the short blocks at the end of one grid
+  // overlap with the long blocks at the start of the next.
   AuxScope aux(st);   // joined again on every way out
   for (int which = 0; which < 2; ++which) {
-    cudaStream_t sk = (G == 1 && which == 1) ? aux.aux(0) : st;
-    for (int g = 0; g < G; ++g) {
-      OgemmArgs p = {};
-      p.I = S; p.J = DH; p.C = S; p.lda = S; p.H = Hkv; p.a_b = (long long)H * S * S; p.a_h = (long long)S * S;
-      p.h_mul = G; p.h_add = g; p.range_mode = 1; p.window = window;
-      p.A = which == 0 ? (const void*)Pb : (const void*)dSt;
-      if (which == 0) { p.B = dout; p.ldb = ld_out; p.b_b = (long long)S * ld_out; }
-      else { p.B = q; p.ldb = ld; p.b_b = (long long)S * ld; }
-      p.b_h = DH;
-      if (g > 0) { p.acc_in = carry; p.acc_ld = DH; p.acc_b = (long long)Hkv * S * DH; p.acc_h = (long long)S * DH; }
-      if (g == G - 1) {
-        p.out = which == 0 ? dv : dk; p.ldo = ld_d; p.o_b = (long long)S * ld_d; p.o_h = DH;
-        rc = ogemm_wb_launch<STRIDED, STRIDED, false, true>(p, B * Hkv, sk);
-      } else {
-        p.out = carry; p.ldo = DH; p.o_b = (long long)Hkv * S * DH; p.o_h = (long long)S * DH;
-        rc = ogemm_wb_launch<STRIDED, STRIDED, false, false>(p, B * Hkv, sk);
-      }
-      if (rc != DET_OK) return rc;
-    }
+    OgemmArgs p = {};
+    p.I = S; p.J = DH; p.C = S; p.lda = S; p.H = Hkv; p.a_b = (long long)H * S * S; p.a_h = (long long)S * S;
+    p.nG = G; p.b_div = 1; p.range_mode = 1; p.window = window;
+    p.A = which == 0 ? Pb : dSt;
+    p.B = which == 0 ? dout : q;
+    p.ldb = which == 0 ? ld_out : ld;
+    p.b_b = (long long)S * p.ldb; p.b_h = DH;
+    p.out = which == 0 ? dv : dk; p.ldo = ld_d; p.o_b = (long long)S * ld_d; p.o_h = DH;
+    rc = ogemm_launch<STRIDED, STRIDED, false, true, 1>(p, B * Hkv, 3, which == 0 ? st : aux.aux(0));
+    if (rc != DET_OK) return rc;
   }
-  // dQ[i,c] = sum over visible keys j ascending of dS~[i,j] k[j,c]
   OgemmArgs p = {};
   p.I = S; p.J = DH; p.C = S; p.lda = S; p.H = H; p.a_b = (long long)H * S * S; p.a_h = (long long)S * S;
-  p.A = dSt; p.B = k; p.ldb = ld; p.b_b = (long long)S * ld; p.b_h = DH; p.b_div = G;
+  p.A = dSt; p.B = k; p.ldb = ld; p.b_b = (long long)S * ld; p.b_h = DH; p.nG = 1; p.b_div = G;
   p.out = dq; p.ldo = ld_d; p.o_b = (long long)S * ld_d; p.o_h = DH; p.range_mode = 2; p.window = window;
-  if (fixq) {
-    // per block of 128 keys the ordered f32 sum, accumulated over the blocks in 64-bit fixed point (Sec. 3.2)
-    rc = ogemm_fix_launch<CONTIG, STRIDED, false>(p, B * H, aux.aux(1));
-  } else {
-    rc = ogemm_wb_launch<CONTIG, STRIDED, false, true>(p, B * H, aux.aux(1));
-  }
+  // fixq: per block of 128 keys the ordered f32 sum, accumulated over the blocks in 64-bit fixed point (Sec. 3.2)
+  if (fixq) rc = ogemm_run<CONTIG, STRIDED, false, true, OgFix, true>(p, B * H, aux.aux(1));
+  else rc = ogemm_launch<CONTIG, STRIDED, false, true, 1>(p, B * H, 3, aux.aux(1));
   if (rc != DET_OK) return rc;
   if (!aux.join()) return DET_ERR_CUDA;
   DET_CHECK_LAUNCH();

@@ -3,9 +3,9 @@
 // Every output is ONE f32 accumulator that starts at +0 (or at the value already in the output) and
 // receives its terms in ascending order of the contraction index, each term an exact bf16 x bf16 product
 // added with a separate rounding.  That fixes the order, so these GEMMs run on the FP32 ALUs:
-// 128x256 output tile per CTA, 8x16 register tile per consumer thread, 16-deep slabs staged through a three-slot
-// shared-memory ring as f32 by dedicated producer warps (k_ogemm_ws in ogemm_core.cuh), packed two-lane FP32
-// instructions.  Because the product of two
+// 128x256 output tile per CTA (smaller ones where those leave SMs idle: og_pick), 8x16 register tile per consumer thread,
+// 16-deep slabs staged through a shared-memory ring as f32 by dedicated producer warps (k_ogemm in ogemm_core.cuh), packed
+// two-lane FP32 instructions.  Because the product of two
 // bf16 values is exact in binary32, "multiply, then add" and a fused multiply-add round the same exact sum
 // once and give the same bits, unless the product is subnormal (the unfused product is then flushed to zero,
 // the fused one is not).  Each slab is therefore checked for factors below 2^-63 while it is staged; clean
@@ -19,7 +19,8 @@ using namespace det;
 // and fills the idle SMs (aux_fork / aux_join keep plain stream order for the caller).
 static OgemmArgs plain_args(const void* A, const void* B, void* out, int I, int J, int C, int lda, int ldb, int ldo, int init) {
   OgemmArgs p = {};
-  p.A = A; p.B = B; p.out = out; p.I = I; p.J = J; p.C = C; p.lda = lda; p.ldb = ldb; p.ldo = ldo; p.init = init; p.H = 1;
+  p.A = A; p.B = B; p.out = out; p.I = I; p.J = J; p.C = C; p.lda = lda; p.ldb = ldb; p.ldo = ldo; p.init = init;
+  p.H = 1; p.nG = 1; p.b_div = 1;
   return p;
 }
 
@@ -27,7 +28,7 @@ extern "C" int det_lmhead_fwd(const det_bf16* H, const det_bf16* W, int M, int V
   if (!H || !W || !logits || M <= 0 || V <= 0 || K <= 0) return DET_ERR_ARG;
   if (K % 16 || V % 4) return DET_ERR_SHAPE;
   if (!aligned16(H) || !aligned16(W) || !aligned16(logits)) return DET_ERR_ALIGN;
-  int rc = ogemm_ws_launch<CONTIG, CONTIG, false, false>(plain_args(H, W, logits, M, V, K, K, K, V, 0), (cudaStream_t)stream);
+  int rc = ogemm_launch<CONTIG, CONTIG, false, false, 0>(plain_args(H, W, logits, M, V, K, K, K, V, 0), 1, 1, (cudaStream_t)stream);
   if (rc != DET_OK) return rc;
   DET_CHECK_LAUNCH();
   return DET_OK;
@@ -41,10 +42,10 @@ extern "C" int det_lmhead_bwd(const float* dlogits, const det_bf16* H, const det
   cudaStream_t st = (cudaStream_t)stream;
   AuxScope aux(st);   // the auxiliary streams start where the caller's stream stands now; joined on every way out
   // dH[m,k] = sum over v ascending of bf16(dlogits[m,v]) * W[v,k]
-  int rc = ogemm_ws_launch<CONTIG, STRIDED, true, true>(plain_args(dlogits, W, dH, M, K, V, V, K, K, 0), st);
+  int rc = ogemm_launch<CONTIG, STRIDED, true, true, 0>(plain_args(dlogits, W, dH, M, K, V, V, K, K, 0), 1, 1, st);
   if (rc != DET_OK) return rc;
   // dW[v,k] (+)= sum over m ascending of bf16(dlogits[m,v]) * H[m,k], beside the first kernel
-  rc = ogemm_ws_launch<STRIDED, STRIDED, true, false>(plain_args(dlogits, H, dW, V, K, M, V, K, K, first_chunk ? 0 : 1),
+  rc = ogemm_launch<STRIDED, STRIDED, true, false, 0>(plain_args(dlogits, H, dW, V, K, M, V, K, K, first_chunk ? 0 : 1), 1, 1,
                                                       aux.aux(0));
   if (rc != DET_OK) return rc;
   if (!aux.join()) return DET_ERR_CUDA;

@@ -44,3 +44,51 @@ def test_hash_batch(det, sizes):
     raw = host(roots).tobytes()
     for i, b in enumerate(blobs):
         assert raw[32 * i:32 * i + 32].hex() == oracle.tensor_hash(b), (i, sizes[i])
+
+
+# LM head at sizes where the tile choice of the ordered contractions changes (32x64, 64x128, 128x128, 128x256) with ragged
+# rows and columns; the last one has a grid of several full rounds in the weight gradient
+@pytest.mark.parametrize("M,V,K", [(8, 16, 16), (40, 80, 48), (136, 2064, 80), (392, 4112, 176), (1032, 8208, 32), (264, 16400, 528)])
+def test_lmhead_tiles(det, M, V, K):
+    H, W = synth.normal_bf16((M, K), 1.0, seed=M, tid=1), synth.normal_bf16((V, K), 0.05, seed=M, tid=2)
+    lg = empty((M, V), F)
+    det.det_lmhead_fwd(dev(H), dev(W), M, V, K, lg)
+    _sync()
+    assert_same_bits(host(lg), oracle.lmhead_fwd(H, W), "logits")
+    g = synth.normal_f32((M, V), 1e-3, seed=M, tid=3)
+    dH, dW = empty((M, K), np.uint16), empty((V, K), F)
+    det.det_lmhead_bwd(dev(g), dev(H), dev(W), M, V, K, dH, dW, 1)
+    _sync()
+    dH_o, dW_o = oracle.lmhead_bwd(g, H, W)
+    assert_same_bits(host(dH, np.uint16), dH_o, "dH")
+    assert_same_bits(host(dW), dW_o, "dW")
+
+
+# attention at head and row counts where the rows per CTA change (32, 64, 128 rows), S off the 128 grid, windows that start
+# and end inside a block, grouped heads (one accumulator over the whole group)
+@pytest.mark.parametrize("B,H,Hkv,S,W", [(1, 2, 2, 576, 0), (1, 40, 40, 320, 0), (2, 80, 80, 192, 0), (1, 3, 3, 704, 256),
+                                         (1, 60, 60, 448, 128), (3, 64, 64, 320, 128), (1, 8, 2, 384, 0), (1, 6, 1, 448, 128)])
+@pytest.mark.parametrize("fixq", [False, True])
+def test_attention_row_blocks(det, B, H, Hkv, S, W, fixq):
+    HD, KD = H * 128, Hkv * 128
+    ld = HD + 2 * KD
+    qkv = synth.normal_bf16((B * S, ld), 1.0, seed=S + H, tid=1)
+    dout = synth.normal_bf16((B * S, HD), 0.1, seed=S + H, tid=2)
+    x = dev(qkv)
+    q = x.data_ptr()
+    k, v = q + 2 * HD, q + 2 * (HD + KD)
+    out, lse = empty((B * S, HD), np.uint16), empty((B, H, S), F)
+    det.det_attn_fwd(q, k, v, ld, B, H, S, out, HD, lse, Hkv=Hkv, window=W)
+    _sync()
+    oout, olse = oracle.attn_fwd(qkv, B, H, S, Hkv=Hkv, window=W)
+    assert_same_bits(host(lse), olse, "lse")
+    assert_same_bits(host(out, np.uint16), oout, "out")
+    dqkv = empty((B * S, ld), np.uint16)
+    d = dqkv.data_ptr()
+    bwd, need = (det.det_attn_bwd_fixq, det.det_attn_bwd_fixq_ws_bytes) if fixq else (det.det_attn_bwd, det.det_attn_bwd_ws_bytes)
+    bwd(dev(dout), q, k, v, out, lse, ld, HD, B, H, S, d, d + 2 * HD, d + 2 * (HD + KD), ld, ws(need(B, H, S, Hkv)), Hkv=Hkv, window=W)
+    _sync()
+    want = oracle.attn_bwd(dout, qkv, oout, olse, B, H, S, Hkv=Hkv, window=W, fixq=fixq)
+    got = host(dqkv, np.uint16)
+    for name, lo, hi in (("dq", 0, HD), ("dk", HD, HD + KD), ("dv", HD + KD, ld)):
+        assert_same_bits(got[:, lo:hi], want[:, lo:hi], name)
