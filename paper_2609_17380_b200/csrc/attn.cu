@@ -25,16 +25,18 @@ __device__ __forceinline__ bool tiny1(float v) { return (__float_as_uint(v) * 2u
 // ---------------------------------------------------------------------------------------------
 // forward, warp-specialised; CTA = FQ queries of one (batch, head).
 //
-// A consumer warp owns 8 whole query rows: a lane holds 8 rows x 4 adjacent columns (keys while the logits are
-// formed, head dimensions during P.V), so the row operand is one address for the whole warp (q^T [dim][query] and
-// P~ [key][query] in shared memory) and the column operand one 16-byte word per lane: three loads per 16
-// packed multiply-adds.  A row's 128 logits of a key block sit in one warp, so its maximum and its row sum (the
-// adjacent pairwise tree: four slots in the lane, then lanes 1, 2, 4, 8, 16 apart) are warp shuffles, P~ of the warp's
-// rows is written and read by that warp alone, and the running maximum, sum and rescale factor of row i live in lane i.
+// A consumer warp owns 8 whole query rows: lane 2t + r holds rows 4r .. 4r+3 and 8 columns (keys 8t .. 8t+7 while the logits
+// are formed, head dimensions {4t.., 64 + 4t..} during P.V).  The row operand (q^T [dim][query], P~ [key][query] in
+// shared memory) is one 16-byte load of two cycles, the column operand two loads of two cycles (neighbouring lanes read the
+// same word), for 16 packed multiply-adds; with 8 rows x 4 columns a lane the column load alone took four cycles and the
+// shared-memory port was busy all the time (4 x 16 heads x 2048: 1.56 -> 1.48 ms).  A row's 128 logits of a key block sit in one warp, so its
+// maximum and its row sum (the adjacent pairwise tree: eight slots in the lane, then lanes 2, 4, 8, 16 apart) are warp
+// shuffles, P~ of the warp's rows is written and read by that warp alone, and the running maximum, sum and rescale factor
+// of a row live in one lane.
 // K and V arrive through an mbarrier-guarded ring of 16-deep slabs filled by four producer warps (K: 16 head dimensions
 // x 128 keys, eight per block; V: 16 keys x 128 dimensions, eight per block), so no block-wide barrier is left in the
-// loop and consumer warps are not coupled to each other.  The softmax evaluates its 32 exponentials per lane as one
-// straight-line block of branch-free chains and reduces the 8 rows with 9 shuffles per reduction.
+// loop and consumer warps are not coupled to each other.  The softmax evaluates its 32 exponentials per lane two at a time
+// as one straight-line block of branch-free chains and reduces the 8 rows with 5 shuffles per reduction.
 // On the diagonal block a warp stops P.V after the last key any of its rows may see.
 // WIN: row i sees the keys j in (i - W, i] (W a multiple of 128): the tile loop starts at the tile of q0 - W, and a row
 // skips a tile that holds none of its keys (its statistics stay untouched: alpha = 1, all weights 0).
@@ -43,71 +45,62 @@ __device__ __forceinline__ bool tiny1(float v) { return (__float_as_uint(v) * 2u
 constexpr int FK = 128;
 constexpr int AF_RW = 8;                      // query rows per consumer warp
 constexpr int AF_PROD = 128;
+// A slab row: the first and the second four columns of a lane lie 80 apart (4t and 80 + 4t), so that a warp's loads of
+// either half are 256 adjacent bytes and the key-wise stores of K stay free of bank conflicts.
+constexpr int AF_HI = 80, AF_BP = 148;
 // Rows per CTA, ring slots, slabs in flight in the producers' registers, CTAs per SM, registers per consumer and producer thread after the hand-over.
-// A CTA of 128 rows has the best rate (26.6 us per row block and key block on a full GPU, against 14.1 us for 64 rows and
-// 8.1 us for 32), but its chain of key blocks is the longest: alone on its SM 26.6, 18 and 14 us per key block.
+// A CTA of 128 rows has the best rate (25.1 us per row block and key block on a full GPU, against 13.2 us for 64 rows and
+// 7.5 us for 32), but its chain of key blocks is the longest: alone on its SM 25.1, 17 and 13 us per key block.
 template <int FQ_, int SLOTS_, int PF_, int CPS_, int RC_, int RP_>
 struct AfTile {
   static constexpr int FQ = FQ_, LQ = FQ_ + 4, SLOTS = SLOTS_, PF = PF_, CPS = CPS_, RC = RC_, RP = RP_;
   static constexpr int CONS = (FQ / AF_RW) * 32, THREADS = CONS + AF_PROD;
-  static constexpr size_t SMEM = (size_t)(DH * LQ + FK * FQ + SLOTS * OK * (OT + 4)) * sizeof(float);
+  static constexpr size_t SMEM = (size_t)(DH * LQ + FK * FQ + SLOTS * OK * AF_BP) * sizeof(float);
   // setmaxnreg: the counts after the hand-over must fit into what the block was launched with, or the increase never returns
   static_assert(CONS * RC + AF_PROD * RP <= (65536 / (CPS * THREADS) / 8 * 8) * THREADS, "register hand-over exceeds the block's allocation");
 };
 typedef AfTile<128, 8, 4, 1, 104, 64> AfTall;
-typedef AfTile<64, 5, 2, 2, 96, 48> AfHalf;
+typedef AfTile<64, 4, 2, 2, 96, 48> AfHalf;
 typedef AfTile<32, 4, 3, 3, 104, 56> AfShort;
 
-// one 16-deep slab: (row i, column c) += A[k][row i of the warp] * B[k][4 lane + c], accumulators laid out as RP() says.
-// Chunk g (rows 4g .. 4g+3) of step k is at ap + k * a_ld + ((chunk0 + g) ^ (PSWZ ? swizzle of the key : 0)) * 4.
+// one 16-deep slab: (row i of the lane, column c) += A[k][row] * B[k][c].  The lane's four rows of step k are chunk
+// `chunk` ^ (PSWZ ? swizzle of the key : 0) of row k of A.
 template <bool FUSED, bool PSWZ>
-__device__ __forceinline__ void mac_8x4(const float* __restrict__ ap, int a_ld, int chunk0, int key0,
-                                        const float (*Bs)[OT + 4], int lane, float2 (&acc)[AF_RW / 2][4]) {
+__device__ __forceinline__ void mac_4x8(const float* __restrict__ ap, int a_ld, int chunk, int key0,
+                                        const float (*Bs)[AF_BP], int tx, float2 (&acc)[4][4]) {
 #pragma unroll
   for (int k = 0; k < OK; ++k) {
-    const int sw = PSWZ ? (((key0 + k) >> 2) & 7) : 0;
-    float4 a[AF_RW / 4];
+    const int sw = PSWZ ? (((key0 + k) >> 3) & 3) << 1 : 0;
+    const float4 a4 = *reinterpret_cast<const float4*>(ap + (size_t)k * a_ld + ((chunk ^ sw) << 2));
+    const float4 b0 = *reinterpret_cast<const float4*>(&Bs[k][4 * tx]), b1 = *reinterpret_cast<const float4*>(&Bs[k][AF_HI + 4 * tx]);
+    const float a[4] = {a4.x, a4.y, a4.z, a4.w};
+    const float2 b[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y), make_float2(b1.z, b1.w)};
 #pragma unroll
-    for (int g = 0; g < AF_RW / 4; ++g) a[g] = *reinterpret_cast<const float4*>(ap + (size_t)k * a_ld + (((chunk0 + g) ^ sw) << 2));
-    const float4 bv = *reinterpret_cast<const float4*>(&Bs[k][4 * lane]);
-    const float bs[4] = {bv.x, bv.y, bv.z, bv.w};
+    for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const float2 bb = make_float2(bs[c], bs[c]);
-#pragma unroll
-      for (int g = 0; g < AF_RW / 4; ++g) {
+      for (int i = 0; i < 4; ++i) {
         if (FUSED) {
-          acc[2 * g][c] = __ffma2_rn(make_float2(a[g].x, a[g].y), bb, acc[2 * g][c]);
-          acc[2 * g + 1][c] = __ffma2_rn(make_float2(a[g].z, a[g].w), bb, acc[2 * g + 1][c]);
+          acc[i][j] = __ffma2_rn(make_float2(a[i], a[i]), b[j], acc[i][j]);
         } else {  // scalar on purpose: a packed multiply + add pair would be contracted by ptxas
-          acc[2 * g][c].x = fadd(acc[2 * g][c].x, fmul(a[g].x, bs[c]));
-          acc[2 * g][c].y = fadd(acc[2 * g][c].y, fmul(a[g].y, bs[c]));
-          acc[2 * g + 1][c].x = fadd(acc[2 * g + 1][c].x, fmul(a[g].z, bs[c]));
-          acc[2 * g + 1][c].y = fadd(acc[2 * g + 1][c].y, fmul(a[g].w, bs[c]));
+          acc[i][j].x = fadd(acc[i][j].x, fmul(a[i], b[j].x));
+          acc[i][j].y = fadd(acc[i][j].y, fmul(a[i], b[j].y));
         }
       }
-    }
   }
 }
-// element (row i, column c) of a row-paired accumulator set (pair [i/2][c] holds rows i, i+1 of column c, so the row
-// operand's register pairs come straight out of its 16-byte loads and only the four column values are duplicated into
-// pairs); i is a compile-time constant wherever this is used
-#define RP(acc, i, c) (((i) & 1) ? (acc)[(i) >> 1][c].y : (acc)[(i) >> 1][c].x)
-// Reduction of 8 rows across the warp (x[i]: this lane's value for row i) with partners 1, 2, 4, 8, 16 lanes apart in that
-// order, which for sums is the adjacent pairwise tree over the lanes.  Instead of 8 butterflies of five shuffles the first
-// three stages halve the rows a lane carries (it sends its partner the half the partner keeps): 4 + 2 + 1 + 1 + 1 shuffles,
-// and lane L ends with the result of row ROW_OF_LANE(L); both operand orders of an addition or a maximum give the same bits.
+// Reduction of a lane's four rows over the sixteen lanes that hold them, with partners 2, 4, 8, 16 lanes apart in that
+// order, which for sums is the adjacent pairwise tree over the lanes.  The first two stages halve the rows a lane carries (it
+// sends its partner the half the partner keeps): 2 + 1 + 1 + 1 shuffles, and lane L ends with the result of row
+// ROW_OF_LANE(L) of the warp; both operand orders of an addition or a maximum give the same bits.
 #define ROW_OF_LANE(L) ((((L) & 1) << 2) | ((L) & 2) | (((L) & 4) >> 2))
-#define ROW_LANE(i) ROW_OF_LANE(i)   /* a lane that holds row i (the bit reversal is its own inverse) */
+#define LANE_OF_ROW(i) ((lane & 1) | ((i) & 2) | (((i) & 1) << 2))   /* a lane that holds row i of this lane's four */
 template <bool SUM>
-__device__ __forceinline__ float rows_reduce(const float (&x)[AF_RW], int lane) {
+__device__ __forceinline__ float rows_reduce(const float (&x)[4], int lane) {
   auto op = [](float a, float b) { return SUM ? fadd(a, b) : fmaxf(a, b); };
-  const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4;
-  float b[4], c[2];
+  const bool b1 = lane & 2, b2 = lane & 4;
+  float c[2];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) b[j] = op(b0 ? x[4 + j] : x[j], __shfl_xor_sync(0xffffffffu, b0 ? x[j] : x[4 + j], 1));
-#pragma unroll
-  for (int j = 0; j < 2; ++j) c[j] = op(b1 ? b[2 + j] : b[j], __shfl_xor_sync(0xffffffffu, b1 ? b[j] : b[2 + j], 2));
+  for (int j = 0; j < 2; ++j) c[j] = op(b1 ? x[2 + j] : x[j], __shfl_xor_sync(0xffffffffu, b1 ? x[j] : x[2 + j], 2));
   float d = op(b2 ? c[1] : c[0], __shfl_xor_sync(0xffffffffu, b2 ? c[0] : c[1], 4));
   d = op(d, __shfl_xor_sync(0xffffffffu, d, 8));
   return op(d, __shfl_xor_sync(0xffffffffu, d, 16));
@@ -122,7 +115,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
   extern __shared__ __align__(16) float sm[];
   float(*Qs)[LQ] = reinterpret_cast<float(*)[LQ]>(sm);                         // [dim][query]
   float* Ps = sm + DH * LQ;                                                    // [key][query], 16-byte chunks swizzled
-  float(*Ring)[OK][OT + 4] = reinterpret_cast<float(*)[OK][OT + 4]>(sm + DH * LQ + FK * FQ);
+  float(*Ring)[OK][AF_BP] = reinterpret_cast<float(*)[OK][AF_BP]>(sm + DH * LQ + FK * FQ);
   __shared__ __align__(16) int tiny_s[AF_SLOTS][AF_PROD / 32];
   __shared__ int tiny_q_s, abort_s;
   __shared__ __align__(8) uint64_t bar_full[AF_SLOTS], bar_empty[AF_SLOTS];
@@ -193,18 +186,19 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
       }
     };
     // unpack, test for factors below 2^-63 and store: K as [dimension][key] (thread = key), V as [key][dimension]
-    auto store = [&](int ph, float (*dst)[OT + 4], const uint4 (&w)[2]) -> bool {
+    const int kcol = (pt & 4 ? AF_HI : 0) + (pt >> 3) * 4 + (pt & 3), vcol = 4 * vf + (vf >= 16 ? AF_HI - 64 : 0);
+    auto store = [&](int ph, float (*dst)[AF_BP], const uint4 (&w)[2]) -> bool {
       uint32_t tiny = 0;
       const uint32_t words[8] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w};
 #pragma unroll
       for (int i = 0; i < 8; ++i) word_tiny(words[i], tiny);
       if (ph < 8) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) { dst[2 * i][pt] = word_lo(words[i]); dst[2 * i + 1][pt] = word_hi(words[i]); }
+        for (int i = 0; i < 8; ++i) { dst[2 * i][kcol] = word_lo(words[i]); dst[2 * i + 1][kcol] = word_hi(words[i]); }
       } else {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          *reinterpret_cast<float4*>(&dst[vk + 4 * i][4 * vf]) =
+          *reinterpret_cast<float4*>(&dst[vk + 4 * i][vcol]) =
               make_float4(word_lo(words[2 * i]), word_hi(words[2 * i]), word_lo(words[2 * i + 1]), word_hi(words[2 * i + 1]));
       }
       return words_tiny(tiny);
@@ -234,11 +228,13 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
   const int tiny_q = tiny_q_s;
   const int wrow = warp * AF_RW;                      // first row of this warp inside the query block
   float m_mine = __int_as_float(0xff800000), l_mine = 0.0f, alpha_mine = 0.0f;   // row ROW_OF_LANE(lane) of the warp
-  float2 o[AF_RW / 2][4];                                   // rows (2a, 2a+1) x column c
+  const int r2 = lane & 1, tx = lane >> 1, lrow = wrow + 4 * r2;   // this lane's rows lrow .. lrow + 3, columns of tx
+  const float2 one = same2(c_one);
+  float2 o[4][4];                                     // row lrow + i, column pair j
 #pragma unroll
-  for (int a = 0; a < AF_RW / 2; ++a)
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) o[a][c] = make_float2(0.0f, 0.0f);
+    for (int j = 0; j < 4; ++j) o[i][j] = make_float2(0.0f, 0.0f);
   bool ok = true;
   // the next slab is waited for (and its below-2^-63 flags fetched) one slab ahead of its use
   int tiny_cur = 0, slot = 0, nslot = 0, left = nslab;
@@ -262,33 +258,32 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     const int j0 = jt * FK;
     const bool diag = (jt == ntiles - 1);           // only the last block of a row block reaches past the diagonal
     const bool edge = WIN && j0 <= q0 + FQ - 1 - W;  // some row's window starts inside or after this block
-    // ---- logits: acc[i] = sum over the 128 dimensions ascending of q[row i][d] k[key][d], keys 4 lane .. 4 lane + 3 ----
-    float2 acc[AF_RW / 2][4];
+    // ---- logits: sum over the 128 dimensions ascending of q[row][d] k[key][d], keys 8 tx .. 8 tx + 7 ----
+    float2 acc[4][4];
 #pragma unroll
-    for (int a = 0; a < AF_RW / 2; ++a)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) acc[a][c] = make_float2(0.0f, 0.0f);
+      for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
     for (int sl = 0; sl < 8; ++sl) {
       const int tiny = tiny_q | tiny_cur;
       if (!acquire()) { ok = false; break; }          // the next slab's flags travel while this one is multiplied
-      const float* ap = &Qs[sl * OK][wrow];
-      if (tiny) mac_8x4<false, false>(ap, LQ, 0, 0, Ring[slot], lane, acc);
-      else mac_8x4<true, false>(ap, LQ, 0, 0, Ring[slot], lane, acc);
+      const float* ap = &Qs[sl * OK][lrow];
+      if (tiny) mac_4x8<false, false>(ap, LQ, 0, 0, Ring[slot], tx, acc);
+      else mac_4x8<true, false>(ap, LQ, 0, 0, Ring[slot], tx, acc);
       release();
     }
     if (!ok) break;
     // ---- online softmax of the warp's 8 rows ----
-    float rm[AF_RW];
+    float rm[4];
+    const int key = j0 + 8 * tx, row = q0 + lrow;
 #pragma unroll
-    for (int i = 0; i < AF_RW; ++i) {
-      const int row = q0 + wrow + i;
+    for (int i = 0; i < 4; ++i) {
       float mt = __int_as_float(0xff800000);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float sv = fmul(RP(acc, i, e), ATT_SCALE);
-        RP(acc, i, e) = sv;
-        const int key = j0 + 4 * lane + e;
-        if ((!diag || key <= row) && (!edge || key > row - W)) mt = fmaxf(mt, sv);
+      for (int j = 0; j < 4; ++j) {
+        acc[i][j] = mul2(acc[i][j], same2(ATT_SCALE));
+        if ((!diag || key + 2 * j <= row + i) && (!edge || key + 2 * j > row + i - W)) mt = fmaxf(mt, acc[i][j].x);
+        if ((!diag || key + 2 * j + 1 <= row + i) && (!edge || key + 2 * j + 1 > row + i - W)) mt = fmaxf(mt, acc[i][j].y);
       }
       rm[i] = mt;
     }
@@ -299,55 +294,63 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     if (edge && j0 + FK - 1 <= q0 + wrow + ROW_OF_LANE(lane) - W) alpha_mine = 1.0f;
     m_mine = m_new;
 #pragma unroll
-    for (int i = 0; i < AF_RW; ++i) rm[i] = __shfl_sync(0xffffffffu, m_new, ROW_LANE(i));
+    for (int i = 0; i < 4; ++i) rm[i] = __shfl_sync(0xffffffffu, m_new, LANE_OF_ROW(i));
     bool tp = false;
     // 32 independent exponentials in one straight-line block (no branch, no shuffle in between), so that their
     // dependent chains interleave; invisible pairs are zeroed afterwards (their arguments may be anything)
 #pragma unroll
-    for (int i = 0; i < AF_RW; ++i)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) RP(acc, i, e) = det_exp_le0(fsub(RP(acc, i, e), rm[i]));
+      for (int j = 0; j < 4; ++j) acc[i][j] = det_exp_le0_2(add2(acc[i][j], same2(-rm[i]), one), one);
     if (diag) {
 #pragma unroll
-      for (int i = 0; i < AF_RW; ++i)
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (j0 + 4 * lane + e > q0 + wrow + i) RP(acc, i, e) = 0.0f;
+        for (int j = 0; j < 4; ++j) {
+          if (key + 2 * j > row + i) acc[i][j].x = 0.0f;
+          if (key + 2 * j + 1 > row + i) acc[i][j].y = 0.0f;
+        }
     }
     if (edge) {
 #pragma unroll
-      for (int i = 0; i < AF_RW; ++i)
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (j0 + 4 * lane + e <= q0 + wrow + i - W) RP(acc, i, e) = 0.0f;
+        for (int j = 0; j < 4; ++j) {
+          if (key + 2 * j <= row + i - W) acc[i][j].x = 0.0f;
+          if (key + 2 * j + 1 <= row + i - W) acc[i][j].y = 0.0f;
+        }
     }
+    uint32_t tw = 0;
 #pragma unroll
-    for (int i = 0; i < AF_RW; ++i) {
-      float p[4] = {RP(acc, i, 0), RP(acc, i, 1), RP(acc, i, 2), RP(acc, i, 3)};
-      rm[i] = fadd(fadd(p[0], p[1]), fadd(p[2], p[3]));      // the lane's four adjacent slots of the block's row sum
+    for (int i = 0; i < 4; ++i) {
+      // the lane's eight adjacent slots of the block's row sum
+      rm[i] = fadd(fadd(fadd(acc[i][0].x, acc[i][0].y), fadd(acc[i][1].x, acc[i][1].y)),
+                   fadd(fadd(acc[i][2].x, acc[i][2].y), fadd(acc[i][3].x, acc[i][3].y)));
 #pragma unroll
-      for (int e = 0; e < 4; ++e) { p[e] = bf2f(f2bf(p[e])); tp |= tiny1(p[e]); RP(acc, i, e) = p[e]; }
-    }
-    // the rest of the adjacent tree over the block's 128 slots: lanes 1, 2, 4, 8, 16 apart
-    l_mine = fadd(fmul(l_mine, alpha_mine), rows_reduce<true>(rm, lane));
-    // P~ of the warp's rows: key row 4 lane + e, chunk of rows 4g .. 4g+3
-    __syncwarp();                                    // the previous block's P.V loads are done
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      float* prow = Ps + (size_t)(4 * lane + e) * FQ;
-#pragma unroll
-      for (int g = 0; g < AF_RW / 4; ++g) {
-        const float4 t = make_float4(RP(acc, 4 * g, e), RP(acc, 4 * g + 1, e), RP(acc, 4 * g + 2, e), RP(acc, 4 * g + 3, e));
-        *reinterpret_cast<float4*>(prow + ((((wrow >> 2) + g) ^ (lane & 7)) << 2)) = t;
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t w = pack_bf2(acc[i][j].x, acc[i][j].y);
+        word_tiny(w, tw);
+        acc[i][j] = make_float2(word_lo(w), word_hi(w));
       }
+    }
+    tp = words_tiny(tw);
+    // the rest of the adjacent tree over the block's 128 slots: lanes 2, 4, 8, 16 apart
+    l_mine = fadd(fmul(l_mine, alpha_mine), rows_reduce<true>(rm, lane));
+    // P~ of the lane's rows: key rows 8 tx + c, one chunk of four rows each
+    __syncwarp();                                    // the previous block's P.V loads are done
+    float* pchunk = Ps + (size_t)(8 * tx) * FQ + (((lrow >> 2) ^ ((tx & 3) << 1)) << 2);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      *reinterpret_cast<float4*>(pchunk + (2 * j) * FQ) = make_float4(acc[0][j].x, acc[1][j].x, acc[2][j].x, acc[3][j].x);
+      *reinterpret_cast<float4*>(pchunk + (2 * j + 1) * FQ) = make_float4(acc[0][j].y, acc[1][j].y, acc[2][j].y, acc[3][j].y);
     }
     const int tiny_p = __any_sync(0xffffffffu, tp);  // also orders the stores before the loads below
     __syncwarp();
     // ---- u = P~ . V over the block's keys ascending from +0, then o = o * alpha + u ----
 #pragma unroll
-    for (int a = 0; a < AF_RW / 2; ++a)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) acc[a][c] = make_float2(0.0f, 0.0f);
+      for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
     // on the diagonal the warp's rows see no key beyond its last row, the CTA's none beyond its own last row
     const int last_slab = diag ? (q0 - j0 + wrow + AF_RW - 1) / OK : 7, last_block = diag ? (q0 - j0 + FQ - 1) / OK : 7;
     for (int sl = 0; sl <= last_block; ++sl) {
@@ -355,17 +358,17 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
       if (!acquire()) { ok = false; break; }
       if (sl <= last_slab) {
         const float* ap = Ps + (size_t)(sl * OK) * FQ;
-        if (tiny) mac_8x4<false, true>(ap, FQ, wrow >> 2, sl * OK, Ring[slot], lane, acc);
-        else mac_8x4<true, true>(ap, FQ, wrow >> 2, sl * OK, Ring[slot], lane, acc);
+        if (tiny) mac_4x8<false, true>(ap, FQ, lrow >> 2, sl * OK, Ring[slot], tx, acc);
+        else mac_4x8<true, true>(ap, FQ, lrow >> 2, sl * OK, Ring[slot], tx, acc);
       }
       release();
     }
     if (!ok) break;
 #pragma unroll
-    for (int i = 0; i < AF_RW; ++i) {  // scalar: the product o * alpha is rounded before the add
-      const float al = __shfl_sync(0xffffffffu, alpha_mine, ROW_LANE(i));
+    for (int i = 0; i < 4; ++i) {  // the product o * alpha is rounded before the add
+      const float2 al = same2(__shfl_sync(0xffffffffu, alpha_mine, LANE_OF_ROW(i)));
 #pragma unroll
-      for (int c = 0; c < 4; ++c) RP(o, i, c) = fadd(fmul(RP(o, i, c), al), RP(acc, i, c));
+      for (int j = 0; j < 4; ++j) o[i][j] = add2(mul2(o[i][j], al), acc[i][j], one);
     }
   }
   if (!ok) return;
@@ -374,19 +377,20 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
   if (lane < AF_RW && q0 + wrow + ROW_OF_LANE(lane) < S) lse[((size_t)b * H + h) * S + q0 + wrow + ROW_OF_LANE(lane)] = lse_mine;
   const float inv_q = qout ? fdiv(1.0f, s_q[0]) : 0.0f;
 #pragma unroll
-  for (int i = 0; i < AF_RW; ++i) {
-    const int row = q0 + wrow + i;
-    const float il = __shfl_sync(0xffffffffu, il_mine, ROW_LANE(i));
+  for (int i = 0; i < 4; ++i) {
+    const int row = q0 + lrow + i;
+    const float il = __shfl_sync(0xffffffffu, il_mine, LANE_OF_ROW(i));
     if (row >= S) continue;
-    uint2 w0;
-    w0.x = pack_bf2(fmul(RP(o, i, 0), il), fmul(RP(o, i, 1), il));
-    w0.y = pack_bf2(fmul(RP(o, i, 2), il), fmul(RP(o, i, 3), il));
-    *reinterpret_cast<uint2*>(out + (row0 + row) * ld_out + (size_t)h * DH + 4 * lane) = w0;
-    if (qout) {   // the output projection's quantiser, applied to the bf16 values just stored
-      const float f0 = bflo(w0.x), f1 = bfhi(w0.x), f2 = bflo(w0.y), f3 = bfhi(w0.y);
-      const uint32_t c = ((uint32_t)(uint8_t)quant1(f0, inv_q)) | ((uint32_t)(uint8_t)quant1(f1, inv_q) << 8) |
-                         ((uint32_t)(uint8_t)quant1(f2, inv_q) << 16) | ((uint32_t)(uint8_t)quant1(f3, inv_q) << 24);
-      *reinterpret_cast<uint32_t*>(qout + (row0 + row) * ld_out + (size_t)h * DH + 4 * lane) = c;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      const float2 x = o[i][2 * g], y = o[i][2 * g + 1];
+      const uint2 w = make_uint2(pack_bf2(fmul(x.x, il), fmul(x.y, il)), pack_bf2(fmul(y.x, il), fmul(y.y, il)));
+      const size_t off = (row0 + row) * ld_out + (size_t)h * DH + 64 * g + 4 * tx;
+      *reinterpret_cast<uint2*>(out + off) = w;
+      if (qout)   // the output projection's quantiser, applied to the bf16 values just stored
+        *reinterpret_cast<uint32_t*>(qout + off) =
+            ((uint32_t)(uint8_t)quant1(bflo(w.x), inv_q)) | ((uint32_t)(uint8_t)quant1(bfhi(w.x), inv_q) << 8) |
+            ((uint32_t)(uint8_t)quant1(bflo(w.y), inv_q) << 16) | ((uint32_t)(uint8_t)quant1(bfhi(w.y), inv_q) << 24);
     }
   }
 }
@@ -597,8 +601,8 @@ static int attn_fwd_run(const det_bf16* q, const det_bf16* k, const det_bf16* v,
 }
 // Rows per CTA: the longest chain of key blocks runs on one SM whatever the others do, and all chains together share the
 // GPU; the figures are the microseconds per key block of a CTA alone on its SM and of one among many, and the row count
-// with the smallest of the larger bounds is taken (16 heads x 832: 0.187 ms with 128 rows, 0.136 with 64, 0.128 with 32;
-// 64 heads x 2048: 1.56, 1.65 and 1.92 ms).
+// with the smallest of the larger bounds is taken (16 heads x 832: 0.178 ms with 128 rows, 0.129 with 64, 0.117 with 32;
+// 64 heads x 2048: 1.48, 1.55 and 1.75 ms).
 struct RowCost { int rows; double alone, full; };
 template <int N>
 static int pick_rows(const RowCost (&c)[N], int heads, int S, int window) {
@@ -619,7 +623,7 @@ static int pick_rows(const RowCost (&c)[N], int heads, int S, int window) {
   return best;
 }
 static int attn_rows(int heads, int S, int window) {
-  const RowCost c[3] = {{128, 26.6, 26.6}, {64, 18.0, 14.1}, {32, 14.0, 8.1}};
+  const RowCost c[3] = {{128, 25.1, 25.1}, {64, 17.0, 13.2}, {32, 13.0, 7.5}};
   return pick_rows(c, heads, S, window);
 }
 static int sdp_rows(int heads, int S, int window) {

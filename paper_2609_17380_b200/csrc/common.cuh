@@ -107,6 +107,53 @@ __device__ __forceinline__ float det_exp_le0(float x) {
 // multiply-add is wanted and proven identical; every multiply-then-add whose product must be rounded on its own is
 // written with the scalar intrinsics, which ptxas never contracts.
 
+// Two lanes of unfused arithmetic per instruction.  A packed multiply followed by a packed ADD would be contracted (above); a
+// packed multiply followed by a packed FUSED multiply-add with a factor that is 1 but not known to the compiler cannot be, and
+// p * 1 + c rounds exactly like p + c.  The factor is read from constant memory.
+static __constant__ float c_one = 1.0f;
+__device__ __forceinline__ unsigned long long f2bits(float2 a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+  return r;
+}
+__device__ __forceinline__ float2 bits2f(unsigned long long r) {
+  float2 a;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
+  return a;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2bits(a)), "l"(f2bits(b)));
+  return bits2f(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  unsigned long long r;
+  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2bits(a)), "l"(f2bits(b)), "l"(f2bits(c)));
+  return bits2f(r);
+}
+__device__ __forceinline__ float2 same2(float a) { return make_float2(a, a); }
+// a + b for an `a` that may be a packed product; one = {1, 1} from constant memory
+__device__ __forceinline__ float2 add2(float2 a, float2 b, float2 one) { return fma2(a, one, b); }
+
+// det_exp_le0 of two arguments, same bits: every product and every sum is rounded on its own, except x - k ln2_hi, whose
+// product is exact (17 significant bits times at most 8 wherever the result is kept) so that one fused instruction rounds
+// the same value once.
+__device__ __forceinline__ float2 det_exp_le0_2(float2 x, float2 one) {
+  const float2 km = add2(mul2(x, same2(0x1.715476p+0f)), same2(12582912.0f), one);
+  const float2 kf = add2(km, same2(-12582912.0f), one);
+  const float2 r = add2(mul2(kf, same2(-0x1.7f7d1cp-20f)), fma2(kf, same2(-0x1.62e400p-1f), x), one);
+  float2 p = add2(mul2(r, same2(0x1.a01a02p-13f)), same2(0x1.6c16c2p-10f), one);
+  p = add2(mul2(p, r), same2(0x1.111112p-7f), one);
+  p = add2(mul2(p, r), same2(0x1.555556p-5f), one);
+  p = add2(mul2(p, r), same2(0x1.555556p-3f), one);
+  p = add2(mul2(p, r), same2(0.5f), one);
+  p = add2(mul2(p, r), same2(1.0f), one);
+  p = add2(mul2(p, r), same2(1.0f), one);
+  const float2 v = mul2(p, make_float2(__int_as_float((int)(__float_as_uint(km.x) << 23) + 0x3f800000),
+                                       __int_as_float((int)(__float_as_uint(km.y) << 23) + 0x3f800000)));
+  return make_float2((x.x < -0x1.5d58a0p+6f) ? 0.0f : v.x, (x.y < -0x1.5d58a0p+6f) ? 0.0f : v.y);
+}
+
 // log: for normal x > 0, x = 2^e m, m in (sqrt(1/2), sqrt(2)], s = (m-1)/(m+1), z = s^2,
 // log m = 2 s (1 + z/3 + z^2/5 + z^3/7 + z^4/9).
 __device__ __forceinline__ float det_log(float x) {

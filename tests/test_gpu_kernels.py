@@ -92,3 +92,15 @@ def test_attention_row_blocks(det, B, H, Hkv, S, W, fixq):
     got = host(dqkv, np.uint16)
     for name, lo, hi in (("dq", 0, HD), ("dk", HD, HD + KD), ("dv", HD + KD, ld)):
         assert_same_bits(got[:, lo:hi], want[:, lo:hi], name)
+
+
+# the two-lane exponential: a dense grid of arguments, the ends of the kept range, subnormal, infinite and NaN arguments
+def test_two_lane_exponential(det):
+    x = np.concatenate([np.linspace(-90, 0, 400001), np.linspace(-87.4, -87.2, 20001), [0.0, -0.0, -1e-40, -1e-30, -200.0, -1e30, -np.inf, np.nan]]).astype(F)
+    a, got, want = dev(x), empty(x.shape, F), empty(x.shape, F)
+    det.det_test_prim(11, a, None, got)
+    det.det_test_prim(5, a, None, want)
+    _sync()
+    n = np.isnan(x)
+    assert_same_bits(host(got)[~n], host(want)[~n], "exp")
+    assert np.isnan(host(got)[n]).all()
