@@ -527,6 +527,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     Lr[a] = i < S ? lse[bh * S + i] : 0.0f;
     Dr[a] = i < S ? delta[bh * S + i] : 0.0f;
   }
+  const float2 one = same2(c_one);
   int slot = 0;
   uint32_t par = 0;
   bool ok = true;
@@ -548,31 +549,49 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
       if (++slot == SDP_SLOTS) { slot = 0; par ^= 1u; }
     }
     if (!ok) break;
+    // P = exp(S*scale - L) and dS, two pairs at a time; the argument is at most 0 whenever L is the row's own logsumexp, and
+    // then the exponential without the overflow range applies (same bits), but L is an input, so four pairs that hold
+    // a positive argument take the general form.  Only the block at the diagonal and those at the window's start mask.
+    const bool masked = j0 + OT - 1 > i0 || (W > 0 && j0 <= i0 + TM - 1 - W);
 #pragma unroll
     for (int a = 0; a < 8; ++a) {
       const int i = i0 + (a >> 2) * (TM / 2) + ty * 4 + (a & 3);
       if (i >= S) continue;
+      const float2 L2 = same2(-Lr[a]), D2 = same2(-Dr[a]);
 #pragma unroll
       for (int g = 0; g < 2; ++g) {
         const int jb = j0 + g * 64 + tx * 4;
         if (jb >= S) continue;
-        const float sv[4] = {sa[a][2 * g].x, sa[a][2 * g].y, sa[a][2 * g + 1].x, sa[a][2 * g + 1].y};
-        const float dv4[4] = {da[a][2 * g].x, da[a][2 * g].y, da[a][2 * g + 1].x, da[a][2 * g + 1].y};
-        float pv[4], dsv[4];
+        float2 x[2], pv[2], ds[2];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {   // branch-free (selects), so that the exponentials' chains interleave
-          const bool vis = jb + e <= i && (W == 0 || jb + e > i - W);
-          const float pe = det_exp(fsub(fmul(sv[e], ATT_SCALE), Lr[a]));
-          const float de = fmul(fmul(pe, fsub(dv4[e], Dr[a])), ATT_SCALE);
-          pv[e] = vis ? pe : 0.0f;
-          dsv[e] = vis ? de : 0.0f;
+        for (int t = 0; t < 2; ++t) x[t] = add2(mul2(sa[a][2 * g + t], same2(ATT_SCALE)), L2, one);
+        bool vis[4] = {true, true, true, true};
+        if (masked) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) vis[e] = jb + e <= i && (W == 0 || jb + e > i - W);
+          x[0] = make_float2(vis[0] ? x[0].x : 0.0f, vis[1] ? x[0].y : 0.0f);
+          x[1] = make_float2(vis[2] ? x[1].x : 0.0f, vis[3] ? x[1].y : 0.0f);
+        }
+        if (x[0].x > 0.0f || x[0].y > 0.0f || x[1].x > 0.0f || x[1].y > 0.0f) {
+#pragma unroll
+          for (int t = 0; t < 2; ++t) pv[t] = make_float2(det_exp(x[t].x), det_exp(x[t].y));
+        } else {
+#pragma unroll
+          for (int t = 0; t < 2; ++t) pv[t] = det_exp_le0_2(x[t], one);
+        }
+#pragma unroll
+        for (int t = 0; t < 2; ++t) ds[t] = mul2(mul2(pv[t], add2(da[a][2 * g + t], D2, one)), same2(ATT_SCALE));
+        if (masked) {
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {
+            pv[t] = make_float2(vis[2 * t] ? pv[t].x : 0.0f, vis[2 * t + 1] ? pv[t].y : 0.0f);
+            ds[t] = make_float2(vis[2 * t] ? ds[t].x : 0.0f, vis[2 * t + 1] ? ds[t].y : 0.0f);
+          }
         }
         const size_t off = (bh * S + i) * S + jb;
-        uint2 u;
-        u.x = pack_bf2(pv[0], pv[1]); u.y = pack_bf2(pv[2], pv[3]);        // P~ = bf16(P) is all the value gradient needs
-        *reinterpret_cast<uint2*>(Pb + off) = u;
-        u.x = pack_bf2(dsv[0], dsv[1]); u.y = pack_bf2(dsv[2], dsv[3]);
-        *reinterpret_cast<uint2*>(dSt + off) = u;
+        // P~ = bf16(P) is all the value gradient needs
+        *reinterpret_cast<uint2*>(Pb + off) = make_uint2(pack_bf2(pv[0].x, pv[0].y), pack_bf2(pv[1].x, pv[1].y));
+        *reinterpret_cast<uint2*>(dSt + off) = make_uint2(pack_bf2(ds[0].x, ds[0].y), pack_bf2(ds[1].x, ds[1].y));
       }
     }
   }

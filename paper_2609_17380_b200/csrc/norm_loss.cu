@@ -472,17 +472,21 @@ __global__ void __launch_bounds__(XT) k_xent_fwd(const float* __restrict__ logit
   for (int w = 1; w < XT / 32; ++w) m = fmaxf(m, red[w]);
   const int nl = (V + 255) >> 8;
   // every argument z - m is <= 0 (or NaN), so the exponential without the overflow range applies
+  const float2 one = same2(c_one);
   const int nfull = V >> 8;  // leaves that lie wholly inside the row: no existence tests in their tree
   for (int leaf = warp; leaf < nfull; leaf += XT / 32) {
     const int e0 = leaf * 256 + lane * 8;
     // second and last read of the row: streaming loads, so that these lines leave L2 before the rows still waiting
     // between their two sweeps (the rows in flight on all SMs together fill most of L2)
     const float4 a0 = __ldcs(reinterpret_cast<const float4*>(z + e0)), a1 = __ldcs(reinterpret_cast<const float4*>(z + e0 + 4));
+    const float2 z8[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y), make_float2(a1.z, a1.w)};
     float e[8];
-    e[0] = det_exp_le0(fsub(a0.x, m)); e[1] = det_exp_le0(fsub(a0.y, m));          // branch-free: the chains interleave
-    e[2] = det_exp_le0(fsub(a0.z, m)); e[3] = det_exp_le0(fsub(a0.w, m));
-    e[4] = det_exp_le0(fsub(a1.x, m)); e[5] = det_exp_le0(fsub(a1.y, m));
-    e[6] = det_exp_le0(fsub(a1.z, m)); e[7] = det_exp_le0(fsub(a1.w, m));
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {          // branch-free, two at a time: the chains interleave
+      const float2 v = det_exp_le0_2(add2(z8[t], same2(-m), one), one);
+      e[2 * t] = v.x;
+      e[2 * t + 1] = v.y;
+    }
     const float s = warp_tree_full(tree8_full(e));
     if (lane == 0) leafs[leaf] = s;
   }
@@ -536,6 +540,7 @@ __global__ void __launch_bounds__(256) k_xent_bwd(float* __restrict__ logits, co
   const int i0 = blockIdx.x * 2048 + threadIdx.x * 4;
   if (i0 >= V) return;
   const bool two = i0 + 1024 < V;
+  const float2 one = same2(c_one);
   for (int row = blockIdx.y; row < rows; row += gridDim.y) {
     float* z = logits + (size_t)row * V;
     const int t = target[row];
@@ -551,7 +556,11 @@ __global__ void __launch_bounds__(256) k_xent_bwd(float* __restrict__ logits, co
     float p[8];
     if (!pos) {
 #pragma unroll
-      for (int k = 0; k < 8; ++k) p[k] = det_exp_le0(x[k]);
+      for (int k = 0; k < 8; k += 2) {
+        const float2 v = det_exp_le0_2(make_float2(x[k], x[k + 1]), one);
+        p[k] = v.x;
+        p[k + 1] = v.y;
+      }
     } else {
 #pragma unroll
       for (int k = 0; k < 8; ++k) p[k] = det_exp(x[k]);
