@@ -309,6 +309,10 @@ typedef struct {
 /* p: bf16 (pdtype DET_BF16) or f32 (DET_F32) parameters, updated in place; g, m, v f32 */
 int det_adamw_step(const det_adamw_desc* h, int pdtype, void* p, const float* g, float* m, float* v, size_t n,
                    void* stream);
+/* The update of many tensors at once: descs, pdtypes, p, g, m, v, n are HOST arrays of ntensors entries.  With coef_dev (device
+ * scalar, may be NULL) every g[t][i] is first multiplied by *coef_dev and stored, exactly as det_scale_inplace does. */
+int det_adamw_batch(const det_adamw_desc* descs, const int* pdtypes, void* const* p, float* const* g, float* const* m,
+                    float* const* v, const size_t* n, int ntensors, const float* coef_dev, void* stream);
 
 /* ---- tensor hash (Appendix B: per-step state hash, here on the device) --------------------------------
  * Level 1: SHA-256 of every 4 KiB chunk of the raw bytes (last chunk may be shorter).  While more than 128

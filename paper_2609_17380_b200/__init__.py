@@ -368,6 +368,15 @@ def det_adamw_step(desc, pdtype, p, g, m, v, n):
                                                    C.c_size_t(n), _stream()))
 
 
+def det_adamw_batch(descs, pdtypes, ps, gs, ms, vs, coef_dev=None):
+    """One launch for many tensors; coef_dev: device scalar every gradient is multiplied with first (in place)."""
+    k = len(ps)
+    table = lambda ts: (C.c_void_p * k)(*[t.data_ptr() for t in ts])
+    _check("det_adamw_batch", load().det_adamw_batch((det_adamw_desc * k)(*descs), (C.c_int * k)(*pdtypes), table(ps), table(gs),
+                                                     table(ms), table(vs), (C.c_size_t * k)(*[t.numel() for t in ps]), C.c_int(k),
+                                                     _ptr(coef_dev), _stream()))
+
+
 def det_tensor_hash_ws_bytes(nbytes):
     return load().det_tensor_hash_ws_bytes(C.c_size_t(nbytes))
 
@@ -385,16 +394,15 @@ def det_tensor_hash(p, nbytes, ws):
     return bytes(out).hex()
 
 
-def _byte_counts(tensors):
-    return (C.c_size_t * len(tensors))(*[t.numel() * t.element_size() for t in tensors])
-
-
-def det_tensor_hash_batch_ws_bytes(tensors):
-    return load().det_tensor_hash_batch_ws_bytes(_byte_counts(tensors), C.c_int(len(tensors)))
+def det_tensor_hash_batch_ws_bytes(nbytes):
+    """nbytes: byte counts of the tensors, or the tensors themselves."""
+    counts = [n if isinstance(n, int) else n.numel() * n.element_size() for n in nbytes]
+    return load().det_tensor_hash_batch_ws_bytes((C.c_size_t * len(counts))(*counts), C.c_int(len(counts)))
 
 
 def det_tensor_hash_batch(tensors, roots_dev, ws):
     """Queues the hashes of all tensors together; root t lands at roots_dev[32 t : 32 t + 32] in stream order."""
-    ptrs = (C.c_void_p * len(tensors))(*[t.data_ptr() for t in tensors])
-    _check("det_tensor_hash_batch", load().det_tensor_hash_batch(ptrs, _byte_counts(tensors), C.c_int(len(tensors)),
-                                                                 _ptr(roots_dev), *_ws(ws), _stream()))
+    k = len(tensors)
+    ptrs = (C.c_void_p * k)(*[t.data_ptr() for t in tensors])
+    counts = (C.c_size_t * k)(*[t.numel() * t.element_size() for t in tensors])
+    _check("det_tensor_hash_batch", load().det_tensor_hash_batch(ptrs, counts, C.c_int(k), _ptr(roots_dev), *_ws(ws), _stream()))

@@ -247,6 +247,66 @@ __device__ __forceinline__ void smem_tree(float* buf, int n) {
   }
 }
 
+constexpr int SUM_CHUNK = 16384;
+// The sum of chunk `base` .. base + SUM_CHUNK of x[0..n): a perfect subtree, or the ragged last one with existence
+// predicates.  All 256 threads of the CTA call it; thread 0 gets the result.
+template <bool SQ>
+__device__ __forceinline__ float chunk_sum(const float* __restrict__ x, long long base, long long n, float (&wsum)[8]) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float s[8], r;
+  const bool full = base + SUM_CHUNK <= n;
+  if (full) {
+    float4 a[8], b[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float4* p = reinterpret_cast<const float4*>(x + base + (warp * 8 + j) * 256 + lane * 8);
+      a[j] = __ldg(p);
+      b[j] = __ldg(p + 1);
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      float v[8] = {a[j].x, a[j].y, a[j].z, a[j].w, b[j].x, b[j].y, b[j].z, b[j].w};
+      if (SQ) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) v[t] = fmul(v[t], v[t]);
+      }
+      s[j] = warp_tree_full(tree8_full(v));
+    }
+    r = fadd(fadd(fadd(s[0], s[1]), fadd(s[2], s[3])), fadd(fadd(s[4], s[5]), fadd(s[6], s[7])));
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const long long lf = base + (warp * 8 + j) * 256;
+      const long long e0 = lf + lane * 8;
+      float v[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        float u = (e0 + t < n) ? x[e0 + t] : 0.0f;
+        v[t] = SQ ? fmul(u, u) : u;
+      }
+      s[j] = lf < n ? warp_tree(tree8(v, e0, n), lf, 8, n) : 0.0f;
+    }
+    r = reg_tree<8>(s, base + (long long)warp * 2048, 256, n);
+  }
+  if (lane == 0) wsum[warp] = r;
+  __syncthreads();
+  r = 0.0f;
+  if (threadIdx.x == 0) {
+    if (full) {
+      r = fadd(fadd(fadd(wsum[0], wsum[1]), fadd(wsum[2], wsum[3])), fadd(fadd(wsum[4], wsum[5]), fadd(wsum[6], wsum[7])));
+    } else {
+      float w[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) w[j] = wsum[j];
+      r = reg_tree<8>(w, base, 2048, n);
+      // a lone element is carried by the tree without any addition; flush it explicitly, as every value that enters or
+      // leaves an operation is flushed
+      if (n == 1 && !(__float_as_uint(r) & 0x7f800000u)) r = __uint_as_float(__float_as_uint(r) & 0x80000000u);
+    }
+  }
+  return r;
+}
+
 __device__ __forceinline__ void or_status(int* status, int bit) {
   if (status) atomicOr(status, bit);
 }

@@ -210,52 +210,78 @@ __global__ void __launch_bounds__(256) k_accum_result(ResultOp op, size_t n) {
 // AdamW
 // ------------------------------------------------------------------------------------------------
 struct AdamScalars { float b1, b2, omb1, omb2, eps, stepsz, isb2, decay; };
-template <bool BF>
-__global__ void __launch_bounds__(256) k_adamw(AdamScalars h, void* __restrict__ p, const float* __restrict__ g,
-                                               float* __restrict__ m, float* __restrict__ v, size_t n) {
-  size_t i = ((size_t)blockIdx.x * 256 + threadIdx.x) * 4;
-  if (i >= n) return;
-  const int cnt = (n - i) < 4 ? (int)(n - i) : 4;
-  float pv[4], gv[4], mv[4], vv[4];
-  if (cnt == 4) {
-    float4 t = *reinterpret_cast<const float4*>(g + i); gv[0] = t.x; gv[1] = t.y; gv[2] = t.z; gv[3] = t.w;
-    t = *reinterpret_cast<const float4*>(m + i); mv[0] = t.x; mv[1] = t.y; mv[2] = t.z; mv[3] = t.w;
-    t = *reinterpret_cast<const float4*>(v + i); vv[0] = t.x; vv[1] = t.y; vv[2] = t.z; vv[3] = t.w;
+constexpr int ADAM_JOBS = 128;   // tensors per launch
+// Job j: tensors p[j] (bf16 or f32), g[j], m[j], v[j] of n[j] elements, scalars h[j]; its blocks (1024 elements each) have the
+// numbers first[j] .. first[j + 1] - 1.
+struct AdamJobs {
+  int n;
+  uint32_t first[ADAM_JOBS + 1];
+  void* p[ADAM_JOBS];
+  float* g[ADAM_JOBS];
+  float* m[ADAM_JOBS];
+  float* v[ADAM_JOBS];
+  size_t len[ADAM_JOBS];
+  AdamScalars h[ADAM_JOBS];
+  uint8_t bf[ADAM_JOBS];
+};
+__device__ __forceinline__ void adam1(const AdamScalars& h, float& p, float g, float& m, float& v) {
+  m = fadd(fmul(h.b1, m), fmul(h.omb1, g));
+  v = fadd(fmul(h.b2, v), fmul(h.omb2, fmul(g, g)));
+  const float den = fadd(fmul(fsqrt(v), h.isb2), h.eps);
+  p = fsub(fmul(p, h.decay), fmul(h.stepsz, fdiv(m, den)));
+}
+// CLIP: g *= *coef first, stored (the clip of the global norm fused into the pass that reads g anyway: 26 bytes per
+// parameter instead of 22 + 8 in two passes)
+template <bool BF, bool CLIP>
+__device__ __forceinline__ void adam_block(const AdamScalars& h, float c, void* __restrict__ p, float* __restrict__ g,
+                                           float* __restrict__ m, float* __restrict__ v, size_t i, size_t n) {
+  uint16_t* pb = reinterpret_cast<uint16_t*>(p);
+  float* pf = reinterpret_cast<float*>(p);
+  if (i + 4 <= n) {
+    const float4 g4 = *reinterpret_cast<const float4*>(g + i), m4 = *reinterpret_cast<const float4*>(m + i);
+    const float4 v4 = *reinterpret_cast<const float4*>(v + i);
+    float gv[4] = {g4.x, g4.y, g4.z, g4.w}, mv[4] = {m4.x, m4.y, m4.z, m4.w}, vv[4] = {v4.x, v4.y, v4.z, v4.w}, pv[4];
     if (BF) {
-      uint2 u = *reinterpret_cast<const uint2*>(reinterpret_cast<uint16_t*>(p) + i);
+      const uint2 u = *reinterpret_cast<const uint2*>(pb + i);
       pv[0] = bflo(u.x); pv[1] = bfhi(u.x); pv[2] = bflo(u.y); pv[3] = bfhi(u.y);
     } else {
-      t = *reinterpret_cast<const float4*>(reinterpret_cast<float*>(p) + i); pv[0] = t.x; pv[1] = t.y; pv[2] = t.z; pv[3] = t.w;
+      const float4 t = *reinterpret_cast<const float4*>(pf + i);
+      pv[0] = t.x; pv[1] = t.y; pv[2] = t.z; pv[3] = t.w;
     }
-  } else {
-    for (int k = 0; k < 4; ++k) {
-      bool ok = k < cnt;
-      gv[k] = ok ? g[i + k] : 0.f; mv[k] = ok ? m[i + k] : 0.f; vv[k] = ok ? v[i + k] : 0.f;
-      pv[k] = ok ? (BF ? bf2f(reinterpret_cast<uint16_t*>(p)[i + k]) : reinterpret_cast<float*>(p)[i + k]) : 0.f;
-    }
-  }
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    mv[k] = fadd(fmul(h.b1, mv[k]), fmul(h.omb1, gv[k]));
-    vv[k] = fadd(fmul(h.b2, vv[k]), fmul(h.omb2, fmul(gv[k], gv[k])));
-    float den = fadd(fmul(fsqrt(vv[k]), h.isb2), h.eps);
-    pv[k] = fsub(fmul(pv[k], h.decay), fmul(h.stepsz, fdiv(mv[k], den)));
-  }
-  if (cnt == 4) {
+    for (int k = 0; k < 4; ++k) {
+      if (CLIP) gv[k] = fmul(gv[k], c);
+      adam1(h, pv[k], gv[k], mv[k], vv[k]);
+    }
+    if (CLIP) *reinterpret_cast<float4*>(g + i) = make_float4(gv[0], gv[1], gv[2], gv[3]);
     *reinterpret_cast<float4*>(m + i) = make_float4(mv[0], mv[1], mv[2], mv[3]);
     *reinterpret_cast<float4*>(v + i) = make_float4(vv[0], vv[1], vv[2], vv[3]);
-    if (BF) {
-      uint2 u; u.x = pack_bf2(pv[0], pv[1]); u.y = pack_bf2(pv[2], pv[3]);
-      *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(p) + i) = u;
-    } else {
-      *reinterpret_cast<float4*>(reinterpret_cast<float*>(p) + i) = make_float4(pv[0], pv[1], pv[2], pv[3]);
-    }
+    if (BF) *reinterpret_cast<uint2*>(pb + i) = make_uint2(pack_bf2(pv[0], pv[1]), pack_bf2(pv[2], pv[3]));
+    else *reinterpret_cast<float4*>(pf + i) = make_float4(pv[0], pv[1], pv[2], pv[3]);
   } else {
-    for (int k = 0; k < cnt; ++k) {
-      m[i + k] = mv[k]; v[i + k] = vv[k];
-      if (BF) reinterpret_cast<uint16_t*>(p)[i + k] = f2bf(pv[k]); else reinterpret_cast<float*>(p)[i + k] = pv[k];
+    for (; i < n; ++i) {
+      float gk = g[i], mk = m[i], vk = v[i], pk = BF ? bf2f(pb[i]) : pf[i];
+      if (CLIP) g[i] = gk = fmul(gk, c);
+      adam1(h, pk, gk, mk, vk);
+      m[i] = mk;
+      v[i] = vk;
+      if (BF) pb[i] = f2bf(pk); else pf[i] = pk;
     }
   }
+}
+template <bool CLIP>
+__global__ void __launch_bounds__(256) k_adamw(const __grid_constant__ AdamJobs jobs, const float* __restrict__ coef) {
+  int lo = 0, hi = jobs.n - 1;         // the last job whose first block is <= this one
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (jobs.first[mid] <= blockIdx.x) lo = mid; else hi = mid - 1;
+  }
+  const size_t i = ((size_t)(blockIdx.x - jobs.first[lo]) * 256 + threadIdx.x) * 4, n = jobs.len[lo];
+  if (i >= n) return;
+  const AdamScalars h = jobs.h[lo];
+  const float c = CLIP ? coef[0] : 1.0f;
+  if (jobs.bf[lo]) adam_block<true, CLIP>(h, c, jobs.p[lo], jobs.g[lo], jobs.m[lo], jobs.v[lo], i, n);
+  else adam_block<false, CLIP>(h, c, jobs.p[lo], jobs.g[lo], jobs.m[lo], jobs.v[lo], i, n);
 }
 
 static double ipow(double b, int e) {
@@ -423,12 +449,13 @@ extern "C" int det_grad_accum_result(det_accum* st, float* g_out, void* stream) 
   return DET_OK;
 }
 
-extern "C" int det_adamw_step(const det_adamw_desc* d, int pdtype, void* p, const float* g, float* m, float* v,
-                              size_t n, void* stream) {
+static int adamw_check(const det_adamw_desc* d, int pdtype, const void* p, const float* g, const float* m, const float* v) {
   if (!d || !p || !g || !m || !v || d->step < 1 || (pdtype != DET_F32 && pdtype != DET_BF16)) return DET_ERR_ARG;
   if (!aligned16(g) || !aligned16(m) || !aligned16(v) || (((uintptr_t)p) & 7u)) return DET_ERR_ALIGN;
   if (pdtype == DET_F32 && !aligned16(p)) return DET_ERR_ALIGN;
-  if (!n) return DET_OK;
+  return DET_OK;
+}
+static AdamScalars adamw_scalars(const det_adamw_desc* d) {
   const double bc1 = 1.0 - ipow(d->beta1, d->step), bc2 = 1.0 - ipow(d->beta2, d->step);
   AdamScalars h;
   h.b1 = (float)d->beta1; h.b2 = (float)d->beta2;
@@ -437,9 +464,46 @@ extern "C" int det_adamw_step(const det_adamw_desc* d, int pdtype, void* p, cons
   h.stepsz = (float)(d->lr / bc1);
   h.isb2 = (float)(1.0 / sqrt(bc2));
   h.decay = (float)(1.0 - d->lr * d->weight_decay);
-  unsigned grid = (unsigned)((n + 1023) / 1024);
-  if (pdtype == DET_BF16) k_adamw<true><<<DET_L(grid), 256, 0, (cudaStream_t)stream>>>(h, p, g, m, v, n);
-  else k_adamw<false><<<DET_L(grid), 256, 0, (cudaStream_t)stream>>>(h, p, g, m, v, n);
-  DET_CHECK_LAUNCH();
+  return h;
+}
+// One launch for many tensors: the 87 tensors of a 12-layer model took 87 launches of 9.9 us on average for 0.6 ms of
+// memory traffic.
+extern "C" int det_adamw_batch(const det_adamw_desc* descs, const int* pdtypes, void* const* p, float* const* g, float* const* m,
+                               float* const* v, const size_t* n, int ntensors, const float* coef_dev, void* stream) {
+  if (ntensors < 0 || (ntensors && (!descs || !pdtypes || !p || !g || !m || !v || !n))) return DET_ERR_ARG;
+  for (int t = 0; t < ntensors; ++t) {
+    if (!n[t]) continue;
+    const int rc = adamw_check(&descs[t], pdtypes[t], p[t], g[t], m[t], v[t]);
+    if (rc != DET_OK) return rc;
+  }
+  for (int t = 0; t < ntensors;) {
+    AdamJobs jobs;
+    jobs.n = 0;
+    size_t c = 0;
+    for (; t < ntensors && jobs.n < ADAM_JOBS; ++t) {
+      if (!n[t]) continue;
+      const size_t blocks = (n[t] + 1023) / 1024;
+      if (c + blocks > 0x7fffffffull) { if (!jobs.n) return DET_ERR_SHAPE; break; }
+      const int j = jobs.n++;
+      jobs.first[j] = (uint32_t)c;
+      jobs.p[j] = p[t]; jobs.g[j] = g[t]; jobs.m[j] = m[t]; jobs.v[j] = v[t];
+      jobs.len[j] = n[t];
+      jobs.h[j] = adamw_scalars(&descs[t]);
+      jobs.bf[j] = pdtypes[t] == DET_BF16;
+      c += blocks;
+    }
+    if (!jobs.n) break;
+    jobs.first[jobs.n] = (uint32_t)c;
+    if (coef_dev) k_adamw<true><<<DET_L((unsigned)c), 256, 0, (cudaStream_t)stream>>>(jobs, coef_dev);
+    else k_adamw<false><<<DET_L((unsigned)c), 256, 0, (cudaStream_t)stream>>>(jobs, nullptr);
+    DET_CHECK_LAUNCH();
+  }
   return DET_OK;
+}
+extern "C" int det_adamw_step(const det_adamw_desc* d, int pdtype, void* p, const float* g, float* m, float* v,
+                              size_t n, void* stream) {
+  const int rc = adamw_check(d, pdtype, p, g, m, v);
+  if (rc != DET_OK || !n) return rc;
+  float* gw = const_cast<float*>(g);      // without a clip coefficient g is only read
+  return det_adamw_batch(d, &pdtype, &p, &gw, &m, &v, &n, 1, nullptr, stream);
 }

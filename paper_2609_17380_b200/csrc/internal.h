@@ -12,6 +12,10 @@ int note_launch();
 size_t sum_ws_floats(size_t n);
 // out[0] = det_sum(x[0..n)) (squares: of x^2); launches on st, scratch in ws (sum_ws_floats(n) floats)
 int sum_launch(const float* x, size_t n, int squares, float* out, float* ws, cudaStream_t st);
+// the levels of det_sum(x[0..n)) above SUM_CHUNK nodes: x and n become what is left, ws what is free of the scratch
+void sum_to_chunk(const float*& x, size_t& n, float*& ws, cudaStream_t st);
+// out[0] = gs * det_sum(x[0..n)), the scaling in the launch that finishes the sum; n >= 1, scratch as for sum_launch
+int sum_scaled_launch(const float* x, size_t n, float gs, float* out, float* ws, cudaStream_t st);
 
 // Epilogue descriptions.  All data-dependent scalars are read from device memory.
 enum { EPI_RAW = 0, EPI_FWD = 1, EPI_DX = 2, EPI_DW = 3 };

@@ -493,7 +493,6 @@ __global__ void k_su_finish(const uint32_t* amax, int rotated, float* s_u) {
   const int am = (int)amax[0];
   s_u[0] = (am > 0) ? fdiv(__int2float_rn(am), 127.0f) : 0.0f;
 }
-__global__ void k_dsx_finish(const float* sum, float gs, float* ds_x) { ds_x[0] = fmul(gs, sum[0]); }
 
 }  // namespace det
 
@@ -672,8 +671,7 @@ extern "C" int det_linear_bwd(const det_bf16* dY, const det_bf16* X, const int8_
   rc = igemm_launch(EPI_DW, GqT, ZqT, N, K, M, ew, status_dev, aux.aux(0));
   if (rc != DET_OK) return rc;
   const size_t np = (size_t)M * (K / 128);
-  sum_launch(partial, np, 0, sscr, sscr + 64, st);
-  k_dsx_finish<<<DET_L(1), 1, 0, st>>>(sscr, (float)(1.0 / sqrt((double)M * (double)K * 127.0)), ds_x);
+  sum_scaled_launch(partial, np, (float)(1.0 / sqrt((double)M * (double)K * 127.0)), ds_x, sscr, st);
   DET_CHECK_LAUNCH();
   if (!aux.join()) return DET_ERR_CUDA;
   return DET_OK;

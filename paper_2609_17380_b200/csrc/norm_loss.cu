@@ -524,11 +524,16 @@ __global__ void __launch_bounds__(XT) k_xent_fwd(const float* __restrict__ logit
   }
 }
 
-__global__ void k_xent_finish(const float* ce_sum, const float* z_sum, float inv_rows, float z_weight,
-                              float* loss_mean, float* z_mean) {
-  float ce = fmul(ce_sum[0], inv_rows), zm = fmul(z_sum[0], inv_rows);
+// the last levels of both sums (n <= SUM_CHUNK nodes each) and the means
+__global__ void __launch_bounds__(256) k_xent_finish(const float* __restrict__ ce, const float* __restrict__ zsq, int n, float inv_rows,
+                                                     float z_weight, float* loss_mean, float* z_mean) {
+  __shared__ float wsum[8];
+  const float c = fmul(chunk_sum<false>(ce, 0, n, wsum), inv_rows);
+  __syncthreads();
+  const float zm = fmul(chunk_sum<false>(zsq, 0, n, wsum), inv_rows);
+  if (threadIdx.x) return;
   z_mean[0] = zm;
-  loss_mean[0] = (z_weight != 0.0f) ? fadd(ce, fmul(z_weight, zm)) : ce;
+  loss_mean[0] = (z_weight != 0.0f) ? fadd(c, fmul(z_weight, zm)) : c;
 }
 
 // Each thread takes two groups of four adjacent logits of a row, 1024 columns apart (every access of a warp covers whole
@@ -687,7 +692,7 @@ extern "C" int det_rmsnorm_bwd(int io, const void* dy, const void* x, const void
 extern "C" size_t det_xent_ws_bytes(int rows, int V) {
   (void)V;
   size_t r = align_up((size_t)(rows > 0 ? rows : 1), 64);
-  return (r + 128 + sum_ws_floats((size_t)rows)) * sizeof(float);
+  return (r + 2 * sum_ws_floats((size_t)rows)) * sizeof(float);
 }
 
 extern "C" int det_xent_fwd(const float* logits, const int32_t* target, int rows, int V, float z_weight,
@@ -699,14 +704,16 @@ extern "C" int det_xent_fwd(const float* logits, const int32_t* target, int rows
   if (ws_bytes < det_xent_ws_bytes(rows, V)) return DET_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   float* zsq = (float*)ws;
-  float* sums = zsq + align_up((size_t)rows, 64);
-  float* scratch = sums + 128;
+  float* scratch = zsq + align_up((size_t)rows, 64);
   const int nl = (V + 255) / 256;
   size_t sh = (size_t)(nl < 32 ? 32 : nl) * sizeof(float);
   k_xent_fwd<<<DET_L(rows), XT, sh, st>>>(logits, target, V, loss_row, lse, zsq, status_dev);
-  sum_launch(loss_row, (size_t)rows, 0, sums, scratch, st);
-  sum_launch(zsq, (size_t)rows, 0, sums + 64, scratch, st);
-  k_xent_finish<<<DET_L(1), 1, 0, st>>>(sums, sums + 64, (float)(1.0 / (double)rows), z_weight, loss_mean, z_mean);
+  const float* ce = loss_row;
+  const float* zs = zsq;
+  size_t n = (size_t)rows, nz = (size_t)rows;
+  sum_to_chunk(ce, n, scratch, st);
+  sum_to_chunk(zs, nz, scratch, st);
+  k_xent_finish<<<DET_L(1), 256, 0, st>>>(ce, zs, (int)n, (float)(1.0 / (double)rows), z_weight, loss_mean, z_mean);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }

@@ -86,70 +86,39 @@ int dev_sm_count() {
 }
 unsigned long long launches() { return g_launches.load(std::memory_order_relaxed); }
 
-constexpr int SUM_CHUNK = 16384;
-
 template <bool SQ>
 __global__ void __launch_bounds__(256) k_sum_chunk(const float* __restrict__ x, long long n, float* __restrict__ partial) {
   __shared__ float wsum[8];
-  const long long base = (long long)blockIdx.x * SUM_CHUNK;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float s[8];
-  if (base + SUM_CHUNK <= n) {
-    float4 a[8], b[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float4* p = reinterpret_cast<const float4*>(x + base + (warp * 8 + j) * 256 + lane * 8);
-      a[j] = __ldg(p);
-      b[j] = __ldg(p + 1);
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      float v[8] = {a[j].x, a[j].y, a[j].z, a[j].w, b[j].x, b[j].y, b[j].z, b[j].w};
-      if (SQ) {
-#pragma unroll
-        for (int t = 0; t < 8; ++t) v[t] = fmul(v[t], v[t]);
-      }
-      s[j] = warp_tree_full(tree8_full(v));
-    }
-    float r = fadd(fadd(fadd(s[0], s[1]), fadd(s[2], s[3])), fadd(fadd(s[4], s[5]), fadd(s[6], s[7])));
-    if (lane == 0) wsum[warp] = r;
-    __syncthreads();
-    if (threadIdx.x == 0)
-      partial[blockIdx.x] = fadd(fadd(fadd(wsum[0], wsum[1]), fadd(wsum[2], wsum[3])),
-                                 fadd(fadd(wsum[4], wsum[5]), fadd(wsum[6], wsum[7])));
-    return;
-  }
-  // ragged last chunk: same tree with existence predicates
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const long long lf = base + (warp * 8 + j) * 256;
-    const long long e0 = lf + lane * 8;
-    float v[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      float u = (e0 + t < n) ? x[e0 + t] : 0.0f;
-      v[t] = SQ ? fmul(u, u) : u;
-    }
-    s[j] = warp_tree(tree8(v, e0, n), lf, 8, n);
-  }
-  float r = reg_tree<8>(s, base + (long long)warp * 2048, 256, n);
-  if (lane == 0) wsum[warp] = r;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float w[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) w[j] = wsum[j];
-    partial[blockIdx.x] = reg_tree<8>(w, base, 2048, n);
-  }
+  const float r = chunk_sum<SQ>(x, (long long)blockIdx.x * SUM_CHUNK, n, wsum);
+  if (threadIdx.x == 0) partial[blockIdx.x] = r;
 }
 
-// A lone element (n == 1) is carried by the tree without any addition; flush it explicitly, as every
-// value that enters or leaves an operation is flushed.
-__global__ void k_flush1(const float* x, float* out, int sq) {
-  float v = x[0];
-  uint32_t u = __float_as_uint(v);
-  if (!(u & 0x7f800000u)) v = __uint_as_float(u & 0x80000000u);
-  out[0] = sq ? fmul(v, v) : v;
+// One level of the sums of many tensors: job j is x[j][0..len[j]), its chunks are the blocks from first[j] on (a multiple of
+// four where there are several, so that the next level's loads are aligned), and block c leaves its sum in out[c], or in
+// per[who[j]] where the job has no other chunk.
+constexpr int SUM_JOBS = 256;
+struct SumJobs {
+  int n;
+  uint32_t first[SUM_JOBS + 1];
+  const float* x[SUM_JOBS];
+  long long len[SUM_JOBS];
+  int who[SUM_JOBS];
+};
+template <bool SQ>
+__global__ void __launch_bounds__(256) k_sum_jobs(const __grid_constant__ SumJobs jobs, float* __restrict__ out, float* __restrict__ per) {
+  __shared__ float wsum[8];
+  int lo = 0, hi = jobs.n - 1;         // the last job whose first block is <= this one
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (jobs.first[mid] <= blockIdx.x) lo = mid; else hi = mid - 1;
+  }
+  const long long base = (long long)(blockIdx.x - jobs.first[lo]) * SUM_CHUNK;
+  if (base >= jobs.len[lo]) return;    // a block that only aligns the next job
+  const float r = chunk_sum<SQ>(jobs.x[lo], base, jobs.len[lo], wsum);
+  if (threadIdx.x == 0) {
+    if (jobs.len[lo] <= SUM_CHUNK) per[jobs.who[lo]] = r;
+    else out[blockIdx.x] = r;
+  }
 }
 
 static inline long long nchunks(long long n) { return (n + SUM_CHUNK - 1) / SUM_CHUNK; }
@@ -164,7 +133,6 @@ size_t sum_ws_floats(size_t n) {
 
 int sum_launch(const float* x, size_t n, int squares, float* out, float* ws, cudaStream_t st) {
   if (n == 0) { cudaMemsetAsync(out, 0, sizeof(float), st); return DET_OK; }
-  if (n == 1) { k_flush1<<<DET_L(1), 1, 0, st>>>(x, out, squares); return DET_OK; }
   const float* src = x;
   long long cur = (long long)n;
   bool sq = squares != 0;
@@ -183,8 +151,35 @@ int sum_launch(const float* x, size_t n, int squares, float* out, float* ws, cud
   return DET_OK;
 }
 
-__global__ void k_norm_finish(const float* total, float max_norm, float* norm_out, float* coef_out, int* status) {
-  float nrm = fsqrt(total[0]);
+// det_sum(x[0..n)), n <= SUM_CHUNK, times gs (the last levels of a sum and the scaling that follows it, in one launch)
+__global__ void __launch_bounds__(256) k_sum_scaled(const float* __restrict__ x, int n, float gs, float* __restrict__ out) {
+  __shared__ float wsum[8];
+  const float r = chunk_sum<false>(x, 0, n, wsum);
+  if (threadIdx.x == 0) out[0] = fmul(gs, r);
+}
+// Reduces x[0..n) until at most SUM_CHUNK nodes are left; x and n become what is left, ws what is free of the scratch.
+void sum_to_chunk(const float*& x, size_t& n, float*& ws, cudaStream_t st) {
+  while (n > (size_t)SUM_CHUNK) {
+    const size_t c = (size_t)nchunks((long long)n);
+    k_sum_chunk<false><<<DET_L((unsigned)c), 256, 0, st>>>(x, (long long)n, ws);
+    x = ws;
+    ws += align_up(c, 64);
+    n = c;
+  }
+}
+int sum_scaled_launch(const float* x, size_t n, float gs, float* out, float* ws, cudaStream_t st) {
+  sum_to_chunk(x, n, ws, st);
+  k_sum_scaled<<<DET_L(1), 256, 0, st>>>(x, (int)n, gs, out);
+  return DET_OK;
+}
+
+// the tree over the per-tensor sums (n <= SUM_CHUNK), the norm and the clip coefficient
+__global__ void __launch_bounds__(256) k_norm_finish(const float* __restrict__ per, int n, float max_norm, float* norm_out,
+                                                     float* coef_out, int* status) {
+  __shared__ float wsum[8];
+  const float total = n ? chunk_sum<false>(per, 0, n, wsum) : 0.0f;
+  if (threadIdx.x) return;
+  float nrm = fsqrt(total);
   norm_out[0] = nrm;
   float coef = 1.0f;
   if (max_norm > 0.0f) coef = fminf(1.0f, fdiv(max_norm, fadd(nrm, 1e-6f)));
@@ -267,13 +262,24 @@ extern "C" int det_sum(const float* x, size_t n, int squares, float* out, void* 
   return rc;
 }
 
+// Workspace: the per-tensor sums, then the chunk sums of one group of tensors (all levels), then the levels above
+// SUM_CHUNK tensors.
 extern "C" size_t det_grad_norm_ws_bytes(const size_t* n_elems, int ntensors) {
-  size_t mx = 0;
-  for (int t = 0; t < ntensors; ++t) mx = n_elems[t] > mx ? n_elems[t] : mx;
-  return (align_up((size_t)(ntensors > 0 ? ntensors : 1), 64) + 64 + sum_ws_floats(mx) +
-          sum_ws_floats((size_t)(ntensors > 0 ? ntensors : 1))) * sizeof(float);
+  size_t most = 0;
+  for (int t0 = 0; t0 < ntensors; t0 += SUM_JOBS) {
+    size_t need = 0;
+    for (int t = t0; t < ntensors && t < t0 + SUM_JOBS; ++t) {
+      long long c = (long long)n_elems[t];
+      do { c = nchunks(c); need += (size_t)c + 4; } while (c > 1);
+    }
+    most = need + 4 * 64 > most ? need + 4 * 64 : most;                 // every level starts at a multiple of 64
+  }
+  const size_t nt = (size_t)(ntensors > 0 ? ntensors : 1);
+  return (align_up(nt, 64) + 64 + align_up(most, 64) + sum_ws_floats(nt)) * sizeof(float);
 }
 
+// The sums of squares of all tensors run level by level together: a launch of its own per tensor and level (138 for a
+// model of 87 tensors, 4 us each and one after the other) cost more than the 187 M values take to read.
 extern "C" int det_grad_norm(const float* const* g_ptrs, const size_t* n_elems, int ntensors, float max_norm,
                              float* norm_out, float* coef_out, void* ws, size_t ws_bytes, void* stream,
                              int* status_dev) {
@@ -285,9 +291,47 @@ extern "C" int det_grad_norm(const float* const* g_ptrs, const size_t* n_elems, 
   float* per = (float*)ws;
   float* total = per + align_up((size_t)(ntensors > 0 ? ntensors : 1), 64);
   float* scratch = total + 64;
-  for (int t = 0; t < ntensors; ++t) sum_launch(g_ptrs[t], n_elems[t], 1, per + t, scratch, st);
-  sum_launch(per, (size_t)ntensors, 0, total, scratch, st);
-  k_norm_finish<<<DET_L(1), 1, 0, st>>>(total, max_norm, norm_out, coef_out, status_dev);
+  bool empty = false;
+  for (int t = 0; t < ntensors; ++t) empty |= n_elems[t] == 0;
+  if (empty) cudaMemsetAsync(per, 0, (size_t)ntensors * sizeof(float), st);   // a tensor without elements has the sum +0
+  for (int t0 = 0; t0 < ntensors; t0 += SUM_JOBS) {
+    SumJobs jobs;
+    jobs.n = 0;
+    for (int t = t0; t < ntensors && t < t0 + SUM_JOBS; ++t) {
+      if (!n_elems[t]) continue;
+      jobs.x[jobs.n] = g_ptrs[t];
+      jobs.len[jobs.n] = (long long)n_elems[t];
+      jobs.who[jobs.n++] = t;
+    }
+    float* out = scratch;
+    bool sq = true;
+    while (jobs.n) {
+      long long c = 0;
+      for (int j = 0; j < jobs.n; ++j) {
+        if (jobs.len[j] > SUM_CHUNK) c = (c + 3) / 4 * 4;
+        jobs.first[j] = (uint32_t)c;
+        c += nchunks(jobs.len[j]);
+      }
+      if (c > 0x7fffffffll) return DET_ERR_SHAPE;
+      jobs.first[jobs.n] = (uint32_t)c;
+      if (sq) k_sum_jobs<true><<<DET_L((unsigned)c), 256, 0, st>>>(jobs, out, per);
+      else k_sum_jobs<false><<<DET_L((unsigned)c), 256, 0, st>>>(jobs, out, per);
+      int m = 0;
+      for (int j = 0; j < jobs.n; ++j)
+        if (jobs.len[j] > SUM_CHUNK) { jobs.x[m] = out + jobs.first[j]; jobs.len[m] = nchunks(jobs.len[j]); jobs.who[m] = jobs.who[j]; ++m; }
+      jobs.n = m;
+      out += align_up((size_t)c, 64);
+      sq = false;
+    }
+  }
+  int n = ntensors;
+  const float* src = per;
+  if (n > SUM_CHUNK) {
+    sum_launch(per, (size_t)n, 0, total, scratch, st);
+    src = total;
+    n = 1;
+  }
+  k_norm_finish<<<DET_L(1), 256, 0, st>>>(src, n, max_norm, norm_out, coef_out, status_dev);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }

@@ -151,7 +151,8 @@ class Replay:
         wsb = max(det.det_attn_bwd_fixq_ws_bytes(B, H, S, Hkv) if cfg.dq_fixed else det.det_attn_bwd_ws_bytes(B, H, S, Hkv),
                   det.det_xent_ws_bytes(T, V), det.det_rmsnorm_bwd_ws_bytes(T, D),
                   det.det_lsq_weight_scale_ws_bytes(2 * Fh, D), det.det_lsq_act_scale_init_ws_bytes(T * max(Fh, D)),
-                  *[det.det_tensor_hash_batch_ws_bytes([t for _, t in self._hash_jobs(per)]) for per in (True, False)],
+                  *[det.det_tensor_hash_batch_ws_bytes(own + [4 * g] * 3) for own in                      # per tensor, or the flat buffers
+                    ([_numel(shape) * (2 if kind == "bf16" else 4) for _, shape, kind in self.specs], [2 * p, 16 * L])],
                   det.det_sum_ws_bytes(g), 1 << 20,
                   (max(det.det_lmhead_fwd_v2_ws_bytes(T, V, D), det.det_lmhead_bwd_v2_ws_bytes(T, V, D)) if cfg.arith == 2 else 0),
                   *[det.det_linear_bwd_ws_bytes(T, N, K) for (N, K) in ((QW, D), (D, D), (2 * Fh, D), (D, Fh))])
@@ -403,12 +404,15 @@ class Replay:
         cfg = self.cfg
         views = [self.g(self.gout, name) for name, _, _ in self.specs]
         det.det_grad_norm(views, cfg.clip, self.norm, self.coef, self.ws, self.status)
-        det.det_scale_inplace(self.gout, self.n_grad, self.coef)
+        descs, kinds = [], []
         for name, shape, kind in self.specs:
             decay = cfg.wd if (name == "lm_head" or name.split(".")[-1] in LINEARS) else 0.0
-            desc = det.det_adamw_desc(cfg.lr, cfg.betas[0], cfg.betas[1], cfg.eps, decay, cfg.step)
-            det.det_adamw_step(desc, det.DET_BF16 if kind == "bf16" else det.DET_F32, self.p(name), self.g(self.gout, name),
-                               self.g(self.m, name), self.g(self.v, name), _numel(shape))
+            descs.append(det.det_adamw_desc(cfg.lr, cfg.betas[0], cfg.betas[1], cfg.eps, decay, cfg.step))
+            kinds.append(det.DET_BF16 if kind == "bf16" else det.DET_F32)
+        names = [name for name, _, _ in self.specs]
+        # the clip coefficient is applied to the gradient in the same pass (every element of gout belongs to one tensor)
+        det.det_adamw_batch(descs, kinds, [self.p(x) for x in names], views, [self.g(self.m, x) for x in names],
+                            [self.g(self.v, x) for x in names], self.coef)
 
     def _hash_jobs(self, per_tensor):
         jobs = [(name, self.p(name)) for name, _, _ in self.specs] if per_tensor else [("params_bf16", self.pbf), ("steps_f32", self.sx)]

@@ -104,3 +104,47 @@ def test_two_lane_exponential(det):
     n = np.isnan(x)
     assert_same_bits(host(got)[~n], host(want)[~n], "exp")
     assert np.isnan(host(got)[n]).all()
+
+
+# global norm over many tensors in common launches: more tensors than one launch takes, empty and one-element ones, lengths
+# around a chunk of 16384 and around the second level (16384 chunks would be 2^28 elements: 40 chunks stand for it)
+@pytest.mark.parametrize("sizes", [[0], [1], [16384, 16385, 0, 1, 300, 16383, 655361, 8, 65536], [(977 * i) % 40000 for i in range(520)]])
+def test_grad_norm_many_tensors(det, sizes):
+    import torch
+    g = [synth.normal_f32((n,), 1e-3, seed=len(sizes), tid=i) if n else np.zeros(0, F) for i, n in enumerate(sizes)]
+    if sizes == [1]:
+        g = [np.array([1e-40], F)]              # a lone subnormal is flushed
+    d = [dev(x) for x in g]
+    norm, coef, status = empty((1,), F), empty((1,), F), torch.zeros(1, dtype=torch.int32, device="cuda")
+    det.det_grad_norm(d, 0.5, norm, coef, ws(det.det_grad_norm_ws_bytes(d)), status)
+    _sync()
+    n_o, c_o = oracle.grad_norm(g, 0.5)
+    assert_same_bits(host(norm), np.array([n_o], F), "norm")
+    assert_same_bits(host(coef), np.array([c_o], F), "coef")
+    assert int(status.item()) == 0
+
+
+# AdamW of many tensors in one launch with the clip coefficient applied on the way: both parameter types, lengths off the
+# 4- and 1024-element grid, empty tensors, more tensors than one launch takes, different decay per tensor
+@pytest.mark.parametrize("sizes,clip", [([1, 3, 4, 5, 1023, 1024, 1025, 0, 4100], True), ([2048, 7], False), ([(37 * i) % 600 for i in range(300)], True)])
+def test_adamw_many_tensors(det, sizes, clip):
+    rng = np.random.default_rng(len(sizes))
+    coef = F(0.3125 + 1e-3)
+    kinds = [int(i % 3 != 2) for i in range(len(sizes))]
+    wd = [0.1 if i % 2 else 0.0 for i in range(len(sizes))]
+    p = [synth.to_bf16(rng.standard_normal(n, dtype=F)) if k else rng.standard_normal(n, dtype=F) for n, k in zip(sizes, kinds)]
+    g, m = [[rng.standard_normal(n, dtype=F) * F(s) for n in sizes] for s in (1e-2, 1e-3)]
+    v = [np.abs(rng.standard_normal(n, dtype=F)) * F(1e-5) for n in sizes]
+    dp, dg, dm, dv = [[dev(x) for x in t] for t in (p, g, m, v)]
+    descs = [det.det_adamw_desc(3e-4, 0.9, 0.95, 1e-8, w, 3) for w in wd]
+    det.det_adamw_batch(descs, kinds, dp, dg, dm, dv, dev(np.array([coef], F)) if clip else None)
+    _sync()
+    for i, n in enumerate(sizes):
+        if not n:
+            continue
+        go = oracle.scale(g[i], coef) if clip else g[i]
+        po, mo, vo = oracle.adamw(p[i], go, m[i], v[i], 3e-4, 0.9, 0.95, 1e-8, wd[i], 3)
+        assert_same_bits(host(dg[i]), go, "g %d" % i)
+        assert_same_bits(host(dp[i], p[i].dtype), po, "p %d" % i)
+        assert_same_bits(host(dm[i]), mo, "m %d" % i)
+        assert_same_bits(host(dv[i]), vo, "v %d" % i)
