@@ -8,20 +8,10 @@
 // Backward: P = exp(S*scale - L) recomputed; every one of the five contractions (S, dP, dV, dK, dQ) is a batched
 // ordered contraction with one sequential accumulator per output (ogemm_core.cuh); bf16(P) and bf16(dS) go through
 // global scratch, so nothing is accumulated with atomics.
-#include "ogemm_core.cuh"
+#include "attn_core.cuh"
 
 namespace det {
 
-#define ATT_SCALE 0x1.6a09e6p-4f
-constexpr int DH = 128;
-
-__device__ __forceinline__ void unpack8a(const uint4& u, float v[8]) {
-  v[0] = bflo(u.x); v[1] = bfhi(u.x); v[2] = bflo(u.y); v[3] = bfhi(u.y);
-  v[4] = bflo(u.z); v[5] = bfhi(u.z); v[6] = bflo(u.w); v[7] = bfhi(u.w);
-}
-
-// conservative test for 0 < |v| < 2^-63 (also true for subnormal v, which only selects the slower exact path)
-__device__ __forceinline__ bool tiny1(float v) { return (__float_as_uint(v) * 2u - 1u) < 0x3fffffffu; }
 // ---------------------------------------------------------------------------------------------
 // forward, warp-specialised; CTA = FQ queries of one (batch, head).
 //
@@ -42,12 +32,6 @@ __device__ __forceinline__ bool tiny1(float v) { return (__float_as_uint(v) * 2u
 // skips a tile that holds none of its keys (its statistics stay untouched: alpha = 1, all weights 0).
 // Hkv key/value heads serve H query heads (head h reads key/value head h / (H/Hkv)).
 // ---------------------------------------------------------------------------------------------
-constexpr int FK = 128;
-constexpr int AF_RW = 8;                      // query rows per consumer warp
-constexpr int AF_PROD = 128;
-// A slab row: the first and the second four columns of a lane lie 80 apart (4t and 80 + 4t), so that a warp's loads of
-// either half are 256 adjacent bytes and the key-wise stores of K stay free of bank conflicts.
-constexpr int AF_HI = 80, AF_BP = 148;
 // Rows per CTA, ring slots, slabs in flight in the producers' registers, CTAs per SM, registers per consumer and producer thread after the hand-over.
 // A CTA of 128 rows has the best rate (25.1 us per row block and key block on a full GPU, against 13.2 us for 64 rows and
 // 7.5 us for 32), but its chain of key blocks is the longest: alone on its SM 25.1, 17 and 13 us per key block.
@@ -63,48 +47,6 @@ typedef AfTile<128, 8, 4, 1, 104, 64> AfTall;
 typedef AfTile<64, 4, 2, 2, 96, 48> AfHalf;
 typedef AfTile<32, 4, 3, 3, 104, 56> AfShort;
 
-// one 16-deep slab: (row i of the lane, column c) += A[k][row] * B[k][c].  The lane's four rows of step k are chunk
-// `chunk` ^ (PSWZ ? swizzle of the key : 0) of row k of A.
-template <bool FUSED, bool PSWZ>
-__device__ __forceinline__ void mac_4x8(const float* __restrict__ ap, int a_ld, int chunk, int key0,
-                                        const float (*Bs)[AF_BP], int tx, float2 (&acc)[4][4]) {
-#pragma unroll
-  for (int k = 0; k < OK; ++k) {
-    const int sw = PSWZ ? (((key0 + k) >> 3) & 3) << 1 : 0;
-    const float4 a4 = *reinterpret_cast<const float4*>(ap + (size_t)k * a_ld + ((chunk ^ sw) << 2));
-    const float4 b0 = *reinterpret_cast<const float4*>(&Bs[k][4 * tx]), b1 = *reinterpret_cast<const float4*>(&Bs[k][AF_HI + 4 * tx]);
-    const float a[4] = {a4.x, a4.y, a4.z, a4.w};
-    const float2 b[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y), make_float2(b1.z, b1.w)};
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (FUSED) {
-          acc[i][j] = __ffma2_rn(make_float2(a[i], a[i]), b[j], acc[i][j]);
-        } else {  // scalar on purpose: a packed multiply + add pair would be contracted by ptxas
-          acc[i][j].x = fadd(acc[i][j].x, fmul(a[i], b[j].x));
-          acc[i][j].y = fadd(acc[i][j].y, fmul(a[i], b[j].y));
-        }
-      }
-  }
-}
-// Reduction of a lane's four rows over the sixteen lanes that hold them, with partners 2, 4, 8, 16 lanes apart in that
-// order, which for sums is the adjacent pairwise tree over the lanes.  The first two stages halve the rows a lane carries (it
-// sends its partner the half the partner keeps): 2 + 1 + 1 + 1 shuffles, and lane L ends with the result of row
-// ROW_OF_LANE(L) of the warp; both operand orders of an addition or a maximum give the same bits.
-#define ROW_OF_LANE(L) ((((L) & 1) << 2) | ((L) & 2) | (((L) & 4) >> 2))
-#define LANE_OF_ROW(i) ((lane & 1) | ((i) & 2) | (((i) & 1) << 2))   /* a lane that holds row i of this lane's four */
-template <bool SUM>
-__device__ __forceinline__ float rows_reduce(const float (&x)[4], int lane) {
-  auto op = [](float a, float b) { return SUM ? fadd(a, b) : fmaxf(a, b); };
-  const bool b1 = lane & 2, b2 = lane & 4;
-  float c[2];
-#pragma unroll
-  for (int j = 0; j < 2; ++j) c[j] = op(b1 ? x[2 + j] : x[j], __shfl_xor_sync(0xffffffffu, b1 ? x[j] : x[2 + j], 2));
-  float d = op(b2 ? c[1] : c[0], __shfl_xor_sync(0xffffffffu, b2 ? c[0] : c[1], 4));
-  d = op(d, __shfl_xor_sync(0xffffffffu, d, 8));
-  return op(d, __shfl_xor_sync(0xffffffffu, d, 16));
-}
 template <class T, bool WIN>
 __global__ void __launch_bounds__(T::THREADS, T::CPS)
     k_attn_fwd(const uint16_t* __restrict__ q, const uint16_t* __restrict__ k, const uint16_t* __restrict__ v, int ld,
@@ -273,69 +215,19 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
       release();
     }
     if (!ok) break;
-    // ---- online softmax of the warp's 8 rows ----
-    float rm[4];
-    const int key = j0 + 8 * tx, row = q0 + lrow;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float mt = __int_as_float(0xff800000);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        acc[i][j] = mul2(acc[i][j], same2(ATT_SCALE));
-        if ((!diag || key + 2 * j <= row + i) && (!edge || key + 2 * j > row + i - W)) mt = fmaxf(mt, acc[i][j].x);
-        if ((!diag || key + 2 * j + 1 <= row + i) && (!edge || key + 2 * j + 1 > row + i - W)) mt = fmaxf(mt, acc[i][j].y);
-      }
-      rm[i] = mt;
-    }
-    // the lane that owns row r (see rows_reduce) updates its running maximum (a row sees at least one key of a block it
-    // visits, so the maximum is a number) and the rescale factor of what it has accumulated
-    const float m_new = fmaxf(m_mine, rows_reduce<false>(rm, lane));
-    alpha_mine = det_exp_le0(fsub(m_mine, m_new));
-    if (edge && j0 + FK - 1 <= q0 + wrow + ROW_OF_LANE(lane) - W) alpha_mine = 1.0f;
-    m_mine = m_new;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) rm[i] = __shfl_sync(0xffffffffu, m_new, LANE_OF_ROW(i));
-    bool tp = false;
-    // 32 independent exponentials in one straight-line block (no branch, no shuffle in between), so that their
-    // dependent chains interleave; invisible pairs are zeroed afterwards (their arguments may be anything)
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = det_exp_le0_2(add2(acc[i][j], same2(-rm[i]), one), one);
-    if (diag) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (key + 2 * j > row + i) acc[i][j].x = 0.0f;
-          if (key + 2 * j + 1 > row + i) acc[i][j].y = 0.0f;
-        }
-    }
-    if (edge) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (key + 2 * j <= row + i - W) acc[i][j].x = 0.0f;
-          if (key + 2 * j + 1 <= row + i - W) acc[i][j].y = 0.0f;
-        }
-    }
+    // ---- online softmax of the warp's 8 rows; the row sums take the weights before their rounding to bf16 ----
+    softmax_block(acc, j0 + 8 * tx, q0 + lrow, q0 + wrow + ROW_OF_LANE(lane), j0 + FK - 1, W, diag, edge, lane, m_mine, l_mine,
+                  alpha_mine, one);
     uint32_t tw = 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      // the lane's eight adjacent slots of the block's row sum
-      rm[i] = fadd(fadd(fadd(acc[i][0].x, acc[i][0].y), fadd(acc[i][1].x, acc[i][1].y)),
-                   fadd(fadd(acc[i][2].x, acc[i][2].y), fadd(acc[i][3].x, acc[i][3].y)));
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const uint32_t w = pack_bf2(acc[i][j].x, acc[i][j].y);
         word_tiny(w, tw);
         acc[i][j] = make_float2(word_lo(w), word_hi(w));
       }
-    }
-    tp = words_tiny(tw);
-    // the rest of the adjacent tree over the block's 128 slots: lanes 2, 4, 8, 16 apart
-    l_mine = fadd(fmul(l_mine, alpha_mine), rows_reduce<true>(rm, lane));
+    const bool tp = words_tiny(tw);
     // P~ of the lane's rows: key rows 8 tx + c, one chunk of four rows each
     __syncwarp();                                    // the previous block's P.V loads are done
     float* pchunk = Ps + (size_t)(8 * tx) * FQ + (((lrow >> 2) ^ ((tx & 3) << 1)) << 2);

@@ -7,93 +7,71 @@
 // and the rescale o = o * alpha + u stay in ordered f32 exactly as in the full-precision kernel (attn.cu); lse is the
 // same as there.
 //
-// CTA = 128 queries of one (batch, head), 512 threads, one CTA per SM.  Logits: 4 x 8 register tiles on the FP32 pipe
-// as in attn.cu.  The quantised weights (A operand, [query][key]) and the quantised, transposed values (B operand,
-// [dim][key]) are written by the threads into shared memory in the 128-byte-swizzled K-major layout the MMA expects;
-// one thread issues four tcgen05.mma.kind::i8 (M = N = 128, K = 32 each) into a 128-column TMEM accumulator and
-// commits to an mbarrier; every warp then loads its 32 lanes x 32 columns of the accumulator.  In that phase a thread
-// owns one query row and 32 output dimensions.  The wait on the mbarrier is bounded: on expiry the kernel raises
-// DET_DEV_TIMEOUT in *status, skips the remaining tiles, frees its TMEM and returns.
-#include "tc05.cuh"
-#include "internal.h"
+// CTA = 128 queries of one (batch, head), one CTA per SM, warp-specialised like the full-precision kernel (attn.cu):
+//   warps 0-15   consumers: 8 whole query rows each; logits on the FP32 pipe from the slab ring, softmax, quantised weights
+//                (A operand, [query][key]) into shared memory in the 128-byte-swizzled K-major layout the MMA expects
+//   warps 16-19  producers: the key block as eight 16-deep slabs into the ring, then the block absmax of V and the
+//                quantised, transposed values (B operand, [dim][key]), double-buffered; between the two one thread issues
+//                four tcgen05.mma.kind::i8 (M = N = 128, K = 32 each) of the block before into a 128-column TMEM accumulator
+//                once both its operands are there, and commits to an mbarrier
+// A consumer warp collects the product of block t after its logits of block t + 1, so the tensor-core product, the other warps'
+// softmax and the quantisation of V run behind the multiply loop (with block-wide phases, each waiting for the one before,
+// forward and backward of 16 heads x 4096 at window 512 took 1.69 ms, 1.55 now).  In that step a thread owns one query row and 32 output
+// dimensions.  Every wait on an mbarrier is bounded: on expiry the kernel raises DET_DEV_TIMEOUT in *status, all roles skip what
+// is left, and the kernel frees its TMEM and returns.
+#include "attn_core.cuh"
 
 namespace det {
 
-#define ATT_SCALE 0x1.6a09e6p-4f
-constexpr int PD = 128;                 // head dimension
-constexpr int PQ = 128, PK = 128, PTH = 512;
-constexpr int PLQ = PQ + 4;
-// shared memory: Q f32 [dim][query], K f32 [dim][key], then (1024-byte aligned) q_p int8 [query][key], q_v int8 [dim][key]
-constexpr size_t PV8_SMEM = (size_t)(2 * PD * PLQ) * sizeof(float) + 1024 + 2 * PQ * PK;
-
-__device__ __forceinline__ void unpack8p(const uint4& u, float v[8]) {
-  v[0] = bflo(u.x); v[1] = bfhi(u.x); v[2] = bflo(u.y); v[3] = bfhi(u.y);
-  v[4] = bflo(u.z); v[5] = bfhi(u.z); v[6] = bflo(u.w); v[7] = bfhi(u.w);
-}
-__device__ __forceinline__ bool tiny1p(float v) { return (__float_as_uint(v) * 2u - 1u) < 0x3fffffffu; }
+constexpr int PQ = 128, PK = 128, PLQ = PQ + 4, PV_SLOTS = 8;
+constexpr int PV_CONS = 512, PV_PROD = 128, PV_THREADS = PV_CONS + PV_PROD;
+// shared memory: Q f32 [dim][query], the slab ring, then (1024-byte aligned) q_p int8 [query][key], q_v int8 [2][dim][key]
+constexpr size_t PV8_SMEM = (size_t)(DH * PLQ + PV_SLOTS * OK * AF_BP) * sizeof(float) + 1024 + 3 * PQ * PK;
+// setmaxnreg: 104 registers for consumers, 64 for producers
+static_assert(PV_CONS * 104 + PV_PROD * 64 <= (65536 / PV_THREADS / 8 * 8) * PV_THREADS, "register hand-over exceeds the block's allocation");
 
 // byte offset of element (row, col) of a 128 x 128 int8 K-major tile with 128-byte swizzle (16-byte chunks of a row
 // are permuted by the row index modulo 8)
 __device__ __forceinline__ int swz(int row, int col) { return row * 128 + ((((col >> 4) ^ (row & 7))) << 4) + (col & 15); }
 
-template <bool FUSED>
-__device__ __forceinline__ void mac_4x8p(const float (*As)[PLQ], const float (*Bs)[PLQ], int ty, int tx, float2 (&acc)[4][4]) {
-#pragma unroll 8
-  for (int k = 0; k < PD; ++k) {
-    const float4 a0 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-    const float4 b0 = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-    const float4 b1 = *reinterpret_cast<const float4*>(&Bs[k][64 + tx * 4]);
-    const float av[4] = {a0.x, a0.y, a0.z, a0.w};
-    const float2 b[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y), make_float2(b1.z, b1.w)};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 a = make_float2(av[i], av[i]);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (FUSED) {
-          acc[i][j] = __ffma2_rn(a, b[j], acc[i][j]);
-        } else {  // scalar on purpose: a packed multiply + add pair would be contracted by ptxas
-          acc[i][j].x = fadd(acc[i][j].x, fmul(av[i], b[j].x));
-          acc[i][j].y = fadd(acc[i][j].y, fmul(av[i], b[j].y));
-        }
-      }
-    }
-  }
-}
-
-__global__ void __launch_bounds__(PTH, 1)
+__global__ void __launch_bounds__(PV_THREADS, 1)
     k_attn_fwd_pv8(const uint16_t* __restrict__ q, const uint16_t* __restrict__ k, const uint16_t* __restrict__ v, int ld, int H,
                    int Hkv, int S, int W, uint16_t* __restrict__ out, int ld_out, float* __restrict__ lse, int* status) {
   extern __shared__ __align__(16) unsigned char psm8[];
   float(*Qs)[PLQ] = reinterpret_cast<float(*)[PLQ]>(psm8);
-  float(*Ks)[PLQ] = reinterpret_cast<float(*)[PLQ]>(psm8 + (size_t)PD * PLQ * sizeof(float));
-  uint8_t* ops = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(psm8 + (size_t)2 * PD * PLQ * sizeof(float)) + 1023) &
-                                            ~(uintptr_t)1023);
+  float(*Ring)[OK][AF_BP] = reinterpret_cast<float(*)[OK][AF_BP]>(psm8 + (size_t)DH * PLQ * sizeof(float));
+  uint8_t* ops = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(psm8 + (size_t)(DH * PLQ + PV_SLOTS * OK * AF_BP) * sizeof(float)) + 1023) & ~(uintptr_t)1023);
   int8_t* Pq = reinterpret_cast<int8_t*>(ops);              // A operand: [query][key]
-  int8_t* Vq = reinterpret_cast<int8_t*>(ops + PQ * PK);    // B operand: [dim][key]
-  __shared__ float alpha_s[PQ], l_s[PQ], m_s[PQ];
-  __shared__ uint32_t vmax_s, tmem_base_s;
-  __shared__ __align__(8) uint64_t bar;
-  __shared__ int abort_s;
+  int8_t* Vq = reinterpret_cast<int8_t*>(ops + PQ * PK);    // B operand: two buffers [dim][key]
+  __shared__ float alpha_s[2][PQ], l_s[PQ], cs_s[4], vmax_s[2][4];
+  __shared__ __align__(16) int tiny_s[PV_SLOTS][4];
+  __shared__ int tiny_q_s, abort_s;
+  __shared__ uint32_t tmem_base_s;
+  __shared__ __align__(8) uint64_t bar_full[PV_SLOTS], bar_empty[PV_SLOTS], bar_p, bar_v[2], bar_mma;
   volatile int* abort_flag = &abort_s;
 
   const int qb = gridDim.y - 1 - blockIdx.y;  // longest rows first
-  const int h = blockIdx.x % H, b = blockIdx.x / H;
+  const int h = blockIdx.x % H, b = blockIdx.x / H, hk = h / (H / Hkv);
   const int q0 = qb * PQ;
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const size_t row0 = (size_t)b * S;
-  const int hk = h / (H / Hkv);
-  const uint16_t* qp = q + row0 * ld + (size_t)h * PD;
-  const uint16_t* kp = k + row0 * ld + (size_t)hk * PD;
-  const uint16_t* vp = v + row0 * ld + (size_t)hk * PD;
+  const uint16_t* qp = q + row0 * ld + (size_t)h * DH;
+  const uint16_t* kp = k + row0 * ld + (size_t)hk * DH;
+  const uint16_t* vp = v + row0 * ld + (size_t)hk * DH;
+  const int jt0 = (W > 0 && q0 > W) ? (q0 - W) / PK : 0, nt = q0 / PK + 1 - jt0;     // key blocks of this CTA
 
   if (tid == 0) {
-    mbar_init(&bar, 1);
+    for (int s = 0; s < PV_SLOTS; ++s) { mbar_init(&bar_full[s], 4); mbar_init(&bar_empty[s], PV_CONS / 32); }
+    mbar_init(&bar_p, PV_CONS / 32);
+    mbar_init(&bar_v[0], 4);
+    mbar_init(&bar_v[1], 4);
+    mbar_init(&bar_mma, 1);
     abort_s = 0;
-    vmax_s = 0;
+    tiny_q_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) {
+  if (warp == 16) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(128u)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -102,189 +80,239 @@ __global__ void __launch_bounds__(PTH, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
-  // accumulator phase: this thread owns query row orow and the 32 output dimensions starting at ocol
-  const int orow = (warp & 3) * 32 + lane, ocol = (warp >> 2) * 32;
-  const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)ocol;
-
-  uint4 rw[4];
-  auto fetch = [&](const uint16_t* base, int j0, bool key_major) {
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int idx = tid + PTH * it;
-      const int key = key_major ? (idx & 127) : (idx >> 4), ch = key_major ? (idx >> 7) : (idx & 15);
-      rw[it] = (j0 + key < S) ? __ldg(reinterpret_cast<const uint4*>(base + (size_t)(j0 + key) * ld + ch * 8))
-                              : make_uint4(0u, 0u, 0u, 0u);
-    }
-  };
-  const int jt0 = (W > 0 && q0 > W) ? (q0 - W) / PK : 0;
-  fetch(kp, jt0 * PK, true);
-  bool tq = false;
-#pragma unroll
-  for (int it = 0; it < 4; ++it) {
-    const int idx = tid + PTH * it, r = idx & 127, ch = idx >> 7;
-    float t[8];
-    if (q0 + r < S) unpack8p(__ldg(reinterpret_cast<const uint4*>(qp + (size_t)(q0 + r) * ld + ch * 8)), t);
-    else {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) t[e] = 0.0f;
-    }
-#pragma unroll
-    for (int e = 0; e < 8; ++e) { tq |= tiny1p(t[e]); Qs[ch * 8 + e][r] = t[e]; }
-  }
-  const int tiny_q = __syncthreads_or(tq);
-  float m[4], l[4], o[32];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) { m[i] = __int_as_float(0xff800000); l[i] = 0.0f; }
-#pragma unroll
-  for (int c = 0; c < 32; ++c) o[c] = 0.0f;
-  const int ntiles = q0 / PK + 1;
-  constexpr uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(PD >> 3) << 17) | ((uint32_t)(PQ >> 4) << 24);
-  uint32_t phase = 0;
-  bool ok = true;
-  for (int jt = jt0; jt < ntiles; ++jt) {
-    const int j0 = jt * PK;
-    // ---- K tile (fetched during the previous tile), transposed, f32 ----
-    bool tk = false;
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int idx = tid + PTH * it, key = idx & 127, ch = idx >> 7;
+  {  // q^T of the query block, staged once by everybody
+    bool tq = false;
+    for (int idx = tid; idx < PQ * 16; idx += PV_THREADS) {
+      const int r = idx % PQ, ch = idx / PQ;
       float t[8];
-      unpack8p(rw[it], t);
+      if (q0 + r < S) unpack8a(__ldg(reinterpret_cast<const uint4*>(qp + (size_t)(q0 + r) * ld + ch * 8)), t);
+      else {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) { tk |= tiny1p(t[e]); Ks[ch * 8 + e][key] = t[e]; }
-    }
-    fetch(vp, j0, false);   // V words travel while the logits are computed
-    const int tiny_k = __syncthreads_or(tk);
-    float2 s[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) s[i][e] = make_float2(0.0f, 0.0f);
-    if (tiny_q || tiny_k) mac_4x8p<false>(Qs, Ks, ty, tx, s);
-    else mac_4x8p<true>(Qs, Ks, ty, tx, s);
-    // ---- block absmax of V (all 128 keys x 128 dims of the tile) ----
-    float vm = 0.0f;
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      float t[8];
-      unpack8p(rw[it], t);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) vm = fmaxf(vm, fabsf(t[e]));
-    }
-#pragma unroll
-    for (int w = 16; w; w >>= 1) vm = fmaxf(vm, __shfl_xor_sync(0xffffffffu, vm, w));
-    if (lane == 0 && vm > 0.0f) atomicMax(&vmax_s, __float_as_uint(vm));
-    // ---- online softmax statistics per row; quantised weights to the A operand ----
-    const bool diag = (jt == ntiles - 1);
-    const bool edge = W > 0 && j0 <= q0 + PQ - 1 - W;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int rl = ty * 4 + i;
-      const int row = q0 + rl;
-      const bool rowvalid = !(edge && j0 + PK - 1 <= row - W);
-      float sv[8] = {s[i][0].x, s[i][0].y, s[i][1].x, s[i][1].y, s[i][2].x, s[i][2].y, s[i][3].x, s[i][3].y};
-      float mt = m[i];
-      bool valid[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int key = j0 + ((e < 4) ? (tx * 4 + e) : (64 + tx * 4 + e - 4));
-        valid[e] = (!diag || key <= row) && (!edge || key > row - W);
-        sv[e] = fmul(sv[e], ATT_SCALE);
-        if (valid[e]) mt = fmaxf(mt, sv[e]);
+        for (int x = 0; x < 8; ++x) t[x] = 0.0f;
       }
 #pragma unroll
-      for (int w = 1; w < 16; w <<= 1) mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, w));
-      const float al0 = det_exp_le0(fsub(m[i], mt));
-      const float al = rowvalid ? al0 : 1.0f;
-      float p[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) p[e] = det_exp_le0(fsub(sv[e], mt));   // branch-free, so the eight chains interleave
-#pragma unroll
-      for (int e = 0; e < 8; ++e) p[e] = valid[e] ? p[e] : 0.0f;
-      uint32_t w0 = 0, w1 = 0;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        w0 |= ((uint32_t)(int)rintf(fmul(p[e], 127.0f))) << (8 * e);
-        w1 |= ((uint32_t)(int)rintf(fmul(p[4 + e], 127.0f))) << (8 * e);
-      }
-      *reinterpret_cast<uint32_t*>(Pq + swz(rl, tx * 4)) = w0;
-      *reinterpret_cast<uint32_t*>(Pq + swz(rl, 64 + tx * 4)) = w1;
-      float h0 = fadd(fadd(p[0], p[1]), fadd(p[2], p[3]));
-      float h1 = fadd(fadd(p[4], p[5]), fadd(p[6], p[7]));
-#pragma unroll
-      for (int w = 1; w < 16; w <<= 1) {
-        h0 = fadd(h0, __shfl_xor_sync(0xffffffffu, h0, w));
-        h1 = fadd(h1, __shfl_xor_sync(0xffffffffu, h1, w));
-      }
-      l[i] = fadd(fmul(l[i], al), fadd(h0, h1));
-      m[i] = mt;
-      if (tx == 0) alpha_s[rl] = al;
+      for (int x = 0; x < 8; ++x) { tq |= tiny1(t[x]); Qs[ch * 8 + x][r] = t[x]; }
     }
-    __syncthreads();  // vmax_s is complete; every thread is done with K
-    const float am = __uint_as_float(vmax_s);
-    const float s_v = (am > 0.0f) ? fdiv(am, 127.0f) : 0.0f, inv_v = (am > 0.0f) ? fdiv(127.0f, am) : 0.0f;
-    const float cs = fdiv(s_v, 127.0f);
-    // ---- quantised, transposed values to the B operand ----
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int idx = tid + PTH * it, key = idx >> 4, ch = idx & 15;
-      float vv[8];
-      unpack8p(rw[it], vv);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const float t = fminf(fmaxf(fmul(vv[e], inv_v), -128.0f), 127.0f);
-        Vq[swz(ch * 8 + e, key)] = (int8_t)(int)rintf(t);
-      }
-    }
-    if (jt + 1 < ntiles) fetch(kp, j0 + PK, true);   // next K travels during the tensor-core product
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    tc_fence_before();
-    __syncthreads();
-    if (tid == 0) {
-      vmax_s = 0;
-      tc_fence_after();
-      const uint64_t da = make_smem_desc(smem_u32(Pq)), db = make_smem_desc(smem_u32(Vq));
-#pragma unroll
-      for (int k4 = 0; k4 < PK / 32; ++k4) umma_i8(tmem_base, da + (uint64_t)(k4 * 2), db + (uint64_t)(k4 * 2), idesc, k4 ? 1u : 0u);
-      umma_commit(&bar);
-    }
-    if (ok && !mbar_wait(&bar, phase, abort_flag, status)) ok = false;
-    ok = __all_sync(0xffffffffu, ok);   // the TMEM load below is warp-collective
-    phase ^= 1u;
-    tc_fence_after();
-    if (ok) {
-      uint32_t r[32];
-      tmem_ld32(taddr, r);
-      const float al = alpha_s[orow];
-#pragma unroll
-      for (int c = 0; c < 32; ++c) o[c] = fadd(fmul(o[c], al), fmul(__int2float_rn((int)r[c]), cs));
-    }
-    tc_fence_before();
-    if (!__syncthreads_and(ok)) break;   // operands, alpha and the accumulator may be overwritten by the next tile
-  }
-  // row statistics travel from the logit mapping (4 rows per thread) to the accumulator mapping (1 row per thread)
-  if (tx == 0) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { l_s[ty * 4 + i] = l[i]; m_s[ty * 4 + i] = m[i]; }
+    if (__any_sync(__activemask(), tq) && lane == 0) atomicOr(&tiny_q_s, 1);
   }
   __syncthreads();
-  const int row = q0 + orow;
-  if (row < S && !abort_s) {
-    const float lr = l_s[orow];
-    const float il = fdiv(1.0f, lr);
-    uint16_t* op = out + (row0 + row) * ld_out + (size_t)h * PD + ocol;
+
+  if (warp >= 16) {
+    // ------------------------------- producers -------------------------------
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    const int pt = tid - PV_CONS, pw = pt >> 5;
+    const int kcol = (pt & 4 ? AF_HI : 0) + (pt >> 3) * 4 + (pt & 3);
+    int slot = 0;
+    uint32_t par = 1;
+    bool ok = true;                                  // after a failed wait nothing is staged, but every barrier below is still met
+    constexpr uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(DH >> 3) << 17) | ((uint32_t)(PQ >> 4) << 24);
+    auto product = [&](int t) {                      // of block t, by one thread, once weights and values are there
+      if (pt == 0 && mbar_wait(&bar_v[t & 1], (uint32_t)(t >> 1) & 1u, abort_flag, status) &&
+          mbar_wait(&bar_p, (uint32_t)t & 1u, abort_flag, status)) {
+        tc_fence_after();
+        const uint64_t da = make_smem_desc(smem_u32(Pq)), db = make_smem_desc(smem_u32(Vq + (t & 1) * (PQ * PK)));
 #pragma unroll
-    for (int c = 0; c < 32; c += 8) {
-      uint4 w;
-      w.x = pack_bf2(fmul(o[c], il), fmul(o[c + 1], il)); w.y = pack_bf2(fmul(o[c + 2], il), fmul(o[c + 3], il));
-      w.z = pack_bf2(fmul(o[c + 4], il), fmul(o[c + 5], il)); w.w = pack_bf2(fmul(o[c + 6], il), fmul(o[c + 7], il));
-      *reinterpret_cast<uint4*>(op + c) = w;
+        for (int k4 = 0; k4 < PK / 32; ++k4) umma_i8(tmem_base, da + (uint64_t)(k4 * 2), db + (uint64_t)(k4 * 2), idesc, k4 ? 1u : 0u);
+        umma_commit(&bar_mma);
+      }
+      __syncwarp();
+    };
+    for (int t = 0; t < nt; ++t) {
+      const int j0 = (jt0 + t) * PK;
+      {  // K: slab sl holds head dimensions 16 sl .. of the 128 keys (thread = key), four slabs in flight
+        const bool in = j0 + pt < S;
+        const uint4* src = reinterpret_cast<const uint4*>(kp + (size_t)(j0 + pt) * ld);
+        uint4 raw[4][2];
+        auto fetch = [&](int sl, uint4 (&w)[2]) {
+          w[0] = in ? __ldg(src + 2 * sl) : make_uint4(0u, 0u, 0u, 0u);
+          w[1] = in ? __ldg(src + 2 * sl + 1) : make_uint4(0u, 0u, 0u, 0u);
+        };
+#pragma unroll
+        for (int d = 0; d < 4; ++d) fetch(d, raw[d]);
+#pragma unroll
+        for (int sl = 0; sl < 8; ++sl) {
+          ok = ok && mbar_wait(&bar_empty[slot], par, abort_flag, status);
+          const uint4 w0 = raw[sl & 3][0], w1 = raw[sl & 3][1];
+          const uint32_t words[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+          uint32_t tw = 0;
+          if (ok) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              word_tiny(words[i], tw);
+              Ring[slot][2 * i][kcol] = word_lo(words[i]);
+              Ring[slot][2 * i + 1][kcol] = word_hi(words[i]);
+            }
+          }
+          if (sl < 4) fetch(sl + 4, raw[sl & 3]);
+          const int any = __any_sync(0xffffffffu, words_tiny(tw));
+          if (lane == 0) { tiny_s[slot][pw] = any; }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bar_full[slot]);
+          if (++slot == PV_SLOTS) { slot = 0; par ^= 1u; }
+        }
+      }
+      if (t > 0) product(t - 1);
+      // V: block absmax (128 keys x 128 dims), then the quantised transposed operand
+      float vm = 0.0f;
+#pragma unroll 8
+      for (int it = 0; it < 16; ++it) {
+        const int key = j0 + it * 8 + (pt >> 4);
+        if (key < S) {
+          float x[8];
+          unpack8a(__ldg(reinterpret_cast<const uint4*>(vp + (size_t)key * ld + (pt & 15) * 8)), x);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) vm = fmaxf(vm, fabsf(x[e]));
+        }
+      }
+#pragma unroll
+      for (int w = 16; w; w >>= 1) vm = fmaxf(vm, __shfl_xor_sync(0xffffffffu, vm, w));
+      if (lane == 0) vmax_s[t & 1][pw] = vm;
+      // past this barrier the products up to block t - 2 are done and buffer t & 1 is free: the first warp has been through
+      // product(t - 1), which every consumer warp announced only after it had collected block t - 2
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      const float am = fmaxf(fmaxf(vmax_s[t & 1][0], vmax_s[t & 1][1]), fmaxf(vmax_s[t & 1][2], vmax_s[t & 1][3]));
+      const float s_v = (am > 0.0f) ? fdiv(am, 127.0f) : 0.0f, inv_v = (am > 0.0f) ? fdiv(127.0f, am) : 0.0f;
+      if (ok) {
+        if (pt == 0) cs_s[t & 3] = fdiv(s_v, 127.0f);
+        int8_t* dst = Vq + (t & 1) * (PQ * PK);
+        const int key = j0 + 4 * lane;               // four adjacent keys x eight dimensions a step: one word per dimension
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int ch = pw * 4 + c;
+          uint4 u[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            u[i] = key + i < S ? __ldg(reinterpret_cast<const uint4*>(vp + (size_t)(key + i) * ld + ch * 8)) : make_uint4(0u, 0u, 0u, 0u);
+          float x[4][8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) unpack8a(u[i], x[i]);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            uint32_t w = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w |= (uint32_t)(uint8_t)quant1(x[i][e], inv_v) << (8 * i);
+            *reinterpret_cast<uint32_t*>(dst + swz(ch * 8 + e, 4 * lane)) = w;
+          }
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar_v[t & 1]);
     }
-    if (ocol == 0) lse[((size_t)b * H + h) * S + row] = fadd(m_s[orow], det_log(lr));
+    product(nt - 1);
+  } else {
+    // ------------------------------- consumers -------------------------------
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+    const int tiny_q = tiny_q_s;
+    const int wrow = warp * AF_RW, r2 = lane & 1, tx = lane >> 1, lrow = wrow + 4 * r2;
+    // accumulator phase: this thread owns query row orow and the 32 output dimensions starting at ocol
+    const int orow = (warp & 3) * 32 + lane, ocol = (warp >> 2) * 32;
+    const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)ocol;
+    const float2 one = same2(c_one);
+    float m_mine = __int_as_float(0xff800000), l_mine = 0.0f, alpha_mine = 0.0f;   // row ROW_OF_LANE(lane) of the warp
+    float2 o[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) o[c] = make_float2(0.0f, 0.0f);
+    // o = o * alpha + u of block t, once its product is there
+    auto collect = [&](int t) -> bool {
+      bool ok = mbar_wait(&bar_p, (uint32_t)t & 1u, abort_flag, status) && mbar_wait(&bar_mma, (uint32_t)t & 1u, abort_flag, status);
+      if (!__all_sync(0xffffffffu, ok)) return false;   // the TMEM load below is warp-collective
+      tc_fence_after();
+      const float2 al = same2(alpha_s[t & 1][orow]), cs = same2(cs_s[t & 3]);
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        uint32_t r[16];
+        tmem_ld16_nowait(taddr + 16 * hf, r);
+        tmem_wait_ld();
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const float2 u = make_float2(__int2float_rn((int)r[2 * c]), __int2float_rn((int)r[2 * c + 1]));
+          o[8 * hf + c] = add2(mul2(o[8 * hf + c], al), mul2(u, cs), one);
+        }
+      }
+      tc_fence_before();
+      return true;
+    };
+    bool ok = true;
+    int slot = 0;
+    uint32_t par = 0;
+    for (int t = 0; t < nt && ok; ++t) {
+      const int j0 = (jt0 + t) * PK;
+      const bool diag = t == nt - 1;                 // only the last block of a row block reaches past the diagonal
+      const bool edge = W > 0 && j0 <= q0 + PQ - 1 - W;  // some row's window starts inside or after this block
+      float2 acc[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
+      for (int sl = 0; sl < 8; ++sl) {
+        if (!mbar_wait(&bar_full[slot], par, abort_flag, status)) { ok = false; break; }
+        const int4 t4 = *reinterpret_cast<const int4*>(tiny_s[slot]);
+        const float* ap = &Qs[sl * OK][lrow];
+        if (tiny_q | t4.x | t4.y | t4.z | t4.w) mac_4x8<false, false>(ap, PLQ, 0, 0, Ring[slot], tx, acc);
+        else mac_4x8<true, false>(ap, PLQ, 0, 0, Ring[slot], tx, acc);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar_empty[slot]);
+        if (++slot == PV_SLOTS) { slot = 0; par ^= 1u; }
+      }
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok && t > 0) ok = collect(t - 1);
+      if (!ok) break;
+      softmax_block(acc, j0 + 8 * tx, q0 + lrow, q0 + wrow + ROW_OF_LANE(lane), j0 + PK - 1, W, diag, edge, lane, m_mine, l_mine,
+                    alpha_mine, one);
+      if (lane < AF_RW) alpha_s[t & 1][wrow + ROW_OF_LANE(lane)] = alpha_mine;
+      // q_p = rne(127 p) of the lane's 4 x 8 weights (0 <= 127 p <= 127: adding 1.5 2^23 leaves the integer in the low byte)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        uint32_t w[2];
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          const float2 x = add2(mul2(acc[i][2 * g], same2(127.0f)), same2(12582912.0f), one);
+          const float2 y = add2(mul2(acc[i][2 * g + 1], same2(127.0f)), same2(12582912.0f), one);
+          w[g] = __byte_perm(__byte_perm(__float_as_uint(x.x), __float_as_uint(x.y), 0x0040),
+                             __byte_perm(__float_as_uint(y.x), __float_as_uint(y.y), 0x0040), 0x5410);
+        }
+        *reinterpret_cast<uint2*>(Pq + swz(lrow + i, 8 * tx)) = make_uint2(w[0], w[1]);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar_p);
+    }
+    if (ok) ok = collect(nt - 1);
+    // row sums travel from the logit mapping (a lane per row) to the accumulator mapping (a row per thread)
+    if (lane < AF_RW) {
+      const int r = wrow + ROW_OF_LANE(lane);
+      l_s[r] = l_mine;
+      if (q0 + r < S && ok) lse[((size_t)b * H + h) * S + q0 + r] = fadd(m_mine, det_log(l_mine));
+    }
+    asm volatile("bar.sync 2, 512;" ::: "memory");
+    const int row = q0 + orow;
+    if (row < S && ok) {
+      const float il = fdiv(1.0f, l_s[orow]);
+      uint16_t* op = out + (row0 + row) * ld_out + (size_t)h * DH + ocol;
+#pragma unroll
+      for (int c = 0; c < 16; c += 4) {
+        uint4 w;
+        w.x = pack_bf2(fmul(o[c].x, il), fmul(o[c].y, il));
+        w.y = pack_bf2(fmul(o[c + 1].x, il), fmul(o[c + 1].y, il));
+        w.z = pack_bf2(fmul(o[c + 2].x, il), fmul(o[c + 2].y, il));
+        w.w = pack_bf2(fmul(o[c + 3].x, il), fmul(o[c + 3].y, il));
+        *reinterpret_cast<uint4*>(op + 2 * c) = w;
+      }
+    }
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(128u) : "memory");
+  if (abort_s) {   // give copies and products in flight time to land before the TMEM goes
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000ll) { }
+    __syncthreads();
+  }
+  if (warp == 16) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(128u) : "memory");
+  }
 }
 
 }  // namespace det
@@ -294,12 +322,12 @@ using namespace det;
 extern "C" int det_attn_fwd_int8pv(const det_bf16* q, const det_bf16* k, const det_bf16* v, int ld, int B, int H, int Hkv, int S,
                                    int window, det_bf16* out, int ld_out, float* lse, void* stream, int* status_dev) {
   if (!q || !k || !v || !out || !lse || B <= 0 || H <= 0 || Hkv <= 0 || S <= 0 || window < 0) return DET_ERR_ARG;
-  if (S % 64 || ld % 8 || ld_out % 8 || ld < H * PD || ld_out < H * PD || H % Hkv || window % 128) return DET_ERR_SHAPE;
+  if (S % 64 || ld % 8 || ld_out % 8 || ld < H * DH || ld_out < H * DH || H % Hkv || window % 128) return DET_ERR_SHAPE;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out)) return DET_ERR_ALIGN;
   static DevOnce once = {};
   if (dev_ensure_smem(once, (const void*)k_attn_fwd_pv8, PV8_SMEM) != DET_OK) return DET_ERR_CUDA;
   dim3 grid(H * B, (S + PQ - 1) / PQ);
-  k_attn_fwd_pv8<<<DET_L(grid), PTH, PV8_SMEM, (cudaStream_t)stream>>>(q, k, v, ld, H, Hkv, S, window, out, ld_out, lse, status_dev);
+  k_attn_fwd_pv8<<<DET_L(grid), PV_THREADS, PV8_SMEM, (cudaStream_t)stream>>>(q, k, v, ld, H, Hkv, S, window, out, ld_out, lse, status_dev);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
