@@ -4,12 +4,12 @@
 //
 //   C[i,j] = sum_k A[i,k] * B[j,k]        A: int8 [I,K] row-major, B: int8 [J,K] row-major (both K-major)
 //
-// One persistent CTA per SM, 192 threads:
-//   warp 0    TMA producer: 128-byte-swizzled tiles of A (128 x 128 B) and B (BN x 128 B) into a 4-stage ring
-//   warp 1    allocates TMEM (512 columns = two BN=256 accumulators) and issues tcgen05.mma.kind::i8
+// One persistent CTA per SM, tiles of 128 x BN (BN = 256, 128 or 64):
+//   warp 0    TMA producer: 128-byte-swizzled tiles of A (128 x 128 B) and B (BN x 128 B) into a ring of 4 to 8 stages
+//   warp 1    allocates TMEM (two BN-column accumulators) and issues tcgen05.mma.kind::i8
 //             (M=128, N=BN, K=32 per instruction, 4 per stage); tcgen05.commit releases ring slots
-//   warps 2-5 epilogue: tcgen05.ld of the int32 accumulator (lane = row), dequantise / mask in registers,
-//             stores; overlaps with the next tile's MMAs through the second accumulator
+//   the rest  epilogue: tcgen05.ld of the int32 accumulator (lane = row), dequantise / mask in registers, stores in whole
+//             row segments through a staging tile; overlaps with the next tile's MMAs through the second accumulator
 // Every mbarrier wait is bounded: on expiry the kernel raises DET_DEV_TIMEOUT in *status, stops issuing
 // work, lets in-flight copies land, frees its TMEM and returns.
 #include "tc05.cuh"
@@ -20,8 +20,12 @@ namespace det {
 
 constexpr int BM = 128;
 constexpr int BK = 128;  // bytes (= int8 elements) per stage along K
-constexpr int STAGES = 4;
-constexpr int GEMM_THREADS = 192;
+// eight epilogue warps (two per TMEM lane quarter, half of the columns each), four for the narrow tile
+template <int BN> struct IgTile {
+  static constexpr int STAGES = BN == 256 ? 4 : (BN == 128 ? 6 : 8), EW = BN == 64 ? 4 : 8, CW = BN / (EW / 4);
+  static constexpr int THREADS = 64 + 32 * EW, TCOLS = 2 * BN;
+  static constexpr size_t SMEM = (size_t)STAGES * (BM * BK + BN * BK) + EW * 4096 + 1024;
+};
 // Tile order: the dimension with fewer tiles runs fastest, so that the CTAs resident at one time share the smaller
 // operand's tiles and the larger operand streams through L2 once.
 __device__ __forceinline__ void tile_origin(int tile, int tiles_i, int tiles_j, int bn, int& i0, int& j0) {
@@ -73,136 +77,108 @@ __device__ __forceinline__ void rows32_to_lanes(uint8_t* stage, const uint4 (&pr
   for (int v = 0; v < 4; ++v) w[v] = *reinterpret_cast<const uint4*>(stage + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4));
 }
 
-// Epilogue of one accumulator row: this lane owns TMEM lane `taddr`'s row (output row `row`), columns j0 .. j0+BN.
-// With a staging tile (`stage`, 4 KiB per warp) the outputs are written through store_rows32.
-template <int BN, int EPI>
+// Epilogue of one accumulator row: this lane owns TMEM lane `taddr`'s row (output row `row`), columns j0 .. j0+CW.
+// The outputs are written through store_rows32 and the reference operand is read the same way, one chunk of 32 ahead (`stage`: 4 KiB
+// per warp).  DX leaves the partial sums of dXhat * phi of every 64 columns (an aligned subtree of the fixed tree).
+template <int CW, int EPI>
 __device__ __forceinline__ void epi_row(const EpiParams& ep, uint32_t taddr, int row, int J, int j0, float cscale,
-                                        float inv_s, float sx, uint8_t* stage = nullptr) {
-      const size_t rbase = (size_t)row * J + j0;
-      const size_t wbase = (size_t)(row - (int)(threadIdx.x & 31)) * J + j0;  // the warp's first row
-      if (EPI == EPI_DW) inv_s = fdiv(1.0f, ep.s_w[row]);
+                                        float inv_s, float sx, uint8_t* stage) {
+  const size_t wbase = (size_t)(row - (int)(threadIdx.x & 31)) * J + j0;  // the warp's first row
+  constexpr bool REF = EPI == EPI_DX || EPI == EPI_DW;
+  if (EPI == EPI_DW) inv_s = fdiv(1.0f, ep.s_w[row]);
+  uint4 pre[4];
+  if (REF) fetch_rows32(reinterpret_cast<const uint8_t*>(ep.ref + wbase), (size_t)J * 2, pre);
 #pragma unroll 1
-      for (int h = 0; h < BN / 128; ++h) {
-      float grp[4];
-      uint4 pre[4];
-      const bool staged_ref = (EPI == EPI_DX || EPI == EPI_DW) && stage != nullptr;
-      if (staged_ref) fetch_rows32(reinterpret_cast<const uint8_t*>(ep.ref + wbase + h * 128), (size_t)J * 2, pre);
+  for (int h = 0; h < CW / 64; ++h) {
+    float grp[2];
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
-        const int c0 = h * 128 + cc * 32;
-        uint32_t r[32];
-        tmem_ld32(taddr + (uint32_t)c0, r);
-        uint4 refw[4];
-        if (EPI == EPI_DX || EPI == EPI_DW) {
-          if (staged_ref) {
-            rows32_to_lanes(stage, pre, refw);
-            if (cc < 3) fetch_rows32(reinterpret_cast<const uint8_t*>(ep.ref + wbase + c0 + 32), (size_t)J * 2, pre);
-          } else {
-            const uint4* rr = reinterpret_cast<const uint4*>(ep.ref + rbase + c0);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) refw[v] = __ldg(rr + v);
-          }
-        }
-        if (EPI == EPI_RAW) {
-          uint4 o[8];
-#pragma unroll
-          for (int v = 0; v < 8; ++v) o[v] = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
-          if (stage) store_rows32<8>(stage, reinterpret_cast<uint8_t*>(reinterpret_cast<int32_t*>(ep.out) + wbase + c0), (size_t)J * 4, o);
-          else {
-            uint4* og = reinterpret_cast<uint4*>(reinterpret_cast<int32_t*>(ep.out) + rbase + c0);
-#pragma unroll
-            for (int v = 0; v < 8; ++v) og[v] = o[v];
-          }
-        } else if (EPI == EPI_FWD) {
-          const float4* sw = reinterpret_cast<const float4*>(ep.s_w + j0 + c0);
-          uint4 o[4];
-#pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            float4 w0 = __ldg(sw + 2 * v), w1 = __ldg(sw + 2 * v + 1);
-            float f[8];
-            f[0] = fmul(__int2float_rn((int)r[8 * v + 0]), fmul(sx, w0.x));
-            f[1] = fmul(__int2float_rn((int)r[8 * v + 1]), fmul(sx, w0.y));
-            f[2] = fmul(__int2float_rn((int)r[8 * v + 2]), fmul(sx, w0.z));
-            f[3] = fmul(__int2float_rn((int)r[8 * v + 3]), fmul(sx, w0.w));
-            f[4] = fmul(__int2float_rn((int)r[8 * v + 4]), fmul(sx, w1.x));
-            f[5] = fmul(__int2float_rn((int)r[8 * v + 5]), fmul(sx, w1.y));
-            f[6] = fmul(__int2float_rn((int)r[8 * v + 6]), fmul(sx, w1.z));
-            f[7] = fmul(__int2float_rn((int)r[8 * v + 7]), fmul(sx, w1.w));
-            o[v] = make_uint4(pack_bf2(f[0], f[1]), pack_bf2(f[2], f[3]), pack_bf2(f[4], f[5]), pack_bf2(f[6], f[7]));
-          }
-          if (stage) store_rows32<4>(stage, reinterpret_cast<uint8_t*>(reinterpret_cast<uint16_t*>(ep.out) + wbase + c0), (size_t)J * 2, o);
-          else {
-            uint4* og = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(ep.out) + rbase + c0);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) og[v] = o[v];
-          }
-        } else if (EPI == EPI_DX) {
-          uint4 o[4];
-          float term[32];
-#pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            uint4 xu = refw[v];
-            const uint32_t xs[4] = {xu.x, xu.y, xu.z, xu.w};
-            float g[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const float xv = (e & 1) ? bfhi(xs[e >> 1]) : bflo(xs[e >> 1]);
-              const float gx = fmul(__int2float_rn((int)r[8 * v + e]), cscale);
-              const float t = fmul(xv, inv_s);
-              const bool in_range = (t >= -128.0f) && (t <= 127.0f);
-              const float phi = t < -128.0f ? -128.0f : (t > 127.0f ? 127.0f : fsub(rintf(t), t));
-              g[e] = in_range ? gx : 0.0f;
-              term[8 * v + e] = fmul(gx, phi);
-            }
-            o[v] = make_uint4(pack_bf2(g[0], g[1]), pack_bf2(g[2], g[3]), pack_bf2(g[4], g[5]), pack_bf2(g[6], g[7]));
-          }
-          if (stage) store_rows32<4>(stage, reinterpret_cast<uint8_t*>(reinterpret_cast<uint16_t*>(ep.out) + wbase + c0), (size_t)J * 2, o);
-          else {
-            uint4* og = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(ep.out) + rbase + c0);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) og[v] = o[v];
-          }
-          // adjacent tree over this lane's 32 columns
-#pragma unroll
-          for (int w = 1; w < 32; w <<= 1)
-#pragma unroll
-            for (int e = 0; e < 32; e += 2 * w) term[e] = fadd(term[e], term[e + w]);
-          grp[cc] = term[0];
-        } else {  // EPI_DW
-          uint4 o[8];
-#pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            uint4 wu = refw[v];
-            const uint32_t wsr[4] = {wu.x, wu.y, wu.z, wu.w};
-            float g[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const float wv = (e & 1) ? bfhi(wsr[e >> 1]) : bflo(wsr[e >> 1]);
-              const float t = fmul(wv, inv_s);
-              const bool in_range = (t >= -128.0f) && (t <= 127.0f);
-              g[e] = in_range ? fmul(__int2float_rn((int)r[8 * v + e]), cscale) : 0.0f;
-            }
-            o[2 * v] = make_uint4(__float_as_uint(g[0]), __float_as_uint(g[1]), __float_as_uint(g[2]), __float_as_uint(g[3]));
-            o[2 * v + 1] = make_uint4(__float_as_uint(g[4]), __float_as_uint(g[5]), __float_as_uint(g[6]), __float_as_uint(g[7]));
-          }
-          if (stage) store_rows32<8>(stage, reinterpret_cast<uint8_t*>(reinterpret_cast<float*>(ep.out) + wbase + c0), (size_t)J * 4, o);
-          else {
-            uint4* og = reinterpret_cast<uint4*>(reinterpret_cast<float*>(ep.out) + rbase + c0);
-#pragma unroll
-            for (int v = 0; v < 8; ++v) og[v] = o[v];
-          }
-        }
+    for (int cc = 0; cc < 2; ++cc) {
+      const int c0 = h * 64 + cc * 32;
+      uint32_t r[32];
+      tmem_ld32(taddr + (uint32_t)c0, r);
+      uint4 refw[4];
+      if (REF) {
+        rows32_to_lanes(stage, pre, refw);
+        if (c0 + 32 < CW) fetch_rows32(reinterpret_cast<const uint8_t*>(ep.ref + wbase + c0 + 32), (size_t)J * 2, pre);
       }
-      if (EPI == EPI_DX)
-        ep.ds_partial[(size_t)row * (J / 128) + (j0 / 128) + h] = fadd(fadd(grp[0], grp[1]), fadd(grp[2], grp[3]));
+      if (EPI == EPI_RAW) {
+        uint4 o[8];
+#pragma unroll
+        for (int v = 0; v < 8; ++v) o[v] = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
+        store_rows32<8>(stage, reinterpret_cast<uint8_t*>(reinterpret_cast<int32_t*>(ep.out) + wbase + c0), (size_t)J * 4, o);
+      } else if (EPI == EPI_FWD) {
+        const float4* sw = reinterpret_cast<const float4*>(ep.s_w + j0 + c0);
+        uint4 o[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          float4 w0 = __ldg(sw + 2 * v), w1 = __ldg(sw + 2 * v + 1);
+          float f[8];
+          f[0] = fmul(__int2float_rn((int)r[8 * v + 0]), fmul(sx, w0.x));
+          f[1] = fmul(__int2float_rn((int)r[8 * v + 1]), fmul(sx, w0.y));
+          f[2] = fmul(__int2float_rn((int)r[8 * v + 2]), fmul(sx, w0.z));
+          f[3] = fmul(__int2float_rn((int)r[8 * v + 3]), fmul(sx, w0.w));
+          f[4] = fmul(__int2float_rn((int)r[8 * v + 4]), fmul(sx, w1.x));
+          f[5] = fmul(__int2float_rn((int)r[8 * v + 5]), fmul(sx, w1.y));
+          f[6] = fmul(__int2float_rn((int)r[8 * v + 6]), fmul(sx, w1.z));
+          f[7] = fmul(__int2float_rn((int)r[8 * v + 7]), fmul(sx, w1.w));
+          o[v] = make_uint4(pack_bf2(f[0], f[1]), pack_bf2(f[2], f[3]), pack_bf2(f[4], f[5]), pack_bf2(f[6], f[7]));
+        }
+        store_rows32<4>(stage, reinterpret_cast<uint8_t*>(reinterpret_cast<uint16_t*>(ep.out) + wbase + c0), (size_t)J * 2, o);
+      } else if (EPI == EPI_DX) {
+        uint4 o[4];
+        float term[32];
+        const float2 one = same2(c_one);
+#pragma unroll
+        for (int v = 0; v < 16; ++v) {
+          const uint32_t xs = reinterpret_cast<const uint32_t*>(refw)[v];
+          const float2 gx = mul2(make_float2(__int2float_rn((int)r[2 * v]), __int2float_rn((int)r[2 * v + 1])), same2(cscale));
+          const float2 t = mul2(make_float2(bflo(xs), bfhi(xs)), same2(inv_s));
+          // t held to [-128, 127]; rne(t) - t where it holds t itself (a NaN included: it compares neither below nor above)
+          const float2 tc = make_float2(fminf(fmaxf(t.x, -128.0f), 127.0f), fminf(fmaxf(t.y, -128.0f), 127.0f));
+          const float2 d = add2(add2(add2(t, same2(12582912.0f), one), same2(-12582912.0f), one), make_float2(-t.x, -t.y), one);
+          const float2 phi = make_float2((t.x < tc.x || t.x > tc.x) ? tc.x : d.x, (t.y < tc.y || t.y > tc.y) ? tc.y : d.y);
+          reinterpret_cast<uint32_t*>(o)[v] = pack_bf2(t.x == tc.x ? gx.x : 0.0f, t.y == tc.y ? gx.y : 0.0f);
+          const float2 p = mul2(gx, phi);
+          term[2 * v] = p.x;
+          term[2 * v + 1] = p.y;
+        }
+        store_rows32<4>(stage, reinterpret_cast<uint8_t*>(reinterpret_cast<uint16_t*>(ep.out) + wbase + c0), (size_t)J * 2, o);
+        // adjacent tree over this lane's 32 columns
+#pragma unroll
+        for (int w = 1; w < 32; w <<= 1)
+#pragma unroll
+          for (int e = 0; e < 32; e += 2 * w) term[e] = fadd(term[e], term[e + w]);
+        grp[cc] = term[0];
+      } else {  // EPI_DW
+        uint4 o[8];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          uint4 wu = refw[v];
+          const uint32_t wsr[4] = {wu.x, wu.y, wu.z, wu.w};
+          float g[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            const float wv = (e & 1) ? bfhi(wsr[e >> 1]) : bflo(wsr[e >> 1]);
+            const float t = fmul(wv, inv_s);
+            const bool in_range = (t >= -128.0f) && (t <= 127.0f);
+            g[e] = in_range ? fmul(__int2float_rn((int)r[8 * v + e]), cscale) : 0.0f;
+          }
+          o[2 * v] = make_uint4(__float_as_uint(g[0]), __float_as_uint(g[1]), __float_as_uint(g[2]), __float_as_uint(g[3]));
+          o[2 * v + 1] = make_uint4(__float_as_uint(g[4]), __float_as_uint(g[5]), __float_as_uint(g[6]), __float_as_uint(g[7]));
+        }
+        store_rows32<8>(stage, reinterpret_cast<uint8_t*>(reinterpret_cast<float*>(ep.out) + wbase + c0), (size_t)J * 4, o);
       }
+    }
+    if (EPI == EPI_DX) ep.ds_partial[(size_t)row * (J / 64) + (j0 / 64) + h] = fadd(grp[0], grp[1]);
+  }
 }
 
 template <int BN, int EPI>
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
+__global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
     k_igemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, EpiParams ep, int I, int J,
             int K, int* status) {
   constexpr int STAGE_A = BM * BK, STAGE_B = BN * BK, STAGE_BYTES = STAGE_A + STAGE_B;
+  constexpr int STAGES = IgTile<BN>::STAGES, EW = IgTile<BN>::EW, CW = IgTile<BN>::CW;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t bar_full[STAGES], bar_empty[STAGES], bar_tfull[2], bar_tempty[2];
@@ -213,7 +189,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&bar_empty[s], 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(&bar_tfull[a], 1); mbar_init(&bar_tempty[a], 4); }
+    for (int a = 0; a < 2; ++a) { mbar_init(&bar_tfull[a], 1); mbar_init(&bar_tempty[a], EW); }
     abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -221,7 +197,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512u)
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"((uint32_t)IgTile<BN>::TCOLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -281,7 +257,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       }
     }
   } else {
-    const int q = warp & 3;  // TMEM lane quarter this warp may read
+    const int q = warp & 3, part = (warp - 2) >> 2;  // TMEM lane quarter this warp may read; its share of the columns
+    uint8_t* stage = smem + STAGES * STAGE_BYTES + (warp - 2) * 4096;  // this warp's 32 x 128-byte staging tile
     int it = 0;
     bool ok = true;
     float cscale, inv_s, sx;
@@ -293,7 +270,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         tile_origin(tile, tiles_i, tiles_j, BN, i0, j0);
       if (!mbar_wait(&bar_tfull[acc], acc_phase, abort_flag, status)) { ok = false; break; }
       tc_fence_after();
-      epi_row<BN, EPI>(ep, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN), i0 + q * 32 + lane, J, j0, cscale, inv_s, sx);
+      epi_row<CW, EPI>(ep, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + part * CW), i0 + q * 32 + lane, J,
+                       j0 + part * CW, cscale, inv_s, sx, stage);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar_tempty[acc]);
@@ -309,7 +287,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   }
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)IgTile<BN>::TCOLS) : "memory");
   }
 }
 
@@ -529,14 +507,14 @@ bool make_map(CUtensorMap* tm, const int8_t* base, int rows, int K, int box_rows
 template <int BN, int EPI>
 static int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const EpiParams& ep, int I, int J, int K, int* status,
                       cudaStream_t st) {
-  constexpr size_t smem = (size_t)STAGES * (BM * BK + BN * BK) + 1024;
+  typedef IgTile<BN> T;
   static DevOnce once = {};
-  if (dev_ensure_smem(once, (const void*)k_igemm<BN, EPI>, smem) != DET_OK) return DET_ERR_CUDA;
+  if (dev_ensure_smem(once, (const void*)k_igemm<BN, EPI>, T::SMEM) != DET_OK) return DET_ERR_CUDA;
   const int sms = dev_sm_count();
   if (sms <= 0) return DET_ERR_CUDA;
   const int tiles = (I / BM) * (J / BN);
   const int grid = tiles < sms ? tiles : sms;
-  k_igemm<BN, EPI><<<DET_L(grid), GEMM_THREADS, smem, st>>>(ta, tb, ep, I, J, K, status);
+  k_igemm<BN, EPI><<<DET_L(grid), T::THREADS, T::SMEM, st>>>(ta, tb, ep, I, J, K, status);
   if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return DET_ERR_CUDA; }
   return DET_OK;
 }
@@ -557,37 +535,55 @@ static int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const EpiPa
   return DET_OK;
 }
 
-// Two-CTA 256 x 256 tiles when both output dimensions are multiples of 256 (unless force_one_cta), else the one-CTA kernel.
+// Which tile: whole rounds of tiles over the SMs, each the longer of its multiply loop and its epilogue, and once the other of the
+// two.  Measured, in microseconds: a 128-deep step costs 0.37 with 256-column tiles and 0.30 with narrower ones (bound by the
+// tensor pipe and by L2), the epilogue of a tile what the table says.  A small grid is bound by the epilogue of one tile, which a
+// narrow tile shortens and spreads over more SMs (1024 x 1024 x 1024: 11.1, 10.6, 8.5, 8.5 forward and 16.7, 15.3, 12.6, 10.5
+// input gradient for 256 x 256 pairs and 256, 128, 64 columns); over many rounds the pairs run a few percent faster
+// than their rounds say (16384 x 2048 x 8192: 166, 171, 265, 520), over few of them the 256-column tiles of one CTA.
+// Returns the columns of a one-CTA tile, or 512 for the CTA pair (256 x 256).
+static int igemm_pick(int epi, int I, int J, int K, int force_one_cta) {
+  const int sms = dev_sm_count() > 0 ? dev_sm_count() : 1;
+  struct { int bn, bi, bj, units; double step, turn, epi[4]; } const c[4] = {     // epi: RAW, FWD, DX, DW
+      {512, 256, 256, sms / 2, 0.365, 0.9, {6.6, 4.2, 10.0, 6.6}}, {256, 128, 256, sms, 0.375, 0.5, {6.2, 4.0, 9.3, 6.2}},
+      {128, 128, 128, sms, 0.30, 0.5, {3.8, 1.7, 5.7, 3.8}}, {64, 128, 64, sms, 0.30, 0.5, {1.8, 1.7, 3.7, 1.8}}};
+  int best = 0;
+  double best_t = 0.0;
+  for (int i = force_one_cta ? 1 : 0; i < 4; ++i) {
+    if (I % c[i].bi || J % c[i].bj || !c[i].units) continue;
+    const long long tiles = (long long)(I / c[i].bi) * (J / c[i].bj), rounds = (tiles + c[i].units - 1) / c[i].units;
+    const double loop = (K / BK) * c[i].step, e = c[i].epi[epi];
+    double t = rounds * ((loop > e ? loop : e) + c[i].turn) + (loop > e ? e : loop);
+    if (c[i].bn == 512 && rounds >= 6) t *= 0.95;
+    if (!best || t < best_t) { best = c[i].bn; best_t = t; }
+  }
+  return best;
+}
+template <int EPI>
+static int igemm_tile(int bn, const CUtensorMap& ta, const CUtensorMap& tb, const EpiParams& ep, int I, int J, int K, int* status,
+                      cudaStream_t st) {
+  switch (bn) {
+    case 512: return launch_pair<EPI>(ta, tb, ep, I, J, K, status, st);
+    case 256: return launch_one<256, EPI>(ta, tb, ep, I, J, K, status, st);
+    case 128: return launch_one<128, EPI>(ta, tb, ep, I, J, K, status, st);
+    default: return launch_one<64, EPI>(ta, tb, ep, I, J, K, status, st);
+  }
+}
 int igemm_launch(int epi, const int8_t* A, const int8_t* B, int I, int J, int K, const EpiParams& ep, int* status,
                  cudaStream_t st, int force_one_cta) {
   if (!A || !B || I <= 0 || J <= 0 || K <= 0) return DET_ERR_ARG;
   if (I % BM || J % 128 || K % BK) return DET_ERR_SHAPE;
   if (K >= (1 << 17)) return DET_ERR_RANGE;
   if (!aligned16(A) || !aligned16(B)) return DET_ERR_ALIGN;
-  const int bn = (J % 256 == 0) ? 256 : 128;
+  const int bn = igemm_pick(epi, I, J, K, force_one_cta);
   CUtensorMap ta, tb;
-  if (!force_one_cta && I % 256 == 0 && J % 256 == 0) {
-    if (!make_map(&ta, A, I, K, 128) || !make_map(&tb, B, J, K, 128)) return DET_ERR_CUDA;
-    switch (epi) {
-      case EPI_RAW: return launch_pair<EPI_RAW>(ta, tb, ep, I, J, K, status, st);
-      case EPI_FWD: return launch_pair<EPI_FWD>(ta, tb, ep, I, J, K, status, st);
-      case EPI_DX: return launch_pair<EPI_DX>(ta, tb, ep, I, J, K, status, st);
-      case EPI_DW: return launch_pair<EPI_DW>(ta, tb, ep, I, J, K, status, st);
-    }
-    return DET_ERR_ARG;
-  }
-  if (!make_map(&ta, A, I, K, BM) || !make_map(&tb, B, J, K, bn)) return DET_ERR_CUDA;
-#define DET_GEMM_CASE(E)                                                     \
-  case E:                                                                    \
-    return bn == 256 ? launch_one<256, E>(ta, tb, ep, I, J, K, status, st)   \
-                     : launch_one<128, E>(ta, tb, ep, I, J, K, status, st);
+  if (!make_map(&ta, A, I, K, 128) || !make_map(&tb, B, J, K, bn == 512 ? 128 : bn)) return DET_ERR_CUDA;
   switch (epi) {
-    DET_GEMM_CASE(EPI_RAW)
-    DET_GEMM_CASE(EPI_FWD)
-    DET_GEMM_CASE(EPI_DX)
-    DET_GEMM_CASE(EPI_DW)
+    case EPI_RAW: return igemm_tile<EPI_RAW>(bn, ta, tb, ep, I, J, K, status, st);
+    case EPI_FWD: return igemm_tile<EPI_FWD>(bn, ta, tb, ep, I, J, K, status, st);
+    case EPI_DX: return igemm_tile<EPI_DX>(bn, ta, tb, ep, I, J, K, status, st);
+    case EPI_DW: return igemm_tile<EPI_DW>(bn, ta, tb, ep, I, J, K, status, st);
   }
-#undef DET_GEMM_CASE
   return DET_ERR_ARG;
 }
 

@@ -28,7 +28,7 @@ struct EpiParams {
   const float* s_u;       // DX: step of the rotated weights
   const uint16_t* ref;    // DX: X bf16 [I,J]; DW: W bf16 [I,J] (range masks)
   float rot;              // 2^-7 with rotation, 1 without
-  float* ds_partial;      // DX: [I, J/128] partial sums of dXhat * phi
+  float* ds_partial;      // DX: [I, J/64] partial sums of dXhat * phi
 };
 
 // Independent kernels of one call may run side by side so that the partial last wave of one grid is filled by blocks of

@@ -595,7 +595,7 @@ static size_t bwd_ws_layout(int M, int N, int K, size_t* oA, size_t* oG, size_t*
   *oA = off; off += align_up((size_t)M * N, 256);
   *oG = off; off += align_up((size_t)M * N, 256);
   *oZ = off; off += align_up((size_t)M * K, 256);
-  const size_t np = (size_t)M * (K / 128);
+  const size_t np = (size_t)M * (K / 64);
   *oP = off; off += align_up(np * sizeof(float), 256);
   *oS = off; off += align_up((sum_ws_floats(np) + 64) * sizeof(float), 256);
   return off;
@@ -670,7 +670,7 @@ extern "C" int det_linear_bwd(const det_bf16* dY, const det_bf16* X, const int8_
   if (rc != DET_OK) return rc;
   rc = igemm_launch(EPI_DW, GqT, ZqT, N, K, M, ew, status_dev, aux.aux(0));
   if (rc != DET_OK) return rc;
-  const size_t np = (size_t)M * (K / 128);
+  const size_t np = (size_t)M * (K / 64);
   sum_scaled_launch(partial, np, (float)(1.0 / sqrt((double)M * (double)K * 127.0)), ds_x, sscr, st);
   DET_CHECK_LAUNCH();
   if (!aux.join()) return DET_ERR_CUDA;

@@ -148,3 +148,29 @@ def test_adamw_many_tensors(det, sizes, clip):
         assert_same_bits(host(dp[i], p[i].dtype), po, "p %d" % i)
         assert_same_bits(host(dm[i]), mo, "m %d" % i)
         assert_same_bits(host(dv[i]), vo, "v %d" % i)
+
+
+# LSQ linear at sizes where the tile of the int8 GEMMs changes (64, 128, 256 columns, CTA pairs), with a last round that is
+# nearly empty and with dimensions that only narrow tiles divide
+@pytest.mark.parametrize("M,N,K", [(128, 128, 128), (384, 640, 384), (1024, 3072, 1024), (1664, 3072, 1024)])
+def test_linear_tiles(det, M, N, K):
+    import torch
+    X, W = synth.normal_bf16((M, K), 1.0, seed=M, tid=1), synth.normal_bf16((N, K), 0.02, seed=M, tid=2)
+    dY = synth.normal_bf16((M, N), 0.01, seed=M, tid=3)
+    X[::7, ::11] = synth.to_bf16(np.array([40.0], F))[0]           # outside the quantiser's range: masked gradient, clamped phi
+    sw, sx = oracle.lsq_weight_scale(W), oracle.lsq_act_scale_init(synth.normal_bf16((M, K), 1.0, seed=M, tid=1))
+    oY, oqX, oqW = oracle.linear_fwd(X, W, sx, sw)
+    odX, odW, ods = oracle.linear_bwd(dY, X, W, sx, sw, hb=128)
+    dX_, dW_, s_w, s_x = dev(X), dev(W), dev(sw), dev(sx)
+    qW, qWt, s_u = empty((N, K), np.int8), empty((K, N), np.int8), empty((1,), F)
+    det.det_lsq_quantize_weight(dW_, s_w, N, K, 128, qW, qWt, s_u, ws(det.det_lsq_quantize_weight_ws_bytes(N, K)))
+    Y, qX, status = empty((M, N), np.uint16), empty((M, K), np.int8), torch.zeros(1, dtype=torch.int32, device="cuda")
+    det.det_linear_fwd(dX_, qW, s_x, s_w, M, N, K, Y, qX, status)
+    gX, gW, gs = empty((M, K), np.uint16), empty((N, K), F), empty((1,), F)
+    det.det_linear_bwd(dev(dY), dX_, qX, dW_, qWt, s_x, s_w, s_u, M, N, K, 128, gX, gW, gs, ws(det.det_linear_bwd_ws_bytes(M, N, K)), status)
+    _sync()
+    assert int(status.item()) == 0
+    assert_same_bits(host(Y, np.uint16), oY, "Y")
+    assert_same_bits(host(gX, np.uint16), odX, "dX")
+    assert_same_bits(host(gW), odW, "dW")
+    assert_same_bits(host(gs), ods, "ds_x")
