@@ -101,7 +101,7 @@ class Replay:
         self.specs = param_specs(cfg)
         D, Fh, V, L, T = cfg.d_model, cfg.ffn, cfg.vocab, cfg.n_layers, cfg.tokens_per_microbatch
         assert D == cfg.n_heads * 128, "head_dim is 128"
-        self.goff, self.poff = {}, {}
+        self.goff, self.poff, self._views = {}, {}, {}
         self.shape = dict((n, sh) for n, sh, _ in self.specs)
         g = p = 0
         for name, shape, kind in self.specs:
@@ -123,7 +123,7 @@ class Replay:
         self.lin = {}
         for l in range(L):
             for w, (N, K) in zip(LINEARS, ((cfg.qkv_width, D), (D, D), (2 * Fh, D), (D, Fh))):
-                self.lin[(l, w)] = dict(N=N, K=K, s_w=z(N, F32), qW=z(N * K, I8), qWt=z(N * K, I8), s_u=z(1, F32))
+                self.lin[(l, w)] = dict(name="l%d.%s" % (l, w), N=N, K=K, s_w=z(N, F32), qW=z(N * K, I8), qWt=z(N * K, I8), s_u=z(1, F32))
         e = lambda n, dt: torch.empty(n, dtype=dt, device=device)
         QW, Hkv = cfg.qkv_width, cfg.kv_heads
         self.head_ops = cfg.qk_norm or cfg.rope_tables is not None
@@ -185,16 +185,29 @@ class Replay:
         return {k: (len(v), sum(a.elapsed_time(b) for a, b in v)) for k, v in (self.prof or {}).items()}
 
     # ---- parameter access ------------------------------------------------------------------------------
+    def _view(self, which, name):
+        """The part of the buffer self.<which> that belongs to one parameter, sliced once per buffer."""
+        buf = getattr(self, which)
+        cache = self._views.get(which)
+        if cache is None or cache[0] is not buf:
+            cache = self._views[which] = (buf, {})
+        v = cache[1].get(name)
+        if v is None:
+            if which == "sx":
+                lo, n = 4 * int(name.split(".")[0][1:]), 4
+            else:
+                lo, n = (self.poff if which == "pbf" else self.goff)[name], _numel(self.shape[name])
+            v = cache[1][name] = buf[lo:lo + n]
+        return v
+
     def p(self, name):
-        shape = self.shape[name]
-        if name.endswith("s_x"):
-            l = int(name.split(".")[0][1:])
-            return self.sx[4 * l:4 * l + 4]
-        return self.pbf[self.poff[name]:self.poff[name] + _numel(shape)]
+        return self._view("sx" if name.endswith("s_x") else "pbf", name)
 
     def g(self, buf, name):
-        shape = self.shape[name]
-        return buf[self.goff[name]:self.goff[name] + _numel(shape)]
+        for which in ("gmb", "gout", "m", "v"):
+            if buf is getattr(self, which):
+                return self._view(which, name)
+        return buf[self.goff[name]:self.goff[name] + _numel(self.shape[name])]
 
     def load_params(self, params):
         """params: dict name -> numpy (uint16 bf16 bits, float32 steps)."""
@@ -246,7 +259,7 @@ class Replay:
         """Start of an optimizer step: re-pin every weight step from the current weights and quantise."""
         hb = self.cfg.hadamard_block
         for (l, w), d in self.lin.items():
-            W = self.p("l%d.%s" % (l, w))
+            W = self.p(d["name"])
             det.det_lsq_weight_scale(W, d["N"], d["K"], 0, d["s_w"], self.ws)
             det.det_lsq_quantize_weight(W, d["s_w"], d["N"], d["K"], hb, d["qW"], d["qWt"], d["s_u"], self.ws)
 
@@ -336,7 +349,7 @@ class Replay:
 
     def _linear_bwd(self, l, w, idx, dY, X, qx, M, dX):
         d = self.lin[(l, w)]
-        name = "l%d.%s" % (l, w)
+        name = d["name"]
         sx = self.sx[4 * l + idx:4 * l + idx + 1]
         ds = self.g(self.gmb, "l%d.s_x" % l)[idx:idx + 1]
         with self.span("linear_bwd"):
