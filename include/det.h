@@ -154,6 +154,15 @@ size_t det_rmsnorm_bwd_ws_bytes(int rows, int D);
 int det_rmsnorm_bwd(int io, const void* dy, const void* x, const void* gamma, const float* rstd, int rows, int D,
                     void* dx, float* dgamma, void* ws, size_t ws_bytes, void* stream);
 
+/* The norms with the residual stream beside them, bf16, D <= 2048; every output has the bits of the two calls:
+ *   det_residual_rmsnorm_fwd = det_residual_add(a, b -> sum), then det_rmsnorm_fwd of sum (with qy also det_rmsnorm_fwd_q's codes;
+ *     s_q / qy may be NULL).  sum and y overlap neither a nor b.
+ *   det_rmsnorm_bwd_residual = det_rmsnorm_bwd, then det_residual_add(res, its dx -> dx).  dx may be res. */
+int det_residual_rmsnorm_fwd(const det_bf16* a, const det_bf16* b, const det_bf16* gamma, int rows, int D, float eps,
+                             det_bf16* sum, det_bf16* y, float* rstd, const float* s_q, int8_t* qy, void* stream);
+int det_rmsnorm_bwd_residual(const det_bf16* dy, const det_bf16* x, const det_bf16* gamma, const float* rstd, int rows, int D,
+                             const det_bf16* res, det_bf16* dx, float* dgamma, void* ws, size_t ws_bytes, void* stream);
+
 /* ---- per-head operations of the attention block (Sec. 3.1 "QK-norm", "RoPE") --------------------------
  * Rows of 128 values (one head of one token) inside wider token rows: element (t, h, i) of x sits at
  * x[t*ld + h*128 + i]; ld, ld_y, ... are row strides in elements (multiples of 4, >= nh*128); pointers 8-byte

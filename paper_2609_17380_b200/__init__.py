@@ -64,7 +64,7 @@ _SIGNATURES = {
     "det_grad_accum_result": "ippp", "det_adamw_step": "ipippppzp", "det_adamw_batch": "ipppppppipp",
     "det_tensor_hash_ws_bytes": "zz", "det_tensor_hash_async": "ipzppzp", "det_tensor_hash": "ipzppzp",
     "det_tensor_hash_batch_ws_bytes": "zpi", "det_tensor_hash_batch": "ippippzp", "det_test_prim": "iipppzp",
-    "det_test_igemm_tn": "ippiiipipp", "det_test_wait_timeout": "iplp",
+    "det_residual_rmsnorm_fwd": "ipppiifpppppp", "det_rmsnorm_bwd_residual": "ippppiippppzp", "det_test_igemm_tn": "ippiiipipp", "det_test_wait_timeout": "iplp",
 }
 
 _lib = None
@@ -226,6 +226,11 @@ def det_rmsnorm_fwd_q(x, gamma, rows, D, eps, y, rstd, s_q, qy):
                                                          _ptr(y), _ptr(rstd), _ptr(s_q), _ptr(qy), _stream()))
 
 
+def det_residual_rmsnorm_fwd(a, b, gamma, rows, D, eps, sum_out, y, rstd, s_q=None, qy=None):
+    _check("det_residual_rmsnorm_fwd", load().det_residual_rmsnorm_fwd(_ptr(a), _ptr(b), _ptr(gamma), rows, D, eps, _ptr(sum_out), _ptr(y),
+                                                                       _ptr(rstd), _ptr(s_q), _ptr(qy), _stream()))
+
+
 def det_headnorm_fwd(x, ld, T, nh, eps, y, ld_y, rstd):
     _check("det_headnorm_fwd", load().det_headnorm_fwd(_ptr(x), ld, T, nh, eps, _ptr(y),
                                                        ld_y, _ptr(rstd), _stream()))
@@ -248,6 +253,11 @@ def det_rmsnorm_bwd_ws_bytes(rows, D):
 def det_rmsnorm_bwd(io, dy, x, gamma, rstd, rows, D, dx, dgamma, ws):
     _check("det_rmsnorm_bwd", load().det_rmsnorm_bwd(io, _ptr(dy), _ptr(x), _ptr(gamma), _ptr(rstd), rows,
                                                      D, _ptr(dx), _ptr(dgamma), *_ws(ws), _stream()))
+
+
+def det_rmsnorm_bwd_residual(dy, x, gamma, rstd, rows, D, res, dx, dgamma, ws):
+    _check("det_rmsnorm_bwd_residual", load().det_rmsnorm_bwd_residual(_ptr(dy), _ptr(x), _ptr(gamma), _ptr(rstd), rows, D, _ptr(res),
+                                                                       _ptr(dx), _ptr(dgamma), *_ws(ws), _stream()))
 
 
 def det_xent_ws_bytes(rows, V):

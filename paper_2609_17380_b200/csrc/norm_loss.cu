@@ -42,7 +42,8 @@ template <bool BF>
 __global__ void __launch_bounds__(256, 4) k_rmsnorm_fwd8(const void* __restrict__ x, const void* __restrict__ gamma, int rows,
                                                          int D, float eps, float invD, void* __restrict__ y,
                                                          float* __restrict__ rstd, const float* __restrict__ s_q = nullptr,
-                                                         int8_t* __restrict__ qy = nullptr) {
+                                                         int8_t* __restrict__ qy = nullptr, const void* __restrict__ res = nullptr,
+                                                         void* __restrict__ sum = nullptr) {
   __shared__ float leaf_sum[2][4][8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int e0 = warp * 256 + lane * 8;
@@ -60,6 +61,20 @@ __global__ void __launch_bounds__(256, 4) k_rmsnorm_fwd8(const void* __restrict_
       else {
 #pragma unroll
         for (int t = 0; t < 8; ++t) xr[a][t] = 0.0f;
+      }
+    }
+    if (BF && res) {   // the residual sum in front of the norm: x + res, rounded and stored, is what is normalised
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const long long row = r0 + 4 * pass + a;
+        if (row >= rows || !have) continue;
+        float b[8];
+        load8<BF>(res, (size_t)row * D + e0, b);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) xr[a][t] = fadd(xr[a][t], b[t]);
+        store8<BF>(sum, (size_t)row * D + e0, xr[a]);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) xr[a][t] = bf2f(f2bf(xr[a][t]));
       }
     }
 #pragma unroll
@@ -116,7 +131,7 @@ __global__ void __launch_bounds__(256, 4) k_rmsnorm_fwd8(const void* __restrict_
 template <bool BF, bool DG>
 __global__ void __launch_bounds__(256, 3) k_rmsnorm_bwd8(const void* __restrict__ dy, const void* __restrict__ x,
                                                         const void* __restrict__ gamma, const float* __restrict__ rstd,
-                                                        int rows, int D, float invD, void* __restrict__ dx,
+                                                        int rows, int D, float invD, void* dx, const void* res,
                                                         float* __restrict__ partial8, int* __restrict__ tickets) {
   constexpr int RPP = BF ? 4 : 2, NPASS = 8 / RPP;
   __shared__ float leaf_sum[2][RPP][8];
@@ -198,6 +213,12 @@ __global__ void __launch_bounds__(256, 3) k_rmsnorm_bwd8(const void* __restrict_
         float o[8];
 #pragma unroll
         for (int t = 0; t < 8; ++t) o[t] = fmul(rs[a], fsub(w[a][t], fmul(xh[a][t], c)));
+        if (BF && res) {   // the gradient that bypasses the norm, added to the rounded one (res may be dx)
+          float b[8];
+          load8<BF>(res, (size_t)row * D + e0, b);
+#pragma unroll
+          for (int t = 0; t < 8; ++t) o[t] = fadd(b[t], bf2f(f2bf(o[t])));
+        }
         store8<BF>(dx, (size_t)row * D + e0, o);
       }
     }
@@ -626,16 +647,16 @@ extern "C" size_t det_rmsnorm_bwd_ws_bytes(int rows, int D) {
 
 template <bool BF>
 static int rmsnorm_bwd8_launch(const void* dy, const void* x, const void* gamma, const float* rstd, int rows, int D,
-                               float invD, void* dx, float* dgamma, float* ws, cudaStream_t st) {
+                               float invD, void* dx, const void* res, float* dgamma, float* ws, cudaStream_t st) {
   const int nb8 = (rows + 7) / 8, nb256 = (rows + 255) / 256;
   if (!dgamma) {
-    k_rmsnorm_bwd8<BF, false><<<DET_L(nb8), 256, 0, st>>>(dy, x, gamma, rstd, rows, D, invD, dx, nullptr, nullptr);
+    k_rmsnorm_bwd8<BF, false><<<DET_L(nb8), 256, 0, st>>>(dy, x, gamma, rstd, rows, D, invD, dx, res, nullptr, nullptr);
     return DET_OK;
   }
   float* partial8 = ws;
   float* partial256 = ws + align_up((size_t)nb8 * D, 64);
   int* tickets = reinterpret_cast<int*>(partial256 + align_up((size_t)nb256 * D, 64));   // one per block of 256 columns (<= 8)
-  k_rmsnorm_bwd8<BF, true><<<DET_L(nb8), 256, 0, st>>>(dy, x, gamma, rstd, rows, D, invD, dx, partial8, tickets);
+  k_rmsnorm_bwd8<BF, true><<<DET_L(nb8), 256, 0, st>>>(dy, x, gamma, rstd, rows, D, invD, dx, res, partial8, tickets);
   // the second launch overlaps its start-up with the first kernel's tail (programmatic dependent launch); the kernel
   // itself waits for the first grid to complete before it reads anything
   cudaLaunchConfig_t cfg = {};
@@ -669,8 +690,8 @@ extern "C" int det_rmsnorm_bwd(int io, const void* dy, const void* x, const void
   }
   const float invD = (float)(1.0 / (double)D);
   if (D <= 2048) {
-    int rc = (io == DET_BF16) ? rmsnorm_bwd8_launch<true>(dy, x, gamma, rstd, rows, D, invD, dx, dgamma, (float*)ws, st)
-                              : rmsnorm_bwd8_launch<false>(dy, x, gamma, rstd, rows, D, invD, dx, dgamma, (float*)ws, st);
+    int rc = (io == DET_BF16) ? rmsnorm_bwd8_launch<true>(dy, x, gamma, rstd, rows, D, invD, dx, nullptr, dgamma, (float*)ws, st)
+                              : rmsnorm_bwd8_launch<false>(dy, x, gamma, rstd, rows, D, invD, dx, nullptr, dgamma, (float*)ws, st);
     if (rc != DET_OK) return rc;
     DET_CHECK_LAUNCH();
     return DET_OK;
@@ -685,6 +706,36 @@ extern "C" int det_rmsnorm_bwd(int io, const void* dy, const void* x, const void
     else k_dgamma_partial<false><<<DET_L(g2), 256, 0, st>>>(dy, x, rstd, rows, D, (float*)ws);
     k_col_tree<<<DET_L((D + 127) / 128), 128, 0, st>>>((float*)ws, nb, D, dgamma, rows);
   }
+  DET_CHECK_LAUNCH();
+  return DET_OK;
+}
+
+extern "C" int det_residual_rmsnorm_fwd(const det_bf16* a, const det_bf16* b, const det_bf16* gamma, int rows, int D, float eps,
+                                        det_bf16* sum, det_bf16* y, float* rstd, const float* s_q, int8_t* qy, void* stream) {
+  if (!a || !b || !sum || !y || !rstd || (qy && !s_q) || rows < 0 || D <= 0) return DET_ERR_ARG;
+  if (D % 8 || D > 2048) return DET_ERR_SHAPE;
+  if (!aligned16(a) || !aligned16(b) || !aligned16(sum) || !aligned16(y) || (gamma && !aligned16(gamma)) || (((uintptr_t)qy) & 7u))
+    return DET_ERR_ALIGN;
+  if (rows == 0) return DET_OK;
+  k_rmsnorm_fwd8<true><<<DET_L((rows + 7) / 8), 256, 0, (cudaStream_t)stream>>>(a, gamma, rows, D, eps, (float)(1.0 / (double)D), y,
+                                                                              rstd, s_q, qy, b, sum);
+  DET_CHECK_LAUNCH();
+  return DET_OK;
+}
+
+extern "C" int det_rmsnorm_bwd_residual(const det_bf16* dy, const det_bf16* x, const det_bf16* gamma, const float* rstd, int rows,
+                                        int D, const det_bf16* res, det_bf16* dx, float* dgamma, void* ws, size_t ws_bytes, void* stream) {
+  if (!dy || !x || !rstd || !res || !dx || rows < 0 || D <= 0) return DET_ERR_ARG;
+  if (D % 8 || D > 2048) return DET_ERR_SHAPE;
+  if (!aligned16(x) || !aligned16(dy) || !aligned16(res) || !aligned16(dx) || (gamma && !aligned16(gamma))) return DET_ERR_ALIGN;
+  if (dgamma && (!ws || !aligned16(ws) || ws_bytes < det_rmsnorm_bwd_ws_bytes(rows, D))) return DET_ERR_WORKSPACE;
+  cudaStream_t st = (cudaStream_t)stream;
+  if (rows == 0) {
+    if (dgamma) cudaMemsetAsync(dgamma, 0, (size_t)D * sizeof(float), st);
+    return DET_OK;
+  }
+  int rc = rmsnorm_bwd8_launch<true>(dy, x, gamma, rstd, rows, D, (float)(1.0 / (double)D), dx, res, dgamma, (float*)ws, st);
+  if (rc != DET_OK) return rc;
   DET_CHECK_LAUNCH();
   return DET_OK;
 }

@@ -114,6 +114,7 @@ class Replay:
         z = lambda n, dt: torch.zeros(n, dtype=dt, device=device)
         self.pbf = z(p, I16)                       # bf16 parameters (bit patterns), canonical order
         self.sx = z(L * 4, F32)                    # LSQ activation steps, [layer, (qkv, o, gu, down)]
+        self._sx = [[self.sx[4 * l + i:4 * l + i + 1] for i in range(4)] for l in range(L)]
         self.m, self.v = z(g, F32), z(g, F32)      # Adam moments, gradient layout
         self.gmb = z(g, F32)                       # gradient of the current micro-batch
         self.gout_padded = z(max(g, gout_len or 0), F32)
@@ -266,7 +267,7 @@ class Replay:
     def _linear(self, l, w, idx, X, M, Y, qx, calibrate, prequantised=False):
         """prequantised: the kernel that produced X already wrote its int8 codes into qx."""
         d = self.lin[(l, w)]
-        sx = self.sx[4 * l + idx:4 * l + idx + 1]
+        sx = self._sx[l][idx]
         if calibrate:
             det.det_lsq_act_scale_init(X, M * d["K"], sx, self.ws)
         with self.span("linear_fwd"):
@@ -275,30 +276,51 @@ class Replay:
             else:
                 det.det_linear_fwd(X, d["qW"], sx, d["s_w"], M, d["N"], d["K"], Y, qx, self.status)
 
+    def _norm(self, a, b, x, gain, y, rstd, s_q=None, qy=None):
+        """y = RMSNorm of x, after x = a + b unless a is None; with s_q the next linear's int8 input too."""
+        T, D = self.cfg.tokens_per_microbatch, self.cfg.d_model
+        g = self.p(gain)
+        if a is not None and D <= 2048:
+            det.det_residual_rmsnorm_fwd(a, b, g, T, D, 1e-6, x, y, rstd, s_q, qy if s_q is not None else None)
+            return
+        if a is not None:
+            det.det_residual_add(a, b, T * D, x)
+        if s_q is not None:
+            det.det_rmsnorm_fwd_q(x, g, T, D, 1e-6, y, rstd, s_q, qy)
+        else:
+            det.det_rmsnorm_fwd(det.DET_BF16, x, g, T, D, 1e-6, y, rstd)
+
+    def _norm_bwd(self, dy, x, gain, rstd, dx, tmp):
+        """dx += gradient through the norm (rounded on its own first); the gain's gradient goes to its place."""
+        T, D = self.cfg.tokens_per_microbatch, self.cfg.d_model
+        g, dg = self.p(gain), self.g(self.gmb, gain)
+        if D <= 2048:
+            det.det_rmsnorm_bwd_residual(dy, x, g, rstd, T, D, dx, dx, dg, self.ws)
+            return
+        det.det_rmsnorm_bwd(det.DET_BF16, dy, x, g, rstd, T, D, tmp, dg, self.ws)
+        det.det_residual_add(dx, tmp, T * D, dx)
+
     def forward(self, tokens_mb, calibrate=False):
         cfg = self.cfg
         D, Fh, V, L, T = cfg.d_model, cfg.ffn, cfg.vocab, cfg.n_layers, cfg.tokens_per_microbatch
         B, H, S = cfg.micro_batch, cfg.n_heads, cfg.seq
         self.tok.copy_(tokens_mb[:, :-1].reshape(-1))
         self.lab.copy_(tokens_mb[:, 1:].reshape(-1))
-        x = self.tmp[0][:T * D]
         Hkv, QW = cfg.kv_heads, cfg.qkv_width
+        x = self.act[0]["x"] if L else self.xf
         if cfg.embed_norm:
             det.det_embed_fwd(self.tok, T, self.p("embed"), V, D, self.x_emb)
             det.det_rmsnorm_fwd(det.DET_BF16, self.x_emb, self.p("embed_norm"), T, D, 1e-6, x, self.rstd_emb)
         else:
             det.det_embed_fwd(self.tok, T, self.p("embed"), V, D, x)
+        # outside the calibration pass every activation step is known before its activation is produced, so the
+        # producers write the next linear's int8 input themselves (same bits as the separate quantiser pass)
+        fuse = self.fuse_quant and not calibrate and D <= 2048
+        dn, res = self.tmp[1][:T * D], None           # the residual sum that ends a layer runs with the norm that starts the next
         for l in range(L):
             a = self.act[l]
-            a["x"].copy_(x)
-            # outside the calibration pass every activation step is known before its activation is produced, so the
-            # producers write the next linear's int8 input themselves (same bits as the separate quantiser pass)
-            fuse = self.fuse_quant and not calibrate and D <= 2048
-            sxl = self.sx[4 * l:4 * l + 4]
-            if fuse:
-                det.det_rmsnorm_fwd_q(a["x"], self.p("l%d.attn_norm" % l), T, D, 1e-6, a["n1"], a["rstd1"], sxl[0:1], a["qx_qkv"])
-            else:
-                det.det_rmsnorm_fwd(det.DET_BF16, a["x"], self.p("l%d.attn_norm" % l), T, D, 1e-6, a["n1"], a["rstd1"])
+            sxl = self._sx[l]
+            self._norm(res, dn, a["x"], "l%d.attn_norm" % l, a["n1"], a["rstd1"], sxl[0] if fuse else None, a["qx_qkv"])
             self._linear(l, "w_qkv", 0, a["n1"], T, a["qkv"], a["qx_qkv"], calibrate, fuse)
             qp = vp = a["qkv"].data_ptr()
             if self.head_ops:
@@ -316,28 +338,22 @@ class Replay:
                     det.det_attn_fwd_int8pv(qp, qp + 2 * D, vp + 2 * (D + 128 * Hkv), QW, B, H, S, a["att"], D, a["lse"],
                                             self.status, Hkv=Hkv, window=cfg.layer_window(l))
                 elif fuse:
-                    det.det_attn_fwd_q(qp, qp + 2 * D, vp + 2 * (D + 128 * Hkv), QW, B, H, S, a["att"], D, a["lse"], sxl[1:2],
+                    det.det_attn_fwd_q(qp, qp + 2 * D, vp + 2 * (D + 128 * Hkv), QW, B, H, S, a["att"], D, a["lse"], sxl[1],
                                        a["qx_o"], Hkv=Hkv, window=cfg.layer_window(l))
                 else:
                     det.det_attn_fwd(qp, qp + 2 * D, vp + 2 * (D + 128 * Hkv), QW, B, H, S, a["att"], D, a["lse"], Hkv=Hkv,
                                      window=cfg.layer_window(l))
             o = self.tmp[1][:T * D]
             self._linear(l, "w_o", 1, a["att"], T, o, a["qx_o"], calibrate, fuse and not cfg.pv_int8)
-            det.det_residual_add(a["x"], o, T * D, a["h"])
-            if fuse:
-                det.det_rmsnorm_fwd_q(a["h"], self.p("l%d.ffn_norm" % l), T, D, 1e-6, a["n2"], a["rstd2"], sxl[2:3], a["qx_gu"])
-            else:
-                det.det_rmsnorm_fwd(det.DET_BF16, a["h"], self.p("l%d.ffn_norm" % l), T, D, 1e-6, a["n2"], a["rstd2"])
+            self._norm(a["x"], o, a["h"], "l%d.ffn_norm" % l, a["n2"], a["rstd2"], sxl[2] if fuse else None, a["qx_gu"])
             self._linear(l, "w_gu", 2, a["n2"], T, a["gu"], a["qx_gu"], calibrate, fuse)
             if fuse:
-                det.det_swiglu_fwd_q(a["gu"], T, Fh, a["a"], sxl[3:4], a["qx_down"])
+                det.det_swiglu_fwd_q(a["gu"], T, Fh, a["a"], sxl[3], a["qx_down"])
             else:
                 det.det_swiglu_fwd(a["gu"], T, Fh, a["a"])
-            dn = self.tmp[1][:T * D]
             self._linear(l, "w_down", 3, a["a"], T, dn, a["qx_down"], calibrate, fuse)
-            det.det_residual_add(a["h"], dn, T * D, x)
-        self.xf.copy_(x)
-        det.det_rmsnorm_fwd(det.DET_BF16, self.xf, self.p("final_norm"), T, D, 1e-6, self.nf, self.rstdf)
+            res = a["h"]
+        self._norm(res, dn, self.xf, "final_norm", self.nf, self.rstdf)
         with self.span("lmhead_fwd"):
             if cfg.arith == 2:
                 det.det_lmhead_fwd_v2(self.nf, self.p("lm_head"), T, V, D, self.logits, self.ws, self.status)
@@ -350,7 +366,7 @@ class Replay:
     def _linear_bwd(self, l, w, idx, dY, X, qx, M, dX):
         d = self.lin[(l, w)]
         name = d["name"]
-        sx = self.sx[4 * l + idx:4 * l + idx + 1]
+        sx = self._sx[l][idx]
         ds = self.g(self.gmb, "l%d.s_x" % l)[idx:idx + 1]
         with self.span("linear_bwd"):
             det.det_linear_bwd(dY, X, qx, self.p(name), d["qWt"], sx, d["s_w"], d["s_u"], M, d["N"], d["K"],
@@ -381,13 +397,9 @@ class Replay:
             det.det_swiglu_bwd(d_a, a["gu"], T, Fh, d_gu)
             d_n2 = t0[:T * D]
             self._linear_bwd(l, "w_gu", 2, d_gu, a["n2"], a["qx_gu"], T, d_n2)
-            d_h2 = t2[:T * D]
-            det.det_rmsnorm_bwd(det.DET_BF16, d_n2, a["h"], self.p("l%d.ffn_norm" % l), a["rstd2"], T, D, d_h2,
-                                self.g(self.gmb, "l%d.ffn_norm" % l), self.ws)
-            d_h = t1[:T * D]
-            det.det_residual_add(dx, d_h2, T * D, d_h)            # in place over dx
+            self._norm_bwd(d_n2, a["h"], "l%d.ffn_norm" % l, a["rstd2"], dx, t2[:T * D])      # dx: gradient of h from here on
             d_att = t0[:T * D]
-            self._linear_bwd(l, "w_o", 1, d_h, a["att"], a["qx_o"], T, d_att)
+            self._linear_bwd(l, "w_o", 1, dx, a["att"], a["qx_o"], T, d_att)
             Hkv, QW = cfg.kv_heads, cfg.qkv_width
             d_qkv = t2[:T * QW]
             vp, dp = a["qkv"].data_ptr(), d_qkv.data_ptr()
@@ -402,10 +414,7 @@ class Replay:
                 det.det_headnorm_bwd(d_qkv, QW, a["qkv"], QW, a["rstd_qk"], T, H + Hkv, d_qkv, QW)
             d_n1 = t0[:T * D]
             self._linear_bwd(l, "w_qkv", 0, d_qkv, a["n1"], a["qx_qkv"], T, d_n1)
-            d_x1 = t2[:T * D]
-            det.det_rmsnorm_bwd(det.DET_BF16, d_n1, a["x"], self.p("l%d.attn_norm" % l), a["rstd1"], T, D, d_x1,
-                                self.g(self.gmb, "l%d.attn_norm" % l), self.ws)
-            det.det_residual_add(d_h, d_x1, T * D, dx)            # dx aliases d_h: in place
+            self._norm_bwd(d_n1, a["x"], "l%d.attn_norm" % l, a["rstd1"], dx, t2[:T * D])     # and of x
         if cfg.embed_norm:
             d_emb = t0[:T * D]
             det.det_rmsnorm_bwd(det.DET_BF16, dx, self.x_emb, self.p("embed_norm"), self.rstd_emb, T, D, d_emb,

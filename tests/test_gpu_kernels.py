@@ -174,3 +174,27 @@ def test_linear_tiles(det, M, N, K):
     assert_same_bits(host(gX, np.uint16), odX, "dX")
     assert_same_bits(host(gW), odW, "dW")
     assert_same_bits(host(gs), ods, "ds_x")
+
+
+# the norms with the residual stream beside them: rows off the block of eight, D off the leaf of 256, with and without codes
+@pytest.mark.parametrize("rows,D,q", [(1, 8, True), (13, 1000, False), (300, 2048, True), (64, 384, True)])
+def test_norms_with_residual(det, rows, D, q):
+    a, b, dy, res = [synth.normal_bf16((rows, D), 1.0, seed=rows, tid=t) for t in range(4)]
+    gain = synth.normal_bf16((D,), 0.1, mean=1.0, seed=rows, tid=9)
+    s = np.array([0.03], F)
+    h, y, rstd, qy = empty((rows, D), np.uint16), empty((rows, D), np.uint16), empty((rows,), F), empty((rows, D), np.int8)
+    det.det_residual_rmsnorm_fwd(dev(a), dev(b), dev(gain), rows, D, 1e-6, h, y, rstd, dev(s) if q else None, qy if q else None)
+    _sync()
+    ho = oracle.residual_add(a, b)
+    yo, ro = oracle.rmsnorm_fwd(ho, gain, 1e-6, bf=True)
+    assert_same_bits(host(h, np.uint16), ho, "sum")
+    assert_same_bits(host(y, np.uint16), yo, "y")
+    assert_same_bits(host(rstd), ro.reshape(-1), "rstd")
+    if q:
+        assert_same_bits(host(qy).reshape(-1), np.asarray(oracle.lsq_quantize(yo, s, False)).reshape(-1).view(np.int8), "codes")
+    dx, dg = dev(res), empty((D,), F)
+    det.det_rmsnorm_bwd_residual(dev(dy), dev(ho), dev(gain), rstd, rows, D, dx, dx, dg, ws(det.det_rmsnorm_bwd_ws_bytes(rows, D)))
+    _sync()
+    dxo, dgo = oracle.rmsnorm_bwd(dy, ho, gain, ro, bf=True)
+    assert_same_bits(host(dx, np.uint16), oracle.residual_add(res, dxo), "dx")
+    assert_same_bits(host(dg), dgo.reshape(-1), "dgain")
