@@ -190,17 +190,17 @@ struct ResultOp {
   float inv_rep;
   float* dst;
 };
-__global__ void __launch_bounds__(256) k_accum_result(ResultOp op, size_t n) {
+// The parameter struct stays in constant space and the loop runs over the partials there are: unrolled to the 34 there may be,
+// the 33 tests per thread held the pass at 3.1 TB/s (RESRATE now).
+__global__ void __launch_bounds__(256) k_accum_result(const __grid_constant__ ResultOp op, size_t n) {
   size_t i = ((size_t)blockIdx.x * 256 + threadIdx.x) * 4;
   if (i >= n) return;
   float4 a = *reinterpret_cast<const float4*>(op.part[0] + i);
   float v[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-  for (int s = 1; s < 34; ++s) {
-    if (s < op.n) {
-      float4 t = *reinterpret_cast<const float4*>(op.part[s] + i);
-      v[0] = fadd(t.x, v[0]); v[1] = fadd(t.y, v[1]); v[2] = fadd(t.z, v[2]); v[3] = fadd(t.w, v[3]);
-    }
+#pragma unroll 1
+  for (int s = 1; s < op.n; ++s) {
+    float4 t = *reinterpret_cast<const float4*>(op.part[s] + i);
+    v[0] = fadd(t.x, v[0]); v[1] = fadd(t.y, v[1]); v[2] = fadd(t.z, v[2]); v[3] = fadd(t.w, v[3]);
   }
   *reinterpret_cast<float4*>(op.dst + i) =
       make_float4(fmul(v[0], op.inv_rep), fmul(v[1], op.inv_rep), fmul(v[2], op.inv_rep), fmul(v[3], op.inv_rep));
