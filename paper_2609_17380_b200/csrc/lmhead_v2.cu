@@ -8,7 +8,7 @@
 // hardware takes them, and the epilogue forms I = 2^14 hh + 2^7 (hl + lh) + ll in 64 bits and rounds I 2^(Ea + Eb - 280)
 // to binary32 ONCE.  Nothing about the result depends on tiling, order or hardware.
 //
-//   k_slice_rows   one warp per row: row exponent (integer maximum), then the two int8 slices
+//   k_slice_rows   one warp (or CTA) per row: row exponent (integer maximum), then the two int8 slices
 //   k_igemm_sl     persistent, one CTA per SM, 128 x 128 output tile; warp 0 streams the FOUR operand tiles of a 128-deep
 //                  step (H hi, H lo, W hi, W lo: 64 KiB) through a three-stage TMA ring, warp 1 issues the sixteen MMAs of
 //                  the step into three TMEM accumulators (hh | hl + lh | ll, 128 columns each), warps 2-5 combine and round.
@@ -33,29 +33,38 @@ __device__ __forceinline__ void load8_bits(const void* X, size_t idx, uint32_t (
     w[0] = u.x; w[1] = u.y; w[2] = u.z; w[3] = u.w;
   }
 }
-template <bool F32>
+// WPR warps per row: one, or the eight of a CTA where a row is long and the rows are few (one warp walks 32768 values twice at
+// the latency of its loads: 1024 rows of 32768 f32 values 0.163 ms, 0.059 with eight).
+template <bool F32, int WPR>
 __global__ void __launch_bounds__(256) k_slice_rows(const void* __restrict__ X, int R, int K, int8_t* __restrict__ hi,
                                                     int8_t* __restrict__ lo, int32_t* __restrict__ E) {
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  __shared__ int key_s[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row = WPR == 1 ? (int)blockIdx.x * 8 + warp : (int)blockIdx.x;
   if (row >= R) return;
-  int e = 0, bad = 0;
-  for (int i = lane; i < K / 8; i += 32) {
+  const int first = WPR == 1 ? lane : (int)threadIdx.x, n8 = K / 8;
+  int key = 0;                                       // exponent, bit 30: an infinity or a NaN
+#pragma unroll 4
+  for (int i = first; i < n8; i += 32 * WPR) {
     uint32_t w[4];
     load8_bits<F32>(X, (size_t)row * K + 8 * (size_t)i, w);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const int e0 = (w[j] >> 7) & 0xFF, e1 = (w[j] >> 23) & 0xFF;
-      bad |= (e0 == 255) | (e1 == 255);
-      e = max(e, max(e0, e1));
+      const int e0 = (w[j] >> 7) & 0xFF, e1 = (w[j] >> 23) & 0xFF, e = max(e0, e1);
+      key = max(key, e == 255 ? (255 | (1 << 30)) : e);
     }
   }
+  key = __reduce_max_sync(0xffffffffu, key);
+  if (WPR > 1) {
+    if (lane == 0) key_s[warp] = key;
+    __syncthreads();
 #pragma unroll
-  for (int s = 16; s; s >>= 1) {
-    e = max(e, __shfl_xor_sync(0xffffffffu, e, s));
-    bad |= __shfl_xor_sync(0xffffffffu, bad, s);
+    for (int w = 0; w < 8; ++w) key = max(key, key_s[w]);
   }
-  if (lane == 0) E[row] = e | (bad ? (1 << 30) : 0);
-  for (int i = lane; i < K / 8; i += 32) {
+  if (first == 0) E[row] = key;
+  const int e = key & 0xFF;
+#pragma unroll 2
+  for (int i = first; i < n8; i += 32 * WPR) {
     uint32_t w[4];
     load8_bits<F32>(X, (size_t)row * K + 8 * (size_t)i, w);
     uint32_t h8[2] = {0u, 0u}, l8[2] = {0u, 0u};
@@ -70,6 +79,12 @@ __global__ void __launch_bounds__(256) k_slice_rows(const void* __restrict__ X, 
     *reinterpret_cast<uint2*>(hi + (size_t)row * K + 8 * i) = make_uint2(h8[0], h8[1]);
     *reinterpret_cast<uint2*>(lo + (size_t)row * K + 8 * i) = make_uint2(l8[0], l8[1]);
   }
+}
+template <bool F32>
+static void slice_rows_launch(const void* X, int R, int K, int8_t* hi, int8_t* lo, int32_t* E, cudaStream_t st) {
+  // eight warps per row once a row holds a few rounds for each of them, unless a warp per row fills the GPU anyway
+  if (K >= 4096 && R < 64 * 4 * dev_sm_count()) k_slice_rows<F32, 8><<<DET_L(R), 256, 0, st>>>(X, R, K, hi, lo, E);
+  else k_slice_rows<F32, 1><<<DET_L((R + 7) / 8), 256, 0, st>>>(X, R, K, hi, lo, E);
 }
 
 // Slicing along the OTHER index, for the gradient contractions: the exponent of column c is taken over the rows r, and the
@@ -386,8 +401,8 @@ extern "C" int det_lmhead_fwd_v2(const det_bf16* H, const det_bf16* W, int M, in
   uint8_t* base = (uint8_t*)ws;
   int8_t *Ah = (int8_t*)(base + oAh), *Al = (int8_t*)(base + oAl), *Bh = (int8_t*)(base + oBh), *Bl = (int8_t*)(base + oBl);
   int32_t *Ea = (int32_t*)(base + oEa), *Eb = (int32_t*)(base + oEb);
-  k_slice_rows<false><<<DET_L((M + 7) / 8), 256, 0, st>>>(H, M, K, Ah, Al, Ea);
-  k_slice_rows<false><<<DET_L((V + 7) / 8), 256, 0, st>>>(W, V, K, Bh, Bl, Eb);
+  slice_rows_launch<false>(H, M, K, Ah, Al, Ea, st);
+  slice_rows_launch<false>(W, V, K, Bh, Bl, Eb, st);
   DET_CHECK_LAUNCH();
   return sliced_gemm<false>(Ah, Al, Bh, Bl, Ea, Eb, logits, M, V, K, status_dev, st);
 }
@@ -421,7 +436,7 @@ extern "C" int det_lmhead_bwd_v2(const float* dlogits, const det_bf16* H, const 
   int8_t *WTh = (int8_t*)(b + o[4]), *WTl = (int8_t*)(b + o[5]), *HTh = (int8_t*)(b + o[6]), *HTl = (int8_t*)(b + o[7]);
   int32_t *Eg = (int32_t*)(b + o[8]), *EgT = (int32_t*)(b + o[9]), *EWT = (int32_t*)(b + o[10]), *EHT = (int32_t*)(b + o[11]);
   cudaMemsetAsync(EgT, 0, o[11] - o[9] + align_up((size_t)K * 4, 256), st);        // the three column-exponent arrays
-  k_slice_rows<true><<<DET_L((M + 7) / 8), 256, 0, st>>>(dlogits, M, V, gh, gl, Eg);
+  slice_rows_launch<true>(dlogits, M, V, gh, gl, Eg, st);
   k_col_exp<true><<<DET_L(dim3(V / 128, M / 128)), 128, 0, st>>>(dlogits, M, V, EgT);
   k_col_exp<false><<<DET_L(dim3(K / 128, V / 128)), 128, 0, st>>>(W, V, K, EWT);
   k_col_exp<false><<<DET_L(dim3(K / 128, M / 128)), 128, 0, st>>>(H, M, K, EHT);

@@ -64,6 +64,26 @@ def test_lmhead_tiles(det, M, V, K):
     assert_same_bits(host(dW), dW_o, "dW")
 
 
+# version-2 gradients where a row of logits is long enough for eight warps (4096 values), and one step below
+@pytest.mark.parametrize("M,V,K", [(128, 3968, 128), (128, 4096, 128), (256, 8320, 128)])
+def test_lmhead_v2_long_rows(det, M, V, K):
+    import torch
+    from oracle import v2
+    H, W = synth.normal_bf16((M, K), 1.0, seed=V, tid=1), synth.normal_bf16((V, K), 0.05, seed=V, tid=2)
+    g = synth.normal_f32((M, V), 1e-3, seed=V, tid=3)
+    g[5, V - 1] = np.inf                                          # seen by one warp: its row of dH and its row of dW are NaN
+    dH, dW = empty((M, K), np.uint16), empty((V, K), F)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    det.det_lmhead_bwd_v2(dev(g), dev(H), dev(W), M, V, K, dH, dW, ws(det.det_lmhead_bwd_v2_ws_bytes(M, V, K)), status)
+    _sync()
+    assert int(status.item()) == 0
+    want_H, want_W = v2.lmhead_bwd(g, H, W)
+    got_H, got_W = host(dH, np.uint16), host(dW)
+    assert np.isnan(synth.from_bf16(got_H[5])).all() and np.isnan(got_W[V - 1]).all()
+    assert_same_bits(np.delete(got_H, 5, 0), np.delete(want_H, 5, 0), "version-2 dH")
+    assert_same_bits(got_W[:-1], want_W[:-1], "version-2 dW")
+
+
 # attention at head and row counts where the rows per CTA change (32, 64, 128 rows), S off the 128 grid, windows that start
 # and end inside a block, grouped heads (one accumulator over the whole group)
 @pytest.mark.parametrize("B,H,Hkv,S,W", [(1, 2, 2, 576, 0), (1, 40, 40, 320, 0), (2, 80, 80, 192, 0), (1, 3, 3, 704, 256),
