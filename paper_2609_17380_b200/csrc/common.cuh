@@ -250,13 +250,16 @@ __device__ __forceinline__ void smem_tree(float* buf, int n) {
 constexpr int SUM_CHUNK = 16384;
 // The sum of chunk `base` .. base + SUM_CHUNK of x[0..n): a perfect subtree, or the ragged last one with existence
 // predicates.  All 256 threads of the CTA call it; thread 0 gets the result.
+// The ragged form deals its leaves out over the warps (a sum of 2048 values has eight: one warp walking them behind scalar
+// loads took 7 us) and the first warp pairs the leaf sums.
+constexpr int SUM_LEAVES = SUM_CHUNK / 256;
 template <bool SQ>
-__device__ __forceinline__ float chunk_sum(const float* __restrict__ x, long long base, long long n, float (&wsum)[8]) {
+__device__ __forceinline__ float chunk_sum(const float* __restrict__ x, long long base, long long n, float (&leaf)[SUM_LEAVES]) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float s[8], r;
-  const bool full = base + SUM_CHUNK <= n;
-  if (full) {
+  const bool vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+  if (base + SUM_CHUNK <= n && vec) {
     float4 a[8], b[8];
+    float s[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const float4* p = reinterpret_cast<const float4*>(x + base + (warp * 8 + j) * 256 + lane * 8);
@@ -272,38 +275,43 @@ __device__ __forceinline__ float chunk_sum(const float* __restrict__ x, long lon
       }
       s[j] = warp_tree_full(tree8_full(v));
     }
-    r = fadd(fadd(fadd(s[0], s[1]), fadd(s[2], s[3])), fadd(fadd(s[4], s[5]), fadd(s[6], s[7])));
-  } else {
+    if (lane == 0) leaf[warp] = fadd(fadd(fadd(s[0], s[1]), fadd(s[2], s[3])), fadd(fadd(s[4], s[5]), fadd(s[6], s[7])));
+    __syncthreads();
+    return threadIdx.x ? 0.0f : fadd(fadd(fadd(leaf[0], leaf[1]), fadd(leaf[2], leaf[3])), fadd(fadd(leaf[4], leaf[5]), fadd(leaf[6], leaf[7])));
+  }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const long long lf = base + (warp * 8 + j) * 256;
-      const long long e0 = lf + lane * 8;
-      float v[8];
+  for (int h = 0; h < 2; ++h) {
+    float v[4][8];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        float u = (e0 + t < n) ? x[e0 + t] : 0.0f;
-        v[t] = SQ ? fmul(u, u) : u;
+    for (int j = 0; j < 4; ++j) {
+      const long long e0 = base + ((4 * h + j) * 8 + warp) * 256 + lane * 8;
+      if (vec && e0 + 8 <= n) {
+        const float4 p = __ldg(reinterpret_cast<const float4*>(x + e0)), q = __ldg(reinterpret_cast<const float4*>(x + e0) + 1);
+        v[j][0] = p.x; v[j][1] = p.y; v[j][2] = p.z; v[j][3] = p.w; v[j][4] = q.x; v[j][5] = q.y; v[j][6] = q.z; v[j][7] = q.w;
+      } else {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) v[j][t] = (e0 + t < n) ? x[e0 + t] : 0.0f;
       }
-      s[j] = lf < n ? warp_tree(tree8(v, e0, n), lf, 8, n) : 0.0f;
     }
-    r = reg_tree<8>(s, base + (long long)warp * 2048, 256, n);
-  }
-  if (lane == 0) wsum[warp] = r;
-  __syncthreads();
-  r = 0.0f;
-  if (threadIdx.x == 0) {
-    if (full) {
-      r = fadd(fadd(fadd(wsum[0], wsum[1]), fadd(wsum[2], wsum[3])), fadd(fadd(wsum[4], wsum[5]), fadd(wsum[6], wsum[7])));
-    } else {
-      float w[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) w[j] = wsum[j];
-      r = reg_tree<8>(w, base, 2048, n);
-      // a lone element is carried by the tree without any addition; flush it explicitly, as every value that enters or
-      // leaves an operation is flushed
-      if (n == 1 && !(__float_as_uint(r) & 0x7f800000u)) r = __uint_as_float(__float_as_uint(r) & 0x80000000u);
+    for (int j = 0; j < 4; ++j) {
+      const int l = (4 * h + j) * 8 + warp;
+      const long long lf = base + l * 256;
+      if (SQ) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) v[j][t] = fmul(v[j][t], v[j][t]);
+      }
+      const float s = lf < n ? warp_tree(tree8(v[j], lf + lane * 8, n), lf, 8, n) : 0.0f;
+      if (lane == 0) leaf[l] = s;
     }
   }
+  __syncthreads();
+  if (warp) return 0.0f;
+  float r = (base + (2 * lane + 1) * 256 < n) ? fadd(leaf[2 * lane], leaf[2 * lane + 1]) : leaf[2 * lane];
+  r = warp_tree(r, base, 512, n);
+  // a lone element is carried by the tree without any addition; flush it explicitly, as every value that enters or
+  // leaves an operation is flushed
+  if (n == 1 && !(__float_as_uint(r) & 0x7f800000u)) r = __uint_as_float(__float_as_uint(r) & 0x80000000u);
   return r;
 }
 

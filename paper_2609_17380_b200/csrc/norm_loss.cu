@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(XT) k_xent_fwd(const float* __restrict__ logit
 // the last levels of both sums (n <= SUM_CHUNK nodes each) and the means
 __global__ void __launch_bounds__(256) k_xent_finish(const float* __restrict__ ce, const float* __restrict__ zsq, int n, float inv_rows,
                                                      float z_weight, float* loss_mean, float* z_mean) {
-  __shared__ float wsum[8];
+  __shared__ float wsum[SUM_LEAVES];
   const float c = fmul(chunk_sum<false>(ce, 0, n, wsum), inv_rows);
   __syncthreads();
   const float zm = fmul(chunk_sum<false>(zsq, 0, n, wsum), inv_rows);

@@ -88,7 +88,7 @@ unsigned long long launches() { return g_launches.load(std::memory_order_relaxed
 
 template <bool SQ>
 __global__ void __launch_bounds__(256) k_sum_chunk(const float* __restrict__ x, long long n, float* __restrict__ partial) {
-  __shared__ float wsum[8];
+  __shared__ float wsum[SUM_LEAVES];
   const float r = chunk_sum<SQ>(x, (long long)blockIdx.x * SUM_CHUNK, n, wsum);
   if (threadIdx.x == 0) partial[blockIdx.x] = r;
 }
@@ -106,7 +106,7 @@ struct SumJobs {
 };
 template <bool SQ>
 __global__ void __launch_bounds__(256) k_sum_jobs(const __grid_constant__ SumJobs jobs, float* __restrict__ out, float* __restrict__ per) {
-  __shared__ float wsum[8];
+  __shared__ float wsum[SUM_LEAVES];
   int lo = 0, hi = jobs.n - 1;         // the last job whose first block is <= this one
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -153,7 +153,7 @@ int sum_launch(const float* x, size_t n, int squares, float* out, float* ws, cud
 
 // det_sum(x[0..n)), n <= SUM_CHUNK, times gs (the last levels of a sum and the scaling that follows it, in one launch)
 __global__ void __launch_bounds__(256) k_sum_scaled(const float* __restrict__ x, int n, float gs, float* __restrict__ out) {
-  __shared__ float wsum[8];
+  __shared__ float wsum[SUM_LEAVES];
   const float r = chunk_sum<false>(x, 0, n, wsum);
   if (threadIdx.x == 0) out[0] = fmul(gs, r);
 }
@@ -176,7 +176,7 @@ int sum_scaled_launch(const float* x, size_t n, float gs, float* out, float* ws,
 // the tree over the per-tensor sums (n <= SUM_CHUNK), the norm and the clip coefficient
 __global__ void __launch_bounds__(256) k_norm_finish(const float* __restrict__ per, int n, float max_norm, float* norm_out,
                                                      float* coef_out, int* status) {
-  __shared__ float wsum[8];
+  __shared__ float wsum[SUM_LEAVES];
   const float total = n ? chunk_sum<false>(per, 0, n, wsum) : 0.0f;
   if (threadIdx.x) return;
   float nrm = fsqrt(total);
