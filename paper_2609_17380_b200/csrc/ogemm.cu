@@ -42,7 +42,8 @@ extern "C" int det_lmhead_bwd(const float* dlogits, const det_bf16* H, const det
   cudaStream_t st = (cudaStream_t)stream;
   AuxScope aux(st);   // the auxiliary streams start where the caller's stream stands now; joined on every way out
   // dH[m,k] = sum over v ascending of bf16(dlogits[m,v]) * W[v,k]
-  int rc = ogemm_launch<CONTIG, STRIDED, true, true, 0>(plain_args(dlogits, W, dH, M, K, V, V, K, K, 0), 1, 1, st);
+  int rc = ogemm_launch<CONTIG, STRIDED, true, true, 0>(plain_args(dlogits, W, dH, M, K, V, V, K, K, 0), 1, 1, st,
+                                                    (double)M * V * K / OG_RATES[0].full);   // beside the weight gradient
   if (rc != DET_OK) return rc;
   // dW[v,k] (+)= sum over m ascending of bf16(dlogits[m,v]) * H[m,k], beside the first kernel
   rc = ogemm_launch<STRIDED, STRIDED, true, false, 0>(plain_args(dlogits, H, dW, V, K, M, V, K, K, first_chunk ? 0 : 1), 1, 1,

@@ -419,18 +419,20 @@ static int ogemm_run(const OgemmArgs& p, int batches, cudaStream_t st) {
 // of the larger bounds is taken.
 struct OgRate { int tm, tn; float alone, full; };     // cycles per step of a CTA alone on its SM; multiply-adds per cycle and SM of a full one
 constexpr OgRate OG_RATES[4] = {{128, 256, 311.0f, 106.0f}, {128, 128, 174.0f, 103.0f}, {64, 128, 110.0f, 89.0f}, {32, 64, 71.0f, 61.0f}};
-// share: how many such contractions run side by side
-static int og_pick(const OgemmArgs& p, int batches, int share, int widest) {
+// share: how many such contractions run side by side; beside: SM-cycles of other work that is queued to fill the SMs that a small
+// grid leaves idle (the head's two gradients at 384 tokens: 96 CTAs of 64 x 128 and the weight gradient on the other SMs,
+// head and loss forward and backward 4.34 ms; 384 CTAs of 32 x 64 on all of them and the weight gradient behind, 5.27 ms)
+static int og_pick(const OgemmArgs& p, int batches, int share, int widest, double beside) {
   const int sms = dev_sm_count() > 0 ? dev_sm_count() : 1;
   int best = widest;
   double best_t = 0.0;
   for (int c = widest; c < 4; ++c) {
     const OgRate r = OG_RATES[c];
     const double ni = (p.I + r.tm - 1) / r.tm, nj = (p.J + r.tn - 1) / r.tn;
+    const double tiles = ni * nj * batches;
     double longest, total;           // steps of the contraction: of one tile, and summed over the tiles
     if (p.range_mode == 0) {
       longest = p.C;
-      const double tiles = ni * nj * batches;
       const long long rounds = ((long long)tiles + sms - 1) / sms;
       total = tiles > sms ? (double)rounds * sms * p.C : tiles * p.C;     // tiles of equal length: whole rounds
     } else {
@@ -443,7 +445,8 @@ static int og_pick(const OgemmArgs& p, int batches, int share, int widest) {
     const double a = longest * p.nG * r.alone, b = share * total * p.nG * r.tm * r.tn / (r.full * sms);
     // the last chains of a causal grid run beside idle SMs: half a chain, on average (three contractions side by side, 16 heads
     // on 4 x 4096: 4.36 ms for the backward with square tiles, 4.07 with half ones; 16 x 16 heads x 2048: 3.43 and 3.56)
-    const double full = p.range_mode ? b + 0.5 * a : b, t = a > full ? a : full;
+    const double full = p.range_mode ? b + 0.5 * a : b, alone = a > full ? a : full;
+    const double busy = tiles <= sms ? tiles * a : alone * sms, t = (busy + beside) / sms > alone ? (busy + beside) / sms : alone;
     if (c == widest || t < (p.range_mode ? 1.0 : 0.95) * best_t) { best = c; best_t = t; }
   }
   return best;
@@ -452,8 +455,8 @@ template <int WIDEST> struct OgFirst { typedef OgWide T; };
 template <> struct OgFirst<1> { typedef OgSquare T; };
 // WIDEST: 0, or 1 where the output has no 256 columns (the head dimension of the attention contractions is 128)
 template <int AMODE, int BMODE, bool AF32, bool OUT_BF16, int WIDEST>
-static int ogemm_launch(const OgemmArgs& p, int batches, int share, cudaStream_t st) {
-  switch (og_pick(p, batches, share, WIDEST)) {
+static int ogemm_launch(const OgemmArgs& p, int batches, int share, cudaStream_t st, double beside = 0.0) {
+  switch (og_pick(p, batches, share, WIDEST, beside)) {
     case 0: return ogemm_run<AMODE, BMODE, AF32, OUT_BF16, typename OgFirst<WIDEST>::T>(p, batches, st);
     case 1: return ogemm_run<AMODE, BMODE, AF32, OUT_BF16, OgSquare>(p, batches, st);
     case 2: return ogemm_run<AMODE, BMODE, AF32, OUT_BF16, OgHalf>(p, batches, st);
