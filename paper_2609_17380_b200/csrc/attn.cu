@@ -308,17 +308,21 @@ __global__ void __launch_bounds__(256) k_attn_delta(const uint16_t* __restrict__
 }
 
 // ---------------------------------------------------------------------------------------------
-// backward, first half: P and dS of one block of 128 queries against every visible block of 128 keys.
+// backward, first half: P and dS of every block of TM queries against every visible block of 128 keys.
 // Warp-specialised like the LM-head kernel: the CTA keeps q^T and dO^T of its query block in shared memory; four
 // producer warps stream the key and value blocks through a three-slot ring of 16-dimension slabs (a "full" and an
 // "empty" mbarrier per slot, bounded waits); eight consumer warps accumulate S = q.k^T and dP = dO.v^T together (two
 // 8 x 8 register tiles per thread, each logit one ascending sum over the 128 dimensions) and, per key block, apply
 // P = exp(S*scale - L) and dS = (P (dP - Delta)) scale and store bf16(P) and bf16(dS).  The producers already fetch
 // the next key block while the consumers are in that epilogue, and consumer warps are not coupled to each other.
+// Nothing is carried from one key block to the next, so the blocks of all heads are numbered (head, query block, key block) and
+// every CTA of a resident grid takes an equal run of them; where a run enters another query block the consumers stage its rows.
+// One query block per CTA, 4 x 16 heads x 2048 (query blocks of up to 16 key blocks, 1024 of them): 1.564 ms, equal runs 1.597; but
+// 16 x 4096 at window 512 0.545 and 0.478 ms, 2 x 8 x 1088 0.215 and 0.145, 8 x 1024 0.210 and 0.066, 16 x 832 0.166 and 0.099; 16 x 4096
+// 1.528, 1.547 and with the short runs at the end 1.526.
 // ---------------------------------------------------------------------------------------------
-// Rows per CTA (TM), ring slots, CTAs per SM, registers per consumer and producer thread.  128 rows: 26.8 us per row
-// block and key block on a full GPU, 24 alone; 64 rows: 15.8 and 19 us, for grids bound by the longest chain (8 heads x
-// 1024: 0.214 ms with 128 rows, 0.169 with 64).
+// Rows per block (TM), ring slots, CTAs per SM, registers per consumer and producer thread.  A block of 128 rows takes 24.5 us, one
+// of 64 rows 18.4 alone and 15.8 beside another; both 12 us for the launch, the first rows and the first slabs.
 template <int TM_, int SLOTS_, int CPS_, int RC_, int RP_>
 struct SdpTile {
   static constexpr int TM = TM_, SLOTS = SLOTS_, CPS = CPS_, RC = RC_, RP = RP_;
@@ -329,12 +333,52 @@ struct SdpTile {
 typedef SdpTile<128, 3, 1, 216, 72> SdpTall;
 typedef SdpTile<64, 2, 2, 200, 56> SdpHalf;
 
+// named barrier of the first `threads` threads; the second form also tells whether any of them came with `x`
+__device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+__device__ __forceinline__ int bar_or(int id, int threads, bool x) {
+  int any;
+  asm volatile("{\n.reg .pred p, q;\nsetp.ne.s32 p, %1, 0;\nbar.red.or.pred q, %2, %3, p;\nselp.s32 %0, 1, 0, q;\n}"
+               : "=r"(any) : "r"((int)x), "r"(id), "r"(threads) : "memory");
+  return any;
+}
+// key blocks that the query block at i0 sees: first one, and how many
+__host__ __device__ __forceinline__ int sdp_first(int i0, int W) { return W > 0 && i0 > W ? (i0 - W) / OT : 0; }
+__host__ __device__ __forceinline__ int sdp_blocks(int i0, int W) { return i0 / OT + 1 - sdp_first(i0, W); }
+// runs of blocks: n_long equal ones over the first `head` blocks, then n_short equal ones over the rest; or (heads != 0) one
+// run per query block of the `heads` heads, the last query blocks first
+struct SdpRuns {
+  int n_long, head, n_short, total, heads;
+  __device__ __forceinline__ int start(int c) const {
+    return c <= n_long ? (int)((long long)head * c / n_long) : head + (int)((long long)(total - head) * (c - n_long) / n_short);
+  }
+};
+// position in the numbering of the blocks
+struct SdpAt {
+  int bh, i0, jt;
+  __device__ __forceinline__ SdpAt(int bh_, int i0_, int jt_) : bh(bh_), i0(i0_), jt(jt_) {}
+  __device__ __forceinline__ SdpAt(int w, int per_head, int tm, int W) {
+    bh = w / per_head;
+    w -= bh * per_head;
+    i0 = 0;
+    for (int n = sdp_blocks(0, W); w >= n; n = sdp_blocks(i0, W)) { w -= n; i0 += tm; }
+    jt = sdp_first(i0, W) + w;
+  }
+  __device__ __forceinline__ bool next(int S, int tm, int W) {   // true: another query block
+    if (++jt <= i0 / OT) return false;
+    i0 += tm;
+    if (i0 >= S) { i0 = 0; ++bh; }
+    jt = sdp_first(i0, W);
+    return true;
+  }
+};
+
 template <class T>
 __global__ void __launch_bounds__(T::THREADS, T::CPS)
     k_attn_sdp(const uint16_t* __restrict__ dout, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k,
                const uint16_t* __restrict__ v, const float* __restrict__ lse, const float* __restrict__ delta, int ld,
-               int ld_out, int H, int Hkv, int S, int W, uint16_t* __restrict__ Pb, uint16_t* __restrict__ dSt) {
-  constexpr int TM = T::TM, SDP_SLOTS = T::SLOTS, SDP_CONS = T::CONS, SDP_THREADS = T::THREADS;
+               int ld_out, int H, int Hkv, int S, int W, int per_head, const SdpRuns runs, uint16_t* __restrict__ Pb,
+               uint16_t* __restrict__ dSt) {
+  constexpr int TM = T::TM, SDP_SLOTS = T::SLOTS, SDP_CONS = T::CONS;
   extern __shared__ __align__(16) unsigned char osm[];
   typedef float(*Full)[TM + 4];
   Full Qs = reinterpret_cast<Full>(osm);                                            // [dim][query]
@@ -342,43 +386,25 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
   float(*Ks)[OK][OT + 4] = reinterpret_cast<float(*)[OK][OT + 4]>(osm + (size_t)2 * DH * (TM + 4) * sizeof(float));
   float(*Vs)[OK][OT + 4] = Ks + SDP_SLOTS;
   __shared__ __align__(16) int tiny_s[SDP_SLOTS][OG_PROD / 32];
-  __shared__ int tiny_qo, abort_s;
+  __shared__ int abort_s;
   __shared__ __align__(8) uint64_t bar_full[SDP_SLOTS], bar_empty[SDP_SLOTS];
   volatile int* abort_flag = &abort_s;
-  const int it = gridDim.y - 1 - blockIdx.y;        // longest rows first
-  const int h = blockIdx.x % H, b = blockIdx.x / H, hk = h / (H / Hkv);
-  const int i0 = it * TM, jt_hi = i0 / OT;
   const int tid = threadIdx.x, lane = tid & 31;
-  const size_t row0 = (size_t)b * S;
-  const uint16_t* qp = q + row0 * ld + (size_t)h * DH;
-  const uint16_t* op = dout + row0 * ld_out + (size_t)h * DH;
-  const uint16_t* kp = k + row0 * ld + (size_t)hk * DH;
-  const uint16_t* vp = v + row0 * ld + (size_t)hk * DH;
-  const int jt_lo = (W > 0 && i0 > W) ? (i0 - W) / OT : 0;
-  const int nslab = (jt_hi - jt_lo + 1) * (DH / OK);
+  int w_lo = 0, w_hi;
+  SdpAt at(0, 0, 0);
+  if (runs.heads) {
+    const int c = blockIdx.x, i0 = ((int)gridDim.x - 1 - c) / runs.heads * TM;
+    at = SdpAt(c % runs.heads, i0, sdp_first(i0, W));
+    w_hi = sdp_blocks(i0, W);
+  } else {
+    w_lo = runs.start(blockIdx.x);
+    w_hi = runs.start(blockIdx.x + 1);
+    at = SdpAt(w_lo, per_head, TM, W);
+  }
   if (tid == 0) {
     for (int s = 0; s < SDP_SLOTS; ++s) { mbar_init(&bar_full[s], OG_PROD / 32); mbar_init(&bar_empty[s], SDP_CONS / 32); }
-    tiny_qo = 0;
     abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  {  // q^T and dO^T of the query block, staged once by everybody
-    bool tq = false;
-    for (int idx = tid; idx < 2 * TM * 16; idx += SDP_THREADS) {
-      const int which = idx >= TM * 16, e = idx - which * TM * 16, r = e % TM, ch = e / TM;
-      const uint16_t* src = which ? op + (size_t)(i0 + r) * ld_out : qp + (size_t)(i0 + r) * ld;
-      float t[8];
-      if (i0 + r < S) unpack8a(__ldg(reinterpret_cast<const uint4*>(src + ch * 8)), t);
-      else {
-#pragma unroll
-        for (int x = 0; x < 8; ++x) t[x] = 0.0f;
-      }
-      Full dst = which ? Os : Qs;
-#pragma unroll
-      for (int x = 0; x < 8; ++x) { tq |= tiny1(t[x]); dst[ch * 8 + x][r] = t[x]; }
-    }
-    if (__any_sync(0xffffffffu, tq) && lane == 0) atomicOr(&tiny_qo, 1);
   }
   __syncthreads();
   if (tid >= SDP_CONS) {
@@ -386,18 +412,27 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(T::RP));
     const int pt = tid - SDP_CONS, pw = pt >> 5;
     OgRaw<CONTIG, false, OT> rk, rv;
-    og_fetch<CONTIG, false, OT>(kp, S, DH, ld, jt_lo * OT, 0, pt, rk);
-    og_fetch<CONTIG, false, OT>(vp, S, DH, ld, jt_lo * OT, 0, pt, rv);
+    const uint16_t *kp, *vp;
+    auto head = [&]() {
+      const size_t o = (size_t)(at.bh / H) * S * ld + (size_t)(at.bh % H / (H / Hkv)) * DH;
+      kp = k + o;
+      vp = v + o;
+    };
+    head();
+    og_fetch<CONTIG, false, OT>(kp, S, DH, ld, at.jt * OT, 0, pt, rk);
+    og_fetch<CONTIG, false, OT>(vp, S, DH, ld, at.jt * OT, 0, pt, rv);
     int slot = 0;
     uint32_t par = 1;
+    const int nslab = (w_hi - w_lo) * (DH / OK);
     for (int s = 0; s < nslab; ++s) {
       if (!mbar_wait(&bar_empty[slot], par, abort_flag, nullptr)) break;
       bool tiny = og_store<CONTIG, false, OT>(Ks[slot], pt, rk);
       tiny |= og_store<CONTIG, false, OT>(Vs[slot], pt, rv);
       if (s + 1 < nslab) {
-        const int j0n = (jt_lo + (s + 1) / (DH / OK)) * OT, c0n = ((s + 1) % (DH / OK)) * OK;
-        og_fetch<CONTIG, false, OT>(kp, S, DH, ld, j0n, c0n, pt, rk);
-        og_fetch<CONTIG, false, OT>(vp, S, DH, ld, j0n, c0n, pt, rv);
+        if ((s + 1) % (DH / OK) == 0 && at.next(S, TM, W)) head();
+        const int c0n = ((s + 1) % (DH / OK)) * OK;
+        og_fetch<CONTIG, false, OT>(kp, S, DH, ld, at.jt * OT, c0n, pt, rk);
+        og_fetch<CONTIG, false, OT>(vp, S, DH, ld, at.jt * OT, c0n, pt, rv);
       }
       const int any = __any_sync(0xffffffffu, tiny);
       if (lane == 0) tiny_s[slot][pw] = any;
@@ -410,80 +445,115 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
   // --------------------------------- consumers ---------------------------------
   asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(T::RC));
   const int ty = (tid >> 5) * 2 + (tid & 1), tx = (lane >> 1);   // neighbouring lanes share their columns (see og_lane)
-  const int tqo = tiny_qo;
-  const size_t bh = (size_t)b * H + h;
+  int tqo = 0;                                     // a value below 2^-63 among the rows
   float Lr[8], Dr[8];
+  // q^T and dO^T of the query block, and its rows' logsumexp and Delta: everything is on its way before the barrier
+  auto stage = [&](int bh, int i0) {
+    const size_t row = (size_t)(bh / H) * S + i0;
+    const int h = bh % H;
+    uint4 u[2][8];                                 // TM x 16 pieces of 16 bytes each: eight per thread
 #pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    const int i = i0 + (a >> 2) * (TM / 2) + ty * 4 + (a & 3);
-    Lr[a] = i < S ? lse[bh * S + i] : 0.0f;
-    Dr[a] = i < S ? delta[bh * S + i] : 0.0f;
-  }
+    for (int c = 0; c < 8; ++c) {
+      const int e = c * SDP_CONS + tid, x = e % TM, ch = e / TM;
+      const bool in = i0 + x < S;
+      u[0][c] = in ? __ldg(reinterpret_cast<const uint4*>(q + (row + x) * ld + (size_t)h * DH + ch * 8)) : make_uint4(0u, 0u, 0u, 0u);
+      u[1][c] = in ? __ldg(reinterpret_cast<const uint4*>(dout + (row + x) * ld_out + (size_t)h * DH + ch * 8)) : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const int i = i0 + (a >> 2) * (TM / 2) + ty * 4 + (a & 3);
+      Lr[a] = i < S ? lse[(size_t)bh * S + i] : 0.0f;
+      Dr[a] = i < S ? delta[(size_t)bh * S + i] : 0.0f;
+    }
+    bool tq = false;
+    bar_sync(1, SDP_CONS);                         // the rows before are not needed any more
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const int e = c * SDP_CONS + tid, x = e % TM, ch = e / TM;
+      float t[8];
+      unpack8a(u[0][c], t);
+#pragma unroll
+      for (int y = 0; y < 8; ++y) { tq |= tiny1(t[y]); Qs[ch * 8 + y][x] = t[y]; }
+      unpack8a(u[1][c], t);
+#pragma unroll
+      for (int y = 0; y < 8; ++y) { tq |= tiny1(t[y]); Os[ch * 8 + y][x] = t[y]; }
+    }
+    tqo = bar_or(1, SDP_CONS, tq);
+  };
   const float2 one = same2(c_one);
   int slot = 0;
   uint32_t par = 0;
   bool ok = true;
-  for (int jt = jt_lo; jt <= jt_hi && ok; ++jt) {
-    const int j0 = jt * OT;
-    float2 sa[8][4], da[8][4];
+  for (int w = w_lo; w < w_hi;) {
+    const int i0 = at.i0, jt0 = at.jt, jt1 = min(jt0 + w_hi - w, i0 / OT + 1);
+    const size_t bh = (size_t)at.bh;
+    stage(at.bh, i0);                              // after a wait that ran out, too: the other warps stand at its barriers
+    w += jt1 - jt0;
+    at.jt = jt1 - 1;
+    at.next(S, TM, W);
+    for (int jt = jt0; jt < jt1 && ok; ++jt) {
+      const int j0 = jt * OT;
+      float2 sa[8][4], da[8][4];
 #pragma unroll
-    for (int a = 0; a < 8; ++a)
+      for (int a = 0; a < 8; ++a)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) { sa[a][c] = make_float2(0.f, 0.f); da[a][c] = make_float2(0.f, 0.f); }
-    for (int sl = 0; sl < DH / OK; ++sl) {
-      if (!mbar_wait(&bar_full[slot], par, abort_flag, nullptr)) { ok = false; break; }
-      const int4 t4 = *reinterpret_cast<const int4*>(tiny_s[slot]);
-      const int tiny = tqo | t4.x | t4.y | t4.z | t4.w;
-      if (tiny) { slab_mac<false, TM, OT, 8>(Qs + sl * OK, Ks[slot], ty, tx, sa); slab_mac<false, TM, OT, 8>(Os + sl * OK, Vs[slot], ty, tx, da); }
-      else { slab_mac<true, TM, OT, 8>(Qs + sl * OK, Ks[slot], ty, tx, sa); slab_mac<true, TM, OT, 8>(Os + sl * OK, Vs[slot], ty, tx, da); }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bar_empty[slot]);
-      if (++slot == SDP_SLOTS) { slot = 0; par ^= 1u; }
-    }
-    if (!ok) break;
-    // P = exp(S*scale - L) and dS, two pairs at a time; the argument is at most 0 whenever L is the row's own logsumexp, and
-    // then the exponential without the overflow range applies (same bits), but L is an input, so four pairs that hold
-    // a positive argument take the general form.  Only the block at the diagonal and those at the window's start mask.
-    const bool masked = j0 + OT - 1 > i0 || (W > 0 && j0 <= i0 + TM - 1 - W);
+        for (int c = 0; c < 4; ++c) { sa[a][c] = make_float2(0.f, 0.f); da[a][c] = make_float2(0.f, 0.f); }
+      for (int sl = 0; sl < DH / OK && ok; ++sl) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&bar_full[slot], par, abort_flag, nullptr));
+        if (!ok) break;
+        const int4 t4 = *reinterpret_cast<const int4*>(tiny_s[slot]);
+        const int tiny = tqo | t4.x | t4.y | t4.z | t4.w;
+        if (tiny) { slab_mac<false, TM, OT, 8>(Qs + sl * OK, Ks[slot], ty, tx, sa); slab_mac<false, TM, OT, 8>(Os + sl * OK, Vs[slot], ty, tx, da); }
+        else { slab_mac<true, TM, OT, 8>(Qs + sl * OK, Ks[slot], ty, tx, sa); slab_mac<true, TM, OT, 8>(Os + sl * OK, Vs[slot], ty, tx, da); }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar_empty[slot]);
+        if (++slot == SDP_SLOTS) { slot = 0; par ^= 1u; }
+      }
+      if (!ok) break;
+      // P = exp(S*scale - L) and dS, two pairs at a time; the argument is at most 0 whenever L is the row's own logsumexp, and
+      // then the exponential without the overflow range applies (same bits), but L is an input, so four pairs that hold
+      // a positive argument take the general form.  Only the block at the diagonal and those at the window's start mask.
+      const bool masked = j0 + OT - 1 > i0 || (W > 0 && j0 <= i0 + TM - 1 - W);
 #pragma unroll
-    for (int a = 0; a < 8; ++a) {
-      const int i = i0 + (a >> 2) * (TM / 2) + ty * 4 + (a & 3);
-      if (i >= S) continue;
-      const float2 L2 = same2(-Lr[a]), D2 = same2(-Dr[a]);
+      for (int a = 0; a < 8; ++a) {
+        const int i = i0 + (a >> 2) * (TM / 2) + ty * 4 + (a & 3);
+        if (i >= S) continue;
+        const float2 L2 = same2(-Lr[a]), D2 = same2(-Dr[a]);
 #pragma unroll
-      for (int g = 0; g < 2; ++g) {
-        const int jb = j0 + g * 64 + tx * 4;
-        if (jb >= S) continue;
-        float2 x[2], pv[2], ds[2];
+        for (int g = 0; g < 2; ++g) {
+          const int jb = j0 + g * 64 + tx * 4;
+          if (jb >= S) continue;
+          float2 x[2], pv[2], ds[2];
 #pragma unroll
-        for (int t = 0; t < 2; ++t) x[t] = add2(mul2(sa[a][2 * g + t], same2(ATT_SCALE)), L2, one);
-        bool vis[4] = {true, true, true, true};
-        if (masked) {
+          for (int t = 0; t < 2; ++t) x[t] = add2(mul2(sa[a][2 * g + t], same2(ATT_SCALE)), L2, one);
+          bool vis[4] = {true, true, true, true};
+          if (masked) {
 #pragma unroll
-          for (int e = 0; e < 4; ++e) vis[e] = jb + e <= i && (W == 0 || jb + e > i - W);
-          x[0] = make_float2(vis[0] ? x[0].x : 0.0f, vis[1] ? x[0].y : 0.0f);
-          x[1] = make_float2(vis[2] ? x[1].x : 0.0f, vis[3] ? x[1].y : 0.0f);
-        }
-        if (x[0].x > 0.0f || x[0].y > 0.0f || x[1].x > 0.0f || x[1].y > 0.0f) {
-#pragma unroll
-          for (int t = 0; t < 2; ++t) pv[t] = make_float2(det_exp(x[t].x), det_exp(x[t].y));
-        } else {
-#pragma unroll
-          for (int t = 0; t < 2; ++t) pv[t] = det_exp_le0_2(x[t], one);
-        }
-#pragma unroll
-        for (int t = 0; t < 2; ++t) ds[t] = mul2(mul2(pv[t], add2(da[a][2 * g + t], D2, one)), same2(ATT_SCALE));
-        if (masked) {
-#pragma unroll
-          for (int t = 0; t < 2; ++t) {
-            pv[t] = make_float2(vis[2 * t] ? pv[t].x : 0.0f, vis[2 * t + 1] ? pv[t].y : 0.0f);
-            ds[t] = make_float2(vis[2 * t] ? ds[t].x : 0.0f, vis[2 * t + 1] ? ds[t].y : 0.0f);
+            for (int e = 0; e < 4; ++e) vis[e] = jb + e <= i && (W == 0 || jb + e > i - W);
+            x[0] = make_float2(vis[0] ? x[0].x : 0.0f, vis[1] ? x[0].y : 0.0f);
+            x[1] = make_float2(vis[2] ? x[1].x : 0.0f, vis[3] ? x[1].y : 0.0f);
           }
+          if (x[0].x > 0.0f || x[0].y > 0.0f || x[1].x > 0.0f || x[1].y > 0.0f) {
+#pragma unroll
+            for (int t = 0; t < 2; ++t) pv[t] = make_float2(det_exp(x[t].x), det_exp(x[t].y));
+          } else {
+#pragma unroll
+            for (int t = 0; t < 2; ++t) pv[t] = det_exp_le0_2(x[t], one);
+          }
+#pragma unroll
+          for (int t = 0; t < 2; ++t) ds[t] = mul2(mul2(pv[t], add2(da[a][2 * g + t], D2, one)), same2(ATT_SCALE));
+          if (masked) {
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+              pv[t] = make_float2(vis[2 * t] ? pv[t].x : 0.0f, vis[2 * t + 1] ? pv[t].y : 0.0f);
+              ds[t] = make_float2(vis[2 * t] ? ds[t].x : 0.0f, vis[2 * t + 1] ? ds[t].y : 0.0f);
+            }
+          }
+          const size_t off = (bh * S + i) * S + jb;
+          // P~ = bf16(P) is all the value gradient needs
+          *reinterpret_cast<uint2*>(Pb + off) = make_uint2(pack_bf2(pv[0].x, pv[0].y), pack_bf2(pv[1].x, pv[1].y));
+          *reinterpret_cast<uint2*>(dSt + off) = make_uint2(pack_bf2(ds[0].x, ds[0].y), pack_bf2(ds[1].x, ds[1].y));
         }
-        const size_t off = (bh * S + i) * S + jb;
-        // P~ = bf16(P) is all the value gradient needs
-        *reinterpret_cast<uint2*>(Pb + off) = make_uint2(pack_bf2(pv[0].x, pv[0].y), pack_bf2(pv[1].x, pv[1].y));
-        *reinterpret_cast<uint2*>(dSt + off) = make_uint2(pack_bf2(ds[0].x, ds[0].y), pack_bf2(ds[1].x, ds[1].y));
       }
     }
   }
@@ -537,11 +607,6 @@ static int attn_rows(int heads, int S, int window) {
   const RowCost c[3] = {{128, 25.1, 25.1}, {64, 17.0, 13.2}, {32, 13.0, 7.5}};
   return pick_rows(c, heads, S, window);
 }
-static int sdp_rows(int heads, int S, int window) {
-  const RowCost c[2] = {{128, 24.5, 26.8}, {64, 19.0, 15.8}};
-  return pick_rows(c, heads, S, window);
-}
-
 static int attn_fwd_impl(const det_bf16* q, const det_bf16* k, const det_bf16* v, int ld, int B, int H, int Hkv, int S,
                          int window, det_bf16* out, int ld_out, float* lse, const float* s_q, int8_t* qout, void* stream) {
   if (!q || !k || !v || !out || !lse || B <= 0 || H <= 0 || Hkv <= 0 || S <= 0 || window < 0) return DET_ERR_ARG;
@@ -580,12 +645,26 @@ extern "C" size_t det_attn_bwd_fixq_ws_bytes(int B, int H, int Hkv, int S) { ret
 
 template <class T>
 static int sdp_run(const det_bf16* dout, const det_bf16* q, const det_bf16* k, const det_bf16* v, const float* lse,
-                   const float* delta, int ld, int ld_out, int B, int H, int Hkv, int S, int window, uint16_t* Pb, uint16_t* dSt,
-                   cudaStream_t st) {
+                   const float* delta, int ld, int ld_out, int B, int H, int Hkv, int S, int window, int per_head, uint16_t* Pb,
+                   uint16_t* dSt, cudaStream_t st) {
   static DevOnce once = {};
   if (dev_ensure_smem(once, (const void*)k_attn_sdp<T>, T::SMEM) != DET_OK) return DET_ERR_CUDA;
-  const dim3 grid(H * B, (S + T::TM - 1) / T::TM);
-  k_attn_sdp<T><<<DET_L(grid), T::THREADS, T::SMEM, st>>>(dout, q, k, v, lse, delta, ld, ld_out, H, Hkv, S, window, Pb, dSt);
+  const int total = B * H * per_head, slots = dev_sm_count() * T::CPS;
+  // Runs of equal length, with a sixteenth of the blocks left for the SMs that finish first where a run is long; whole query blocks
+  // only where those are long (the start of a CTA weighs little) and many (the hardware's order balances them)
+  const int rows = (S + T::TM - 1) / T::TM, longest = sdp_blocks((rows - 1) * T::TM, window);
+  SdpRuns runs = {total < slots ? total : slots, total, 0, total, 0};
+  int ctas = runs.n_long;
+  if (longest >= 12 && (long long)rows * B * H >= 6 * slots) {
+    runs.heads = B * H;
+    ctas = rows * B * H;
+  } else if (total >= 16 * slots) {
+    runs.head = total - total / 16;
+    runs.n_short = 2 * slots;
+    ctas += runs.n_short;
+  }
+  k_attn_sdp<T><<<DET_L(ctas), T::THREADS, T::SMEM, st>>>(dout, q, k, v, lse, delta, ld, ld_out, H, Hkv, S, window, per_head, runs, Pb,
+                                                          dSt);
   return DET_OK;
 }
 
@@ -612,9 +691,16 @@ static int attn_bwd_impl(const det_bf16* dout, const det_bf16* q, const det_bf16
   DET_CHECK_LAUNCH();
   // P[i,j] = exp(scale * sum_d q[i,d] k[j,d] - L_i) for visible (i,j) (f32; tiles without a visible pair are never
   // touched) and dS[i,j] = bf16((P[i,j] * (sum_d dO[i,d] v[j,d] - Delta_i)) * scale); both sums ascend over the 128 dims
-  int rc = sdp_rows(B * H, S, window) == 128
-               ? sdp_run<SdpTall>(dout, q, k, v, lse, delta, ld, ld_out, B, H, Hkv, S, window, Pb, dSt, st)
-               : sdp_run<SdpHalf>(dout, q, k, v, lse, delta, ld, ld_out, B, H, Hkv, S, window, Pb, dSt, st);
+  // blocks of 64 rows where those leave every CTA with one block at most (2 heads x 128: 0.027 against 0.035 ms); with more of them
+  // the tall ones have the better rate (8 x 1024: 0.076 and 0.066 ms)
+  int tall = 0, half = 0;
+  for (int i0 = 0; i0 < S; i0 += 64) {
+    half += sdp_blocks(i0, window);
+    if (i0 % 128 == 0) tall += sdp_blocks(i0, window);
+  }
+  int rc = (long long)B * H * half <= dev_sm_count()
+               ? sdp_run<SdpHalf>(dout, q, k, v, lse, delta, ld, ld_out, B, H, Hkv, S, window, half, Pb, dSt, st)
+               : sdp_run<SdpTall>(dout, q, k, v, lse, delta, ld, ld_out, B, H, Hkv, S, window, tall, Pb, dSt, st);
   if (rc != DET_OK) return rc;
   DET_CHECK_LAUNCH();
   // dV[j,c] = sum over the query heads g of the group, then over queries i >= j ascending, of P~[i,j] dO[i,c];

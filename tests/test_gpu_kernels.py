@@ -114,6 +114,28 @@ def test_attention_row_blocks(det, B, H, Hkv, S, W, fixq):
         assert_same_bits(got[:, lo:hi], want[:, lo:hi], name)
 
 
+# the backward's blocks in equal runs, in runs with short ones at the end, and by whole query blocks: heads of one call against the
+# same heads in calls of their own
+@pytest.mark.parametrize("B,H,S", [(1, 3, 1344), (1, 18, 2048), (4, 16, 2048)])
+def test_attention_backward_heads_apart(det, B, H, S):
+    def run(B, H, qkv, dout):
+        HD, x = H * 128, dev(qkv)
+        q = x.data_ptr()
+        out, lse, dqkv = empty((B * S, HD), np.uint16), empty((B, H, S), F), empty((B * S, 3 * HD), np.uint16)
+        det.det_attn_fwd(q, q + 2 * HD, q + 4 * HD, 3 * HD, B, H, S, out, HD, lse)
+        d = dqkv.data_ptr()
+        det.det_attn_bwd(dev(dout), q, q + 2 * HD, q + 4 * HD, out, lse, 3 * HD, HD, B, H, S, d, d + 2 * HD, d + 4 * HD, 3 * HD,
+                         ws(det.det_attn_bwd_ws_bytes(B, H, S)))
+        _sync()
+        return host(dqkv, np.uint16).reshape(B, S, 3, H, 128)
+    qkv = synth.normal_bf16((B * S, 3 * H * 128), 1.0, seed=H, tid=1).reshape(B, S, 3, H, 128)
+    dout = synth.normal_bf16((B * S, H * 128), 0.1, seed=H, tid=2).reshape(B, S, H, 128)
+    got = run(B, H, qkv, dout)
+    for b, h in ((0, 0), (B - 1, H // 2), (B - 1, H - 1)):
+        want = run(1, 1, np.ascontiguousarray(qkv[b:b + 1, :, :, h:h + 1]), np.ascontiguousarray(dout[b:b + 1, :, h:h + 1]))
+        assert_same_bits(got[b, :, :, h], want[0, :, :, 0], "gradients of head %d" % h)
+
+
 # the two-lane exponential: a dense grid of arguments, the ends of the kept range, subnormal, infinite and NaN arguments
 def test_two_lane_exponential(det):
     x = np.concatenate([np.linspace(-90, 0, 400001), np.linspace(-87.4, -87.2, 20001), [0.0, -0.0, -1e-40, -1e-30, -200.0, -1e30, -np.inf, np.nan]]).astype(F)
