@@ -102,10 +102,8 @@ __global__ void __launch_bounds__(256) k_quantize(const uint16_t* __restrict__ X
 // ---- Walsh-Hadamard operand preparation -----------------------------------------------------------
 // Unnormalised butterflies, stages h = 1..64, (a, b) -> (a + b, a - b) for index pairs (i, i + h).
 
-// (1) rotation along the row (contiguous) direction: A = rotate_n(dY[m,n] * s_w[n]).
-//     A warp owns one 128-element block: a lane holds 4 adjacent elements (stages 1, 2 in registers,
-//     stages 4..64 by shuffles).  PASS 0 records the absmax, PASS 1 quantises.
-template <int PASS, bool ROT>
+// (1) without the rotation: A = dY[m,n] * s_w[n], PASS 0 records the absmax, PASS 1 quantises.  A lane holds 4 adjacent elements.
+template <int PASS>
 __global__ void __launch_bounds__(256) k_rot_rows(const uint16_t* __restrict__ dY, const float* __restrict__ s_w, int M,
                                                   int N, uint32_t* __restrict__ amax, int8_t* __restrict__ Aq) {
   // a warp owns RB consecutive 128-element blocks of one row and issues all its loads before any arithmetic
@@ -139,19 +137,6 @@ __global__ void __launch_bounds__(256) k_rot_rows(const uint16_t* __restrict__ d
     for (int r = 0; r < RB; ++r) {
       const int n0 = (nb0 + r) * 128 + lane * 4;
       float v[4] = {fmul(bflo(u[r].x), w[r].x), fmul(bfhi(u[r].x), w[r].y), fmul(bflo(u[r].y), w[r].z), fmul(bfhi(u[r].y), w[r].w)};
-      if (ROT) {
-        float a0 = fadd(v[0], v[1]), a1 = fsub(v[0], v[1]), a2 = fadd(v[2], v[3]), a3 = fsub(v[2], v[3]);
-        v[0] = fadd(a0, a2); v[2] = fsub(a0, a2); v[1] = fadd(a1, a3); v[3] = fsub(a1, a3);
-#pragma unroll
-        for (int hl = 1; hl < 32; hl <<= 1) {
-          const bool upper = lane & hl;
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            float o = __shfl_xor_sync(0xffffffffu, v[e], hl);
-            v[e] = upper ? fsub(o, v[e]) : fadd(v[e], o);
-          }
-        }
-      }
       if (PASS == 0) {
         local = fmaxf(local, fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3]))));
       } else if (n0 < N) {
@@ -170,59 +155,27 @@ __global__ void __launch_bounds__(256) k_rot_rows(const uint16_t* __restrict__ d
   }
 }
 
-// (2) rotation along the row-index (strided) direction with a transposed int8 result:
-//     in [R, C] (bf16 for G = dY, int8 for Z = qX and U = qW)  ->  out int8 [C, R],
-//     out[c, r] = quantise(rotate_r(in[:, c]))[r].  A thread owns one column of a 128-row block: 128 values in
-//     registers (a warp reads 32 adjacent columns of each row, i.e. whole 32/64-byte sectors), the seven butterfly
-//     stages run in registers, and the thread writes its 128 quantised values as one contiguous 128-byte run of the
-//     transposed output.  Each stage touches disjoint pairs, so the rounding order per element is fixed.
-template <bool ISF, int PASS, bool ROT>
-__global__ void __launch_bounds__(128) k_rotc(const void* __restrict__ in, int R, int C, uint32_t* __restrict__ amax,
+// (2) without the rotation, transposed: G = dY as int8 [N, M], a thread per column of a 128-row block (a warp reads 32 adjacent
+//     columns of each row, and a thread writes one contiguous 128-byte run).
+template <int PASS>
+__global__ void __launch_bounds__(128) k_rotc(const uint16_t* __restrict__ in, int R, int C, uint32_t* __restrict__ amax,
                                               int8_t* __restrict__ outT) {
   const int col = blockIdx.x * 128 + threadIdx.x;
   const int r0 = blockIdx.y * 128;
-  float vf[ISF ? 128 : 1];
-  int vi[ISF ? 1 : 128];
-  if (ISF) {
-    const uint16_t* p = reinterpret_cast<const uint16_t*>(in) + (size_t)r0 * C + col;
+  float vf[128];
+  const uint16_t* p = in + (size_t)r0 * C + col;
 #pragma unroll
-    for (int i = 0; i < 128; ++i) vf[i] = bf2f(__ldg(p + (size_t)i * C));
-  } else {
-    const int8_t* p = reinterpret_cast<const int8_t*>(in) + (size_t)r0 * C + col;
-#pragma unroll
-    for (int i = 0; i < 128; ++i) vi[i] = (int)__ldg(p + (size_t)i * C);
-  }
-  if (ROT) {
-#pragma unroll
-    for (int h = 1; h < 128; h <<= 1) {
-#pragma unroll
-      for (int i = 0; i < 128; ++i) {
-        if (!(i & h)) {
-          if (ISF) { const float a = vf[i], b = vf[i + h]; vf[i] = fadd(a, b); vf[i + h] = fsub(a, b); }
-          else { const int a = vi[i], b = vi[i + h]; vi[i] = a + b; vi[i + h] = a - b; }
-        }
-      }
-    }
-  }
+  for (int i = 0; i < 128; ++i) vf[i] = bf2f(__ldg(p + (size_t)i * C));
   if (PASS == 0) {
     uint32_t local = 0;
 #pragma unroll
-    for (int i = 0; i < 128; ++i) {
-      if (ISF) local = max(local, __float_as_uint(fabsf(vf[i])));
-      else local = max(local, (uint32_t)abs(vi[i]));
-    }
+    for (int i = 0; i < 128; ++i) local = max(local, __float_as_uint(fabsf(vf[i])));
 #pragma unroll
     for (int w = 16; w; w >>= 1) local = max(local, __shfl_xor_sync(0xffffffffu, local, w));
     if ((threadIdx.x & 31) == 0 && local > *reinterpret_cast<volatile uint32_t*>(amax)) atomicMax(amax, local);
   } else {
-    float inv = 0.0f;
-    if (ISF) {
-      const float am = __uint_as_float(amax[0]);
-      inv = (am > 0.0f) ? fdiv(127.0f, am) : 0.0f;
-    } else if (ROT) {
-      const int am = (int)amax[0];
-      inv = (am > 0) ? fdiv(127.0f, __int2float_rn(am)) : 0.0f;
-    }
+    const float am = __uint_as_float(amax[0]);
+    const float inv = (am > 0.0f) ? fdiv(127.0f, am) : 0.0f;
     uint4* dst = reinterpret_cast<uint4*>(outT + (size_t)col * R + r0);
 #pragma unroll
     for (int g = 0; g < 8; ++g) {
@@ -231,31 +184,19 @@ __global__ void __launch_bounds__(128) k_rotc(const void* __restrict__ in, int R
       for (int k = 0; k < 4; ++k) {
         uint32_t o = 0;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int i = g * 16 + k * 4 + e;
-          int8_t qv;
-          if (ISF) qv = quant1(vf[i], inv);
-          else if (ROT) qv = quant1(__int2float_rn(vi[i]), inv);
-          else qv = (int8_t)vi[i];
-          o |= ((uint32_t)(uint8_t)qv) << (8 * e);
-        }
+        for (int e = 0; e < 4; ++e) o |= ((uint32_t)(uint8_t)quant1(vf[g * 16 + k * 4 + e], inv)) << (8 * e);
         w[k] = o;
       }
       dst[g] = make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
 }
-
-// (2b) the int8 operands (Z = qX, U = qW) through shared memory: the CTA loads its 128 x 128 tile with whole 128-byte row
-//      segments (eight lanes per row), every thread takes one column from the tile (a warp reads 32 adjacent bytes of a
-//      row: one wavefront), rotates it in registers (exact integers, |value| <= 2^14), and in PASS 1 the quantised columns
-//      go back through the tile so that the transposed output is written as whole 128-byte lines as well (the version this
-//      replaced read one byte and wrote sixteen per lane in 32 different lines per instruction; the values are the same).
-template <int PASS, bool ROT>
-__global__ void __launch_bounds__(128) k_rotc8(const int8_t* __restrict__ in, int R, int C, uint32_t* __restrict__ amax,
-                                               int8_t* __restrict__ outT) {
+// and the int8 operand: transposed through shared memory, whole 128-byte lines on both sides; s_u (or null) becomes 1
+__global__ void __launch_bounds__(128) k_transpose8(const int8_t* __restrict__ in, int R, int C, int8_t* __restrict__ outT,
+                                                    float* __restrict__ s_u) {
   __shared__ __align__(16) uint8_t tile[128 * 128];
   const int t = threadIdx.x, c0 = blockIdx.x * 128, r0 = blockIdx.y * 128;
+  if (s_u && blockIdx.x == 0 && blockIdx.y == 0 && t == 0) s_u[0] = 1.0f;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int r = i * 16 + (t >> 3), ch = t & 7;
@@ -263,50 +204,15 @@ __global__ void __launch_bounds__(128) k_rotc8(const int8_t* __restrict__ in, in
         __ldg(reinterpret_cast<const uint4*>(in + (size_t)(r0 + r) * C + c0 + ch * 16));
   }
   __syncthreads();
-  int vi[128];
+  uint32_t w[32];
 #pragma unroll
-  for (int i = 0; i < 128; ++i) vi[i] = (int)(int8_t)tile[i * 128 + t];
-  if (ROT) {
-#pragma unroll
-    for (int h = 1; h < 128; h <<= 1) {
-#pragma unroll
-      for (int i = 0; i < 128; ++i) {
-        if (!(i & h)) { const int a = vi[i], b = vi[i + h]; vi[i] = a + b; vi[i + h] = a - b; }
-      }
-    }
-  }
-  if (PASS == 0) {
-    uint32_t local = 0;
-#pragma unroll
-    for (int i = 0; i < 128; ++i) local = max(local, (uint32_t)abs(vi[i]));
-#pragma unroll
-    for (int w = 16; w; w >>= 1) local = max(local, __shfl_xor_sync(0xffffffffu, local, w));
-    if ((t & 31) == 0 && local > *reinterpret_cast<volatile uint32_t*>(amax)) atomicMax(amax, local);
-    return;
-  }
-  float inv = 0.0f;
-  if (ROT) {
-    const int am = (int)amax[0];
-    inv = (am > 0) ? fdiv(127.0f, __int2float_rn(am)) : 0.0f;
-  }
+  for (int k = 0; k < 32; ++k)
+    w[k] = (uint32_t)tile[(4 * k) * 128 + t] | ((uint32_t)tile[(4 * k + 1) * 128 + t] << 8) | ((uint32_t)tile[(4 * k + 2) * 128 + t] << 16) |
+           ((uint32_t)tile[(4 * k + 3) * 128 + t] << 24);
   __syncthreads();                       // everybody has read its column: the tile becomes the transposed output tile
 #pragma unroll
-  for (int g = 0; g < 8; ++g) {
-    uint32_t w[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      uint32_t o = 0;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int i = g * 16 + k * 4 + e;
-        const int8_t qv = ROT ? quant1(__int2float_rn(vi[i]), inv) : (int8_t)vi[i];
-        o |= ((uint32_t)(uint8_t)qv) << (8 * e);
-      }
-      w[k] = o;
-    }
-    // row t of the transposed tile (column c0 + t of the input), sixteen-byte pieces XOR-swizzled by row
-    *reinterpret_cast<uint4*>(tile + t * 128 + ((g ^ (t & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-  }
+  for (int g = 0; g < 8; ++g)            // row t of it, sixteen-byte pieces XOR-swizzled by row
+    *reinterpret_cast<uint4*>(tile + t * 128 + ((g ^ (t & 7)) << 4)) = make_uint4(w[4 * g], w[4 * g + 1], w[4 * g + 2], w[4 * g + 3]);
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -371,18 +277,23 @@ __device__ __forceinline__ void quant_pack128(const float2 (&v)[64], float inv, 
   }
 }
 __device__ __forceinline__ bool finite1(float x) { return (__float_as_uint(x) & 0x7f800000u) != 0x7f800000u; }
-__device__ __forceinline__ void amax_publish(float local, uint32_t* amax) {
-#pragma unroll
-  for (int w = 16; w; w >>= 1) local = fmaxf(local, __shfl_xor_sync(0xffffffffu, local, w));
-  if ((threadIdx.x & 31) == 0 && local > 0.0f && __float_as_uint(local) > *reinterpret_cast<volatile uint32_t*>(amax))
-    atomicMax(amax, __float_as_uint(local));
-}
 
-//     The kernel is persistent and software-pipelined: a CTA walks over tiles, the raw bf16 tile of the NEXT step travels
-//     into the other half of a double buffer (16-byte asynchronous copies, chunks XOR-swizzled by row so that a thread reads
+//     The kernel is persistent and software-pipelined: a CTA walks over tiles, the raw tile of the NEXT step travels
+//     into the other half of a double buffer (16-byte asynchronous copies, bf16 chunks XOR-swizzled by row so that a thread reads
 //     its row with conflict-free 16-byte loads and its column with 2-byte loads) while the current one is rotated, so no
 //     global-load latency and no convert-and-store pass sits between the butterflies; the finished int8 rows leave through
 //     the buffer that has just been consumed, as whole 128-byte lines.
+//
+// (4) the int8 operand (Z = qX for the weight gradient, U = qW for the weights) in the same launch, as further tiles: a thread rotates
+//     one column, as f32 (exact integers up to 2^14).  The byte becomes 2^23 + 128 + x by its exponent bits, one subtraction
+//     for two values takes the offset away, and the butterflies are the packed ones (as 32-bit integers they took the
+//     half-rate integer pipe: 896 instructions of two cycles instead of 512 that make up 896 cycles of the FP32 pipe).
+//
+//     The code is straight-line and as long as the work on a tile.  Where no CTA has more than one tile, fetching it is what takes the
+//     time, and rows of dY, columns of dY and columns of Z go through ONE copy of the butterflies and of the quantiser in a
+//     rolled loop (PREP_ONE; second pass of 256 tokens x 512, cold: 7.4 us in one launch, 27 with a copy for each).  Over
+//     many tiles the copies are the faster form (first pass over 16384 tokens x 16384: 0.20 against 0.23 ms), dY in one launch (PREP_Y), Z in
+//     another (PREP_Z) beside it.
 constexpr size_t PREP2_SMEM = (size_t)2 * PT * 256 + 2 * PT * sizeof(float);
 
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
@@ -392,36 +303,86 @@ __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gsrc) : "memory");
 }
 
-template <int PASS>
-__global__ void __launch_bounds__(PT, 3) k_prep_dy2(const uint16_t* __restrict__ dY, const float* __restrict__ s_w, int M, int N,
-                                                    uint32_t* __restrict__ amax, int8_t* __restrict__ Aq,
-                                                    int8_t* __restrict__ GqT) {
+// The maxima of pass 0 for A, G and Z: a word per CTA where the scratch has room for it, else one, zeroed before and raised by
+// atomics.  Pass 1 reduces them and its first CTA leaves the results in final[0..2].
+struct PrepMax {
+  uint32_t* part[3];
+  int n[3];
+  uint32_t* final;
+};
+struct PrepArgs {
+  const uint16_t* dY;      // [M, N] or null
+  const float* s_w;
+  const int8_t* Z;         // [M, K]
+  int M, N, K;
+  int8_t *Aq, *GqT, *ZqT;
+  PrepMax mx;
+  float* s_u;              // the step of Z, or null
+};
+
+__device__ __forceinline__ uint32_t block_max(uint32_t x, uint32_t (&box)[PT / 32]) {
+  x = __reduce_max_sync(0xffffffffu, x);
+  if ((threadIdx.x & 31) == 0) box[threadIdx.x >> 5] = x;
+  __syncthreads();
+  x = max(max(box[0], box[1]), max(box[2], box[3]));
+  __syncthreads();
+  return x;
+}
+
+enum { PREP_ONE, PREP_Y, PREP_Z };
+template <int PASS, int KIND>
+__global__ void __launch_bounds__(PT, 3) k_prep(const __grid_constant__ PrepArgs p) {
   extern __shared__ __align__(16) uint8_t pbuf[];
+  __shared__ uint32_t box[PT / 32];
   float* swb = reinterpret_cast<float*>(pbuf + 2 * PT * 256);      // [2][128]
-  const int t = threadIdx.x;
-  const int ntn = N / PT, ntiles = ntn * (M / PT);
+  const int t = threadIdx.x, M = p.M, N = p.N, K = p.K;
+  const int ntn = N / PT, ntk = K / PT, ntiles_y = KIND != PREP_Z && p.dY ? ntn * (M / PT) : 0;
+  const int ntiles = ntiles_y + (KIND != PREP_Y ? ntk * (M / PT) : 0);
+  auto z_tile = [&](int tile) { return KIND == PREP_Z || (KIND == PREP_ONE && tile >= ntiles_y); };
   auto issue = [&](int tile, int b) {
-    const int n0 = (tile % ntn) * PT, m0 = (tile / ntn) * PT;
     uint8_t* dst = pbuf + b * (PT * 256);
+    if (!z_tile(tile)) {
+      const int n0 = (tile % ntn) * PT, m0 = (tile / ntn) * PT;
 #pragma unroll
-    for (int it = 0; it < 16; ++it) {
-      const int r = it * 8 + (t >> 4), c = t & 15;
-      cp_async16(dst + r * 256 + ((c ^ (r & 7)) << 4), dY + (size_t)(m0 + r) * N + n0 + c * 8);
+      for (int it = 0; it < 16; ++it) {
+        const int r = it * 8 + (t >> 4), c = t & 15;
+        cp_async16(dst + r * 256 + ((c ^ (r & 7)) << 4), p.dY + (size_t)(m0 + r) * N + n0 + c * 8);
+      }
+      cp_async4(swb + b * PT + t, p.s_w + n0 + t);
+    } else {
+      const int z = tile - ntiles_y, c0 = (z % ntk) * PT, m0 = (z / ntk) * PT;
+      const int8_t* src = p.Z + (size_t)(m0 + (t >> 3)) * K + c0 + (t & 7) * 16;
+#pragma unroll
+      for (int it = 0; it < 8; ++it) cp_async16(dst + (it * 16 + (t >> 3)) * 128 + (t & 7) * 16, src + (size_t)it * 16 * K);
     }
-    cp_async4(swb + b * PT + t, s_w + n0 + t);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  float invA = 0.0f, invG = 0.0f;
-  bool fastA = false, fastG = false;
-  if (PASS == 1) {
-    const float a = __uint_as_float(amax[0]), g = __uint_as_float(amax[1]);
-    invA = (a > 0.0f) ? fdiv(127.0f, a) : 0.0f;
-    invG = (g > 0.0f) ? fdiv(127.0f, g) : 0.0f;
-    fastA = finite1(a) && finite1(invA);
-    fastG = finite1(g) && finite1(invG);
-  }
-  float maxA = 0.0f, maxG = 0.0f;
   if ((int)blockIdx.x < ntiles) issue(blockIdx.x, 0);
+  float inv[3] = {0.0f, 0.0f, 0.0f};                   // of A, G, Z
+  bool fast[3] = {false, false, false};
+  if (PASS == 1) {
+    uint32_t m[3] = {0u, 0u, 0u};
+    for (int i = t; i < max(p.mx.n[0], p.mx.n[2]); i += PT) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        if ((KIND == PREP_ONE || (k == 2) == (KIND == PREP_Z)) && i < p.mx.n[k]) m[k] = max(m[k], p.mx.part[k][i]);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (KIND != PREP_ONE && (k == 2) != (KIND == PREP_Z)) continue;
+      m[k] = block_max(m[k], box);
+      const float a = __uint_as_float(m[k]);
+      inv[k] = (a > 0.0f) ? fdiv(127.0f, a) : 0.0f;
+      fast[k] = finite1(a) && finite1(inv[k]);
+    }
+    if (blockIdx.x == 0 && t == 0) {
+      const float z = __uint_as_float(m[2]);
+      if (p.mx.final && KIND != PREP_Z) { p.mx.final[0] = m[0]; p.mx.final[1] = m[1]; }
+      if (p.mx.final && KIND != PREP_Y) p.mx.final[2] = (uint32_t)z;
+      if (p.s_u && KIND != PREP_Y) p.s_u[0] = (z > 0.0f) ? fdiv(z, 127.0f) : 0.0f;
+    }
+  }
+  float mx[3] = {0.0f, 0.0f, 0.0f};
   int i = 0;
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
     const int b = i & 1, next = tile + gridDim.x;
@@ -433,65 +394,131 @@ __global__ void __launch_bounds__(PT, 3) k_prep_dy2(const uint16_t* __restrict__
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     __syncthreads();                                   // tile i has landed for every thread
-    const uint8_t* buf = pbuf + b * (PT * 256);
-    const float* sw = swb + b * PT;
-    const int n0 = (tile % ntn) * PT, m0 = (tile / ntn) * PT;
-    float2 v[64];
-    uint32_t qa[32], qg[32];
-    // row t of the tile, scaled by the weight steps (scalar multiplies: the products are rounded before any add)
+    uint8_t* buf = pbuf + b * (PT * 256);
+    const bool isz = z_tile(tile);
+    uint32_t qa[32];
+    auto rotate = [&](int dir) {
+      float2 v[64];
+      if (dir == 0) {   // row t of the tile, scaled by the weight steps (scalar multiplies: the products are rounded before any add)
+        const float* sw = swb + b * PT;
 #pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const uint4 u = *reinterpret_cast<const uint4*>(buf + t * 256 + ((c ^ (t & 7)) << 4));
-      const float4 w0 = *reinterpret_cast<const float4*>(&sw[8 * c]), w1 = *reinterpret_cast<const float4*>(&sw[8 * c + 4]);
-      v[4 * c] = make_float2(fmul(bflo(u.x), w0.x), fmul(bfhi(u.x), w0.y));
-      v[4 * c + 1] = make_float2(fmul(bflo(u.y), w0.z), fmul(bfhi(u.y), w0.w));
-      v[4 * c + 2] = make_float2(fmul(bflo(u.z), w1.x), fmul(bfhi(u.z), w1.y));
-      v[4 * c + 3] = make_float2(fmul(bflo(u.w), w1.z), fmul(bfhi(u.w), w1.w));
-    }
-    wht128_pairs(v);
-    if (PASS == 0) maxA = fmaxf(maxA, absmax128(v));
-    else if (fastA && finite1(v[0].x)) quant_pack128<true>(v, invA, qa);
-    else quant_pack128<false>(v, invA, qa);
-    // column t of the tile, transposed output
-    const int cc = t >> 3, cw = (t & 7) * 2;
+        for (int c = 0; c < 16; ++c) {
+          const uint4 u = *reinterpret_cast<const uint4*>(buf + t * 256 + ((c ^ (t & 7)) << 4));
+          const float4 w0 = *reinterpret_cast<const float4*>(&sw[8 * c]), w1 = *reinterpret_cast<const float4*>(&sw[8 * c + 4]);
+          v[4 * c] = make_float2(fmul(bflo(u.x), w0.x), fmul(bfhi(u.x), w0.y));
+          v[4 * c + 1] = make_float2(fmul(bflo(u.y), w0.z), fmul(bfhi(u.y), w0.w));
+          v[4 * c + 2] = make_float2(fmul(bflo(u.z), w1.x), fmul(bfhi(u.z), w1.y));
+          v[4 * c + 3] = make_float2(fmul(bflo(u.w), w1.z), fmul(bfhi(u.w), w1.w));
+        }
+      } else if (dir == 1) {   // column t, transposed output
+        const int cc = t >> 3, cw = (t & 7) * 2;
 #pragma unroll
-    for (int p = 0; p < 64; ++p) {
-      const uint16_t lo = *reinterpret_cast<const uint16_t*>(buf + (2 * p) * 256 + ((cc ^ ((2 * p) & 7)) << 4) + cw);
-      const uint16_t hi = *reinterpret_cast<const uint16_t*>(buf + (2 * p + 1) * 256 + ((cc ^ ((2 * p + 1) & 7)) << 4) + cw);
-      v[p] = make_float2(bf2f(lo), bf2f(hi));
-    }
-    wht128_pairs(v);
-    if (PASS == 0) { maxG = fmaxf(maxG, absmax128(v)); continue; }
-    if (fastG && finite1(v[0].x)) quant_pack128<true>(v, invG, qg);
-    else quant_pack128<false>(v, invG, qg);
-    // hand-over through the consumed buffer: two tiles of 128 rows x 128 bytes, sixteen-byte pieces XOR-swizzled by row
-    __syncthreads();
-    uint8_t* stg = pbuf + b * (PT * 256);
+        for (int q = 0; q < 64; ++q) {
+          const uint16_t lo = *reinterpret_cast<const uint16_t*>(buf + (2 * q) * 256 + ((cc ^ ((2 * q) & 7)) << 4) + cw);
+          const uint16_t hi = *reinterpret_cast<const uint16_t*>(buf + (2 * q + 1) * 256 + ((cc ^ ((2 * q + 1) & 7)) << 4) + cw);
+          v[q] = make_float2(bf2f(lo), bf2f(hi));
+        }
+      } else {
+        const float2 off = make_float2(-8388736.0f, -8388736.0f);
 #pragma unroll
-    for (int g = 0; g < 8; ++g) {
-      const int off = t * 128 + ((g ^ (t & 7)) << 4);
-      *reinterpret_cast<uint4*>(stg + off) = make_uint4(qa[4 * g], qa[4 * g + 1], qa[4 * g + 2], qa[4 * g + 3]);
-      *reinterpret_cast<uint4*>(stg + 16384 + off) = make_uint4(qg[4 * g], qg[4 * g + 1], qg[4 * g + 2], qg[4 * g + 3]);
-    }
-    __syncthreads();
+        for (int q = 0; q < 64; ++q)
+          v[q] = __fadd2_rn(make_float2(__uint_as_float(buf[2 * q * 128 + t] ^ 0x4b000080u),
+                                        __uint_as_float(buf[(2 * q + 1) * 128 + t] ^ 0x4b000080u)), off);
+      }
+      wht128_pairs(v);
+      if (PASS == 0) {
+        const float m = absmax128(v);
+        if (dir == 0) mx[0] = fmaxf(mx[0], m);
+        else if (dir == 1) mx[1] = fmaxf(mx[1], m);
+        else mx[2] = fmaxf(mx[2], m);
+        return;
+      }
+      uint32_t q[32];
+      const float iv = dir == 0 ? inv[0] : (dir == 1 ? inv[1] : inv[2]);
+      if ((dir == 0 ? fast[0] : (dir == 1 ? fast[1] : fast[2])) && finite1(v[0].x)) quant_pack128<true>(v, iv, q);
+      else quant_pack128<false>(v, iv, q);
+      if (dir == 0) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int idx = k * PT + t, r = idx >> 3, piece = idx & 7;
-      const int off = r * 128 + ((piece ^ (r & 7)) << 4);
-      *reinterpret_cast<uint4*>(Aq + (size_t)(m0 + r) * N + n0 + piece * 16) = *reinterpret_cast<const uint4*>(stg + off);
-      *reinterpret_cast<uint4*>(GqT + (size_t)(n0 + r) * M + m0 + piece * 16) = *reinterpret_cast<const uint4*>(stg + 16384 + off);
+        for (int k = 0; k < 32; ++k) qa[k] = q[k];
+        return;
+      }
+      // hand-over through the consumed buffer: tiles of 128 rows x 128 bytes, sixteen-byte pieces XOR-swizzled by row
+      __syncthreads();
+#pragma unroll
+      for (int g = 0; g < 8; ++g) {
+        const int off = t * 128 + ((g ^ (t & 7)) << 4);
+        *reinterpret_cast<uint4*>(buf + off) = make_uint4(q[4 * g], q[4 * g + 1], q[4 * g + 2], q[4 * g + 3]);
+        if (dir == 1) *reinterpret_cast<uint4*>(buf + 16384 + off) = make_uint4(qa[4 * g], qa[4 * g + 1], qa[4 * g + 2], qa[4 * g + 3]);
+      }
+      __syncthreads();
+      const int z = tile - ntiles_y, m0 = (isz ? z / ntk : tile / ntn) * PT, c0 = (isz ? z % ntk : tile % ntn) * PT;
+      int8_t* dst = (isz ? p.ZqT : p.GqT) + (size_t)c0 * M + m0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int idx = k * PT + t, rr = idx >> 3, piece = idx & 7;
+        const int off = rr * 128 + ((piece ^ (rr & 7)) << 4);
+        *reinterpret_cast<uint4*>(dst + (size_t)rr * M + piece * 16) = *reinterpret_cast<const uint4*>(buf + off);
+        if (dir == 1) *reinterpret_cast<uint4*>(p.Aq + (size_t)(m0 + rr) * N + c0 + piece * 16) = *reinterpret_cast<const uint4*>(buf + 16384 + off);
+      }
+    };
+    if (KIND == PREP_Y) {
+      rotate(0);
+      rotate(1);
+    } else if (KIND == PREP_Z) {
+      rotate(2);
+    } else {
+#pragma unroll 1
+      for (int dir = isz ? 2 : 0; dir < (isz ? 3 : 2); ++dir) rotate(dir);
     }
   }
   if (PASS == 0) {
-    amax_publish(maxA, amax + 0);
-    amax_publish(maxG, amax + 1);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (KIND != PREP_ONE && (k == 2) != (KIND == PREP_Z)) continue;
+      const uint32_t x = block_max(__float_as_uint(mx[k]), box);     // non-negative floats order as integers
+      if (t) continue;
+      if (p.mx.n[k] > 1) p.mx.part[k][blockIdx.x] = x;
+      else if (x > *reinterpret_cast<volatile uint32_t*>(p.mx.part[k])) atomicMax(p.mx.part[k], x);
+    }
   }
 }
-
-__global__ void k_su_finish(const uint32_t* amax, int rotated, float* s_u) {
-  if (!rotated) { s_u[0] = 1.0f; return; }
-  const int am = (int)amax[0];
-  s_u[0] = (am > 0) ? fdiv(__int2float_rn(am), 127.0f) : 0.0f;
+template <int KIND>
+static int prep_pass(int pass, const PrepArgs& p, int grid, cudaStream_t st) {
+  static DevOnce once0 = {}, once1 = {};
+  const auto kern = pass ? k_prep<1, KIND> : k_prep<0, KIND>;
+  if (dev_ensure_smem(pass ? once1 : once0, (const void*)kern, PREP2_SMEM) != DET_OK) return DET_ERR_CUDA;
+  kern<<<DET_L(grid), PT, PREP2_SMEM, st>>>(p);
+  return DET_OK;
+}
+// both passes, three CTAs per SM or one per tile; `words` of scratch for the maxima
+static int prep_launch(PrepArgs p, uint32_t* scratch, int words, cudaStream_t st) {
+  const int sms = dev_sm_count();
+  if (sms <= 0) return DET_ERR_CUDA;
+  const long long ty = p.dY ? (long long)(p.M / PT) * (p.N / PT) : 0, tz = (long long)(p.M / PT) * (p.K / PT);
+  const bool one = ty + tz <= 3 * sms;
+  const int gy = one ? (int)(ty + tz) : (int)(ty < 3 * sms ? ty : 3 * sms), gz = one ? gy : (int)(tz < 3 * sms ? tz : 3 * sms);
+  const int n[3] = {gy, gy, gz};
+  const bool room = 2 * gy + gz <= words;
+  for (int k = 0, at = 0; k < 3; at += p.mx.n[k++]) {
+    p.mx.n[k] = room ? n[k] : 1;
+    p.mx.part[k] = scratch + at;
+  }
+  if ((!room || gy <= 1 || gz <= 1) && cudaMemsetAsync(scratch, 0, 4 * (size_t)(p.mx.n[0] + p.mx.n[1] + p.mx.n[2]), st) != cudaSuccess)
+    return DET_ERR_CUDA;
+  if (one) {
+    const int rc = prep_pass<PREP_ONE>(0, p, gy, st);
+    return rc != DET_OK ? rc : prep_pass<PREP_ONE>(1, p, gy, st);
+  }
+  AuxScope aux(st);   // the tiles of Z do not depend on those of dY
+  for (int pass = 0; pass < 2; ++pass) {
+    if (ty) {
+      const int rc = prep_pass<PREP_Y>(pass, p, gy, st);
+      if (rc != DET_OK) return rc;
+    }
+    const int rc = prep_pass<PREP_Z>(pass, p, gz, ty ? aux.aux(1) : st);
+    if (rc != DET_OK) return rc;
+  }
+  return aux.join() ? DET_OK : DET_ERR_CUDA;
 }
 
 }  // namespace det
@@ -549,16 +576,14 @@ extern "C" int det_lsq_quantize_weight(const det_bf16* W, const float* s_w, int 
   const size_t n16 = (size_t)N * K / 16;
   k_quantize<<<DET_L((unsigned)((n16 + 255) / 256)), 256, 0, st>>>(W, n16, K / 16, s_w, 1, qW);
   if (qWt_bwd) {
-    uint32_t* amax = (uint32_t*)ws;
-    cudaMemsetAsync(amax, 0, 256, st);
-    dim3 grid(K / 128, N / 128);
     if (hadamard_block) {
-      k_rotc8<0, true><<<DET_L(grid), 128, 0, st>>>(qW, N, K, amax, nullptr);
-      k_rotc8<1, true><<<DET_L(grid), 128, 0, st>>>(qW, N, K, amax, qWt_bwd);
+      PrepArgs pa = {};
+      pa.Z = qW; pa.M = N; pa.K = K; pa.ZqT = qWt_bwd; pa.s_u = s_u;
+      const int rc = prep_launch(pa, (uint32_t*)ws, 64, st);
+      if (rc != DET_OK) return rc;
     } else {
-      k_rotc8<1, false><<<DET_L(grid), 128, 0, st>>>(qW, N, K, amax, qWt_bwd);
+      k_transpose8<<<DET_L(dim3(K / 128, N / 128)), 128, 0, st>>>(qW, N, K, qWt_bwd, s_u);
     }
-    k_su_finish<<<DET_L(1), 1, 0, st>>>(amax, hadamard_block != 0, s_u);
   }
   DET_CHECK_LAUNCH();
   return DET_OK;
@@ -626,33 +651,23 @@ extern "C" int det_linear_bwd(const det_bf16* dY, const det_bf16* X, const int8_
   float* partial = (float*)(base + oP);
   float* sscr = (float*)(base + oS);
   const bool rot = hadamard_block != 0;
-  cudaMemsetAsync(amax, 0, 256, st);
-  const size_t ngrp = (size_t)M * ((N / 128 + 7) / 8);  // warp groups of 8 blocks
-  const unsigned g1 = (unsigned)((ngrp + 7) / 8);
-  dim3 gG(N / 128, M / 128), gZ(K / 128, M / 128);
   if (rot) {
-    static DevOnce once0 = {}, once1 = {};
-    if (dev_ensure_smem(once0, (const void*)k_prep_dy2<0>, PREP2_SMEM) != DET_OK ||
-        dev_ensure_smem(once1, (const void*)k_prep_dy2<1>, PREP2_SMEM) != DET_OK)
-      return DET_ERR_CUDA;
-    const int sms = dev_sm_count();
-    if (sms <= 0) return DET_ERR_CUDA;
-    const int ptiles = (M / PT) * (N / PT);
-    const unsigned gP = (unsigned)(ptiles < 3 * sms ? ptiles : 3 * sms);   // persistent: three CTAs per SM
-    // the rotation of the saved int8 activations does not depend on dY: it runs beside the two passes over dY
-    AuxScope az(st);
-    cudaStream_t sz = az.aux(1);
-    k_prep_dy2<0><<<DET_L(gP), PT, PREP2_SMEM, st>>>(dY, s_w, M, N, amax, nullptr, nullptr);
-    k_rotc8<0, true><<<DET_L(gZ), 128, 0, sz>>>(qX, M, K, amax + 2, nullptr);
-    k_prep_dy2<1><<<DET_L(gP), PT, PREP2_SMEM, st>>>(dY, s_w, M, N, amax, Aq, GqT);
-    k_rotc8<1, true><<<DET_L(gZ), 128, 0, sz>>>(qX, M, K, amax + 2, ZqT);
-    if (!az.join()) return DET_ERR_CUDA;
+    // the maxima of pass 0 lie in dW until the weight-gradient GEMM writes it (N K >= 16384 values)
+    PrepArgs pa = {};
+    pa.dY = dY; pa.s_w = s_w; pa.Z = qX; pa.M = M; pa.N = N; pa.K = K; pa.Aq = Aq; pa.GqT = GqT; pa.ZqT = ZqT;
+    pa.mx.final = amax;
+    const int rc = prep_launch(pa, (uint32_t*)dW, 16384, st);
+    if (rc != DET_OK) return rc;
   } else {
-    k_rot_rows<0, false><<<DET_L(g1), 256, 0, st>>>(dY, s_w, M, N, amax + 0, nullptr);
-    k_rotc<true, 0, false><<<DET_L(gG), 128, 0, st>>>(dY, M, N, amax + 1, nullptr);
-    k_rot_rows<1, false><<<DET_L(g1), 256, 0, st>>>(dY, s_w, M, N, amax + 0, Aq);
-    k_rotc<true, 1, false><<<DET_L(gG), 128, 0, st>>>(dY, M, N, amax + 1, GqT);
-    k_rotc8<1, false><<<DET_L(gZ), 128, 0, st>>>(qX, M, K, amax + 2, ZqT);
+    cudaMemsetAsync(amax, 0, 256, st);
+    const size_t ngrp = (size_t)M * ((N / 128 + 7) / 8);  // warp groups of 8 blocks
+    const unsigned g1 = (unsigned)((ngrp + 7) / 8);
+    dim3 gG(N / 128, M / 128);
+    k_rot_rows<0><<<DET_L(g1), 256, 0, st>>>(dY, s_w, M, N, amax + 0, nullptr);
+    k_rotc<0><<<DET_L(gG), 128, 0, st>>>(dY, M, N, amax + 1, nullptr);
+    k_rot_rows<1><<<DET_L(g1), 256, 0, st>>>(dY, s_w, M, N, amax + 0, Aq);
+    k_rotc<1><<<DET_L(gG), 128, 0, st>>>(dY, M, N, amax + 1, GqT);
+    k_transpose8<<<DET_L(dim3(K / 128, M / 128)), 128, 0, st>>>(qX, M, K, ZqT, nullptr);
   }
   DET_CHECK_LAUNCH();
   const float rotf = rot ? 0x1p-7f : 1.0f;

@@ -192,6 +192,29 @@ def test_adamw_many_tensors(det, sizes, clip):
         assert_same_bits(host(dv[i]), vo, "v %d" % i)
 
 
+# the rotated transposed weight codes, two columns per integer: codes at both ends of the range (all of one sign, so that the plain
+# sum is +-2^14), a column block without a partner, more than one tile per CTA
+@pytest.mark.parametrize("N,K", [(128, 128), (256, 384), (3072, 8320)])
+def test_weight_rotation(det, N, K):
+    rng = np.random.default_rng(N + K)
+    W = np.where(rng.random((N, K)) < 0.5, -1.0, 1.0)
+    W[:, 0], W[:, 1], W[:128, K - 1] = 1.0, -1.0, -1.0
+    W[:, 2:64:3] = 1e-3 * rng.integers(-128, 128, (N, len(range(2, 64, 3))))
+    q = np.clip(np.rint(synth.from_bf16(synth.to_bf16(W.astype(F))) * (F(1.0) / F(1e-3))), -128, 127).astype(np.int64)
+    v = q.reshape(N // 128, 128, K)
+    for h in (1, 2, 4, 8, 16, 32, 64):
+        v = v.reshape(N // 128, 64 // h, 2, h, K)
+        v = np.stack((v[:, :, 0] + v[:, :, 1], v[:, :, 0] - v[:, :, 1]), axis=2).reshape(N // 128, 128, K)
+    am = np.abs(v).max()
+    want = np.rint(v.astype(F) * (F(127.0) / F(am))).astype(np.int8).reshape(N, K).T
+    qW, qWt, s_u = empty((N, K), np.int8), empty((K, N), np.int8), empty((1,), F)
+    det.det_lsq_quantize_weight(dev(synth.to_bf16(W.astype(F))), dev(np.full(N, 1e-3, F)), N, K, 128, qW, qWt, s_u, ws(256))
+    _sync()
+    assert_same_bits(host(qW, np.int8), q.astype(np.int8), "codes")
+    assert_same_bits(host(qWt, np.int8), np.ascontiguousarray(want), "rotated codes")
+    assert_same_bits(host(s_u), np.array([F(am) / F(127.0)], F), "step")
+
+
 # LSQ linear at sizes where the tile of the int8 GEMMs changes (64, 128, 256 columns, CTA pairs), with a last round that is
 # nearly empty and with dimensions that only narrow tiles divide
 @pytest.mark.parametrize("M,N,K", [(128, 128, 128), (384, 640, 384), (1024, 3072, 1024), (1664, 3072, 1024)])
