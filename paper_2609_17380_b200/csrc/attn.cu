@@ -294,6 +294,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
 // Delta_i = adjacent tree over the 128 dims of dO_ic * O_ic; one warp per (b, h, i)
 __global__ void __launch_bounds__(256) k_attn_delta(const uint16_t* __restrict__ dout, const uint16_t* __restrict__ out,
                                                     int ld_out, int H, int S, size_t nrows, float* __restrict__ delta) {
+  grid_dep();
   const size_t w = (size_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= nrows) return;  // w = (b*H + h)*S + i
@@ -687,7 +688,7 @@ static int attn_bwd_impl(const det_bf16* dout, const det_bf16* q, const det_bf16
   uint16_t* dSt = (uint16_t*)((uint8_t*)ws + matP);
   float* delta = (float*)((uint8_t*)ws + matP + matS);
   const size_t nrows = (size_t)B * H * S;
-  k_attn_delta<<<DET_L((unsigned)((nrows + 7) / 8)), 256, 0, st>>>(dout, out, ld_out, H, S, nrows, delta);
+  launch_after(k_attn_delta, (unsigned)((nrows + 7) / 8), 256, 0, st, dout, out, ld_out, H, S, nrows, delta);
   DET_CHECK_LAUNCH();
   // P[i,j] = exp(scale * sum_d q[i,d] k[j,d] - L_i) for visible (i,j) (f32; tiles without a visible pair are never
   // touched) and dS[i,j] = bf16((P[i,j] * (sum_d dO[i,d] v[j,d] - Delta_i)) * scale); both sums ascend over the 128 dims

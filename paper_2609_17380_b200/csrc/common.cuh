@@ -248,6 +248,16 @@ __device__ __forceinline__ void smem_tree(float* buf, int n) {
 }
 
 constexpr int SUM_CHUNK = 16384;
+// First thing, by every thread, in a kernel launched by launch_after: the kernel before it on the stream is complete and its results
+// are visible when this returns, and the next one may start coming in.  Before it, a kernel may only touch what is older than
+// the kernel before, or its own shared memory.  Returns 0, as a value that exists only after the wait: an index that it is
+// added to keeps a load of constant data that opens the kernel behind the wait.
+__device__ __forceinline__ int grid_dep() {
+  int zero;
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;\n\tmov.u32 %0, 0;" : "=r"(zero) : : "memory");
+  return zero;
+}
+
 // The sum of chunk `base` .. base + SUM_CHUNK of x[0..n): a perfect subtree, or the ragged last one with existence
 // predicates.  All 256 threads of the CTA call it; thread 0 gets the result.
 // The ragged form deals its leaves out over the warps (a sum of 2048 values has eight: one warp walking them behind scalar

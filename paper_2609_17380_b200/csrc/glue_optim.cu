@@ -23,6 +23,7 @@ __device__ __forceinline__ uint4 pack8(const float v[8]) {
 __global__ void __launch_bounds__(256) k_swiglu_fwd(const uint16_t* __restrict__ gu, int rows, int F,
                                                     uint16_t* __restrict__ h, const float* __restrict__ s_q = nullptr,
                                                     int8_t* __restrict__ qh = nullptr) {
+  grid_dep();
   const size_t per_row = (size_t)F / 8;
   size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= per_row * rows) return;
@@ -43,6 +44,7 @@ __global__ void __launch_bounds__(256) k_swiglu_fwd(const uint16_t* __restrict__
 
 __global__ void __launch_bounds__(256) k_swiglu_bwd(const uint16_t* __restrict__ dh, const uint16_t* __restrict__ gu,
                                                     int rows, int F, uint16_t* __restrict__ dgu) {
+  grid_dep();
   const size_t per_row = (size_t)F / 8;
   size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= per_row * rows) return;
@@ -74,7 +76,7 @@ __global__ void __launch_bounds__(256) k_residual(const uint16_t* a, const uint1
 
 __global__ void __launch_bounds__(256) k_embed_fwd(const int32_t* __restrict__ tok, const uint16_t* __restrict__ E, int V,
                                                    int D, uint16_t* __restrict__ y) {
-  const int t = blockIdx.x;
+  const int t = blockIdx.x + grid_dep();
   int v = tok[t];
   v = v < 0 ? 0 : (v >= V ? V - 1 : v);
   const uint4* src = reinterpret_cast<const uint4*>(E + (size_t)v * D);
@@ -89,7 +91,7 @@ __global__ void __launch_bounds__(256) k_embed_bwd(const int32_t* __restrict__ t
   __shared__ int s_flag;
   __shared__ int s_list[256];
   __shared__ int s_cnt;
-  const int p = blockIdx.x;
+  const int p = blockIdx.x + grid_dep();
   const int v = tok[p];
   if (v < 0 || v >= V) return;
   if (threadIdx.x == 0) s_flag = 0;
@@ -157,6 +159,7 @@ struct AccumOp {
   float* dst;
 };
 __global__ void __launch_bounds__(256) k_accum(AccumOp op, size_t n) {
+  grid_dep();
   size_t i = ((size_t)blockIdx.x * 256 + threadIdx.x) * 4;
   if (i >= n) return;
   float4 g = *reinterpret_cast<const float4*>(op.g + i);
@@ -193,6 +196,7 @@ struct ResultOp {
 // The parameter struct stays in constant space and the loop runs over the partials there are: unrolled to the 34 there may be,
 // the 33 tests per thread held the pass at 3.1 TB/s (6.6 TB/s now, 188 M values).
 __global__ void __launch_bounds__(256) k_accum_result(const __grid_constant__ ResultOp op, size_t n) {
+  grid_dep();
   size_t i = ((size_t)blockIdx.x * 256 + threadIdx.x) * 4;
   if (i >= n) return;
   float4 a = *reinterpret_cast<const float4*>(op.part[0] + i);
@@ -271,6 +275,7 @@ __device__ __forceinline__ void adam_block(const AdamScalars& h, float c, void* 
 }
 template <bool CLIP>
 __global__ void __launch_bounds__(256) k_adamw(const __grid_constant__ AdamJobs jobs, const float* __restrict__ coef) {
+  grid_dep();
   int lo = 0, hi = jobs.n - 1;         // the last job whose first block is <= this one
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -300,7 +305,7 @@ extern "C" int det_swiglu_fwd(const det_bf16* gu, int rows, int F, det_bf16* h, 
   if (!aligned16(gu) || !aligned16(h)) return DET_ERR_ALIGN;
   size_t n = (size_t)rows * (F / 8);
   if (!n) return DET_OK;
-  k_swiglu_fwd<<<DET_L((unsigned)((n + 255) / 256)), 256, 0, (cudaStream_t)stream>>>(gu, rows, F, h);
+  launch_after(k_swiglu_fwd, (unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream, gu, rows, F, h, nullptr, nullptr);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
@@ -310,7 +315,7 @@ extern "C" int det_swiglu_fwd_q(const det_bf16* gu, int rows, int F, det_bf16* h
   if (!aligned16(gu) || !aligned16(h) || (((uintptr_t)qh) & 7u)) return DET_ERR_ALIGN;
   size_t n = (size_t)rows * (F / 8);
   if (!n) return DET_OK;
-  k_swiglu_fwd<<<DET_L((unsigned)((n + 255) / 256)), 256, 0, (cudaStream_t)stream>>>(gu, rows, F, h, s_q, qh);
+  launch_after(k_swiglu_fwd, (unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream, gu, rows, F, h, s_q, qh);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
@@ -320,7 +325,7 @@ extern "C" int det_swiglu_bwd(const det_bf16* dh, const det_bf16* gu, int rows, 
   if (!aligned16(gu) || !aligned16(dh) || !aligned16(dgu)) return DET_ERR_ALIGN;
   size_t n = (size_t)rows * (F / 8);
   if (!n) return DET_OK;
-  k_swiglu_bwd<<<DET_L((unsigned)((n + 255) / 256)), 256, 0, (cudaStream_t)stream>>>(dh, gu, rows, F, dgu);
+  launch_after(k_swiglu_bwd, (unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream, dh, gu, rows, F, dgu);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
@@ -338,7 +343,7 @@ extern "C" int det_embed_fwd(const int32_t* tok, int T, const det_bf16* E, int V
   if (D % 8) return DET_ERR_SHAPE;
   if (!aligned16(E) || !aligned16(y)) return DET_ERR_ALIGN;
   if (!T) return DET_OK;
-  k_embed_fwd<<<DET_L(T), 256, 0, (cudaStream_t)stream>>>(tok, E, V, D, y);
+  launch_after(k_embed_fwd, T, 256, 0, (cudaStream_t)stream, tok, E, V, D, y);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
@@ -348,7 +353,7 @@ extern "C" int det_embed_bwd(const int32_t* tok, int T, const det_bf16* dy, int 
   if (!aligned16(dy) || !aligned16(dE)) return DET_ERR_ALIGN;
   cudaStream_t st = (cudaStream_t)stream;
   cudaMemsetAsync(dE, 0, (size_t)V * D * sizeof(float), st);
-  if (T) k_embed_bwd<<<DET_L(T), 256, 0, st>>>(tok, T, dy, V, D, dE);
+  if (T) launch_after(k_embed_bwd, T, 256, 0, st, tok, T, dy, V, D, dE);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
@@ -428,7 +433,7 @@ extern "C" int det_grad_accum_push(det_accum* st, const float* g, void* stream) 
   }
   if (dst_slot < 0) return DET_ERR_ARG;
   op.dst = st->bufs + (size_t)dst_slot * n;
-  if (n) k_accum<<<DET_L((unsigned)((n / 4 + 255) / 256)), 256, 0, (cudaStream_t)stream>>>(op, n);
+  if (n) launch_after(k_accum, (unsigned)((n / 4 + 255) / 256), 256, 0, (cudaStream_t)stream, op, n);
   for (int l = 0; l < npop; ++l) st->free_mask |= (1ull << popped[l]);
   st->pushes++;
   DET_CHECK_LAUNCH();
@@ -444,7 +449,7 @@ extern "C" int det_grad_accum_result(det_accum* st, float* g_out, void* stream) 
   for (int s = 0; s < st->nstack; ++s) op.part[s] = st->bufs + (size_t)st->slot[st->nstack - 1 - s] * st->n;
   op.inv_rep = (float)(1.0 / (double)st->dp_replicate);
   op.dst = g_out;
-  if (st->n) k_accum_result<<<DET_L((unsigned)((st->n / 4 + 255) / 256)), 256, 0, (cudaStream_t)stream>>>(op, st->n);
+  if (st->n) launch_after(k_accum_result, (unsigned)((st->n / 4 + 255) / 256), 256, 0, (cudaStream_t)stream, op, st->n);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
@@ -494,8 +499,8 @@ extern "C" int det_adamw_batch(const det_adamw_desc* descs, const int* pdtypes, 
     }
     if (!jobs.n) break;
     jobs.first[jobs.n] = (uint32_t)c;
-    if (coef_dev) k_adamw<true><<<DET_L((unsigned)c), 256, 0, (cudaStream_t)stream>>>(jobs, coef_dev);
-    else k_adamw<false><<<DET_L((unsigned)c), 256, 0, (cudaStream_t)stream>>>(jobs, nullptr);
+    if (coef_dev) launch_after(k_adamw<true>, (unsigned)c, 256, 0, (cudaStream_t)stream, jobs, coef_dev);
+    else launch_after(k_adamw<false>, (unsigned)c, 256, 0, (cudaStream_t)stream, jobs, nullptr);
     DET_CHECK_LAUNCH();
   }
   return DET_OK;

@@ -110,6 +110,7 @@ __device__ __forceinline__ ShaMsg sha_msg(const HashJobs& jobs, uint32_t chunk) 
 // instruction per cycle and scheduler make 0.87 TB/s the ceiling at 1.965 GHz, and 1 GiB is hashed at 0.84 TB/s (additions
 // written as integer multiply-adds, meant for another pipe, measured 0.81: they take the same issue slots).
 __global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJobs jobs, uint8_t* __restrict__ out) {
+  grid_dep();
   const uint32_t c = blockIdx.x * 64 + threadIdx.x;
   if (c >= jobs.first[jobs.n]) return;
   const ShaMsg msg = sha_msg<false>(jobs, c);
@@ -152,6 +153,7 @@ __global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJ
 constexpr int SF_CH = 8, SF_PITCH = 68;
 template <bool ROOT>
 __global__ void __launch_bounds__(32) k_sha_few(const __grid_constant__ HashJobs jobs, uint8_t* __restrict__ out) {
+  grid_dep();
   __shared__ __align__(16) uint32_t ws[4 * SF_CH * SF_PITCH];
   constexpr uint32_t K[64] = {SHA_K_LIST};
   const int ch = threadIdx.x >> 2, sub = threadIdx.x & 3;
@@ -235,8 +237,8 @@ static int hash_level(const HashJobs& jobs, uint8_t* out, cudaStream_t st) {
   if (!n) return DET_OK;
   const int sms = dev_sm_count();
   if (sms <= 0) return DET_ERR_CUDA;
-  if (n <= (uint32_t)sms * 4 * SF_CH) k_sha_few<false><<<DET_L((n + SF_CH - 1) / SF_CH), 32, 0, st>>>(jobs, out);
-  else k_sha_chunks<<<DET_L((n + 63) / 64), 64, 0, st>>>(jobs, out);
+  if (n <= (uint32_t)sms * 4 * SF_CH) launch_after(k_sha_few<false>, (n + SF_CH - 1) / SF_CH, 32, 0, st, jobs, out);
+  else launch_after(k_sha_chunks, (n + 63) / 64, 64, 0, st, jobs, out);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
@@ -305,7 +307,7 @@ extern "C" int det_tensor_hash_batch(const void* const* ptrs, const size_t* nbyt
       out += c * 32;
       lv.n = m;
     }
-    k_sha_few<true><<<DET_L((n + SF_CH - 1) / SF_CH), 32, 0, st>>>(root, roots_dev + (size_t)t0 * 32);
+    launch_after(k_sha_few<true>, (n + SF_CH - 1) / SF_CH, 32, 0, st, root, roots_dev + (size_t)t0 * 32);
     DET_CHECK_LAUNCH();
   }
   return DET_OK;

@@ -13,6 +13,7 @@ constexpr int HD = 128;
 // times 2^-7.  Lane l holds elements 4l .. 4l+3.
 __global__ void __launch_bounds__(256) k_headnorm_fwd(const uint16_t* __restrict__ x, int ld, size_t nrows, int nh, float eps,
                                                       uint16_t* __restrict__ y, int ld_y, float* __restrict__ rstd) {
+  grid_dep();
   const size_t w = (size_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= nrows) return;
@@ -33,6 +34,7 @@ __global__ void __launch_bounds__(256) k_headnorm_fwd(const uint16_t* __restrict
 __global__ void __launch_bounds__(256) k_headnorm_bwd(const uint16_t* __restrict__ dy, int ld_dy, const uint16_t* __restrict__ x,
                                                       int ld, const float* __restrict__ rstd, size_t nrows, int nh,
                                                       uint16_t* __restrict__ dx, int ld_dx) {
+  grid_dep();
   const size_t w = (size_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= nrows) return;
@@ -59,6 +61,7 @@ __global__ void __launch_bounds__(256) k_headnorm_bwd(const uint16_t* __restrict
 __global__ void __launch_bounds__(256) k_rope(const uint16_t* __restrict__ x, int ld, size_t nrows, int nh, int S,
                                               const float* __restrict__ cs, const float* __restrict__ sn, int inverse,
                                               uint16_t* __restrict__ y, int ld_y) {
+  grid_dep();
   const size_t w = (size_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= nrows) return;
@@ -90,7 +93,7 @@ extern "C" int det_headnorm_fwd(const det_bf16* x, int ld, int T, int nh, float 
   if (!head_args_ok(ld, T, nh) || !head_args_ok(ld_y, T, nh)) return DET_ERR_SHAPE;
   if ((((uintptr_t)x) | ((uintptr_t)y)) & 7u) return DET_ERR_ALIGN;
   const size_t nrows = (size_t)T * nh;
-  k_headnorm_fwd<<<DET_L((unsigned)((nrows + 7) / 8)), 256, 0, (cudaStream_t)stream>>>(x, ld, nrows, nh, eps, y, ld_y, rstd);
+  launch_after(k_headnorm_fwd, (unsigned)((nrows + 7) / 8), 256, 0, (cudaStream_t)stream, x, ld, nrows, nh, eps, y, ld_y, rstd);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
@@ -101,7 +104,7 @@ extern "C" int det_headnorm_bwd(const det_bf16* dy, int ld_dy, const det_bf16* x
   if (!head_args_ok(ld, T, nh) || !head_args_ok(ld_dy, T, nh) || !head_args_ok(ld_dx, T, nh)) return DET_ERR_SHAPE;
   if ((((uintptr_t)x) | ((uintptr_t)dy) | ((uintptr_t)dx)) & 7u) return DET_ERR_ALIGN;
   const size_t nrows = (size_t)T * nh;
-  k_headnorm_bwd<<<DET_L((unsigned)((nrows + 7) / 8)), 256, 0, (cudaStream_t)stream>>>(dy, ld_dy, x, ld, rstd, nrows, nh, dx,
+  launch_after(k_headnorm_bwd, (unsigned)((nrows + 7) / 8), 256, 0, (cudaStream_t)stream, dy, ld_dy, x, ld, rstd, nrows, nh, dx,
                                                                                      ld_dx);
   DET_CHECK_LAUNCH();
   return DET_OK;
@@ -113,7 +116,7 @@ extern "C" int det_rope(const det_bf16* x, int ld, int T, int nh, int S, const f
   if (!head_args_ok(ld, T, nh) || !head_args_ok(ld_y, T, nh)) return DET_ERR_SHAPE;
   if (((((uintptr_t)x) | ((uintptr_t)y)) & 3u) || ((((uintptr_t)cos_tab) | ((uintptr_t)sin_tab)) & 7u)) return DET_ERR_ALIGN;
   const size_t nrows = (size_t)T * nh;
-  k_rope<<<DET_L((unsigned)((nrows + 7) / 8)), 256, 0, (cudaStream_t)stream>>>(x, ld, nrows, nh, S, cos_tab, sin_tab, inverse, y,
+  launch_after(k_rope, (unsigned)((nrows + 7) / 8), 256, 0, (cudaStream_t)stream, x, ld, nrows, nh, S, cos_tab, sin_tab, inverse, y,
                                                                             ld_y);
   DET_CHECK_LAUNCH();
   return DET_OK;

@@ -205,6 +205,7 @@ __global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
+  grid_dep();
 
   const int tiles_i = I / BM, tiles_j = J / BN;
   const int num_tiles = tiles_i * tiles_j;
@@ -387,6 +388,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
   cluster_sync_all();  // the peer's barriers are initialised before anything can signal them
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
+  grid_dep();
 
   const int tiles_i = I / 256, tiles_j = J / BN2;
   const int num_tiles = tiles_i * tiles_j;
@@ -514,7 +516,7 @@ static int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const EpiPar
   if (sms <= 0) return DET_ERR_CUDA;
   const int tiles = (I / BM) * (J / BN);
   const int grid = tiles < sms ? tiles : sms;
-  k_igemm<BN, EPI><<<DET_L(grid), T::THREADS, T::SMEM, st>>>(ta, tb, ep, I, J, K, status);
+  launch_after(k_igemm<BN, EPI>, grid, T::THREADS, T::SMEM, st, ta, tb, ep, I, J, K, status);
   if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return DET_ERR_CUDA; }
   return DET_OK;
 }
@@ -530,7 +532,7 @@ static int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const EpiPa
   const int tiles = (I / 256) * (J / BN2);
   int clusters = sms / 2;
   if (tiles < clusters) clusters = tiles;
-  k_igemm2<EPI><<<DET_L(2 * clusters), GEMM2_THREADS, smem, st>>>(ta, tb, ep, I, J, K, status);
+  launch_after(k_igemm2<EPI>, 2 * clusters, GEMM2_THREADS, smem, st, ta, tb, ep, I, J, K, status);
   if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return DET_ERR_CUDA; }
   return DET_OK;
 }

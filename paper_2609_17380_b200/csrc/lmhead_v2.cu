@@ -38,6 +38,7 @@ __device__ __forceinline__ void load8_bits(const void* X, size_t idx, uint32_t (
 template <bool F32, int WPR>
 __global__ void __launch_bounds__(256) k_slice_rows(const void* __restrict__ X, int R, int K, int8_t* __restrict__ hi,
                                                     int8_t* __restrict__ lo, int32_t* __restrict__ E) {
+  grid_dep();
   __shared__ int key_s[8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = WPR == 1 ? (int)blockIdx.x * 8 + warp : (int)blockIdx.x;
@@ -83,8 +84,8 @@ __global__ void __launch_bounds__(256) k_slice_rows(const void* __restrict__ X, 
 template <bool F32>
 static void slice_rows_launch(const void* X, int R, int K, int8_t* hi, int8_t* lo, int32_t* E, cudaStream_t st) {
   // eight warps per row once a row holds a few rounds for each of them, unless a warp per row fills the GPU anyway
-  if (K >= 4096 && R < 64 * 4 * dev_sm_count()) k_slice_rows<F32, 8><<<DET_L(R), 256, 0, st>>>(X, R, K, hi, lo, E);
-  else k_slice_rows<F32, 1><<<DET_L((R + 7) / 8), 256, 0, st>>>(X, R, K, hi, lo, E);
+  if (K >= 4096 && R < 64 * 4 * dev_sm_count()) launch_after(k_slice_rows<F32, 8>, R, 256, 0, st, X, R, K, hi, lo, E);
+  else launch_after(k_slice_rows<F32, 1>, (R + 7) / 8, 256, 0, st, X, R, K, hi, lo, E);
 }
 
 // Slicing along the OTHER index, for the gradient contractions: the exponent of column c is taken over the rows r, and the
@@ -94,7 +95,7 @@ static void slice_rows_launch(const void* X, int R, int K, int8_t* hi, int8_t* l
 //                 registers as packed bytes, out through a swizzled shared-memory tile as whole 128-byte lines
 template <bool F32>
 __global__ void __launch_bounds__(128) k_col_exp(const void* __restrict__ X, int R, int C, int32_t* __restrict__ E) {
-  const int c = blockIdx.x * 128 + threadIdx.x, r0 = blockIdx.y * 128;
+  const int c = blockIdx.x * 128 + threadIdx.x + grid_dep(), r0 = blockIdx.y * 128;
   int key = 0;
 #pragma unroll 8
   for (int i = 0; i < 128; ++i) {
@@ -109,7 +110,7 @@ template <bool F32>
 __global__ void __launch_bounds__(128) k_slice_cols(const void* __restrict__ X, int R, int C, const int32_t* __restrict__ E,
                                                     int8_t* __restrict__ hiT, int8_t* __restrict__ loT) {
   __shared__ __align__(16) uint8_t tile[2][128 * 128];
-  const int t = threadIdx.x, c0 = blockIdx.x * 128, r0 = blockIdx.y * 128;
+  const int t = threadIdx.x, c0 = blockIdx.x * 128 + grid_dep(), r0 = blockIdx.y * 128;
   const int e = E[c0 + t] & 0xFF;
   uint32_t hw[32], lw[32];
 #pragma unroll
@@ -197,6 +198,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
+  grid_dep();
   const int tiles_i = I / SL_T, tiles_j = J / SL_T, per_z = tiles_i * tiles_j, num_tiles = p.Z * per_z, kblocks = K / SL_BK;
   // tile t -> problem z, row tile it, column tile jt (the rows run fastest: the CTAs resident at one time share a tile of
   // B and stream A through L2); false when the tile does not exist; [k_lo, k_hi) = its steps along the contraction
@@ -355,7 +357,7 @@ int sliced_gemm_launch(const int8_t* Ah, const int8_t* Al, const int8_t* Bh, con
   const int sms = dev_sm_count();
   if (sms <= 0) return DET_ERR_CUDA;
   const long long tiles = (long long)p.Z * (p.I / SL_T) * (p.J / SL_T);
-  k_igemm_sl<<<DET_L((unsigned)(tiles < sms ? tiles : sms)), SL_THREADS, SL_SMEM, st>>>(tAh, tAl, tBh, tBl, p, status);
+  launch_after(k_igemm_sl, (unsigned)(tiles < sms ? tiles : sms), SL_THREADS, SL_SMEM, st, tAh, tAl, tBh, tBl, p, status);
   if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return DET_ERR_CUDA; }
   return DET_OK;
 }
@@ -437,12 +439,12 @@ extern "C" int det_lmhead_bwd_v2(const float* dlogits, const det_bf16* H, const 
   int32_t *Eg = (int32_t*)(b + o[8]), *EgT = (int32_t*)(b + o[9]), *EWT = (int32_t*)(b + o[10]), *EHT = (int32_t*)(b + o[11]);
   cudaMemsetAsync(EgT, 0, o[11] - o[9] + align_up((size_t)K * 4, 256), st);        // the three column-exponent arrays
   slice_rows_launch<true>(dlogits, M, V, gh, gl, Eg, st);
-  k_col_exp<true><<<DET_L(dim3(V / 128, M / 128)), 128, 0, st>>>(dlogits, M, V, EgT);
-  k_col_exp<false><<<DET_L(dim3(K / 128, V / 128)), 128, 0, st>>>(W, V, K, EWT);
-  k_col_exp<false><<<DET_L(dim3(K / 128, M / 128)), 128, 0, st>>>(H, M, K, EHT);
-  k_slice_cols<true><<<DET_L(dim3(V / 128, M / 128)), 128, 0, st>>>(dlogits, M, V, EgT, gTh, gTl);
-  k_slice_cols<false><<<DET_L(dim3(K / 128, V / 128)), 128, 0, st>>>(W, V, K, EWT, WTh, WTl);
-  k_slice_cols<false><<<DET_L(dim3(K / 128, M / 128)), 128, 0, st>>>(H, M, K, EHT, HTh, HTl);
+  launch_after(k_col_exp<true>, dim3(V / 128, M / 128), 128, 0, st, dlogits, M, V, EgT);
+  launch_after(k_col_exp<false>, dim3(K / 128, V / 128), 128, 0, st, W, V, K, EWT);
+  launch_after(k_col_exp<false>, dim3(K / 128, M / 128), 128, 0, st, H, M, K, EHT);
+  launch_after(k_slice_cols<true>, dim3(V / 128, M / 128), 128, 0, st, dlogits, M, V, EgT, gTh, gTl);
+  launch_after(k_slice_cols<false>, dim3(K / 128, V / 128), 128, 0, st, W, V, K, EWT, WTh, WTl);
+  launch_after(k_slice_cols<false>, dim3(K / 128, M / 128), 128, 0, st, H, M, K, EHT, HTh, HTl);
   DET_CHECK_LAUNCH();
   // dH[m,k] = bf16(contraction over the vocabulary of row m of g with column k of W)
   int rc = sliced_gemm<true>(gh, gl, WTh, WTl, Eg, EWT, dH, M, K, V, status_dev, st);

@@ -17,6 +17,7 @@ __device__ __forceinline__ void unpack8u(const uint4& u, float v[8]) {
 // per output channel: one warp per row of W, K <= 8192
 __global__ void __launch_bounds__(256) k_wscale_rows(const uint16_t* __restrict__ W, int N, int K, float invK,
                                                      float* __restrict__ s_w) {
+  grid_dep();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = blockIdx.x * 8 + warp;
   if (row >= N) return;
@@ -81,6 +82,7 @@ __global__ void k_scale_finish(const float* sum, float inv_n, float* out, int co
 // rows x cols bf16 -> int8, step per row (per_row) or one step for the tensor; cols % 16 == 0
 __global__ void __launch_bounds__(256) k_quantize(const uint16_t* __restrict__ X, size_t n16, int cols16,
                                                   const float* __restrict__ s, int per_row, int8_t* __restrict__ q) {
+  grid_dep();
   size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= n16) return;
   const float inv = fdiv(1.0f, s[per_row ? (i / cols16) : 0]);
@@ -357,7 +359,9 @@ __global__ void __launch_bounds__(PT, 3) k_prep(const __grid_constant__ PrepArgs
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  if ((int)blockIdx.x < ntiles) issue(blockIdx.x, 0);
+  if (PASS == 0) grid_dep();
+  if ((int)blockIdx.x < ntiles) issue(blockIdx.x, 0);     // the second pass reads what is older than the first
+  if (PASS == 1) grid_dep();
   float inv[3] = {0.0f, 0.0f, 0.0f};                   // of A, G, Z
   bool fast[3] = {false, false, false};
   if (PASS == 1) {
@@ -487,7 +491,7 @@ static int prep_pass(int pass, const PrepArgs& p, int grid, cudaStream_t st) {
   static DevOnce once0 = {}, once1 = {};
   const auto kern = pass ? k_prep<1, KIND> : k_prep<0, KIND>;
   if (dev_ensure_smem(pass ? once1 : once0, (const void*)kern, PREP2_SMEM) != DET_OK) return DET_ERR_CUDA;
-  kern<<<DET_L(grid), PT, PREP2_SMEM, st>>>(p);
+  launch_after(kern, grid, PT, PREP2_SMEM, st, p);
   return DET_OK;
 }
 // both passes, three CTAs per SM or one per tile; `words` of scratch for the maxima
@@ -550,7 +554,7 @@ extern "C" int det_lsq_weight_scale(const det_bf16* W, int N, int K, int per_ten
     if (!ws || ws_bytes < det_lsq_weight_scale_ws_bytes(N, K)) return DET_ERR_WORKSPACE;
     abs_mean_scale(W, (size_t)N * K, s_w, N, (float*)ws, st);
   } else {
-    k_wscale_rows<<<DET_L((N + 7) / 8), 256, 0, st>>>(W, N, K, (float)(1.0 / (double)K), s_w);
+    launch_after(k_wscale_rows, (N + 7) / 8, 256, 0, st, W, N, K, (float)(1.0 / (double)K), s_w);
   }
   DET_CHECK_LAUNCH();
   return DET_OK;
@@ -574,7 +578,7 @@ extern "C" int det_lsq_quantize_weight(const det_bf16* W, const float* s_w, int 
   if (qWt_bwd && (!ws || ws_bytes < 256)) return DET_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   const size_t n16 = (size_t)N * K / 16;
-  k_quantize<<<DET_L((unsigned)((n16 + 255) / 256)), 256, 0, st>>>(W, n16, K / 16, s_w, 1, qW);
+  launch_after(k_quantize, (unsigned)((n16 + 255) / 256), 256, 0, st, W, n16, K / 16, s_w, 1, qW);
   if (qWt_bwd) {
     if (hadamard_block) {
       PrepArgs pa = {};
@@ -597,7 +601,7 @@ extern "C" int det_linear_fwd(const det_bf16* X, const int8_t* qW, const float* 
   if (!aligned16(X) || !aligned16(qW) || !aligned16(Y) || !aligned16(qX_save) || !aligned16(s_w)) return DET_ERR_ALIGN;
   cudaStream_t st = (cudaStream_t)stream;
   const size_t n16 = (size_t)M * K / 16;
-  k_quantize<<<DET_L((unsigned)((n16 + 255) / 256)), 256, 0, st>>>(X, n16, K / 16, s_x, 0, qX_save);
+  launch_after(k_quantize, (unsigned)((n16 + 255) / 256), 256, 0, st, X, n16, K / 16, s_x, 0, qX_save);
   DET_CHECK_LAUNCH();
   EpiParams ep = {};
   ep.out = Y; ep.s_x = s_x; ep.s_w = s_w;

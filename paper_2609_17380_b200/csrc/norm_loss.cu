@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(256, 4) k_rmsnorm_fwd8(const void* __restrict_
                                                          float* __restrict__ rstd, const float* __restrict__ s_q = nullptr,
                                                          int8_t* __restrict__ qy = nullptr, const void* __restrict__ res = nullptr,
                                                          void* __restrict__ sum = nullptr) {
+  grid_dep();
   __shared__ float leaf_sum[2][4][8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int e0 = warp * 256 + lane * 8;
@@ -133,6 +134,7 @@ __global__ void __launch_bounds__(256, 3) k_rmsnorm_bwd8(const void* __restrict_
                                                         const void* __restrict__ gamma, const float* __restrict__ rstd,
                                                         int rows, int D, float invD, void* dx, const void* res,
                                                         float* __restrict__ partial8, int* __restrict__ tickets) {
+  grid_dep();
   constexpr int RPP = BF ? 4 : 2, NPASS = 8 / RPP;
   __shared__ float leaf_sum[2][RPP][8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -141,7 +143,6 @@ __global__ void __launch_bounds__(256, 3) k_rmsnorm_bwd8(const void* __restrict_
   const bool full = (D & 255) == 0;
   const long long r0 = (long long)blockIdx.x * 8;
   if (DG && blockIdx.x == 0 && (int)threadIdx.x < ((D + 255) >> 8)) tickets[threadIdx.x] = 0;   // for the kernel that follows
-  if (DG) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // its blocks may start coming in; they wait for this grid
   float pair0[8], node[8];                        // column tree: a pair of rows waiting for the next pair; rows 0 .. 3
 #pragma unroll
   for (int t = 0; t < 8; ++t) { pair0[t] = 0.0f; node[t] = 0.0f; }
@@ -239,9 +240,7 @@ __global__ void __launch_bounds__(256) k_colsum32(const float* __restrict__ part
   __shared__ int last_s;
   const int col = blockIdx.x * 256 + threadIdx.x;
   const int g = blockIdx.y;
-  // launched as a programmatic dependent of the kernel that writes partial8: its blocks may be resident before that
-  // kernel has drained; nothing of its results is read before this wait returns
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  grid_dep();
   if (col < D) {
     float s[32];
 #pragma unroll
@@ -467,7 +466,7 @@ __global__ void __launch_bounds__(XT) k_xent_fwd(const float* __restrict__ logit
   extern __shared__ float leafs[];  // ceil(V/256) floats, >= 32
   __shared__ float red[XT / 32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const float* z = logits + (size_t)blockIdx.x * V;
+  const float* z = logits + (size_t)(blockIdx.x + grid_dep()) * V;
   float m = __int_as_float(0xff800000);
   {
     auto ld4 = [&](const float* p) { return *reinterpret_cast<const float4*>(p); };
@@ -548,6 +547,7 @@ __global__ void __launch_bounds__(XT) k_xent_fwd(const float* __restrict__ logit
 // the last levels of both sums (n <= SUM_CHUNK nodes each) and the means
 __global__ void __launch_bounds__(256) k_xent_finish(const float* __restrict__ ce, const float* __restrict__ zsq, int n, float inv_rows,
                                                      float z_weight, float* loss_mean, float* z_mean) {
+  grid_dep();
   __shared__ float wsum[SUM_LEAVES];
   const float c = fmul(chunk_sum<false>(ce, 0, n, wsum), inv_rows);
   __syncthreads();
@@ -563,6 +563,7 @@ __global__ void __launch_bounds__(256) k_xent_finish(const float* __restrict__ c
 // general form for its eight values.
 __global__ void __launch_bounds__(256) k_xent_bwd(float* __restrict__ logits, const int32_t* __restrict__ target,
                                                   const float* __restrict__ lse, int rows, int V, float z_weight, float scale) {
+  grid_dep();
   const int i0 = blockIdx.x * 2048 + threadIdx.x * 4;
   if (i0 >= V) return;
   const bool two = i0 + 1024 < V;
@@ -618,10 +619,10 @@ extern "C" int det_rmsnorm_fwd(int io, const void* x, const void* gamma, int row
   const float invD = (float)(1.0 / (double)D);
   dim3 grid((rows + 7) / 8);
   if (io == DET_BF16) {
-    if (D <= 2048) k_rmsnorm_fwd8<true><<<DET_L(grid), 256, 0, st>>>(x, gamma, rows, D, eps, invD, y, rstd);
+    if (D <= 2048) launch_after(k_rmsnorm_fwd8<true>, grid, 256, 0, st, x, gamma, rows, D, eps, invD, y, rstd, nullptr, nullptr, nullptr, nullptr);
     else k_rmsnorm_fwd<true, 0><<<DET_L(grid), 256, 0, st>>>(x, gamma, rows, D, eps, invD, y, rstd);
   } else {
-    if (D <= 2048) k_rmsnorm_fwd8<false><<<DET_L(grid), 256, 0, st>>>(x, gamma, rows, D, eps, invD, y, rstd);
+    if (D <= 2048) launch_after(k_rmsnorm_fwd8<false>, grid, 256, 0, st, x, gamma, rows, D, eps, invD, y, rstd, nullptr, nullptr, nullptr, nullptr);
     else k_rmsnorm_fwd<false, 0><<<DET_L(grid), 256, 0, st>>>(x, gamma, rows, D, eps, invD, y, rstd);
   }
   DET_CHECK_LAUNCH();
@@ -634,8 +635,8 @@ extern "C" int det_rmsnorm_fwd_q(const det_bf16* x, const det_bf16* gamma, int r
   if (D % 8 || D > 2048) return DET_ERR_SHAPE;
   if (!aligned16(x) || !aligned16(y) || (gamma && !aligned16(gamma)) || (((uintptr_t)qy) & 7u)) return DET_ERR_ALIGN;
   if (rows == 0) return DET_OK;
-  k_rmsnorm_fwd8<true><<<DET_L((rows + 7) / 8), 256, 0, (cudaStream_t)stream>>>(x, gamma, rows, D, eps, (float)(1.0 / (double)D), y,
-                                                                              rstd, s_q, qy);
+  launch_after(k_rmsnorm_fwd8<true>, (rows + 7) / 8, 256, 0, (cudaStream_t)stream, x, gamma, rows, D, eps, (float)(1.0 / (double)D), y,
+                                                                              rstd, s_q, qy, nullptr, nullptr);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
@@ -650,30 +651,17 @@ static int rmsnorm_bwd8_launch(const void* dy, const void* x, const void* gamma,
                                float invD, void* dx, const void* res, float* dgamma, float* ws, cudaStream_t st) {
   const int nb8 = (rows + 7) / 8, nb256 = (rows + 255) / 256;
   if (!dgamma) {
-    k_rmsnorm_bwd8<BF, false><<<DET_L(nb8), 256, 0, st>>>(dy, x, gamma, rstd, rows, D, invD, dx, res, nullptr, nullptr);
+    launch_after(k_rmsnorm_bwd8<BF, false>, nb8, 256, 0, st, dy, x, gamma, rstd, rows, D, invD, dx, res, nullptr, nullptr);
     return DET_OK;
   }
   float* partial8 = ws;
   float* partial256 = ws + align_up((size_t)nb8 * D, 64);
   int* tickets = reinterpret_cast<int*>(partial256 + align_up((size_t)nb256 * D, 64));   // one per block of 256 columns (<= 8)
-  k_rmsnorm_bwd8<BF, true><<<DET_L(nb8), 256, 0, st>>>(dy, x, gamma, rstd, rows, D, invD, dx, res, partial8, tickets);
+  launch_after(k_rmsnorm_bwd8<BF, true>, nb8, 256, 0, st, dy, x, gamma, rstd, rows, D, invD, dx, res, partial8, tickets);
   // the second launch overlaps its start-up with the first kernel's tail (programmatic dependent launch); the kernel
   // itself waits for the first grid to complete before it reads anything
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((D + 255) / 256, nb256);
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  note_launch();
-  if (cudaLaunchKernelEx(&cfg, k_colsum32, (const float*)partial8, nb8, rows, D, partial256, nb256, tickets, dgamma) != cudaSuccess) {
-    cudaGetLastError();
-    return DET_ERR_CUDA;
-  }
+  launch_after(k_colsum32, dim3((D + 255) / 256, nb256), 256, 0, st, (const float*)partial8, nb8, rows, D, partial256, nb256, tickets, dgamma);
+  DET_CHECK_LAUNCH();
   return DET_OK;
 }
 
@@ -717,7 +705,7 @@ extern "C" int det_residual_rmsnorm_fwd(const det_bf16* a, const det_bf16* b, co
   if (!aligned16(a) || !aligned16(b) || !aligned16(sum) || !aligned16(y) || (gamma && !aligned16(gamma)) || (((uintptr_t)qy) & 7u))
     return DET_ERR_ALIGN;
   if (rows == 0) return DET_OK;
-  k_rmsnorm_fwd8<true><<<DET_L((rows + 7) / 8), 256, 0, (cudaStream_t)stream>>>(a, gamma, rows, D, eps, (float)(1.0 / (double)D), y,
+  launch_after(k_rmsnorm_fwd8<true>, (rows + 7) / 8, 256, 0, (cudaStream_t)stream, a, gamma, rows, D, eps, (float)(1.0 / (double)D), y,
                                                                               rstd, s_q, qy, b, sum);
   DET_CHECK_LAUNCH();
   return DET_OK;
@@ -758,13 +746,13 @@ extern "C" int det_xent_fwd(const float* logits, const int32_t* target, int rows
   float* scratch = zsq + align_up((size_t)rows, 64);
   const int nl = (V + 255) / 256;
   size_t sh = (size_t)(nl < 32 ? 32 : nl) * sizeof(float);
-  k_xent_fwd<<<DET_L(rows), XT, sh, st>>>(logits, target, V, loss_row, lse, zsq, status_dev);
+  launch_after(k_xent_fwd, rows, XT, sh, st, logits, target, V, loss_row, lse, zsq, status_dev);
   const float* ce = loss_row;
   const float* zs = zsq;
   size_t n = (size_t)rows, nz = (size_t)rows;
   sum_to_chunk(ce, n, scratch, st);
   sum_to_chunk(zs, nz, scratch, st);
-  k_xent_finish<<<DET_L(1), 256, 0, st>>>(ce, zs, (int)n, (float)(1.0 / (double)rows), z_weight, loss_mean, z_mean);
+  launch_after(k_xent_finish, 1, 256, 0, st, ce, zs, (int)n, (float)(1.0 / (double)rows), z_weight, loss_mean, z_mean);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
@@ -775,7 +763,7 @@ extern "C" int det_xent_bwd(float* logits_inout, const int32_t* target, const fl
   if (V % 4) return DET_ERR_SHAPE;
   if (!aligned16(logits_inout)) return DET_ERR_ALIGN;
   dim3 grid((V + 2047) / 2048, rows < 65535 ? rows : 65535);
-  k_xent_bwd<<<DET_L(grid), 256, 0, (cudaStream_t)stream>>>(logits_inout, target, lse, rows, V, z_weight, scale);
+  launch_after(k_xent_bwd, grid, 256, 0, (cudaStream_t)stream, logits_inout, target, lse, rows, V, z_weight, scale);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }

@@ -88,6 +88,7 @@ unsigned long long launches() { return g_launches.load(std::memory_order_relaxed
 
 template <bool SQ>
 __global__ void __launch_bounds__(256) k_sum_chunk(const float* __restrict__ x, long long n, float* __restrict__ partial) {
+  grid_dep();
   __shared__ float wsum[SUM_LEAVES];
   const float r = chunk_sum<SQ>(x, (long long)blockIdx.x * SUM_CHUNK, n, wsum);
   if (threadIdx.x == 0) partial[blockIdx.x] = r;
@@ -106,6 +107,7 @@ struct SumJobs {
 };
 template <bool SQ>
 __global__ void __launch_bounds__(256) k_sum_jobs(const __grid_constant__ SumJobs jobs, float* __restrict__ out, float* __restrict__ per) {
+  grid_dep();
   __shared__ float wsum[SUM_LEAVES];
   int lo = 0, hi = jobs.n - 1;         // the last job whose first block is <= this one
   while (lo < hi) {
@@ -140,8 +142,8 @@ int sum_launch(const float* x, size_t n, int squares, float* out, float* ws, cud
   while (true) {
     long long c = nchunks(cur);
     float* dst = (c == 1) ? out : w;
-    if (sq) k_sum_chunk<true><<<DET_L((unsigned)c), 256, 0, st>>>(src, cur, dst);
-    else k_sum_chunk<false><<<DET_L((unsigned)c), 256, 0, st>>>(src, cur, dst);
+    if (sq) launch_after(k_sum_chunk<true>, (unsigned)c, 256, 0, st, src, cur, dst);
+    else launch_after(k_sum_chunk<false>, (unsigned)c, 256, 0, st, src, cur, dst);
     if (c == 1) break;
     w += align_up((size_t)c, 64);
     src = dst;
@@ -153,6 +155,7 @@ int sum_launch(const float* x, size_t n, int squares, float* out, float* ws, cud
 
 // det_sum(x[0..n)), n <= SUM_CHUNK, times gs (the last levels of a sum and the scaling that follows it, in one launch)
 __global__ void __launch_bounds__(256) k_sum_scaled(const float* __restrict__ x, int n, float gs, float* __restrict__ out) {
+  grid_dep();
   __shared__ float wsum[SUM_LEAVES];
   const float r = chunk_sum<false>(x, 0, n, wsum);
   if (threadIdx.x == 0) out[0] = fmul(gs, r);
@@ -161,7 +164,7 @@ __global__ void __launch_bounds__(256) k_sum_scaled(const float* __restrict__ x,
 void sum_to_chunk(const float*& x, size_t& n, float*& ws, cudaStream_t st) {
   while (n > (size_t)SUM_CHUNK) {
     const size_t c = (size_t)nchunks((long long)n);
-    k_sum_chunk<false><<<DET_L((unsigned)c), 256, 0, st>>>(x, (long long)n, ws);
+    launch_after(k_sum_chunk<false>, (unsigned)c, 256, 0, st, x, (long long)n, ws);
     x = ws;
     ws += align_up(c, 64);
     n = c;
@@ -169,13 +172,14 @@ void sum_to_chunk(const float*& x, size_t& n, float*& ws, cudaStream_t st) {
 }
 int sum_scaled_launch(const float* x, size_t n, float gs, float* out, float* ws, cudaStream_t st) {
   sum_to_chunk(x, n, ws, st);
-  k_sum_scaled<<<DET_L(1), 256, 0, st>>>(x, (int)n, gs, out);
+  launch_after(k_sum_scaled, 1, 256, 0, st, x, (int)n, gs, out);
   return DET_OK;
 }
 
 // the tree over the per-tensor sums (n <= SUM_CHUNK), the norm and the clip coefficient
 __global__ void __launch_bounds__(256) k_norm_finish(const float* __restrict__ per, int n, float max_norm, float* norm_out,
                                                      float* coef_out, int* status) {
+  grid_dep();
   __shared__ float wsum[SUM_LEAVES];
   const float total = n ? chunk_sum<false>(per, 0, n, wsum) : 0.0f;
   if (threadIdx.x) return;
@@ -314,8 +318,8 @@ extern "C" int det_grad_norm(const float* const* g_ptrs, const size_t* n_elems, 
       }
       if (c > 0x7fffffffll) return DET_ERR_SHAPE;
       jobs.first[jobs.n] = (uint32_t)c;
-      if (sq) k_sum_jobs<true><<<DET_L((unsigned)c), 256, 0, st>>>(jobs, out, per);
-      else k_sum_jobs<false><<<DET_L((unsigned)c), 256, 0, st>>>(jobs, out, per);
+      if (sq) launch_after(k_sum_jobs<true>, (unsigned)c, 256, 0, st, jobs, out, per);
+      else launch_after(k_sum_jobs<false>, (unsigned)c, 256, 0, st, jobs, out, per);
       int m = 0;
       for (int j = 0; j < jobs.n; ++j)
         if (jobs.len[j] > SUM_CHUNK) { jobs.x[m] = out + jobs.first[j]; jobs.len[m] = nchunks(jobs.len[j]); jobs.who[m] = jobs.who[j]; ++m; }
@@ -331,7 +335,7 @@ extern "C" int det_grad_norm(const float* const* g_ptrs, const size_t* n_elems, 
     src = total;
     n = 1;
   }
-  k_norm_finish<<<DET_L(1), 256, 0, st>>>(src, n, max_norm, norm_out, coef_out, status_dev);
+  launch_after(k_norm_finish, 1, 256, 0, st, src, n, max_norm, norm_out, coef_out, status_dev);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
