@@ -35,46 +35,64 @@ namespace det {
 // Rows per CTA, ring slots, slabs in flight in the producers' registers, CTAs per SM, registers per consumer and producer thread after the hand-over.
 // A CTA of 128 rows has the best rate (25.1 us per row block and key block on a full GPU, against 13.2 us for 64 rows and
 // 7.5 us for 32), but its chain of key blocks is the longest: alone on its SM 25.1, 17 and 13 us per key block.
-template <int FQ_, int SLOTS_, int PF_, int CPS_, int RC_, int RP_>
+// GR groups of consumer and producer warps take the key blocks of the CTA's rows in turn: logits and P.V of a block need nothing of
+// the block before but its running maximum, which passes from warp to warp through shared memory, and group 1 hands its u, row
+// sums and rescale factors to group 0, which alone forms o and l, in block order.  Two groups shorten the chain, 13 to 9.9 us per
+// key block, and lose rate (9.8 against 7.5 us per 32 rows and key block): 8 heads x 1024 0.119 ms with 32 rows, 0.088 with two groups;
+// 16 x 832 0.119 and 0.117; two sequences of 8 x 1088 0.167 and 0.189.
+template <int FQ_, int SLOTS_, int PF_, int CPS_, int RC_, int RP_, int GR_ = 1>
 struct AfTile {
-  static constexpr int FQ = FQ_, LQ = FQ_ + 4, SLOTS = SLOTS_, PF = PF_, CPS = CPS_, RC = RC_, RP = RP_;
-  static constexpr int CONS = (FQ / AF_RW) * 32, THREADS = CONS + AF_PROD;
-  static constexpr size_t SMEM = (size_t)(DH * LQ + FK * FQ + SLOTS * OK * AF_BP) * sizeof(float);
+  static constexpr int FQ = FQ_, LQ = FQ_ + 4, SLOTS = SLOTS_, PF = PF_, CPS = CPS_, RC = RC_, RP = RP_, GR = GR_;
+  static constexpr int GCONS = (FQ / AF_RW) * 32, CONS = GR * GCONS, THREADS = CONS + GR * AF_PROD;
+  static constexpr size_t SMEM = (size_t)(DH * LQ + GR * (FK * FQ + SLOTS * OK * AF_BP) + (GR - 1) * FQ * DH) * sizeof(float);
   // setmaxnreg: the counts after the hand-over must fit into what the block was launched with, or the increase never returns
-  static_assert(CONS * RC + AF_PROD * RP <= (65536 / (CPS * THREADS) / 8 * 8) * THREADS, "register hand-over exceeds the block's allocation");
+  static_assert(CONS * RC + GR * AF_PROD * RP <= (65536 / (CPS * THREADS) / 8 * 8) * THREADS, "register hand-over exceeds the block's allocation");
 };
 typedef AfTile<128, 8, 4, 1, 104, 64> AfTall;
 typedef AfTile<64, 4, 2, 2, 96, 48> AfHalf;
 typedef AfTile<32, 4, 3, 3, 104, 56> AfShort;
+typedef AfTile<32, 4, 3, 1, 136, 64, 2> AfPair;
 
 template <class T, bool WIN>
 __global__ void __launch_bounds__(T::THREADS, T::CPS)
     k_attn_fwd(const uint16_t* __restrict__ q, const uint16_t* __restrict__ k, const uint16_t* __restrict__ v, int ld,
                int H, int Hkv, int S, int Warg, uint16_t* __restrict__ out, int ld_out, float* __restrict__ lse,
                const float* __restrict__ s_q, int8_t* __restrict__ qout) {
-  constexpr int FQ = T::FQ, LQ = T::LQ, AF_SLOTS = T::SLOTS, AF_PF = T::PF, AF_CONS = T::CONS, AF_THREADS = T::THREADS;
+  constexpr int FQ = T::FQ, LQ = T::LQ, AF_SLOTS = T::SLOTS, AF_PF = T::PF, AF_CONS = T::CONS, AF_THREADS = T::THREADS, GR = T::GR;
+  constexpr int GWARPS = T::GCONS / 32;
   const int W = WIN ? Warg : 0;
   extern __shared__ __align__(16) float sm[];
   float(*Qs)[LQ] = reinterpret_cast<float(*)[LQ]>(sm);                         // [dim][query]
-  float* Ps = sm + DH * LQ;                                                    // [key][query], 16-byte chunks swizzled
-  float(*Ring)[OK][AF_BP] = reinterpret_cast<float(*)[OK][AF_BP]>(sm + DH * LQ + FK * FQ);
-  __shared__ __align__(16) int tiny_s[AF_SLOTS][AF_PROD / 32];
+  __shared__ __align__(16) int tiny_g[GR][AF_SLOTS][AF_PROD / 32];
   __shared__ int tiny_q_s, abort_s;
-  __shared__ __align__(8) uint64_t bar_full[AF_SLOTS], bar_empty[AF_SLOTS];
+  __shared__ __align__(8) uint64_t full_g[GR][AF_SLOTS], empty_g[GR][AF_SLOTS];
+  // between the two groups, per warp: maxima passed on by either, group 1's sums and factors, "u is there", "u has been read"
+  __shared__ float max_g[GR][FQ], sum_g[FQ], alpha_g[FQ];
+  __shared__ __align__(8) uint64_t bar_max[GR][GWARPS], bar_u[GWARPS], bar_ufree[GWARPS];
   volatile int* abort_flag = &abort_s;
   const int qb = gridDim.y - 1 - blockIdx.y;          // longest rows first
   const int h = blockIdx.x % H, b = blockIdx.x / H, hk = h / (H / Hkv);
   const int q0 = qb * FQ;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int grp = GR == 1 ? 0 : (tid < AF_CONS ? tid / T::GCONS : (tid - AF_CONS) / AF_PROD), warp = (tid >> 5) - grp * GWARPS;   // consumers' warp
+  float* Ps = sm + DH * LQ + grp * (FK * FQ);                                  // [key][query], 16-byte chunks swizzled
+  float(*Ring)[OK][AF_BP] = reinterpret_cast<float(*)[OK][AF_BP]>(sm + DH * LQ + GR * FK * FQ) + grp * AF_SLOTS;
+  float4* U = reinterpret_cast<float4*>(sm + DH * LQ + GR * (FK * FQ + AF_SLOTS * OK * AF_BP));   // [4][thread of the group]
+  int(*tiny_s)[AF_PROD / 32] = tiny_g[grp];
+  uint64_t *bar_full = full_g[grp], *bar_empty = empty_g[grp];
   const size_t row0 = (size_t)b * S;
   const uint16_t* qp = q + row0 * ld + (size_t)h * DH;
   const uint16_t* kp = k + row0 * ld + (size_t)hk * DH;
   const uint16_t* vp = v + row0 * ld + (size_t)hk * DH;
-  const int jt0 = (WIN && q0 > W) ? (q0 - W) / FK : 0, ntiles = q0 / FK + 1;
+  const int jt0 = ((WIN && q0 > W) ? (q0 - W) / FK : 0) + grp, ntiles = q0 / FK + 1;   // this group's first block
   // the last block ends with the last slab of 16 value rows that the CTA's last query may see
-  const int nslab = (ntiles - jt0) * 16 - 7 + (q0 % FK + FQ - 1) / OK;
+  const int mine = ntiles > jt0 ? (ntiles - jt0 + GR - 1) / GR : 0;
+  const int nslab = mine * 16 - ((ntiles - 1 - jt0) % GR == 0 && mine ? 7 - (q0 % FK + FQ - 1) / OK : 0);
   if (tid == 0) {
-    for (int s = 0; s < AF_SLOTS; ++s) { mbar_init(&bar_full[s], AF_PROD / 32); mbar_init(&bar_empty[s], AF_CONS / 32); }
+    for (int g = 0; g < GR; ++g)
+      for (int s = 0; s < AF_SLOTS; ++s) { mbar_init(&full_g[g][s], AF_PROD / 32); mbar_init(&empty_g[g][s], GWARPS); }
+    if (GR > 1)
+      for (int w = 0; w < GWARPS; ++w) { mbar_init(&bar_max[0][w], 1); mbar_init(&bar_max[GR - 1][w], 1); mbar_init(&bar_u[w], 1); mbar_init(&bar_ufree[w], 1); }
     tiny_q_s = 0;
     abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -99,7 +117,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
   if (tid >= AF_CONS) {
     // ------------------------------- producers -------------------------------
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(T::RP));
-    const int pt = tid - AF_CONS, pw = pt >> 5;
+    const int pt = (tid - AF_CONS) % AF_PROD, pw = pt >> 5;
     // Slab s of the block sequence: block s / 16; s % 16 < 8: K, head dimensions 16 (s % 16) .. (thread = key, two
     // 16-byte words); else V, keys 16 (s % 16 - 8) .. (thread = four dimensions of keys kk, kk + 4, kk + 8, kk + 12).
     // AF_PF slabs are in flight in registers, so that the latency of a global load is spread over several slabs.
@@ -108,7 +126,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     const int vf = pt & 31, vk = pt >> 5;            // V: dimensions 4 vf .. 4 vf + 3 of keys vk, vk + 4, vk + 8, vk + 12
     auto fetch = [&](int sn, uint4 (&w)[2]) {
       if (sn >= nslab) return;
-      const int j0n = (jt0 + (sn >> 4)) * FK, phn = sn & 15;
+      const int j0n = (jt0 + GR * (sn >> 4)) * FK, phn = sn & 15;
       if (phn < 8) {
         const int key = j0n + pt;
         const uint4* src = reinterpret_cast<const uint4*>(kp + (size_t)key * ld + phn * OK);
@@ -196,7 +214,25 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     if (++slot == AF_SLOTS) slot = 0;
   };
   ok = acquire();
-  for (int jt = jt0; jt < ntiles && ok; ++jt) {
+  // o = o * alpha + u and l = l * alpha + sum of group 1's block of round `rd`
+  auto take = [&](int rd) -> bool {
+    if (!__all_sync(0xffffffffu, mbar_wait(&bar_u[warp], (uint32_t)rd & 1u, abort_flag, nullptr))) return false;
+    const int own = wrow + ROW_OF_LANE(lane);
+    l_mine = fadd(fmul(l_mine, alpha_g[own]), sum_g[own]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float2 al = same2(alpha_g[lrow + i]);
+      const float4 x = U[(2 * i) * T::GCONS + tid], y = U[(2 * i + 1) * T::GCONS + tid];
+      const float2 u[4] = {make_float2(x.x, x.y), make_float2(x.z, x.w), make_float2(y.x, y.y), make_float2(y.z, y.w)};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) o[i][j] = add2(mul2(o[i][j], al), u[j], one);
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&bar_ufree[warp]);
+    return true;
+  };
+  int rd = 0;
+  for (int jt = jt0; jt < ntiles && ok; jt += GR, ++rd) {
     const int j0 = jt * FK;
     const bool diag = (jt == ntiles - 1);           // only the last block of a row block reaches past the diagonal
     const bool edge = WIN && j0 <= q0 + FQ - 1 - W;  // some row's window starts inside or after this block
@@ -216,8 +252,20 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     }
     if (!ok) break;
     // ---- online softmax of the warp's 8 rows; the row sums take the weights before their rounding to bf16 ----
-    softmax_block(acc, j0 + 8 * tx, q0 + lrow, q0 + wrow + ROW_OF_LANE(lane), j0 + FK - 1, W, diag, edge, lane, m_mine, l_mine,
-                  alpha_mine, one);
+    const float sum = softmax_block(
+        acc, j0 + 8 * tx, q0 + lrow, q0 + wrow + ROW_OF_LANE(lane), j0 + FK - 1, W, diag, edge, lane, m_mine, alpha_mine, one,
+        [&](float m) {
+          if (GR == 1 || (grp == 0 && rd == 0)) return m;
+          ok = __all_sync(0xffffffffu, mbar_wait(&bar_max[GR - 1 - grp][warp], (uint32_t)(grp ? rd : rd - 1) & 1u, abort_flag, nullptr));
+          return max_g[GR - 1 - grp][wrow + ROW_OF_LANE(lane)];
+        },
+        [&](float m) {
+          if (GR == 1) return;
+          if (lane < AF_RW) max_g[grp][wrow + ROW_OF_LANE(lane)] = m;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bar_max[grp][warp]);
+        });
+    if (!ok) break;
     uint32_t tw = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -256,6 +304,20 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
       release();
     }
     if (!ok) break;
+    if (GR > 1 && grp == 1) {   // hand u over once the last one has been read
+      if (rd > 0 && !__all_sync(0xffffffffu, mbar_wait(&bar_ufree[warp], (uint32_t)(rd - 1) & 1u, abort_flag, nullptr))) { ok = false; break; }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        U[(2 * i) * T::GCONS + tid - T::GCONS] = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+        U[(2 * i + 1) * T::GCONS + tid - T::GCONS] = make_float4(acc[i][2].x, acc[i][2].y, acc[i][3].x, acc[i][3].y);
+      }
+      if (lane < AF_RW) { sum_g[wrow + ROW_OF_LANE(lane)] = sum; alpha_g[wrow + ROW_OF_LANE(lane)] = alpha_mine; }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar_u[warp]);
+      continue;
+    }
+    if (GR > 1 && rd > 0 && !take(rd - 1)) { ok = false; break; }
+    l_mine = fadd(fmul(l_mine, alpha_mine), sum);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {  // the product o * alpha is rounded before the add
       const float2 al = same2(__shfl_sync(0xffffffffu, alpha_mine, LANE_OF_ROW(i)));
@@ -263,7 +325,11 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
       for (int j = 0; j < 4; ++j) o[i][j] = add2(mul2(o[i][j], al), acc[i][j], one);
     }
   }
-  if (!ok) return;
+  if (!ok || grp) return;
+  if (GR > 1 && (ntiles - jt0) % GR == 0) {   // the last block was group 1's
+    if (!take(rd - 1)) return;
+    m_mine = max_g[GR - 1][wrow + ROW_OF_LANE(lane)];
+  }
   const float il_mine = fdiv(1.0f, l_mine);
   const float lse_mine = fadd(m_mine, det_log(l_mine));
   if (lane < AF_RW && q0 + wrow + ROW_OF_LANE(lane) < S) lse[((size_t)b * H + h) * S + q0 + wrow + ROW_OF_LANE(lane)] = lse_mine;
@@ -585,7 +651,7 @@ static int attn_fwd_run(const det_bf16* q, const det_bf16* k, const det_bf16* v,
 // GPU; the figures are the microseconds per key block of a CTA alone on its SM and of one among many, and the row count
 // with the smallest of the larger bounds is taken (16 heads x 832: 0.178 ms with 128 rows, 0.129 with 64, 0.117 with 32;
 // 64 heads x 2048: 1.48, 1.55 and 1.75 ms).
-struct RowCost { int rows; double alone, full; };
+struct RowCost { int rows; double alone, full; };   // rows: 33 for 32 rows with two groups
 template <int N>
 static int pick_rows(const RowCost (&c)[N], int heads, int S, int window) {
   const int sms = dev_sm_count() > 0 ? dev_sm_count() : 1;
@@ -593,7 +659,7 @@ static int pick_rows(const RowCost (&c)[N], int heads, int S, int window) {
   double best_t = 0.0;
   for (int i = 0; i < N; ++i) {
     double longest = 0.0, total = 0.0;
-    for (int q0 = 0; q0 < S; q0 += c[i].rows) {
+    for (int q0 = 0; q0 < S; q0 += c[i].rows & ~1) {
       const int lo = window && q0 > window ? (q0 - window) / FK : 0;
       const double tiles = q0 / FK + 1 - lo;
       total += tiles;
@@ -605,7 +671,7 @@ static int pick_rows(const RowCost (&c)[N], int heads, int S, int window) {
   return best;
 }
 static int attn_rows(int heads, int S, int window) {
-  const RowCost c[3] = {{128, 25.1, 25.1}, {64, 17.0, 13.2}, {32, 13.0, 7.5}};
+  const RowCost c[4] = {{128, 25.1, 25.1}, {64, 17.0, 13.2}, {32, 13.0, 7.5}, {33, 9.9, 9.8}};
   return pick_rows(c, heads, S, window);
 }
 static int attn_fwd_impl(const det_bf16* q, const det_bf16* k, const det_bf16* v, int ld, int B, int H, int Hkv, int S,
@@ -618,6 +684,7 @@ static int attn_fwd_impl(const det_bf16* q, const det_bf16* k, const det_bf16* v
   switch (attn_rows(B * H, S, window)) {
     case 128: rc = attn_fwd_run<AfTall>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, (cudaStream_t)stream); break;
     case 64: rc = attn_fwd_run<AfHalf>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, (cudaStream_t)stream); break;
+    case 33: rc = attn_fwd_run<AfPair>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, (cudaStream_t)stream); break;
     default: rc = attn_fwd_run<AfShort>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, (cudaStream_t)stream);
   }
   if (rc != DET_OK) return rc;

@@ -65,11 +65,13 @@ __device__ __forceinline__ float rows_reduce(const float (&x)[4], int lane) {
   return op(d, __shfl_xor_sync(0xffffffffu, d, 16));
 }
 // Online softmax of one key block for the warp's 8 rows: acc (the logits of rows `row` .. row + 3 and keys `key` .. key + 7 of this
-// lane, without the scale) becomes the weights exp(s - m), invisible pairs +0; the running maximum, row sum and
-// rescale factor of row ROW_OF_LANE(lane) of the warp (row `own`) are updated.  diag: the block reaches past some row; edge: some
+// lane, without the scale) becomes the weights exp(s - m), invisible pairs +0; the running maximum and the rescale factor of row
+// ROW_OF_LANE(lane) of the warp (row `own`) are updated, and the block's row sum is returned.  before(m) gives the maximum up to the
+// block before, after(m) takes the one up to this block (the identity and nothing where one warp sees all blocks).  diag: the block reaches past some row; edge: some
 // row's window starts inside or after it (last: the block's last key).
-__device__ __forceinline__ void softmax_block(float2 (&acc)[4][4], int key, int row, int own, int last, int W, bool diag, bool edge,
-                                              int lane, float& m_mine, float& l_mine, float& alpha_mine, float2 one) {
+template <class Before, class After>
+__device__ __forceinline__ float softmax_block(float2 (&acc)[4][4], int key, int row, int own, int last, int W, bool diag, bool edge,
+                                               int lane, float& m_mine, float& alpha_mine, float2 one, Before before, After after) {
   float rm[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -84,8 +86,9 @@ __device__ __forceinline__ void softmax_block(float2 (&acc)[4][4], int key, int 
   }
   // a row sees at least one key of a block it visits, so its maximum is a number; in a block that holds none of its keys its
   // statistics stay untouched
-  const float m_new = fmaxf(m_mine, rows_reduce<false>(rm, lane));
-  alpha_mine = det_exp_le0(fsub(m_mine, m_new));
+  const float m_block = rows_reduce<false>(rm, lane), m_old = before(m_mine), m_new = fmaxf(m_old, m_block);
+  after(m_new);
+  alpha_mine = det_exp_le0(fsub(m_old, m_new));
   if (edge && last <= own - W) alpha_mine = 1.0f;
   m_mine = m_new;
 #pragma unroll
@@ -119,7 +122,7 @@ __device__ __forceinline__ void softmax_block(float2 (&acc)[4][4], int key, int 
     rm[i] = fadd(fadd(fadd(acc[i][0].x, acc[i][0].y), fadd(acc[i][1].x, acc[i][1].y)),
                  fadd(fadd(acc[i][2].x, acc[i][2].y), fadd(acc[i][3].x, acc[i][3].y)));
   // the rest of the adjacent tree over the block's 128 slots: lanes 2, 4, 8, 16 apart
-  l_mine = fadd(fmul(l_mine, alpha_mine), rows_reduce<true>(rm, lane));
+  return rows_reduce<true>(rm, lane);
 }
 
 }  // namespace det

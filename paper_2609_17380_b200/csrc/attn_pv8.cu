@@ -258,8 +258,9 @@ __global__ void __launch_bounds__(PV_THREADS, 1)
       ok = __all_sync(0xffffffffu, ok);
       if (ok && t > 0) ok = collect(t - 1);
       if (!ok) break;
-      softmax_block(acc, j0 + 8 * tx, q0 + lrow, q0 + wrow + ROW_OF_LANE(lane), j0 + PK - 1, W, diag, edge, lane, m_mine, l_mine,
-                    alpha_mine, one);
+      const float sum = softmax_block(acc, j0 + 8 * tx, q0 + lrow, q0 + wrow + ROW_OF_LANE(lane), j0 + PK - 1, W, diag, edge, lane,
+                                      m_mine, alpha_mine, one, [](float m) { return m; }, [](float) {});
+      l_mine = fadd(fmul(l_mine, alpha_mine), sum);
       if (lane < AF_RW) alpha_s[t & 1][wrow + ROW_OF_LANE(lane)] = alpha_mine;
       // q_p = rne(127 p) of the lane's 4 x 8 weights (0 <= 127 p <= 127: adding 1.5 2^23 leaves the integer in the low byte)
 #pragma unroll
