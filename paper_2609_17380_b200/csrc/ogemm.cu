@@ -40,16 +40,16 @@ extern "C" int det_lmhead_bwd(const float* dlogits, const det_bf16* H, const det
   if (K % 16 || V % 16 || M % 8) return DET_ERR_SHAPE;
   if (!aligned16(dlogits) || !aligned16(H) || !aligned16(W) || !aligned16(dH) || !aligned16(dW)) return DET_ERR_ALIGN;
   cudaStream_t st = (cudaStream_t)stream;
-  AuxScope aux(st);   // the auxiliary streams start where the caller's stream stands now; joined on every way out
-  // dH[m,k] = sum over v ascending of bf16(dlogits[m,v]) * W[v,k]
-  int rc = ogemm_launch<CONTIG, STRIDED, true, true, 0>(plain_args(dlogits, W, dH, M, K, V, V, K, K, 0), 1, 1, st,
-                                                    (double)M * V * K / OG_RATES[0].full);   // beside the weight gradient
+  // dH[m,k] = sum over v ascending of bf16(dlogits[m,v]) * W[v,k]; dW[v,k] (+)= sum over m ascending of bf16(dlogits[m,v]) * H[m,k].
+  // The two are independent, and dW fills the SMs that dH leaves.  It must come second: with its CTAs first on the SMs the chains of dH
+  // start when dW is nearly done (384 tokens: 7.3 instead of 4.3 ms for head and loss, which two streams left to chance).
+  OgemmArgs h = plain_args(dlogits, W, dH, M, K, V, V, K, K, 0), w = plain_args(dlogits, H, dW, V, K, M, V, K, K, first_chunk ? 0 : 1);
+  h.order = OG_LEAD;
+  w.order = OG_FILL;
+  int rc = ogemm_launch<CONTIG, STRIDED, true, true, 0>(h, 1, 1, st, (double)M * V * K / OG_RATES[0].full);
   if (rc != DET_OK) return rc;
-  // dW[v,k] (+)= sum over m ascending of bf16(dlogits[m,v]) * H[m,k], beside the first kernel
-  rc = ogemm_launch<STRIDED, STRIDED, true, false, 0>(plain_args(dlogits, H, dW, V, K, M, V, K, K, first_chunk ? 0 : 1), 1, 1,
-                                                      aux.aux(0));
+  rc = ogemm_launch<STRIDED, STRIDED, true, false, 0>(w, 1, 1, st);
   if (rc != DET_OK) return rc;
-  if (!aux.join()) return DET_ERR_CUDA;
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
