@@ -145,9 +145,13 @@ class Replay:
         self.tmp = [e(T * max(QW, 2 * Fh), I16) for _ in range(3)]   # gradient scratch activations
         self.tok = e(T, I32)
         self.lab = e(T, I32)
-        self.norm, self.coef = e(1, F32), e(1, F32)
-        self.status = z(1, I32)
-        self.roots = z(32 * 8, torch.uint8)        # hash roots of one step, read back with one copy
+        # what a step reports lies in one buffer and comes back in one copy: status, norm and clip coefficient, hash roots, losses
+        nr, n_mb = 32 * (max(len(self.specs), 2) + 3), cfg.mesh[0] * cfg.mesh[1] * cfg.mesh[2]
+        self._out = z(16 + nr + 4 * n_mb, torch.uint8)
+        self.status = self._out[0:4].view(I32)
+        self.norm, self.coef = self._out[4:8].view(F32), self._out[8:12].view(F32)
+        self.roots = self._out[16:16 + nr]
+        self._losses = self._out[16 + nr:].view(F32)
         B, H, S = cfg.micro_batch, cfg.n_heads, cfg.seq
         wsb = max(det.det_attn_bwd_fixq_ws_bytes(B, H, S, Hkv) if cfg.dq_fixed else det.det_attn_bwd_ws_bytes(B, H, S, Hkv),
                   det.det_xent_ws_bytes(T, V), det.det_rmsnorm_bwd_ws_bytes(T, D),
@@ -304,8 +308,8 @@ class Replay:
         cfg = self.cfg
         D, Fh, V, L, T = cfg.d_model, cfg.ffn, cfg.vocab, cfg.n_layers, cfg.tokens_per_microbatch
         B, H, S = cfg.micro_batch, cfg.n_heads, cfg.seq
-        self.tok.copy_(tokens_mb[:, :-1].reshape(-1))
-        self.lab.copy_(tokens_mb[:, 1:].reshape(-1))
+        self.tok.view(B, S).copy_(tokens_mb[:, :-1])
+        self.lab.view(B, S).copy_(tokens_mb[:, 1:])
         Hkv, QW = cfg.kv_heads, cfg.qkv_width
         x = self.act[0]["x"] if L else self.xf
         if cfg.embed_norm:
@@ -440,15 +444,20 @@ class Replay:
         jobs = [(name, self.p(name)) for name, _, _ in self.specs] if per_tensor else [("params_bf16", self.pbf), ("steps_f32", self.sx)]
         return jobs + [("grad", self.gout), ("adam_m", self.m), ("adam_v", self.v)]
 
+    def _queue_hashes(self, per_tensor):
+        jobs = self._hash_jobs(per_tensor)
+        det.det_tensor_hash_batch([t for _, t in jobs], self.roots, self.ws)
+        return [name for name, _ in jobs]
+
+    @staticmethod
+    def _hex(names, raw):
+        return {name: raw[32 * i:32 * i + 32].hex() for i, name in enumerate(names)}
+
     def hashes(self, per_tensor=True):
         """State hashes of the step (Appendix B).  All of them are queued as one batch with the roots finished on the
         device; the roots come back in ONE copy, so the whole set costs one synchronisation."""
-        jobs = self._hash_jobs(per_tensor)
-        if self.roots.numel() < 32 * len(jobs):
-            self.roots = torch.empty(32 * len(jobs), dtype=torch.uint8, device=self.dev)
-        det.det_tensor_hash_batch([t for _, t in jobs], self.roots, self.ws)
-        raw = self.roots[:32 * len(jobs)].cpu().numpy().tobytes()
-        return {name: raw[32 * i:32 * i + 32].hex() for i, (name, _) in enumerate(jobs)}
+        names = self._queue_hashes(per_tensor)
+        return self._hex(names, self.roots.cpu().numpy().tobytes())
 
     def calibrate(self, tokens_mb):
         """Untimed: set every activation step from the first micro-batch (LSQ initialisation rule)."""
@@ -462,11 +471,12 @@ class Replay:
             self.prepare_weights()
         st = det.det_accum()
         det.det_grad_accum_init(st, cfg.mesh[0], cfg.mesh[1], cfg.mesh[2], self.n_grad, self.abufs)
-        losses = torch.empty(tokens.shape[0], dtype=F32, device=self.dev)
-        for mb in range(tokens.shape[0]):
+        n_mb = tokens.shape[0]
+        losses = self._losses if n_mb == self._losses.numel() else torch.empty(n_mb, dtype=F32, device=self.dev)
+        for mb in range(n_mb):
             torch.cuda.nvtx.range_push("microbatch%d" % mb)      # lets a profiler select one micro-batch
+            self.loss_mean = losses[mb:mb + 1]
             self.forward(tokens[mb])
-            losses[mb:mb + 1].copy_(self.loss_mean)
             self.backward()
             with self.span("grad_accum"):
                 det.det_grad_accum_push(st, self.gmb)
@@ -475,12 +485,14 @@ class Replay:
         with self.span("optimizer"):
             self.optimizer()
         with self.span("hash"):
-            h = self.hashes(per_tensor_hashes)
-        res = {"hashes": h, "status": int(self.status.item())}
+            names = self._queue_hashes(per_tensor_hashes)
+            out = self._out.cpu().numpy()          # the step's one synchronisation
+        scalars = out[4:12].view(np.float32)
+        res = {"hashes": self._hex(names, out[16:].tobytes()), "status": int(out[:4].view(np.int32)[0])}
         if want_losses:
-            ls = losses.cpu().numpy()
+            ls = (out[16 + self.roots.numel():].view(np.float32) if losses is self._losses else losses.cpu().numpy())
             res.update(losses=[float(x) for x in ls], loss=float(np.mean(ls.astype(np.float64))),
-                       grad_norm=float(self.norm.item()), coef=float(self.coef.item()))
+                       grad_norm=float(scalars[0]), coef=float(scalars[1]))
         return res
 
 
