@@ -72,7 +72,7 @@ _lib = None
 
 def load():
     """Load libdet.so; raises if it has not been built (python -m paper_2609_17380_b200.build)."""
-    global _lib
+    global _lib, _ptr, _stream
     if _lib is None:
         if not os.path.exists(_SO):
             raise ImportError("libdet.so is missing: build it with `python paper_2609_17380_b200/build.py` "
@@ -82,19 +82,20 @@ def load():
             fn = getattr(lib, name)
             fn.restype = _CTYPES[sig[0]]
             fn.argtypes = [_CTYPES[c] for c in sig[1:]]
+        from . import _binding
+        _ptr, _stream = _binding.ptr, _binding.stream
         _lib = lib
     return _lib
 
 
 def _ptr(t):
-    if t is None or isinstance(t, int):
-        return t
-    assert t.is_cuda and t.is_contiguous(), "tensors must be contiguous CUDA tensors"
-    return t.data_ptr()
+    load()                       # replaces this function and _stream by the native ones
+    return _ptr(t)
 
 
 def _stream():
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    load()
+    return _stream()
 
 
 def _check(fn, rc):

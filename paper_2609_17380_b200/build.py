@@ -1,4 +1,4 @@
-"""Builds libdet.so (CUDA, sm_100a only) in-tree with nvcc.
+"""Builds libdet.so (CUDA, sm_100a only) in-tree with nvcc, and _binding.so, the Python binding's argument conversion.
 
 Flags that matter for the arithmetic: -fmad=false (never contract a*b+c), -ftz=true (flush subnormal
 inputs and results), -prec-div=true / -prec-sqrt=true (IEEE division and square root).
@@ -10,6 +10,7 @@ from concurrent.futures import ThreadPoolExecutor
 _DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_DIR, "csrc")
 OUT = os.path.join(_DIR, "libdet.so")
+BINDING = os.path.join(_DIR, "_binding.so")
 SOURCES = ["reduce.cu", "norm_loss.cu", "glue_optim.cu", "hash.cu", "igemm.cu", "lsq.cu", "ogemm.cu", "attn.cu", "attn_pv8.cu", "headops.cu", "sum_static.cu", "lmhead_v2.cu", "attn_v2.cu"]
 HEADERS = ["common.cuh", "internal.h", "ogemm_core.cuh", "attn_core.cuh", "tc05.cuh", "v2_slice.cuh", os.path.join("..", "..", "include", "det.h"),
            os.path.join("..", "..", "include", "det_test.h")]
@@ -31,6 +32,24 @@ def _stale(target, deps):
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_binding(force=False):
+    """_binding.so from csrc/binding.cpp against the installed torch."""
+    src = os.path.join(CSRC, "binding.cpp")
+    if not force and not _stale(BINDING, [src]):
+        return BINDING
+    import sysconfig
+    import torch
+    from torch.utils import cpp_extension
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    inc = cpp_extension.include_paths("cuda") + [sysconfig.get_paths()["include"]]
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI]
+    cmd += [x for i in inc for x in ("-isystem", i)] + [src, "-o", BINDING, "-L", lib, "-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10", "-lc10_cuda"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("g++ failed for binding.cpp:\n%s" % r.stderr)
+    return BINDING
+
+
 def build(force=False, verbose=False):
     hdrs = [os.path.join(CSRC, h) for h in HEADERS]
     objdir = os.path.join(_DIR, "build")
@@ -50,7 +69,9 @@ def build(force=False, verbose=False):
         return o
 
     with ThreadPoolExecutor(max_workers=8) as ex:
+        binding = ex.submit(build_binding, force)
         objs = list(ex.map(compile_one, SOURCES))
+        binding.result()
     if force or _stale(OUT, objs):
         cmd = [nvcc, "-shared", "-o", OUT] + objs + ["-gencode", "arch=compute_100a,code=sm_100a", "-lcudart_static", "-ldl",
                                                      "-lrt", "-lpthread"]

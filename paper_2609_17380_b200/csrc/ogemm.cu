@@ -14,9 +14,6 @@
 
 using namespace det;
 
-// The two gradient contractions of the LM head are independent; the input-gradient grid (512 blocks on 148 SMs at
-// the benchmark shape) ends in a partial wave, so the weight-gradient kernel runs beside it on an auxiliary stream
-// and fills the idle SMs (aux_fork / aux_join keep plain stream order for the caller).
 static OgemmArgs plain_args(const void* A, const void* B, void* out, int I, int J, int C, int lda, int ldb, int ldo, int init) {
   OgemmArgs p = {};
   p.A = A; p.B = B; p.out = out; p.I = I; p.J = J; p.C = C; p.lda = lda; p.ldb = ldb; p.ldo = ldo; p.init = init;
