@@ -258,6 +258,15 @@ __device__ __forceinline__ int grid_dep() {
   return zero;
 }
 
+// A kernel launched by launch_after that depends on nothing of the kernel before it, only on older ones, fills the SMs that one
+// leaves as soon as all CTAs of that one are running: it skips the wait, and one CTA of it, the last, waits here at its end, so that
+// whatever comes after this kernel on the stream comes after both.
+__device__ __forceinline__ void grid_fill_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_fill_end() {
+  if (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // The sum of chunk `base` .. base + SUM_CHUNK of x[0..n): a perfect subtree, or the ragged last one with existence
 // predicates.  All 256 threads of the CTA call it; thread 0 gets the result.
 // The ragged form deals its leaves out over the warps (a sum of 2048 values has eight: one warp walking them behind scalar

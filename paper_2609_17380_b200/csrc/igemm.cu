@@ -176,7 +176,7 @@ __device__ __forceinline__ void epi_row(const EpiParams& ep, uint32_t taddr, int
 template <int BN, int EPI>
 __global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
     k_igemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, EpiParams ep, int I, int J,
-            int K, int* status) {
+            int K, int* status, int fill) {
   constexpr int STAGE_A = BM * BK, STAGE_B = BN * BK, STAGE_BYTES = STAGE_A + STAGE_B;
   constexpr int STAGES = IgTile<BN>::STAGES, EW = IgTile<BN>::EW, CW = IgTile<BN>::CW;
   extern __shared__ uint8_t smem_raw[];
@@ -205,7 +205,8 @@ __global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
-  grid_dep();
+  if (fill) grid_fill_begin();
+  else grid_dep();
 
   const int tiles_i = I / BM, tiles_j = J / BN;
   const int num_tiles = tiles_i * tiles_j;
@@ -290,6 +291,7 @@ __global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)IgTile<BN>::TCOLS) : "memory");
   }
+  if (fill) grid_fill_end();
 }
 
 // ------------------------------------------------------------------------------------------------------------
@@ -357,7 +359,7 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
 template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     k_igemm2(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, EpiParams ep, int I, int J,
-             int K, int* status) {
+             int K, int* status, int fill) {
   constexpr int STAGE_A = 128 * BK, STAGE_B = 128 * BK, STAGE_BYTES = STAGE_A + STAGE_B;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -388,7 +390,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
   cluster_sync_all();  // the peer's barriers are initialised before anything can signal them
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
-  grid_dep();
+  if (fill) grid_fill_begin();
+  else grid_dep();
 
   const int tiles_i = I / 256, tiles_j = J / BN2;
   const int num_tiles = tiles_i * tiles_j;
@@ -477,6 +480,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
   }
+  if (fill) grid_fill_end();
 }
 
 // ---- host side -------------------------------------------------------------------------------
@@ -508,7 +512,7 @@ bool make_map(CUtensorMap* tm, const int8_t* base, int rows, int K, int box_rows
 
 template <int BN, int EPI>
 static int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const EpiParams& ep, int I, int J, int K, int* status,
-                      cudaStream_t st) {
+                      cudaStream_t st, int fill) {
   typedef IgTile<BN> T;
   static DevOnce once = {};
   if (dev_ensure_smem(once, (const void*)k_igemm<BN, EPI>, T::SMEM) != DET_OK) return DET_ERR_CUDA;
@@ -516,14 +520,14 @@ static int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const EpiPar
   if (sms <= 0) return DET_ERR_CUDA;
   const int tiles = (I / BM) * (J / BN);
   const int grid = tiles < sms ? tiles : sms;
-  launch_after(k_igemm<BN, EPI>, grid, T::THREADS, T::SMEM, st, ta, tb, ep, I, J, K, status);
+  launch_after(k_igemm<BN, EPI>, grid, T::THREADS, T::SMEM, st, ta, tb, ep, I, J, K, status, fill);
   if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return DET_ERR_CUDA; }
   return DET_OK;
 }
 
 template <int EPI>
 static int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const EpiParams& ep, int I, int J, int K, int* status,
-                       cudaStream_t st) {
+                       cudaStream_t st, int fill) {
   constexpr size_t smem = (size_t)STAGES2 * (2 * 128 * BK) + 8 * 4096 + 1024;
   static DevOnce once = {};
   if (dev_ensure_smem(once, (const void*)k_igemm2<EPI>, smem) != DET_OK) return DET_ERR_CUDA;
@@ -532,7 +536,7 @@ static int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const EpiPa
   const int tiles = (I / 256) * (J / BN2);
   int clusters = sms / 2;
   if (tiles < clusters) clusters = tiles;
-  launch_after(k_igemm2<EPI>, 2 * clusters, GEMM2_THREADS, smem, st, ta, tb, ep, I, J, K, status);
+  launch_after(k_igemm2<EPI>, 2 * clusters, GEMM2_THREADS, smem, st, ta, tb, ep, I, J, K, status, fill);
   if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return DET_ERR_CUDA; }
   return DET_OK;
 }
@@ -563,16 +567,16 @@ static int igemm_pick(int epi, int I, int J, int K, int force_one_cta) {
 }
 template <int EPI>
 static int igemm_tile(int bn, const CUtensorMap& ta, const CUtensorMap& tb, const EpiParams& ep, int I, int J, int K, int* status,
-                      cudaStream_t st) {
+                      cudaStream_t st, int fill) {
   switch (bn) {
-    case 512: return launch_pair<EPI>(ta, tb, ep, I, J, K, status, st);
-    case 256: return launch_one<256, EPI>(ta, tb, ep, I, J, K, status, st);
-    case 128: return launch_one<128, EPI>(ta, tb, ep, I, J, K, status, st);
-    default: return launch_one<64, EPI>(ta, tb, ep, I, J, K, status, st);
+    case 512: return launch_pair<EPI>(ta, tb, ep, I, J, K, status, st, fill);
+    case 256: return launch_one<256, EPI>(ta, tb, ep, I, J, K, status, st, fill);
+    case 128: return launch_one<128, EPI>(ta, tb, ep, I, J, K, status, st, fill);
+    default: return launch_one<64, EPI>(ta, tb, ep, I, J, K, status, st, fill);
   }
 }
 int igemm_launch(int epi, const int8_t* A, const int8_t* B, int I, int J, int K, const EpiParams& ep, int* status,
-                 cudaStream_t st, int force_one_cta) {
+                 cudaStream_t st, int force_one_cta, int fill) {
   if (!A || !B || I <= 0 || J <= 0 || K <= 0) return DET_ERR_ARG;
   if (I % BM || J % 128 || K % BK) return DET_ERR_SHAPE;
   if (K >= (1 << 17)) return DET_ERR_RANGE;
@@ -581,10 +585,10 @@ int igemm_launch(int epi, const int8_t* A, const int8_t* B, int I, int J, int K,
   CUtensorMap ta, tb;
   if (!make_map(&ta, A, I, K, 128) || !make_map(&tb, B, J, K, bn == 512 ? 128 : bn)) return DET_ERR_CUDA;
   switch (epi) {
-    case EPI_RAW: return igemm_tile<EPI_RAW>(bn, ta, tb, ep, I, J, K, status, st);
-    case EPI_FWD: return igemm_tile<EPI_FWD>(bn, ta, tb, ep, I, J, K, status, st);
-    case EPI_DX: return igemm_tile<EPI_DX>(bn, ta, tb, ep, I, J, K, status, st);
-    case EPI_DW: return igemm_tile<EPI_DW>(bn, ta, tb, ep, I, J, K, status, st);
+    case EPI_RAW: return igemm_tile<EPI_RAW>(bn, ta, tb, ep, I, J, K, status, st, fill);
+    case EPI_FWD: return igemm_tile<EPI_FWD>(bn, ta, tb, ep, I, J, K, status, st, fill);
+    case EPI_DX: return igemm_tile<EPI_DX>(bn, ta, tb, ep, I, J, K, status, st, fill);
+    case EPI_DW: return igemm_tile<EPI_DW>(bn, ta, tb, ep, I, J, K, status, st, fill);
   }
   return DET_ERR_ARG;
 }
