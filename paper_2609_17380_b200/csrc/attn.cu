@@ -773,9 +773,9 @@ static int attn_bwd_impl(const det_bf16* dout, const det_bf16* q, const det_bf16
   DET_CHECK_LAUNCH();
   // dV[j,c] = sum over the query heads g of the group, then over queries i >= j ascending, of P~[i,j] dO[i,c];
   // dK[j,c] likewise with dS~ and q; dQ[i,c] = sum over visible keys j ascending of dS~[i,j] k[j,c].  The three are
-  // independent of each other and run side by side on auxiliary streams, so that the short blocks at the end of one grid
-  // overlap with the long blocks at the start of the next.
-  AuxScope aux(st);   // joined again on every way out
+  // independent of each other: each fills the SMs that the one before it leaves, so that the short blocks at the end of one grid
+  // overlap with the long blocks at the start of the next (on three streams, 16 heads x 4096 with window 512: 1.472 ms forward and backward
+  // against 1.425, two sequences of 8 x 1088 0.514 against 0.511).
   for (int which = 0; which < 2; ++which) {
     OgemmArgs p = {};
     p.I = S; p.J = DH; p.C = S; p.lda = S; p.H = Hkv; p.a_b = (long long)H * S * S; p.a_h = (long long)S * S;
@@ -785,7 +785,8 @@ static int attn_bwd_impl(const det_bf16* dout, const det_bf16* q, const det_bf16
     p.ldb = which == 0 ? ld_out : ld;
     p.b_b = (long long)S * p.ldb; p.b_h = DH;
     p.out = which == 0 ? dv : dk; p.ldo = ld_d; p.o_b = (long long)S * ld_d; p.o_h = DH;
-    rc = ogemm_launch<STRIDED, STRIDED, false, true, 1>(p, B * Hkv, 3, which == 0 ? st : aux.aux(0));
+    p.order = which == 0 ? OG_LEAD : OG_LEAD | OG_FILL;
+    rc = ogemm_launch<STRIDED, STRIDED, false, true, 1>(p, B * Hkv, 3, st);
     if (rc != DET_OK) return rc;
   }
   OgemmArgs p = {};
@@ -793,10 +794,10 @@ static int attn_bwd_impl(const det_bf16* dout, const det_bf16* q, const det_bf16
   p.A = dSt; p.B = k; p.ldb = ld; p.b_b = (long long)S * ld; p.b_h = DH; p.nG = 1; p.b_div = G;
   p.out = dq; p.ldo = ld_d; p.o_b = (long long)S * ld_d; p.o_h = DH; p.range_mode = 2; p.window = window;
   // fixq: per block of 128 keys the ordered f32 sum, accumulated over the blocks in 64-bit fixed point (Sec. 3.2)
-  if (fixq) rc = ogemm_run<CONTIG, STRIDED, false, true, OgFix, true>(p, B * H, aux.aux(1));
-  else rc = ogemm_launch<CONTIG, STRIDED, false, true, 1>(p, B * H, 3, aux.aux(1));
+  p.order = OG_FILL;
+  if (fixq) rc = ogemm_run<CONTIG, STRIDED, false, true, OgFix, true>(p, B * H, st);
+  else rc = ogemm_launch<CONTIG, STRIDED, false, true, 1>(p, B * H, 3, st);
   if (rc != DET_OK) return rc;
-  if (!aux.join()) return DET_ERR_CUDA;
   DET_CHECK_LAUNCH();
   return DET_OK;
 }

@@ -208,10 +208,9 @@ struct OgemmArgs {
   int window;           // sliding window W (multiple of 128; 0 = none): only |query - key| < W contributes
   int range_mode;       // 0: whole contraction; 1: c >= first row of the tile (causal, per key); 2: c < last row + 1 of the tile
                         // (with a window, mode 1 also stops at c < i0 + W + TM and mode 2 starts at c >= i0 - W)
-  int order;            // OG_PLAIN; or OG_LEAD, the next launch is OG_FILL; OG_FILL: independent of the launch before, takes the SMs
-                        // that are left once all CTAs of that one are running, and ends after it
+  int order;            // OG_LEAD: the next launch is OG_FILL; OG_FILL: independent of the launch before, fills the SMs that it leaves
 };
-enum { OG_PLAIN, OG_LEAD, OG_FILL };
+enum { OG_LEAD = 1, OG_FILL = 2 };
 
 // Tile TM x TN, thread tile 8 x CT, LY lanes of a warp along the rows, ST ring slots, PF slabs in flight in the producers'
 // registers, CPS CTAs per SM; RC / RP: registers of a consumer / producer thread after the hand-over (0: none).
@@ -283,7 +282,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS) k_ogemm(const OgemmArgs p)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  if (p.order == OG_LEAD) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (p.order & OG_LEAD) grid_fill_begin();
   // use n of a slot completes phase n of its barriers: the consumers wait with parity n & 1, the producers, one use
   // behind, with the opposite one
   if (tid >= T::CONS) {
@@ -402,9 +401,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS) k_ogemm(const OgemmArgs p)
       }
     }
   }
-  // one CTA that ends after the launch before is enough for the whole grid to do so
-  if (p.order == OG_FILL && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (p.order & OG_FILL) grid_fill_end();
 }
 
 template <int AMODE, int BMODE, bool AF32, bool OUT_BF16, class T, bool FIX = false>
@@ -415,7 +412,7 @@ static int ogemm_run(const OgemmArgs& p, int batches, cudaStream_t st) {
   if (dev_ensure_smem(once, (const void*)kern, smem) != DET_OK) return DET_ERR_CUDA;
   const unsigned ni = (unsigned)((p.I + T::TM - 1) / T::TM), nj = (unsigned)((p.J + T::TN - 1) / T::TN);
   const dim3 grid = p.range_mode ? dim3(nj, (unsigned)batches, ni) : dim3(nj, ni, (unsigned)batches);
-  if (p.order == OG_FILL) launch_after(kern, grid, T::THREADS, smem, st, p);
+  if (p.order & OG_FILL) launch_after(kern, grid, T::THREADS, smem, st, p);
   else kern<<<DET_L(grid), T::THREADS, smem, st>>>(p);
   return DET_OK;
 }
