@@ -146,98 +146,111 @@ __global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJ
   sha_store(out + (size_t)c * 32, h);
 }
 
-// Few chunks: eight chains per warp, four lanes each.  Only the 64 rounds of a block depend on the block before, so the
-// four lanes of a chain expand the schedules of its next four blocks side by side (schedule word + round constant through
-// shared memory) and the chain itself is rounds alone: 14 instructions a round instead of 22 on the pipe that sets the pace
-// of a single warp, 0.085 ms for 65 blocks instead of 0.137 ms.
+// Few chunks: eight chains per CTA, four lanes each.  Only the 64 rounds of a block depend on the block before, so the four lanes
+// of a chain expand the schedules of its next four blocks side by side (schedule word + round constant, through shared memory)
+// and the chain itself is rounds alone: 14 instructions a round on the half-rate integer pipe instead of 22, ordered so that a and
+// e depend on the round before through one rotation, one exclusive or and one addition each.  While there are schedulers to
+// spare a second warp does the expanding, double-buffered.  65 blocks: 0.137 ms with a thread per chunk, 0.089 with
+// one warp per CTA, 0.076 with two.
 constexpr int SF_CH = 8, SF_PITCH = 68;
 template <bool ROOT>
-__global__ void __launch_bounds__(32) k_sha_few(const __grid_constant__ HashJobs jobs, uint8_t* __restrict__ out) {
+__global__ void __launch_bounds__(64) k_sha_few(const __grid_constant__ HashJobs jobs, uint8_t* __restrict__ out) {
   grid_dep();
-  __shared__ __align__(16) uint32_t ws[4 * SF_CH * SF_PITCH];
+  __shared__ __align__(16) uint32_t ws[2][4 * SF_CH * SF_PITCH];
   constexpr uint32_t K[64] = {SHA_K_LIST};
-  const int ch = threadIdx.x >> 2, sub = threadIdx.x & 3;
+  const int ch = (threadIdx.x & 31) >> 2, sub = threadIdx.x & 3;
+  const bool pair = blockDim.x == 64, expand = threadIdx.x >= 32;
   const uint32_t c = blockIdx.x * SF_CH + ch;
   const bool have = c < jobs.first[jobs.n];
   ShaMsg msg = {};
   uint32_t nb = 0;
   if (have) { msg = sha_msg<ROOT>(jobs, c); nb = msg.blocks(); }
   const uint32_t full = have ? msg.len / 64 : 0, nbmax = __reduce_max_sync(0xffffffffu, nb);
+  uint4 nx[4];
+  auto fetch = [&](uint32_t b) {
+    if (b < full) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) nx[k] = __ldg(reinterpret_cast<const uint4*>(msg.p + (size_t)b * 64) + k);
+    }
+  };
+  auto schedule = [&](uint32_t b, uint32_t* row) {   // of block b, whose words are in nx
+    if (b >= nb) return;
+    uint32_t w[16];
+    if (b < full) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint4 u = nx[k];
+        w[4 * k] = bswap(u.x); w[4 * k + 1] = bswap(u.y); w[4 * k + 2] = bswap(u.z); w[4 * k + 3] = bswap(u.w);
+      }
+    } else {
+      uint32_t t[16];
+      msg.ragged_block(b, t);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) w[k] = t[k];
+    }
+    fetch(b + 4);
+#pragma unroll
+    for (int i = 0; i < 64; i += 4) {
+      uint32_t t[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int j = i + k;
+        if (j >= 16) w[j & 15] += small_s0(w[(j + 1) & 15]) + w[(j + 9) & 15] + small_s1(w[(j + 14) & 15]);
+        t[k] = w[j & 15] + K[j];
+      }
+      *reinterpret_cast<uint4*>(row + i) = make_uint4(t[0], t[1], t[2], t[3]);
+    }
+  };
   uint32_t h[8];
   sha_init(h);
-  uint4 nx[4];
-  if ((uint32_t)sub < full) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) nx[k] = __ldg(reinterpret_cast<const uint4*>(msg.p + sub * 64) + k);
-  }
-  for (uint32_t b0 = 0; b0 < nbmax; b0 += 4) {
-    const uint32_t mine = b0 + sub;
-    if (mine < nb) {
-      uint32_t w[16];
-      if (mine < full) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const uint4 u = nx[k];
-          w[4 * k] = bswap(u.x); w[4 * k + 1] = bswap(u.y); w[4 * k + 2] = bswap(u.z); w[4 * k + 3] = bswap(u.w);
-        }
-      } else {
-        uint32_t t[16];
-        msg.ragged_block(mine, t);
-#pragma unroll
-        for (int k = 0; k < 16; ++k) w[k] = t[k];
-      }
-      if (mine + 4 < full) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) nx[k] = __ldg(reinterpret_cast<const uint4*>(msg.p + (mine + 4) * 64) + k);
-      }
-      uint32_t* row = ws + (sub * SF_CH + ch) * SF_PITCH;
-#pragma unroll
-      for (int i = 0; i < 64; i += 4) {
-        uint32_t t[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int j = i + k;
-          if (j >= 16) w[j & 15] += small_s0(w[(j + 1) & 15]) + w[(j + 9) & 15] + small_s1(w[(j + 14) & 15]);
-          t[k] = w[j & 15] + K[j];
-        }
-        *reinterpret_cast<uint4*>(row + i) = make_uint4(t[0], t[1], t[2], t[3]);
-      }
-    }
-    __syncwarp();
+  // a pair: the expanding warp is four blocks ahead; a single warp does one after the other
+  if (!pair || expand) fetch(sub);
+  for (int b0 = pair ? -4 : 0; b0 < (int)nbmax; b0 += 4) {
+    uint32_t* next = ws[pair ? (b0 / 4 + 1) & 1 : 0];
+    const uint32_t* cur = ws[pair ? (b0 / 4) & 1 : 0];
+    if (!pair || expand) schedule((uint32_t)(b0 + (pair ? 4 : 0) + sub), next + (sub * SF_CH + ch) * SF_PITCH);
+    if (!pair) __syncwarp();
+    if (!expand && b0 >= 0) {
 #pragma unroll 1
-    for (int s = 0; s < 4; ++s) {
-      if (b0 + s < nb) {
-        const uint32_t* row = ws + (s * SF_CH + ch) * SF_PITCH;
-        uint32_t a = h[0], b = h[1], cc = h[2], d = h[3], e = h[4], f = h[5], g = h[6], hh = h[7];
+      for (int s = 0; s < 4; ++s) {
+        if ((uint32_t)(b0 + s) < nb) {
+          const uint32_t* row = cur + (s * SF_CH + ch) * SF_PITCH;
+          uint32_t a = h[0], b = h[1], cc = h[2], d = h[3], e = h[4], f = h[5], g = h[6], hh = h[7];
 #pragma unroll
-        for (int i = 0; i < 64; i += 4) {
-          const uint4 u = *reinterpret_cast<const uint4*>(row + i);
-          const uint32_t wk[4] = {u.x, u.y, u.z, u.w};
+          for (int i = 0; i < 64; i += 4) {
+            const uint4 u = *reinterpret_cast<const uint4*>(row + i);
+            const uint32_t wk[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const uint32_t dx = wk[k] + hh + d;
-            const uint32_t en = big_s1(e) + sha_ch(e, f, g) + dx;
-            const uint32_t q = big_s0(a) + sha_maj(a, b, cc) - d;
-            hh = g; g = f; f = e; e = en; d = cc; cc = b; b = a; a = q + en;
+            for (int k = 0; k < 4; ++k) {
+              const uint32_t dx = wk[k] + hh + d;
+              const uint32_t en = big_s1(e) + sha_ch(e, f, g) + dx;
+              const uint32_t an = big_s0(a) + sha_maj(a, b, cc) + (en - d);
+              hh = g; g = f; f = e; e = en; d = cc; cc = b; b = a; a = an;
+            }
           }
+          h[0] += a; h[1] += b; h[2] += cc; h[3] += d; h[4] += e; h[5] += f; h[6] += g; h[7] += hh;
         }
-        h[0] += a; h[1] += b; h[2] += cc; h[3] += d; h[4] += e; h[5] += f; h[6] += g; h[7] += hh;
       }
     }
-    __syncwarp();
+    __syncthreads();
   }
-  if (have && sub == 0) sha_store(out + (size_t)c * 32, h);
+  if (have && !expand && sub == 0) sha_store(out + (size_t)c * 32, h);
 }
 
-// The rule: as long as four lanes per chain leave at most one warp on a scheduler, the chain's latency is what counts and
-// the few-chunk form is the faster one (1000 chunks: 0.085 against 0.140 ms); with two warps per scheduler both take
-// about the same time (9000 chunks: 0.157 and 0.141 ms), beyond that a thread per chunk wins.
+// The rule: as long as the warps of this form do not outnumber the schedulers, the chain's latency is what counts (3144 chunks: 0.097 ms with one warp
+// per CTA, 0.134 with two, 0.140 with a thread per chunk); with
+// two warps per scheduler both forms take about the same time (9000 chunks: 0.157 and 0.141 ms), beyond that a thread per
+// chunk wins.
+static void sha_few_launch(bool root, const HashJobs& jobs, uint32_t n, uint8_t* out, int sms, cudaStream_t st) {
+  const unsigned ctas = (n + SF_CH - 1) / SF_CH;
+  launch_after(root ? k_sha_few<true> : k_sha_few<false>, ctas, ctas <= 2u * (unsigned)sms ? 64 : 32, 0, st, jobs, out);
+}
 static int hash_level(const HashJobs& jobs, uint8_t* out, cudaStream_t st) {
   const uint32_t n = jobs.first[jobs.n];
   if (!n) return DET_OK;
   const int sms = dev_sm_count();
   if (sms <= 0) return DET_ERR_CUDA;
-  if (n <= (uint32_t)sms * 4 * SF_CH) launch_after(k_sha_few<false>, (n + SF_CH - 1) / SF_CH, 32, 0, st, jobs, out);
+  if (n <= (uint32_t)sms * 4 * SF_CH) sha_few_launch(false, jobs, n, out, sms, st);
   else launch_after(k_sha_chunks, (n + 63) / 64, 64, 0, st, jobs, out);
   DET_CHECK_LAUNCH();
   return DET_OK;
@@ -273,6 +286,8 @@ extern "C" int det_tensor_hash_batch(const void* const* ptrs, const size_t* nbyt
   }
   if (!aligned16(roots_dev)) return DET_ERR_ALIGN;
   if (!ws || !aligned16(ws) || ws_bytes < det_tensor_hash_batch_ws_bytes(nbytes, ntensors)) return DET_ERR_WORKSPACE;
+  const int sms = dev_sm_count();
+  if (sms <= 0) return DET_ERR_CUDA;
   cudaStream_t st = (cudaStream_t)stream;
   for (int t0 = 0; t0 < ntensors; t0 += HASH_JOBS) {
     const int n = ntensors - t0 < HASH_JOBS ? ntensors - t0 : HASH_JOBS;
@@ -307,7 +322,7 @@ extern "C" int det_tensor_hash_batch(const void* const* ptrs, const size_t* nbyt
       out += c * 32;
       lv.n = m;
     }
-    launch_after(k_sha_few<true>, (n + SF_CH - 1) / SF_CH, 32, 0, st, root, roots_dev + (size_t)t0 * 32);
+    sha_few_launch(true, root, (uint32_t)n, roots_dev + (size_t)t0 * 32, sms, st);
     DET_CHECK_LAUNCH();
   }
   return DET_OK;
