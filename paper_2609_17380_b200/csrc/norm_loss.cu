@@ -37,27 +37,33 @@ __device__ __forceinline__ void store8(void* p, size_t idx, const float v[8]) {
 // ------------------------------------------------------------------------------------------------
 // A warp per LEAF (256 columns, 8 adjacent columns per lane), a CTA of 8 warps per block of 8 rows in two passes of four
 // rows: 16 values and 8 loads in flight per lane, four CTAs per SM; the leaf sums of a row meet in shared memory (one
-// barrier per pass) and every thread forms the row's tree over its leaves itself.
-template <bool BF>
+// barrier per pass) and every thread forms the row's tree over its leaves itself.  Rows of at most 1024 columns need only some of
+// the warps: the eight rows are then dealt out to 2, 4 or 8 groups of warps and take one pass (cold, 128 rows of 256: 10.3 -> 4.1 us;
+// 1664 of 1024: 12.6 -> 8.9).
+// WPR warps per row; RowGroups: groups per CTA, rows per group and pass.
+template <int WPR>
+struct RowGroups { static constexpr int GROUPS = 8 / WPR, ROWS = WPR < 4 ? WPR : 4; };
+template <bool BF, int WPR>
 __global__ void __launch_bounds__(256, 4) k_rmsnorm_fwd8(const void* __restrict__ x, const void* __restrict__ gamma, int rows,
                                                          int D, float eps, float invD, void* __restrict__ y,
                                                          float* __restrict__ rstd, const float* __restrict__ s_q = nullptr,
                                                          int8_t* __restrict__ qy = nullptr, const void* __restrict__ res = nullptr,
                                                          void* __restrict__ sum = nullptr) {
   grid_dep();
-  __shared__ float leaf_sum[2][4][8];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __shared__ float leaf_sum[8][8];
+  constexpr int ROWS = RowGroups<WPR>::ROWS, STEP = RowGroups<WPR>::GROUPS * ROWS;
+  const int grp = (threadIdx.x >> 5) / WPR, warp = (threadIdx.x >> 5) % WPR, lane = threadIdx.x & 31;
   const int e0 = warp * 256 + lane * 8;
   const bool have = e0 < D;
   const bool full = (D & 255) == 0;
   const long long r0 = (long long)blockIdx.x * 8;
   const float inv_q = (BF && qy) ? fdiv(1.0f, s_q[0]) : 0.0f;
 #pragma unroll 1
-  for (int pass = 0; pass < 2; ++pass) {
-    float xr[4][8];
+  for (int first = grp * ROWS; first < 8; first += STEP) {   // this group's rows of the pass
+    float xr[ROWS][8];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const long long row = r0 + 4 * pass + a;
+    for (int a = 0; a < ROWS; ++a) {
+      const long long row = r0 + first + a;
       if (row < rows && have) load8<BF>(x, (size_t)row * D + e0, xr[a]);
       else {
 #pragma unroll
@@ -66,8 +72,8 @@ __global__ void __launch_bounds__(256, 4) k_rmsnorm_fwd8(const void* __restrict_
     }
     if (BF && res) {   // the residual sum in front of the norm: x + res, rounded and stored, is what is normalised
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const long long row = r0 + 4 * pass + a;
+      for (int a = 0; a < ROWS; ++a) {
+        const long long row = r0 + first + a;
         if (row >= rows || !have) continue;
         float b[8];
         load8<BF>(res, (size_t)row * D + e0, b);
@@ -79,27 +85,27 @@ __global__ void __launch_bounds__(256, 4) k_rmsnorm_fwd8(const void* __restrict_
       }
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
+    for (int a = 0; a < ROWS; ++a) {
       float sq[8];
 #pragma unroll
       for (int t = 0; t < 8; ++t) sq[t] = fmul(xr[a][t], xr[a][t]);
       const float t8 = tree8_full(sq);
       const float leaf = full ? warp_tree_full(t8) : warp_tree(t8, (long long)warp * 256, 8, D);
-      if (lane == 0) leaf_sum[pass][a][warp] = leaf;
+      if (lane == 0) leaf_sum[first + a][warp] = leaf;
     }
     __syncthreads();
     float g[8];
     if (gamma && have) load8<BF>(gamma, e0, g);
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const long long row = r0 + 4 * pass + a;
+    for (int a = 0; a < ROWS; ++a) {
+      const long long row = r0 + first + a;
       float L[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) L[j] = leaf_sum[pass][a][j];
+      for (int j = 0; j < 8; ++j) L[j] = leaf_sum[first + a][j];
       const float ss = reg_tree<8>(L, 0, 256, D);          // a leaf beyond D does not exist
       const float rs = fdiv(1.0f, fsqrt(fadd(fmul(ss, invD), eps)));
       if (row >= rows) continue;
-      if (threadIdx.x == a) rstd[row] = rs;
+      if (warp == 0 && lane == a) rstd[row] = rs;
       if (!have) continue;
       float o[8];
       if (gamma) {
@@ -129,15 +135,19 @@ __global__ void __launch_bounds__(256, 4) k_rmsnorm_fwd8(const void* __restrict_
 // 0.065-0.070 ms without the gain gradient, i.e. 0.9 of the copy bandwidth).  The row sums go through shared memory: one
 // value per leaf and row, one barrier per pass.
 // RPP rows per pass: 2 for f32 rows, 4 for bf16 rows (16 values and 64 bytes of loads in flight per lane and tensor either way).
-template <bool BF, bool DG>
+// bf16 rows of at most 1024 columns: groups of warps as in the forward kernel, one pass; the groups' nodes of the column tree meet in
+// shared memory (cold, 128 rows of 256: 13.3 -> 4.1 us; 1024 of 1024: 14.3 -> 8.7).
+template <bool BF, bool DG, int WPR>
 __global__ void __launch_bounds__(256, 3) k_rmsnorm_bwd8(const void* __restrict__ dy, const void* __restrict__ x,
                                                         const void* __restrict__ gamma, const float* __restrict__ rstd,
                                                         int rows, int D, float invD, void* dx, const void* res,
                                                         float* __restrict__ partial8, int* __restrict__ tickets) {
   grid_dep();
-  constexpr int RPP = BF ? 4 : 2, NPASS = 8 / RPP;
-  __shared__ float leaf_sum[2][RPP][8];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  static_assert(BF || WPR == 8, "f32 rows take the passes one after the other");
+  constexpr int RPP = BF ? RowGroups<WPR>::ROWS : 2, GROUPS = RowGroups<WPR>::GROUPS;
+  __shared__ float leaf_sum[8][8];
+  __shared__ __align__(16) float nodes[DG && GROUPS > 1 ? 8 : 1][32][8];
+  const int grp = (threadIdx.x >> 5) / WPR, warp = (threadIdx.x >> 5) % WPR, lane = threadIdx.x & 31;
   const int e0 = warp * 256 + lane * 8;
   const bool have = e0 < D;                       // this lane's 8 columns exist (D is a multiple of 8)
   const bool full = (D & 255) == 0;
@@ -147,8 +157,8 @@ __global__ void __launch_bounds__(256, 3) k_rmsnorm_bwd8(const void* __restrict_
 #pragma unroll
   for (int t = 0; t < 8; ++t) { pair0[t] = 0.0f; node[t] = 0.0f; }
 #pragma unroll 1
-  for (int pass = 0; pass < NPASS; ++pass) {
-    const long long first = r0 + RPP * pass;
+  for (int pass = 0, f = grp * RPP; f < 8; f += GROUPS * RPP, ++pass) {
+    const long long first = r0 + f;
     float w[RPP][8], xh[RPP][8], rs[RPP];
 #pragma unroll
     for (int a = 0; a < RPP; ++a) {
@@ -170,12 +180,16 @@ __global__ void __launch_bounds__(256, 3) k_rmsnorm_bwd8(const void* __restrict_
                 // iff its first row does, else the left one is carried up unchanged)
 #pragma unroll
       for (int t = 0; t < 8; ++t) {
-        const float d0 = fmul(w[0][t], xh[0][t]), d1 = fmul(w[1][t], xh[1][t]);
-        const float pa = (first + 1 < rows) ? fadd(d0, d1) : d0;
-        if (RPP == 4) {
-          const float d2 = fmul(w[RPP - 2][t], xh[RPP - 2][t]), d3 = fmul(w[RPP - 1][t], xh[RPP - 1][t]);
-          const float pb = (first + 3 < rows) ? fadd(d2, d3) : d2;
-          const float four = (first + 2 < rows) ? fadd(pa, pb) : pa;
+        const float d0 = fmul(w[0][t], xh[0][t]);
+        float pa = d0;
+        if (RPP > 1) pa = (first + 1 < rows) ? fadd(d0, fmul(w[RPP > 1][t], xh[RPP > 1][t])) : d0;
+        if (BF) {
+          float four = pa;
+          if (RPP == 4) {
+            const float d2 = fmul(w[RPP / 2][t], xh[RPP / 2][t]), d3 = fmul(w[RPP - 1][t], xh[RPP - 1][t]);
+            const float pb = (first + 3 < rows) ? fadd(d2, d3) : d2;
+            four = (first + 2 < rows) ? fadd(pa, pb) : pa;
+          }
           node[t] = (pass == 0) ? four : ((r0 + 4 < rows) ? fadd(node[t], four) : node[t]);
         } else if ((pass & 1) == 0) {
           pair0[t] = pa;
@@ -183,6 +197,11 @@ __global__ void __launch_bounds__(256, 3) k_rmsnorm_bwd8(const void* __restrict_
           const float four = (first < rows) ? fadd(pair0[t], pa) : pair0[t];
           node[t] = (pass == 1) ? four : ((r0 + 4 < rows) ? fadd(node[t], four) : node[t]);
         }
+      }
+      if (GROUPS > 1) {
+        float4* mine = reinterpret_cast<float4*>(nodes[threadIdx.x >> 5][lane]);
+        mine[0] = make_float4(node[0], node[1], node[2], node[3]);
+        mine[1] = make_float4(node[4], node[5], node[6], node[7]);
       }
     }
     if (gamma && have) {
@@ -200,7 +219,7 @@ __global__ void __launch_bounds__(256, 3) k_rmsnorm_bwd8(const void* __restrict_
       for (int t = 0; t < 8; ++t) pr[t] = fmul(w[a][t], xh[a][t]);
       const float t8 = tree8_full(pr);
       const float leaf = full ? warp_tree_full(t8) : warp_tree(t8, (long long)warp * 256, 8, D);
-      if (lane == 0) leaf_sum[pass & 1][a][warp] = leaf;
+      if (lane == 0) leaf_sum[f + a][warp] = leaf;
     }
     __syncthreads();
 #pragma unroll
@@ -208,7 +227,7 @@ __global__ void __launch_bounds__(256, 3) k_rmsnorm_bwd8(const void* __restrict_
       const long long row = first + a;
       float L[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) L[j] = leaf_sum[pass & 1][a][j];
+      for (int j = 0; j < 8; ++j) L[j] = leaf_sum[f + a][j];
       const float c = fmul(reg_tree<8>(L, 0, 256, D), invD);   // the row's tree over its leaves (a leaf beyond D does not exist)
       if (row < rows && have) {
         float o[8];
@@ -222,6 +241,17 @@ __global__ void __launch_bounds__(256, 3) k_rmsnorm_bwd8(const void* __restrict_
         }
         store8<BF>(dx, (size_t)row * D + e0, o);
       }
+    }
+  }
+  if (DG && GROUPS > 1) {   // the tree over the groups' nodes, each of RPP rows
+    __syncthreads();
+    if (grp) return;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      float n[GROUPS];
+#pragma unroll
+      for (int g = 0; g < GROUPS; ++g) n[g] = nodes[g * WPR + warp][lane][t];
+      node[t] = reg_tree<GROUPS>(n, r0, RPP, rows);
     }
   }
   if (DG && have) {
@@ -605,6 +635,19 @@ __global__ void __launch_bounds__(256) k_xent_bwd(float* __restrict__ logits, co
   }
 }
 
+// the variant for rows of D columns
+template <bool BF>
+static auto fwd8_kernel(int D) {
+  return D <= 256 ? k_rmsnorm_fwd8<BF, 1> : (D <= 512 ? k_rmsnorm_fwd8<BF, 2> : (D <= 1024 ? k_rmsnorm_fwd8<BF, 4> : k_rmsnorm_fwd8<BF, 8>));
+}
+template <bool BF, bool DG>
+static auto bwd8_kernel(int D) {
+  if constexpr (BF)
+    return D <= 256 ? k_rmsnorm_bwd8<BF, DG, 1> : (D <= 512 ? k_rmsnorm_bwd8<BF, DG, 2> : (D <= 1024 ? k_rmsnorm_bwd8<BF, DG, 4> : k_rmsnorm_bwd8<BF, DG, 8>));
+  else
+    return &k_rmsnorm_bwd8<BF, DG, 8>;
+}
+
 }  // namespace det
 
 using namespace det;
@@ -619,10 +662,10 @@ extern "C" int det_rmsnorm_fwd(int io, const void* x, const void* gamma, int row
   const float invD = (float)(1.0 / (double)D);
   dim3 grid((rows + 7) / 8);
   if (io == DET_BF16) {
-    if (D <= 2048) launch_after(k_rmsnorm_fwd8<true>, grid, 256, 0, st, x, gamma, rows, D, eps, invD, y, rstd, nullptr, nullptr, nullptr, nullptr);
+    if (D <= 2048) launch_after(fwd8_kernel<true>(D), grid, 256, 0, st, x, gamma, rows, D, eps, invD, y, rstd, nullptr, nullptr, nullptr, nullptr);
     else k_rmsnorm_fwd<true, 0><<<DET_L(grid), 256, 0, st>>>(x, gamma, rows, D, eps, invD, y, rstd);
   } else {
-    if (D <= 2048) launch_after(k_rmsnorm_fwd8<false>, grid, 256, 0, st, x, gamma, rows, D, eps, invD, y, rstd, nullptr, nullptr, nullptr, nullptr);
+    if (D <= 2048) launch_after(fwd8_kernel<false>(D), grid, 256, 0, st, x, gamma, rows, D, eps, invD, y, rstd, nullptr, nullptr, nullptr, nullptr);
     else k_rmsnorm_fwd<false, 0><<<DET_L(grid), 256, 0, st>>>(x, gamma, rows, D, eps, invD, y, rstd);
   }
   DET_CHECK_LAUNCH();
@@ -635,7 +678,7 @@ extern "C" int det_rmsnorm_fwd_q(const det_bf16* x, const det_bf16* gamma, int r
   if (D % 8 || D > 2048) return DET_ERR_SHAPE;
   if (!aligned16(x) || !aligned16(y) || (gamma && !aligned16(gamma)) || (((uintptr_t)qy) & 7u)) return DET_ERR_ALIGN;
   if (rows == 0) return DET_OK;
-  launch_after(k_rmsnorm_fwd8<true>, (rows + 7) / 8, 256, 0, (cudaStream_t)stream, x, gamma, rows, D, eps, (float)(1.0 / (double)D), y,
+  launch_after(fwd8_kernel<true>(D), (rows + 7) / 8, 256, 0, (cudaStream_t)stream, x, gamma, rows, D, eps, (float)(1.0 / (double)D), y,
                                                                               rstd, s_q, qy, nullptr, nullptr);
   DET_CHECK_LAUNCH();
   return DET_OK;
@@ -651,13 +694,13 @@ static int rmsnorm_bwd8_launch(const void* dy, const void* x, const void* gamma,
                                float invD, void* dx, const void* res, float* dgamma, float* ws, cudaStream_t st) {
   const int nb8 = (rows + 7) / 8, nb256 = (rows + 255) / 256;
   if (!dgamma) {
-    launch_after(k_rmsnorm_bwd8<BF, false>, nb8, 256, 0, st, dy, x, gamma, rstd, rows, D, invD, dx, res, nullptr, nullptr);
+    launch_after(bwd8_kernel<BF, false>(D), nb8, 256, 0, st, dy, x, gamma, rstd, rows, D, invD, dx, res, nullptr, nullptr);
     return DET_OK;
   }
   float* partial8 = ws;
   float* partial256 = ws + align_up((size_t)nb8 * D, 64);
   int* tickets = reinterpret_cast<int*>(partial256 + align_up((size_t)nb256 * D, 64));   // one per block of 256 columns (<= 8)
-  launch_after(k_rmsnorm_bwd8<BF, true>, nb8, 256, 0, st, dy, x, gamma, rstd, rows, D, invD, dx, res, partial8, tickets);
+  launch_after(bwd8_kernel<BF, true>(D), nb8, 256, 0, st, dy, x, gamma, rstd, rows, D, invD, dx, res, partial8, tickets);
   // the second launch overlaps its start-up with the first kernel's tail (programmatic dependent launch); the kernel
   // itself waits for the first grid to complete before it reads anything
   launch_after(k_colsum32, dim3((D + 255) / 256, nb256), 256, 0, st, (const float*)partial8, nb8, rows, D, partial256, nb256, tickets, dgamma);
@@ -705,7 +748,7 @@ extern "C" int det_residual_rmsnorm_fwd(const det_bf16* a, const det_bf16* b, co
   if (!aligned16(a) || !aligned16(b) || !aligned16(sum) || !aligned16(y) || (gamma && !aligned16(gamma)) || (((uintptr_t)qy) & 7u))
     return DET_ERR_ALIGN;
   if (rows == 0) return DET_OK;
-  launch_after(k_rmsnorm_fwd8<true>, (rows + 7) / 8, 256, 0, (cudaStream_t)stream, a, gamma, rows, D, eps, (float)(1.0 / (double)D), y,
+  launch_after(fwd8_kernel<true>(D), (rows + 7) / 8, 256, 0, (cudaStream_t)stream, a, gamma, rows, D, eps, (float)(1.0 / (double)D), y,
                                                                               rstd, s_q, qy, b, sum);
   DET_CHECK_LAUNCH();
   return DET_OK;

@@ -242,7 +242,8 @@ def test_linear_tiles(det, M, N, K):
 
 
 # the norms with the residual stream beside them: rows off the block of eight, D off the leaf of 256, with and without codes
-@pytest.mark.parametrize("rows,D,q", [(1, 8, True), (13, 1000, False), (300, 2048, True), (64, 384, True)])
+@pytest.mark.parametrize("rows,D,q", [(1, 8, True), (13, 1000, False), (300, 2048, True), (64, 384, True), (21, 256, True), (22, 512, False),
+                                      (23, 1024, True), (9, 1032, True), (515, 200, False)])
 def test_norms_with_residual(det, rows, D, q):
     a, b, dy, res = [synth.normal_bf16((rows, D), 1.0, seed=rows, tid=t) for t in range(4)]
     gain = synth.normal_bf16((D,), 0.1, mean=1.0, seed=rows, tid=9)
