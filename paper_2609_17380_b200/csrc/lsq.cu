@@ -291,9 +291,10 @@ __device__ __forceinline__ bool finite1(float x) { return (__float_as_uint(x) & 
 //     for two values takes the offset away, and the butterflies are the packed ones (as 32-bit integers they took the
 //     half-rate integer pipe: 896 instructions of two cycles instead of 512 that make up 896 cycles of the FP32 pipe).
 //
-//     The code is straight-line and as long as the work on a tile.  Where no CTA has more than one tile, fetching it is what takes the
-//     time, and rows of dY, columns of dY and columns of Z go through ONE copy of the butterflies and of the quantiser in a
-//     rolled loop (PREP_ONE; second pass of 256 tokens x 512, cold: 7.4 us in one launch, 27 with a copy for each).  Over
+//     The code is straight-line and as long as the work on a tile.  Where a CTA has one tile or two, fetching it is what takes the
+//     time, and rows of dY, columns of dY and columns of Z are work of different CTAs and go through ONE copy of the butterflies
+//     and of the quantiser (PREP_ONE; second pass of 256 tokens x 512, cold: 5.8 us, 7.4 with rows and columns of a tile one
+//     after the other in a CTA, 27 with a copy of the code for each).  Over
 //     many tiles the copies are the faster form (first pass over 16384 tokens x 16384: 0.20 against 0.23 ms), dY in one launch (PREP_Y), Z in
 //     another (PREP_Z) beside it.
 constexpr size_t PREP2_SMEM = (size_t)2 * PT * 256 + 2 * PT * sizeof(float);
@@ -332,19 +333,22 @@ __device__ __forceinline__ uint32_t block_max(uint32_t x, uint32_t (&box)[PT / 3
 }
 
 enum { PREP_ONE, PREP_Y, PREP_Z };
+constexpr int PREP_ONE_ROUNDS = 2;
 template <int PASS, int KIND>
 __global__ void __launch_bounds__(PT, 3) k_prep(const __grid_constant__ PrepArgs p) {
   extern __shared__ __align__(16) uint8_t pbuf[];
   __shared__ uint32_t box[PT / 32];
   float* swb = reinterpret_cast<float*>(pbuf + 2 * PT * 256);      // [2][128]
   const int t = threadIdx.x, M = p.M, N = p.N, K = p.K;
-  const int ntn = N / PT, ntk = K / PT, ntiles_y = KIND != PREP_Z && p.dY ? ntn * (M / PT) : 0;
+  const int ntn = N / PT, ntk = K / PT, tiles_y = KIND != PREP_Z && p.dY ? ntn * (M / PT) : 0;
+  const int ntiles_y = KIND == PREP_ONE ? 2 * tiles_y : tiles_y;      // one by one: rows of all tiles of dY, then their columns
   const int ntiles = ntiles_y + (KIND != PREP_Y ? ntk * (M / PT) : 0);
   auto z_tile = [&](int tile) { return KIND == PREP_Z || (KIND == PREP_ONE && tile >= ntiles_y); };
+  auto y_tile = [&](int tile) { return KIND == PREP_ONE && tile >= tiles_y ? tile - tiles_y : tile; };
   auto issue = [&](int tile, int b) {
     uint8_t* dst = pbuf + b * (PT * 256);
     if (!z_tile(tile)) {
-      const int n0 = (tile % ntn) * PT, m0 = (tile / ntn) * PT;
+      const int n0 = (y_tile(tile) % ntn) * PT, m0 = (y_tile(tile) / ntn) * PT;
 #pragma unroll
       for (int it = 0; it < 16; ++it) {
         const int r = it * 8 + (t >> 4), c = t & 15;
@@ -441,7 +445,7 @@ __global__ void __launch_bounds__(PT, 3) k_prep(const __grid_constant__ PrepArgs
       const float iv = dir == 0 ? inv[0] : (dir == 1 ? inv[1] : inv[2]);
       if ((dir == 0 ? fast[0] : (dir == 1 ? fast[1] : fast[2])) && finite1(v[0].x)) quant_pack128<true>(v, iv, q);
       else quant_pack128<false>(v, iv, q);
-      if (dir == 0) {
+      if (KIND != PREP_ONE && dir == 0) {
 #pragma unroll
         for (int k = 0; k < 32; ++k) qa[k] = q[k];
         return;
@@ -452,17 +456,19 @@ __global__ void __launch_bounds__(PT, 3) k_prep(const __grid_constant__ PrepArgs
       for (int g = 0; g < 8; ++g) {
         const int off = t * 128 + ((g ^ (t & 7)) << 4);
         *reinterpret_cast<uint4*>(buf + off) = make_uint4(q[4 * g], q[4 * g + 1], q[4 * g + 2], q[4 * g + 3]);
-        if (dir == 1) *reinterpret_cast<uint4*>(buf + 16384 + off) = make_uint4(qa[4 * g], qa[4 * g + 1], qa[4 * g + 2], qa[4 * g + 3]);
+        if (KIND == PREP_Y) *reinterpret_cast<uint4*>(buf + 16384 + off) = make_uint4(qa[4 * g], qa[4 * g + 1], qa[4 * g + 2], qa[4 * g + 3]);
       }
       __syncthreads();
-      const int z = tile - ntiles_y, m0 = (isz ? z / ntk : tile / ntn) * PT, c0 = (isz ? z % ntk : tile % ntn) * PT;
-      int8_t* dst = (isz ? p.ZqT : p.GqT) + (size_t)c0 * M + m0;
+      const int z = tile - ntiles_y, y = y_tile(tile), m0 = (isz ? z / ntk : y / ntn) * PT, c0 = (isz ? z % ntk : y % ntn) * PT;
+      const bool rows = KIND == PREP_ONE && dir == 0;
+      const size_t pitch = rows ? N : M;
+      int8_t* dst = rows ? p.Aq + (size_t)m0 * N + c0 : (isz ? p.ZqT : p.GqT) + (size_t)c0 * M + m0;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const int idx = k * PT + t, rr = idx >> 3, piece = idx & 7;
         const int off = rr * 128 + ((piece ^ (rr & 7)) << 4);
-        *reinterpret_cast<uint4*>(dst + (size_t)rr * M + piece * 16) = *reinterpret_cast<const uint4*>(buf + off);
-        if (dir == 1) *reinterpret_cast<uint4*>(p.Aq + (size_t)(m0 + rr) * N + c0 + piece * 16) = *reinterpret_cast<const uint4*>(buf + 16384 + off);
+        *reinterpret_cast<uint4*>(dst + (size_t)rr * pitch + piece * 16) = *reinterpret_cast<const uint4*>(buf + off);
+        if (KIND == PREP_Y) *reinterpret_cast<uint4*>(p.Aq + (size_t)(m0 + rr) * N + c0 + piece * 16) = *reinterpret_cast<const uint4*>(buf + 16384 + off);
       }
     };
     if (KIND == PREP_Y) {
@@ -471,8 +477,7 @@ __global__ void __launch_bounds__(PT, 3) k_prep(const __grid_constant__ PrepArgs
     } else if (KIND == PREP_Z) {
       rotate(2);
     } else {
-#pragma unroll 1
-      for (int dir = isz ? 2 : 0; dir < (isz ? 3 : 2); ++dir) rotate(dir);
+      rotate(isz ? 2 : (tile >= tiles_y ? 1 : 0));
     }
   }
   if (PASS == 0) {
@@ -499,8 +504,9 @@ static int prep_launch(PrepArgs p, uint32_t* scratch, int words, cudaStream_t st
   const int sms = dev_sm_count();
   if (sms <= 0) return DET_ERR_CUDA;
   const long long ty = p.dY ? (long long)(p.M / PT) * (p.N / PT) : 0, tz = (long long)(p.M / PT) * (p.K / PT);
-  const bool one = ty + tz <= 3 * sms;
-  const int gy = one ? (int)(ty + tz) : (int)(ty < 3 * sms ? ty : 3 * sms), gz = one ? gy : (int)(tz < 3 * sms ? tz : 3 * sms);
+  const long long items = 2 * ty + tz;
+  const bool one = items <= PREP_ONE_ROUNDS * 3 * sms;
+  const int gy = one ? (int)(items < 3 * sms ? items : 3 * sms) : (int)(ty < 3 * sms ? ty : 3 * sms), gz = one ? gy : (int)(tz < 3 * sms ? tz : 3 * sms);
   const int n[3] = {gy, gy, gz};
   const bool room = 2 * gy + gz <= words;
   for (int k = 0, at = 0; k < 3; at += p.mx.n[k++]) {
