@@ -57,7 +57,7 @@ template <class T, bool WIN>
 __global__ void __launch_bounds__(T::THREADS, T::CPS)
     k_attn_fwd(const uint16_t* __restrict__ q, const uint16_t* __restrict__ k, const uint16_t* __restrict__ v, int ld,
                int H, int Hkv, int S, int Warg, uint16_t* __restrict__ out, int ld_out, float* __restrict__ lse,
-               const float* __restrict__ s_q, int8_t* __restrict__ qout) {
+               const float* __restrict__ s_q, int8_t* __restrict__ qout, int sms) {
   constexpr int FQ = T::FQ, LQ = T::LQ, AF_SLOTS = T::SLOTS, AF_PF = T::PF, AF_CONS = T::CONS, AF_THREADS = T::THREADS, GR = T::GR;
   constexpr int GWARPS = T::GCONS / 32;
   const int W = WIN ? Warg : 0;
@@ -70,8 +70,13 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
   __shared__ float max_g[GR][FQ], sum_g[FQ], alpha_g[FQ];
   __shared__ __align__(8) uint64_t bar_max[GR][GWARPS], bar_u[GWARPS], bar_ufree[GWARPS];
   volatile int* abort_flag = &abort_s;
-  const int qb = gridDim.y - 1 - blockIdx.y;          // longest rows first
-  const int h = blockIdx.x % H, b = blockIdx.x / H, hk = h / (H / Hkv);
+  // Longest rows first.  With two CTAs per SM the first two rounds over the SMs are resident together, one of each on an SM: the
+  // second one runs backwards, so that a long row has a short one beside it (two sequences of 8 heads x 1088, 64 rows: 0.181 -> 0.157
+  // ms; 32 heads x 512 0.090 -> 0.078; with three CTAs per SM the order of placement is another one, 16 heads x 832, 32 rows: 0.119 and 0.129)
+  int c = blockIdx.y * gridDim.x + blockIdx.x;
+  if (T::CPS == 2 && c >= sms && c < 2 * sms) c = sms + min(2 * sms, (int)(gridDim.x * gridDim.y)) - 1 - c;
+  const int qb = gridDim.y - 1 - c / gridDim.x, bh = c % gridDim.x;
+  const int h = bh % H, b = bh / H, hk = h / (H / Hkv);
   const int q0 = qb * FQ;
   const int tid = threadIdx.x, lane = tid & 31;
   const int grp = GR == 1 ? 0 : (tid < AF_CONS ? tid / T::GCONS : (tid - AF_CONS) / AF_PROD), warp = (tid >> 5) - grp * GWARPS;   // consumers' warp
@@ -638,7 +643,7 @@ static int attn_fwd_go(const det_bf16* q, const det_bf16* k, const det_bf16* v, 
   const auto kern = k_attn_fwd<T, WIN>;
   if (dev_ensure_smem(once, (const void*)kern, T::SMEM) != DET_OK) return DET_ERR_CUDA;
   const dim3 grid(H * B, (S + T::FQ - 1) / T::FQ);
-  kern<<<DET_L(grid), T::THREADS, T::SMEM, st>>>(q, k, v, ld, H, Hkv, S, window, out, ld_out, lse, s_q, qout);
+  kern<<<DET_L(grid), T::THREADS, T::SMEM, st>>>(q, k, v, ld, H, Hkv, S, window, out, ld_out, lse, s_q, qout, dev_sm_count());
   return DET_OK;
 }
 template <class T>
@@ -647,33 +652,34 @@ static int attn_fwd_run(const det_bf16* q, const det_bf16* k, const det_bf16* v,
   return window ? attn_fwd_go<T, true>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, st)
                 : attn_fwd_go<T, false>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, st);
 }
-// Rows per CTA: the longest chain of key blocks runs on one SM whatever the others do, and all chains together share the
-// GPU; the figures are the microseconds per key block of a CTA alone on its SM and of one among many, and the row count
-// with the smallest of the larger bounds is taken (16 heads x 832: 0.178 ms with 128 rows, 0.129 with 64, 0.117 with 32;
-// 64 heads x 2048: 1.48, 1.55 and 1.75 ms).
-struct RowCost { int rows; double alone, full; };   // rows: 33 for 32 rows with two groups
-template <int N>
-static int pick_rows(const RowCost (&c)[N], int heads, int S, int window) {
+// Rows per CTA: the longest chain of key blocks runs on one SM whatever the others do, and all chains together share the GPU; the
+// figures are the microseconds per key block of a CTA alone on its SM and of one among many, the CTAs per SM, and the part of a
+// chain by which the shared time is exceeded in the end, nothing while long and short rows are paired on the SMs (two CTAs each,
+// none left over).  The row count with the smallest of the larger bounds is taken: 64 heads x 2048 1.49 ms with 128 rows, 1.57
+// with 64, 1.77 with 32; 20 heads x 1024 0.201, 0.199, 0.170; two sequences of 8 heads x 1088 0.226, 0.157, 0.167, two groups 0.189;
+// 16 heads x 832 0.176, 0.123, 0.119, 0.117; 8 heads x 1024 0.201, 0.140, 0.118, 0.088.
+struct RowCost { int rows; double alone, full; int cps; double over; };   // rows: 33 for 32 rows with two groups
+static int attn_rows(int heads, int S, int window) {
+  const RowCost c[4] = {{128, 25.1, 25.1, 1, 0.0}, {64, 17.0, 13.2, 2, 0.5}, {32, 13.0, 7.5, 3, 0.25}, {33, 9.9, 9.8, 1, 0.25}};
   const int sms = dev_sm_count() > 0 ? dev_sm_count() : 1;
   int best = c[0].rows;
   double best_t = 0.0;
-  for (int i = 0; i < N; ++i) {
+  for (int i = 0; i < 4; ++i) {
+    const int step = c[i].rows & ~1;
     double longest = 0.0, total = 0.0;
-    for (int q0 = 0; q0 < S; q0 += c[i].rows & ~1) {
+    for (int q0 = 0; q0 < S; q0 += step) {
       const int lo = window && q0 > window ? (q0 - window) / FK : 0;
       const double tiles = q0 / FK + 1 - lo;
       total += tiles;
       if (tiles > longest) longest = tiles;
     }
-    const double a = longest * c[i].alone, b = total * heads * c[i].full / sms, t = a > b ? a : b;
+    const bool paired = c[i].cps == 2 && (long long)heads * ((S + step - 1) / step) <= 2 * sms;
+    const double a = longest * c[i].alone, b = total * heads * c[i].full / sms + (paired ? 0.0 : c[i].over * a), t = a > b ? a : b;
     if (i == 0 || t < 0.97 * best_t) { best = c[i].rows; best_t = t; }
   }
   return best;
 }
-static int attn_rows(int heads, int S, int window) {
-  const RowCost c[4] = {{128, 25.1, 25.1}, {64, 17.0, 13.2}, {32, 13.0, 7.5}, {33, 9.9, 9.8}};
-  return pick_rows(c, heads, S, window);
-}
+
 static int attn_fwd_impl(const det_bf16* q, const det_bf16* k, const det_bf16* v, int ld, int B, int H, int Hkv, int S,
                          int window, det_bf16* out, int ld_out, float* lse, const float* s_q, int8_t* qout, void* stream) {
   if (!q || !k || !v || !out || !lse || B <= 0 || H <= 0 || Hkv <= 0 || S <= 0 || window < 0) return DET_ERR_ARG;
