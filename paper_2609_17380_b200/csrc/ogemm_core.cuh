@@ -208,9 +208,10 @@ struct OgemmArgs {
   int window;           // sliding window W (multiple of 128; 0 = none): only |query - key| < W contributes
   int range_mode;       // 0: whole contraction; 1: c >= first row of the tile (causal, per key); 2: c < last row + 1 of the tile
                         // (with a window, mode 1 also stops at c < i0 + W + TM and mode 2 starts at c >= i0 - W)
-  int order;            // OG_LEAD: the next launch is OG_FILL; OG_FILL: independent of the launch before, fills the SMs that it leaves
+  int order;            // OG_LEAD: the next launch is OG_FILL; OG_FILL: independent of the launch before, fills the SMs that it leaves;
+                        // OG_BACK: a causal grid with its shortest contractions first
 };
-enum { OG_LEAD = 1, OG_FILL = 2 };
+enum { OG_LEAD = 1, OG_FILL = 2, OG_BACK = 4 };
 
 // Tile TM x TN, thread tile 8 x CT, LY lanes of a warp along the rows, ST ring slots, PF slabs in flight in the producers'
 // registers, CPS CTAs per SM; RC / RP: registers of a consumer / producer thread after the hand-over (0: none).
@@ -261,9 +262,10 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS) k_ogemm(const OgemmArgs p)
   __shared__ __align__(8) uint64_t bar_full[ST], bar_empty[ST];
   __shared__ int abort_s;
   volatile int* abort_flag = &abort_s;
-  // causal grids: the row tile is the slowest grid index, longest contraction first
+  // causal grids: the row tile is the slowest grid index, longest contraction first (OG_BACK: last)
   const bool causal = p.range_mode != 0;
-  const int ti = causal ? (p.range_mode == 2 ? (int)(gridDim.z - 1 - blockIdx.z) : (int)blockIdx.z) : (int)blockIdx.y;
+  const bool down = (p.range_mode == 2) != ((p.order & OG_BACK) != 0);
+  const int ti = causal ? (down ? (int)(gridDim.z - 1 - blockIdx.z) : (int)blockIdx.z) : (int)blockIdx.y;
   const int zidx = causal ? (int)blockIdx.y : (int)blockIdx.z;
   const int i0 = ti * TM, j0 = blockIdx.x * TN;
   const long long zb = zidx / p.H, zh = zidx % p.H;
