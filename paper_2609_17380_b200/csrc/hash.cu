@@ -43,16 +43,32 @@ __device__ __forceinline__ uint32_t sha_maj(uint32_t a, uint32_t b, uint32_t c) 
 __device__ __forceinline__ uint32_t small_s0(uint32_t w) { return rotr32(w, 7) ^ rotr32(w, 18) ^ (w >> 3); }
 __device__ __forceinline__ uint32_t small_s1(uint32_t w) { return rotr32(w, 17) ^ rotr32(w, 19) ^ (w >> 10); }
 
-// one compression: 64 rounds with the message schedule kept in a rolling window of 16 words
-__device__ __forceinline__ void sha_rounds(uint32_t (&h)[8], uint32_t (&w)[16]) {
+// a + b on the multiply-add pipe, with `one` a 1 that the compiler does not know
+__constant__ uint32_t c_one_u = 1u;
+__device__ __forceinline__ uint32_t opaque_one() {
+  uint32_t one;
+  asm volatile("mov.u32 %0, %1;" : "=r"(one) : "r"(c_one_u));
+  return one;
+}
+__device__ __forceinline__ uint32_t add_mad(uint32_t a, uint32_t b, uint32_t one) {
+  uint32_t d;
+  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(one), "r"(b));
+  return d;
+}
+// one compression: 64 rounds with the message schedule kept in a rolling window of 16 words.  The integer pipe is what a
+// thread per chunk is bound by (96 % busy with 21 logic, shift and add instructions a round, 1 GiB at 0.86 TB/s), while the
+// multiply-add pipe idles, so most additions go there: 1.03 TB/s with the ones below, 0.86 to 1.02 with other choices (all
+// of the schedule 1.02, without the schedule 1.01, the round constant's too 0.92).
+__device__ __forceinline__ void sha_rounds(uint32_t (&h)[8], uint32_t (&w)[16], uint32_t one) {
   constexpr uint32_t K[64] = {SHA_K_LIST};
   uint32_t a = h[0], b = h[1], c = h[2], d = h[3], e = h[4], f = h[5], g = h[6], hh = h[7];
 #pragma unroll
   for (int i = 0; i < 64; ++i) {
-    if (i >= 16) w[i & 15] += small_s0(w[(i + 1) & 15]) + w[(i + 9) & 15] + small_s1(w[(i + 14) & 15]);
-    const uint32_t t1 = hh + big_s1(e) + sha_ch(e, f, g) + K[i] + w[i & 15];
-    const uint32_t t2 = big_s0(a) + sha_maj(a, b, c);
-    hh = g; g = f; f = e; e = d + t1; d = c; c = b; b = a; a = t1 + t2;
+    if (i >= 16)
+      w[i & 15] = add_mad(add_mad(w[(i + 9) & 15], small_s1(w[(i + 14) & 15]), one), w[i & 15] + small_s0(w[(i + 1) & 15]), one);
+    const uint32_t t1 = add_mad(big_s1(e), add_mad(sha_ch(e, f, g), add_mad(hh, w[i & 15] + K[i], one), one), one);
+    const uint32_t t2 = add_mad(big_s0(a), sha_maj(a, b, c), one);
+    hh = g; g = f; f = e; e = add_mad(d, t1, one); d = c; c = b; b = a; a = add_mad(t2, t1, one);
   }
   h[0] += a; h[1] += b; h[2] += c; h[3] += d; h[4] += e; h[5] += f; h[6] += g; h[7] += hh;
 }
@@ -106,14 +122,14 @@ __device__ __forceinline__ ShaMsg sha_msg(const HashJobs& jobs, uint32_t chunk) 
   return m;
 }
 
-// Many chunks: a thread per chunk.  Bound by the integer pipe: 22 logic, shift and add instructions a round at half an
-// instruction per cycle and scheduler make 0.87 TB/s the ceiling at 1.965 GHz, and 1 GiB is hashed at 0.84 TB/s (additions
-// written as integer multiply-adds, meant for another pipe, measured 0.81: they take the same issue slots).
+// Many chunks: a thread per chunk, the next 64-byte block on its way while the rounds of the current one run (sha_rounds says what
+// bounds it).
 __global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJobs jobs, uint8_t* __restrict__ out) {
   grid_dep();
   const uint32_t c = blockIdx.x * 64 + threadIdx.x;
   if (c >= jobs.first[jobs.n]) return;
   const ShaMsg msg = sha_msg<false>(jobs, c);
+  const uint32_t one = opaque_one();
   uint32_t h[8], w[16];
   sha_init(h);
   const uint32_t full = msg.len / 64, nb = msg.blocks();
@@ -141,7 +157,7 @@ __global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJ
 #pragma unroll
       for (int k = 0; k < 16; ++k) w[k] = t[k];
     }
-    sha_rounds(h, w);
+    sha_rounds(h, w, one);
   }
   sha_store(out + (size_t)c * 32, h);
 }
