@@ -295,9 +295,11 @@ __device__ __forceinline__ bool finite1(float x) { return (__float_as_uint(x) & 
 //     time, and rows of dY, columns of dY and columns of Z are work of different CTAs and go through ONE copy of the butterflies
 //     and of the quantiser (PREP_ONE; second pass of 256 tokens x 512, cold: 5.8 us, 7.4 with rows and columns of a tile one
 //     after the other in a CTA, 27 with a copy of the code for each).  Over
-//     many tiles the copies are the faster form (first pass over 16384 tokens x 16384: 0.20 against 0.23 ms), dY in one launch (PREP_Y), Z in
+//     many tiles the copies are the faster form (first pass over 16384 tokens x 16384: 0.17 against 0.20 ms), dY in one launch (PREP_Y), Z in
 //     another (PREP_Z) beside it.
-constexpr size_t PREP2_SMEM = (size_t)2 * PT * 256 + 2 * PT * sizeof(float);
+// All shared memory is dynamic: sixteen bytes of static shared memory in front of the buffers put their rows across 128-byte lines
+// and cost 10 % of the first pass (16384 tokens x 16384: 0.191 ms instead of 0.174).
+constexpr size_t PREP2_SMEM = (size_t)2 * PT * 256 + 2 * PT * sizeof(float) + (PT / 32) * sizeof(uint32_t);
 
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gsrc) : "memory");
@@ -323,7 +325,7 @@ struct PrepArgs {
   float* s_u;              // the step of Z, or null
 };
 
-__device__ __forceinline__ uint32_t block_max(uint32_t x, uint32_t (&box)[PT / 32]) {
+__device__ __forceinline__ uint32_t block_max(uint32_t x, uint32_t* box) {
   x = __reduce_max_sync(0xffffffffu, x);
   if ((threadIdx.x & 31) == 0) box[threadIdx.x >> 5] = x;
   __syncthreads();
@@ -337,8 +339,8 @@ constexpr int PREP_ONE_ROUNDS = 2;
 template <int PASS, int KIND>
 __global__ void __launch_bounds__(PT, 3) k_prep(const __grid_constant__ PrepArgs p) {
   extern __shared__ __align__(16) uint8_t pbuf[];
-  __shared__ uint32_t box[PT / 32];
   float* swb = reinterpret_cast<float*>(pbuf + 2 * PT * 256);      // [2][128]
+  uint32_t* box = reinterpret_cast<uint32_t*>(swb + 2 * PT);
   const int t = threadIdx.x, M = p.M, N = p.N, K = p.K;
   const int ntn = N / PT, ntk = K / PT, tiles_y = KIND != PREP_Z && p.dY ? ntn * (M / PT) : 0;
   const int ntiles_y = KIND == PREP_ONE ? 2 * tiles_y : tiles_y;      // one by one: rows of all tiles of dY, then their columns
