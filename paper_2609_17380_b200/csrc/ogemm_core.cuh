@@ -453,7 +453,11 @@ static int og_pick(const OgemmArgs& p, int batches, int share, int widest, doubl
     // the last chains of a causal grid run beside idle SMs: half a chain, on average (three contractions side by side, 16 heads
     // on 4 x 4096: 4.36 ms for the backward with square tiles, 4.07 with half ones; 16 x 16 heads x 2048: 3.43 and 3.56)
     const double full = p.range_mode ? b + 0.5 * a : b, alone = a > full ? a : full;
-    const double busy = tiles <= sms ? tiles * a : alone * sms, t = (busy + beside) / sms > alone ? (busy + beside) / sms : alone;
+    // what is queued beside also fills the last round of a grid of several (8192 tokens: 512 tiles of 128 x 256 are 3.5 rounds, and
+    // the head's two gradients take 1.4 ms of 55 less than with 128 x 128 tiles of dH)
+    const double each = (double)p.C * p.nG * r.tm * r.tn / r.full;
+    const double busy = tiles <= sms ? tiles * a : (beside > 0.0 ? tiles * each : alone * sms);
+    const double t = (busy + beside) / sms > (beside > 0.0 ? a : alone) ? (busy + beside) / sms : (beside > 0.0 ? a : alone);
     if (c == widest || t < (p.range_mode ? 1.0 : 0.95) * best_t) { best = c; best_t = t; }
   }
   return best;
