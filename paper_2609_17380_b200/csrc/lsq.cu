@@ -109,6 +109,7 @@ template <int PASS>
 __global__ void __launch_bounds__(256) k_rot_rows(const uint16_t* __restrict__ dY, const float* __restrict__ s_w, int M,
                                                   int N, uint32_t* __restrict__ amax, int8_t* __restrict__ Aq) {
   // a warp owns RB consecutive 128-element blocks of one row and issues all its loads before any arithmetic
+  grid_dep();
   constexpr int RB = 8;
   const int lane = threadIdx.x & 31;
   const int gpr = (N / 128 + RB - 1) / RB;  // warp groups per row
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(256) k_rot_rows(const uint16_t* __restrict__ d
 template <int PASS>
 __global__ void __launch_bounds__(128) k_rotc(const uint16_t* __restrict__ in, int R, int C, uint32_t* __restrict__ amax,
                                               int8_t* __restrict__ outT) {
-  const int col = blockIdx.x * 128 + threadIdx.x;
+  const int col = blockIdx.x * 128 + threadIdx.x + grid_dep();
   const int r0 = blockIdx.y * 128;
   float vf[128];
   const uint16_t* p = in + (size_t)r0 * C + col;
@@ -197,7 +198,7 @@ __global__ void __launch_bounds__(128) k_rotc(const uint16_t* __restrict__ in, i
 __global__ void __launch_bounds__(128) k_transpose8(const int8_t* __restrict__ in, int R, int C, int8_t* __restrict__ outT,
                                                     float* __restrict__ s_u) {
   __shared__ __align__(16) uint8_t tile[128 * 128];
-  const int t = threadIdx.x, c0 = blockIdx.x * 128, r0 = blockIdx.y * 128;
+  const int t = threadIdx.x, c0 = blockIdx.x * 128 + grid_dep(), r0 = blockIdx.y * 128;
   if (s_u && blockIdx.x == 0 && blockIdx.y == 0 && t == 0) s_u[0] = 1.0f;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -594,7 +595,7 @@ extern "C" int det_lsq_quantize_weight(const det_bf16* W, const float* s_w, int 
       const int rc = prep_launch(pa, (uint32_t*)ws, 64, st);
       if (rc != DET_OK) return rc;
     } else {
-      k_transpose8<<<DET_L(dim3(K / 128, N / 128)), 128, 0, st>>>(qW, N, K, qWt_bwd, s_u);
+      launch_after(k_transpose8, dim3(K / 128, N / 128), 128, 0, st, qW, N, K, qWt_bwd, s_u);
     }
   }
   DET_CHECK_LAUNCH();
@@ -675,11 +676,11 @@ extern "C" int det_linear_bwd(const det_bf16* dY, const det_bf16* X, const int8_
     const size_t ngrp = (size_t)M * ((N / 128 + 7) / 8);  // warp groups of 8 blocks
     const unsigned g1 = (unsigned)((ngrp + 7) / 8);
     dim3 gG(N / 128, M / 128);
-    k_rot_rows<0><<<DET_L(g1), 256, 0, st>>>(dY, s_w, M, N, amax + 0, nullptr);
-    k_rotc<0><<<DET_L(gG), 128, 0, st>>>(dY, M, N, amax + 1, nullptr);
-    k_rot_rows<1><<<DET_L(g1), 256, 0, st>>>(dY, s_w, M, N, amax + 0, Aq);
-    k_rotc<1><<<DET_L(gG), 128, 0, st>>>(dY, M, N, amax + 1, GqT);
-    k_transpose8<<<DET_L(dim3(K / 128, M / 128)), 128, 0, st>>>(qX, M, K, ZqT, nullptr);
+    launch_after(k_rot_rows<0>, g1, 256, 0, st, dY, s_w, M, N, amax + 0, nullptr);
+    launch_after(k_rotc<0>, gG, 128, 0, st, dY, M, N, amax + 1, nullptr);
+    launch_after(k_rot_rows<1>, g1, 256, 0, st, dY, s_w, M, N, amax + 0, Aq);
+    launch_after(k_rotc<1>, gG, 128, 0, st, dY, M, N, amax + 1, GqT);
+    launch_after(k_transpose8, dim3(K / 128, M / 128), 128, 0, st, qX, M, K, ZqT, nullptr);
   }
   DET_CHECK_LAUNCH();
   const float rotf = rot ? 0x1p-7f : 1.0f;

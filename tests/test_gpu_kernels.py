@@ -23,18 +23,19 @@ def _sync():
     torch.cuda.synchronize()
 
 
-# chunk counts of a launch around the rule between the two hash kernels (a warp of eight chains per scheduler: 8 * 4 * SMs),
+# chunk counts of a launch around the rule between the two hash kernels (a warp of eight chains per scheduler: 8 * 4 * SMs) and
+# between one and two warps per eight chains (half of that),
 # tensors of one, two and three levels, an empty one, byte counts off the 4- and 64-byte grid, more tensors than one
 # launch takes
 @pytest.mark.parametrize("sizes", [
     [16, 0, 4096, 4095, 4097, 61, 64, 55, 56, 128 * 4096, 128 * 4096 + 1, 0],
-    "edge", "edge+1", [128 * 128 * 4096 + 4096 + 48, 5000, 129 * 4096 + 3],
+    "edge", "edge+1", "pair", "pair+1", [128 * 128 * 4096 + 4096 + 48, 5000, 129 * 4096 + 3],
     [(37 * i) % 9000 for i in range(300)],
 ])
 def test_hash_batch(det, sizes):
     if isinstance(sizes, str):
-        edge = 8 * 4 * det.det_device_sm_count()
-        sizes = [4096 * (edge - 200) + 4096 * (sizes != "edge"), 4096 * 199 + 777]
+        edge = 8 * (4 if "edge" in sizes else 2) * det.det_device_sm_count()
+        sizes = [4096 * (edge - 200) + 4096 * sizes.endswith("+1"), 4096 * 199 + 777]
     rng = np.random.default_rng(len(sizes))
     blobs = [rng.integers(0, 256, n).astype(np.uint8) for n in sizes]
     tensors = [dev(b) for b in blobs]
@@ -216,8 +217,8 @@ def test_weight_rotation(det, N, K):
 
 
 # LSQ linear at sizes where the tile of the int8 GEMMs changes (64, 128, 256 columns, CTA pairs), with a last round that is
-# nearly empty and with dimensions that only narrow tiles divide
-@pytest.mark.parametrize("M,N,K", [(128, 128, 128), (384, 640, 384), (1024, 3072, 1024), (1664, 3072, 1024)])
+# nearly empty and with dimensions that only narrow tiles divide; the operand preparation with one item, two items and many tiles per CTA
+@pytest.mark.parametrize("M,N,K", [(128, 128, 128), (384, 640, 384), (1024, 3072, 1024), (1664, 3072, 1024), (2048, 3072, 1024)])
 def test_linear_tiles(det, M, N, K):
     import torch
     X, W = synth.normal_bf16((M, K), 1.0, seed=M, tid=1), synth.normal_bf16((N, K), 0.02, seed=M, tid=2)
