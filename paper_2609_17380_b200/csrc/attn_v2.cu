@@ -31,7 +31,7 @@ __device__ __forceinline__ const uint16_t* head_row(const uint16_t* X, int ld, i
 // rows of a head-packed bf16 tensor -> slices [Z*S, 128] and exponents [Z*S]; one warp per row, four values per lane
 __global__ void __launch_bounds__(256) k_slice_heads(const uint16_t* __restrict__ X, int ld, int H, int S, int rows,
                                                      int8_t* __restrict__ hi, int8_t* __restrict__ lo, int32_t* __restrict__ E) {
-  const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int r = blockIdx.x * 8 + (threadIdx.x >> 5) + grid_dep(), lane = threadIdx.x & 31;
   if (r >= rows) return;
   const int z = r / S, i = r - z * S;
   const uint2 w = __ldg(reinterpret_cast<const uint2*>(head_row(X, ld, H, S, z, i) + lane * 4));
@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(256) k_slice_heads(const uint16_t* __restrict_
 // [z*128 + c][position].  grid (1, S/128, Z), thread = dimension.
 __global__ void __launch_bounds__(128) k_col_exp_heads(const uint16_t* __restrict__ X, int ld, int H, int S,
                                                        int32_t* __restrict__ E) {
-  const int c = threadIdx.x, r0 = blockIdx.y * 128, z = blockIdx.z;
+  const int c = threadIdx.x, r0 = blockIdx.y * 128, z = blockIdx.z + grid_dep();
   const uint16_t* base = head_row(X, ld, H, S, z, r0) + c;
   int key = 0;
 #pragma unroll 8
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(128) k_slice_cols_heads(const uint16_t* __rest
                                                           const int32_t* __restrict__ E, int8_t* __restrict__ hiT,
                                                           int8_t* __restrict__ loT) {
   __shared__ __align__(16) uint8_t tile[2][128 * 128];
-  const int t = threadIdx.x, r0 = blockIdx.y * 128, z = blockIdx.z;
+  const int t = threadIdx.x, r0 = blockIdx.y * 128, z = blockIdx.z + grid_dep();
   const uint16_t* base = head_row(X, ld, H, S, z, r0) + t;
   const int e = E[z * 128 + t] & 0xFF;
   uint32_t hw[32], lw[32];
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256) k_softmax_v2(const float* __restrict__ Sr
   __shared__ float leafs[32];
   __shared__ float redf[8];
   __shared__ int redi[8];
-  const int row = blockIdx.x, i = row % S, n = i + 1;
+  const int row = blockIdx.x + grid_dep(), i = row % S, n = i + 1;
   const int kend = ((i >> 7) + 1) << 7;           // the keys the row tile's contraction runs over
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nl = (n + 255) >> 8;                  // leaves of the row
@@ -261,10 +261,10 @@ extern "C" int det_attn_fwd_v2(const det_bf16* q, const det_bf16* k, const det_b
   int32_t *Eq = (int32_t*)(w + L.Eq), *Ek = (int32_t*)(w + L.Ek), *Ev = (int32_t*)(w + L.Ev), *Ep = (int32_t*)(w + L.Ep);
   float *Sraw = (float*)(w + L.Sraw), *invl = (float*)(w + L.invl);
   if (cudaMemsetAsync(Ev, 0, (size_t)Z * 128 * 4, st) != cudaSuccess) return DET_ERR_CUDA;
-  k_slice_heads<<<DET_L((rows + 7) / 8), 256, 0, st>>>(q, ld, H, S, rows, Qh, Ql, Eq);
-  k_slice_heads<<<DET_L((rows + 7) / 8), 256, 0, st>>>(k, ld, H, S, rows, Kh, Kl, Ek);
-  k_col_exp_heads<<<DET_L(dim3(1, S / 128, Z)), 128, 0, st>>>(v, ld, H, S, Ev);
-  k_slice_cols_heads<<<DET_L(dim3(1, S / 128, Z)), 128, 0, st>>>(v, ld, H, S, Ev, VTh, VTl);
+  launch_after(k_slice_heads, (rows + 7) / 8, 256, 0, st, q, ld, H, S, rows, Qh, Ql, Eq);
+  launch_after(k_slice_heads, (rows + 7) / 8, 256, 0, st, k, ld, H, S, rows, Kh, Kl, Ek);
+  launch_after(k_col_exp_heads, dim3(1, S / 128, Z), 128, 0, st, v, ld, H, S, Ev);
+  launch_after(k_slice_cols_heads, dim3(1, S / 128, Z), 128, 0, st, v, ld, H, S, Ev, VTh, VTl);
   DET_CHECK_LAUNCH();
   SlArgs a = {};
   a.Ea = Eq; a.Eb = Ek; a.out = Sraw; a.rowscale = nullptr;
@@ -272,8 +272,8 @@ extern "C" int det_attn_fwd_v2(const det_bf16* q, const det_bf16* k, const det_b
   a.causal_tiles = 1; a.krange = 0; a.epi = SL_F32;
   int rc = sliced_gemm_launch(Qh, Ql, Kh, Kl, a, status_dev, st);
   if (rc != DET_OK) return rc;
-  if (S <= 2048) k_softmax_v2<1><<<DET_L(rows), 256, 0, st>>>(Sraw, S, lse, invl, Ph, Pl, Ep);
-  else k_softmax_v2<SM2_LPW><<<DET_L(rows), 256, 0, st>>>(Sraw, S, lse, invl, Ph, Pl, Ep);
+  if (S <= 2048) launch_after(k_softmax_v2<1>, rows, 256, 0, st, Sraw, S, lse, invl, Ph, Pl, Ep);
+  else launch_after(k_softmax_v2<SM2_LPW>, rows, 256, 0, st, Sraw, S, lse, invl, Ph, Pl, Ep);
   DET_CHECK_LAUNCH();
   SlArgs u = {};
   u.Ea = Ep; u.Eb = Ev; u.out = out; u.rowscale = invl;
