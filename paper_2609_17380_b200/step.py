@@ -304,12 +304,19 @@ class Replay:
         det.det_rmsnorm_bwd(det.DET_BF16, dy, x, g, rstd, T, D, tmp, dg, self.ws)
         det.det_residual_add(dx, tmp, T * D, dx)
 
+    def _set_tokens(self, dst, part):
+        """dst <- the tokens of a micro-batch, row after row; rows of another length count as one sequence of tokens."""
+        if part.shape == (self.cfg.micro_batch, self.cfg.seq):
+            dst.view(part.shape).copy_(part)          # without a contiguous copy in between
+        else:
+            dst.copy_(part.reshape(-1))
+
     def forward(self, tokens_mb, calibrate=False):
         cfg = self.cfg
         D, Fh, V, L, T = cfg.d_model, cfg.ffn, cfg.vocab, cfg.n_layers, cfg.tokens_per_microbatch
         B, H, S = cfg.micro_batch, cfg.n_heads, cfg.seq
-        self.tok.view(B, S).copy_(tokens_mb[:, :-1])
-        self.lab.view(B, S).copy_(tokens_mb[:, 1:])
+        self._set_tokens(self.tok, tokens_mb[:, :-1])
+        self._set_tokens(self.lab, tokens_mb[:, 1:])
         Hkv, QW = cfg.kv_heads, cfg.qkv_width
         x = self.act[0]["x"] if L else self.xf
         if cfg.embed_norm:

@@ -1,0 +1,41 @@
+"""The step driver's host side (buffers, views, what it hands to the library), on the CPU with the library's calls recorded."""
+import pytest
+import torch
+
+import paper_2609_17380_b200 as det
+from paper_2609_17380_b200 import step as dstep
+
+HOST = ("det_accum", "det_adamw_desc", "det_grad_accum_nbufs")
+
+
+@pytest.fixture
+def calls(monkeypatch):
+    """(name, arguments) of every library call that would launch something."""
+    log = []
+    for name in dir(det):
+        if name.startswith("det_") and not name.endswith("ws_bytes") and name not in HOST:
+            monkeypatch.setattr(det, name, lambda *a, _name=name, **k: log.append((_name, a)))
+    return log
+
+
+def _replay(**kw):
+    cfg = dict(n_layers=2, d_model=256, n_heads=2, ffn=256, vocab=512, seq=64, micro_batch=2, mesh=(1, 2, 1))
+    cfg.update(kw)
+    return dstep.Replay(dstep.ModelConfig(**cfg), device="cpu")
+
+
+# tokens of a micro-batch: [rows, sequence + 1] of the configuration, or any rows whose tokens come to the same number
+@pytest.mark.parametrize("shape", [(2, 65), (1, 129), (4, 33), (128, 2)])
+def test_tokens_accepted(calls, shape):
+    r = _replay()
+    t = torch.arange(shape[0] * shape[1], dtype=torch.int32).reshape(shape)
+    r.forward(t)
+    assert torch.equal(r.tok, t[:, :-1].reshape(-1)) and torch.equal(r.lab, t[:, 1:].reshape(-1))
+
+
+# too few or too many are refused, one row for all sequences and one token for all positions among them
+@pytest.mark.parametrize("shape", [(1, 65), (2, 2), (2, 64), (3, 65), (2, 1)])
+def test_tokens_refused(calls, shape):
+    r = _replay()
+    with pytest.raises(RuntimeError):
+        r.forward(torch.zeros(shape, dtype=torch.int32))
