@@ -482,8 +482,8 @@ class Replay:
         losses = self._losses if n_mb == self._losses.numel() else torch.empty(n_mb, dtype=F32, device=self.dev)
         for mb in range(n_mb):
             torch.cuda.nvtx.range_push("microbatch%d" % mb)      # lets a profiler select one micro-batch
-            self.loss_mean = losses[mb:mb + 1]
             self.forward(tokens[mb])
+            losses[mb:mb + 1].copy_(self.loss_mean)
             self.backward()
             with self.span("grad_accum"):
                 det.det_grad_accum_push(st, self.gmb)

@@ -39,3 +39,23 @@ def test_tokens_refused(calls, shape):
     r = _replay()
     with pytest.raises(RuntimeError):
         r.forward(torch.zeros(shape, dtype=torch.int32))
+
+
+# loss_mean is one buffer: who holds it sees the loss of the latest forward pass, and a forward pass after a step leaves what
+# the step reports alone
+def test_loss_buffer_stays(calls, monkeypatch):
+    r, n = _replay(), [0.0]
+
+    def xent(logits, target, rows, V, z, loss_row, lse, loss_mean, *rest):
+        n[0] += 1.0
+        loss_mean.fill_(n[0])
+
+    monkeypatch.setattr(det, "det_xent_fwd", xent)
+    monkeypatch.setattr(torch.cuda.nvtx, "range_push", lambda *a: None)
+    monkeypatch.setattr(torch.cuda.nvtx, "range_pop", lambda *a: None)
+    held = r.loss_mean
+    tokens = torch.zeros((2, 2, 65), dtype=torch.int32)
+    assert r.step(tokens)["losses"] == [1.0, 2.0]
+    assert held is r.loss_mean and held.item() == 2.0
+    r.forward(tokens[0])
+    assert held.item() == 3.0 and r._losses.tolist() == [1.0, 2.0]
