@@ -114,7 +114,6 @@ class Replay:
         z = lambda n, dt: torch.zeros(n, dtype=dt, device=device)
         self.pbf = z(p, I16)                       # bf16 parameters (bit patterns), canonical order
         self.sx = z(L * 4, F32)                    # LSQ activation steps, [layer, (qkv, o, gu, down)]
-        self._sx = [[self.sx[4 * l + i:4 * l + i + 1] for i in range(4)] for l in range(L)]
         self.m, self.v = z(g, F32), z(g, F32)      # Adam moments, gradient layout
         self.gmb = z(g, F32)                       # gradient of the current micro-batch
         self.gout_padded = z(max(g, gout_len or 0), F32)
@@ -191,18 +190,21 @@ class Replay:
 
     # ---- parameter access ------------------------------------------------------------------------------
     def _view(self, which, name):
-        """The part of the buffer self.<which> that belongs to one parameter, sliced once per buffer."""
+        """The part of the buffer self.<which> that belongs to one parameter (or, by (layer, linear), to one activation step),
+        sliced once for as long as the buffer and its memory are the same ones."""
         buf = getattr(self, which)
         cache = self._views.get(which)
-        if cache is None or cache[0] is not buf:
-            cache = self._views[which] = (buf, {})
-        v = cache[1].get(name)
+        if cache is None or cache[0] is not buf or cache[1] != buf.data_ptr():
+            cache = self._views[which] = (buf, buf.data_ptr(), {})
+        v = cache[2].get(name)
         if v is None:
-            if which == "sx":
-                lo, n = 4 * int(name.split(".")[0][1:]), 4
-            else:
+            if which != "sx":
                 lo, n = (self.poff if which == "pbf" else self.goff)[name], _numel(self.shape[name])
-            v = cache[1][name] = buf[lo:lo + n]
+            elif isinstance(name, tuple):
+                lo, n = 4 * name[0] + name[1], 1
+            else:
+                lo, n = 4 * int(name.split(".")[0][1:]), 4
+            v = cache[2][name] = buf[lo:lo + n]
         return v
 
     def p(self, name):
@@ -271,7 +273,7 @@ class Replay:
     def _linear(self, l, w, idx, X, M, Y, qx, calibrate, prequantised=False):
         """prequantised: the kernel that produced X already wrote its int8 codes into qx."""
         d = self.lin[(l, w)]
-        sx = self._sx[l][idx]
+        sx = self._view("sx", (l, idx))
         if calibrate:
             det.det_lsq_act_scale_init(X, M * d["K"], sx, self.ws)
         with self.span("linear_fwd"):
@@ -330,7 +332,7 @@ class Replay:
         dn, res = self.tmp[1][:T * D], None           # the residual sum that ends a layer runs with the norm that starts the next
         for l in range(L):
             a = self.act[l]
-            sxl = self._sx[l]
+            sxl = [self._view("sx", (l, i)) for i in range(4)] if fuse else None
             self._norm(res, dn, a["x"], "l%d.attn_norm" % l, a["n1"], a["rstd1"], sxl[0] if fuse else None, a["qx_qkv"])
             self._linear(l, "w_qkv", 0, a["n1"], T, a["qkv"], a["qx_qkv"], calibrate, fuse)
             qp = vp = a["qkv"].data_ptr()
@@ -377,7 +379,7 @@ class Replay:
     def _linear_bwd(self, l, w, idx, dY, X, qx, M, dX):
         d = self.lin[(l, w)]
         name = d["name"]
-        sx = self._sx[l][idx]
+        sx = self._view("sx", (l, idx))
         ds = self.g(self.gmb, "l%d.s_x" % l)[idx:idx + 1]
         with self.span("linear_bwd"):
             det.det_linear_bwd(dY, X, qx, self.p(name), d["qWt"], sx, d["s_w"], d["s_u"], M, d["N"], d["K"],

@@ -59,3 +59,37 @@ def test_loss_buffer_stays(calls, monkeypatch):
     assert held is r.loss_mean and held.item() == 2.0
     r.forward(tokens[0])
     assert held.item() == 3.0 and r._losses.tolist() == [1.0, 2.0]
+
+
+# a buffer of the state replaced, or given other memory, between two calls: the library gets the memory that is there now
+@pytest.mark.parametrize("swap", ["object", "memory"])
+def test_replaced_buffers_are_used(calls, swap):
+    r = _replay()
+    t = torch.zeros((2, 65), dtype=torch.int32)
+
+    def passes():
+        del calls[:]
+        r.prepare_weights()
+        r.forward(t, calibrate=True)
+        r.forward(t)
+        r.backward()
+        r.optimizer()
+
+    def touched():
+        return {a.data_ptr() for _, args in calls for x in args for a in (x if isinstance(x, list) else [x]) if torch.is_tensor(a)}
+
+    passes()
+    names, old = ("sx", "pbf", "m", "v", "gmb"), {}
+    for n in names:
+        old[n] = getattr(r, n).detach()[:]                  # keeps the old memory, so that no new buffer can be at its address
+        if swap == "object":
+            setattr(r, n, getattr(r, n).clone())
+        else:
+            getattr(r, n).data = getattr(r, n).clone()
+    passes()
+    for n in names:
+        lo = old[n].data_ptr()
+        stale = [p for p in touched() if lo <= p < lo + old[n].numel() * old[n].element_size()]
+        assert not stale, n
+    steps = {r.sx.data_ptr() + 4 * i for i in range(8)}
+    assert steps <= touched()
