@@ -496,13 +496,19 @@ class Replay:
         with self.span("hash"):
             names = self._queue_hashes(per_tensor_hashes)
             out = self._out.cpu().numpy()          # the step's one synchronisation
-        scalars = out[4:12].view(np.float32)
-        res = {"hashes": self._hex(names, out[16:].tobytes()), "status": int(out[:4].view(np.int32)[0])}
+        res = {"hashes": self._hex(names, self._reported(out, self.roots).tobytes()), "status": int(self._reported(out, self.status)[0])}
         if want_losses:
-            ls = (out[16 + self.roots.numel():].view(np.float32) if losses is self._losses else losses.cpu().numpy())
+            ls = self._reported(out, losses)
             res.update(losses=[float(x) for x in ls], loss=float(np.mean(ls.astype(np.float64))),
-                       grad_norm=float(scalars[0]), coef=float(scalars[1]))
+                       grad_norm=float(self._reported(out, self.norm)[0]), coef=float(self._reported(out, self.coef)[0]))
         return res
+
+    def _reported(self, out, t):
+        """What t holds: its part of the report buffer's host copy, or a copy of its own where it lies elsewhere by now."""
+        lo, n = t.data_ptr() - self._out.data_ptr(), t.numel() * t.element_size()
+        if 0 <= lo <= out.size - n:
+            return out[lo:lo + n].view({F32: np.float32, I32: np.int32, torch.uint8: np.uint8}[t.dtype])
+        return t.cpu().numpy()
 
 
 def run_step(cfg, params, tokens, calibrate=True):

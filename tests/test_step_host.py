@@ -18,6 +18,20 @@ def calls(monkeypatch):
     return log
 
 
+@pytest.fixture
+def counted_losses(calls, monkeypatch):
+    """The losses of successive forward passes are 1, 2, ..."""
+    n = [0.0]
+
+    def xent(logits, target, rows, V, z, loss_row, lse, loss_mean, *rest):
+        n[0] += 1.0
+        loss_mean.fill_(n[0])
+
+    monkeypatch.setattr(det, "det_xent_fwd", xent)
+    monkeypatch.setattr(torch.cuda.nvtx, "range_push", lambda *a: None)
+    monkeypatch.setattr(torch.cuda.nvtx, "range_pop", lambda *a: None)
+
+
 def _replay(**kw):
     cfg = dict(n_layers=2, d_model=256, n_heads=2, ffn=256, vocab=512, seq=64, micro_batch=2, mesh=(1, 2, 1))
     cfg.update(kw)
@@ -43,16 +57,8 @@ def test_tokens_refused(calls, shape):
 
 # loss_mean is one buffer: who holds it sees the loss of the latest forward pass, and a forward pass after a step leaves what
 # the step reports alone
-def test_loss_buffer_stays(calls, monkeypatch):
-    r, n = _replay(), [0.0]
-
-    def xent(logits, target, rows, V, z, loss_row, lse, loss_mean, *rest):
-        n[0] += 1.0
-        loss_mean.fill_(n[0])
-
-    monkeypatch.setattr(det, "det_xent_fwd", xent)
-    monkeypatch.setattr(torch.cuda.nvtx, "range_push", lambda *a: None)
-    monkeypatch.setattr(torch.cuda.nvtx, "range_pop", lambda *a: None)
+def test_loss_buffer_stays(calls, counted_losses):
+    r = _replay()
     held = r.loss_mean
     tokens = torch.zeros((2, 2, 65), dtype=torch.int32)
     assert r.step(tokens)["losses"] == [1.0, 2.0]
@@ -93,3 +99,17 @@ def test_replaced_buffers_are_used(calls, swap):
         assert not stale, n
     steps = {r.sx.data_ptr() + 4 * i for i in range(8)}
     assert steps <= touched()
+
+
+# the scalars and roots that a step reports are those of the tensors the library was given, also where one of them was replaced
+def test_replaced_report_is_read(calls, counted_losses, monkeypatch):
+    r = _replay()
+    tokens = torch.zeros((2, 2, 65), dtype=torch.int32)
+    r.status, r.norm, r.coef = torch.tensor([4], dtype=torch.int32), torch.tensor([0.5]), torch.tensor([0.25])
+    monkeypatch.setattr(det, "det_tensor_hash_batch", lambda ts, roots, ws: roots.copy_(torch.arange(roots.numel()) % 251))
+    for moved in (False, True):
+        if moved:
+            r.roots = torch.zeros_like(r.roots)
+        res = r.step(tokens)
+        assert (res["status"], res["grad_norm"], res["coef"]) == (4, 0.5, 0.25)
+        assert res["hashes"]["embed"] == bytes(range(32)).hex()
