@@ -57,3 +57,23 @@ def test_host_side_argument_checks():
     assert lib.det_attn_fwd_v2(a1, a16, a16, 768, 1, 2, 256, a16, 256, a16, a16, big, None, None) == -3       # alignment
     assert lib.det_attn_fwd_v2(a16, a16, a16, 768, 1, 2, 256, a16, 256, a16, a16, ctypes.c_size_t(need - 1), None, None) == -4
     assert lib.det_attn_fwd_v2(None, a16, a16, 768, 1, 2, 256, a16, 256, a16, a16, big, None, None) == -1     # null operand
+
+
+# every tensor of a table is checked as a single argument is: one on the host, one with gaps or one that is too short is refused
+# before anything is launched (no GPU needed: the refusal comes first)
+def test_tables_are_checked():
+    import pytest
+    import torch
+    import paper_2609_17380_b200 as det
+    t = lambda n, dt=torch.float32: torch.zeros(n, dtype=dt)
+    desc = det.det_adamw_desc(1e-3, 0.9, 0.95, 1e-8, 0.0, 1)
+    bf = t(8, torch.int16)
+    for args in (([desc], [det.DET_BF16], [bf], [t(8)], [t(8)], [t(8)]),              # on the host
+                 ([desc], [det.DET_BF16], [bf], [t(4)], [t(8)], [t(8)]),              # a short gradient
+                 ([desc], [det.DET_BF16], [bf], [t(8)], [t(8)], [t(4)]),              # a short moment
+                 ([desc], [det.DET_F32], [bf], [t(8)], [t(8)], [t(8)]),               # 16 bits passed as 32
+                 ([desc], [], [bf], [t(8)], [t(8)], [t(8)])):                         # no type given
+        with pytest.raises(AssertionError):
+            det.det_adamw_batch(*args)
+    with pytest.raises(AssertionError):
+        det.det_tensor_hash_batch([t(64, torch.uint8)], t(32, torch.uint8), t(4096, torch.uint8))
