@@ -33,12 +33,13 @@ def _stale(target, deps):
 
 
 def build_binding(force=False):
-    """_binding.so from csrc/binding.cpp against the installed torch."""
-    src = os.path.join(CSRC, "binding.cpp")
-    if not force and not _stale(BINDING, [src]):
-        return BINDING
+    """_binding.so from csrc/binding.cpp against the installed torch and Python, whose versions are written beside the objects."""
     import sysconfig
     import torch
+    src, stamp = os.path.join(CSRC, "binding.cpp"), os.path.join(_DIR, "build", "_binding.versions")
+    versions = "torch %s, Python %s\n" % (torch.__version__, sysconfig.get_config_var("SOABI"))
+    if not force and not _stale(BINDING, [src]) and os.path.exists(stamp) and open(stamp).read() == versions:
+        return BINDING
     from torch.utils import cpp_extension
     lib = os.path.join(os.path.dirname(torch.__file__), "lib")
     inc = cpp_extension.include_paths("cuda") + [sysconfig.get_paths()["include"]]
@@ -47,6 +48,9 @@ def build_binding(force=False):
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("g++ failed for binding.cpp:\n%s" % r.stderr)
+    os.makedirs(os.path.dirname(stamp), exist_ok=True)
+    with open(stamp, "w") as f:
+        f.write(versions)
     return BINDING
 
 

@@ -77,3 +77,21 @@ def test_tables_are_checked():
             det.det_adamw_batch(*args)
     with pytest.raises(AssertionError):
         det.det_tensor_hash_batch([t(64, torch.uint8)], t(32, torch.uint8), t(4096, torch.uint8))
+
+
+# the binding is compiled against torch's headers: another torch version makes the object stale although its source is older
+def test_binding_follows_the_torch_version(monkeypatch):
+    import subprocess
+    import torch
+    from paper_2609_17380_b200 import build
+    build.build_binding()
+    runs = []
+    monkeypatch.setattr(subprocess, "run", lambda cmd, **k: runs.append(cmd) or subprocess.CompletedProcess(cmd, 1, "", "not run"))
+    build.build_binding()
+    assert not runs                                            # up to date
+    monkeypatch.setattr(torch, "__version__", torch.__version__ + ".1")
+    try:
+        build.build_binding()
+    except RuntimeError:
+        pass
+    assert len(runs) == 1
