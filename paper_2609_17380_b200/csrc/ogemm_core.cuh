@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS) k_ogemm(const OgemmArgs p)
   int slot = 0;
   uint32_t par = 0;
   for (int s = 0; s < nslab; ++s) {
-    if (!mbar_wait(&bar_full[slot], par, abort_flag, nullptr)) { if (FIX) return; break; }   // slot is full
+    if (!mbar_wait(&bar_full[slot], par, abort_flag, nullptr)) break;   // slot is full; after a wait that ran out the outputs are undefined
     const int4 t4 = *reinterpret_cast<const int4*>(tiny_s[slot]);
     if (t4.x | t4.y | t4.z | t4.w) slab_mac<false, TM, TN, CT>(As[slot], Bs[slot], ty, tx, acc);
     else if constexpr (CT == 16) slab_mac_ordered<TM, TN>(As[slot], Bs[slot], ty, tx, acc);

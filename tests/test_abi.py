@@ -95,3 +95,24 @@ def test_binding_follows_the_torch_version(monkeypatch):
     except RuntimeError:
         pass
     assert len(runs) == 1
+
+
+# a filling grid skips the wait at its start, so its last block has to wait at its end on every way out, that after an expired wait
+# included, or what comes next on the stream overlaps the launch before.  No wait can be made to expire from outside: the source is read
+def test_filling_kernels_always_reach_their_end():
+    csrc = os.path.join(ROOT, "paper_2609_17380_b200", "csrc")
+    found = 0
+    for name in sorted(os.listdir(csrc)):
+        if not name.endswith((".cu", ".cuh")) or name == "common.cuh":
+            continue
+        src = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        for body in src.split("__global__")[1:]:
+            if "grid_fill_end()" not in body:
+                continue
+            found += 1
+            body = body[:body.index("grid_fill_end()")]
+            if "setmaxnreg.inc" in body:                        # producer warps leave on their own; the consumers go to the end
+                body = body[body.index("setmaxnreg.inc"):]
+            body = re.sub(r"\[&\]\([^)]*\)(?: -> \w+)? \{.*?\n  \};", "", body, flags=re.S)      # a lambda returns to its caller
+            assert not re.search(r"\breturn\b", body), name
+    assert found >= 3
