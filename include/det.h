@@ -14,15 +14,15 @@
  *  - work is asynchronous on `stream` (a cudaStream_t passed as void*; NULL = default stream), except
  *    det_tensor_hash which synchronises that stream (det_tensor_hash_async does not).  Kernels are launched as
  *    programmatic dependents of each other where that pays: they wait on the device for what they depend on, and what comes
- *    after them on the stream comes after all of them.  Large calls of det_linear_bwd and det_lsq_quantize_weight run independent
+ *    after them on the stream comes after all of them.  Large calls of det_linear_bwd run independent
  *    kernels side by side on two auxiliary streams per device that
  *    the library creates on first use: they start where `stream` stands when the call is made and `stream` waits
  *    for them on every way out of the call (error returns included), so the caller still sees plain stream order.
  *    What the library keeps between calls is per DEVICE and set up under a lock on first use there: those two streams,
  *    the one-time opt-in of each kernel for large shared memory, the SM count, and the address of det_sum_static's
  *    scratch.  None of it outlives a cudaDeviceReset (do not call the library again after one).  No mode or option
- *    is process-wide.  Calls for one device may come from several host threads, except that two calls of the two
- *    functions above on one device at the same time would share the auxiliary streams: give those one thread per device;
+ *    is process-wide.  Calls for one device may come from several host threads, except that two calls of
+ *    det_linear_bwd on one device at the same time would share the auxiliary streams: give those one thread per device;
  *  - data-dependent scalars (LSQ steps, norms, losses) are device scalars so that no call forces a sync;
  *  - device-detected conditions (bad target index, a bounded wait that expired, a non-finite norm) are
  *    OR-ed into *status_dev (device int, may be NULL) as DET_DEV_* bits; kernels never trap;

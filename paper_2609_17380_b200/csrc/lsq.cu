@@ -522,13 +522,14 @@ static int prep_launch(PrepArgs p, uint32_t* scratch, int words, cudaStream_t st
     const int rc = prep_pass<PREP_ONE>(0, p, gy, st);
     return rc != DET_OK ? rc : prep_pass<PREP_ONE>(1, p, gy, st);
   }
+  if (!ty) {            // weights: everything stays on the caller's stream, and the call shares nothing with other threads
+    const int rc = prep_pass<PREP_Z>(0, p, gz, st);
+    return rc != DET_OK ? rc : prep_pass<PREP_Z>(1, p, gz, st);
+  }
   AuxScope aux(st);   // the tiles of Z do not depend on those of dY
   for (int pass = 0; pass < 2; ++pass) {
-    if (ty) {
-      const int rc = prep_pass<PREP_Y>(pass, p, gy, st);
-      if (rc != DET_OK) return rc;
-    }
-    const int rc = prep_pass<PREP_Z>(pass, p, gz, ty ? aux.aux(1) : st);
+    int rc = prep_pass<PREP_Y>(pass, p, gy, st);
+    if (rc == DET_OK) rc = prep_pass<PREP_Z>(pass, p, gz, aux.aux(1));
     if (rc != DET_OK) return rc;
   }
   return aux.join() ? DET_OK : DET_ERR_CUDA;

@@ -265,3 +265,39 @@ def test_norms_with_residual(det, rows, D, q):
     dxo, dgo = oracle.rmsnorm_bwd(dy, ho, gain, ro, bf=True)
     assert_same_bits(host(dx, np.uint16), oracle.residual_add(res, dxo), "dx")
     assert_same_bits(host(dg), dgo.reshape(-1), "dgain")
+
+
+# a weight of many tiles stays on the caller's stream: it does not wait for another stream's linear backward, whose kernels on the
+# auxiliary streams stand behind 0.2 s of other work
+def test_weight_quantisation_waits_for_nobody(det):
+    import time
+    import torch
+    M, N, K = 2048, 3072, 1024                                     # large enough for the auxiliary streams
+    X, dY, W = [dev(synth.normal_bf16(s, 0.1, seed=1, tid=t)) for t, s in enumerate(((M, K), (M, N), (N, K)))]
+    sw, one = dev(np.full(N, 1e-3, F)), dev(np.ones(1, F))
+    qX, qWt, status = dev(np.ones((M, K), np.int8)), dev(np.ones((K, N), np.int8)), torch.zeros(1, dtype=torch.int32, device="cuda")
+    dX, dW, ds, wb = empty((M, K), np.uint16), empty((N, K), F), empty((1,), F), ws(det.det_linear_bwd_ws_bytes(M, N, K))
+    big = dev(synth.normal_bf16((3072, 8320), 0.1, seed=2, tid=0))
+    out = [(empty((3072, 8320), np.int8), empty((8320, 3072), np.int8), empty((1,), F), ws(256)) for _ in range(8)]
+    backward = lambda: det.det_linear_bwd(dY, X, qX, W, qWt, one, sw, one, M, N, K, 128, dX, dW, ds, wb, status)
+    weights = lambda o: det.det_lsq_quantize_weight(big, sw, 3072, 8320, 128, o[0], o[1], o[2], o[3])
+    backward()                                                     # everything is loaded before it counts
+    weights(out[0])
+    _sync()
+    first, others, slept = torch.cuda.Stream(), [torch.cuda.Stream() for _ in out], torch.cuda.Event()
+    with torch.cuda.stream(first):
+        torch.cuda._sleep(400_000_000)
+        slept.record()
+        backward()
+    done = []
+    for s, o in zip(others, out):                                  # several: two streams can share a hardware queue
+        with torch.cuda.stream(s):
+            weights(o)
+            done.append(torch.cuda.Event())
+            done[-1].record()
+    free = False
+    end = time.monotonic() + 30
+    while not free and not slept.query() and time.monotonic() < end:
+        free = any(e.query() for e in done) and not slept.query()
+    _sync()
+    assert free
