@@ -50,7 +50,9 @@ __device__ __forceinline__ uint32_t opaque_one() {
   asm volatile("mov.u32 %0, %1;" : "=r"(one) : "r"(c_one_u));
   return one;
 }
+template <bool MAD>
 __device__ __forceinline__ uint32_t add_mad(uint32_t a, uint32_t b, uint32_t one) {
+  if (!MAD) return a + b;
   uint32_t d;
   asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(one), "r"(b));
   return d;
@@ -59,16 +61,18 @@ __device__ __forceinline__ uint32_t add_mad(uint32_t a, uint32_t b, uint32_t one
 // thread per chunk is bound by (96 % busy with 21 logic, shift and add instructions a round, 1 GiB at 0.86 TB/s), while the
 // multiply-add pipe idles, so most additions go there: 1.03 TB/s with the ones below, 0.86 to 1.02 with other choices (all
 // of the schedule 1.02, without the schedule 1.01, the round constant's too 0.92).
+template <bool MAD>
 __device__ __forceinline__ void sha_rounds(uint32_t (&h)[8], uint32_t (&w)[16], uint32_t one) {
   constexpr uint32_t K[64] = {SHA_K_LIST};
+  auto add = [one](uint32_t x, uint32_t y) { return add_mad<MAD>(x, y, one); };
   uint32_t a = h[0], b = h[1], c = h[2], d = h[3], e = h[4], f = h[5], g = h[6], hh = h[7];
 #pragma unroll
   for (int i = 0; i < 64; ++i) {
     if (i >= 16)
-      w[i & 15] = add_mad(add_mad(w[(i + 9) & 15], small_s1(w[(i + 14) & 15]), one), w[i & 15] + small_s0(w[(i + 1) & 15]), one);
-    const uint32_t t1 = add_mad(big_s1(e), add_mad(sha_ch(e, f, g), add_mad(hh, w[i & 15] + K[i], one), one), one);
-    const uint32_t t2 = add_mad(big_s0(a), sha_maj(a, b, c), one);
-    hh = g; g = f; f = e; e = add_mad(d, t1, one); d = c; c = b; b = a; a = add_mad(t2, t1, one);
+      w[i & 15] = add(add(w[(i + 9) & 15], small_s1(w[(i + 14) & 15])), w[i & 15] + small_s0(w[(i + 1) & 15]));
+    const uint32_t t1 = add(big_s1(e), add(sha_ch(e, f, g), add(hh, w[i & 15] + K[i])));
+    const uint32_t t2 = add(big_s0(a), sha_maj(a, b, c));
+    hh = g; g = f; f = e; e = add(d, t1); d = c; c = b; b = a; a = add(t2, t1);
   }
   h[0] += a; h[1] += b; h[2] += c; h[3] += d; h[4] += e; h[5] += f; h[6] += g; h[7] += hh;
 }
@@ -127,6 +131,7 @@ __device__ __forceinline__ ShaMsg sha_msg(const HashJobs& jobs, uint32_t chunk) 
 
 // Many chunks: a thread per chunk, the next 64-byte block on its way while the rounds of the current one run (sha_rounds says what
 // bounds it).
+template <bool MAD>
 __global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJobs jobs, uint8_t* __restrict__ out) {
   grid_dep();
   const uint32_t c = blockIdx.x * 64 + threadIdx.x;
@@ -160,7 +165,7 @@ __global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJ
 #pragma unroll
       for (int k = 0; k < 16; ++k) w[k] = t[k];
     }
-    sha_rounds(h, w, one);
+    sha_rounds<MAD>(h, w, one);
   }
   sha_store(out + (size_t)c * 32, h);
 }
@@ -170,7 +175,7 @@ __global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJ
 // and the chain itself is rounds alone: 14 instructions a round on the half-rate integer pipe instead of 22, ordered so that a and
 // e depend on the round before through one rotation, one exclusive or and one addition each.  While there are schedulers to
 // spare a second warp does the expanding, double-buffered.  65 blocks: 0.137 ms with a thread per chunk, 0.089 with
-// one warp per CTA, 0.076 with two.
+// one warp per CTA, 0.076 with two; with the padding a word at a time 0.118, 0.077 and 0.066.
 constexpr int SF_CH = 8, SF_PITCH = 68;
 template <bool ROOT>
 __global__ void __launch_bounds__(64) k_sha_few(const __grid_constant__ HashJobs jobs, uint8_t* __restrict__ out) {
@@ -256,10 +261,12 @@ __global__ void __launch_bounds__(64) k_sha_few(const __grid_constant__ HashJobs
   if (have && !expand && sub == 0) sha_store(out + (size_t)c * 32, h);
 }
 
-// The rule: as long as the warps of this form do not outnumber the schedulers, the chain's latency is what counts (3144 chunks: 0.097 ms with one warp
-// per CTA, 0.134 with two, 0.140 with a thread per chunk); with
-// two warps per scheduler both forms take about the same time (9000 chunks: 0.157 and 0.141 ms), beyond that a thread per
-// chunk wins.
+// The rule, 65 blocks a chunk, 148 SMs of four schedulers.  Where the latency of a chain is what counts the form with the shorter chain
+// is taken: four lanes per chunk and a second warp while there are schedulers to spare (8 to 2368 chunks: 0.066 ms, one warp 0.077, a
+// thread per chunk 0.118), one warp while its warps do not outnumber the schedulers (up to 4736 chunks: 0.079, 0.125, 0.118), then
+// a thread per chunk with plain additions up to one warp per scheduler (6000: 0.118, four lanes 0.145, the multiply-add pipe's longer
+// latency 0.127; 18944: 0.125, 0.282, 0.133).  Beyond that the integer pipe is what counts (20480: 0.211 plain, 0.178; 65536: 0.406, 0.339;
+// 262144: 1.33, 1.08).
 static void sha_few_launch(bool root, const HashJobs& jobs, uint32_t n, uint8_t* out, int sms, cudaStream_t st) {
   const unsigned ctas = (n + SF_CH - 1) / SF_CH;
   launch_after(root ? k_sha_few<true> : k_sha_few<false>, ctas, ctas <= 2u * (unsigned)sms ? 64 : 32, 0, st, jobs, out);
@@ -270,7 +277,7 @@ static int hash_level(const HashJobs& jobs, uint8_t* out, cudaStream_t st) {
   const int sms = dev_sm_count();
   if (sms <= 0) return DET_ERR_CUDA;
   if (n <= (uint32_t)sms * 4 * SF_CH) sha_few_launch(false, jobs, n, out, sms, st);
-  else launch_after(k_sha_chunks, (n + 63) / 64, 64, 0, st, jobs, out);
+  else launch_after(n <= (uint32_t)sms * 4 * 32 ? k_sha_chunks<false> : k_sha_chunks<true>, (n + 63) / 64, 64, 0, st, jobs, out);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }

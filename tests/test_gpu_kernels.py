@@ -23,19 +23,20 @@ def _sync():
     torch.cuda.synchronize()
 
 
-# chunk counts of a launch around the rule between the two hash kernels (a warp of eight chains per scheduler: 8 * 4 * SMs) and
-# between one and two warps per eight chains (half of that),
-# byte counts around every place that the padding of a block can start at, tensors of one, two and three levels, an empty one, byte counts off the 4- and 64-byte grid, more tensors than one
+# chunk counts of a launch around the rule between the two hash kernels (a warp of eight chains per scheduler: 8 * 4 * SMs),
+# between one and two warps per eight chains (half of that) and between plain and multiply-add additions (a warp of 32 chunks per
+# scheduler), byte counts around every place that the padding of a block can start at,
+# tensors of one, two and three levels, an empty one, byte counts off the 4- and 64-byte grid, more tensors than one
 # launch takes
 @pytest.mark.parametrize("sizes", [
     [16, 0, 4096, 4095, 4097, 61, 64, 55, 56, 128 * 4096, 128 * 4096 + 1, 0],
-    "edge", "edge+1", "pair", "pair+1", list(range(1, 130)) + [4096 + i for i in range(1, 65)], [128 * 128 * 4096 + 4096 + 48, 5000, 129 * 4096 + 3],
+    "edge", "edge+1", "pair", "pair+1", "flat", "flat+1", list(range(1, 130)) + [4096 + i for i in range(1, 65)], [128 * 128 * 4096 + 4096 + 48, 5000, 129 * 4096 + 3],
     [(37 * i) % 9000 for i in range(300)],
 ])
 def test_hash_batch(det, sizes):
     if isinstance(sizes, str):
-        edge = 8 * (4 if "edge" in sizes else 2) * det.det_device_sm_count()
-        sizes = [4096 * (edge - 200) + 4096 * sizes.endswith("+1"), 4096 * 199 + 777]
+        edge = {"edge": 32, "pair": 16, "flat": 128}[sizes.split("+")[0]] * det.det_device_sm_count()
+        sizes = [4096 * (edge - 200) + 4096 * sizes.endswith("+1"), 4096 * 199 + 777]          # edge or edge + 1 chunks
     rng = np.random.default_rng(len(sizes))
     blobs = [rng.integers(0, 256, n).astype(np.uint8) for n in sizes]
     tensors = [dev(b) for b in blobs]
