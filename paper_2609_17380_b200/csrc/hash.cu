@@ -130,10 +130,10 @@ __device__ __forceinline__ ShaMsg sha_msg(const HashJobs& jobs, uint32_t chunk) 
 }
 
 // Many chunks: a thread per chunk, the next 64-byte block on its way while the rounds of the current one run (sha_rounds says what
-// bounds it).
+// bounds it).  A plain launch that lets nothing in early: CTAs of the next level that wait on the same SMs cost these chains up to twice
+// their time (whole hash of 10240 chunks 0.463 -> 0.228 ms, of 65536 0.784 -> 0.485, of 262144 1.53 -> 1.23).
 template <bool MAD>
 __global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJobs jobs, uint8_t* __restrict__ out) {
-  grid_dep();
   const uint32_t c = blockIdx.x * 64 + threadIdx.x;
   if (c >= jobs.first[jobs.n]) return;
   const ShaMsg msg = sha_msg<false>(jobs, c);
@@ -277,7 +277,8 @@ static int hash_level(const HashJobs& jobs, uint8_t* out, cudaStream_t st) {
   const int sms = dev_sm_count();
   if (sms <= 0) return DET_ERR_CUDA;
   if (n <= (uint32_t)sms * 4 * SF_CH) sha_few_launch(false, jobs, n, out, sms, st);
-  else launch_after(n <= (uint32_t)sms * 4 * 32 ? k_sha_chunks<false> : k_sha_chunks<true>, (n + 63) / 64, 64, 0, st, jobs, out);
+  else if (n <= (uint32_t)sms * 4 * 32) k_sha_chunks<false><<<DET_L((n + 63) / 64), 64, 0, st>>>(jobs, out);
+  else k_sha_chunks<true><<<DET_L((n + 63) / 64), 64, 0, st>>>(jobs, out);
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
