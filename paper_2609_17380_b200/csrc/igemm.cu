@@ -551,7 +551,7 @@ static int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const EpiPa
 static int igemm_pick(int epi, int I, int J, int K, int force_one_cta) {
   const int sms = dev_sm_count() > 0 ? dev_sm_count() : 1;
   struct { int bn, bi, bj, units; double step, turn, epi[4]; } const c[4] = {     // epi: RAW, FWD, DX, DW
-      {512, 256, 256, sms / 2, 0.365, 0.9, {6.6, 4.2, 10.0, 6.6}}, {256, 128, 256, sms, 0.375, 0.5, {6.2, 4.0, 9.3, 6.2}},
+      {512, 256, 256, sms / 2, 0.365, 0.9, {6.6, 4.2, 10.0, 6.6}}, {256, 128, 256, sms, 0.375, 0.5, {8.4, 4.0, 9.3, 6.2}},
       {128, 128, 128, sms, 0.30, 0.5, {3.8, 1.7, 5.7, 3.8}}, {64, 128, 64, sms, 0.30, 0.5, {1.8, 1.7, 3.7, 1.8}}};
   int best = 0;
   double best_t = 0.0;
