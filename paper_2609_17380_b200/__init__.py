@@ -64,7 +64,8 @@ _SIGNATURES = {
     "det_grad_accum_result": "ippp", "det_adamw_step": "ipippppzp", "det_adamw_batch": "ipppppppipp",
     "det_tensor_hash_ws_bytes": "zz", "det_tensor_hash_async": "ipzppzp", "det_tensor_hash": "ipzppzp",
     "det_tensor_hash_batch_ws_bytes": "zpi", "det_tensor_hash_batch": "ippippzp", "det_test_prim": "iipppzp",
-    "det_residual_rmsnorm_fwd": "ipppiifpppppp", "det_rmsnorm_bwd_residual": "ippppiippppzp", "det_test_igemm_tn": "ippiiipipp", "det_test_wait_timeout": "iplp",
+    "det_residual_rmsnorm_fwd": "ipppiifpppppp", "det_rmsnorm_bwd_residual": "ippppiippppzp", "det_test_igemm_tn": "ippiiipipp", "det_test_lmhead_tile": "iiippiiipip",
+    "det_test_wait_timeout": "iplp",
 }
 
 _lib = None
@@ -376,6 +377,10 @@ def det_attn_fwd_v2(q, k, v, ld, B, H, S, out, ld_out, lse, ws, status_dev=None)
 def det_lmhead_bwd(dlogits, H, W, M, V, K, dH, dW, first_chunk):
     _check("det_lmhead_bwd", load().det_lmhead_bwd(_ptr(dlogits), _ptr(H), _ptr(W), M, V, K,
                                                    _ptr(dH), _ptr(dW), first_chunk, _stream()))
+
+
+def det_test_lmhead_tile(which, tile, A, B, M, V, K, out, first_chunk=1):
+    _check("det_test_lmhead_tile", load().det_test_lmhead_tile(which, tile, _ptr(A), _ptr(B), M, V, K, _ptr(out), first_chunk, _stream()))
 
 
 # ---- gradient accumulation, AdamW, hash ---------------------------------------------------------------------------

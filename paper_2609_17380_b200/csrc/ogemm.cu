@@ -11,6 +11,7 @@
 // the fused one is not).  Each slab is therefore checked for factors below 2^-63 while it is staged; clean
 // slabs use the fused instruction, the others the two-instruction sequence.
 #include "ogemm_core.cuh"
+#include "../../include/det_test.h"
 
 using namespace det;
 
@@ -46,6 +47,22 @@ extern "C" int det_lmhead_bwd(const float* dlogits, const det_bf16* H, const det
   int rc = ogemm_launch<CONTIG, STRIDED, true, true, 0>(h, 1, 1, st, (double)M * V * K / OG_RATES[0].full);
   if (rc != DET_OK) return rc;
   rc = ogemm_launch<STRIDED, STRIDED, true, false, 0>(w, 1, 1, st);
+  if (rc != DET_OK) return rc;
+  DET_CHECK_LAUNCH();
+  return DET_OK;
+}
+
+// The three contractions of the head one by one, with the tile (an index into OG_RATES) given instead of picked
+extern "C" int det_test_lmhead_tile(int which, int tile, const void* A, const det_bf16* B, int M, int V, int K, void* out, int first_chunk,
+                                    void* stream) {
+  if (!A || !B || !out || M <= 0 || V <= 0 || K <= 0 || which < 0 || which > 2 || tile < 0 || tile > 3) return DET_ERR_ARG;
+  if (K % 16 || V % (which ? 16 : 4) || (which && M % 8)) return DET_ERR_SHAPE;
+  if (!aligned16(A) || !aligned16(B) || !aligned16(out)) return DET_ERR_ALIGN;
+  cudaStream_t st = (cudaStream_t)stream;
+  int rc;
+  if (which == 0) rc = ogemm_tile<CONTIG, CONTIG, false, false, 0>(tile, plain_args(A, B, out, M, V, K, K, K, V, 0), 1, st);
+  else if (which == 1) rc = ogemm_tile<CONTIG, STRIDED, true, true, 0>(tile, plain_args(A, B, out, M, K, V, V, K, K, 0), 1, st);
+  else rc = ogemm_tile<STRIDED, STRIDED, true, false, 0>(tile, plain_args(A, B, out, V, K, M, V, K, K, first_chunk ? 0 : 1), 1, st);
   if (rc != DET_OK) return rc;
   DET_CHECK_LAUNCH();
   return DET_OK;

@@ -466,13 +466,17 @@ template <int WIDEST> struct OgFirst { typedef OgWide T; };
 template <> struct OgFirst<1> { typedef OgSquare T; };
 // WIDEST: 0, or 1 where the output has no 256 columns (the head dimension of the attention contractions is 128)
 template <int AMODE, int BMODE, bool AF32, bool OUT_BF16, int WIDEST>
-static int ogemm_launch(const OgemmArgs& p, int batches, int share, cudaStream_t st, double beside = 0.0) {
-  switch (og_pick(p, batches, share, WIDEST, beside)) {
+static int ogemm_tile(int tile, const OgemmArgs& p, int batches, cudaStream_t st) {
+  switch (tile) {
     case 0: return ogemm_run<AMODE, BMODE, AF32, OUT_BF16, typename OgFirst<WIDEST>::T>(p, batches, st);
     case 1: return ogemm_run<AMODE, BMODE, AF32, OUT_BF16, OgSquare>(p, batches, st);
     case 2: return ogemm_run<AMODE, BMODE, AF32, OUT_BF16, OgHalf>(p, batches, st);
     default: return ogemm_run<AMODE, BMODE, AF32, OUT_BF16, OgSmall>(p, batches, st);
   }
+}
+template <int AMODE, int BMODE, bool AF32, bool OUT_BF16, int WIDEST>
+static int ogemm_launch(const OgemmArgs& p, int batches, int share, cudaStream_t st, double beside = 0.0) {
+  return ogemm_tile<AMODE, BMODE, AF32, OUT_BF16, WIDEST>(og_pick(p, batches, share, WIDEST, beside), p, batches, st);
 }
 
 }  // namespace det

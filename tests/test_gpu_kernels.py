@@ -48,8 +48,8 @@ def test_hash_batch(det, sizes):
         assert raw[32 * i:32 * i + 32].hex() == oracle.tensor_hash(b), (i, sizes[i])
 
 
-# LM head at sizes where the tile choice of the ordered contractions changes (32x64, 64x128, 128x128, 128x256) with ragged
-# rows and columns; the last one has a grid of several full rounds in the weight gradient
+# LM head through its entry points, ragged rows and columns; at these sizes the dispatch takes 32x64 and 128x128 tiles (every tile is run by
+# test_lmhead_every_tile); the last one has a grid of several full rounds in the weight gradient
 @pytest.mark.parametrize("M,V,K", [(8, 16, 16), (40, 80, 48), (136, 2064, 80), (392, 4112, 176), (1032, 8208, 32), (264, 16400, 528)])
 def test_lmhead_tiles(det, M, V, K):
     H, W = synth.normal_bf16((M, K), 1.0, seed=M, tid=1), synth.normal_bf16((V, K), 0.05, seed=M, tid=2)
@@ -64,6 +64,34 @@ def test_lmhead_tiles(det, M, V, K):
     dH_o, dW_o = oracle.lmhead_bwd(g, H, W)
     assert_same_bits(host(dH, np.uint16), dH_o, "dH")
     assert_same_bits(host(dW), dW_o, "dW")
+
+
+# the three contractions of the head on each of the four tiles: one tile and less, ragged rows and columns in the last tile of either
+# direction, one slab and many, a weight gradient that goes on from a chunk before, slabs with values whose products can be subnormal
+@pytest.mark.parametrize("tile", [0, 1, 2, 3])
+@pytest.mark.parametrize("M,V,K,tiny", [(8, 16, 16, False), (136, 272, 304, False), (200, 528, 80, True), (392, 784, 560, True)])
+def test_lmhead_every_tile(det, tile, M, V, K, tiny):
+    H, W = synth.normal_bf16((M, K), 1.0, seed=M, tid=1), synth.normal_bf16((V, K), 0.05, seed=M, tid=2)
+    g = synth.normal_f32((M, V), 1e-3, seed=M, tid=3)
+    if tiny:
+        rng = np.random.default_rng(M)
+        for a in (H, W, g):
+            at = rng.integers(0, a.size, 12)
+            v = (F(2.0) ** rng.integers(-66, -61, 12)).astype(F)
+            a.reshape(-1)[at] = v if a is g else synth.to_bf16(v)
+    dH_, dW_, dg = dev(H), dev(W), dev(g)
+    lg, dH, dW = empty((M, V), F), empty((M, K), np.uint16), empty((V, K), F)
+    det.det_test_lmhead_tile(0, tile, dH_, dW_, M, V, K, lg)
+    det.det_test_lmhead_tile(1, tile, dg, dW_, M, V, K, dH)
+    det.det_test_lmhead_tile(2, tile, dg, dH_, M, V, K, dW, 1)
+    _sync()
+    dH_o, dW_o = oracle.lmhead_bwd(g, H, W)
+    assert_same_bits(host(lg), oracle.lmhead_fwd(H, W), "logits")
+    assert_same_bits(host(dH, np.uint16), dH_o, "dH")
+    assert_same_bits(host(dW), dW_o, "dW")
+    det.det_test_lmhead_tile(2, tile, dg, dH_, M, V, K, dW, 0)
+    _sync()
+    assert_same_bits(host(dW), oracle.lmhead_bwd(g, H, W, dW_o)[1], "dW continued")
 
 
 # version-2 gradients where a row of logits is long enough for eight warps (4096 values), and one step below
@@ -194,7 +222,7 @@ def test_adamw_many_tensors(det, sizes, clip):
         assert_same_bits(host(dv[i]), vo, "v %d" % i)
 
 
-# the rotated transposed weight codes, two columns per integer: codes at both ends of the range (all of one sign, so that the plain
+# the rotated transposed weight codes: codes at both ends of the range (all of one sign, so that the plain
 # sum is +-2^14), a column block without a partner, more than one tile per CTA
 @pytest.mark.parametrize("N,K", [(128, 128), (256, 384), (3072, 8320)])
 def test_weight_rotation(det, N, K):
@@ -218,8 +246,9 @@ def test_weight_rotation(det, N, K):
 
 
 # LSQ linear at sizes where the tile of the int8 GEMMs changes (64, 128, 256 columns, CTA pairs), with a last round that is
-# nearly empty and with dimensions that only narrow tiles divide; the operand preparation with one item, two items and many tiles per CTA
-@pytest.mark.parametrize("M,N,K", [(128, 128, 128), (384, 640, 384), (1024, 3072, 1024), (1664, 3072, 1024), (2048, 3072, 1024)])
+# nearly empty and with dimensions that only narrow tiles divide; the operand preparation one item per CTA, two, and (the last) more tiles of dY and of Z than CTAs,
+# so that a CTA's buffers change places
+@pytest.mark.parametrize("M,N,K", [(128, 128, 128), (384, 640, 384), (1024, 3072, 1024), (1664, 3072, 1024), (2048, 3072, 1024), (10240, 768, 896)])
 def test_linear_tiles(det, M, N, K):
     import torch
     X, W = synth.normal_bf16((M, K), 1.0, seed=M, tid=1), synth.normal_bf16((N, K), 0.02, seed=M, tid=2)
@@ -302,3 +331,25 @@ def test_weight_quantisation_waits_for_nobody(det):
         free = any(e.query() for e in done) and not slept.query()
     _sync()
     assert free
+
+
+# the forward pass with int8 P.V over many key blocks: nine and eleven per row block (with the last row block ragged), six in a window,
+# so that the two value buffers, the four block scales and the barriers' parities come round again; every block of 128 keys has a value
+# range of its own, so that a stale scale or buffer shows
+@pytest.mark.parametrize("B,H,Hkv,S,W", [(1, 2, 2, 1088, 0), (2, 2, 1, 1344, 0), (1, 4, 2, 1472, 640)])
+def test_int8_pv_many_blocks(det, B, H, Hkv, S, W):
+    import torch
+    HD, KD = H * 128, Hkv * 128
+    ld = HD + 2 * KD
+    x = synth.from_bf16(synth.normal_bf16((B * S, ld), 1.0, seed=S, tid=1)).astype(F)
+    x[:, HD + KD:] *= (F(3.0) ** ((np.arange(B * S) % S // 128 * 5) % 7 - 3).astype(F))[:, None]
+    qkv = synth.to_bf16(x)
+    d = dev(qkv)
+    q = d.data_ptr()
+    out, lse, status = empty((B * S, HD), np.uint16), empty((B, H, S), F), torch.zeros(1, dtype=torch.int32, device="cuda")
+    det.det_attn_fwd_int8pv(q, q + 2 * HD, q + 2 * (HD + KD), ld, B, H, S, out, HD, lse, status, Hkv=Hkv, window=W)
+    _sync()
+    assert int(status.item()) == 0
+    oout, olse = oracle.attn_fwd(qkv, B, H, S, Hkv=Hkv, window=W, int8_pv=True)
+    assert_same_bits(host(lse), olse, "lse")
+    assert_same_bits(host(out, np.uint16), oout, "out")
