@@ -59,7 +59,8 @@ typedef enum {
 
 /* bits OR-ed into *status_dev by kernels */
 #define DET_DEV_TARGET 1    /* cross-entropy target outside [0, V) */
-#define DET_DEV_TIMEOUT 2   /* a bounded in-kernel wait expired; outputs of that launch are undefined */
+#define DET_DEV_TIMEOUT 2   /* a bounded in-kernel wait expired; outputs of that launch are undefined (calls without a status_dev
+                             * argument, the ordered attention and LM-head calls among them, cannot report it) */
 #define DET_DEV_NONFINITE 4 /* non-finite gradient norm */
 
 typedef enum { DET_F32 = 0, DET_BF16 = 1 } det_dtype;

@@ -714,7 +714,7 @@ extern "C" size_t det_attn_bwd_ws_bytes(int B, int H, int Hkv, int S) {
   return 2 * align_up((size_t)B * H * S * S * 2, 256) + align_up((size_t)B * H * S * 4, 256);
 }
 
-// the fixed-point variant keeps its 64-bit accumulators in registers: no extra scratch
+// the fixed-point variant keeps its 64-bit totals in shared memory (k_ogemm): no extra scratch
 extern "C" size_t det_attn_bwd_fixq_ws_bytes(int B, int H, int Hkv, int S) { return det_attn_bwd_ws_bytes(B, H, Hkv, S); }
 
 template <class T>
@@ -782,9 +782,11 @@ static int attn_bwd_impl(const det_bf16* dout, const det_bf16* q, const det_bf16
   // independent of each other: each fills the SMs that the one before it leaves, so that the short blocks at the end of one grid
   // overlap with the long blocks at the start of the next (on three streams, 16 heads x 4096 with window 512: 1.472 ms forward and backward
   // against 1.425, two sequences of 8 x 1088 0.514 against 0.511).
-  // While the tiles of dV are resident at once, the dK tiles that join them start with the shortest, so that long and short ones share
+  // While dV has at most two 64-row tiles per SM (whatever tile og_pick takes), all of them resident at once, the dK tiles that join them
+  // start with the shortest, so that long and short ones share
   // an SM: 8 heads x 1024 0.174 -> 0.163 ms for the whole backward, two sequences of 8 x 1088 0.344 -> 0.330; with more tiles, or with
-  // the long chains of grouped heads, the longest dK must not come last (16 heads on 4 x 4096: 3.40 and 3.80 ms).
+  // the long chains of grouped heads, the longest dK must not come last (16 heads on 4 x 4096: 3.40 and 3.80 ms).  Grids of 128-row
+  // tiles that are resident although they have more 64-row tiles than that (8 heads x 2432 to 4096) keep the longest first.
   const bool pair = G == 1 && (long long)B * H * ((S + 63) / 64) <= 2 * dev_sm_count();
   for (int which = 0; which < 2; ++which) {
     OgemmArgs p = {};

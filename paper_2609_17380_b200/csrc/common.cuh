@@ -261,6 +261,10 @@ __device__ __forceinline__ int grid_dep() {
 // A kernel launched by launch_after that depends on nothing of the kernel before it, only on older ones, fills the SMs that one
 // leaves as soon as all CTAs of that one are running: it skips the wait, and one CTA of it, the last, waits here at its end, so that
 // whatever comes after this kernel on the stream comes after both.
+// What is older than the launch before has to be complete when that one triggers: it waits before it triggers (grid_dep), or it is a
+// plain launch that triggers at once (nothing older runs when it starts), or it is itself a filling launch behind one of these and this
+// kernel depends on neither.  Nothing checks that: behind a launch_after kernel that triggers without a wait, a filling one reads too
+// early.  Used so by ogemm_run (OG_LEAD on a plain launch, then OG_FILL) and by igemm_launch (fill = 1 behind another k_igemm).
 __device__ __forceinline__ void grid_fill_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_fill_end() {
   if (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
