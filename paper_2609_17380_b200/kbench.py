@@ -10,6 +10,7 @@ MB for profiler captures.  Rates are algorithmic bytes (or integer / floating-po
 import argparse
 import json
 import sys
+import time
 
 import torch
 
@@ -26,9 +27,18 @@ def flush_l2():
     _flush.zero_()
 
 
+SETTLE_S = 0.25   # a case behind one that drew the power limit starts at that one's lower clock for some 50 ms of work
+
+
 def timeit(fn, iters, warm=2):
+    """Median of `iters` calls, after `warm` calls and, where more than one is timed, as many more as it takes the clock to settle."""
     for _ in range(warm):
         fn()
+    torch.cuda.synchronize()
+    end = time.monotonic() + SETTLE_S
+    while iters > 1 and time.monotonic() < end:
+        fn()
+        torch.cuda.synchronize()
     ts = []
     for _ in range(iters):
         flush_l2()
