@@ -258,6 +258,12 @@ __device__ __forceinline__ int grid_dep() {
   return zero;
 }
 
+// The wait alone: the next kernel comes in when this one is complete.  CTAs that come in while every SM holds some of this one are packed, as
+// many on an SM as fit before the next SM gets any (behind 160 CTAs of 64 threads: 20 CTAs of 64 threads on 2 SMs, 148 of 256
+// threads on 19; one per SM when they come in after the end).  That costs nothing where they fill the GPU or wait for memory, but chains
+// that share a scheduler, or a grid meant to be one CTA per SM, take several times as long.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // A kernel launched by launch_after that depends on nothing of the kernel before it, only on older ones, fills the SMs that one
 // leaves as soon as all CTAs of that one are running: it skips the wait, and one CTA of it, the last, waits here at its end, so that
 // whatever comes after this kernel on the stream comes after both.

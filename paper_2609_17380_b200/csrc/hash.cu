@@ -130,8 +130,9 @@ __device__ __forceinline__ ShaMsg sha_msg(const HashJobs& jobs, uint32_t chunk) 
 }
 
 // Many chunks: a thread per chunk, the next 64-byte block on its way while the rounds of the current one run (sha_rounds says what
-// bounds it).  A plain launch that lets nothing in early: CTAs of the next level that wait on the same SMs cost these chains up to twice
-// their time (whole hash of 10240 chunks 0.463 -> 0.228 ms, of 65536 0.784 -> 0.485, of 262144 1.53 -> 1.23).
+// bounds it).  A plain launch that lets nothing in early: the few CTAs of the next level would be packed on two or three SMs (grid_wait in
+// common.cuh) and their chains share the schedulers there (whole hash of 10240 chunks 0.463 -> 0.228 ms, of 65536 0.784 -> 0.485, of 262144
+// 1.53 -> 1.23).
 template <bool MAD>
 __global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJobs jobs, uint8_t* __restrict__ out) {
   const uint32_t c = blockIdx.x * 64 + threadIdx.x;

@@ -35,10 +35,12 @@ __device__ __forceinline__ void load8_bits(const void* X, size_t idx, uint32_t (
 }
 // WPR warps per row: one, or the eight of a CTA where a row is long and the rows are few (one warp walks 32768 values twice at
 // the latency of its loads: 1024 rows of 32768 f32 values 0.163 ms, 0.059 with eight).
+// Neither this kernel nor the sliced contraction lets the next one in before it is complete: with that, logits of 384 tokens x 8064 x 640
+// took 39.0 us and 31.4 without (36.9 as plain launches), 1024 tokens 58.2, 52.7 and 53.3; both gradients of 1664 x 512 x 256 80.4 and 65.0.
 template <bool F32, int WPR>
 __global__ void __launch_bounds__(256) k_slice_rows(const void* __restrict__ X, int R, int K, int8_t* __restrict__ hi,
                                                     int8_t* __restrict__ lo, int32_t* __restrict__ E) {
-  grid_dep();
+  grid_wait();
   __shared__ int key_s[8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = WPR == 1 ? (int)blockIdx.x * 8 + warp : (int)blockIdx.x;
@@ -247,7 +249,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
-  grid_dep();
+  grid_wait();
   const int tiles_i = I / SL_T, tiles_j = J / SL_T, per_z = tiles_i * tiles_j, num_tiles = p.Z * per_z, kblocks = K / SL_BK;
   // tile t -> problem z, row tile it, column tile jt (the rows run fastest: the CTAs resident at one time share a tile of
   // B and stream A through L2); false when the tile does not exist; [k_lo, k_hi) = its steps along the contraction
