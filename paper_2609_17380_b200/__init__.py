@@ -408,15 +408,14 @@ def det_adamw_step(desc, pdtype, p, g, m, v, n):
 
 def det_adamw_batch(descs, pdtypes, ps, gs, ms, vs, coef_dev=None):
     """One launch for many tensors; coef_dev: device scalar every gradient is multiplied with first (in place)."""
-    k = len(ps)
-    table = lambda ts: (C.c_void_p * k)(*[_ptr(t) for t in ts])
-    assert k == len(descs) == len(pdtypes) == len(gs) == len(ms) == len(vs), "one entry per tensor in every list"
-    for kind, p, g, m, v in zip(pdtypes, ps, gs, ms, vs):
-        assert p.numel() == g.numel() == m.numel() == v.numel() and p.element_size() == (2 if kind == DET_BF16 else 4), \
-            "parameter, gradient and moments of a tensor differ in size"
+    k, numel = len(ps), torch.Tensor.numel
+    table = lambda ts: (C.c_void_p * k)(*map(_ptr, ts))
+    counts = list(map(numel, ps))
+    assert k == len(descs) == len(pdtypes) and all(list(map(numel, ts)) == counts for ts in (gs, ms, vs)) and \
+        [2 if kind == DET_BF16 else 4 for kind in pdtypes] == list(map(torch.Tensor.element_size, ps)), \
+        "one entry per tensor in every list; parameter, gradient and moments of a tensor have the same number of elements"
     _check("det_adamw_batch", load().det_adamw_batch((det_adamw_desc * k)(*descs), (C.c_int * k)(*pdtypes), table(ps), table(gs),
-                                                     table(ms), table(vs), (C.c_size_t * k)(*[t.numel() for t in ps]), k,
-                                                     _ptr(coef_dev), _stream()))
+                                                     table(ms), table(vs), (C.c_size_t * k)(*counts), k, _ptr(coef_dev), _stream()))
 
 
 def det_tensor_hash_ws_bytes(nbytes):
@@ -445,6 +444,6 @@ def det_tensor_hash_batch_ws_bytes(nbytes):
 def det_tensor_hash_batch(tensors, roots_dev, ws):
     """Queues the hashes of all tensors together; root t lands at roots_dev[32 t : 32 t + 32] in stream order."""
     k = len(tensors)
-    ptrs = (C.c_void_p * k)(*[_ptr(t) for t in tensors])
+    ptrs = (C.c_void_p * k)(*map(_ptr, tensors))
     counts = (C.c_size_t * k)(*[t.numel() * t.element_size() for t in tensors])
     _check("det_tensor_hash_batch", load().det_tensor_hash_batch(ptrs, counts, k, _ptr(roots_dev), *_ws(ws), _stream()))

@@ -89,6 +89,18 @@ def _numel(shape):
     return n
 
 
+class _Views(dict):
+    """Parts of a flat buffer by name, sliced on first use; good for as long as the buffer and its memory are the same ones."""
+
+    def __init__(self, buf, parts):
+        self.buf, self.address, self.parts = buf, buf.data_ptr(), parts
+
+    def __missing__(self, name):
+        lo, n = self.parts[name]
+        v = self[name] = self.buf[lo:lo + n]
+        return v
+
+
 class Replay:
     """Device state of the replay: parameters, optimizer moments, gradient buffers, saved activations."""
 
@@ -101,7 +113,7 @@ class Replay:
         self.specs = param_specs(cfg)
         D, Fh, V, L, T = cfg.d_model, cfg.ffn, cfg.vocab, cfg.n_layers, cfg.tokens_per_microbatch
         assert D == cfg.n_heads * 128, "head_dim is 128"
-        self.goff, self.poff, self._views = {}, {}, {}
+        self.goff, self.poff = {}, {}
         self.shape = dict((n, sh) for n, sh, _ in self.specs)
         g = p = 0
         for name, shape, kind in self.specs:
@@ -111,6 +123,15 @@ class Replay:
                 self.poff[name] = p
                 p += _numel(shape)
         self.n_grad = g
+        # where a parameter lies in the flat buffers, and by (layer, linear) a single activation step and its gradient
+        grads = {n: (lo, _numel(self.shape[n])) for n, lo in self.goff.items()}
+        steps = {"l%d.s_x" % l: (4 * l, 4) for l in range(L)}
+        for l in range(L):
+            steps.update({(l, i): (4 * l + i, 1) for i in range(4)})
+            grads.update({(l, i): (self.goff["l%d.s_x" % l] + i, 1) for i in range(4)})
+        self._views = {}
+        self._parts = dict(pbf={n: (lo, _numel(self.shape[n])) for n, lo in self.poff.items()}, sx=steps, gmb=grads, gout=grads, m=grads,
+                           v=grads)
         z = lambda n, dt: torch.zeros(n, dtype=dt, device=device)
         self.pbf = z(p, I16)                       # bf16 parameters (bit patterns), canonical order
         self.sx = z(L * 4, F32)                    # LSQ activation steps, [layer, (qkv, o, gu, down)]
@@ -189,31 +210,22 @@ class Replay:
         return {k: (len(v), sum(a.elapsed_time(b) for a, b in v)) for k, v in (self.prof or {}).items()}
 
     # ---- parameter access ------------------------------------------------------------------------------
-    def _view(self, which, name):
-        """The part of the buffer self.<which> that belongs to one parameter (or, by (layer, linear), to one activation step),
-        sliced once for as long as the buffer and its memory are the same ones."""
-        buf = getattr(self, which)
-        cache = self._views.get(which)
-        if cache is None or cache[0] is not buf or cache[1] != buf.data_ptr():
-            cache = self._views[which] = (buf, buf.data_ptr(), {})
-        v = cache[2].get(name)
-        if v is None:
-            if which != "sx":
-                lo, n = (self.poff if which == "pbf" else self.goff)[name], _numel(self.shape[name])
-            elif isinstance(name, tuple):
-                lo, n = 4 * name[0] + name[1], 1
-            else:
-                lo, n = 4 * int(name.split(".")[0][1:]), 4
-            v = cache[2][name] = buf[lo:lo + n]
-        return v
+    def _fresh(self):
+        """The views by buffer name, those of buffers that were replaced or given other memory since the last call made anew.  Called at
+        the start of every pass; within one the buffers stay."""
+        for which, parts in self._parts.items():
+            buf, v = getattr(self, which), self._views.get(which)
+            if v is None or v.buf is not buf or v.address != buf.data_ptr():
+                self._views[which] = _Views(buf, parts)
+        return self._views
 
     def p(self, name):
-        return self._view("sx" if name.endswith("s_x") else "pbf", name)
+        return self._fresh()["sx" if name.endswith("s_x") else "pbf"][name]
 
     def g(self, buf, name):
         for which in ("gmb", "gout", "m", "v"):
             if buf is getattr(self, which):
-                return self._view(which, name)
+                return self._fresh()[which][name]
         return buf[self.goff[name]:self.goff[name] + _numel(self.shape[name])]
 
     def load_params(self, params):
@@ -264,16 +276,16 @@ class Replay:
     # ---- step pieces --------------------------------------------------------------------------------------
     def prepare_weights(self):
         """Start of an optimizer step: re-pin every weight step from the current weights and quantise."""
-        hb = self.cfg.hadamard_block
-        for (l, w), d in self.lin.items():
-            W = self.p(d["name"])
+        hb, P = self.cfg.hadamard_block, self._fresh()["pbf"]
+        for d in self.lin.values():
+            W = P[d["name"]]
             det.det_lsq_weight_scale(W, d["N"], d["K"], 0, d["s_w"], self.ws)
             det.det_lsq_quantize_weight(W, d["s_w"], d["N"], d["K"], hb, d["qW"], d["qWt"], d["s_u"], self.ws)
 
     def _linear(self, l, w, idx, X, M, Y, qx, calibrate, prequantised=False):
         """prequantised: the kernel that produced X already wrote its int8 codes into qx."""
         d = self.lin[(l, w)]
-        sx = self._view("sx", (l, idx))
+        sx = self._views["sx"][l, idx]
         if calibrate:
             det.det_lsq_act_scale_init(X, M * d["K"], sx, self.ws)
         with self.span("linear_fwd"):
@@ -285,7 +297,7 @@ class Replay:
     def _norm(self, a, b, x, gain, y, rstd, s_q=None, qy=None):
         """y = RMSNorm of x, after x = a + b unless a is None; with s_q the next linear's int8 input too."""
         T, D = self.cfg.tokens_per_microbatch, self.cfg.d_model
-        g = self.p(gain)
+        g = self._views["pbf"][gain]
         if a is not None and D <= 2048:
             det.det_residual_rmsnorm_fwd(a, b, g, T, D, 1e-6, x, y, rstd, s_q, qy if s_q is not None else None)
             return
@@ -299,7 +311,7 @@ class Replay:
     def _norm_bwd(self, dy, x, gain, rstd, dx, tmp):
         """dx += gradient through the norm (rounded on its own first); the gain's gradient goes to its place."""
         T, D = self.cfg.tokens_per_microbatch, self.cfg.d_model
-        g, dg = self.p(gain), self.g(self.gmb, gain)
+        g, dg = self._views["pbf"][gain], self._views["gmb"][gain]
         if D <= 2048:
             det.det_rmsnorm_bwd_residual(dy, x, g, rstd, T, D, dx, dx, dg, self.ws)
             return
@@ -317,22 +329,24 @@ class Replay:
         cfg = self.cfg
         D, Fh, V, L, T = cfg.d_model, cfg.ffn, cfg.vocab, cfg.n_layers, cfg.tokens_per_microbatch
         B, H, S = cfg.micro_batch, cfg.n_heads, cfg.seq
+        views = self._fresh()
+        P, X = views["pbf"], views["sx"]
         self._set_tokens(self.tok, tokens_mb[:, :-1])
         self._set_tokens(self.lab, tokens_mb[:, 1:])
         Hkv, QW = cfg.kv_heads, cfg.qkv_width
         x = self.act[0]["x"] if L else self.xf
         if cfg.embed_norm:
-            det.det_embed_fwd(self.tok, T, self.p("embed"), V, D, self.x_emb)
-            det.det_rmsnorm_fwd(det.DET_BF16, self.x_emb, self.p("embed_norm"), T, D, 1e-6, x, self.rstd_emb)
+            det.det_embed_fwd(self.tok, T, P["embed"], V, D, self.x_emb)
+            det.det_rmsnorm_fwd(det.DET_BF16, self.x_emb, P["embed_norm"], T, D, 1e-6, x, self.rstd_emb)
         else:
-            det.det_embed_fwd(self.tok, T, self.p("embed"), V, D, x)
+            det.det_embed_fwd(self.tok, T, P["embed"], V, D, x)
         # outside the calibration pass every activation step is known before its activation is produced, so the
         # producers write the next linear's int8 input themselves (same bits as the separate quantiser pass)
         fuse = self.fuse_quant and not calibrate and D <= 2048
         dn, res = self.tmp[1][:T * D], None           # the residual sum that ends a layer runs with the norm that starts the next
         for l in range(L):
             a = self.act[l]
-            sxl = [self._view("sx", (l, i)) for i in range(4)] if fuse else None
+            sxl = [X[l, i] for i in range(4)] if fuse else None
             self._norm(res, dn, a["x"], "l%d.attn_norm" % l, a["n1"], a["rstd1"], sxl[0] if fuse else None, a["qx_qkv"])
             self._linear(l, "w_qkv", 0, a["n1"], T, a["qkv"], a["qx_qkv"], calibrate, fuse)
             qp = vp = a["qkv"].data_ptr()
@@ -369,39 +383,39 @@ class Replay:
         self._norm(res, dn, self.xf, "final_norm", self.nf, self.rstdf)
         with self.span("lmhead_fwd"):
             if cfg.arith == 2:
-                det.det_lmhead_fwd_v2(self.nf, self.p("lm_head"), T, V, D, self.logits, self.ws, self.status)
+                det.det_lmhead_fwd_v2(self.nf, P["lm_head"], T, V, D, self.logits, self.ws, self.status)
             else:
-                det.det_lmhead_fwd(self.nf, self.p("lm_head"), T, V, D, self.logits)
+                det.det_lmhead_fwd(self.nf, P["lm_head"], T, V, D, self.logits)
         with self.span("xent_fwd"):
             det.det_xent_fwd(self.logits, self.lab, T, V, cfg.z_weight, self.loss_row, self.lse_x, self.loss_mean,
                              self.z_mean, self.ws, self.status)
 
     def _linear_bwd(self, l, w, idx, dY, X, qx, M, dX):
         d = self.lin[(l, w)]
-        name = d["name"]
-        sx = self._view("sx", (l, idx))
-        ds = self.g(self.gmb, "l%d.s_x" % l)[idx:idx + 1]
+        P, G, name = self._views["pbf"], self._views["gmb"], d["name"]
         with self.span("linear_bwd"):
-            det.det_linear_bwd(dY, X, qx, self.p(name), d["qWt"], sx, d["s_w"], d["s_u"], M, d["N"], d["K"],
-                               self.cfg.hadamard_block, dX, self.g(self.gmb, name), ds, self.ws, self.status)
+            det.det_linear_bwd(dY, X, qx, P[name], d["qWt"], self._views["sx"][l, idx], d["s_w"], d["s_u"], M, d["N"], d["K"],
+                               self.cfg.hadamard_block, dX, G[name], G[l, idx], self.ws, self.status)
 
     def backward(self):
         cfg = self.cfg
         D, Fh, V, L, T = cfg.d_model, cfg.ffn, cfg.vocab, cfg.n_layers, cfg.tokens_per_microbatch
         B, H, S = cfg.micro_batch, cfg.n_heads, cfg.seq
+        views = self._fresh()
+        P, G = views["pbf"], views["gmb"]
         with self.span("xent_bwd"):
             det.det_xent_bwd(self.logits, self.lab, self.lse_x, T, V, cfg.z_weight, 1.0 / T)
         t0, t1, t2 = self.tmp
         d_nf = t0[:T * D]
         with self.span("lmhead_bwd"):
             if cfg.arith == 2:
-                det.det_lmhead_bwd_v2(self.logits, self.nf, self.p("lm_head"), T, V, D, d_nf, self.g(self.gmb, "lm_head"),
+                det.det_lmhead_bwd_v2(self.logits, self.nf, P["lm_head"], T, V, D, d_nf, G["lm_head"],
                                       self.ws, self.status)
             else:
-                det.det_lmhead_bwd(self.logits, self.nf, self.p("lm_head"), T, V, D, d_nf, self.g(self.gmb, "lm_head"), 1)
+                det.det_lmhead_bwd(self.logits, self.nf, P["lm_head"], T, V, D, d_nf, G["lm_head"], 1)
         dx = t1[:T * D]
-        det.det_rmsnorm_bwd(det.DET_BF16, d_nf, self.xf, self.p("final_norm"), self.rstdf, T, D, dx,
-                            self.g(self.gmb, "final_norm"), self.ws)
+        det.det_rmsnorm_bwd(det.DET_BF16, d_nf, self.xf, P["final_norm"], self.rstdf, T, D, dx,
+                            G["final_norm"], self.ws)
         for l in reversed(range(L)):
             a = self.act[l]
             d_a = t0[:T * Fh]
@@ -430,27 +444,32 @@ class Replay:
             self._norm_bwd(d_n1, a["x"], "l%d.attn_norm" % l, a["rstd1"], dx, t2[:T * D])     # and of x
         if cfg.embed_norm:
             d_emb = t0[:T * D]
-            det.det_rmsnorm_bwd(det.DET_BF16, dx, self.x_emb, self.p("embed_norm"), self.rstd_emb, T, D, d_emb,
-                                self.g(self.gmb, "embed_norm"), self.ws)
+            det.det_rmsnorm_bwd(det.DET_BF16, dx, self.x_emb, P["embed_norm"], self.rstd_emb, T, D, d_emb,
+                                G["embed_norm"], self.ws)
             dx = d_emb
-        det.det_embed_bwd(self.tok, T, dx, V, D, self.g(self.gmb, "embed"))
+        det.det_embed_bwd(self.tok, T, dx, V, D, G["embed"])
 
     def optimizer(self):
         cfg = self.cfg
-        views = [self.g(self.gout, name) for name, _, _ in self.specs]
-        det.det_grad_norm(views, cfg.clip, self.norm, self.coef, self.ws, self.status)
+        views, names = self._fresh(), [name for name, _, _ in self.specs]
+        part = lambda which: [views[which][name] for name in names]
+        grads = part("gout")
+        det.det_grad_norm(grads, cfg.clip, self.norm, self.coef, self.ws, self.status)
         descs, kinds = [], []
         for name, shape, kind in self.specs:
             decay = cfg.wd if (name == "lm_head" or name.split(".")[-1] in LINEARS) else 0.0
             descs.append(det.det_adamw_desc(cfg.lr, cfg.betas[0], cfg.betas[1], cfg.eps, decay, cfg.step))
             kinds.append(det.DET_BF16 if kind == "bf16" else det.DET_F32)
-        names = [name for name, _, _ in self.specs]
         # the clip coefficient is applied to the gradient in the same pass (every element of gout belongs to one tensor)
-        det.det_adamw_batch(descs, kinds, [self.p(x) for x in names], views, [self.g(self.m, x) for x in names],
-                            [self.g(self.v, x) for x in names], self.coef)
+        params = [views["sx" if kind == "f32" else "pbf"][name] for name, _, kind in self.specs]
+        det.det_adamw_batch(descs, kinds, params, grads, part("m"), part("v"), self.coef)
 
     def _hash_jobs(self, per_tensor):
-        jobs = [(name, self.p(name)) for name, _, _ in self.specs] if per_tensor else [("params_bf16", self.pbf), ("steps_f32", self.sx)]
+        if per_tensor:
+            views = self._fresh()
+            jobs = [(name, views["sx" if kind == "f32" else "pbf"][name]) for name, _, kind in self.specs]
+        else:
+            jobs = [("params_bf16", self.pbf), ("steps_f32", self.sx)]
         return jobs + [("grad", self.gout), ("adam_m", self.m), ("adam_v", self.v)]
 
     def _queue_hashes(self, per_tensor):
