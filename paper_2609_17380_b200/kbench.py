@@ -27,18 +27,16 @@ def flush_l2():
     _flush.zero_()
 
 
-SETTLE_S = 0.25   # a case behind one that drew the power limit starts at that one's lower clock for some 50 ms of work
+SETTLE_S = 0.25   # a case right behind one that drew the power limit starts at that one's lower clock
 
 
-def timeit(fn, iters, warm=2):
-    """Median of `iters` calls, after `warm` calls and, where more than one is timed, as many more as it takes the clock to settle."""
+def timeit(fn, iters, warm=3):
+    """Median of `iters` calls after `warm` calls, from a GPU that has been idle for long enough to have its clock back."""
+    torch.cuda.synchronize()
+    if iters > 1:
+        time.sleep(SETTLE_S)
     for _ in range(warm):
         fn()
-    torch.cuda.synchronize()
-    end = time.monotonic() + SETTLE_S
-    while iters > 1 and time.monotonic() < end:
-        fn()
-        torch.cuda.synchronize()
     ts = []
     for _ in range(iters):
         flush_l2()
@@ -270,7 +268,7 @@ def main():
     for name in names:
         fn, work, unit = cases[name](args.small)
         torch.cuda.synchronize()
-        ms = timeit(fn, args.iters, warm=1 if args.iters == 1 else 2)
+        ms = timeit(fn, args.iters, warm=1 if args.iters == 1 else 3)
         rate = work / (ms / 1e3)
         res[name] = {"ms": round(ms, 4), "rate": rate / 1e9 if unit == "B" else rate / 1e12,
                      "unit": "GB/s" if unit == "B" else ("TOP/s" if unit == "op" else "TFLOP/s")}
