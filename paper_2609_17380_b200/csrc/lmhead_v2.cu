@@ -11,7 +11,7 @@
 //   k_slice_rows   one warp (or CTA) per row: row exponent (integer maximum), then the two int8 slices
 //   k_igemm_sl     persistent, one CTA per SM, 128 x 128 output tile; warp 0 streams the FOUR operand tiles of a 128-deep
 //                  step (H hi, H lo, W hi, W lo: 64 KiB) through a three-stage TMA ring, warp 1 issues the sixteen MMAs of
-//                  the step into three TMEM accumulators (hh | hl + lh | ll, 128 columns each), warps 2-5 combine and round.
+//                  the step into three TMEM accumulators (hh | hl + lh | ll, 128 columns each), sixteen more combine and round.
 // Every mbarrier wait is bounded (DET_DEV_TIMEOUT), as in igemm.cu.
 #include "tc05.cuh"
 #include "internal.h"
@@ -315,7 +315,10 @@ __device__ __forceinline__ bool sl_tile(const SlArgs& p, int z, int row, int j0,
 // j0 <= i0 exist.  krange: 0 the whole contraction; 1 only the steps up to and including the row tile's own (a causal
 // product whose contracted index is the key); 2 only the steps from the row tile's own on (contracted index = query).
 // epi: SL_F32 | SL_BF16 | SL_BF16_ROWSCALE (the rounded result times rowscale[z*I + i] in binary32, then bf16).
-__global__ void __launch_bounds__(SL_THREADS, 1)
+// SPLIT > 1: a cluster of SPLIT CTAs computes ONE tile (krange 0, no causal filter): each takes a part of the steps, and the integers meet in
+// shared memory before the one rounding.
+template <int SPLIT>
+__global__ void __cluster_dims__(SPLIT, 1, 1) __launch_bounds__(SL_THREADS, 1)
     k_igemm_sl(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__ CUtensorMap tmAl,
                const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmBl, const SlArgs p, int* status) {
   const int I = p.I, J = p.J, K = p.K;
@@ -326,6 +329,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
   __shared__ int abort_s;
   volatile int* abort_flag = &abort_s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = SPLIT > 1 ? (int)cluster_ctarank() : 0;
   if (threadIdx.x == 0) {
     for (int s = 0; s < SL_STAGES; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&bar_empty[s], 1); }
     mbar_init(&bar_tfull, 1);
@@ -352,15 +356,17 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
     i0 = it * SL_T; j0 = jt * SL_T;
     k_lo = (p.krange == 2) ? it : 0;
     k_hi = (p.krange == 1) ? min(kblocks, it + 1) : kblocks;
+    if (SPLIT > 1) { k_lo = kblocks * rank / SPLIT; k_hi = kblocks * (rank + 1) / SPLIT; }
     return !(p.causal_tiles && jt > it);
   };
 
+  const int first_tile = (int)blockIdx.x / SPLIT, next_tile = (int)gridDim.x / SPLIT;
   if (warp == 0) {
     if (lane == 0) {
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+      for (int tile = first_tile; tile < num_tiles && ok; tile += next_tile) {
         int z, i0, j0, k_lo, k_hi;
         if (!tile_of(tile, z, i0, j0, k_lo, k_hi)) continue;
         for (int kb = k_lo; kb < k_hi; ++kb) {
@@ -382,7 +388,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
       int stage = 0, it = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+      for (int tile = first_tile; tile < num_tiles && ok; tile += next_tile) {
         int z, i0, j0, k_lo, k_hi;
         if (!tile_of(tile, z, i0, j0, k_lo, k_hi)) continue;
         if (!mbar_wait(&bar_tempty, ((uint32_t)it & 1u) ^ 1u, abort_flag, status)) { ok = false; break; }   // accumulators drained
@@ -415,7 +421,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
     int it = 0;
     bool ok = true;
     const uint32_t tcols = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(part * 32);
-    // the totals of 16 of this warp's columns
+    // the totals of 16 of this warp's columns, of this CTA's part of the contraction
     auto totals = [&](int sub, long long (&T)[16]) {
       uint32_t hh[16], cr[16], ll[16];
       tmem_ld16_nowait(tcols + (uint32_t)(sub * 16), hh);
@@ -425,13 +431,50 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
 #pragma unroll
       for (int c = 0; c < 16; ++c) T[c] = sl_total(hh[c], cr[c], ll[c]);
     };
-    for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+    // SPLIT: CTA r of the cluster finishes the columns r * 128 / SPLIT .. and gets the others' totals of them into its ring, which is free once
+    // every CTA's MMAs are done: [sender][column of its share][row]
+    const int owner = part * SPLIT / 4;
+    constexpr int SHARE = SL_T / SPLIT;
+    const uint32_t xrow = (uint32_t)((part * 32 - owner * SHARE) * SL_T + q * 32 + lane) * 8u;
+    if (SPLIT > 1) {
+      ok = __all_sync(0xffffffffu, mbar_wait(&bar_tfull, 0u, abort_flag, status));
+      tc_fence_after();
+      cluster_sync_all();
+      if (ok && owner != rank) {
+        const uint32_t dst = mapa_u32(smem_u32(smem), (uint32_t)owner) + (uint32_t)((rank - (rank > owner ? 1 : 0)) * SHARE * SL_T) * 8u + xrow;
+#pragma unroll 1
+        for (int sub = 0; sub < 2; ++sub) {
+          long long T[16];
+          totals(sub, T);
+#pragma unroll
+          for (int c = 0; c < 16; ++c)
+            asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(dst + (uint32_t)((sub * 16 + c) * SL_T) * 8u), "l"(T[c]) : "memory");
+        }
+      }
+      cluster_sync_all();
+      ok = ok && owner == rank;
+    }
+    for (int tile = first_tile; tile < num_tiles && ok; tile += next_tile) {
       int z, i0, j0, k_lo, k_hi;
       if (!tile_of(tile, z, i0, j0, k_lo, k_hi)) continue;
       ok = sl_tile<16>(p, z, i0 + q * 32 + lane, j0, part, stage, [&]() { return mbar_wait(&bar_tfull, (uint32_t)it & 1u, abort_flag, status); },
-                       [&](int c0, long long (&T)[16]) { totals(c0 / 16, T); }, [&]() { mbar_arrive(&bar_tempty); });
+                       [&](int c0, long long (&T)[16]) {
+        totals(c0 / 16, T);
+        if (SPLIT > 1) {
+#pragma unroll
+          for (int src = 0; src < SPLIT - 1; ++src)
+#pragma unroll
+            for (int c = 0; c < 16; ++c)
+              T[c] += *reinterpret_cast<const long long*>(smem + (size_t)(src * SHARE + c0 + c) * SL_T * 8 + xrow);
+        }
+      }, [&]() { mbar_arrive(&bar_tempty); });
       ++it;
     }
+  }
+  if (SPLIT > 1 && warp < 2) {   // the two meetings of the cluster, with the epilogue warps
+    __syncwarp();
+    cluster_sync_all();
+    cluster_sync_all();
   }
   __syncthreads();
   if (abort_s) {
@@ -445,6 +488,146 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
   }
 }
 
+// CTA pairs (cta_group::2): a pair computes 256 x 128 results.  CTA r stages its own 128 rows of both slices of A and ONE slice of the
+// 128 rows of B, the high one in CTA 0, the low one in CTA 1: side by side they are the 256 columns of one MMA, so that A hi times
+// both is hh | hl and A lo times both lh | ll, two MMAs of 256 x 256 where a single CTA issues four of 128 x 128.  A CTA reads 48
+// instead of 64 KiB per 128-deep step, and what all SMs together read from L2 is what bounds the single CTAs (some 10 TB/s; 8192 x 50304 x
+// 2048: 2.43 -> 2.28 ms).  The four accumulators fill TMEM; hl and lh are added in the epilogue.
+constexpr int SLP_STAGES = 4, SLP_STAGE_BYTES = 3 * SL_TILE;
+static_assert(SLP_STAGES * SLP_STAGE_BYTES == SL_STAGES * SL_STAGE_BYTES, "the pair's ring is as large as the single CTA's");
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SL_THREADS, 1)
+    k_igemm_sl_pair(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__ CUtensorMap tmAl,
+                    const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmBl, const SlArgs p, int* status) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  __shared__ __align__(8) uint64_t bar_full[SLP_STAGES], bar_empty[SLP_STAGES], bar_tfull, bar_tempty;
+  __shared__ uint32_t tmem_base_s;
+  __shared__ int abort_s;
+  volatile int* abort_flag = &abort_s;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = (int)cluster_ctarank();
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < SLP_STAGES; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&bar_empty[s], 1); }
+    mbar_init(&bar_tfull, 1);
+    mbar_init(&bar_tempty, 2 * SL_EPI_WARPS);
+    abort_s = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();   // the peer's barriers are initialised before anything can signal them
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_base_s;
+  grid_wait();
+  const int tiles_i = p.I / (2 * SL_T), per_z = tiles_i * (p.J / SL_T), num_tiles = p.Z * per_z, kblocks = p.K / SL_BK;
+  const int first = (int)blockIdx.x >> 1, step = (int)gridDim.x >> 1;
+  auto tile_of = [&](int t, int& z, int& i0, int& j0) {
+    z = t / per_z;
+    const int r = t - z * per_z;
+    i0 = (r % tiles_i) * (2 * SL_T); j0 = (r / tiles_i) * SL_T;
+  };
+  if (warp == 0) {
+    if (lane == 0) {
+      int stage = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      const CUtensorMap* tmB = rank ? &tmBl : &tmBh;
+      for (int tile = first; tile < num_tiles && ok; tile += step) {
+        int z, i0, j0;
+        tile_of(tile, z, i0, j0);
+        const int arow = z * p.I + i0 + rank * SL_T, brow = z * p.J + j0;
+        for (int kb = 0; kb < kblocks; ++kb) {
+          if (!mbar_wait(&bar_empty[stage], phase ^ 1u, abort_flag, status)) { ok = false; break; }
+          if (rank == 0) mbar_expect_tx(&bar_full[stage], 2 * SLP_STAGE_BYTES);   // both CTAs' tiles complete on this barrier
+          uint8_t* sa = smem + stage * SLP_STAGE_BYTES;
+          tma_load_2d_pair(sa, &tmAh, kb * SL_BK, arow, &bar_full[stage]);
+          tma_load_2d_pair(sa + SL_TILE, &tmAl, kb * SL_BK, arow, &bar_full[stage]);
+          tma_load_2d_pair(sa + 2 * SL_TILE, tmB, kb * SL_BK, brow, &bar_full[stage]);
+          if (++stage == SLP_STAGES) { stage = 0; phase ^= 1u; }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0 && rank == 0) {
+      // instruction descriptor: D = S32, A = B = signed 8-bit, both K-major, N = 256, M = 256 (two CTAs x 128)
+      constexpr uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+      int stage = 0, it = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      for (int tile = first; tile < num_tiles && ok; tile += step, ++it) {
+        if (!mbar_wait(&bar_tempty, ((uint32_t)it & 1u) ^ 1u, abort_flag, status)) { ok = false; break; }   // accumulators drained
+        tc_fence_after();
+        for (int kb = 0; kb < kblocks; ++kb) {
+          if (!mbar_wait(&bar_full[stage], phase, abort_flag, status)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t sa = smem_u32(smem + stage * SLP_STAGE_BYTES);
+          const uint64_t ah = make_smem_desc(sa), al = make_smem_desc(sa + SL_TILE), b = make_smem_desc(sa + 2 * SL_TILE);
+#pragma unroll
+          for (int k4 = 0; k4 < SL_BK / 32; ++k4) {
+            const uint64_t o = (uint64_t)(k4 * 2);
+            const uint32_t more = (kb || k4) ? 1u : 0u;
+            umma_i8_pair(tmem_base, ah + o, b + o, idesc, more);            // hh | hl
+            umma_i8_pair(tmem_base + 256u, al + o, b + o, idesc, more);     // lh | ll
+          }
+          umma_commit_pair(&bar_empty[stage]);
+          if (++stage == SLP_STAGES) { stage = 0; phase ^= 1u; }
+        }
+        if (ok) umma_commit_pair(&bar_tfull);
+      }
+    }
+  } else {
+    const int q = warp & 3, part = (warp - 2) >> 2;  // TMEM lane quarter this warp may read; its 32 of the 128 columns
+    uint8_t* stage = smem + SLP_STAGES * SLP_STAGE_BYTES + (warp - 2) * 2048;
+    const uint32_t tcols = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(part * 32), tempty = mapa_u32(smem_u32(&bar_tempty), 0);
+    int it = 0;
+    for (int tile = first; tile < num_tiles; tile += step, ++it) {
+      int z, i0, j0;
+      tile_of(tile, z, i0, j0);
+      if (!sl_tile<8>(p, z, i0 + rank * SL_T + q * 32 + lane, j0, part, stage, [&]() { return mbar_wait(&bar_tfull, (uint32_t)it & 1u, abort_flag, status); },
+                      [&](int c0, long long (&T)[8]) {
+        uint32_t hh[8], hl[8], lh[8], ll[8];
+        tmem_ld8_nowait(tcols + (uint32_t)c0, hh);
+        tmem_ld8_nowait(tcols + 128u + (uint32_t)c0, hl);
+        tmem_ld8_nowait(tcols + 256u + (uint32_t)c0, lh);
+        tmem_ld8_nowait(tcols + 384u + (uint32_t)c0, ll);
+        tmem_wait_ld();
+#pragma unroll
+        for (int c = 0; c < 8; ++c) T[c] = sl_total(hh[c], hl[c] + lh[c], ll[c]);
+      }, [&]() { mbar_arrive_remote(tempty); })) break;
+    }
+  }
+  // both CTAs meet before either leaves (the peer may still signal this CTA's barriers or read its tiles)
+  __syncthreads();
+  if (abort_s) {
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000ll) { }
+  }
+  cluster_sync_all();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+  }
+}
+
+template <class Kern>
+static int sl_go(Kern kern, DevOnce& once, long long ctas, const CUtensorMap& tAh, const CUtensorMap& tAl, const CUtensorMap& tBh,
+                 const CUtensorMap& tBl, const SlArgs& p, int* status, cudaStream_t st) {
+  if (dev_ensure_smem(once, (const void*)kern, SL_SMEM) != DET_OK) return DET_ERR_CUDA;
+  launch_after(kern, (unsigned)ctas, SL_THREADS, SL_SMEM, st, tAh, tAl, tBh, tBl, p, status);
+  if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return DET_ERR_CUDA; }
+  return DET_OK;
+}
+
 // host: Z sliced contractions in one launch (see k_igemm_sl); the slices of problem z are rows z*I.. / z*J.. of A / B
 int sliced_gemm_launch(const int8_t* Ah, const int8_t* Al, const int8_t* Bh, const int8_t* Bl, const SlArgs& p, int* status,
                        cudaStream_t st) {
@@ -454,14 +637,22 @@ int sliced_gemm_launch(const int8_t* Ah, const int8_t* Al, const int8_t* Bh, con
   if (!make_map(&tAh, Ah, p.Z * p.I, p.K, SL_T) || !make_map(&tAl, Al, p.Z * p.I, p.K, SL_T) ||
       !make_map(&tBh, Bh, p.Z * p.J, p.K, SL_T) || !make_map(&tBl, Bl, p.Z * p.J, p.K, SL_T))
     return DET_ERR_CUDA;
-  static DevOnce once = {};
-  if (dev_ensure_smem(once, (const void*)k_igemm_sl, SL_SMEM) != DET_OK) return DET_ERR_CUDA;
-  const int sms = dev_sm_count();
+  static DevOnce once[4] = {};
+  const int sms = dev_sm_count(), steps = p.K / SL_BK;
   if (sms <= 0) return DET_ERR_CUDA;
   const long long tiles = (long long)p.Z * (p.I / SL_T) * (p.J / SL_T);
-  launch_after(k_igemm_sl, (unsigned)(tiles < sms ? tiles : sms), SL_THREADS, SL_SMEM, st, tAh, tAl, tBh, tBl, p, status);
-  if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return DET_ERR_CUDA; }
-  return DET_OK;
+  const bool whole = !p.krange && !p.causal_tiles;      // every tile takes every step
+  // Few tiles with a long contraction (a token gradient of 1024 x 1024 has 64 tiles of 256 steps) leave SMs idle: two or four CTAs share a
+  // tile (1024 x 1024 x 32768: 0.170 -> 0.114 ms).  A part is at least eight steps (the exchange costs about four); clusters of four find room
+  // on some seven eighths of the SMs.
+  if (whole && tiles * 4 <= sms - sms / 8 && steps >= 32) return sl_go(k_igemm_sl<4>, once[0], tiles * 4, tAh, tAl, tBh, tBl, p, status, st);
+  if (whole && tiles * 2 <= sms && steps >= 16) return sl_go(k_igemm_sl<2>, once[1], tiles * 2, tAh, tAl, tBh, tBl, p, status, st);
+  // pairs wherever their tile fits (causal and row-tied problems are written for tiles of 128 rows)
+  if (whole && p.I % (2 * SL_T) == 0 && sms >= 2) {
+    const long long pairs = tiles / 2 < sms / 2 ? tiles / 2 : sms / 2;
+    return sl_go(k_igemm_sl_pair, once[2], 2 * pairs, tAh, tAl, tBh, tBl, p, status, st);
+  }
+  return sl_go(k_igemm_sl<1>, once[3], tiles < sms ? tiles : sms, tAh, tAl, tBh, tBl, p, status, st);
 }
 
 }  // namespace det

@@ -114,6 +114,26 @@ def test_lmhead_v2_long_rows(det, M, V, K):
     assert_same_bits(got_W[:-1], want_W[:-1], "version-2 dW")
 
 
+# version-2 contraction where the CTAs that share a tile change (16 and 32 steps, 32 and 74 tiles), CTA pairs with one round and several,
+# and operands whose exponents cross the range in which every result is a normal number, in both directions
+@pytest.mark.parametrize("M,V,K,spread", [(128, 128, 1920, False), (128, 128, 2048, False), (256, 128, 4096, True), (128, 4224, 4096, False),
+                                          (128, 9600, 2048, False), (256, 384, 256, True), (256, 20480, 128, False), (768, 6912, 384, True)])
+def test_lmhead_v2_shared_tiles(det, M, V, K, spread):
+    import torch
+    from oracle import v2
+    H, W = synth.normal_bf16((M, K), 1.0, seed=V + K, tid=1), synth.normal_bf16((V, K), 0.05, seed=V + K, tid=2)
+    if spread:                                                    # rows of H from 2^-70 to 2^70 times, blocks of W by 2^60 either way
+        h = synth.from_bf16(H) * np.exp2(np.linspace(-70, 70, M).round())[:, None]
+        w = synth.from_bf16(W) * np.exp2(60.0 * ((np.arange(V) // 64) % 3 - 1))[:, None]
+        H, W = synth.to_bf16(h.astype(F)), synth.to_bf16(w.astype(F))
+    lg = empty((M, V), F)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    det.det_lmhead_fwd_v2(dev(H), dev(W), M, V, K, lg, ws(det.det_lmhead_fwd_v2_ws_bytes(M, V, K)), status)
+    _sync()
+    assert int(status.item()) == 0
+    assert_same_bits(host(lg), v2.lmhead_fwd(H, W), "version-2 logits")
+
+
 # attention at head and row counts where the rows per CTA change (32, 64, 128 rows), S off the 128 grid, windows that start
 # and end inside a block, grouped heads (one accumulator over the whole group)
 @pytest.mark.parametrize("B,H,Hkv,S,W", [(1, 2, 2, 576, 0), (1, 40, 40, 320, 0), (2, 80, 80, 192, 0), (1, 3, 3, 704, 256),
