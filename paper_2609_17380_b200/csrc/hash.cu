@@ -173,8 +173,10 @@ __global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJ
 
 // Few chunks: eight chains per CTA, four lanes each.  Only the 64 rounds of a block depend on the block before, so the four lanes
 // of a chain expand the schedules of its next four blocks side by side (schedule word + round constant, through shared memory)
-// and the chain itself is rounds alone: 14 instructions a round on the half-rate integer pipe instead of 22, ordered so that a and
-// e depend on the round before through one rotation, one exclusive or and one addition each.  While there are schedulers to
+// and the chain itself is rounds alone: 12 instructions a round on the half-rate integer pipe instead of 22, ordered so that a and
+// e depend on the round before through one rotation, one exclusive or and one addition each.  A warp alone on its scheduler is bound by
+// that pipe, two cycles an instruction, so the additions that nothing waits for (schedule word + h + d, maj - d) go to the
+// multiply-add pipe: all levels of 1 MiB 151.3 -> 146.1 us, one chunk 84.9 -> 82.6 (all additions there: slower, by their latency).  While there are schedulers to
 // spare a second warp does the expanding, double-buffered.  65 blocks: 0.137 ms with a thread per chunk, 0.089 with
 // one warp per CTA, 0.076 with two; with the padding a word at a time 0.118, 0.077 and 0.066.
 constexpr int SF_CH = 8, SF_PITCH = 68;
@@ -226,6 +228,7 @@ __global__ void __launch_bounds__(64) k_sha_few(const __grid_constant__ HashJobs
       *reinterpret_cast<uint4*>(row + i) = make_uint4(t[0], t[1], t[2], t[3]);
     }
   };
+  const uint32_t one = opaque_one(), minus_one = 0u - one;
   uint32_t h[8];
   sha_init(h);
   // a pair: the expanding warp is four blocks ahead; a single warp does one after the other
@@ -247,9 +250,9 @@ __global__ void __launch_bounds__(64) k_sha_few(const __grid_constant__ HashJobs
             const uint32_t wk[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              const uint32_t dx = wk[k] + hh + d;
+              const uint32_t dx = add_mad<true>(add_mad<true>(wk[k], hh, one), d, one);
               const uint32_t en = big_s1(e) + sha_ch(e, f, g) + dx;
-              const uint32_t an = big_s0(a) + sha_maj(a, b, cc) + (en - d);
+              const uint32_t an = big_s0(a) + add_mad<true>(d, sha_maj(a, b, cc), minus_one) + en;
               hh = g; g = f; f = e; e = en; d = cc; cc = b; b = a; a = an;
             }
           }
