@@ -68,6 +68,32 @@ _SIGNATURES = {
     "det_test_wait_timeout": "iplp",
 }
 
+# The entry points that csrc/binding.cpp calls directly: what it makes of each Python argument (letters as above; w: a workspace tensor or None,
+# passed as address and size; s: the current stream, no argument of its own).
+_PATTERNS = {
+    "det_sum": "pzipws", "det_sum_static": "pzips", "det_scale_inplace": "pzps", "det_lsq_weight_scale": "piiipws",
+    "det_lsq_act_scale_init": "pzpws", "det_lsq_quantize_weight": "ppiiipppws", "det_linear_fwd": "ppppiiippsp",
+    "det_linear_fwd_q": "ppppiiipsp", "det_linear_bwd": "ppppppppiiiipppwsp", "det_rmsnorm_fwd": "ippiifpps",
+    "det_rmsnorm_fwd_q": "ppiifpppps", "det_residual_rmsnorm_fwd": "pppiifppppps", "det_headnorm_fwd": "piiifpips",
+    "det_headnorm_bwd": "pipipiipis", "det_rope": "piiiippipis", "det_rmsnorm_bwd": "ippppiippws",
+    "det_rmsnorm_bwd_residual": "ppppiipppws", "det_xent_fwd": "ppiifppppwsp", "det_xent_bwd": "pppiiffs", "det_attn_fwd": "pppiiiiiipips",
+    "det_attn_fwd_q": "pppiiiiiipippps", "det_attn_fwd_int8pv": "pppiiiiiipipsp", "det_attn_bwd": "ppppppiiiiiiipppiws",
+    "det_attn_bwd_fixq": "ppppppiiiiiiipppiws", "det_swiglu_fwd": "piips", "det_swiglu_fwd_q": "piippps", "det_swiglu_bwd": "ppiips",
+    "det_residual_add": "ppzps", "det_embed_fwd": "pipiips", "det_embed_bwd": "pipiips", "det_lmhead_fwd": "ppiiips",
+    "det_lmhead_fwd_v2": "ppiiipwsp", "det_lmhead_bwd": "pppiiippis", "det_lmhead_bwd_v2": "pppiiippwsp",
+    "det_attn_fwd_v2": "pppiiiipipwsp", "det_tensor_hash_async": "pzpws",
+}
+
+
+class _Calls:
+    """The callables by name, there once the library is loaded."""
+
+    def __getattr__(self, name):
+        load()
+        return self.__dict__[name]
+
+
+_c = _Calls()
 _lib = None
 
 
@@ -85,6 +111,7 @@ def load():
             fn.argtypes = [_CTYPES[c] for c in sig[1:]]
         from . import _binding
         _ptr, _stream = _binding.ptr, _binding.stream
+        _c.__dict__.update(_binding.bind(_SO, _PATTERNS, _check))
         _lib = lib
     return _lib
 
@@ -127,7 +154,7 @@ def det_sum_ws_bytes(n):
 
 
 def det_sum(x, n, squares, out, ws):
-    _check("det_sum", load().det_sum(_ptr(x), n, squares, _ptr(out), *_ws(ws), _stream()))
+    _c.det_sum(x, n, squares, out, ws)
 
 
 def det_sum_static_max_n():
@@ -136,7 +163,7 @@ def det_sum_static_max_n():
 
 def det_sum_static(x, n, squares, out):
     """det_sum without a workspace argument: scratch lives in a fixed array inside the library (see det.h)."""
-    _check("det_sum_static", load().det_sum_static(_ptr(x), n, squares, _ptr(out), _stream()))
+    _c.det_sum_static(x, n, squares, out)
 
 
 def _tensor_table(tensors):
@@ -157,7 +184,7 @@ def det_grad_norm(tensors, max_norm, norm_out, coef_out, ws, status_dev=None):
 
 
 def det_scale_inplace(g, n, coef_dev):
-    _check("det_scale_inplace", load().det_scale_inplace(_ptr(g), n, _ptr(coef_dev), _stream()))
+    _c.det_scale_inplace(g, n, coef_dev)
 
 
 # ---- LSQ int8 linear -------------------------------------------------------------------------------------
@@ -166,8 +193,7 @@ def det_lsq_weight_scale_ws_bytes(N, K):
 
 
 def det_lsq_weight_scale(W, N, K, per_tensor, s_w, ws):
-    _check("det_lsq_weight_scale", load().det_lsq_weight_scale(_ptr(W), N, K, per_tensor,
-                                                               _ptr(s_w), *_ws(ws), _stream()))
+    _c.det_lsq_weight_scale(W, N, K, per_tensor, s_w, ws)
 
 
 def det_lsq_act_scale_init_ws_bytes(n):
@@ -175,7 +201,7 @@ def det_lsq_act_scale_init_ws_bytes(n):
 
 
 def det_lsq_act_scale_init(X, n, s_x, ws):
-    _check("det_lsq_act_scale_init", load().det_lsq_act_scale_init(_ptr(X), n, _ptr(s_x), *_ws(ws), _stream()))
+    _c.det_lsq_act_scale_init(X, n, s_x, ws)
 
 
 def det_lsq_quantize_weight_ws_bytes(N, K):
@@ -183,19 +209,15 @@ def det_lsq_quantize_weight_ws_bytes(N, K):
 
 
 def det_lsq_quantize_weight(W, s_w, N, K, hadamard_block, qW, qWt_bwd, s_u, ws):
-    _check("det_lsq_quantize_weight", load().det_lsq_quantize_weight(
-        _ptr(W), _ptr(s_w), N, K, hadamard_block, _ptr(qW), _ptr(qWt_bwd), _ptr(s_u), *_ws(ws),
-        _stream()))
+    _c.det_lsq_quantize_weight(W, s_w, N, K, hadamard_block, qW, qWt_bwd, s_u, ws)
 
 
 def det_linear_fwd(X, qW, s_x, s_w, M, N, K, Y, qX_save, status_dev=None):
-    _check("det_linear_fwd", load().det_linear_fwd(_ptr(X), _ptr(qW), _ptr(s_x), _ptr(s_w), M, N,
-                                                   K, _ptr(Y), _ptr(qX_save), _stream(), _ptr(status_dev)))
+    _c.det_linear_fwd(X, qW, s_x, s_w, M, N, K, Y, qX_save, status_dev)
 
 
 def det_linear_fwd_q(qX, qW, s_x, s_w, M, N, K, Y, status_dev=None):
-    _check("det_linear_fwd_q", load().det_linear_fwd_q(_ptr(qX), _ptr(qW), _ptr(s_x), _ptr(s_w), M, N,
-                                                       K, _ptr(Y), _stream(), _ptr(status_dev)))
+    _c.det_linear_fwd_q(qX, qW, s_x, s_w, M, N, K, Y, status_dev)
 
 
 def det_linear_bwd_ws_bytes(M, N, K):
@@ -203,9 +225,7 @@ def det_linear_bwd_ws_bytes(M, N, K):
 
 
 def det_linear_bwd(dY, X, qX, W, qWt_bwd, s_x, s_w, s_u, M, N, K, hadamard_block, dX, dW, ds_x, ws, status_dev=None):
-    _check("det_linear_bwd", load().det_linear_bwd(
-        _ptr(dY), _ptr(X), _ptr(qX), _ptr(W), _ptr(qWt_bwd), _ptr(s_x), _ptr(s_w), _ptr(s_u), M, N,
-        K, hadamard_block, _ptr(dX), _ptr(dW), _ptr(ds_x), *_ws(ws), _stream(), _ptr(status_dev)))
+    _c.det_linear_bwd(dY, X, qX, W, qWt_bwd, s_x, s_w, s_u, M, N, K, hadamard_block, dX, dW, ds_x, ws, status_dev)
 
 
 def det_test_wait_timeout(status_dev, limit_cycles):
@@ -219,33 +239,27 @@ def det_test_igemm_tn(A, B, I, J, K, Cout, force_one_cta=0, status_dev=None):
 
 # ---- RMSNorm, cross-entropy ---------------------------------------------------------------------------------
 def det_rmsnorm_fwd(io, x, gamma, rows, D, eps, y, rstd):
-    _check("det_rmsnorm_fwd", load().det_rmsnorm_fwd(io, _ptr(x), _ptr(gamma), rows, D,
-                                                     eps, _ptr(y), _ptr(rstd), _stream()))
+    _c.det_rmsnorm_fwd(io, x, gamma, rows, D, eps, y, rstd)
 
 
 def det_rmsnorm_fwd_q(x, gamma, rows, D, eps, y, rstd, s_q, qy):
-    _check("det_rmsnorm_fwd_q", load().det_rmsnorm_fwd_q(_ptr(x), _ptr(gamma), rows, D, eps,
-                                                         _ptr(y), _ptr(rstd), _ptr(s_q), _ptr(qy), _stream()))
+    _c.det_rmsnorm_fwd_q(x, gamma, rows, D, eps, y, rstd, s_q, qy)
 
 
 def det_residual_rmsnorm_fwd(a, b, gamma, rows, D, eps, sum_out, y, rstd, s_q=None, qy=None):
-    _check("det_residual_rmsnorm_fwd", load().det_residual_rmsnorm_fwd(_ptr(a), _ptr(b), _ptr(gamma), rows, D, eps, _ptr(sum_out), _ptr(y),
-                                                                       _ptr(rstd), _ptr(s_q), _ptr(qy), _stream()))
+    _c.det_residual_rmsnorm_fwd(a, b, gamma, rows, D, eps, sum_out, y, rstd, s_q, qy)
 
 
 def det_headnorm_fwd(x, ld, T, nh, eps, y, ld_y, rstd):
-    _check("det_headnorm_fwd", load().det_headnorm_fwd(_ptr(x), ld, T, nh, eps, _ptr(y),
-                                                       ld_y, _ptr(rstd), _stream()))
+    _c.det_headnorm_fwd(x, ld, T, nh, eps, y, ld_y, rstd)
 
 
 def det_headnorm_bwd(dy, ld_dy, x, ld, rstd, T, nh, dx, ld_dx):
-    _check("det_headnorm_bwd", load().det_headnorm_bwd(_ptr(dy), ld_dy, _ptr(x), ld, _ptr(rstd), T,
-                                                       nh, _ptr(dx), ld_dx, _stream()))
+    _c.det_headnorm_bwd(dy, ld_dy, x, ld, rstd, T, nh, dx, ld_dx)
 
 
 def det_rope(x, ld, T, nh, S, cos_tab, sin_tab, inverse, y, ld_y):
-    _check("det_rope", load().det_rope(_ptr(x), ld, T, nh, S, _ptr(cos_tab), _ptr(sin_tab),
-                                       int(inverse), _ptr(y), ld_y, _stream()))
+    _c.det_rope(x, ld, T, nh, S, cos_tab, sin_tab, int(inverse), y, ld_y)
 
 
 def det_rmsnorm_bwd_ws_bytes(rows, D):
@@ -253,13 +267,11 @@ def det_rmsnorm_bwd_ws_bytes(rows, D):
 
 
 def det_rmsnorm_bwd(io, dy, x, gamma, rstd, rows, D, dx, dgamma, ws):
-    _check("det_rmsnorm_bwd", load().det_rmsnorm_bwd(io, _ptr(dy), _ptr(x), _ptr(gamma), _ptr(rstd), rows,
-                                                     D, _ptr(dx), _ptr(dgamma), *_ws(ws), _stream()))
+    _c.det_rmsnorm_bwd(io, dy, x, gamma, rstd, rows, D, dx, dgamma, ws)
 
 
 def det_rmsnorm_bwd_residual(dy, x, gamma, rstd, rows, D, res, dx, dgamma, ws):
-    _check("det_rmsnorm_bwd_residual", load().det_rmsnorm_bwd_residual(_ptr(dy), _ptr(x), _ptr(gamma), _ptr(rstd), rows, D, _ptr(res),
-                                                                       _ptr(dx), _ptr(dgamma), *_ws(ws), _stream()))
+    _c.det_rmsnorm_bwd_residual(dy, x, gamma, rstd, rows, D, res, dx, dgamma, ws)
 
 
 def det_xent_ws_bytes(rows, V):
@@ -267,33 +279,24 @@ def det_xent_ws_bytes(rows, V):
 
 
 def det_xent_fwd(logits, target, rows, V, z_weight, loss_row, lse, loss_mean, z_mean, ws, status_dev=None):
-    _check("det_xent_fwd", load().det_xent_fwd(_ptr(logits), _ptr(target), rows, V, z_weight,
-                                               _ptr(loss_row), _ptr(lse), _ptr(loss_mean), _ptr(z_mean), *_ws(ws), _stream(),
-                                               _ptr(status_dev)))
+    _c.det_xent_fwd(logits, target, rows, V, z_weight, loss_row, lse, loss_mean, z_mean, ws, status_dev)
 
 
 def det_xent_bwd(logits_inout, target, lse, rows, V, z_weight, scale):
-    _check("det_xent_bwd", load().det_xent_bwd(_ptr(logits_inout), _ptr(target), _ptr(lse), rows, V,
-                                               z_weight, scale, _stream()))
+    _c.det_xent_bwd(logits_inout, target, lse, rows, V, z_weight, scale)
 
 
 # ---- attention ------------------------------------------------------------------------------------------------
 def det_attn_fwd(q, k, v, ld, B, H, S, out, ld_out, lse, Hkv=None, window=0):
-    _check("det_attn_fwd", load().det_attn_fwd(_ptr(q), _ptr(k), _ptr(v), ld, B, H,
-                                               H if Hkv is None else Hkv, S, window, _ptr(out),
-                                               ld_out, _ptr(lse), _stream()))
+    _c.det_attn_fwd(q, k, v, ld, B, H, H if Hkv is None else Hkv, S, window, out, ld_out, lse)
 
 
 def det_attn_fwd_q(q, k, v, ld, B, H, S, out, ld_out, lse, s_q, qout, Hkv=None, window=0):
-    _check("det_attn_fwd_q", load().det_attn_fwd_q(_ptr(q), _ptr(k), _ptr(v), ld, B, H,
-                                                   H if Hkv is None else Hkv, S, window, _ptr(out),
-                                                   ld_out, _ptr(lse), _ptr(s_q), _ptr(qout), _stream()))
+    _c.det_attn_fwd_q(q, k, v, ld, B, H, H if Hkv is None else Hkv, S, window, out, ld_out, lse, s_q, qout)
 
 
 def det_attn_fwd_int8pv(q, k, v, ld, B, H, S, out, ld_out, lse, status_dev=None, Hkv=None, window=0):
-    _check("det_attn_fwd_int8pv", load().det_attn_fwd_int8pv(_ptr(q), _ptr(k), _ptr(v), ld, B, H,
-                                                             H if Hkv is None else Hkv, S, window,
-                                                             _ptr(out), ld_out, _ptr(lse), _stream(), _ptr(status_dev)))
+    _c.det_attn_fwd_int8pv(q, k, v, ld, B, H, H if Hkv is None else Hkv, S, window, out, ld_out, lse, status_dev)
 
 
 def det_attn_bwd_ws_bytes(B, H, S, Hkv=None):
@@ -301,10 +304,7 @@ def det_attn_bwd_ws_bytes(B, H, S, Hkv=None):
 
 
 def det_attn_bwd(dout, q, k, v, out, lse, ld, ld_out, B, H, S, dq, dk, dv, ld_d, ws, Hkv=None, window=0):
-    _check("det_attn_bwd", load().det_attn_bwd(_ptr(dout), _ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), ld,
-                                               ld_out, B, H, H if Hkv is None else Hkv,
-                                               S, window, _ptr(dq), _ptr(dk), _ptr(dv), ld_d,
-                                               *_ws(ws), _stream()))
+    _c.det_attn_bwd(dout, q, k, v, out, lse, ld, ld_out, B, H, H if Hkv is None else Hkv, S, window, dq, dk, dv, ld_d, ws)
 
 
 def det_attn_bwd_fixq_ws_bytes(B, H, S, Hkv=None):
@@ -312,39 +312,36 @@ def det_attn_bwd_fixq_ws_bytes(B, H, S, Hkv=None):
 
 
 def det_attn_bwd_fixq(dout, q, k, v, out, lse, ld, ld_out, B, H, S, dq, dk, dv, ld_d, ws, Hkv=None, window=0):
-    _check("det_attn_bwd_fixq", load().det_attn_bwd_fixq(_ptr(dout), _ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse),
-                                                         ld, ld_out, B, H,
-                                                         H if Hkv is None else Hkv, S, window,
-                                                         _ptr(dq), _ptr(dk), _ptr(dv), ld_d, *_ws(ws), _stream()))
+    _c.det_attn_bwd_fixq(dout, q, k, v, out, lse, ld, ld_out, B, H, H if Hkv is None else Hkv, S, window, dq, dk, dv, ld_d, ws)
 
 
 # ---- glue --------------------------------------------------------------------------------------------------------
 def det_swiglu_fwd(gu, rows, F, h):
-    _check("det_swiglu_fwd", load().det_swiglu_fwd(_ptr(gu), rows, F, _ptr(h), _stream()))
+    _c.det_swiglu_fwd(gu, rows, F, h)
 
 
 def det_swiglu_fwd_q(gu, rows, F, h, s_q, qh):
-    _check("det_swiglu_fwd_q", load().det_swiglu_fwd_q(_ptr(gu), rows, F, _ptr(h), _ptr(s_q), _ptr(qh), _stream()))
+    _c.det_swiglu_fwd_q(gu, rows, F, h, s_q, qh)
 
 
 def det_swiglu_bwd(dh, gu, rows, F, dgu):
-    _check("det_swiglu_bwd", load().det_swiglu_bwd(_ptr(dh), _ptr(gu), rows, F, _ptr(dgu), _stream()))
+    _c.det_swiglu_bwd(dh, gu, rows, F, dgu)
 
 
 def det_residual_add(a, b, n, y):
-    _check("det_residual_add", load().det_residual_add(_ptr(a), _ptr(b), n, _ptr(y), _stream()))
+    _c.det_residual_add(a, b, n, y)
 
 
 def det_embed_fwd(tok, T, E, V, D, y):
-    _check("det_embed_fwd", load().det_embed_fwd(_ptr(tok), T, _ptr(E), V, D, _ptr(y), _stream()))
+    _c.det_embed_fwd(tok, T, E, V, D, y)
 
 
 def det_embed_bwd(tok, T, dy, V, D, dE):
-    _check("det_embed_bwd", load().det_embed_bwd(_ptr(tok), T, _ptr(dy), V, D, _ptr(dE), _stream()))
+    _c.det_embed_bwd(tok, T, dy, V, D, dE)
 
 
 def det_lmhead_fwd(H, W, M, V, K, logits):
-    _check("det_lmhead_fwd", load().det_lmhead_fwd(_ptr(H), _ptr(W), M, V, K, _ptr(logits), _stream()))
+    _c.det_lmhead_fwd(H, W, M, V, K, logits)
 
 
 def det_lmhead_fwd_v2_ws_bytes(M, V, K):
@@ -352,8 +349,7 @@ def det_lmhead_fwd_v2_ws_bytes(M, V, K):
 
 
 def det_lmhead_fwd_v2(H, W, M, V, K, logits, ws, status_dev=None):
-    _check("det_lmhead_fwd_v2", load().det_lmhead_fwd_v2(_ptr(H), _ptr(W), M, V, K, _ptr(logits),
-                                                         *_ws(ws), _stream(), _ptr(status_dev)))
+    _c.det_lmhead_fwd_v2(H, W, M, V, K, logits, ws, status_dev)
 
 
 def det_lmhead_bwd_v2_ws_bytes(M, V, K):
@@ -361,8 +357,7 @@ def det_lmhead_bwd_v2_ws_bytes(M, V, K):
 
 
 def det_lmhead_bwd_v2(dlogits, H, W, M, V, K, dH, dW, ws, status_dev=None):
-    _check("det_lmhead_bwd_v2", load().det_lmhead_bwd_v2(_ptr(dlogits), _ptr(H), _ptr(W), M, V, K,
-                                                         _ptr(dH), _ptr(dW), *_ws(ws), _stream(), _ptr(status_dev)))
+    _c.det_lmhead_bwd_v2(dlogits, H, W, M, V, K, dH, dW, ws, status_dev)
 
 
 def det_attn_fwd_v2_ws_bytes(B, H, S):
@@ -370,13 +365,11 @@ def det_attn_fwd_v2_ws_bytes(B, H, S):
 
 
 def det_attn_fwd_v2(q, k, v, ld, B, H, S, out, ld_out, lse, ws, status_dev=None):
-    _check("det_attn_fwd_v2", load().det_attn_fwd_v2(_ptr(q), _ptr(k), _ptr(v), ld, B, H, S,
-                                                     _ptr(out), ld_out, _ptr(lse), *_ws(ws), _stream(), _ptr(status_dev)))
+    _c.det_attn_fwd_v2(q, k, v, ld, B, H, S, out, ld_out, lse, ws, status_dev)
 
 
 def det_lmhead_bwd(dlogits, H, W, M, V, K, dH, dW, first_chunk):
-    _check("det_lmhead_bwd", load().det_lmhead_bwd(_ptr(dlogits), _ptr(H), _ptr(W), M, V, K,
-                                                   _ptr(dH), _ptr(dW), first_chunk, _stream()))
+    _c.det_lmhead_bwd(dlogits, H, W, M, V, K, dH, dW, first_chunk)
 
 
 def det_test_lmhead_tile(which, tile, A, B, M, V, K, out, first_chunk=1):
@@ -424,8 +417,7 @@ def det_tensor_hash_ws_bytes(nbytes):
 
 def det_tensor_hash_async(p, nbytes, out32_dev, ws):
     """Queues the hash; the 32-byte root lands in out32_dev (device) in stream order, nothing synchronises."""
-    _check("det_tensor_hash_async", load().det_tensor_hash_async(_ptr(p), nbytes, _ptr(out32_dev), *_ws(ws),
-                                                                 _stream()))
+    _c.det_tensor_hash_async(p, nbytes, out32_dev, ws)
 
 
 def det_tensor_hash(p, nbytes, ws):

@@ -38,7 +38,7 @@ def build_binding(force=False):
     import torch
     src, stamp = os.path.join(CSRC, "binding.cpp"), os.path.join(_DIR, "build", "_binding.versions")
     versions = "torch %s, Python %s\n" % (torch.__version__, sysconfig.get_config_var("SOABI"))
-    if not force and not _stale(BINDING, [src]) and os.path.exists(stamp) and open(stamp).read() == versions:
+    if not force and not _stale(BINDING, [src, os.path.join(_DIR, "..", "include", "det.h")]) and os.path.exists(stamp) and open(stamp).read() == versions:
         return BINDING
     from torch.utils import cpp_extension
     lib = os.path.join(os.path.dirname(torch.__file__), "lib")

@@ -79,6 +79,43 @@ def test_tables_are_checked():
         det.det_tensor_hash_batch([t(64, torch.uint8)], t(32, torch.uint8), t(4096, torch.uint8))
 
 
+# the native callables take what an argument with a declared C type takes (integers of any kind, ctypes objects of that very type) and
+# refuse the rest; a status that is not DET_OK raises.  Rows of no values are refused and no rows return at once, so nothing is launched
+def test_native_calls_convert_and_refuse():
+    import numpy as np
+    import pytest
+    import torch
+    import paper_2609_17380_b200 as det
+    from paper_2609_17380_b200 import _binding
+    det.load()
+    patterns = {n: p.replace("s", "p") for n, p in det._PATTERNS.items()}            # the stream as an argument: no device is touched
+    calls = _binding.bind(det._SO, patterns, det._check)
+    try:
+        swiglu, hash_ = calls["det_swiglu_bwd"], calls["det_tensor_hash_async"]
+        for width in (0, np.int64(0), False, ctypes.c_int(0), 1 << 32):              # 2^32 is 0 in a C int
+            assert swiglu(16, 16, width, 8, 16, None) is None                        # no rows
+            with pytest.raises(det.DetError) as e:
+                swiglu(16, 16, 0, width, 16, None)
+            assert e.value.code == -1
+        for bad in (0.0, "0", None, ctypes.c_long(0)):
+            with pytest.raises(TypeError):
+                swiglu(16, 16, bad, 8, 16, None)
+        for bad in ("x", 1.0):
+            with pytest.raises(TypeError):
+                swiglu(bad, 16, 0, 8, 16, None)
+        with pytest.raises(AssertionError):
+            swiglu(torch.zeros(4), 16, 0, 8, 16, None)                                # not a CUDA tensor
+        with pytest.raises(AttributeError):
+            hash_(16, 0, 16, 16, None)                                                # a workspace has to be a tensor
+        for n in (5, 7):
+            with pytest.raises(TypeError):
+                swiglu(*([0] * n))
+        with pytest.raises(ImportError):
+            _binding.bind(det._SO, dict(patterns, det_swiglu_bwd="pppppp"), det._check)
+    finally:
+        _binding.bind(det._SO, det._PATTERNS, det._check)
+
+
 # the binding is compiled against torch's headers: another torch version makes the object stale although its source is older
 def test_binding_follows_the_torch_version(monkeypatch):
     import subprocess
