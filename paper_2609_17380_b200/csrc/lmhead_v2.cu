@@ -12,6 +12,8 @@
 //   k_igemm_sl     persistent, one CTA per SM, 128 x 128 output tile; warp 0 streams the FOUR operand tiles of a 128-deep
 //                  step (H hi, H lo, W hi, W lo: 64 KiB) through a three-stage TMA ring, warp 1 issues the sixteen MMAs of
 //                  the step into three TMEM accumulators (hh | hl + lh | ll, 128 columns each), sixteen more combine and round.
+//                  Clusters of two or four share a tile with a long contraction
+//   k_igemm_sl_pair  the same by CTA pairs, 256 x 128 output tile, wherever a problem takes every step of every tile
 // Every mbarrier wait is bounded (DET_DEV_TIMEOUT), as in igemm.cu.
 #include "tc05.cuh"
 #include "internal.h"
