@@ -7,6 +7,7 @@
 #include <dlfcn.h>
 #include <string.h>
 
+#include <memory>
 #include <string>
 #include <type_traits>
 #include <utility>
@@ -89,11 +90,11 @@ struct Entry {
   const char* name;
   int (*call)(void*, const Slot*);
   std::string (*kinds)();
-  void* fn;
-  std::string pattern;                         // per Python argument: p i z f, or w a workspace (its address and size); s the current stream
   PyMethodDef def;
 };
-#define DET_ENTRY(f) {#f, &Typed<decltype(f)>::call, &Typed<decltype(f)>::kinds, nullptr, std::string(), {}}
+static PyObject* entry_call(PyObject* self, PyObject* const* args, Py_ssize_t nargs);
+#define DET_ENTRY(f) \
+  {#f, &Typed<decltype(f)>::call, &Typed<decltype(f)>::kinds, {#f, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&entry_call)), METH_FASTCALL, nullptr}}
 static Entry entries[] = {
     DET_ENTRY(det_sum), DET_ENTRY(det_sum_static), DET_ENTRY(det_scale_inplace), DET_ENTRY(det_lsq_weight_scale), DET_ENTRY(det_lsq_act_scale_init),
     DET_ENTRY(det_lsq_quantize_weight), DET_ENTRY(det_linear_fwd), DET_ENTRY(det_linear_fwd_q), DET_ENTRY(det_linear_bwd), DET_ENTRY(det_rmsnorm_fwd),
@@ -103,7 +104,16 @@ static Entry entries[] = {
     DET_ENTRY(det_swiglu_fwd_q), DET_ENTRY(det_swiglu_bwd), DET_ENTRY(det_residual_add), DET_ENTRY(det_embed_fwd), DET_ENTRY(det_embed_bwd),
     DET_ENTRY(det_lmhead_fwd), DET_ENTRY(det_lmhead_fwd_v2), DET_ENTRY(det_lmhead_bwd), DET_ENTRY(det_lmhead_bwd_v2), DET_ENTRY(det_attn_fwd_v2),
     DET_ENTRY(det_tensor_hash_async)};
-static PyObject* raise_status = nullptr;       // raise_status(name, status), set by bind
+
+// One callable that bind returns, owned by the capsule that is its self: nothing is shared between two results of bind.
+struct Callable {
+  const Entry* entry;
+  void* fn;
+  std::string pattern;                         // per Python argument: p i z f, or w a workspace (its address and size); s the current stream
+  PyObject* raise_status = nullptr;            // raise_status(name, status)
+  ~Callable() { Py_XDECREF(raise_status); }
+};
+static void callable_free(PyObject* capsule) { delete static_cast<Callable*>(PyCapsule_GetPointer(capsule, nullptr)); }
 
 // the value of a ctypes object of the given type, after a conversion of the object itself has failed; otherwise that error stands
 template <class T>
@@ -119,14 +129,15 @@ static bool value_of(PyObject* x, const char* type, T& out) {
 }
 static PyObject* entry_call(PyObject* self, PyObject* const* args, Py_ssize_t nargs) {
   HANDLE_TH_ERRORS
-  const Entry* e = static_cast<const Entry*>(PyCapsule_GetPointer(self, nullptr));
+  const Callable* e = static_cast<const Callable*>(PyCapsule_GetPointer(self, nullptr));
   if (!e) return nullptr;
+  const char* name = e->entry->name;
   Slot s[MAX_ARGS];
   int n = 0;
   Py_ssize_t a = 0;
   for (const char c : e->pattern) {
     if (c == 's') { s[n++].u = current_stream(); continue; }
-    if (a == nargs) { PyErr_Format(PyExc_TypeError, "%s: too few arguments", e->name); return nullptr; }
+    if (a == nargs) { PyErr_Format(PyExc_TypeError, "%s: too few arguments", name); return nullptr; }
     PyObject* x = args[a++];
     switch (c) {
       case 'p':
@@ -136,7 +147,7 @@ static PyObject* entry_call(PyObject* self, PyObject* const* args, Py_ssize_t na
         if (!address_of(x, s[n].u)) return nullptr;
         if (x == Py_None) s[n + 1].u = 0;
         else if (THPVariable_Check(x)) s[n + 1].u = THPVariable_Unpack(x).nbytes();
-        else { PyErr_Format(PyExc_AttributeError, "%s: a workspace is a tensor or None", e->name); return nullptr; }
+        else { PyErr_Format(PyExc_AttributeError, "%s: a workspace is a tensor or None", name); return nullptr; }
         n += 2;
         break;
       case 'f': {
@@ -151,12 +162,12 @@ static PyObject* entry_call(PyObject* self, PyObject* const* args, Py_ssize_t na
         ++n;
     }
   }
-  if (a != nargs) { PyErr_Format(PyExc_TypeError, "%s: too many arguments", e->name); return nullptr; }
+  if (a != nargs) { PyErr_Format(PyExc_TypeError, "%s: too many arguments", name); return nullptr; }
   int rc;
   Py_BEGIN_ALLOW_THREADS
-  rc = e->call(e->fn, s);
+  rc = e->entry->call(e->fn, s);
   Py_END_ALLOW_THREADS
-  if (rc != DET_OK) return PyObject_CallFunction(raise_status, "si", e->name, rc);
+  if (rc != DET_OK) return PyObject_CallFunction(e->raise_status, "si", name, rc);
   Py_RETURN_NONE;
   END_HANDLE_TH_ERRORS
 }
@@ -176,23 +187,24 @@ static PyObject* bind(PyObject*, PyObject* args) {
     const char* p = pat ? PyUnicode_AsUTF8(pat) : nullptr;
     std::string kinds;
     for (const char* c = p ? p : ""; *c; ++c) kinds += *c == 'w' ? std::string("pz") : std::string(1, *c == 's' ? 'p' : *c);
-    e.fn = dlsym(lib, e.name);
-    if (!e.fn || !p || kinds != e.kinds()) {
-      PyErr_Format(PyExc_ImportError, "%s: %s", e.name, e.fn ? "the pattern does not fit the declaration" : "not in the library");
+    std::unique_ptr<Callable> own(new Callable);
+    own->entry = &e;
+    own->fn = dlsym(lib, e.name);
+    if (!own->fn || !p || kinds != e.kinds()) {
+      PyErr_Format(PyExc_ImportError, "%s: %s", e.name, own->fn ? "the pattern does not fit the declaration" : "not in the library");
       Py_DECREF(out);
       return nullptr;
     }
-    e.pattern = p;
-    e.def = {e.name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&entry_call)), METH_FASTCALL, nullptr};
-    PyObject* self = PyCapsule_New(&e, nullptr, nullptr);
+    own->pattern = p;
+    own->raise_status = Py_NewRef(raise);
+    PyObject* self = PyCapsule_New(own.get(), nullptr, callable_free);
+    if (self) own.release();
     PyObject* f = self ? PyCFunction_New(&e.def, self) : nullptr;
     Py_XDECREF(self);
     const int bad = f ? PyDict_SetItemString(out, e.name, f) : -1;
     Py_XDECREF(f);
     if (bad) { Py_DECREF(out); return nullptr; }
   }
-  Py_INCREF(raise);
-  Py_XSETREF(raise_status, raise);
   return out;
   END_HANDLE_TH_ERRORS
 }

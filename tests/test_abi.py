@@ -116,6 +116,25 @@ def test_native_calls_convert_and_refuse():
         _binding.bind(det._SO, det._PATTERNS, det._check)
 
 
+# a second bind, one that is refused half-way included, leaves the callables of the first as they are: here they take the
+# stream as an argument, where the package's take the current one
+def test_bound_calls_stay_as_they_were_bound():
+    import pytest
+    import paper_2609_17380_b200 as det
+    from paper_2609_17380_b200 import _binding
+    det.load()
+    patterns = {n: p.replace("s", "p") for n, p in det._PATTERNS.items()}
+    swiglu = _binding.bind(det._SO, patterns, det._check)["det_swiglu_bwd"]
+    other = lambda name, status: 1 / 0
+    _binding.bind(det._SO, det._PATTERNS, other)
+    assert swiglu(16, 16, 0, 8, 16, None) is None
+    with pytest.raises(ImportError):
+        _binding.bind(det._SO, dict(det._PATTERNS, det_tensor_hash_async="p"), other)
+    assert swiglu(16, 16, 0, 8, 16, None) is None
+    with pytest.raises(det.DetError):
+        swiglu(16, 16, 0, 0, 16, None)
+
+
 # the binding is compiled against torch's headers: another torch version makes the object stale although its source is older
 def test_binding_follows_the_torch_version(monkeypatch):
     import subprocess
