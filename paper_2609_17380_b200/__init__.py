@@ -111,7 +111,7 @@ def load():
             fn.argtypes = [_CTYPES[c] for c in sig[1:]]
         from . import _binding
         _ptr, _stream = _binding.ptr, _binding.stream
-        _c.__dict__.update(_binding.bind(_SO, _PATTERNS, _check))
+        _c.__dict__.update(_binding.bind(_SO, _PATTERNS, _check, lib))
         _lib = lib
     return _lib
 

@@ -2,10 +2,9 @@
 // tensor) and the current stream.  bind: callables for entry points of libdet.so that convert their own arguments, tensors, numbers, a
 // workspace and the current stream, call with the interpreter's lock released and raise on a status that is not DET_OK.  One call of 19
 // arguments took some 7 us of the host through a Python expression per argument and ctypes, and those calls, not the GPU,
-// are what a single small linear waits for.
+// are what a single small linear waits for.  Numbers that are no Python int or float go through ctypes as before.
 #include <Python.h>
 #include <dlfcn.h>
-#include <string.h>
 
 #include <memory>
 #include <string>
@@ -110,21 +109,31 @@ struct Callable {
   const Entry* entry;
   void* fn;
   std::string pattern;                         // per Python argument: p i z f, or w a workspace (its address and size); s the current stream
+  PyObject* general = nullptr;                 // the entry point with its C types declared (ctypes)
   PyObject* raise_status = nullptr;            // raise_status(name, status)
-  ~Callable() { Py_XDECREF(raise_status); }
+  ~Callable() { Py_XDECREF(general); Py_XDECREF(raise_status); }
 };
 static void callable_free(PyObject* capsule) { delete static_cast<Callable*>(PyCapsule_GetPointer(capsule, nullptr)); }
 
-// the value of a ctypes object of the given type, after a conversion of the object itself has failed; otherwise that error stands
-template <class T>
-static bool value_of(PyObject* x, const char* type, T& out) {
-  if (strcmp(Py_TYPE(x)->tp_name, type)) return false;
-  PyErr_Clear();
-  PyObject* v = PyObject_GetAttrString(x, "value");
-  if (!v) return false;
-  if constexpr (std::is_same<T, double>::value) out = PyFloat_AsDouble(v);
-  else out = PyLong_AsUnsignedLongLongMask(v);
-  Py_DECREF(v);
+// The call with arguments that are not plain Python numbers: addresses, sizes and the stream as they have been found, the numbers as
+// they came, so that what is taken for a number, and the error for what is not, are those of the declared types.
+static bool call_general(const Callable& e, const Slot* s, PyObject* const* args, int& rc) {
+  PyObject* t = PyTuple_New((Py_ssize_t)e.entry->kinds().size());
+  if (!t) return false;
+  Py_ssize_t n = 0;
+  for (const char c : e.pattern) {
+    if (c != 's') ++args;
+    for (int k = 0; k < (c == 'w' ? 2 : 1); ++k, ++n) {
+      PyObject* x = c == 'i' || c == 'z' || c == 'f' ? Py_NewRef(args[-1]) : PyLong_FromUnsignedLongLong(s[n].u);
+      if (!x) { Py_DECREF(t); return false; }
+      PyTuple_SET_ITEM(t, n, x);
+    }
+  }
+  PyObject* r = PyObject_CallObject(e.general, t);
+  Py_DECREF(t);
+  if (!r) return false;
+  rc = (int)PyLong_AsLong(r);
+  Py_DECREF(r);
   return !PyErr_Occurred();
 }
 static PyObject* entry_call(PyObject* self, PyObject* const* args, Py_ssize_t nargs) {
@@ -133,8 +142,9 @@ static PyObject* entry_call(PyObject* self, PyObject* const* args, Py_ssize_t na
   if (!e) return nullptr;
   const char* name = e->entry->name;
   Slot s[MAX_ARGS];
-  int n = 0;
+  int n = 0, rc;
   Py_ssize_t a = 0;
+  bool plain = true;                           // every number is a Python int or float
   for (const char c : e->pattern) {
     if (c == 's') { s[n++].u = current_stream(); continue; }
     if (a == nargs) { PyErr_Format(PyExc_TypeError, "%s: too few arguments", name); return nullptr; }
@@ -150,34 +160,40 @@ static PyObject* entry_call(PyObject* self, PyObject* const* args, Py_ssize_t na
         else { PyErr_Format(PyExc_AttributeError, "%s: a workspace is a tensor or None", name); return nullptr; }
         n += 2;
         break;
-      case 'f': {
-        double d = PyFloat_AsDouble(x);
-        if (d == -1.0 && PyErr_Occurred() && !value_of(x, "c_float", d)) return nullptr;
-        s[n++].f = static_cast<float>(d);
+      case 'f':
+        plain = plain && (PyFloat_Check(x) || PyLong_Check(x));
+        if (plain) {
+          const double d = PyFloat_AsDouble(x);
+          s[n].f = static_cast<float>(d);
+          if (d == -1.0 && PyErr_Occurred()) { PyErr_Clear(); plain = false; }   // an integer beyond the range
+        }
+        ++n;
         break;
-      }
       default:
-        s[n].u = PyLong_AsUnsignedLongLongMask(x);   // integers of any kind, the C type's own ctypes object
-        if (s[n].u == ~0ull && PyErr_Occurred() && !value_of(x, c == 'i' ? "c_int" : "c_ulong", s[n].u)) return nullptr;
+        plain = plain && PyLong_Check(x);
+        if (plain) s[n].u = PyLong_AsUnsignedLongLongMask(x);
         ++n;
     }
   }
   if (a != nargs) { PyErr_Format(PyExc_TypeError, "%s: too many arguments", name); return nullptr; }
-  int rc;
-  Py_BEGIN_ALLOW_THREADS
-  rc = e->entry->call(e->fn, s);
-  Py_END_ALLOW_THREADS
+  if (plain) {
+    Py_BEGIN_ALLOW_THREADS
+    rc = e->entry->call(e->fn, s);
+    Py_END_ALLOW_THREADS
+  } else if (!call_general(*e, s, args, rc)) {
+    return nullptr;
+  }
   if (rc != DET_OK) return PyObject_CallFunction(e->raise_status, "si", name, rc);
   Py_RETURN_NONE;
   END_HANDLE_TH_ERRORS
 }
 
-// bind(path of libdet.so, {name: pattern}, raise_status) -> {name: callable}
+// bind(path of libdet.so, {name: pattern}, raise_status, the library with its C types declared) -> {name: callable}
 static PyObject* bind(PyObject*, PyObject* args) {
   HANDLE_TH_ERRORS
   const char* path;
-  PyObject *patterns, *raise;
-  if (!PyArg_ParseTuple(args, "sO!O", &path, &PyDict_Type, &patterns, &raise)) return nullptr;
+  PyObject *patterns, *raise, *declared;
+  if (!PyArg_ParseTuple(args, "sO!OO", &path, &PyDict_Type, &patterns, &raise, &declared)) return nullptr;
   void* lib = dlopen(path, RTLD_NOW);
   if (!lib) { PyErr_Format(PyExc_ImportError, "%s", dlerror()); return nullptr; }
   PyObject* out = PyDict_New();
@@ -196,8 +212,9 @@ static PyObject* bind(PyObject*, PyObject* args) {
       return nullptr;
     }
     own->pattern = p;
+    own->general = PyObject_GetAttrString(declared, e.name);
     own->raise_status = Py_NewRef(raise);
-    PyObject* self = PyCapsule_New(own.get(), nullptr, callable_free);
+    PyObject* self = own->general ? PyCapsule_New(own.get(), nullptr, callable_free) : nullptr;
     if (self) own.release();
     PyObject* f = self ? PyCFunction_New(&e.def, self) : nullptr;
     Py_XDECREF(self);

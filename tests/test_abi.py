@@ -79,41 +79,56 @@ def test_tables_are_checked():
         det.det_tensor_hash_batch([t(64, torch.uint8)], t(32, torch.uint8), t(4096, torch.uint8))
 
 
-# the native callables take what an argument with a declared C type takes (integers of any kind, ctypes objects of that very type) and
-# refuse the rest; a status that is not DET_OK raises.  Rows of no values are refused and no rows return at once, so nothing is launched
+# the native callables take what an argument with a declared C type takes (integers of any kind, ctypes objects of that type or of one
+# derived from it, anything with _as_parameter_) and refuse the rest as ctypes does, naming the argument; a status that is not DET_OK
+# raises.  Rows of no values are refused and no rows return at once, so nothing is launched
 def test_native_calls_convert_and_refuse():
     import numpy as np
     import pytest
     import torch
     import paper_2609_17380_b200 as det
     from paper_2609_17380_b200 import _binding
-    det.load()
+    lib = det.load()
     patterns = {n: p.replace("s", "p") for n, p in det._PATTERNS.items()}            # the stream as an argument: no device is touched
-    calls = _binding.bind(det._SO, patterns, det._check)
-    try:
-        swiglu, hash_ = calls["det_swiglu_bwd"], calls["det_tensor_hash_async"]
-        for width in (0, np.int64(0), False, ctypes.c_int(0), 1 << 32):              # 2^32 is 0 in a C int
-            assert swiglu(16, 16, width, 8, 16, None) is None                        # no rows
-            with pytest.raises(det.DetError) as e:
-                swiglu(16, 16, 0, width, 16, None)
-            assert e.value.code == -1
-        for bad in (0.0, "0", None, ctypes.c_long(0)):
-            with pytest.raises(TypeError):
-                swiglu(16, 16, bad, 8, 16, None)
-        for bad in ("x", 1.0):
-            with pytest.raises(TypeError):
-                swiglu(bad, 16, 0, 8, 16, None)
-        with pytest.raises(AssertionError):
-            swiglu(torch.zeros(4), 16, 0, 8, 16, None)                                # not a CUDA tensor
-        with pytest.raises(AttributeError):
-            hash_(16, 0, 16, 16, None)                                                # a workspace has to be a tensor
-        for n in (5, 7):
-            with pytest.raises(TypeError):
-                swiglu(*([0] * n))
-        with pytest.raises(ImportError):
-            _binding.bind(det._SO, dict(patterns, det_swiglu_bwd="pppppp"), det._check)
-    finally:
-        _binding.bind(det._SO, det._PATTERNS, det._check)
+    calls = _binding.bind(det._SO, patterns, det._check, lib)
+    swiglu, hash_, norm = calls["det_swiglu_bwd"], calls["det_tensor_hash_async"], calls["det_rmsnorm_fwd_q"]
+
+    class Rows(ctypes.c_int):
+        pass
+
+    class Width:
+        def __init__(self, v):
+            self._as_parameter_ = v
+
+    for width in (0, np.int64(0), False, ctypes.c_int(0), 1 << 32, torch.tensor(0), Rows(0), Width(0), Width(Rows(0))):   # 2^32 is 0 in a C int
+        assert swiglu(16, 16, width, 8, 16, None) is None                        # no rows
+        with pytest.raises(det.DetError) as e:
+            swiglu(16, 16, 0, width, 16, None)
+        assert e.value.code == -1
+    for eps in (1, 1e-6, 1e300, np.float32(1e-6), np.float64(1e-6), torch.tensor(1e-6), ctypes.c_float(1e-6), Width(1e-6)):
+        with pytest.raises(det.DetError) as e:                                    # rows of no values
+            norm(16, 16, 0, 0, eps, 16, 16, 16, 16, None)
+        assert e.value.code == -1
+    for bad in (0.0, "0", None, ctypes.c_long(0), Width("0")):
+        for call in (swiglu, lib.det_swiglu_bwd):                                 # the same from either
+            with pytest.raises(ctypes.ArgumentError, match="argument 3"):
+                call(16, 16, bad, 8, 16, None)
+    for bad in ("1", None, 10 ** 400, ctypes.c_double(1.0)):
+        for call in (norm, lib.det_rmsnorm_fwd_q):
+            with pytest.raises(ctypes.ArgumentError, match="argument 5"):
+                call(16, 16, 0, 0, bad, 16, 16, 16, 16, None)
+    for bad in ("x", 1.0):
+        with pytest.raises(TypeError):
+            swiglu(bad, 16, 0, 8, 16, None)
+    with pytest.raises(AssertionError):
+        swiglu(torch.zeros(4), 16, 0, 8, 16, None)                                # not a CUDA tensor
+    with pytest.raises(AttributeError):
+        hash_(16, 0, 16, 16, None)                                                # a workspace has to be a tensor
+    for n in (5, 7):
+        with pytest.raises(TypeError):
+            swiglu(*([0] * n))
+    with pytest.raises(ImportError):
+        _binding.bind(det._SO, dict(patterns, det_swiglu_bwd="pppppp"), det._check, lib)
 
 
 # a second bind, one that is refused half-way included, leaves the callables of the first as they are: here they take the
@@ -122,14 +137,14 @@ def test_bound_calls_stay_as_they_were_bound():
     import pytest
     import paper_2609_17380_b200 as det
     from paper_2609_17380_b200 import _binding
-    det.load()
+    lib = det.load()
     patterns = {n: p.replace("s", "p") for n, p in det._PATTERNS.items()}
-    swiglu = _binding.bind(det._SO, patterns, det._check)["det_swiglu_bwd"]
+    swiglu = _binding.bind(det._SO, patterns, det._check, lib)["det_swiglu_bwd"]
     other = lambda name, status: 1 / 0
-    _binding.bind(det._SO, det._PATTERNS, other)
+    _binding.bind(det._SO, det._PATTERNS, other, lib)
     assert swiglu(16, 16, 0, 8, 16, None) is None
     with pytest.raises(ImportError):
-        _binding.bind(det._SO, dict(det._PATTERNS, det_tensor_hash_async="p"), other)
+        _binding.bind(det._SO, dict(det._PATTERNS, det_tensor_hash_async="p"), other, lib)
     assert swiglu(16, 16, 0, 8, 16, None) is None
     with pytest.raises(det.DetError):
         swiglu(16, 16, 0, 0, 16, None)
