@@ -72,8 +72,17 @@ static A slot_as(const Slot& s) {
   else return static_cast<A>(s.u);
 }
 template <class A>
-static constexpr char kind_of() {              // the letters of a signature
-  return std::is_pointer<A>::value ? 'p' : std::is_same<A, float>::value ? 'f' : sizeof(A) == 8 ? 'z' : 'i';
+static constexpr char kind_of() {              // the letters of a signature; v: void*, what a workspace and a stream are declared as
+  return std::is_same<A, void*>::value ? 'v' : std::is_pointer<A>::value ? 'p' : std::is_same<A, float>::value ? 'f' : sizeof(A) == 8 ? 'z' : 'i';
+}
+// whether a pattern gives each C argument what its type takes: a stream and a workspace only where there is a void*
+static bool fits(const char* pattern, const std::string& kinds) {
+  size_t n = 0;
+  for (const char* c = pattern; *c; ++c) {
+    const char k = n < kinds.size() ? kinds[n++] : 0;
+    if (*c == 'w' ? k != 'v' || kinds[n++] != 'z' : *c == 's' ? k != 'v' : *c == 'p' ? k != 'p' && k != 'v' : k != *c || k == 'v') return false;
+  }
+  return n == kinds.size();
 }
 template <class... A, size_t... I>
 static int invoke(int (*fn)(A...), const Slot* s, std::index_sequence<I...>) { return fn(slot_as<A>(s[I])...); }
@@ -201,12 +210,10 @@ static PyObject* bind(PyObject*, PyObject* args) {
   for (Entry& e : entries) {
     PyObject* pat = PyDict_GetItemString(patterns, e.name);
     const char* p = pat ? PyUnicode_AsUTF8(pat) : nullptr;
-    std::string kinds;
-    for (const char* c = p ? p : ""; *c; ++c) kinds += *c == 'w' ? std::string("pz") : std::string(1, *c == 's' ? 'p' : *c);
     std::unique_ptr<Callable> own(new Callable);
     own->entry = &e;
     own->fn = dlsym(lib, e.name);
-    if (!own->fn || !p || kinds != e.kinds()) {
+    if (!own->fn || !p || !fits(p, e.kinds())) {
       PyErr_Format(PyExc_ImportError, "%s: %s", e.name, own->fn ? "the pattern does not fit the declaration" : "not in the library");
       Py_DECREF(out);
       return nullptr;

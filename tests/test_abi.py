@@ -150,6 +150,22 @@ def test_bound_calls_stay_as_they_were_bound():
         swiglu(16, 16, 0, 0, 16, None)
 
 
+# a pattern with the current stream or a workspace where the entry point takes another pointer, the status word say, is refused, and so is
+# one that is too short or too long; the table of C types and the patterns describe the same arguments
+def test_patterns_fit_the_declarations():
+    import pytest
+    import paper_2609_17380_b200 as det
+    from paper_2609_17380_b200 import _binding
+    lib = det.load()
+    for name, bad in (("det_linear_fwd", "ppppiiippps"), ("det_linear_fwd", "sppppiiippp"), ("det_linear_fwd", "ppppiiipps"),
+                      ("det_linear_fwd", "ppppiiippspp"), ("det_sum", "pzipw"), ("det_sum", "pziwws"), ("det_sum", "wipws"), ("det_sum", ""),
+                      ("det_sum", "vzipws"), ("det_sum", "pzipvzs"), ("det_xent_bwd", "pppiifis")):
+        with pytest.raises(ImportError):
+            _binding.bind(det._SO, dict(det._PATTERNS, **{name: bad}), det._check, lib)
+    for name, p in det._PATTERNS.items():
+        assert det._SIGNATURES[name] == "i" + p.replace("w", "pz").replace("s", "p"), name
+
+
 # the binding is compiled against torch's headers: another torch version makes the object stale although its source is older
 def test_binding_follows_the_torch_version(monkeypatch):
     import subprocess
