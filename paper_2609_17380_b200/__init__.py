@@ -90,7 +90,10 @@ class _Calls:
 
     def __getattr__(self, name):
         load()
-        return self.__dict__[name]
+        try:
+            return self.__dict__[name]
+        except KeyError:
+            raise AttributeError(name) from None
 
 
 _c = _Calls()

@@ -166,6 +166,11 @@ def test_patterns_fit_the_declarations():
         assert det._SIGNATURES[name] == "i" + p.replace("w", "pz").replace("s", "p"), name
 
 
+def test_unknown_entry_point_is_an_attribute_error():
+    import paper_2609_17380_b200 as det
+    assert callable(det._c.det_sum) and not hasattr(det._c, "det_no_such_thing")
+
+
 # the binding is compiled against torch's headers: another torch version makes the object stale although its source is older
 def test_binding_follows_the_torch_version(monkeypatch):
     import subprocess
