@@ -233,7 +233,7 @@ __device__ __forceinline__ float sl_float(long long I) {
   return __fmaf_rn(h, 8388608.0f, l);
 }
 // whether every result of this row against columns with exponents lo .. hi is 0 or a normal number whatever I: 2^e and 2^(e + 44) are, with
-// e = ea + eb - 280.  A non-finite row or column (bit 30) is not.
+// e = ea + eb - 280.  For finite rows and columns (the flag of the others, bit 30, would overflow the sums).
 __device__ __forceinline__ bool sl_plain(int ea, int lo, int hi) { return ea + lo >= 154 && ea + hi <= 363; }
 
 // Rounding and stores of one tile, by a warp that owns 32 rows (a lane each) and 32 columns: ready() waits for the tile's MMAs, after
@@ -253,7 +253,7 @@ __device__ __forceinline__ bool sl_tile(const SlArgs& p, int z, int row, int j0,
   const int ebv = p.Eb[(size_t)z * p.J + j0 + part * 32 + lane];
   const int any_bad = __any_sync(0xffffffffu, ((ea | ebv) >> 30) != 0);
   const int ea280 = (ea & 0xFF) - 280;
-  const bool plain = __all_sync(0xffffffffu, sl_plain(ea, __reduce_min_sync(0xffffffffu, ebv), __reduce_max_sync(0xffffffffu, ebv)));
+  const bool plain = !any_bad && __all_sync(0xffffffffu, sl_plain(ea, __reduce_min_sync(0xffffffffu, ebv), __reduce_max_sync(0xffffffffu, ebv)));
   uint32_t* cexp = reinterpret_cast<uint32_t*>(stage);
   __syncwarp();
   cexp[lane] = (uint32_t)ebv << 23;

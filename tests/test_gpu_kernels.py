@@ -134,6 +134,28 @@ def test_lmhead_v2_shared_tiles(det, M, V, K, spread):
     assert_same_bits(host(lg), v2.lmhead_fwd(H, W), "version-2 logits")
 
 
+# rows that are all non-finite for one warp against columns of which one is: every one of its results is NaN, the others stay as they are
+@pytest.mark.parametrize("M,V", [(128, 128), (256, 9728)])
+def test_lmhead_v2_non_finite_warp(det, M, V):
+    import torch
+    from oracle import v2
+    K = 128
+    H, W = synth.normal_bf16((M, K), 1.0, seed=M, tid=1), synth.normal_bf16((V, K), 0.05, seed=M, tid=2)
+    H[32:64, 3] = synth.to_bf16(np.full(32, np.inf, F))
+    H[40:44, 5] = synth.to_bf16(np.full(4, np.nan, F))
+    W[70, 9] = synth.to_bf16(np.array([-np.inf], F))[0]
+    lg = empty((M, V), F)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    det.det_lmhead_fwd_v2(dev(H), dev(W), M, V, K, lg, ws(det.det_lmhead_fwd_v2_ws_bytes(M, V, K)), status)
+    _sync()
+    assert int(status.item()) == 0
+    got, want = host(lg), v2.lmhead_fwd(H, W)
+    bad = np.zeros((M, V), bool)
+    bad[32:64], bad[:, 70] = True, True
+    assert np.array_equal(np.isnan(got), bad) and np.array_equal(np.isnan(want), bad)
+    assert_same_bits(got[~bad], want[~bad], "version-2 logits")
+
+
 # attention at head and row counts where the rows per CTA change (32, 64, 128 rows), S off the 128 grid, windows that start
 # and end inside a block, grouped heads (one accumulator over the whole group)
 @pytest.mark.parametrize("B,H,Hkv,S,W", [(1, 2, 2, 576, 0), (1, 40, 40, 320, 0), (2, 80, 80, 192, 0), (1, 3, 3, 704, 256),
