@@ -232,9 +232,10 @@ __device__ __forceinline__ float sl_float(long long I) {
   const float l = fadd(__uint_as_float(((uint32_t)I & 0x7fffffu) | 0x4b000000u), -8388608.0f);
   return __fmaf_rn(h, 8388608.0f, l);
 }
-// whether every result of this row against columns with exponents lo .. hi is 0 or a normal number whatever I: 2^e and 2^(e + 44) are, with
-// e = ea + eb - 280.  For finite rows and columns (the flag of the others, bit 30, would overflow the sums).
-__device__ __forceinline__ bool sl_plain(int ea, int lo, int hi) { return ea + lo >= 154 && ea + hi <= 363; }
+// whether every result of a row against columns with exponents lo .. hi is 0 or a normal number whatever I: 2^e and 2^(e + 44) are, with
+// e = ea280 + eb.  The row's exponent comes without the flag of a non-finite row, whose results are all replaced anyway; with the flag of
+// a column in hi it is false, and the sum of two flags would overflow.
+__device__ __forceinline__ bool sl_plain(int ea280, int lo, int hi) { return ea280 + lo >= -126 && ea280 + hi <= 83; }
 
 // Rounding and stores of one tile, by a warp that owns 32 rows (a lane each) and 32 columns: ready() waits for the tile's MMAs, after
 // the exponents have been fetched; totals(c, T) gives the integers of columns c .. c + CH - 1; release() is called by one lane once
@@ -253,7 +254,7 @@ __device__ __forceinline__ bool sl_tile(const SlArgs& p, int z, int row, int j0,
   const int ebv = p.Eb[(size_t)z * p.J + j0 + part * 32 + lane];
   const int any_bad = __any_sync(0xffffffffu, ((ea | ebv) >> 30) != 0);
   const int ea280 = (ea & 0xFF) - 280;
-  const bool plain = !any_bad && __all_sync(0xffffffffu, sl_plain(ea, __reduce_min_sync(0xffffffffu, ebv), __reduce_max_sync(0xffffffffu, ebv)));
+  const bool plain = __all_sync(0xffffffffu, sl_plain(ea280, __reduce_min_sync(0xffffffffu, ebv), __reduce_max_sync(0xffffffffu, ebv)));
   uint32_t* cexp = reinterpret_cast<uint32_t*>(stage);
   __syncwarp();
   cexp[lane] = (uint32_t)ebv << 23;
