@@ -13,7 +13,8 @@
 //                  step (H hi, H lo, W hi, W lo: 64 KiB) through a three-stage TMA ring, warp 1 issues the sixteen MMAs of
 //                  the step into three TMEM accumulators (hh | hl + lh | ll, 128 columns each), sixteen more combine and round.
 //                  Clusters of two or four share a tile with a long contraction
-//   k_igemm_sl_pair  the same by CTA pairs, 256 x 128 output tile, wherever a problem takes every step of every tile
+//   k_igemm_sl_pair  the same by CTA pairs, 256 x 128 output tile, where a problem takes every step of every tile, its rows
+//                  come to whole pairs and the steps are not few
 // Every mbarrier wait is bounded (DET_DEV_TIMEOUT), as in igemm.cu.
 #include "tc05.cuh"
 #include "internal.h"
@@ -650,8 +651,13 @@ int sliced_gemm_launch(const int8_t* Ah, const int8_t* Al, const int8_t* Bh, con
   // on some seven eighths of the SMs.
   if (whole && tiles * 4 <= sms - sms / 8 && steps >= 32) return sl_go(k_igemm_sl<4>, once[0], tiles * 4, tAh, tAl, tBh, tBl, p, status, st);
   if (whole && tiles * 2 <= sms && steps >= 16) return sl_go(k_igemm_sl<2>, once[1], tiles * 2, tAh, tAl, tBh, tBl, p, status, st);
-  // pairs wherever their tile fits (causal and row-tied problems are written for tiles of 128 rows)
-  if (whole && p.I % (2 * SL_T) == 0 && sms >= 2) {
+  // Pairs where their tile fits (causal and row-tied problems are written for tiles of 128 rows) and what a step gains has made up for the
+  // launch of clusters, some 2 us, and the longer drain of four accumulators: 15 steps in all rounds together, 6 a tile.  Single CTA
+  // and pair, us, one round (2048 x 1024 results) 12 steps 15.6 and 16.0, 14 17.2 and 17.1, 15 17.9 and 17.7; two (512 x 8064) 7 steps 19.5 and 19.8,
+  // 8 20.9 and 21.0, 10 23.7 and 23.2; four (1024 x 8064) 4 steps 25.9 and 27.1, 6 31.3 and 31.1, 16 65.2 and 58.2; 22 (1024 x 50304)
+  // 1 step 120 and 136, 4 128 and 133, 6 175 and 172, 16 390 and 335.
+  const long long rounds = (tiles + sms - 1) / sms;
+  if (whole && p.I % (2 * SL_T) == 0 && steps >= 6 && rounds * steps >= 15 && sms >= 2) {
     const long long pairs = tiles / 2 < sms / 2 ? tiles / 2 : sms / 2;
     return sl_go(k_igemm_sl_pair, once[2], 2 * pairs, tAh, tAl, tBh, tBl, p, status, st);
   }

@@ -114,10 +114,14 @@ def test_lmhead_v2_long_rows(det, M, V, K):
     assert_same_bits(got_W[:-1], want_W[:-1], "version-2 dW")
 
 
-# version-2 contraction where the CTAs that share a tile change (16 and 32 steps, 32 and 74 tiles), CTA pairs with one round and several,
-# and operands whose exponents cross the range in which every result is a normal number, in both directions
+# version-2 contraction on both sides of where the CTAs that share a tile change (15 and 16 steps; 32 steps with 32 and 33 tiles, 16
+# with 74 and 75) and of where CTA pairs begin (one round of tiles with 14 and 15 steps, two with 7 and 8, three with 5 and 6), and
+# operands whose exponents cross the range in which every result is a normal number, in both directions
 @pytest.mark.parametrize("M,V,K,spread", [(128, 128, 1920, False), (128, 128, 2048, False), (256, 128, 4096, True), (128, 4224, 4096, False),
-                                          (128, 9600, 2048, False), (256, 384, 256, True), (256, 20480, 128, False), (768, 6912, 384, True)])
+                                          (512, 1024, 4096, False), (256, 4736, 2048, False), (128, 9600, 2048, False),
+                                          (256, 5120, 1792, False), (256, 5120, 1920, False), (256, 9728, 896, False), (256, 9728, 1024, False),
+                                          (768, 6912, 640, False), (768, 6912, 768, True),
+                                          (256, 384, 256, True), (256, 20480, 128, False), (768, 6912, 384, True)])
 def test_lmhead_v2_shared_tiles(det, M, V, K, spread):
     import torch
     from oracle import v2
@@ -135,11 +139,10 @@ def test_lmhead_v2_shared_tiles(det, M, V, K, spread):
 
 
 # rows that are all non-finite for one warp against columns of which one is: every one of its results is NaN, the others stay as they are
-@pytest.mark.parametrize("M,V", [(128, 128), (256, 9728)])
-def test_lmhead_v2_non_finite_warp(det, M, V):
+@pytest.mark.parametrize("M,V,K", [(128, 128, 128), (256, 9728, 1024)])
+def test_lmhead_v2_non_finite_warp(det, M, V, K):
     import torch
     from oracle import v2
-    K = 128
     H, W = synth.normal_bf16((M, K), 1.0, seed=M, tid=1), synth.normal_bf16((V, K), 0.05, seed=M, tid=2)
     H[32:64, 3] = synth.to_bf16(np.full(32, np.inf, F))
     H[40:44, 5] = synth.to_bf16(np.full(4, np.nan, F))
