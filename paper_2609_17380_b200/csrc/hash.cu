@@ -176,8 +176,9 @@ __global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJ
 // and the chain itself is rounds alone: 12 instructions a round on the half-rate integer pipe instead of 22, ordered so that a and
 // e depend on the round before through one rotation, one exclusive or and one addition each.  A warp alone on its scheduler is bound by
 // that pipe, two cycles an instruction, so the additions that nothing waits for (schedule word + h + d, maj - d) go to the
-// multiply-add pipe: all levels of 1 MiB 151.3 -> 146.1 us, one chunk 84.9 -> 82.6 (all additions there: slower, by their latency).  While there are schedulers to
-// spare a second warp does the expanding, double-buffered.  65 blocks: 0.137 ms with a thread per chunk, 0.089 with
+// multiply-add pipe: all levels of 1 MiB 138.6 -> 133.0 us, one chunk 72.7 -> 69.9 (all additions there: slower, by their latency).  Their 1 is
+// the grid's height: from constant memory it was a miss that short chains wait for (60 bytes 13.7 -> 14.1 us, 13.8 with this).  While there
+// are schedulers to spare a second warp does the expanding, double-buffered.  65 blocks: 0.137 ms with a thread per chunk, 0.089 with
 // one warp per CTA, 0.076 with two; with the padding a word at a time 0.118, 0.077 and 0.066.
 constexpr int SF_CH = 8, SF_PITCH = 68;
 template <bool ROOT>
@@ -228,7 +229,7 @@ __global__ void __launch_bounds__(64) k_sha_few(const __grid_constant__ HashJobs
       *reinterpret_cast<uint4*>(row + i) = make_uint4(t[0], t[1], t[2], t[3]);
     }
   };
-  const uint32_t one = opaque_one(), minus_one = 0u - one;
+  const uint32_t one = gridDim.y, minus_one = 0u - one;   // 1, which the compiler does not know
   uint32_t h[8];
   sha_init(h);
   // a pair: the expanding warp is four blocks ahead; a single warp does one after the other
