@@ -94,8 +94,11 @@ def test_lmhead_every_tile(det, tile, M, V, K, tiny):
     assert_same_bits(host(dW), oracle.lmhead_bwd(g, H, W, dW_o)[1], "dW continued")
 
 
-# version-2 gradients where a row of logits is long enough for eight warps (4096 values), and one step below
-@pytest.mark.parametrize("M,V,K", [(128, 3968, 128), (128, 4096, 128), (256, 8320, 128)])
+# version-2 gradients where a row of logits is long enough for eight warps (4096 values), and one step below; a token gradient of 36
+# tiles and 16 steps (two CTAs a tile, bf16 results), one of 80 (pairs, bf16 results); the 1B shape's vocabulary, an odd number of row
+# tiles for the weight gradient
+@pytest.mark.parametrize("M,V,K", [(128, 3968, 128), (128, 4096, 128), (256, 8320, 128), (1152, 2048, 512), (1280, 2048, 1024),
+                                   (256, 50304, 128)])
 def test_lmhead_v2_long_rows(det, M, V, K):
     import torch
     from oracle import v2
@@ -136,6 +139,31 @@ def test_lmhead_v2_shared_tiles(det, M, V, K, spread):
     _sync()
     assert int(status.item()) == 0
     assert_same_bits(host(lg), v2.lmhead_fwd(H, W), "version-2 logits")
+
+
+# the longest contraction that is allowed, with the largest slices (bf16 reaches 16320 of 16383): totals up to 2^43.99 of either sign, ties of
+# the one rounding and their neighbours, accumulators that reach their largest, on each form of the contraction (four and two CTAs a tile,
+# one, pairs).  Four kinds of rows and thirty-two of columns, so the oracle takes one of each
+@pytest.mark.parametrize("M,V", [(128, 128), (128, 4224), (128, 9600), (256, 9728)])
+def test_lmhead_v2_largest_totals(det, M, V):
+    import torch
+    from oracle import v2
+    K, big = 65408, F(255.0 / 128)                                # 16320 = 255 * 64
+    h, w = np.full((4, K), big, F), np.full((32, K), big, F)
+    h[1], h[2, ::2], h[3] = -big, -big, F(1.0)                    # h[3]: products of 2^13, so that a column's sum is what is rounded
+    for i in range(32):                                           # sums of 2^29.99 with a tail of 31 .. 33 of 64 (a tie at 32)
+        w[i, 7 + i] = F((32 + 64 * (i % 4 // 2) + (i // 4) % 3 - 1) / 8192.0)
+    w[1::2] *= F(-1.0)
+    w[28:30, 0::3] = F(255.0 / 8192)                              # low slices of 127
+    H, W = synth.to_bf16(h), synth.to_bf16(w)
+    want = np.tile(v2.lmhead_fwd(H, W), (M // 4, V // 32))
+    assert np.abs(want).max() > 65400 * 3.96
+    lg = empty((M, V), F)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    det.det_lmhead_fwd_v2(dev(H).repeat(M // 4, 1), dev(W).repeat(V // 32, 1), M, V, K, lg, ws(det.det_lmhead_fwd_v2_ws_bytes(M, V, K)), status)
+    _sync()
+    assert int(status.item()) == 0
+    assert_same_bits(host(lg), want, "version-2 logits")
 
 
 # rows that are all non-finite for one warp against columns of which one is: every one of its results is NaN, the others stay as they are
