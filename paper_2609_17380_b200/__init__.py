@@ -1,9 +1,11 @@
 """paper_2609_17380_b200: bit-exact, replayable transformer training-step arithmetic on B200.
 
-Thin ctypes binding of libdet.so (see include/det.h).  Every function here has the name and the argument
+Binding of libdet.so (see include/det.h).  Every function here has the name and the argument
 order of its C-ABI entry point and only marshals arguments: torch tensors (CUDA, contiguous) are passed as
-device pointers, the current torch CUDA stream as the stream.  Nothing is computed in Python and there is
-no CPU fallback: importing the binding without the built library raises.
+device pointers, the current torch CUDA stream as the stream.  The stream-ordered entry points are called by
+_binding.so (csrc/binding.cpp), the size queries, the calls with tables and the test hooks through ctypes.
+Nothing is computed in Python and there is no CPU fallback: importing the binding without the built library
+raises.
 """
 import ctypes as C
 import os
@@ -40,7 +42,7 @@ class det_adamw_desc(C.Structure):
 
 
 # Result and arguments of every entry point, one letter each (p pointer, i int, z size_t, f float, l long long, u unsigned long
-# long): with the types declared once a call passes plain Python numbers, which is what a call costs on the host.
+# long): the types that ctypes converts by, also for the calls of the native binding with numbers that are no Python int or float.
 _CTYPES = {"p": C.c_void_p, "i": C.c_int, "z": C.c_size_t, "f": C.c_float, "l": C.c_longlong, "u": C.c_ulonglong}
 _SIGNATURES = {
     "det_device_sm_count": "i", "det_launch_count": "u", "det_sum_ws_bytes": "zz", "det_sum": "ipzippzp",

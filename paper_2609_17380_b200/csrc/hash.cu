@@ -178,8 +178,8 @@ __global__ void __launch_bounds__(64) k_sha_chunks(const __grid_constant__ HashJ
 // that pipe, two cycles an instruction, so the additions that nothing waits for (schedule word + h + d, maj - d) go to the
 // multiply-add pipe: all levels of 1 MiB 138.6 -> 133.0 us, one chunk 72.7 -> 69.9 (all additions there: slower, by their latency).  Their 1 is
 // the grid's height: from constant memory it was a miss that short chains wait for (60 bytes 13.7 -> 14.1 us, 13.8 with this).  While there
-// are schedulers to spare a second warp does the expanding, double-buffered.  65 blocks: 0.137 ms with a thread per chunk, 0.089 with
-// one warp per CTA, 0.076 with two; with the padding a word at a time 0.118, 0.077 and 0.066.
+// are schedulers to spare a second warp does the expanding, double-buffered.  65 blocks: 0.119 ms with a thread per chunk, 0.074 with
+// one warp per CTA, 0.063 with two.
 constexpr int SF_CH = 8, SF_PITCH = 68;
 template <bool ROOT>
 __global__ void __launch_bounds__(64) k_sha_few(const __grid_constant__ HashJobs jobs, uint8_t* __restrict__ out) {
@@ -267,10 +267,10 @@ __global__ void __launch_bounds__(64) k_sha_few(const __grid_constant__ HashJobs
 }
 
 // The rule, 65 blocks a chunk, 148 SMs of four schedulers.  Where the latency of a chain is what counts the form with the shorter chain
-// is taken: four lanes per chunk and a second warp while there are schedulers to spare (8 to 2368 chunks: 0.066 ms, one warp 0.077, a
-// thread per chunk 0.118), one warp while its warps do not outnumber the schedulers (up to 4736 chunks: 0.079, 0.125, 0.118), then
-// a thread per chunk with plain additions up to one warp per scheduler (6000: 0.118, four lanes 0.145, the multiply-add pipe's longer
-// latency 0.127; 18944: 0.125, 0.282, 0.133).  Beyond that the integer pipe is what counts (20480: 0.211 plain, 0.178; 65536: 0.406, 0.339;
+// is taken: four lanes per chunk and a second warp while there are schedulers to spare (8 to 2368 chunks: 0.063 ms, one warp 0.074, a
+// thread per chunk 0.119), one warp while its warps do not outnumber the schedulers (up to 4736 chunks: 0.077, 0.120, 0.120), then
+// a thread per chunk with plain additions up to one warp per scheduler (6000: 0.121, four lanes 0.139, the multiply-add pipe's longer
+// latency 0.129; 18944: 0.123, 0.270, 0.131).  Beyond that the integer pipe is what counts (20480: 0.215 plain, 0.181; 65536: 0.410, 0.342;
 // 262144: 1.33, 1.08).
 static void sha_few_launch(bool root, const HashJobs& jobs, uint32_t n, uint8_t* out, int sms, cudaStream_t st) {
   const unsigned ctas = (n + SF_CH - 1) / SF_CH;

@@ -226,8 +226,9 @@ __device__ __forceinline__ long long sl_total(uint32_t hh, uint32_t cr, uint32_t
   return t;
 }
 // binary32 of I, nearest even, for |I| < 2^44 (fewer than 2^16 terms of at most 16383^2): the bits above the 23 lowest and those 23 are
-// integers that adding 1.5 * 2^23 and 2^23 by their bits makes floats, and one fused multiply-add joins the two with the one rounding
-// (the conversion of a 64-bit integer with a test of its result's range took 34 instructions a result, this takes 11).
+// integers that adding 1.5 * 2^23 and 2^23 by their bits makes floats, and one fused multiply-add joins the two with the one rounding.
+// The whole kernel, polling in its waits included, executed 34.4 warp instructions for 32 results with the conversion of a 64-bit integer and a
+// test of its result's range, and 30.9 with this (logits of 16 heads x 2048, 0.122 -> 0.084 ms with the earlier release below).
 __device__ __forceinline__ float sl_float(long long I) {
   const float h = fadd(__int_as_float((int)(I >> 23) + 0x4b400000), -12582912.0f);
   const float l = fadd(__uint_as_float(((uint32_t)I & 0x7fffffu) | 0x4b000000u), -8388608.0f);
@@ -647,15 +648,16 @@ int sliced_gemm_launch(const int8_t* Ah, const int8_t* Al, const int8_t* Bh, con
   const long long tiles = (long long)p.Z * (p.I / SL_T) * (p.J / SL_T);
   const bool whole = !p.krange && !p.causal_tiles;      // every tile takes every step
   // Few tiles with a long contraction (a token gradient of 1024 x 1024 has 64 tiles of 256 steps) leave SMs idle: two or four CTAs share a
-  // tile (1024 x 1024 x 32768: 0.170 -> 0.114 ms).  A part is at least eight steps (the exchange costs about four); clusters of four find room
-  // on some seven eighths of the SMs.
+  // tile.  A part is at least eight steps (the exchange costs about four); clusters of four find room on some seven eighths of the SMs.
+  // One, two and four CTAs a tile, us: 2 tiles 16 steps 17.4, 13.9, 12.2, 32 steps 28.4, 19.5, 15.0; 64 tiles 8 steps 12.3, 11.9, 16 17.9,
+  // 14.9, 256 186, 106; 36 tiles 16 steps 17.8, 14.4 and, in clusters of four that do not all find room, 23.8; 80 tiles 16 steps 18.6, 27.7.
   if (whole && tiles * 4 <= sms - sms / 8 && steps >= 32) return sl_go(k_igemm_sl<4>, once[0], tiles * 4, tAh, tAl, tBh, tBl, p, status, st);
   if (whole && tiles * 2 <= sms && steps >= 16) return sl_go(k_igemm_sl<2>, once[1], tiles * 2, tAh, tAl, tBh, tBl, p, status, st);
   // Pairs where their tile fits (causal and row-tied problems are written for tiles of 128 rows) and what a step gains has made up for the
   // launch of clusters, some 2 us, and the longer drain of four accumulators: 15 steps in all rounds together, 6 a tile.  Single CTA
   // and pair, us, one round (2048 x 1024 results) 12 steps 15.6 and 16.0, 14 17.2 and 17.1, 15 17.9 and 17.7; two (512 x 8064) 7 steps 19.5 and 19.8,
   // 8 20.9 and 21.0, 10 23.7 and 23.2; four (1024 x 8064) 4 steps 25.9 and 27.1, 6 31.3 and 31.1, 16 65.2 and 58.2; 22 (1024 x 50304)
-  // 1 step 120 and 136, 4 128 and 133, 6 175 and 172, 16 390 and 335.
+  // 1 step 120 and 136, 4 157 and 159, 6 175 and 172, 16 390 and 335.
   const long long rounds = (tiles + sms - 1) / sms;
   if (whole && p.I % (2 * SL_T) == 0 && steps >= 6 && rounds * steps >= 15 && sms >= 2) {
     const long long pairs = tiles / 2 < sms / 2 ? tiles / 2 : sms / 2;
