@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
   Full Os = reinterpret_cast<Full>(osm + (size_t)DH * (TM + 4) * sizeof(float));    // [dim][query] of dO
   float(*Ks)[OK][OT + 4] = reinterpret_cast<float(*)[OK][OT + 4]>(osm + (size_t)2 * DH * (TM + 4) * sizeof(float));
   float(*Vs)[OK][OT + 4] = Ks + SDP_SLOTS;
-  __shared__ __align__(16) int tiny_s[SDP_SLOTS][OG_PROD / 32];
+  __shared__ __align__(4) uint8_t tiny_s[SDP_SLOTS][OG_PROD / 32];
   __shared__ int abort_s;
   __shared__ __align__(8) uint64_t bar_full[SDP_SLOTS], bar_empty[SDP_SLOTS];
   volatile int* abort_flag = &abort_s;
@@ -483,31 +483,35 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     // ------------------------------- producers -------------------------------
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(T::RP));
     const int pt = tid - SDP_CONS, pw = pt >> 5;
-    OgRaw<CONTIG, false, OT> rk, rv;
-    const uint16_t *kp, *vp;
-    auto head = [&]() {
+    typedef OgSide<CONTIG, false, OT> Side;
+    Side sk, sv;
+    Side::Raw rk, rv;
+    auto block = [&]() {                             // the key block `at`
       const size_t o = (size_t)(at.bh / H) * S * ld + (size_t)(at.bh % H / (H / Hkv)) * DH;
-      kp = k + o;
-      vp = v + o;
+      sk.init(k + o, S, ld, at.jt * OT, 0, pt);
+      sv.init(v + o, S, ld, at.jt * OT, 0, pt);
     };
-    head();
-    og_fetch<CONTIG, false, OT>(kp, S, DH, ld, at.jt * OT, 0, pt, rk);
-    og_fetch<CONTIG, false, OT>(vp, S, DH, ld, at.jt * OT, 0, pt, rv);
+    block();
+    sk.fetch(rk, OK, 0, pt);
+    sv.fetch(rv, OK, 0, pt);
     int slot = 0;
     uint32_t par = 1;
     const int nslab = (w_hi - w_lo) * (DH / OK);
     for (int s = 0; s < nslab; ++s) {
       if (!mbar_wait(&bar_empty[slot], par, abort_flag, nullptr)) break;
-      bool tiny = og_store<CONTIG, false, OT>(Ks[slot], pt, rk);
-      tiny |= og_store<CONTIG, false, OT>(Vs[slot], pt, rv);
+      uint32_t least = ~0u;
+      sk.store(Ks[slot], rk, least, pt);
+      sv.store(Vs[slot], rv, least, pt);
       if (s + 1 < nslab) {
-        if ((s + 1) % (DH / OK) == 0 && at.next(S, TM, W)) head();
-        const int c0n = ((s + 1) % (DH / OK)) * OK;
-        og_fetch<CONTIG, false, OT>(kp, S, DH, ld, at.jt * OT, c0n, pt, rk);
-        og_fetch<CONTIG, false, OT>(vp, S, DH, ld, at.jt * OT, c0n, pt, rv);
+        if ((s + 1) % (DH / OK) == 0) {
+          at.next(S, TM, W);
+          block();
+        }
+        sk.fetch(rk, OK, 0, pt);
+        sv.fetch(rv, OK, 0, pt);
       }
-      const int any = __any_sync(0xffffffffu, tiny);
-      if (lane == 0) tiny_s[slot][pw] = any;
+      const int any = __any_sync(0xffffffffu, least_tiny(least));
+      if (lane == 0) tiny_s[slot][pw] = (uint8_t)any;
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar_full[slot]);
       if (++slot == SDP_SLOTS) { slot = 0; par ^= 1u; }
@@ -573,9 +577,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
       for (int sl = 0; sl < DH / OK && ok; ++sl) {
         ok = __all_sync(0xffffffffu, mbar_wait(&bar_full[slot], par, abort_flag, nullptr));
         if (!ok) break;
-        const int4 t4 = *reinterpret_cast<const int4*>(tiny_s[slot]);
-        const int tiny = tqo | t4.x | t4.y | t4.z | t4.w;
-        if (tiny) { slab_mac<false, TM, OT, 8>(Qs + sl * OK, Ks[slot], ty, tx, sa); slab_mac<false, TM, OT, 8>(Os + sl * OK, Vs[slot], ty, tx, da); }
+        if (tqo | *reinterpret_cast<const uint32_t*>(tiny_s[slot])) { slab_mac<false, TM, OT, 8>(Qs + sl * OK, Ks[slot], ty, tx, sa); slab_mac<false, TM, OT, 8>(Os + sl * OK, Vs[slot], ty, tx, da); }
         else { slab_mac<true, TM, OT, 8>(Qs + sl * OK, Ks[slot], ty, tx, sa); slab_mac<true, TM, OT, 8>(Os + sl * OK, Vs[slot], ty, tx, da); }
         __syncwarp();
         if (lane == 0) mbar_arrive(&bar_empty[slot]);

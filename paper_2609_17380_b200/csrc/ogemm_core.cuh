@@ -23,9 +23,11 @@ enum { CONTIG = 0, STRIDED = 1 };
 // two bf16 values is exact in binary32.  Two accumulators are processed per instruction (packed f32x2 arithmetic, each
 // lane rounded on its own).
 //
-// The 8 x 16 tiles (FUSED) fetch the next step's operands before they multiply the current one's and keep that order (volatile):
-// 301 instead of 306 cycles per step of the 128 x 256 tile; other orders of the 64 multiply-adds (rows outermost, zigzag,
-// 2 x 2 blocks) took 302 to 326, and a copy of A with every value doubled, which needs no register pairs to be made, 365.
+// The 8 x 16 and 8 x 4 tiles (FUSED) fetch the next step's operands before they multiply the current one's and keep that order
+// (volatile): 302 instead of 306 cycles per step of the 128 x 256 tile; other orders of the 64 multiply-adds (rows outermost, zigzag,
+// 2 x 2 blocks) took 302 to 326, a copy of A with every value doubled 365, and bf16 words in shared memory that the consumers unpack
+// 335 to 383.  Counters say why: a packed multiply-add holds the issue port of its scheduler for two cycles, and twice the
+// multiply-adds plus everything else comes to 98 % of the cycles, so each further instruction costs its cycle.
 __device__ __forceinline__ float4 lds128_ordered(const float* p) {
   float4 v;
   asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(smem_u32(p)));
@@ -36,31 +38,42 @@ __device__ __forceinline__ void ffma2_ordered(float a, float2 b, float2& c) {
   asm volatile("fma.rn.ftz.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(f2bits(make_float2(a, a))), "l"(f2bits(b)));
   c = bits2f(d);
 }
-template <int TM, int TN>
-__device__ __forceinline__ void slab_mac_ordered(const float (*As)[TM + 4], const float (*Bs)[TN + 4], int ty, int tx, float2 (&acc)[8][8]) {
-  float4 a0 = lds128_ordered(&As[0][ty * 4]), a1 = lds128_ordered(&As[0][TM / 2 + ty * 4]), bn[4];
+// CARRY: the last step of a slab fetches the first operands of the next one, n slabs in all; else one slab.  One warp per scheduler
+// sees the latency of those loads (128 x 128 tiles alone on their SMs 171 -> 165 cycles per step, 32 x 64 56 -> 52), two hide it for each other
+// (128 x 256: 302 -> 308), and the 8 x 8 loop is best left to the compiler (64 x 128 alone: 91 -> 99).
+template <bool CARRY, int TM, int TN, int CT, int LA, int LB>
+__device__ __forceinline__ void slabs_ordered(const float (*As)[LA], const float (*Bs)[LB], int n, int ty, int tx, float2 (&acc)[8][CT / 2]) {
+  const float *pa = &As[0][ty * 4], *pb = &Bs[0][tx * 4];
+  float4 a0 = lds128_ordered(pa), a1 = lds128_ordered(pa + TM / 2), bn[CT / 4];
 #pragma unroll
-  for (int g = 0; g < 4; ++g) bn[g] = lds128_ordered(&Bs[0][g * (TN / 4) + tx * 4]);
+  for (int g = 0; g < CT / 4; ++g) bn[g] = lds128_ordered(pb + g * (TN * 4 / CT));
+#pragma unroll 1
+  do {
+    const float *qa = CARRY && n > 1 ? pa + OK * LA : pa, *qb = CARRY && n > 1 ? pb + OK * LB : pb;   // after the last slab: its first row again
 #pragma unroll
-  for (int k = 0; k < OK; ++k) {
-    const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-    float2 b[8];
+    for (int k = 0; k < OK; ++k) {
+      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      float2 b[CT / 2];
 #pragma unroll
-    for (int g = 0; g < 4; ++g) { b[2 * g] = make_float2(bn[g].x, bn[g].y); b[2 * g + 1] = make_float2(bn[g].z, bn[g].w); }
-    if (k + 1 < OK) {
-      a0 = lds128_ordered(&As[k + 1][ty * 4]);
-      a1 = lds128_ordered(&As[k + 1][TM / 2 + ty * 4]);
+      for (int g = 0; g < CT / 4; ++g) { b[2 * g] = make_float2(bn[g].x, bn[g].y); b[2 * g + 1] = make_float2(bn[g].z, bn[g].w); }
+      if (CARRY || k + 1 < OK) {
+        const float *na = k + 1 < OK ? pa + (k + 1) * LA : qa, *nb = k + 1 < OK ? pb + (k + 1) * LB : qb;
+        a0 = lds128_ordered(na);
+        a1 = lds128_ordered(na + TM / 2);
 #pragma unroll
-      for (int g = 0; g < 4; ++g) bn[g] = lds128_ordered(&Bs[k + 1][g * (TN / 4) + tx * 4]);
+        for (int g = 0; g < CT / 4; ++g) bn[g] = lds128_ordered(nb + g * (TN * 4 / CT));
+      }
+#pragma unroll
+      for (int j = 0; j < CT / 2; ++j)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) ffma2_ordered(av[i], b[j], acc[i][j]);
     }
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int i = 0; i < 8; ++i) ffma2_ordered(av[i], b[j], acc[i][j]);
-  }
+    pa = qa;
+    pb = qb;
+  } while (CARRY && --n > 0);
 }
-template <bool FUSED, int TM, int TN, int CT>
-__device__ __forceinline__ void slab_mac(const float (*As)[TM + 4], const float (*Bs)[TN + 4], int ty, int tx,
+template <bool FUSED, int TM, int TN, int CT, int LA, int LB>
+__device__ __forceinline__ void slab_mac(const float (*As)[LA], const float (*Bs)[LB], int ty, int tx,
                                          float2 (&acc)[8][CT / 2]) {
 #pragma unroll
   for (int k = 0; k < OK; ++k) {
@@ -110,76 +123,110 @@ __device__ __forceinline__ void word_tiny(uint32_t u, uint32_t& m) {
 }
 __device__ __forceinline__ bool words_tiny(uint32_t m) { return (m & 0x80008000u) != 0; }
 
+// The same test on two instructions a word: m, which starts at ~0, becomes the smaller of itself and the magnitudes less one, in
+// which a zero is the largest.
+__device__ __forceinline__ void word_least(uint32_t u, uint32_t& m) { m = __viaddmin_u16x2(u & 0x7fff7fffu, 0xffffffffu, m); }
+__device__ __forceinline__ bool least_tiny(uint32_t m) { return (m & 0xffffu) < 0x1fffu || (m >> 16) < 0x1fffu; }
+
 // One producer thread's share of a slab of ROWS rows x 16 contraction steps, as raw words.  Unit u = thread + 128 i:
-//   CONTIG : a 16-byte word (8 bf16 or 4 f32 contraction indices) of row u mod ROWS: consecutive lanes, consecutive rows
+//   CONTIG : a 16-byte word (8 bf16 or 4 f32 contraction indices) of RPU neighbouring rows: consecutive lanes, consecutive rows.  Two
+//            rows where that leaves a unit for every thread: their values go to shared memory as pairs, half the stores
 //   STRIDED: four consecutive rows 4f .. 4f+3, f = u mod ROWS/4, at one contraction index: consecutive lanes read and store
 //            consecutive words, so the shared-memory stores are free of bank conflicts
+// All units of a thread have the same rows, so a pointer (CONTIG: one per row) is all that fetching a slab needs.  Rows past the
+// last one repeat it: their results are not stored.
+// Every instruction here takes an issue cycle from the consumers of its scheduler (see slabs_ordered).  Running pointers instead of
+// addresses and bounds per load, the two-instruction test and the paired stores took the instructions beside the multiply-adds
+// from 0.30 to 0.25 per multiply-add (LM head forward, 128 x 256 tiles: 308 -> 302 cycles per step; weight gradient 310 -> 302).
 template <int MODE, bool F32IN, int ROWS>
-struct OgRaw {
-  static constexpr int UNITS = MODE == CONTIG ? ROWS * (F32IN ? 4 : 2) : 4 * ROWS;
-  static constexpr int PER = (UNITS + OG_PROD - 1) / OG_PROD;
-  uint4 w[(MODE == STRIDED && !F32IN) ? (PER + 1) / 2 : PER];   // STRIDED bf16: two units share one 16-byte register group
-};
-template <int MODE, bool F32IN, int ROWS>
-__device__ __forceinline__ void og_fetch(const void* base, int rows, int C, int ld, int r0, int c0, int pt,
-                                         OgRaw<MODE, F32IN, ROWS>& raw) {
-  typedef OgRaw<MODE, F32IN, ROWS> R;
-  constexpr int ESZ = F32IN ? 4 : 2;
-  const char* b = reinterpret_cast<const char*>(base);
+struct OgSide {
+  static constexpr int EPW = F32IN ? 4 : 8, ESZ = F32IN ? 4 : 2;          // CONTIG: contraction indices of a 16-byte word
+  static constexpr int RPU = MODE == STRIDED ? 4 : (ROWS * OK / EPW >= 2 * OG_PROD ? 2 : 1);
+  static constexpr int LINE = ROWS / RPU;                                 // units of one group of contraction indices
+  static constexpr int UNITS = LINE * (MODE == STRIDED ? OK : OK / EPW), PER = (UNITS + OG_PROD - 1) / OG_PROD;
+  static constexpr int CSTEP = (OG_PROD / LINE) * (MODE == STRIDED ? 1 : EPW);   // contraction indices from one unit of a thread to the next
+  static constexpr int NP = MODE == STRIDED ? 1 : RPU, WORDS = MODE == STRIDED && !F32IN ? 2 : 4;   // pointers; 32-bit words of a load
+  static_assert(OG_PROD % LINE == 0 && (UNITS % OG_PROD == 0 || PER == 1), "units of a thread share their rows");
+  struct Raw { uint32_t w[PER][NP][WORDS]; };
+  const char* ptr[NP];
+  int c;                       // contraction index of the thread's first unit, relative to the slab's
+
+  __device__ __forceinline__ bool mine(int pt) const { return UNITS % OG_PROD == 0 || pt < UNITS; }
+  __device__ __forceinline__ void init(const void* base, int rows, int ld, int r0, int c0, int pt) {
+    c = (pt / LINE) * (MODE == STRIDED ? 1 : EPW);
 #pragma unroll
-  for (int i = 0; i < R::PER; ++i) {
-    const int u = pt + OG_PROD * i;
-    const bool mine = R::UNITS % OG_PROD == 0 || u < R::UNITS;
+    for (int q = 0; q < NP; ++q) {
+      const int r = min(r0 + RPU * (pt % LINE) + q, rows - (MODE == STRIDED ? 4 : 1));
+      ptr[q] = reinterpret_cast<const char*>(base) + (MODE == CONTIG ? (size_t)r * ld + c0 + c : (size_t)(c0 + c) * ld + r) * ESZ;
+    }
+  }
+  // the next slab, of which `left` contraction indices exist; step: bytes from one contraction index to the next (STRIDED)
+  __device__ __forceinline__ void fetch(Raw& raw, int left, long long step, int pt) {
+    if (!mine(pt)) return;
+    const bool full = left >= OK;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+#pragma unroll
+      for (int q = 0; q < NP; ++q) {
+        const char* src = MODE == CONTIG ? ptr[q] + i * CSTEP * ESZ : ptr[q];
+        uint32_t* w = raw.w[i][q];
+        if (full || c + i * CSTEP < left) {
+          if (WORDS == 4) {
+            const uint4 t = __ldg(reinterpret_cast<const uint4*>(src));
+            w[0] = t.x; w[1] = t.y; w[WORDS - 2] = t.z; w[WORDS - 1] = t.w;
+          } else {
+            const uint2 t = __ldg(reinterpret_cast<const uint2*>(src));
+            w[0] = t.x; w[1] = t.y;
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < WORDS; ++e) w[e] = 0u;
+        }
+      }
+      if (MODE == STRIDED) ptr[0] += CSTEP * step;
+    }
     if (MODE == CONTIG) {
-      const int r = r0 + u % ROWS, c = c0 + (u / ROWS) * (F32IN ? 4 : 8);
-      raw.w[i] = (mine && r < rows && c < C) ? __ldg(reinterpret_cast<const uint4*>(b + ((size_t)r * ld + c) * ESZ))
-                                             : make_uint4(0u, 0u, 0u, 0u);
-    } else {
-      const int r = r0 + 4 * (u % (ROWS / 4)), c = c0 + u / (ROWS / 4);
-      const bool ok = mine && r < rows && c < C;
-      const char* src = b + ((size_t)c * ld + r) * ESZ;
-      if (F32IN) {
-        raw.w[i] = ok ? __ldg(reinterpret_cast<const uint4*>(src)) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int q = 0; q < NP; ++q) ptr[q] += OK * ESZ;
+    }
+  }
+  __device__ __forceinline__ void skip(long long bytes) {
+#pragma unroll
+    for (int q = 0; q < NP; ++q) ptr[q] += bytes;
+  }
+  // unpack, test and store; m: see word_least
+  template <int LD>
+  __device__ __forceinline__ void store(float (*s)[LD], const Raw& raw, uint32_t& m, int pt) const {
+    if (!mine(pt)) return;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      constexpr int NW = MODE == STRIDED ? 2 : EPW / 2;       // words of bf16 pairs
+      uint32_t p[NP][NW];
+#pragma unroll
+      for (int q = 0; q < NP; ++q)
+#pragma unroll
+        for (int e = 0; e < NW; ++e) {
+          p[q][e] = F32IN ? word_of(raw.w[i][q][2 * e], raw.w[i][q][2 * e + 1]) : raw.w[i][q][e];
+          word_least(p[q][e], m);
+        }
+      const int k = c + i * CSTEP, r = RPU * (pt % LINE);
+      if (MODE == STRIDED) {
+        *reinterpret_cast<float4*>(&s[k][r]) = make_float4(word_lo(p[0][0]), word_hi(p[0][0]), word_lo(p[0][1]), word_hi(p[0][1]));
       } else {
-        const uint2 t = ok ? __ldg(reinterpret_cast<const uint2*>(src)) : make_uint2(0u, 0u);
-        if (i & 1) { raw.w[i >> 1].z = t.x; raw.w[i >> 1].w = t.y; }
-        else { raw.w[i >> 1].x = t.x; raw.w[i >> 1].y = t.y; }
+#pragma unroll
+        for (int e = 0; e < NW; ++e) {
+          if (RPU == 2) {
+            *reinterpret_cast<float2*>(&s[k + 2 * e][r]) = make_float2(word_lo(p[0][e]), word_lo(p[NP - 1][e]));
+            *reinterpret_cast<float2*>(&s[k + 2 * e + 1][r]) = make_float2(word_hi(p[0][e]), word_hi(p[NP - 1][e]));
+          } else {
+            s[k + 2 * e][r] = word_lo(p[0][e]);
+            s[k + 2 * e + 1][r] = word_hi(p[0][e]);
+          }
+        }
       }
     }
   }
-}
-// unpack, test and store one thread's share; returns the below-2^-63 flag of its values
-template <int MODE, bool F32IN, int ROWS>
-__device__ __forceinline__ bool og_store(float (*s)[ROWS + 4], int pt, const OgRaw<MODE, F32IN, ROWS>& raw) {
-  typedef OgRaw<MODE, F32IN, ROWS> R;
-  uint32_t m = 0;
-#pragma unroll
-  for (int i = 0; i < R::PER; ++i) {
-    const int u = pt + OG_PROD * i;
-    if (R::UNITS % OG_PROD != 0 && u >= R::UNITS) continue;
-    if (MODE == CONTIG) {
-      constexpr int EPW = F32IN ? 4 : 8;
-      const int r = u % ROWS, k = (u / ROWS) * EPW;
-      const uint4 q = raw.w[i];
-      const uint32_t p[4] = {F32IN ? word_of(q.x, q.y) : q.x, F32IN ? word_of(q.z, q.w) : q.y, q.z, q.w};
-#pragma unroll
-      for (int e = 0; e < EPW / 2; ++e) {
-        word_tiny(p[e], m);
-        s[k + 2 * e][r] = word_lo(p[e]);
-        s[k + 2 * e + 1][r] = word_hi(p[e]);
-      }
-    } else {
-      const int f = u % (ROWS / 4), k = u / (ROWS / 4);
-      uint32_t lo, hi;
-      if (F32IN) { lo = word_of(raw.w[i].x, raw.w[i].y); hi = word_of(raw.w[i].z, raw.w[i].w); }
-      else { lo = (i & 1) ? raw.w[i >> 1].z : raw.w[i >> 1].x; hi = (i & 1) ? raw.w[i >> 1].w : raw.w[i >> 1].y; }
-      word_tiny(lo, m);
-      word_tiny(hi, m);
-      *reinterpret_cast<float4*>(&s[k][4 * f]) = make_float4(word_lo(lo), word_hi(lo), word_lo(hi), word_hi(hi));
-    }
-  }
-  return words_tiny(m);
-}
+};
 
 // f32 -> signed 64-bit fixed point with 48 fractional bits: round to nearest even, saturate, NaN -> 0
 __device__ __forceinline__ long long fix48(float u) {
@@ -213,24 +260,31 @@ struct OgemmArgs {
 };
 enum { OG_LEAD = 1, OG_FILL = 2, OG_BACK = 4 };
 
-// Tile TM x TN, thread tile 8 x CT, LY lanes of a warp along the rows, ST ring slots, PF slabs in flight in the producers'
-// registers, CPS CTAs per SM; RC / RP: registers of a consumer / producer thread after the hand-over (0: none).
-template <int TM_, int TN_, int CT_, int LY_, int ST_, int PF_, int CPS_, int RC_, int RP_>
+// Tile TM x TN, thread tile 8 x CT, LY lanes of a warp along the rows, ST ring slots of HS slabs, PF slabs in flight in the producers'
+// registers, CPS CTAs per SM; RC / RP: registers of a consumer / producer thread after the hand-over (0: none); PAD: floats behind
+// each row of a slab (four instead of none are worth 2 % in every tile; with the 64-bit totals there is no room for them).
+// A hand-over costs a consumer some 35 instructions and, with one warp per scheduler, their latency; over HS slabs it is paid once.
+// Cycles per step of a CTA alone on its SM / multiply-adds per cycle and SM of a full GPU, by slabs per slot: 64 x 128 tiles 1: 103,
+// 97; 2: 97, 99; 4: 92, 102.  32 x 64 tiles 1: 67, 67; 2: 60, 76; 4: 52, 77.  128 x 128 tiles 1: 173, 97; 2: 170, 98; 3: 165, 99.  128 x 256
+// tiles 1 and 2: 302, 108.5; 4 in two slots 308, 105.
+template <int TM_, int TN_, int CT_, int LY_, int ST_, int PF_, int CPS_, int RC_, int RP_, int HS_, bool CARRY_ = false, int PAD_ = 4>
 struct OgTile {
-  static constexpr int TM = TM_, TN = TN_, CT = CT_, LY = LY_, ST = ST_, PF = PF_, CPS = CPS_, RC = RC_, RP = RP_;
+  static constexpr int TM = TM_, TN = TN_, CT = CT_, LY = LY_, ST = ST_, PF = PF_, CPS = CPS_, RC = RC_, RP = RP_, HS = HS_;
+  static constexpr int LA = TM + PAD_, LB = TN + PAD_;                    // floats of a slab row
+  static constexpr bool CARRY = CARRY_;
   static constexpr int CONS = (TM / 8) * (TN / CT), THREADS = CONS + OG_PROD;
-  static constexpr size_t SMEM = (size_t)ST * OK * (TM + 4 + TN + 4) * sizeof(float);
+  static constexpr size_t SMEM = (size_t)ST * HS * OK * (LA + LB) * sizeof(float);
   // what the block is launched with: 65536 registers over CPS blocks, in steps of eight a thread
   static_assert(RC == 0 || CONS * RC + OG_PROD * RP <= (65536 / (CPS * THREADS) / 8 * 8) * THREADS, "register hand-over exceeds the block's allocation");
 };
-// Measured at 2048 contraction steps on full GPUs (multiply-adds per cycle and SM, 128 is the pipe): 106, 103, 89, 61; one CTA
-// on each SM: 311, 174, 110, 71 cycles per step.  Some 30 cycles of every step are not multiply-adds whatever the tile, so
+// Measured at 2048 contraction steps on full GPUs (multiply-adds per cycle and SM, 128 is the pipe): 108.5, 107, 98, 76; one CTA
+// on each SM: 302, 165, 93, 56 cycles per step.  Some 20 to 40 cycles of every step are not multiply-adds whatever the tile, so
 // a smaller tile shortens a chain but never reaches the rate of a larger one.
-typedef OgTile<128, 256, 16, 2, 3, 1, 1, 216, 72> OgWide;
-typedef OgTile<128, 128, 16, 4, 3, 1, 2, 208, 48> OgSquare;
-typedef OgTile<64, 128, 8, 2, 4, 2, 2, 0, 0> OgHalf;
-typedef OgTile<32, 64, 4, 2, 6, 4, 4, 0, 0> OgSmall;
-typedef OgTile<64, 128, 8, 2, 3, 2, 2, 0, 0> OgFix;          // with 64 KiB of 64-bit accumulators beside the ring
+typedef OgTile<128, 256, 16, 2, 2, 1, 1, 216, 72, 2> OgWide;
+typedef OgTile<128, 128, 16, 4, 2, 1, 2, 208, 48, 3, true> OgSquare;
+typedef OgTile<64, 128, 8, 2, 2, 2, 2, 0, 0, 4> OgHalf;
+typedef OgTile<32, 64, 4, 2, 2, 4, 4, 0, 0, 4, true> OgSmall;
+typedef OgTile<64, 128, 8, 2, 2, 1, 2, 0, 0, 2, false, 0> OgFix;       // with 64 KiB of 64-bit accumulators beside the ring
 constexpr size_t OG_FIX_BYTES = (size_t)64 * 128 * 8;
 
 // Position of a consumer thread in the tile.  A 16-byte shared-memory load takes two cycles of the port when neighbouring
@@ -248,17 +302,18 @@ __device__ __forceinline__ void og_lane(int tid, int& ty, int& tx) {
 // shared-memory stores) into a ring of slabs.  Each ring slot has a "full" and an "empty" mbarrier: a producer warp arrives on
 // "full" after its stores, a consumer warp arrives on "empty" after its last read, and everybody only waits for the
 // other side, so consumer warps are not coupled to each other and the multiply pipe never waits for staging
-// instructions of its own warp.  All waits are bounded.
+// instructions of its own warp.  All waits are bounded.  A slot is handed over with HS slabs (first slots of 1
+// and 2 slabs, so that the multiplications start earlier, gained nothing).
 // FIX: the accumulators of a block of 128 contraction indices are converted (48 fractional bits) and added to 64-bit
 // totals after every block.  The totals lie in shared memory, one column per thread (no conflicts): kept in registers they
 // forced 128 x 128 tiles of one CTA per SM at 63 multiply-adds per cycle and SM, 72 this way (0.292 -> 0.245 ms at 16 x 4096, window 512).
 template <int AMODE, int BMODE, bool AF32, bool OUT_BF16, class T, bool FIX>
 __global__ void __launch_bounds__(T::THREADS, T::CPS) k_ogemm(const OgemmArgs p) {
-  constexpr int TM = T::TM, TN = T::TN, CT = T::CT, ST = T::ST, PF = T::PF;
+  constexpr int TM = T::TM, TN = T::TN, LA = T::LA, LB = T::LB, CT = T::CT, ST = T::ST, PF = T::PF, HS = T::HS;
   extern __shared__ __align__(16) unsigned char osm[];
-  float(*As)[OK][TM + 4] = reinterpret_cast<float(*)[OK][TM + 4]>(osm);
-  float(*Bs)[OK][TN + 4] = reinterpret_cast<float(*)[OK][TN + 4]>(osm + (size_t)ST * OK * (TM + 4) * sizeof(float));
-  __shared__ __align__(16) int tiny_s[ST][4];
+  float(*As)[OK][LA] = reinterpret_cast<float(*)[OK][LA]>(osm);
+  float(*Bs)[OK][LB] = reinterpret_cast<float(*)[OK][LB]>(osm + (size_t)ST * HS * OK * LA * sizeof(float));
+  __shared__ __align__(4) uint8_t tiny_s[ST][OG_PROD / 32];
   __shared__ __align__(8) uint64_t bar_full[ST], bar_empty[ST];
   __shared__ int abort_s;
   volatile int* abort_flag = &abort_s;
@@ -291,41 +346,54 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS) k_ogemm(const OgemmArgs p)
     // ------------------------------- producers -------------------------------
     if (T::RP) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(T::RP ? T::RP : 24));
     const int pt = tid - T::CONS, pw = pt >> 5;
-    const long long hA = zh * p.nG, hB = hA / p.b_div;
-    const char* A = reinterpret_cast<const char*>(p.A) + (zb * p.a_b + hA * p.a_h) * (AF32 ? 4 : 2);
-    const char* B = reinterpret_cast<const char*>(p.B) + (zb * p.b_b + hB * p.b_h) * 2;
-    OgRaw<AMODE, AF32, TM> ra[PF];
-    OgRaw<BMODE, false, TN> rb[PF];
-    int fetched = 0, c_next = c_lo;
+    typedef OgSide<AMODE, AF32, TM> SideA;
+    typedef OgSide<BMODE, false, TN> SideB;
+    const long long hA = zh * p.nG, hB = hA / p.b_div, stepA = (long long)p.lda * SideA::ESZ, stepB = (long long)p.ldb * SideB::ESZ;
+    SideA sa;
+    SideB sb;
+    sa.init(reinterpret_cast<const char*>(p.A) + (zb * p.a_b + hA * p.a_h) * SideA::ESZ, p.I, p.lda, i0, c_lo, pt);
+    sb.init(reinterpret_cast<const char*>(p.B) + (zb * p.b_b + hB * p.b_h) * SideB::ESZ, p.J, p.ldb, j0, c_lo, pt);
+    // from behind a head's last slab to the next head's first one
+    const long long turnA = p.a_h * SideA::ESZ - (long long)per_head * OK * (AMODE == STRIDED ? stepA : SideA::ESZ);
+    const long long turnB = p.b_h * SideB::ESZ - (long long)per_head * OK * (BMODE == STRIDED ? stepB : SideB::ESZ);
+    typename SideA::Raw ra[PF];
+    typename SideB::Raw rb[PF];
+    int fetched = 0, left = c_hi - c_lo;
     auto fetch = [&](int d) {
       if (fetched == nslab) return;
-      og_fetch<AMODE, AF32, TM>(A, p.I, c_hi, p.lda, i0, c_next, pt, ra[d]);
-      og_fetch<BMODE, false, TN>(B, p.J, c_hi, p.ldb, j0, c_next, pt, rb[d]);
+      sa.fetch(ra[d], left, stepA, pt);
+      sb.fetch(rb[d], left, stepB, pt);
       ++fetched;
-      c_next += OK;
-      if (c_next >= c_hi) {                                          // on to the next head of the group
-        c_next = c_lo;
-        A += p.a_h * (AF32 ? 4 : 2);
-        B += p.b_h * 2;
+      left -= OK;
+      if (left <= 0) {                                               // on to the next head of the group
+        left = c_hi - c_lo;
+        sa.skip(turnA);
+        sb.skip(turnB);
       }
     };
 #pragma unroll
     for (int d = 0; d < PF; ++d) fetch(d);
     int slot = 0;
-    uint32_t par = 1;
+    uint32_t par = 1, least = ~0u;
     for (int s0 = 0; s0 < nslab; s0 += PF) {
 #pragma unroll
       for (int d = 0; d < PF; ++d) {
         if (s0 + d >= nslab) return;
-        if (!mbar_wait(&bar_empty[slot], par, abort_flag, nullptr)) return;   // the consumers have left this slot
-        bool tiny = og_store<AMODE, AF32, TM>(As[slot], pt, ra[d]);
-        tiny |= og_store<BMODE, false, TN>(Bs[slot], pt, rb[d]);
+        const int sub = HS == 1 ? 0 : (s0 + d) % HS;
+        if (sub == 0) {
+          if (!mbar_wait(&bar_empty[slot], par, abort_flag, nullptr)) return;   // the consumers have left this slot
+          least = ~0u;
+        }
+        sa.store(As[slot * HS + sub], ra[d], least, pt);
+        sb.store(Bs[slot * HS + sub], rb[d], least, pt);
         fetch(d);                                                    // these words travel during the handshake
-        const int any = __any_sync(0xffffffffu, tiny);
-        if (lane == 0) tiny_s[slot][pw] = any;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bar_full[slot]);                 // slot is full (releases the warp's stores)
-        if (++slot == ST) { slot = 0; par ^= 1u; }
+        if (sub == HS - 1 || s0 + d == nslab - 1) {
+          const int any = __any_sync(0xffffffffu, least_tiny(least));
+          if (lane == 0) tiny_s[slot][pw] = (uint8_t)any;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bar_full[slot]);               // slot is full (releases the warp's stores)
+          if (++slot == ST) { slot = 0; par ^= 1u; }
+        }
       }
     }
     return;
@@ -366,10 +434,22 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS) k_ogemm(const OgemmArgs p)
   uint32_t par = 0;
   for (int s = 0; s < nslab; ++s) {
     if (!mbar_wait(&bar_full[slot], par, abort_flag, nullptr)) break;   // slot is full; after a wait that ran out the outputs are undefined
-    const int4 t4 = *reinterpret_cast<const int4*>(tiny_s[slot]);
-    if (t4.x | t4.y | t4.z | t4.w) slab_mac<false, TM, TN, CT>(As[slot], Bs[slot], ty, tx, acc);
-    else if constexpr (CT == 16) slab_mac_ordered<TM, TN>(As[slot], Bs[slot], ty, tx, acc);
-    else slab_mac<true, TM, TN, CT>(As[slot], Bs[slot], ty, tx, acc);
+    const bool tiny = *reinterpret_cast<const uint32_t*>(tiny_s[slot]) != 0;
+    if (T::CARRY && !tiny) {
+      const int n = min(HS, nslab - s);
+      slabs_ordered<true, TM, TN, CT>(As[slot * HS], Bs[slot * HS], n, ty, tx, acc);
+      s += n - 1;
+    } else {
+#pragma unroll 1
+      for (int sub = 0;; ++sub) {
+        const int at = slot * HS + sub;
+        if (tiny) slab_mac<false, TM, TN, CT>(As[at], Bs[at], ty, tx, acc);
+        else if constexpr (CT == 16) slabs_ordered<false, TM, TN, CT>(As[at], Bs[at], 1, ty, tx, acc);
+        else slab_mac<true, TM, TN, CT>(As[at], Bs[at], ty, tx, acc);
+        if (HS == 1 || sub == HS - 1 || s == nslab - 1) break;
+        ++s;
+      }
+    }
     __syncwarp();
     if (lane == 0) mbar_arrive(&bar_empty[slot]);                    // slot may be refilled
     if (++slot == ST) { slot = 0; par ^= 1u; }
@@ -425,7 +505,7 @@ static int ogemm_run(const OgemmArgs& p, int batches, cudaStream_t st) {
 // which falls with the tile (more operand loads per multiply).  Both are measured figures; the tile with the smaller
 // of the larger bounds is taken.
 struct OgRate { int tm, tn; float alone, full; };     // cycles per step of a CTA alone on its SM; multiply-adds per cycle and SM of a full one
-constexpr OgRate OG_RATES[4] = {{128, 256, 311.0f, 106.0f}, {128, 128, 174.0f, 103.0f}, {64, 128, 110.0f, 89.0f}, {32, 64, 71.0f, 61.0f}};
+constexpr OgRate OG_RATES[4] = {{128, 256, 302.0f, 108.5f}, {128, 128, 165.0f, 107.0f}, {64, 128, 93.0f, 98.0f}, {32, 64, 56.0f, 76.0f}};
 // share: how many such contractions run side by side; beside: SM-cycles of other work that is queued to fill the SMs that a small
 // grid leaves idle (the head's two gradients at 384 tokens: 96 CTAs of 64 x 128 and the weight gradient on the other SMs,
 // head and loss forward and backward 4.34 ms; 384 CTAs of 32 x 64 on all of them and the weight gradient behind, 5.27 ms)

@@ -94,6 +94,27 @@ def test_lmhead_every_tile(det, tile, M, V, K, tiny):
     assert_same_bits(host(dW), oracle.lmhead_bwd(g, H, W, dW_o)[1], "dW continued")
 
 
+# contraction lengths around a ring slot of two, three and four slabs of 16 and around the ring's two slots, the last slab of the weight gradient a
+# half one or whole; rows of which the last tile repeats most
+@pytest.mark.parametrize("tile", [0, 1, 2, 3])
+@pytest.mark.parametrize("C", [32, 48, 64, 80, 96, 112, 128, 144])
+def test_lmhead_slots_of_slabs(det, tile, C):
+    H, W = synth.normal_bf16((24, C), 1.0, seed=C, tid=1), synth.normal_bf16((C, C), 0.05, seed=C, tid=2)
+    g = synth.normal_f32((24, C), 1e-3, seed=C, tid=3)
+    lg, dH = empty((24, C), F), empty((24, C), np.uint16)
+    det.det_test_lmhead_tile(0, tile, dev(H), dev(W), 24, C, C, lg)
+    det.det_test_lmhead_tile(1, tile, dev(g), dev(W), 24, C, C, dH)
+    _sync()
+    assert_same_bits(host(lg), oracle.lmhead_fwd(H, W), "logits")
+    assert_same_bits(host(dH, np.uint16), oracle.lmhead_bwd(g, H, W)[0], "dH")
+    for M in (C - 8, C):
+        Hm, gm = synth.normal_bf16((M, 16), 1.0, seed=M, tid=4), synth.normal_f32((M, 32), 1e-3, seed=M, tid=5)
+        dW = empty((32, 16), F)
+        det.det_test_lmhead_tile(2, tile, dev(gm), dev(Hm), M, 32, 16, dW, 1)
+        _sync()
+        assert_same_bits(host(dW), oracle.lmhead_bwd(gm, Hm, synth.normal_bf16((32, 16), 0.05, seed=M, tid=6))[1], "dW")
+
+
 # version-2 gradients where a row of logits is long enough for eight warps (4096 values), and one step below; a token gradient of 36
 # tiles and 16 steps (two CTAs a tile, bf16 results), one of 80 (pairs, bf16 results); the 1B shape's vocabulary, an odd number of row
 # tiles for the weight gradient
