@@ -384,25 +384,35 @@ __global__ void __launch_bounds__(256) k_attn_delta(const uint16_t* __restrict__
 // Warp-specialised like the LM-head kernel: the CTA keeps q^T and dO^T of its query block in shared memory; four
 // producer warps stream the key and value blocks through a three-slot ring of 16-dimension slabs (a "full" and an
 // "empty" mbarrier per slot, bounded waits); eight consumer warps accumulate S = q.k^T and dP = dO.v^T together (two
-// 8 x 8 register tiles per thread, each logit one ascending sum over the 128 dimensions) and, per key block, apply
-// P = exp(S*scale - L) and dS = (P (dP - Delta)) scale and store bf16(P) and bf16(dS).  The producers already fetch
-// the next key block while the consumers are in that epilogue, and consumer warps are not coupled to each other.
+// 8 x 8 register tiles per thread, each logit one ascending sum over the 128 dimensions).  Per key block
+// P = exp(S*scale - L) and dS = (P (dP - Delta)) scale are formed and bf16(P) and bf16(dS) stored.  Consumer warps are not coupled to
+// each other.
+// EPI: that epilogue belongs to four more warps, and the 128 sums of a thread go to them through tensor memory, which is idle
+// otherwise (a store of four instructions; two buffers of 128 columns per consumer warp).  Two consumer warps on a scheduler fall
+// into step and left it idle during their epilogues, a latency-bound 12.5 of 52 thousand cycles a key block; now one multiplies on
+// while the exponentials fill the issue slots it leaves: 16 heads x 2048 0.453 -> 0.406 ms; the whole windowed attention (16 x 4096, forward and
+// backward) 1.380 -> 1.348 ms, two sequences of 8 x 1088 0.478 -> 0.460.  A fourth slot (1.381) and slots of two slabs (1.372) leave less of the
+// memory to the first-level cache and were slower.
+// Without EPI a consumer thread works on its own sums, which is the shorter way where a CTA has one key block.
 // Nothing is carried from one key block to the next, so the blocks of all heads are numbered (head, query block, key block) and
 // every CTA of a resident grid takes an equal run of them; where a run enters another query block the consumers stage its rows.
 // One query block per CTA, 4 x 16 heads x 2048 (query blocks of up to 16 key blocks, 1024 of them): 1.564 ms, equal runs 1.597; but
 // 16 x 4096 at window 512 0.545 and 0.478 ms, 2 x 8 x 1088 0.215 and 0.145, 8 x 1024 0.210 and 0.066, 16 x 832 0.166 and 0.099; 16 x 4096
 // 1.528, 1.547 and with the short runs at the end 1.526.
 // ---------------------------------------------------------------------------------------------
-// Rows per block (TM), ring slots, CTAs per SM, registers per consumer and producer thread.  A block of 128 rows takes 24.5 us, one
+// Rows per block (TM), ring slots, CTAs per SM, registers per consumer, producer and epilogue thread.  A block of 128 rows takes 24.5 us, one
 // of 64 rows 18.4 alone and 15.8 beside another; both 12 us for the launch, the first rows and the first slabs.
-template <int TM_, int SLOTS_, int CPS_, int RC_, int RP_>
+template <int TM_, int SLOTS_, int CPS_, int RC_, int RP_, int RE_ = 0>
 struct SdpTile {
-  static constexpr int TM = TM_, SLOTS = SLOTS_, CPS = CPS_, RC = RC_, RP = RP_;
-  static constexpr int CONS = TM * 2, THREADS = CONS + OG_PROD;
+  static constexpr int TM = TM_, SLOTS = SLOTS_, CPS = CPS_, RC = RC_, RP = RP_, RE = RE_;
+  static constexpr bool EPI = RE > 0;
+  static constexpr int CONS = TM * 2, THREADS = CONS + OG_PROD + (EPI ? 128 : 0);
+  static constexpr int COLS = CONS;                // tensor memory columns of a buffer: 128 for every four consumer warps
   static constexpr size_t SMEM = (size_t)(2 * DH * (TM + 4) + 2 * SLOTS * OK * (OT + 4)) * sizeof(float);
-  static_assert(CONS * RC + OG_PROD * RP <= (65536 / (CPS * THREADS) / 8 * 8) * THREADS, "register hand-over exceeds the block's allocation");
+  static_assert(CONS * RC + OG_PROD * RP + 128 * RE <= (65536 / (CPS * THREADS) / 8 * 8) * THREADS, "register hand-over exceeds the block's allocation");
+  static_assert(!EPI || (CPS == 1 && 2 * COLS <= 512), "two buffers in tensor memory");
 };
-typedef SdpTile<128, 3, 1, 216, 72> SdpTall;
+typedef SdpTile<128, 3, 1, 184, 56, 88> SdpTall;
 typedef SdpTile<64, 2, 2, 200, 56> SdpHalf;
 
 // named barrier of the first `threads` threads; the second form also tells whether any of them came with `x`
@@ -444,6 +454,77 @@ struct SdpAt {
   }
 };
 
+// P and dS of eight keys j0 + 64 g + 4 tx + 0 .. 3 (g = 0, 1) of row i from the sums s = q.k and d = dO.v; P and dS point to the row.
+// The argument of the exponential is at most 0 whenever L is the row's own logsumexp, and then the form without the overflow range
+// applies (same bits), but L is an input, so eight values that hold a positive argument take the general form.
+__device__ __forceinline__ void sdp_row(const float2 (&s)[4], const float2 (&d)[4], float L, float D, int i, int j0, int tx, int S, int W,
+                                        bool masked, float2 one, uint16_t* __restrict__ P, uint16_t* __restrict__ dS) {
+  const float2 L2 = same2(-L), D2 = same2(-D);
+  float2 x[4], pv[4], ds[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) x[t] = add2(mul2(s[t], same2(ATT_SCALE)), L2, one);
+  uint32_t vis = 0xff;
+  if (masked) {
+    vis = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int key = j0 + (e >> 2) * 64 + tx * 4 + (e & 3);
+      if (key <= i && (W == 0 || key > i - W)) vis |= 1u << e;
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) x[t] = make_float2(vis >> (2 * t) & 1 ? x[t].x : 0.0f, vis >> (2 * t + 1) & 1 ? x[t].y : 0.0f);
+  }
+  float top = x[0].x;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) top = fmaxf(top, fmaxf(x[t].x, x[t].y));
+  if (top > 0.0f) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) pv[t] = make_float2(det_exp(x[t].x), det_exp(x[t].y));
+  } else {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) pv[t] = det_exp_le0_2(x[t], one);
+  }
+#pragma unroll
+  for (int t = 0; t < 4; ++t) ds[t] = mul2(mul2(pv[t], add2(d[t], D2, one)), same2(ATT_SCALE));
+  if (masked) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      pv[t] = make_float2(vis >> (2 * t) & 1 ? pv[t].x : 0.0f, vis >> (2 * t + 1) & 1 ? pv[t].y : 0.0f);
+      ds[t] = make_float2(vis >> (2 * t) & 1 ? ds[t].x : 0.0f, vis >> (2 * t + 1) & 1 ? ds[t].y : 0.0f);
+    }
+  }
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
+    const int jb = j0 + g * 64 + tx * 4;
+    if (jb >= S) continue;
+    // P~ = bf16(P) is all the value gradient needs
+    *reinterpret_cast<uint2*>(P + jb) = make_uint2(pack_bf2(pv[2 * g].x, pv[2 * g].y), pack_bf2(pv[2 * g + 1].x, pv[2 * g + 1].y));
+    *reinterpret_cast<uint2*>(dS + jb) = make_uint2(pack_bf2(ds[2 * g].x, ds[2 * g].y), pack_bf2(ds[2 * g + 1].x, ds[2 * g + 1].y));
+  }
+}
+
+// two rows of a thread's sums, S and dP of each, to 32 columns of its lane
+__device__ __forceinline__ void tmem_st_rows(uint32_t taddr, const float2 (&s0)[4], const float2 (&d0)[4], const float2 (&s1)[4],
+                                             const float2 (&d1)[4]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
+      "f"(s0[0].x), "f"(s0[0].y), "f"(s0[1].x), "f"(s0[1].y), "f"(s0[2].x), "f"(s0[2].y), "f"(s0[3].x), "f"(s0[3].y),
+      "f"(d0[0].x), "f"(d0[0].y), "f"(d0[1].x), "f"(d0[1].y), "f"(d0[2].x), "f"(d0[2].y), "f"(d0[3].x), "f"(d0[3].y),
+      "f"(s1[0].x), "f"(s1[0].y), "f"(s1[1].x), "f"(s1[1].y), "f"(s1[2].x), "f"(s1[2].y), "f"(s1[3].x), "f"(s1[3].y),
+      "f"(d1[0].x), "f"(d1[0].y), "f"(d1[1].x), "f"(d1[1].y), "f"(d1[2].x), "f"(d1[2].y), "f"(d1[3].x), "f"(d1[3].y)
+      : "memory");
+}
+// the wait behind tmem_ld16_nowait, with the registers it is for
+__device__ __forceinline__ void tmem_wait_ld16(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]),
+                 "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
+
 template <class T>
 __global__ void __launch_bounds__(T::THREADS, T::CPS)
     k_attn_sdp(const uint16_t* __restrict__ dout, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k,
@@ -460,6 +541,8 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
   __shared__ __align__(4) uint8_t tiny_s[SDP_SLOTS][OG_PROD / 32];
   __shared__ int abort_s;
   __shared__ __align__(8) uint64_t bar_full[SDP_SLOTS], bar_empty[SDP_SLOTS];
+  __shared__ __align__(8) uint64_t sum_full[2][SDP_CONS / 32], sum_empty[2][SDP_CONS / 32];   // the sums of a consumer warp, per buffer
+  __shared__ uint32_t tmem_base_s;
   volatile int* abort_flag = &abort_s;
   const int tid = threadIdx.x, lane = tid & 31;
   int w_lo = 0, w_hi;
@@ -475,11 +558,73 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
   }
   if (tid == 0) {
     for (int s = 0; s < SDP_SLOTS; ++s) { mbar_init(&bar_full[s], OG_PROD / 32); mbar_init(&bar_empty[s], SDP_CONS / 32); }
+    for (int w = 0; w < SDP_CONS / 32; ++w)
+      for (int b = 0; b < 2; ++b) { mbar_init(&sum_full[b][w], 1); mbar_init(&sum_empty[b][w], 1); }
     abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (T::EPI && tid >> 5 == (SDP_CONS + OG_PROD) / 32) {   // first epilogue warp
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"((uint32_t)(2 * T::COLS)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (T::EPI) tc_fence_before();
   __syncthreads();
-  if (tid >= SDP_CONS) {
+  if (T::EPI) tc_fence_after();
+  // the sums of consumer warp w: lanes 32 (w % 4) .., columns 128 (w / 4) .. of a buffer; row a of a thread in columns 16 a ..
+  auto sums_at = [&](int w, int buf) { return tmem_base_s + ((uint32_t)(w & 3) << 21) + (uint32_t)(buf * T::COLS + (w >> 2) * 128); };
+  const float2 one = same2(c_one);
+  if (T::EPI && tid >= SDP_CONS + OG_PROD) {
+    // ------------------------------- epilogue -------------------------------
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(T::EPI ? T::RE : 24));
+    const int tx = lane >> 1;
+    int buf = 0;
+    uint32_t par = 0;
+    bool ok = true;
+    for (int blk = w_lo; blk < w_hi && ok; ++blk) {
+      const int i0 = at.i0, j0 = at.jt * OT;
+      const size_t r0 = (size_t)at.bh * S;
+      const bool masked = j0 + OT - 1 > i0 || (W > 0 && j0 <= i0 + TM - 1 - W);   // the block at the diagonal and those at the window's start
+#pragma unroll 1
+      for (int w = (tid >> 5) & 3; w < SDP_CONS / 32; w += 4) {
+        const int first = i0 + (w * 2 + (lane & 1)) * 4;               // rows first + 0 .. 3 and first + TM / 2 + 0 .. 3
+        // rows past the last one exist only where S is no multiple of TM: their L and Delta are never used
+        float L = first < S ? __ldg(lse + r0 + first) : 0.0f, D = first < S ? __ldg(delta + r0 + first) : 0.0f;
+        ok = __all_sync(0xffffffffu, mbar_wait(&sum_full[buf][w], par, abort_flag, nullptr));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t taddr = sums_at(w, buf);
+        uint32_t r[16];
+        tmem_ld16_nowait(taddr, r);
+        tmem_wait_ld16(r);
+#pragma unroll 1
+        for (int a = 0; a < 8; ++a) {
+          const int i = first + (a >> 2) * (TM / 2) + (a & 3);
+          float2 sv[4], dv[4];
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            sv[t] = make_float2(__uint_as_float(r[2 * t]), __uint_as_float(r[2 * t + 1]));
+            dv[t] = make_float2(__uint_as_float(r[8 + 2 * t]), __uint_as_float(r[9 + 2 * t]));
+          }
+          const float La = L, Da = D;
+          if (a < 7) {                                                  // the next row travels during this one's arithmetic
+            const int n = first + ((a + 1) >> 2) * (TM / 2) + ((a + 1) & 3);
+            tmem_ld16_nowait(taddr + 16 * (a + 1), r);
+            if (n < S) { L = __ldg(lse + r0 + n); D = __ldg(delta + r0 + n); }
+          }
+          if (i < S) sdp_row(sv, dv, La, Da, i, j0, tx, S, W, masked, one, Pb + (r0 + i) * S, dSt + (r0 + i) * S);
+          __syncwarp();
+          if (a < 7) tmem_wait_ld16(r);
+          if (a == 6) {                                                 // everything has been read
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sum_empty[buf][w]);
+          }
+        }
+      }
+      at.next(S, TM, W);
+      if ((buf ^= 1) == 0) par ^= 1u;
+    }
+  } else if (tid >= SDP_CONS) {
     // ------------------------------- producers -------------------------------
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(T::RP));
     const int pt = tid - SDP_CONS, pw = pt >> 5;
@@ -516,8 +661,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
       if (lane == 0) mbar_arrive(&bar_full[slot]);
       if (++slot == SDP_SLOTS) { slot = 0; par ^= 1u; }
     }
-    return;
-  }
+  } else {
   // --------------------------------- consumers ---------------------------------
   asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(T::RC));
   const int ty = (tid >> 5) * 2 + (tid & 1), tx = (lane >> 1);   // neighbouring lanes share their columns (see og_lane)
@@ -537,6 +681,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     }
 #pragma unroll
     for (int a = 0; a < 8; ++a) {
+      if (T::EPI) break;
       const int i = i0 + (a >> 2) * (TM / 2) + ty * 4 + (a & 3);
       Lr[a] = i < S ? lse[(size_t)bh * S + i] : 0.0f;
       Dr[a] = i < S ? delta[(size_t)bh * S + i] : 0.0f;
@@ -556,9 +701,8 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     }
     tqo = bar_or(1, SDP_CONS, tq);
   };
-  const float2 one = same2(c_one);
-  int slot = 0;
-  uint32_t par = 0;
+  int slot = 0, buf = 0;
+  uint32_t par = 0, spar = 1;
   bool ok = true;
   for (int w = w_lo; w < w_hi;) {
     const int i0 = at.i0, jt0 = at.jt, jt1 = min(jt0 + w_hi - w, i0 / OT + 1);
@@ -584,51 +728,36 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
         if (++slot == SDP_SLOTS) { slot = 0; par ^= 1u; }
       }
       if (!ok) break;
-      // P = exp(S*scale - L) and dS, two pairs at a time; the argument is at most 0 whenever L is the row's own logsumexp, and
-      // then the exponential without the overflow range applies (same bits), but L is an input, so four pairs that hold
-      // a positive argument take the general form.  Only the block at the diagonal and those at the window's start mask.
-      const bool masked = j0 + OT - 1 > i0 || (W > 0 && j0 <= i0 + TM - 1 - W);
+      if (T::EPI) {
+        const int w = tid >> 5;
+        ok = __all_sync(0xffffffffu, mbar_wait(&sum_empty[buf][w], spar, abort_flag, nullptr));   // two blocks ago has been read
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t taddr = sums_at(w, buf);
 #pragma unroll
-      for (int a = 0; a < 8; ++a) {
-        const int i = i0 + (a >> 2) * (TM / 2) + ty * 4 + (a & 3);
-        if (i >= S) continue;
-        const float2 L2 = same2(-Lr[a]), D2 = same2(-Dr[a]);
+        for (int a = 0; a < 8; a += 2) tmem_st_rows(taddr + 16 * a, sa[a], da[a], sa[a + 1], da[a + 1]);
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sum_full[buf][w]);
+        if ((buf ^= 1) == 0) spar ^= 1u;
+      } else {
+        const bool masked = j0 + OT - 1 > i0 || (W > 0 && j0 <= i0 + TM - 1 - W);   // the block at the diagonal and those at the window's start
 #pragma unroll
-        for (int g = 0; g < 2; ++g) {
-          const int jb = j0 + g * 64 + tx * 4;
-          if (jb >= S) continue;
-          float2 x[2], pv[2], ds[2];
-#pragma unroll
-          for (int t = 0; t < 2; ++t) x[t] = add2(mul2(sa[a][2 * g + t], same2(ATT_SCALE)), L2, one);
-          bool vis[4] = {true, true, true, true};
-          if (masked) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) vis[e] = jb + e <= i && (W == 0 || jb + e > i - W);
-            x[0] = make_float2(vis[0] ? x[0].x : 0.0f, vis[1] ? x[0].y : 0.0f);
-            x[1] = make_float2(vis[2] ? x[1].x : 0.0f, vis[3] ? x[1].y : 0.0f);
-          }
-          if (x[0].x > 0.0f || x[0].y > 0.0f || x[1].x > 0.0f || x[1].y > 0.0f) {
-#pragma unroll
-            for (int t = 0; t < 2; ++t) pv[t] = make_float2(det_exp(x[t].x), det_exp(x[t].y));
-          } else {
-#pragma unroll
-            for (int t = 0; t < 2; ++t) pv[t] = det_exp_le0_2(x[t], one);
-          }
-#pragma unroll
-          for (int t = 0; t < 2; ++t) ds[t] = mul2(mul2(pv[t], add2(da[a][2 * g + t], D2, one)), same2(ATT_SCALE));
-          if (masked) {
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-              pv[t] = make_float2(vis[2 * t] ? pv[t].x : 0.0f, vis[2 * t + 1] ? pv[t].y : 0.0f);
-              ds[t] = make_float2(vis[2 * t] ? ds[t].x : 0.0f, vis[2 * t + 1] ? ds[t].y : 0.0f);
-            }
-          }
-          const size_t off = (bh * S + i) * S + jb;
-          // P~ = bf16(P) is all the value gradient needs
-          *reinterpret_cast<uint2*>(Pb + off) = make_uint2(pack_bf2(pv[0].x, pv[0].y), pack_bf2(pv[1].x, pv[1].y));
-          *reinterpret_cast<uint2*>(dSt + off) = make_uint2(pack_bf2(ds[0].x, ds[0].y), pack_bf2(ds[1].x, ds[1].y));
+        for (int a = 0; a < 8; ++a) {
+          const int i = i0 + (a >> 2) * (TM / 2) + ty * 4 + (a & 3);
+          if (i < S) sdp_row(sa[a], da[a], Lr[a], Dr[a], i, j0, tx, S, W, masked, one, Pb + (bh * S + i) * S, dSt + (bh * S + i) * S);
         }
       }
+    }
+  }
+  }
+  if (T::EPI) {
+    tc_fence_before();
+    __syncthreads();
+    if (tid >> 5 == (SDP_CONS + OG_PROD) / 32) {
+      tc_fence_after();
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base_s), "r"((uint32_t)(2 * T::COLS)) : "memory");
     }
   }
 }
