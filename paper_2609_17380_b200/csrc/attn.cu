@@ -40,18 +40,23 @@ namespace det {
 // sums and rescale factors to group 0, which alone forms o and l, in block order.  Two groups shorten the chain, 13 to 9.9 us per
 // key block, and lose rate (9.8 against 7.5 us per 32 rows and key block): 8 heads x 1024 0.119 ms with 32 rows, 0.088 with two groups;
 // 16 x 832 0.119 and 0.117; two sequences of 8 x 1088 0.167 and 0.189.
+// Slabs of a ring slot.  The kernel is bound by issue slots (twice the packed multiply-adds plus all other instructions come to 98 % of the
+// cycles), and a hand-over takes a consumer warp some 70 of them: one for two slabs instead of one a slab, waited for where it is needed
+// instead of a slab ahead, with two keys a store in the producers (see OgSide) took 16 heads x 832 from 116 to 107 us.
+constexpr int AF_HS = 2;
 template <int FQ_, int SLOTS_, int PF_, int CPS_, int RC_, int RP_, int GR_ = 1>
 struct AfTile {
   static constexpr int FQ = FQ_, LQ = FQ_ + 4, SLOTS = SLOTS_, PF = PF_, CPS = CPS_, RC = RC_, RP = RP_, GR = GR_;
   static constexpr int GCONS = (FQ / AF_RW) * 32, CONS = GR * GCONS, THREADS = CONS + GR * AF_PROD;
-  static constexpr size_t SMEM = (size_t)(DH * LQ + GR * (FK * FQ + SLOTS * OK * AF_BP) + (GR - 1) * FQ * DH) * sizeof(float);
+  static constexpr size_t SMEM = (size_t)(DH * LQ + GR * (FK * FQ + SLOTS * AF_HS * OK * AF_BP) + (GR - 1) * FQ * DH) * sizeof(float);
+  static_assert(FQ % (AF_HS * OK) == 0, "the last slot of value rows is whole");
   // setmaxnreg: the counts after the hand-over must fit into what the block was launched with, or the increase never returns
   static_assert(CONS * RC + GR * AF_PROD * RP <= (65536 / (CPS * THREADS) / 8 * 8) * THREADS, "register hand-over exceeds the block's allocation");
 };
-typedef AfTile<128, 8, 4, 1, 104, 64> AfTall;
-typedef AfTile<64, 4, 2, 2, 96, 48> AfHalf;
-typedef AfTile<32, 4, 3, 3, 104, 56> AfShort;
-typedef AfTile<32, 4, 3, 1, 136, 64, 2> AfPair;
+typedef AfTile<128, 4, 4, 1, 104, 64> AfTall;
+typedef AfTile<64, 2, 2, 2, 96, 48> AfHalf;
+typedef AfTile<32, 2, 3, 3, 104, 56> AfShort;
+typedef AfTile<32, 2, 3, 1, 136, 64, 2> AfPair;
 
 template <class T, bool WIN>
 __global__ void __launch_bounds__(T::THREADS, T::CPS)
@@ -63,7 +68,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
   const int W = WIN ? Warg : 0;
   extern __shared__ __align__(16) float sm[];
   float(*Qs)[LQ] = reinterpret_cast<float(*)[LQ]>(sm);                         // [dim][query]
-  __shared__ __align__(16) int tiny_g[GR][AF_SLOTS][AF_PROD / 32];
+  __shared__ __align__(4) uint8_t tiny_g[GR][AF_SLOTS][AF_PROD / 32];
   __shared__ int tiny_q_s, abort_s;
   __shared__ __align__(8) uint64_t full_g[GR][AF_SLOTS], empty_g[GR][AF_SLOTS];
   // between the two groups, per warp: maxima passed on by either, group 1's sums and factors, "u is there", "u has been read"
@@ -81,16 +86,16 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
   const int tid = threadIdx.x, lane = tid & 31;
   const int grp = GR == 1 ? 0 : (tid < AF_CONS ? tid / T::GCONS : (tid - AF_CONS) / AF_PROD), warp = (tid >> 5) - grp * GWARPS;   // consumers' warp
   float* Ps = sm + DH * LQ + grp * (FK * FQ);                                  // [key][query], 16-byte chunks swizzled
-  float(*Ring)[OK][AF_BP] = reinterpret_cast<float(*)[OK][AF_BP]>(sm + DH * LQ + GR * FK * FQ) + grp * AF_SLOTS;
-  float4* U = reinterpret_cast<float4*>(sm + DH * LQ + GR * (FK * FQ + AF_SLOTS * OK * AF_BP));   // [4][thread of the group]
-  int(*tiny_s)[AF_PROD / 32] = tiny_g[grp];
+  float(*Ring)[OK][AF_BP] = reinterpret_cast<float(*)[OK][AF_BP]>(sm + DH * LQ + GR * FK * FQ) + grp * (AF_SLOTS * AF_HS);
+  float4* U = reinterpret_cast<float4*>(sm + DH * LQ + GR * (FK * FQ + AF_SLOTS * AF_HS * OK * AF_BP));   // [4][thread of the group]
+  uint8_t(*tiny_s)[AF_PROD / 32] = tiny_g[grp];
   uint64_t *bar_full = full_g[grp], *bar_empty = empty_g[grp];
   const size_t row0 = (size_t)b * S;
   const uint16_t* qp = q + row0 * ld + (size_t)h * DH;
   const uint16_t* kp = k + row0 * ld + (size_t)hk * DH;
   const uint16_t* vp = v + row0 * ld + (size_t)hk * DH;
   const int jt0 = ((WIN && q0 > W) ? (q0 - W) / FK : 0) + grp, ntiles = q0 / FK + 1;   // this group's first block
-  // the last block ends with the last slab of 16 value rows that the CTA's last query may see
+  // the last block ends with the last slab of 16 value rows that the CTA's last query may see, and with that a slot (FQ % 32 = 0)
   const int mine = ntiles > jt0 ? (ntiles - jt0 + GR - 1) / GR : 0;
   const int nslab = mine * 16 - ((ntiles - 1 - jt0) % GR == 0 && mine ? 7 - (q0 % FK + FQ - 1) / OK : 0);
   if (tid == 0) {
@@ -123,64 +128,82 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     // ------------------------------- producers -------------------------------
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(T::RP));
     const int pt = (tid - AF_CONS) % AF_PROD, pw = pt >> 5;
-    // Slab s of the block sequence: block s / 16; s % 16 < 8: K, head dimensions 16 (s % 16) .. (thread = key, two
-    // 16-byte words); else V, keys 16 (s % 16 - 8) .. (thread = four dimensions of keys kk, kk + 4, kk + 8, kk + 12).
+    // Slab s of the block sequence: block s / 16; s % 16 < 8: K, head dimensions 16 (s % 16) .. (thread = eight of them, of two
+    // neighbouring keys); else V, keys 16 (s % 16 - 8) .. (thread = four dimensions of keys kk, kk + 4, kk + 8, kk + 12).
     // AF_PF slabs are in flight in registers, so that the latency of a global load is spread over several slabs.
     // Both kinds are two 16-byte words per thread, so one register array holds whichever kind slab s is.
     uint4 raw[AF_PF][2];
     const int vf = pt & 31, vk = pt >> 5;            // V: dimensions 4 vf .. 4 vf + 3 of keys vk, vk + 4, vk + 8, vk + 12
+    const int kk = 2 * (pt & 63), kd = (pt >> 6) * 8;   // K: keys kk and kk + 1, dimensions kd .. kd + 7 of the slab
+    const size_t row = (size_t)ld * 2;
+    // keys past the last one repeat it: they are never visible.  ksrc, vsrc: this thread's words of the block's first slab
+    const char *ksrc0, *ksrc1, *vsrc;
+    int vleft;                                       // keys of the sequence from the thread's first one on
+    auto block = [&](int j0n) {
+      ksrc0 = reinterpret_cast<const char*>(kp + kd) + min(j0n + kk, S - 1) * row;
+      ksrc1 = reinterpret_cast<const char*>(kp + kd) + min(j0n + kk + 1, S - 1) * row;
+      vsrc = reinterpret_cast<const char*>(vp + 4 * vf) + (j0n + vk) * row;
+      vleft = S - (j0n + vk);
+    };
+    block(jt0 * FK);
     auto fetch = [&](int sn, uint4 (&w)[2]) {
       if (sn >= nslab) return;
-      const int j0n = (jt0 + GR * (sn >> 4)) * FK, phn = sn & 15;
+      const int phn = sn & 15;
+      if (phn == 0 && sn) block((jt0 + GR * (sn >> 4)) * FK);
       if (phn < 8) {
-        const int key = j0n + pt;
-        const uint4* src = reinterpret_cast<const uint4*>(kp + (size_t)key * ld + phn * OK);
-        const bool in = key < S;
-        w[0] = in ? __ldg(src) : make_uint4(0u, 0u, 0u, 0u);
-        w[1] = in ? __ldg(src + 1) : make_uint4(0u, 0u, 0u, 0u);
+        w[0] = __ldg(reinterpret_cast<const uint4*>(ksrc0));
+        w[1] = __ldg(reinterpret_cast<const uint4*>(ksrc1));
+        ksrc0 += 2 * OK;
+        ksrc1 += 2 * OK;
       } else {
-        const int key0 = j0n + (phn - 8) * OK + vk;
         uint2 u[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const int key = key0 + 4 * i;
-          u[i] = key < S ? __ldg(reinterpret_cast<const uint2*>(vp + (size_t)key * ld + 4 * vf)) : make_uint2(0u, 0u);
+          u[i] = 4 * i < vleft ? __ldg(reinterpret_cast<const uint2*>(vsrc)) : make_uint2(0u, 0u);
+          vsrc += 4 * row;
         }
+        vleft -= OK;
         w[0] = make_uint4(u[0].x, u[0].y, u[1].x, u[1].y);
         w[1] = make_uint4(u[2].x, u[2].y, u[3].x, u[3].y);
       }
     };
-    // unpack, test for factors below 2^-63 and store: K as [dimension][key] (thread = key), V as [key][dimension]
-    const int kcol = (pt & 4 ? AF_HI : 0) + (pt >> 3) * 4 + (pt & 3), vcol = 4 * vf + (vf >= 16 ? AF_HI - 64 : 0);
-    auto store = [&](int ph, float (*dst)[AF_BP], const uint4 (&w)[2]) -> bool {
-      uint32_t tiny = 0;
+    // unpack, test for factors below 2^-63 and store: K as [dimension][key], two keys at a time, V as [key][dimension]
+    const int kcol = (kk & 4 ? AF_HI : 0) + (kk >> 3) * 4 + (kk & 3), vcol = 4 * vf + (vf >= 16 ? AF_HI - 64 : 0);
+    auto store = [&](int ph, float (*dst)[AF_BP], const uint4 (&w)[2], uint32_t& least) {
       const uint32_t words[8] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w};
 #pragma unroll
-      for (int i = 0; i < 8; ++i) word_tiny(words[i], tiny);
+      for (int i = 0; i < 8; ++i) word_least(words[i], least);
       if (ph < 8) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) { dst[2 * i][kcol] = word_lo(words[i]); dst[2 * i + 1][kcol] = word_hi(words[i]); }
+        for (int i = 0; i < 4; ++i) {
+          *reinterpret_cast<float2*>(&dst[kd + 2 * i][kcol]) = make_float2(word_lo(words[i]), word_lo(words[4 + i]));
+          *reinterpret_cast<float2*>(&dst[kd + 2 * i + 1][kcol]) = make_float2(word_hi(words[i]), word_hi(words[4 + i]));
+        }
       } else {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
           *reinterpret_cast<float4*>(&dst[vk + 4 * i][vcol]) =
               make_float4(word_lo(words[2 * i]), word_hi(words[2 * i]), word_lo(words[2 * i + 1]), word_hi(words[2 * i + 1]));
       }
-      return words_tiny(tiny);
     };
 #pragma unroll
     for (int d = 0; d < AF_PF; ++d) fetch(d, raw[d]);
     int slot = 0;
-    uint32_t par = 1;
+    uint32_t par = 1, least = ~0u;
     for (int s0 = 0; s0 < nslab; s0 += AF_PF) {
 #pragma unroll
       for (int d = 0; d < AF_PF; ++d) {
-        const int s = s0 + d;
-        if (s >= nslab || !mbar_wait(&bar_empty[slot], par, abort_flag, nullptr)) return;
-        const bool tiny = store(s & 15, Ring[slot], raw[d]);
+        const int s = s0 + d, sub = s % AF_HS;
+        if (s >= nslab) return;
+        if (sub == 0) {
+          if (!mbar_wait(&bar_empty[slot], par, abort_flag, nullptr)) return;
+          least = ~0u;
+        }
+        store(s & 15, Ring[slot * AF_HS + sub], raw[d], least);
         fetch(s + AF_PF, raw[d]);
-        const int any = __any_sync(0xffffffffu, tiny);
-        if (lane == 0) tiny_s[slot][pw] = any;
+        if (sub < AF_HS - 1) continue;
+        const int any = __any_sync(0xffffffffu, least_tiny(least));
+        if (lane == 0) tiny_s[slot][pw] = (uint8_t)any;
         __syncwarp();
         if (lane == 0) mbar_arrive(&bar_full[slot]);
         if (++slot == AF_SLOTS) { slot = 0; par ^= 1u; }
@@ -201,24 +224,19 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
 #pragma unroll
     for (int j = 0; j < 4; ++j) o[i][j] = make_float2(0.0f, 0.0f);
   bool ok = true;
-  // the next slab is waited for (and its below-2^-63 flags fetched) one slab ahead of its use
-  int tiny_cur = 0, slot = 0, nslot = 0, left = nslab;
-  uint32_t npar = 0;
-  auto acquire = [&]() -> bool {
-    if (left == 0) return true;
-    --left;
-    if (!mbar_wait(&bar_full[nslot], npar, abort_flag, nullptr)) return false;
-    const int4 t4 = *reinterpret_cast<const int4*>(tiny_s[nslot]);
-    tiny_cur = t4.x | t4.y | t4.z | t4.w;
-    if (++nslot == AF_SLOTS) { nslot = 0; npar ^= 1u; }
+  int slot = 0;
+  uint32_t par = 0;
+  // the next slot is full: its below-2^-63 flags
+  auto acquire = [&](bool& tiny) -> bool {
+    if (!mbar_wait(&bar_full[slot], par, abort_flag, nullptr)) return false;
+    tiny = *reinterpret_cast<const uint32_t*>(tiny_s[slot]) != 0;
     return true;
   };
   auto release = [&]() {
     __syncwarp();
     if (lane == 0) mbar_arrive(&bar_empty[slot]);
-    if (++slot == AF_SLOTS) slot = 0;
+    if (++slot == AF_SLOTS) { slot = 0; par ^= 1u; }
   };
-  ok = acquire();
   // o = o * alpha + u and l = l * alpha + sum of group 1's block of round `rd`
   auto take = [&](int rd) -> bool {
     if (!__all_sync(0xffffffffu, mbar_wait(&bar_u[warp], (uint32_t)rd & 1u, abort_flag, nullptr))) return false;
@@ -247,12 +265,16 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
-    for (int sl = 0; sl < 8; ++sl) {
-      const int tiny = tiny_q | tiny_cur;
-      if (!acquire()) { ok = false; break; }          // the next slab's flags travel while this one is multiplied
-      const float* ap = &Qs[sl * OK][lrow];
-      if (tiny) mac_4x8<false, false>(ap, LQ, 0, 0, Ring[slot], tx, acc);
-      else mac_4x8<true, false>(ap, LQ, 0, 0, Ring[slot], tx, acc);
+    for (int sl = 0; sl < 8; sl += AF_HS) {
+      bool tiny;
+      if (!acquire(tiny)) { ok = false; break; }
+      tiny |= tiny_q != 0;
+#pragma unroll 1
+      for (int sub = 0; sub < AF_HS; ++sub) {
+        const float* ap = &Qs[(sl + sub) * OK][lrow];
+        if (tiny) mac_4x8<false, false>(ap, LQ, 0, 0, Ring[slot * AF_HS + sub], tx, acc);
+        else mac_4x8<true, false>(ap, LQ, 0, 0, Ring[slot * AF_HS + sub], tx, acc);
+      }
       release();
     }
     if (!ok) break;
@@ -298,13 +320,15 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
       for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
     // on the diagonal the warp's rows see no key beyond its last row, the CTA's none beyond its own last row
     const int last_slab = diag ? (q0 - j0 + wrow + AF_RW - 1) / OK : 7, last_block = diag ? (q0 - j0 + FQ - 1) / OK : 7;
-    for (int sl = 0; sl <= last_block; ++sl) {
-      const int tiny = tiny_p | tiny_cur;
-      if (!acquire()) { ok = false; break; }
-      if (sl <= last_slab) {
-        const float* ap = Ps + (size_t)(sl * OK) * FQ;
-        if (tiny) mac_4x8<false, true>(ap, FQ, lrow >> 2, sl * OK, Ring[slot], tx, acc);
-        else mac_4x8<true, true>(ap, FQ, lrow >> 2, sl * OK, Ring[slot], tx, acc);
+    for (int sl = 0; sl <= last_block; sl += AF_HS) {
+      bool tiny;
+      if (!acquire(tiny)) { ok = false; break; }
+      tiny |= tiny_p != 0;
+#pragma unroll 1
+      for (int sub = 0; sub < AF_HS && sl + sub <= last_slab; ++sub) {
+        const float* ap = Ps + (size_t)((sl + sub) * OK) * FQ;
+        if (tiny) mac_4x8<false, true>(ap, FQ, lrow >> 2, sub * OK, Ring[slot * AF_HS + sub], tx, acc);
+        else mac_4x8<true, true>(ap, FQ, lrow >> 2, sub * OK, Ring[slot * AF_HS + sub], tx, acc);
       }
       release();
     }
