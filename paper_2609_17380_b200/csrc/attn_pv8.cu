@@ -23,10 +23,10 @@
 
 namespace det {
 
-constexpr int PQ = 128, PK = 128, PLQ = PQ + 4, PV_SLOTS = 8;
+constexpr int PQ = 128, PK = 128, PLQ = PQ + 4, PV_SLOTS = 4, PV_HS = 2;   // ring slots, 16-deep slabs of a slot
 constexpr int PV_CONS = 512, PV_PROD = 128, PV_THREADS = PV_CONS + PV_PROD;
 // shared memory: Q f32 [dim][query], the slab ring, then (1024-byte aligned) q_p int8 [query][key], q_v int8 [2][dim][key]
-constexpr size_t PV8_SMEM = (size_t)(DH * PLQ + PV_SLOTS * OK * AF_BP) * sizeof(float) + 1024 + 3 * PQ * PK;
+constexpr size_t PV8_SMEM = (size_t)(DH * PLQ + PV_SLOTS * PV_HS * OK * AF_BP) * sizeof(float) + 1024 + 3 * PQ * PK;
 // setmaxnreg: 104 registers for consumers, 64 for producers
 static_assert(PV_CONS * 104 + PV_PROD * 64 <= (65536 / PV_THREADS / 8 * 8) * PV_THREADS, "register hand-over exceeds the block's allocation");
 
@@ -41,11 +41,11 @@ __global__ void __launch_bounds__(PV_THREADS, 1)
   float(*Qs)[PLQ] = reinterpret_cast<float(*)[PLQ]>(psm8);
   float(*Ring)[OK][AF_BP] = reinterpret_cast<float(*)[OK][AF_BP]>(psm8 + (size_t)DH * PLQ * sizeof(float));
   uint8_t* ops = reinterpret_cast<uint8_t*>(
-      (reinterpret_cast<uintptr_t>(psm8 + (size_t)(DH * PLQ + PV_SLOTS * OK * AF_BP) * sizeof(float)) + 1023) & ~(uintptr_t)1023);
+      (reinterpret_cast<uintptr_t>(psm8 + (size_t)(DH * PLQ + PV_SLOTS * PV_HS * OK * AF_BP) * sizeof(float)) + 1023) & ~(uintptr_t)1023);
   int8_t* Pq = reinterpret_cast<int8_t*>(ops);              // A operand: [query][key]
   int8_t* Vq = reinterpret_cast<int8_t*>(ops + PQ * PK);    // B operand: two buffers [dim][key]
   __shared__ float alpha_s[2][PQ], l_s[PQ], cs_s[4], vmax_s[2][4];
-  __shared__ __align__(16) int tiny_s[PV_SLOTS][4];
+  __shared__ __align__(4) uint8_t tiny_s[PV_SLOTS][4];
   __shared__ int tiny_q_s, abort_s;
   __shared__ uint32_t tmem_base_s;
   __shared__ __align__(8) uint64_t bar_full[PV_SLOTS], bar_empty[PV_SLOTS], bar_p, bar_v[2], bar_mma;
@@ -101,7 +101,8 @@ __global__ void __launch_bounds__(PV_THREADS, 1)
     // ------------------------------- producers -------------------------------
     asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
     const int pt = tid - PV_CONS, pw = pt >> 5;
-    const int kcol = (pt & 4 ? AF_HI : 0) + (pt >> 3) * 4 + (pt & 3);
+    const int kk = 2 * (pt & 63), kd = (pt >> 6) * 8;   // K: keys kk and kk + 1 of a block, dimensions kd .. kd + 7 of a slab
+    const int kcol = (kk & 4 ? AF_HI : 0) + (kk >> 3) * 4 + (kk & 3);
     int slot = 0;
     uint32_t par = 1;
     bool ok = true;                                  // after a failed wait nothing is staged, but every barrier below is still met
@@ -119,33 +120,37 @@ __global__ void __launch_bounds__(PV_THREADS, 1)
     };
     for (int t = 0; t < nt; ++t) {
       const int j0 = (jt0 + t) * PK;
-      {  // K: slab sl holds head dimensions 16 sl .. of the 128 keys (thread = key), four slabs in flight
-        const bool in = j0 + pt < S;
-        const uint4* src = reinterpret_cast<const uint4*>(kp + (size_t)(j0 + pt) * ld);
+      {  // K: slab sl holds head dimensions 16 sl .. of the 128 keys, four slabs in flight; keys past the last one repeat it, they are never visible
+        const uint4* src0 = reinterpret_cast<const uint4*>(kp + (size_t)min(j0 + kk, S - 1) * ld + kd);
+        const uint4* src1 = reinterpret_cast<const uint4*>(kp + (size_t)min(j0 + kk + 1, S - 1) * ld + kd);
         uint4 raw[4][2];
-        auto fetch = [&](int sl, uint4 (&w)[2]) {
-          w[0] = in ? __ldg(src + 2 * sl) : make_uint4(0u, 0u, 0u, 0u);
-          w[1] = in ? __ldg(src + 2 * sl + 1) : make_uint4(0u, 0u, 0u, 0u);
-        };
+        auto fetch = [&](int sl, uint4 (&w)[2]) { w[0] = __ldg(src0 + 2 * sl); w[1] = __ldg(src1 + 2 * sl); };
 #pragma unroll
         for (int d = 0; d < 4; ++d) fetch(d, raw[d]);
+        uint32_t least = ~0u;
 #pragma unroll
         for (int sl = 0; sl < 8; ++sl) {
-          ok = ok && mbar_wait(&bar_empty[slot], par, abort_flag, status);
+          const int sub = sl % PV_HS;
+          if (sub == 0) {
+            ok = ok && mbar_wait(&bar_empty[slot], par, abort_flag, status);
+            least = ~0u;
+          }
           const uint4 w0 = raw[sl & 3][0], w1 = raw[sl & 3][1];
           const uint32_t words[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-          uint32_t tw = 0;
           if (ok) {
+            float(*dst)[AF_BP] = Ring[slot * PV_HS + sub];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              word_tiny(words[i], tw);
-              Ring[slot][2 * i][kcol] = word_lo(words[i]);
-              Ring[slot][2 * i + 1][kcol] = word_hi(words[i]);
+            for (int i = 0; i < 4; ++i) {
+              word_least(words[i], least);
+              word_least(words[4 + i], least);
+              *reinterpret_cast<float2*>(&dst[kd + 2 * i][kcol]) = make_float2(word_lo(words[i]), word_lo(words[4 + i]));
+              *reinterpret_cast<float2*>(&dst[kd + 2 * i + 1][kcol]) = make_float2(word_hi(words[i]), word_hi(words[4 + i]));
             }
           }
           if (sl < 4) fetch(sl + 4, raw[sl & 3]);
-          const int any = __any_sync(0xffffffffu, words_tiny(tw));
-          if (lane == 0) { tiny_s[slot][pw] = any; }
+          if (sub < PV_HS - 1) continue;
+          const int any = __any_sync(0xffffffffu, least_tiny(least));
+          if (lane == 0) { tiny_s[slot][pw] = (uint8_t)any; }
           __syncwarp();
           if (lane == 0) mbar_arrive(&bar_full[slot]);
           if (++slot == PV_SLOTS) { slot = 0; par ^= 1u; }
@@ -245,12 +250,15 @@ __global__ void __launch_bounds__(PV_THREADS, 1)
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
-      for (int sl = 0; sl < 8; ++sl) {
+      for (int sl = 0; sl < 8; sl += PV_HS) {
         if (!mbar_wait(&bar_full[slot], par, abort_flag, status)) { ok = false; break; }
-        const int4 t4 = *reinterpret_cast<const int4*>(tiny_s[slot]);
-        const float* ap = &Qs[sl * OK][lrow];
-        if (tiny_q | t4.x | t4.y | t4.z | t4.w) mac_4x8<false, false>(ap, PLQ, 0, 0, Ring[slot], tx, acc);
-        else mac_4x8<true, false>(ap, PLQ, 0, 0, Ring[slot], tx, acc);
+        const bool tiny = tiny_q != 0 || *reinterpret_cast<const uint32_t*>(tiny_s[slot]) != 0;
+#pragma unroll 1
+        for (int sub = 0; sub < PV_HS; ++sub) {
+          const float* ap = &Qs[(sl + sub) * OK][lrow];
+          if (tiny) mac_4x8<false, false>(ap, PLQ, 0, 0, Ring[slot * PV_HS + sub], tx, acc);
+          else mac_4x8<true, false>(ap, PLQ, 0, 0, Ring[slot * PV_HS + sub], tx, acc);
+        }
         __syncwarp();
         if (lane == 0) mbar_arrive(&bar_empty[slot]);
         if (++slot == PV_SLOTS) { slot = 0; par ^= 1u; }
