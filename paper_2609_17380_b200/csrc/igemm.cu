@@ -173,10 +173,32 @@ __device__ __forceinline__ void epi_row(const EpiParams& ep, uint32_t taddr, int
   }
 }
 
-template <int BN, int EPI>
-__global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
-    k_igemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, EpiParams ep, int I, int J,
-            int K, int* status, int fill) {
+// A product of a launch that has two of them, with the same columns J
+struct IgProduct {
+  CUtensorMap a, b;
+  EpiParams ep;
+  int I, K;
+};
+// The tiles of CTA `b` of `g`, one after the other.  Those of the second product (n1) come behind those of the first (n0), and the
+// CTAs that have one tile of the first less take `lead` tiles of the second while the others are at it.
+struct IgWalk {
+  int n0, n1, b, g, lead;
+  __device__ __forceinline__ bool tile(int it, int& job, int& at) const {
+    job = 0;
+    at = b + it * g;
+    if (at < n0) return true;
+    if (n1 == 0) return false;
+    const int own = b < n0 ? (n0 - b + g - 1) / g : 0, rest = n0 % g, mine = b >= rest ? lead : 0;
+    job = 1;
+    it -= own;
+    at = it < mine ? it * (g - rest) + b - rest : lead * (g - rest) + (it - mine) * g + b;
+    return at < n1;
+  }
+};
+
+template <int BN, int EPI, int EPI2>
+__device__ __forceinline__ void ig_body(const CUtensorMap& tmA, const CUtensorMap& tmB, const EpiParams& ep, int I, int J, int K,
+                                        int* status, int fill, const IgProduct* second, int lead) {
   constexpr int STAGE_A = BM * BK, STAGE_B = BN * BK, STAGE_BYTES = STAGE_A + STAGE_B;
   constexpr int STAGES = IgTile<BN>::STAGES, EW = IgTile<BN>::EW, CW = IgTile<BN>::CW;
   extern __shared__ uint8_t smem_raw[];
@@ -208,24 +230,26 @@ __global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
   if (fill) grid_fill_begin();
   else grid_dep();
 
-  const int tiles_i = I / BM, tiles_j = J / BN;
-  const int num_tiles = tiles_i * tiles_j;
-  const int kblocks = K / BK;
+  constexpr bool TWO = EPI2 >= 0;
+  const int tiles_j = J / BN, tiles_i[2] = {I / BM, TWO ? second->I / BM : 0}, kblocks[2] = {K / BK, TWO ? second->K / BK : 0};
+  const IgWalk walk = {tiles_i[0] * tiles_j, tiles_i[1] * tiles_j, (int)blockIdx.x, (int)gridDim.x, lead};
 
   if (warp == 0) {
     if (lane == 0) {
-      int stage = 0;
+      int stage = 0, job, tile;
       uint32_t phase = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+      for (int it = 0; ok && walk.tile(it, job, tile); ++it) {
+        const bool w = TWO && job;
         int i0, j0;
-        tile_origin(tile, tiles_i, tiles_j, BN, i0, j0);
-        for (int kb = 0; kb < kblocks; ++kb) {
+        tile_origin(tile, w ? tiles_i[1] : tiles_i[0], tiles_j, BN, i0, j0);
+        const CUtensorMap *ma = w ? &second->a : &tmA, *mb = w ? &second->b : &tmB;
+        for (int kb = 0, nk = w ? kblocks[1] : kblocks[0]; kb < nk; ++kb) {
           if (!mbar_wait(&bar_empty[stage], phase ^ 1u, abort_flag, status)) { ok = false; break; }
           mbar_expect_tx(&bar_full[stage], STAGE_BYTES);
           uint8_t* sa = smem + stage * STAGE_BYTES;
-          tma_load_2d(sa, &tmA, kb * BK, i0, &bar_full[stage]);
-          tma_load_2d(sa + STAGE_A, &tmB, kb * BK, j0, &bar_full[stage]);
+          tma_load_2d(sa, ma, kb * BK, i0, &bar_full[stage]);
+          tma_load_2d(sa + STAGE_A, mb, kb * BK, j0, &bar_full[stage]);
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
@@ -234,17 +258,16 @@ __global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
     if (lane == 0) {
       // instruction descriptor: D = S32, A = B = signed 8-bit, both K-major, N = BN, M = 128
       constexpr uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-      int stage = 0;
+      int stage = 0, job, tile;
       uint32_t phase = 0;
-      int it = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++it) {
+      for (int it = 0; ok && walk.tile(it, job, tile); ++it) {
         const int acc = it & 1;
         const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
         if (!mbar_wait(&bar_tempty[acc], acc_phase ^ 1u, abort_flag, status)) { ok = false; break; }
         tc_fence_after();
         const uint32_t tmem_d = tmem_base + (uint32_t)(acc * BN);
-        for (int kb = 0; kb < kblocks; ++kb) {
+        for (int kb = 0, nk = TWO && job ? kblocks[1] : kblocks[0]; kb < nk; ++kb) {
           if (!mbar_wait(&bar_full[stage], phase, abort_flag, status)) { ok = false; break; }
           tc_fence_after();
           const uint32_t sa = smem_u32(smem + stage * STAGE_BYTES);
@@ -261,19 +284,22 @@ __global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
   } else {
     const int q = warp & 3, part = (warp - 2) >> 2;  // TMEM lane quarter this warp may read; its share of the columns
     uint8_t* stage = smem + STAGES * STAGE_BYTES + (warp - 2) * 4096;  // this warp's 32 x 128-byte staging tile
-    int it = 0;
+    int job, tile;
     bool ok = true;
-    float cscale, inv_s, sx;
+    float cscale, inv_s, sx, cscale2 = 1.0f, inv_s2 = 1.0f, sx2 = 1.0f;
     epi_scalars<EPI>(ep, cscale, inv_s, sx);
-    for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++it) {
+    if constexpr (TWO) epi_scalars<EPI2>(second->ep, cscale2, inv_s2, sx2);
+    for (int it = 0; ok && walk.tile(it, job, tile); ++it) {
       const int acc = it & 1;
       const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
       int i0, j0;
-        tile_origin(tile, tiles_i, tiles_j, BN, i0, j0);
+      tile_origin(tile, TWO && job ? tiles_i[1] : tiles_i[0], tiles_j, BN, i0, j0);
       if (!mbar_wait(&bar_tfull[acc], acc_phase, abort_flag, status)) { ok = false; break; }
       tc_fence_after();
-      epi_row<CW, EPI>(ep, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + part * CW), i0 + q * 32 + lane, J,
-                       j0 + part * CW, cscale, inv_s, sx, stage);
+      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + part * CW);
+      if (!TWO || !job) epi_row<CW, EPI>(ep, taddr, i0 + q * 32 + lane, J, j0 + part * CW, cscale, inv_s, sx, stage);
+      if constexpr (TWO)
+        if (job) epi_row<CW, EPI2>(second->ep, taddr, i0 + q * 32 + lane, J, j0 + part * CW, cscale2, inv_s2, sx2, stage);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar_tempty[acc]);
@@ -292,6 +318,18 @@ __global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)IgTile<BN>::TCOLS) : "memory");
   }
   if (fill) grid_fill_end();
+}
+template <int BN, int EPI>
+__global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
+    k_igemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, EpiParams ep, int I, int J, int K,
+            int* status, int fill) {
+  ig_body<BN, EPI, -1>(tmA, tmB, ep, I, J, K, status, fill, nullptr, 0);
+}
+// both gradient products of a linear layer, dX [M, K] over N and dW [N, K] over M, `p` before `s`
+template <int BN, bool W_FIRST>
+__global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
+    k_igemm_grads(const __grid_constant__ IgProduct p, const __grid_constant__ IgProduct s, int J, int* status, int lead) {
+  ig_body<BN, W_FIRST ? EPI_DW : EPI_DX, W_FIRST ? EPI_DX : EPI_DW>(p.a, p.b, p.ep, p.I, J, p.K, status, 0, &s, lead);
 }
 
 // ------------------------------------------------------------------------------------------------------------
@@ -315,7 +353,7 @@ constexpr int GEMM2_THREADS = 64 + 8 * 32;
 template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     k_igemm2(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, EpiParams ep, int I, int J,
-             int K, int* status, int fill) {
+             int K, int* status) {
   constexpr int STAGE_A = 128 * BK, STAGE_B = 128 * BK, STAGE_BYTES = STAGE_A + STAGE_B;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -346,8 +384,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
   cluster_sync_all();  // the peer's barriers are initialised before anything can signal them
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
-  if (fill) grid_fill_begin();
-  else grid_dep();
+  grid_dep();
 
   const int tiles_i = I / 256, tiles_j = J / BN2;
   const int num_tiles = tiles_i * tiles_j;
@@ -436,7 +473,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
   }
-  if (fill) grid_fill_end();
 }
 
 // ---- host side -------------------------------------------------------------------------------
@@ -483,7 +519,7 @@ static int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const EpiPar
 
 template <int EPI>
 static int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const EpiParams& ep, int I, int J, int K, int* status,
-                       cudaStream_t st, int fill) {
+                       cudaStream_t st) {
   constexpr size_t smem = (size_t)STAGES2 * (2 * 128 * BK) + 8 * 4096 + 1024;
   static DevOnce once = {};
   if (dev_ensure_smem(once, (const void*)k_igemm2<EPI>, smem) != DET_OK) return DET_ERR_CUDA;
@@ -492,7 +528,7 @@ static int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const EpiPa
   const int tiles = (I / 256) * (J / BN2);
   int clusters = sms / 2;
   if (tiles < clusters) clusters = tiles;
-  launch_after(k_igemm2<EPI>, 2 * clusters, GEMM2_THREADS, smem, st, ta, tb, ep, I, J, K, status, fill);
+  launch_after(k_igemm2<EPI>, 2 * clusters, GEMM2_THREADS, smem, st, ta, tb, ep, I, J, K, status);
   if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return DET_ERR_CUDA; }
   return DET_OK;
 }
@@ -503,21 +539,27 @@ static int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const EpiPa
 // narrow tile shortens and spreads over more SMs (1024 x 1024 x 1024: 11.1, 10.6, 8.5, 8.5 forward and 16.7, 15.3, 12.6, 10.5
 // input gradient for 256 x 256 pairs and 256, 128, 64 columns); over many rounds the pairs run a few percent faster
 // than their rounds say (16384 x 2048 x 8192: 166, 171, 265, 520), over few of them the 256-column tiles of one CTA.
-// Returns the columns of a one-CTA tile, or 512 for the CTA pair (256 x 256).
-static int igemm_pick(int epi, int I, int J, int K, int force_one_cta) {
+// Returns the columns of a one-CTA tile, or 512 for the CTA pair (256 x 256); *work: its time on a full GPU without the last round's loss.
+struct IgCost { int bn, bi, bj, pair; double step, turn, epi[4]; };               // epi: RAW, FWD, DX, DW
+constexpr IgCost IG_COST[4] = {{512, 256, 256, 1, 0.365, 0.9, {6.6, 4.2, 10.0, 6.6}}, {256, 128, 256, 0, 0.375, 0.5, {8.4, 4.0, 9.3, 6.2}},
+                               {128, 128, 128, 0, 0.30, 0.5, {3.8, 1.7, 5.7, 3.8}}, {64, 128, 64, 0, 0.30, 0.5, {1.8, 1.7, 3.7, 1.8}}};
+static int igemm_pick(int epi, int I, int J, int K, int force_one_cta, double* work = nullptr) {
   const int sms = dev_sm_count() > 0 ? dev_sm_count() : 1;
-  struct { int bn, bi, bj, units; double step, turn, epi[4]; } const c[4] = {     // epi: RAW, FWD, DX, DW
-      {512, 256, 256, sms / 2, 0.365, 0.9, {6.6, 4.2, 10.0, 6.6}}, {256, 128, 256, sms, 0.375, 0.5, {8.4, 4.0, 9.3, 6.2}},
-      {128, 128, 128, sms, 0.30, 0.5, {3.8, 1.7, 5.7, 3.8}}, {64, 128, 64, sms, 0.30, 0.5, {1.8, 1.7, 3.7, 1.8}}};
+  const IgCost* c = IG_COST;
   int best = 0;
   double best_t = 0.0;
   for (int i = force_one_cta ? 1 : 0; i < 4; ++i) {
-    if (I % c[i].bi || J % c[i].bj || !c[i].units) continue;
-    const long long tiles = (long long)(I / c[i].bi) * (J / c[i].bj), rounds = (tiles + c[i].units - 1) / c[i].units;
+    const int units = c[i].pair ? sms / 2 : sms;
+    if (I % c[i].bi || J % c[i].bj || !units) continue;
+    const long long tiles = (long long)(I / c[i].bi) * (J / c[i].bj), rounds = (tiles + units - 1) / units;
     const double loop = (K / BK) * c[i].step, e = c[i].epi[epi];
     double t = rounds * ((loop > e ? loop : e) + c[i].turn) + (loop > e ? e : loop);
     if (c[i].bn == 512 && rounds >= 6) t *= 0.95;
-    if (!best || t < best_t) { best = c[i].bn; best_t = t; }
+    if (!best || t < best_t) {
+      best = c[i].bn;
+      best_t = t;
+      if (work) *work = tiles * ((loop > e ? loop : e) + c[i].turn) / units;
+    }
   }
   return best;
 }
@@ -525,7 +567,7 @@ template <int EPI>
 static int igemm_tile(int bn, const CUtensorMap& ta, const CUtensorMap& tb, const EpiParams& ep, int I, int J, int K, int* status,
                       cudaStream_t st, int fill) {
   switch (bn) {
-    case 512: return launch_pair<EPI>(ta, tb, ep, I, J, K, status, st, fill);
+    case 512: return launch_pair<EPI>(ta, tb, ep, I, J, K, status, st);
     case 256: return launch_one<256, EPI>(ta, tb, ep, I, J, K, status, st, fill);
     case 128: return launch_one<128, EPI>(ta, tb, ep, I, J, K, status, st, fill);
     default: return launch_one<64, EPI>(ta, tb, ep, I, J, K, status, st, fill);
@@ -537,7 +579,7 @@ int igemm_launch(int epi, const int8_t* A, const int8_t* B, int I, int J, int K,
   if (I % BM || J % 128 || K % BK) return DET_ERR_SHAPE;
   if (K >= (1 << 17)) return DET_ERR_RANGE;
   if (!aligned16(A) || !aligned16(B)) return DET_ERR_ALIGN;
-  const int bn = igemm_pick(epi, I, J, K, force_one_cta);
+  const int bn = igemm_pick(epi, I, J, K, force_one_cta || fill);
   CUtensorMap ta, tb;
   if (!make_map(&ta, A, I, K, 128) || !make_map(&tb, B, J, K, bn == 512 ? 128 : bn)) return DET_ERR_CUDA;
   switch (epi) {
@@ -547,6 +589,68 @@ int igemm_launch(int epi, const int8_t* A, const int8_t* B, int I, int J, int K,
     case EPI_DW: return igemm_tile<EPI_DW>(bn, ta, tb, ep, I, J, K, status, st, fill);
   }
   return DET_ERR_ARG;
+}
+
+template <int BN>
+static int grads_tile(bool w_first, const IgProduct& p, const IgProduct& s, int J, int grid, int lead, int* status, cudaStream_t st) {
+  typedef IgTile<BN> T;
+  static DevOnce once[2] = {};
+  const auto kern = w_first ? k_igemm_grads<BN, true> : k_igemm_grads<BN, false>;
+  if (dev_ensure_smem(once[w_first], (const void*)kern, T::SMEM) != DET_OK) return DET_ERR_CUDA;
+  launch_after(kern, grid, T::THREADS, T::SMEM, st, p, s, J, status, lead);
+  if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return DET_ERR_CUDA; }
+  return DET_OK;
+}
+// Both gradient products in one launch, *did, instead of two, the larger ones of which go through a fork to another stream and a join.  The
+// product with the longer tiles comes first; the time of a tile width is that of the CTA that has most to do, and it may exceed
+// the work of the two, each with its own best width, by what two launches and their last rounds lose.  Whole input passes, tokens, rows and columns,
+// microseconds, two launches and one: 512 x 512 x 512 18.5 and 17.3, 1024 x 1024 x 1024 26.1 and 21.8, 1024 x 5632 x 1024 52.3 and 46.0,
+// 6144 x 640 x 1280 62.4 and 58.6, 8192 x 256 x 2048 87.4 and 81.2.  Two launches stay the better ones where one width costs more than that
+// (1024 x 1024 x 2816 34.9 and 35.5, 3200 x 1152 x 256 31.3 and 32.0), where the work is long (128 x 16384 x 4096 151 and 155) and where the
+// sum of the step gradient is (4096 x 256 x 8192 117 and 128: it runs beside the weight gradient).
+int igemm_grads_launch(const int8_t* A, const int8_t* Ut, const EpiParams& ex, const int8_t* Gt, const int8_t* Zt, const EpiParams& ew,
+                       int M, int N, int K, int* status, cudaStream_t st, bool* did) {
+  *did = false;
+  const int sms = dev_sm_count();
+  if (sms <= 0) return DET_ERR_CUDA;
+  double work[2] = {};
+  if (igemm_pick(EPI_DX, M, K, N, 0, &work[0]) == 512 || igemm_pick(EPI_DW, N, K, M, 0, &work[1]) == 512) return DET_OK;
+  int bn = 0, lead = 0, grid = 0;
+  bool w_first = false;
+  double best = 0.0;
+  for (int i = 1; i < 4; ++i) {
+    const IgCost& c = IG_COST[i];
+    if (K % c.bn) continue;
+    const double loop[2] = {(N / BK) * c.step, (M / BK) * c.step}, epi[2] = {c.epi[EPI_DX], c.epi[EPI_DW]};
+    const int tiles[2] = {(M / BM) * (K / c.bn), (N / BM) * (K / c.bn)};
+    double each[2];
+    for (int k = 0; k < 2; ++k) each[k] = (loop[k] > epi[k] ? loop[k] : epi[k]) + c.turn;
+    const int f = each[1] > each[0], g = tiles[0] + tiles[1] < sms ? tiles[0] + tiles[1] : sms;    // f: the first product
+    const int rest = tiles[f] % g, spare = g - rest, n = tiles[1 - f];
+    int l = 0;
+    if (rest) {
+      l = (int)(each[f] / each[1 - f] + 0.5);
+      if (l > (n + spare - 1) / spare) l = (n + spare - 1) / spare;
+    }
+    const int left = n > l * spare ? n - l * spare : 0;
+    const double part = rest ? (each[f] > l * each[1 - f] ? each[f] : l * each[1 - f]) : 0.0;
+    const double tail = loop[1 - f] < epi[1 - f] ? loop[1 - f] : epi[1 - f];
+    const double t = (tiles[f] / g) * each[f] + part + ((left + g - 1) / g) * each[1 - f] + tail;
+    if (!bn || t < best) { bn = c.bn; best = t; lead = l; grid = g; w_first = f; }
+  }
+  if (best > work[0] + work[1] + 5.5 || work[0] + work[1] > 50.0 || (long long)M * (K / 64) > 16ll * 16384) return DET_OK;
+  IgProduct x = {}, w = {};
+  if (!make_map(&x.a, A, M, N, 128) || !make_map(&x.b, Ut, K, N, bn) || !make_map(&w.a, Gt, N, M, 128) || !make_map(&w.b, Zt, K, M, bn))
+    return DET_ERR_CUDA;
+  x.ep = ex; x.I = M; x.K = N;
+  w.ep = ew; w.I = N; w.K = M;
+  *did = true;
+  const IgProduct &p = w_first ? w : x, &s = w_first ? x : w;
+  switch (bn) {
+    case 256: return grads_tile<256>(w_first, p, s, K, grid, lead, status, st);
+    case 128: return grads_tile<128>(w_first, p, s, K, grid, lead, status, st);
+    default: return grads_tile<64>(w_first, p, s, K, grid, lead, status, st);
+  }
 }
 
 }  // namespace det

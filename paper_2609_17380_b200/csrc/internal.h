@@ -81,10 +81,14 @@ int dev_ensure_smem(DevOnce& once, const void* fn, size_t bytes);  // DET_OK or 
 int dev_sm_count();                                                 // SMs of the current device (0 on error)
 
 // C[i,j] = sum_k A[i,k] B[j,k] on the tensor cores with the chosen epilogue; host-side checks included
-// fill != 0: this product does not depend on the kernel before it on the stream and takes the SMs that one leaves (common.cuh)
+// fill != 0: this product does not depend on the kernel before it on the stream and takes the SMs that one leaves (common.cuh); one-CTA kernel
 // force_one_cta != 0 keeps the one-CTA kernel even where the two-CTA tiles would apply (the results are identical)
 int igemm_launch(int epi, const int8_t* A, const int8_t* B, int I, int J, int K, const EpiParams& ep, int* status,
                  cudaStream_t st, int force_one_cta = 0, int fill = 0);
+
+// dX [M,K] = A [M,N] . (Ut [K,N])^T and dW [N,K] = Gt [N,M] . (Zt [K,M])^T in one launch; *did: whether the sizes are for that
+int igemm_grads_launch(const int8_t* A, const int8_t* Ut, const EpiParams& ex, const int8_t* Gt, const int8_t* Zt, const EpiParams& ew,
+                       int M, int N, int K, int* status, cudaStream_t st, bool* did);
 
 // Sliced (arithmetic version 2) contractions: out = round(I 2^(Ea + Eb - 280)) from the int8 slices of both operands,
 // Z problems per launch (lmhead_v2.cu).

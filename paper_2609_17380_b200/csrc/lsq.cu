@@ -691,23 +691,29 @@ extern "C" int det_linear_bwd(const det_bf16* dY, const det_bf16* X, const int8_
   // grad wrt x: [M,K] = A_q [M,N] . (U_q^T [K,N])^T
   EpiParams ex = {};
   ex.out = dX; ex.s_x = s_x; ex.amax1 = amax + 0; ex.s_u = s_u; ex.ref = X; ex.rot = rotf; ex.ds_partial = partial;
-  // The two products are independent.  Small ones stay on one stream, the second filling the SMs that the first leaves: a fork and a
-  // join cost more than the sum of the step gradient behind them (256 tokens, 512 -> 512, forward and backward: 29.9 against 27.4 us).  Large ones are persistent
-  // grids whose blocks leave as their tiles run out; the weight gradient, on an auxiliary stream, moves onto the SMs that the
-  // last partial round of the input gradient leaves idle, and the sum does not wait for it.
   const size_t np = (size_t)M * (K / 64);
   const float gs = (float)(1.0 / sqrt((double)M * (double)K * 127.0));
+  // The two products are independent: one launch where igemm_grads_launch says so.  Of the others, small ones stay on one stream, the
+  // second filling the SMs that the first leaves: a fork and a join cost more than the sum of the step gradient behind them (512 tokens,
+  // 256 -> 2944, backward: 26.8 against 25.1 us, 25.7 in one launch).  Large ones are persistent grids whose blocks leave as their tiles
+  // run out; the weight gradient, on an auxiliary stream, moves onto the SMs that the last partial round of the input
+  // gradient leaves idle, and the sum does not wait for it.
+  bool both;
+  int rc = igemm_grads_launch(Aq, qWt_bwd, ex, GqT, ZqT, ew, M, N, K, status_dev, st, &both);
+  if (rc != DET_OK) return rc;
   const bool small = (long long)(M / 128 + N / 128) * (K / 128) <= dev_sm_count();
-  if (small) {
-    int rc = igemm_launch(EPI_DX, Aq, qWt_bwd, M, K, N, ex, status_dev, st);
-    if (rc == DET_OK) rc = igemm_launch(EPI_DW, GqT, ZqT, N, K, M, ew, status_dev, st, 0, 1);
+  if (!both && small) {
+    rc = igemm_launch(EPI_DX, Aq, qWt_bwd, M, K, N, ex, status_dev, st);
+    if (rc == DET_OK) rc = igemm_launch(EPI_DW, GqT, ZqT, N, K, M, ew, status_dev, st, 1, 1);
     if (rc != DET_OK) return rc;
+  }
+  if (both || small) {
     sum_scaled_launch(partial, np, gs, ds_x, sscr, st);
     DET_CHECK_LAUNCH();
     return DET_OK;
   }
   AuxScope aux(st);   // joined again on every way out
-  int rc = igemm_launch(EPI_DX, Aq, qWt_bwd, M, K, N, ex, status_dev, st);
+  rc = igemm_launch(EPI_DX, Aq, qWt_bwd, M, K, N, ex, status_dev, st);
   if (rc == DET_OK) rc = igemm_launch(EPI_DW, GqT, ZqT, N, K, M, ew, status_dev, aux.aux(0));
   if (rc != DET_OK) return rc;
   sum_scaled_launch(partial, np, gs, ds_x, sscr, st);

@@ -366,6 +366,30 @@ def test_linear_tiles(det, M, N, K):
     assert_same_bits(host(gs), ods, "ds_x")
 
 
+# the two gradient products of a linear in one launch: one tile each, either product first, CTAs with and without a tile of the first one, widths
+# that only 64 columns divide, with and without the rotation; and in two launches on either side of the rule
+@pytest.mark.parametrize("M,N,K,hb", [(128, 128, 128, 128), (2048, 128, 128, 0), (1280, 1408, 384, 128), (640, 384, 896, 0), (1536, 1408, 640, 128),
+                                      (1920, 896, 256, 128), (512, 2944, 256, 128), (3968, 128, 256, 0)])
+def test_linear_gradients_together(det, M, N, K, hb):
+    import torch
+    X, W = synth.normal_bf16((M, K), 1.0, seed=N, tid=1), synth.normal_bf16((N, K), 0.02, seed=N, tid=2)
+    dY = synth.normal_bf16((M, N), 0.01, seed=N, tid=3)
+    sw, sx = oracle.lsq_weight_scale(W), oracle.lsq_act_scale_init(X)
+    odX, odW, ods = oracle.linear_bwd(dY, X, W, sx, sw, hb=hb)
+    dX_, dW_, s_w, s_x = dev(X), dev(W), dev(sw), dev(sx)
+    qW, qWt, s_u = empty((N, K), np.int8), empty((K, N), np.int8), empty((1,), F)
+    det.det_lsq_quantize_weight(dW_, s_w, N, K, hb, qW, qWt, s_u, ws(det.det_lsq_quantize_weight_ws_bytes(N, K)))
+    Y, qX, status = empty((M, N), np.uint16), empty((M, K), np.int8), torch.zeros(1, dtype=torch.int32, device="cuda")
+    det.det_linear_fwd(dX_, qW, s_x, s_w, M, N, K, Y, qX, status)
+    gX, gW, gs = empty((M, K), np.uint16), empty((N, K), F), empty((1,), F)
+    det.det_linear_bwd(dev(dY), dX_, qX, dW_, qWt, s_x, s_w, s_u, M, N, K, hb, gX, gW, gs, ws(det.det_linear_bwd_ws_bytes(M, N, K)), status)
+    _sync()
+    assert int(status.item()) == 0
+    assert_same_bits(host(gX, np.uint16), odX, "dX")
+    assert_same_bits(host(gW), odW, "dW")
+    assert_same_bits(host(gs), ods, "ds_x")
+
+
 # the norms with the residual stream beside them: rows off the block of eight, D off the leaf of 256, with and without codes
 @pytest.mark.parametrize("rows,D,q", [(1, 8, True), (13, 1000, False), (300, 2048, True), (64, 384, True), (21, 256, True), (22, 512, False),
                                       (23, 1024, True), (9, 1032, True), (515, 200, False)])
