@@ -8,6 +8,7 @@
 // Backward: P = exp(S*scale - L) recomputed; every one of the five contractions (S, dP, dV, dK, dQ) is a batched
 // ordered contraction with one sequential accumulator per output (ogemm_core.cuh); bf16(P) and bf16(dS) go through
 // global scratch, so nothing is accumulated with atomics.
+#include <math.h>
 #include "attn_core.cuh"
 
 namespace det {
@@ -809,13 +810,13 @@ static int attn_fwd_run(const det_bf16* q, const det_bf16* k, const det_bf16* v,
 }
 // Rows per CTA: the longest chain of key blocks runs on one SM whatever the others do, and all chains together share the GPU; the
 // figures are the microseconds per key block of a CTA alone on its SM and of one among many, the CTAs per SM, and the part of a
-// chain by which the shared time is exceeded in the end, nothing while long and short rows are paired on the SMs (two CTAs each,
-// none left over).  The row count with the smallest of the larger bounds is taken: 64 heads x 2048 1.49 ms with 128 rows, 1.57
-// with 64, 1.77 with 32; 20 heads x 1024 0.201, 0.199, 0.170; two sequences of 8 heads x 1088 0.226, 0.157, 0.167, two groups 0.189;
-// 16 heads x 832 0.176, 0.123, 0.119, 0.117; 8 heads x 1024 0.201, 0.140, 0.118, 0.088.
-struct RowCost { int rows; double alone, full; int cps; double over; };   // rows: 33 for 32 rows with two groups
+// chain by which the shared time is exceeded in the end, which shrinks with the rounds of CTAs over the GPU's places; nothing while long and
+// short rows are paired on the SMs (two CTAs each, none left over).  The row count with the smallest of the larger bounds is taken.
+// Measured with 128, 64, 32 rows and two groups: 64 heads x 2048 1447, 1500, 1624, 2056 us; 48 x 832 246, 216, 228, 297; 20 x 1024 197, 190,
+// 170, 183; 16 x 1088 220, 145, 153, 166; 16 x 832 171, 115, 108, 103; 8 x 1024 197, 128, 101, 79.
+struct RowCost { int rows; double alone, full; int cps; double over, decay; };   // rows: 33 for 32 rows with two groups
 static int attn_rows(int heads, int S, int window) {
-  const RowCost c[4] = {{128, 25.1, 25.1, 1, 0.0}, {64, 17.0, 13.2, 2, 0.5}, {32, 13.0, 7.5, 3, 0.25}, {33, 9.9, 9.8, 1, 0.25}};
+  const RowCost c[4] = {{128, 24.1, 24.6, 1, 0.3, 1.5}, {64, 15.5, 12.6, 2, 0.55, 2.0}, {32, 10.4, 6.9, 3, 0.5, 1.5}, {33, 8.75, 8.75, 1, 0.15, 0.0}};
   const int sms = dev_sm_count() > 0 ? dev_sm_count() : 1;
   int best = c[0].rows;
   double best_t = 0.0;
@@ -828,8 +829,11 @@ static int attn_rows(int heads, int S, int window) {
       total += tiles;
       if (tiles > longest) longest = tiles;
     }
-    const bool paired = c[i].cps == 2 && (long long)heads * ((S + step - 1) / step) <= 2 * sms;
-    const double a = longest * c[i].alone, b = total * heads * c[i].full / sms + (paired ? 0.0 : c[i].over * a), t = a > b ? a : b;
+    const double rounds = (double)heads * ((S + step - 1) / step) / ((double)c[i].cps * sms);
+    const double over = rounds > 1.0 ? c[i].over * pow(rounds, -c[i].decay) : (c[i].cps == 2 ? 0.0 : c[i].over);
+    const double a = longest * c[i].alone, b = total * heads * c[i].full / sms + over * a;
+    // a window's edge is one more block with masks for a few rows, which the two groups feel most (8 x 1024, window 256: 79, 56, 58, 64 us)
+    const double t = (a > b ? a : b) * (window && i == 3 ? 1.2 : 1.0);
     if (i == 0 || t < 0.97 * best_t) { best = c[i].rows; best_t = t; }
   }
   return best;
