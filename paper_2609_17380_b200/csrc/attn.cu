@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(256) k_attn_delta(const uint16_t* __restrict__
 // while the exponentials fill the issue slots it leaves: 16 heads x 2048 0.453 -> 0.406 ms; the whole windowed attention (16 x 4096, forward and
 // backward) 1.380 -> 1.348 ms, two sequences of 8 x 1088 0.478 -> 0.460.  A fourth slot (1.381) and slots of two slabs (1.372) leave less of the
 // memory to the first-level cache and were slower.
-// Without EPI a consumer thread works on its own sums, which is the shorter way where a CTA has one key block.
+// Without EPI a consumer thread works on its own sums, which is the shorter way where a CTA has a key block or two.
 // Nothing is carried from one key block to the next, so the blocks of all heads are numbered (head, query block, key block) and
 // every CTA of a resident grid takes an equal run of them; where a run enters another query block the consumers stage its rows.
 // One query block per CTA, 4 x 16 heads x 2048 (query blocks of up to 16 key blocks, 1024 of them): 1.564 ms, equal runs 1.597; but
@@ -438,6 +438,7 @@ struct SdpTile {
   static_assert(!EPI || (CPS == 1 && 2 * COLS <= 512), "two buffers in tensor memory");
 };
 typedef SdpTile<128, 3, 1, 184, 56, 88> SdpTall;
+typedef SdpTile<128, 3, 1, 216, 72> SdpLone;
 typedef SdpTile<64, 2, 2, 200, 56> SdpHalf;
 
 // named barrier of the first `threads` threads; the second form also tells whether any of them came with `x`
@@ -925,7 +926,9 @@ static int attn_bwd_impl(const det_bf16* dout, const det_bf16* q, const det_bf16
   // P[i,j] = exp(scale * sum_d q[i,d] k[j,d] - L_i) for visible (i,j) (f32; tiles without a visible pair are never
   // touched) and dS[i,j] = bf16((P[i,j] * (sum_d dO[i,d] v[j,d] - Delta_i)) * scale); both sums ascend over the 128 dims
   // blocks of 64 rows where those leave every CTA with one block at most (2 heads x 128: 0.027 against 0.035 ms); with more of them
-  // the tall ones have the better rate (8 x 1024: 0.076 and 0.066 ms)
+  // the tall ones have the better rate (8 x 1024: 0.076 and 0.066 ms).  Up to a block and three quarters per CTA there is little to multiply
+  // behind the epilogue and the multiplying warps do it themselves (whole backward, with epilogue warps and without: 16 heads x 384, 96
+  // blocks, 82.9 and 79.0 us; 24 x 512, 240 blocks, 138.3 and 137.9; 90 x 256, 270 blocks, 136.4 and 138.5)
   int tall = 0, half = 0;
   for (int i0 = 0; i0 < S; i0 += 64) {
     half += sdp_blocks(i0, window);
@@ -933,6 +936,8 @@ static int attn_bwd_impl(const det_bf16* dout, const det_bf16* q, const det_bf16
   }
   int rc = (long long)B * H * half <= dev_sm_count()
                ? sdp_run<SdpHalf>(dout, q, k, v, lse, delta, ld, ld_out, B, H, Hkv, S, window, half, Pb, dSt, st)
+           : 4ll * B * H * tall <= 7ll * dev_sm_count()
+               ? sdp_run<SdpLone>(dout, q, k, v, lse, delta, ld, ld_out, B, H, Hkv, S, window, tall, Pb, dSt, st)
                : sdp_run<SdpTall>(dout, q, k, v, lse, delta, ld, ld_out, B, H, Hkv, S, window, tall, Pb, dSt, st);
   if (rc != DET_OK) return rc;
   DET_CHECK_LAUNCH();

@@ -238,6 +238,26 @@ def test_attention_row_blocks(det, B, H, Hkv, S, W, fixq):
         assert_same_bits(got[:, lo:hi], want[:, lo:hi], name)
 
 
+# the backward on either side of the number of blocks (seven quarters of the SMs) from which warps of their own form P and dS: heads of two
+# and of three blocks, the latter with half a block at the end and a window
+@pytest.mark.parametrize("per_head,S,W", [(3, 256, 0), (5, 320, 128)])
+@pytest.mark.parametrize("more", [0, 1])
+def test_attention_backward_epilogue_warps(det, per_head, S, W, more):
+    B, H = 1, 7 * det.det_device_sm_count() // 4 // per_head + more
+    HD = H * 128
+    qkv, dout = synth.normal_bf16((S, 3 * HD), 1.0, seed=H, tid=1), synth.normal_bf16((S, HD), 0.1, seed=H, tid=2)
+    x, d = dev(qkv), empty((S, 3 * HD), np.uint16)
+    q, g = x.data_ptr(), d.data_ptr()
+    out, lse = empty((S, HD), np.uint16), empty((B, H, S), F)
+    det.det_attn_fwd(q, q + 2 * HD, q + 4 * HD, 3 * HD, B, H, S, out, HD, lse, window=W)
+    det.det_attn_bwd(dev(dout), q, q + 2 * HD, q + 4 * HD, out, lse, 3 * HD, HD, B, H, S, g, g + 2 * HD, g + 4 * HD, 3 * HD,
+                     ws(det.det_attn_bwd_ws_bytes(B, H, S)), window=W)
+    _sync()
+    oout, olse = oracle.attn_fwd(qkv, B, H, S, window=W)
+    assert_same_bits(host(out, np.uint16), oout, "out")
+    assert_same_bits(host(d, np.uint16), oracle.attn_bwd(dout, qkv, oout, olse, B, H, S, window=W), "gradients")
+
+
 # the backward's blocks in equal runs, in runs with short ones at the end, and by whole query blocks: heads of one call against the
 # same heads in calls of their own
 @pytest.mark.parametrize("B,H,S", [(1, 3, 1344), (1, 18, 2048), (4, 16, 2048)])
