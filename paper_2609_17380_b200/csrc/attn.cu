@@ -34,13 +34,16 @@ namespace det {
 // Hkv key/value heads serve H query heads (head h reads key/value head h / (H/Hkv)).
 // ---------------------------------------------------------------------------------------------
 // Rows per CTA, ring slots, slabs in flight in the producers' registers, CTAs per SM, registers per consumer and producer thread after the hand-over.
-// A CTA of 128 rows has the best rate (25.1 us per row block and key block on a full GPU, against 13.2 us for 64 rows and
-// 7.5 us for 32), but its chain of key blocks is the longest: alone on its SM 25.1, 17 and 13 us per key block.
+// The registers go to the consumers, whose loops spill and reload with fewer: one slab in flight leaves them eight to sixteen more than
+// three or four did (64 heads x 2048, 128 rows, 104 and 112: 1447 and 1415 us; 4 x 4096, 64 rows, 96 and 104: 494 and 479; 20 x 1024,
+// 32 rows, 104, 112 and 120: 170, 153 and 149; 8 x 1024, two groups, 136 and 160: 78.3 and 76.5), and the other warps cover the loads.
+// A CTA of 128 rows has the best rate (23.9 us per row block and key block on a full GPU, against 12.1 us for 64 rows and
+// 6.5 us for 32), but its chain of key blocks is the longest: alone on its SM 23.5, 15.0 and 9.8 us per key block.
 // GR groups of consumer and producer warps take the key blocks of the CTA's rows in turn: logits and P.V of a block need nothing of
 // the block before but its running maximum, which passes from warp to warp through shared memory, and group 1 hands its u, row
-// sums and rescale factors to group 0, which alone forms o and l, in block order.  Two groups shorten the chain, 13 to 9.9 us per
-// key block, and lose rate (9.8 against 7.5 us per 32 rows and key block): 8 heads x 1024 0.119 ms with 32 rows, 0.088 with two groups;
-// 16 x 832 0.119 and 0.117; two sequences of 8 x 1088 0.167 and 0.189.
+// sums and rescale factors to group 0, which alone forms o and l, in block order.  Two groups shorten the chain, 9.8 to 8.6 us per
+// key block, and lose rate (8.6 against 6.5 us per 32 rows and key block): 8 heads x 1024 98 us with 32 rows, 76 with two groups;
+// 16 x 832 106 and 102; 16 x 1088 151 and 163.
 // Slabs of a ring slot.  The kernel is bound by issue slots (twice the packed multiply-adds plus all other instructions come to 98 % of the
 // cycles), and a hand-over takes a consumer warp some 70 of them: one for two slabs instead of one a slab, waited for where it is needed
 // instead of a slab ahead, with two keys a store in the producers (see OgSide) took 16 heads x 832 from 116 to 107 us.
@@ -54,10 +57,10 @@ struct AfTile {
   // setmaxnreg: the counts after the hand-over must fit into what the block was launched with, or the increase never returns
   static_assert(CONS * RC + GR * AF_PROD * RP <= (65536 / (CPS * THREADS) / 8 * 8) * THREADS, "register hand-over exceeds the block's allocation");
 };
-typedef AfTile<128, 4, 4, 1, 104, 64> AfTall;
-typedef AfTile<64, 2, 2, 2, 96, 48> AfHalf;
-typedef AfTile<32, 2, 3, 3, 104, 56> AfShort;
-typedef AfTile<32, 2, 3, 1, 136, 64, 2> AfPair;
+typedef AfTile<128, 4, 1, 1, 112, 32> AfTall;
+typedef AfTile<64, 2, 1, 2, 104, 32> AfHalf;
+typedef AfTile<32, 2, 1, 3, 120, 40> AfShort;
+typedef AfTile<32, 2, 3, 1, 160, 96, 2> AfPair;
 
 template <class T, bool WIN>
 __global__ void __launch_bounds__(T::THREADS, T::CPS)
@@ -811,13 +814,13 @@ static int attn_fwd_run(const det_bf16* q, const det_bf16* k, const det_bf16* v,
 }
 // Rows per CTA: the longest chain of key blocks runs on one SM whatever the others do, and all chains together share the GPU; the
 // figures are the microseconds per key block of a CTA alone on its SM and of one among many, the CTAs per SM, and the part of a
-// chain by which the shared time is exceeded in the end, which shrinks with the rounds of CTAs over the GPU's places; nothing while long and
-// short rows are paired on the SMs (two CTAs each, none left over).  The row count with the smallest of the larger bounds is taken.
-// Measured with 128, 64, 32 rows and two groups: 64 heads x 2048 1447, 1500, 1624, 2056 us; 48 x 832 246, 216, 228, 297; 20 x 1024 197, 190,
-// 170, 183; 16 x 1088 220, 145, 153, 166; 16 x 832 171, 115, 108, 103; 8 x 1024 197, 128, 101, 79.
-struct RowCost { int rows; double alone, full; int cps; double over, decay; };   // rows: 33 for 32 rows with two groups
+// chain by which the shared time is exceeded in the end, which shrinks with the rounds of CTAs over the GPU's places (with 128 rows a key
+// block's time); nothing while long and short rows are paired on the SMs (two CTAs each, none left over).  The row count with the smallest of
+// the larger bounds is taken.  Measured with 64, 32 rows and two groups: 16 heads x 2048 408, 409, 513 us and 386 with 128 rows; 48 x 832 214, 224,
+// 294; 20 x 1024 189, 154, 181; 16 x 1088 146, 151, 163; 16 x 832 116, 106, 102; 8 x 1024 128, 98, 76.
+struct RowCost { int rows; double alone, full; int cps; double over, decay, tail; };   // rows: 33 for 32 rows with two groups; tail: in key blocks
 static int attn_rows(int heads, int S, int window) {
-  const RowCost c[4] = {{128, 24.1, 24.6, 1, 0.3, 1.5}, {64, 15.5, 12.6, 2, 0.55, 2.0}, {32, 10.4, 6.9, 3, 0.5, 1.5}, {33, 8.75, 8.75, 1, 0.15, 0.0}};
+  const RowCost c[4] = {{128, 23.5, 23.9, 1, 0.0, 0.0, 0.9}, {64, 15.0, 12.1, 2, 0.55, 2.0, 0.0}, {32, 9.8, 6.5, 3, 0.5, 1.5, 0.0}, {33, 8.6, 8.6, 1, 0.15, 0.0, 0.0}};
   const int sms = dev_sm_count() > 0 ? dev_sm_count() : 1;
   int best = c[0].rows;
   double best_t = 0.0;
@@ -832,9 +835,11 @@ static int attn_rows(int heads, int S, int window) {
     }
     const double rounds = (double)heads * ((S + step - 1) / step) / ((double)c[i].cps * sms);
     const double over = rounds > 1.0 ? c[i].over * pow(rounds, -c[i].decay) : (c[i].cps == 2 ? 0.0 : c[i].over);
-    const double a = longest * c[i].alone, b = total * heads * c[i].full / sms + over * a;
-    // a window's edge is one more block with masks for a few rows, which the two groups feel most (8 x 1024, window 256: 79, 56, 58, 64 us)
-    const double t = (a > b ? a : b) * (window && i == 3 ? 1.2 : 1.0);
+    const double a = longest * c[i].alone, b = total * heads * c[i].full / sms + over * a + (rounds > 1.0 ? c[i].tail * c[i].alone : 0.0);
+    // a window's edge is one more block with masks for a few rows, which short row blocks feel more (16 x 2048, window 128: 103 us with 128
+    // rows, 115 with 64; 8 x 1024, window 256, two groups 64, 32 rows 58)
+    const double edge[4] = {1.1, 1.3, 1.2, 1.4};
+    const double t = (a > b ? a : b) * (window ? edge[i] : 1.0);
     if (i == 0 || t < 0.97 * best_t) { best = c[i].rows; best_t = t; }
   }
   return best;
