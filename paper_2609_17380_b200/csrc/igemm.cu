@@ -317,13 +317,13 @@ __device__ __forceinline__ void ig_body(const CUtensorMap& tmA, const CUtensorMa
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)IgTile<BN>::TCOLS) : "memory");
   }
-  if (fill) grid_fill_end();
 }
 template <int BN, int EPI>
 __global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
     k_igemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, EpiParams ep, int I, int J, int K,
             int* status, int fill) {
   ig_body<BN, EPI, -1>(tmA, tmB, ep, I, J, K, status, fill, nullptr, 0);
+  if (fill) grid_fill_end();
 }
 // both gradient products of a linear layer, dX [M, K] over N and dW [N, K] over M, `p` before `s`
 template <int BN, bool W_FIRST>
@@ -353,7 +353,7 @@ constexpr int GEMM2_THREADS = 64 + 8 * 32;
 template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     k_igemm2(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, EpiParams ep, int I, int J,
-             int K, int* status) {
+             int K, int* status, int fill) {
   constexpr int STAGE_A = 128 * BK, STAGE_B = 128 * BK, STAGE_BYTES = STAGE_A + STAGE_B;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -384,7 +384,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
   cluster_sync_all();  // the peer's barriers are initialised before anything can signal them
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
-  grid_dep();
+  if (fill) grid_fill_begin();
+  else grid_dep();
 
   const int tiles_i = I / 256, tiles_j = J / BN2;
   const int num_tiles = tiles_i * tiles_j;
@@ -473,6 +474,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
   }
+  if (fill) grid_fill_end();
 }
 
 // ---- host side -------------------------------------------------------------------------------
@@ -519,7 +521,7 @@ static int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const EpiPar
 
 template <int EPI>
 static int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const EpiParams& ep, int I, int J, int K, int* status,
-                       cudaStream_t st) {
+                       cudaStream_t st, int fill) {
   constexpr size_t smem = (size_t)STAGES2 * (2 * 128 * BK) + 8 * 4096 + 1024;
   static DevOnce once = {};
   if (dev_ensure_smem(once, (const void*)k_igemm2<EPI>, smem) != DET_OK) return DET_ERR_CUDA;
@@ -528,7 +530,7 @@ static int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const EpiPa
   const int tiles = (I / 256) * (J / BN2);
   int clusters = sms / 2;
   if (tiles < clusters) clusters = tiles;
-  launch_after(k_igemm2<EPI>, 2 * clusters, GEMM2_THREADS, smem, st, ta, tb, ep, I, J, K, status);
+  launch_after(k_igemm2<EPI>, 2 * clusters, GEMM2_THREADS, smem, st, ta, tb, ep, I, J, K, status, fill);
   if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return DET_ERR_CUDA; }
   return DET_OK;
 }
@@ -567,7 +569,7 @@ template <int EPI>
 static int igemm_tile(int bn, const CUtensorMap& ta, const CUtensorMap& tb, const EpiParams& ep, int I, int J, int K, int* status,
                       cudaStream_t st, int fill) {
   switch (bn) {
-    case 512: return launch_pair<EPI>(ta, tb, ep, I, J, K, status, st);
+    case 512: return launch_pair<EPI>(ta, tb, ep, I, J, K, status, st, fill);
     case 256: return launch_one<256, EPI>(ta, tb, ep, I, J, K, status, st, fill);
     case 128: return launch_one<128, EPI>(ta, tb, ep, I, J, K, status, st, fill);
     default: return launch_one<64, EPI>(ta, tb, ep, I, J, K, status, st, fill);
@@ -579,7 +581,7 @@ int igemm_launch(int epi, const int8_t* A, const int8_t* B, int I, int J, int K,
   if (I % BM || J % 128 || K % BK) return DET_ERR_SHAPE;
   if (K >= (1 << 17)) return DET_ERR_RANGE;
   if (!aligned16(A) || !aligned16(B)) return DET_ERR_ALIGN;
-  const int bn = igemm_pick(epi, I, J, K, force_one_cta || fill);
+  const int bn = igemm_pick(epi, I, J, K, force_one_cta);
   CUtensorMap ta, tb;
   if (!make_map(&ta, A, I, K, 128) || !make_map(&tb, B, J, K, bn == 512 ? 128 : bn)) return DET_ERR_CUDA;
   switch (epi) {

@@ -81,7 +81,7 @@ int dev_ensure_smem(DevOnce& once, const void* fn, size_t bytes);  // DET_OK or 
 int dev_sm_count();                                                 // SMs of the current device (0 on error)
 
 // C[i,j] = sum_k A[i,k] B[j,k] on the tensor cores with the chosen epilogue; host-side checks included
-// fill != 0: this product does not depend on the kernel before it on the stream and takes the SMs that one leaves (common.cuh); one-CTA kernel
+// fill != 0: this product does not depend on the kernel before it on the stream and takes the SMs that one leaves (common.cuh)
 // force_one_cta != 0 keeps the one-CTA kernel even where the two-CTA tiles would apply (the results are identical)
 int igemm_launch(int epi, const int8_t* A, const int8_t* B, int I, int J, int K, const EpiParams& ep, int* status,
                  cudaStream_t st, int force_one_cta = 0, int fill = 0);

@@ -704,7 +704,7 @@ extern "C" int det_linear_bwd(const det_bf16* dY, const det_bf16* X, const int8_
   const bool small = (long long)(M / 128 + N / 128) * (K / 128) <= dev_sm_count();
   if (!both && small) {
     rc = igemm_launch(EPI_DX, Aq, qWt_bwd, M, K, N, ex, status_dev, st);
-    if (rc == DET_OK) rc = igemm_launch(EPI_DW, GqT, ZqT, N, K, M, ew, status_dev, st, 1, 1);
+    if (rc == DET_OK) rc = igemm_launch(EPI_DW, GqT, ZqT, N, K, M, ew, status_dev, st, 0, 1);
     if (rc != DET_OK) return rc;
   }
   if (both || small) {
