@@ -27,6 +27,10 @@ int det_test_igemm_tn(const int8_t* A, const int8_t* B, int I, int J, int K, int
  * so that the time-out path can be exercised without making a real kernel hang. */
 int det_test_wait_timeout(int* status_dev, long long limit_cycles, void* stream);
 
+/* The same wait by a whole warp of which only every other lane waits for nothing: gone_on (device, 32 ints) says for each lane whether it
+ * would go on.  After limit_cycles all of them must have given up together. */
+int det_test_wait_warp(int* gone_on, long long limit_cycles, void* stream);
+
 /* One contraction of the LM head with a tile of the caller's choice (0: 128 x 256, 1: 128 x 128, 2: 64 x 128, 3: 32 x 64), so that a test can
  * run every tile at any size; the result does not depend on it.  which 0: logits f32 [M,V] of A = H, B = W as det_lmhead_fwd; 1: dH bf16
  * [M,K] of A = dlogits (f32), B = W; 2: dW f32 [V,K] of A = dlogits, B = H (first_chunk as there), as det_lmhead_bwd.  Same shape limits. */

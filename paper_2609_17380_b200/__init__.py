@@ -67,7 +67,7 @@ _SIGNATURES = {
     "det_tensor_hash_ws_bytes": "zz", "det_tensor_hash_async": "ipzppzp", "det_tensor_hash": "ipzppzp",
     "det_tensor_hash_batch_ws_bytes": "zpi", "det_tensor_hash_batch": "ippippzp", "det_test_prim": "iipppzp",
     "det_residual_rmsnorm_fwd": "ipppiifpppppp", "det_rmsnorm_bwd_residual": "ippppiippppzp", "det_test_igemm_tn": "ippiiipipp", "det_test_lmhead_tile": "iiippiiipip",
-    "det_test_wait_timeout": "iplp",
+    "det_test_wait_timeout": "iplp", "det_test_wait_warp": "iplp",
 }
 
 # The entry points that csrc/binding.cpp calls directly: what it makes of each Python argument (letters as above; w: a workspace tensor or None,
@@ -235,6 +235,10 @@ def det_linear_bwd(dY, X, qX, W, qWt_bwd, s_x, s_w, s_u, M, N, K, hadamard_block
 
 def det_test_wait_timeout(status_dev, limit_cycles):
     _check("det_test_wait_timeout", load().det_test_wait_timeout(_ptr(status_dev), limit_cycles, _stream()))
+
+
+def det_test_wait_warp(gone_on, limit_cycles):
+    _check("det_test_wait_warp", load().det_test_wait_warp(_ptr(gone_on), limit_cycles, _stream()))
 
 
 def det_test_igemm_tn(A, B, I, J, K, Cout, force_one_cta=0, status_dev=None):

@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
   };
   // o = o * alpha + u and l = l * alpha + sum of group 1's block of round `rd`
   auto take = [&](int rd) -> bool {
-    if (!__all_sync(0xffffffffu, mbar_wait(&bar_u[warp], (uint32_t)rd & 1u, abort_flag, nullptr))) return false;
+    if (!mbar_wait_warp(&bar_u[warp], (uint32_t)rd & 1u, abort_flag, nullptr)) return false;
     const int own = wrow + ROW_OF_LANE(lane);
     l_mine = fadd(fmul(l_mine, alpha_g[own]), sum_g[own]);
 #pragma unroll
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
         acc, j0 + 8 * tx, q0 + lrow, q0 + wrow + ROW_OF_LANE(lane), j0 + FK - 1, W, diag, edge, lane, m_mine, alpha_mine, one,
         [&](float m) {
           if (GR == 1 || (grp == 0 && rd == 0)) return m;
-          ok = __all_sync(0xffffffffu, mbar_wait(&bar_max[GR - 1 - grp][warp], (uint32_t)(grp ? rd : rd - 1) & 1u, abort_flag, nullptr));
+          ok = mbar_wait_warp(&bar_max[GR - 1 - grp][warp], (uint32_t)(grp ? rd : rd - 1) & 1u, abort_flag, nullptr);
           return max_g[GR - 1 - grp][wrow + ROW_OF_LANE(lane)];
         },
         [&](float m) {
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     }
     if (!ok) break;
     if (GR > 1 && grp == 1) {   // hand u over once the last one has been read
-      if (rd > 0 && !__all_sync(0xffffffffu, mbar_wait(&bar_ufree[warp], (uint32_t)(rd - 1) & 1u, abort_flag, nullptr))) { ok = false; break; }
+      if (rd > 0 && !mbar_wait_warp(&bar_ufree[warp], (uint32_t)(rd - 1) & 1u, abort_flag, nullptr)) { ok = false; break; }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         U[(2 * i) * T::GCONS + tid - T::GCONS] = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
         const int first = i0 + (w * 2 + (lane & 1)) * 4;               // rows first + 0 .. 3 and first + TM / 2 + 0 .. 3
         // rows past the last one exist only where S is no multiple of TM: their L and Delta are never used
         float L = first < S ? __ldg(lse + r0 + first) : 0.0f, D = first < S ? __ldg(delta + r0 + first) : 0.0f;
-        ok = __all_sync(0xffffffffu, mbar_wait(&sum_full[buf][w], par, abort_flag, nullptr));
+        ok = mbar_wait_warp(&sum_full[buf][w], par, abort_flag, nullptr);
         if (!ok) break;
         tc_fence_after();
         const uint32_t taddr = sums_at(w, buf);
@@ -672,7 +672,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
     uint32_t par = 1;
     const int nslab = (w_hi - w_lo) * (DH / OK);
     for (int s = 0; s < nslab; ++s) {
-      if (!mbar_wait(&bar_empty[slot], par, abort_flag, nullptr)) break;
+      if (!mbar_wait_warp(&bar_empty[slot], par, abort_flag, nullptr)) break;   // the block's last barrier is for whole warps
       uint32_t least = ~0u;
       sk.store(Ks[slot], rk, least, pt);
       sv.store(Vs[slot], rv, least, pt);
@@ -748,7 +748,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
 #pragma unroll
         for (int c = 0; c < 4; ++c) { sa[a][c] = make_float2(0.f, 0.f); da[a][c] = make_float2(0.f, 0.f); }
       for (int sl = 0; sl < DH / OK && ok; ++sl) {
-        ok = __all_sync(0xffffffffu, mbar_wait(&bar_full[slot], par, abort_flag, nullptr));
+        ok = mbar_wait_warp(&bar_full[slot], par, abort_flag, nullptr);
         if (!ok) break;
         if (tqo | *reinterpret_cast<const uint32_t*>(tiny_s[slot])) { slab_mac<false, TM, OT, 8>(Qs + sl * OK, Ks[slot], ty, tx, sa); slab_mac<false, TM, OT, 8>(Os + sl * OK, Vs[slot], ty, tx, da); }
         else { slab_mac<true, TM, OT, 8>(Qs + sl * OK, Ks[slot], ty, tx, sa); slab_mac<true, TM, OT, 8>(Os + sl * OK, Vs[slot], ty, tx, da); }
@@ -759,7 +759,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS)
       if (!ok) break;
       if (T::EPI) {
         const int w = tid >> 5;
-        ok = __all_sync(0xffffffffu, mbar_wait(&sum_empty[buf][w], spar, abort_flag, nullptr));   // two blocks ago has been read
+        ok = mbar_wait_warp(&sum_empty[buf][w], spar, abort_flag, nullptr);   // two blocks ago has been read
         if (!ok) break;
         tc_fence_after();
         const uint32_t taddr = sums_at(w, buf);

@@ -680,6 +680,26 @@ extern "C" int det_test_wait_timeout(int* status_dev, long long limit_cycles, vo
   return DET_OK;
 }
 
+// Self-test of the wait of a whole warp: even lanes wait for a phase that is over, odd ones for one that nothing completes.
+__global__ void k_selftest_wait_warp(int* gone_on, long long limit) {
+  __shared__ __align__(8) uint64_t bar;
+  __shared__ int abort_s;
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    abort_s = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  gone_on[threadIdx.x] = mbar_wait_warp(&bar, threadIdx.x & 1 ? 0u : 1u, &abort_s, nullptr, limit);
+}
+
+extern "C" int det_test_wait_warp(int* gone_on, long long limit_cycles, void* stream) {
+  if (!gone_on || limit_cycles <= 0 || limit_cycles > 4000000000ll) return DET_ERR_ARG;
+  k_selftest_wait_warp<<<DET_L(1), 32, 0, (cudaStream_t)stream>>>(gone_on, limit_cycles);
+  DET_CHECK_LAUNCH();
+  return DET_OK;
+}
+
 extern "C" int det_test_igemm_tn(const int8_t* A, const int8_t* B, int I, int J, int K, int32_t* C, int force_one_cta,
                                  void* stream, int* status_dev) {
   if (!C) return DET_ERR_ARG;

@@ -52,6 +52,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   }
 }
 
+// The wait of a whole warp: true only if every lane saw the phase.  Each lane polls for itself, so one that has given up can have
+// neighbours that saw the barrier complete; where either way on leads to something the lanes do together, they must take the same one.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
+                                               long long limit = WAIT_LIMIT_CYCLES) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, limit));
+}
+
 __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* tm, int x, int y, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(

@@ -929,6 +929,15 @@ def test_bounded_wait_times_out_and_context_survives(det):
     assert_same_bits(host(out), np.array([oracle.det_sum(x)], F), "sum after a timed-out wait")
 
 
+def test_lanes_of_a_warp_give_up_together(det):
+    """A lane whose wait runs out takes the others of its warp with it, also those that saw their barrier complete."""
+    import torch
+    gone_on = torch.full((32,), 7, dtype=torch.int32, device="cuda")
+    det.det_test_wait_warp(gone_on, 2000000)
+    _sync()
+    assert not gone_on.any()
+
+
 def test_extreme_inputs(det):
     """Saturated softmax, zero rows and non-finite gradients: the degenerate corners of the floating-point ops."""
     import torch
