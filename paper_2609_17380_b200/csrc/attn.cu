@@ -816,10 +816,76 @@ static int attn_fwd_run(const det_bf16* q, const det_bf16* k, const det_bf16* v,
 // figures are the microseconds per key block of a CTA alone on its SM and of one among many, the CTAs per SM, and the part of a
 // chain by which the shared time is exceeded in the end, which shrinks with the rounds of CTAs over the GPU's places (with 128 rows a key
 // block's time); nothing while long and short rows are paired on the SMs (two CTAs each, none left over).  The row count with the smallest of
-// the larger bounds is taken.  Measured with 64, 32 rows and two groups: 16 heads x 2048 408, 409, 513 us and 386 with 128 rows; 48 x 832 214, 224,
-// 294; 20 x 1024 189, 154, 181; 16 x 1088 146, 151, 163; 16 x 832 116, 106, 102; 8 x 1024 128, 98, 76.
+// the larger bounds is taken.  Measured with 128, 64, 32 rows and two groups: 16 heads x 2048 378, 405, 400, 513; 48 x 832 241, 214, 218, 294; 20 x 1024 194, 187, 151, 181;
+// 16 x 1088 216, 140, 150, 163; 16 x 832 169, 112, 104, 101; 8 x 1024 192, 124, 95, 77 us.
 struct RowCost { int rows; double alone, full; int cps; double over, decay, tail; };   // rows: 33 for 32 rows with two groups; tail: in key blocks
+// With a window that is shorter than the sequence all rows but the first ones have chains of one length, so they run in rounds of equal CTAs and
+// a last round costs what the CTAs beside each other on an SM then need: 20 heads x 832 at window 128 take one round of 128 rows
+// (54 us; 64 rows, two CTAs on each SM, 64), 16 x 2048 two (103; 64 rows in two rounds of two CTAs 116, 32 rows 111), 8 x 512 one of
+// two groups (24; 32 rows 30, 128 rows 54).  Forms with one CTA on an SM: the CTAs are dealt out in their order, the longest first, to the SM
+// that is free first.  Forms with several: the larger one of the rounds of the longest chains and of all chains shared out evenly, a part of a
+// mean chain more in the end.  Microseconds of a launch, of a key block and of a CTA beside its key blocks (odd: one more where the second group has a
+// block less), by the CTAs on the SM.  Fitted to 208 shapes (2 to 96 heads x 320 to 4096, windows of 128 to 2048), all four forms measured
+// of each: the form taken is 0.2 % slower than the best one in the mean and 4 % with three exceptions (12 x 832 at window 512 takes 64 or 32 rows,
+// 91 us, two groups 81).  The rule below, which counts on chains of all lengths, was 6 % off in the mean.
+struct WindowCost { int rows, cps; double launch, tail, block[3], cta[3], odd; };
+constexpr int WIN_LENGTHS = 64;
+static int attn_rows_window(int heads, int S, int window) {
+  const WindowCost forms[4] = {{128, 1, 3.58, 0.0, {23.48}, {3.08}, 0.0},
+                               {64, 2, 14.46, 0.32, {16.21, 26.92}, {-6.19, -3.23}, 0.0},
+                               {32, 3, 10.71, 0.24, {11.72, 17.03, 20.96}, {-4.54, -4.94, -0.05}, 0.0},
+                               {33, 1, 3.87, 0.0, {8.63}, {1.9}, 2.14}};
+  const int sms = dev_sm_count() > 0 ? dev_sm_count() : 1;
+  int best = 0;
+  double best_t = 0.0;
+  for (const WindowCost& f : forms) {
+    const int step = f.rows & ~1;
+    int longest = 0;
+    long long count[WIN_LENGTHS] = {}, ctas = 0, blocks = 0;         // CTAs with a chain of so many blocks
+    for (int q0 = 0; q0 < S; q0 += step) {
+      const int n = q0 / FK + 1 - (q0 > window ? (q0 - window) / FK : 0);
+      if (n > longest) longest = n;
+      count[n] += heads;
+      ctas += heads;
+      blocks += (long long)n * heads;
+    }
+    auto chain = [&](double n, int beside) { return n * f.block[beside - 1] + f.cta[beside - 1]; };
+    double t = 0.0;
+    if (f.cps == 1) {
+      struct { double at; long long sms; } free[WIN_LENGTHS + 1] = {{0.0, sms}};   // SMs by the time they are free; a length adds one entry at most
+      int m = 1;
+      for (int n = longest; n > 0; --n)
+        for (long long left = count[n]; left > 0;) {
+          const long long take = left < free[0].sms ? left : free[0].sms;
+          const double end = free[0].at + chain(n, 1) + (n > 1 && n % 2 ? f.odd : 0.0);
+          left -= take;
+          if (take < free[0].sms) {
+            free[0].sms -= take;
+          } else {
+            --m;
+            for (int i = 0; i < m; ++i) free[i] = free[i + 1];
+          }
+          int i = m;
+          for (; i > 0 && free[i - 1].at > end; --i) free[i] = free[i - 1];
+          free[i] = {end, take};
+          ++m;
+        }
+      t = free[m - 1].at;
+    } else {
+      const long long places = (long long)sms * f.cps, full = count[longest], rest = full % places;
+      const double rounds = (full / places) * chain(longest, f.cps) + (rest ? chain(longest, (int)((rest + sms - 1) / sms)) : 0.0);
+      const double shared = (blocks * f.block[f.cps - 1] + ctas * f.cta[f.cps - 1]) / places + f.tail * chain((double)blocks / ctas, 1);
+      t = chain(longest, 1);
+      if (rounds > t) t = rounds;
+      if (ctas > sms && shared > t) t = shared;
+    }
+    t += f.launch;
+    if (!best || t < best_t) { best = f.rows; best_t = t; }
+  }
+  return best;
+}
 static int attn_rows(int heads, int S, int window) {
+  if (window && window / FK + 1 < WIN_LENGTHS) return attn_rows_window(heads, S, window);
   const RowCost c[4] = {{128, 23.5, 23.9, 1, 0.0, 0.0, 0.9}, {64, 15.0, 12.1, 2, 0.55, 2.0, 0.0}, {32, 9.8, 6.5, 3, 0.5, 1.5, 0.0}, {33, 8.6, 8.6, 1, 0.15, 0.0, 0.0}};
   const int sms = dev_sm_count() > 0 ? dev_sm_count() : 1;
   int best = c[0].rows;
@@ -828,18 +894,14 @@ static int attn_rows(int heads, int S, int window) {
     const int step = c[i].rows & ~1;
     double longest = 0.0, total = 0.0;
     for (int q0 = 0; q0 < S; q0 += step) {
-      const int lo = window && q0 > window ? (q0 - window) / FK : 0;
-      const double tiles = q0 / FK + 1 - lo;
+      const double tiles = q0 / FK + 1 - (window && q0 > window ? (q0 - window) / FK : 0);
       total += tiles;
       if (tiles > longest) longest = tiles;
     }
     const double rounds = (double)heads * ((S + step - 1) / step) / ((double)c[i].cps * sms);
     const double over = rounds > 1.0 ? c[i].over * pow(rounds, -c[i].decay) : (c[i].cps == 2 ? 0.0 : c[i].over);
     const double a = longest * c[i].alone, b = total * heads * c[i].full / sms + over * a + (rounds > 1.0 ? c[i].tail * c[i].alone : 0.0);
-    // a window's edge is one more block with masks for a few rows, which short row blocks feel more (16 x 2048, window 128: 103 us with 128
-    // rows, 115 with 64; 8 x 1024, window 256, two groups 64, 32 rows 58)
-    const double edge[4] = {1.1, 1.3, 1.2, 1.4};
-    const double t = (a > b ? a : b) * (window ? edge[i] : 1.0);
+    const double t = a > b ? a : b;
     if (i == 0 || t < 0.97 * best_t) { best = c[i].rows; best_t = t; }
   }
   return best;
@@ -851,6 +913,7 @@ static int attn_fwd_impl(const det_bf16* q, const det_bf16* k, const det_bf16* v
   if (qout && (!s_q || (((uintptr_t)qout) & 3u))) return qout && !s_q ? DET_ERR_ARG : DET_ERR_ALIGN;
   if (S % 64 || ld % 8 || ld_out % 8 || ld < H * DH || ld_out < H * DH || H % Hkv || window % 128) return DET_ERR_SHAPE;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out)) return DET_ERR_ALIGN;
+  if (window >= S) window = 0;                     // no row has a key that far behind it
   int rc;
   switch (attn_rows(B * H, S, window)) {
     case 128: rc = attn_fwd_run<AfTall>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, (cudaStream_t)stream); break;
