@@ -555,26 +555,26 @@ static int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const EpiPa
 // narrow tile shortens and spreads over more SMs (1024 x 1024 x 1024: 11.1, 10.6, 8.5, 8.5 forward and 16.7, 15.3, 12.6, 10.5
 // input gradient for 256 x 256 pairs and 256, 128, 64 columns); over many rounds the pairs run a few percent faster
 // than their rounds say (16384 x 2048 x 8192: 166, 171, 265, 520), over few of them the 256-column tiles of one CTA.
-// Returns the columns of a one-CTA tile, or 512 for the CTA pair (256 x 256); *work: its time on a full GPU without the last round's loss.
+// bn: the columns of a one-CTA tile, or 512 for the CTA pair (256 x 256); work: its time on a full GPU without the last round's loss.
 struct IgCost { int bn, bi, bj, pair; double step, turn, epi[4]; };               // epi: RAW, FWD, DX, DW
 constexpr IgCost IG_COST[4] = {{512, 256, 256, 1, 0.365, 0.9, {6.6, 4.2, 10.0, 6.6}}, {256, 128, 256, 0, 0.375, 0.5, {8.4, 4.0, 9.3, 6.2}},
                                {128, 128, 128, 0, 0.30, 0.5, {3.8, 1.7, 5.7, 3.8}}, {64, 128, 64, 0, 0.30, 0.5, {1.8, 1.7, 3.7, 1.8}}};
-static int igemm_pick(int epi, int I, int J, int K, int force_one_cta, double* work = nullptr) {
+struct IgPlan { int bn, tiles; double each, tail, work; };                        // each: a tile's time, tail: what the last one takes longer
+static IgPlan igemm_pick(int epi, int I, int J, int K, int force_one_cta) {
   const int sms = dev_sm_count() > 0 ? dev_sm_count() : 1;
   const IgCost* c = IG_COST;
-  int best = 0;
+  IgPlan best = {};
   double best_t = 0.0;
   for (int i = force_one_cta ? 1 : 0; i < 4; ++i) {
     const int units = c[i].pair ? sms / 2 : sms;
     if (I % c[i].bi || J % c[i].bj || !units) continue;
     const long long tiles = (long long)(I / c[i].bi) * (J / c[i].bj), rounds = (tiles + units - 1) / units;
-    const double loop = (K / BK) * c[i].step, e = c[i].epi[epi];
-    double t = rounds * ((loop > e ? loop : e) + c[i].turn) + (loop > e ? e : loop);
+    const double loop = (K / BK) * c[i].step, e = c[i].epi[epi], each = (loop > e ? loop : e) + c[i].turn, tail = loop > e ? e : loop;
+    double t = rounds * each + tail;
     if (c[i].bn == 512 && rounds >= 6) t *= 0.95;
-    if (!best || t < best_t) {
-      best = c[i].bn;
+    if (!best.bn || t < best_t) {
+      best = {c[i].bn, (int)tiles, each, tail, tiles * each / units};
       best_t = t;
-      if (work) *work = tiles * ((loop > e ? loop : e) + c[i].turn) / units;
     }
   }
   return best;
@@ -595,7 +595,7 @@ int igemm_launch(int epi, const int8_t* A, const int8_t* B, int I, int J, int K,
   if (I % BM || J % 128 || K % BK) return DET_ERR_SHAPE;
   if (K >= (1 << 17)) return DET_ERR_RANGE;
   if (!aligned16(A) || !aligned16(B)) return DET_ERR_ALIGN;
-  const int bn = igemm_pick(epi, I, J, K, force_one_cta);
+  const int bn = igemm_pick(epi, I, J, K, force_one_cta).bn;
   CUtensorMap ta, tb;
   if (!make_map(&ta, A, I, K, 128) || !make_map(&tb, B, J, K, bn == 512 ? 128 : bn)) return DET_ERR_CUDA;
   switch (epi) {
@@ -617,20 +617,34 @@ static int grads_tile(bool w_first, const IgProduct& p, const IgProduct& s, int 
   if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return DET_ERR_CUDA; }
   return DET_OK;
 }
-// Both gradient products in one launch, *did, instead of two, the larger ones of which go through a fork to another stream and a join.  The
-// product with the longer tiles comes first; the time of a tile width is that of the CTA that has most to do, and it may exceed
-// the work of the two, each with its own best width, by what two launches and their last rounds lose.  Whole input passes, tokens, rows and columns,
-// microseconds, two launches and one: 512 x 512 x 512 18.5 and 17.3, 1024 x 1024 x 1024 26.1 and 21.8, 1024 x 5632 x 1024 52.3 and 46.0,
-// 6144 x 640 x 1280 62.4 and 58.6, 8192 x 256 x 2048 87.4 and 81.2.  Two launches stay the better ones where one width costs more than that
-// (1024 x 1024 x 2816 34.9 and 35.5, 3200 x 1152 x 256 31.3 and 32.0), where the work is long (128 x 16384 x 4096 151 and 155) and where the
-// sum of the step gradient is (4096 x 256 x 8192 117 and 128: it runs beside the weight gradient).
+// When the last CTA of product `w` is done whose CTAs move in behind those of product `x`, first on the SMs that it leaves idle, then as they end
+static double behind_each_other(const IgPlan& x, const IgPlan& w, int sms) {
+  const int gx = x.tiles < sms ? x.tiles : sms, gw = w.tiles < sms ? w.tiles : sms, rest = w.tiles % gw;
+  auto free = [&](int j) {                                            // of the j-th SM to be free
+    j -= sms - gx;
+    return j < 0 ? 0.0 : (x.tiles / gx + (j >= gx - x.tiles % gx)) * x.each + x.tail;
+  };
+  const double few = free(gw - 1) + (w.tiles / gw) * w.each, many = rest ? free(rest - 1) + (w.tiles / gw + 1) * w.each : 0.0;
+  const double wt = (few > many ? few : many) + w.tail, xt = free(sms - 1);
+  return wt > xt ? wt : xt;
+}
+// Both gradient products in one launch, *did, instead of two; fork: the two would be on two streams, else one behind the other.  The product with
+// the longer tiles comes first; the time of a tile width is that of the CTA that has most to do.  Whole input passes, tokens, rows and columns,
+// microseconds, two launches and one, 445 shapes measured:
+//   on one stream one launch is the better one nearly always (512 x 512 x 512 18.6 and 17.4, 1024 x 1024 x 1024 26.2 and 21.6, 2560 x 3584 x 256 53.6
+//     and 45.5), unless its one width costs much more than the two widths of the others (128 x 7424 x 256 32.7 and 33.9);
+//   instead of a fork and a join one launch has to be faster by what it loses: the sum of the step gradient, which runs beside the weight
+//     gradient otherwise, from 16384 partial sums on in two launches (1024 x 5632 x 1024 52.6 and 46.0, 512 x 9216 x 1408 78.7 and 61.8; but 384 x 1408 x
+//     3328 29.0 and 33.8, 3840 x 384 x 768 30.9 and 35.8, 1024 x 2048 x 2816 41.4 and 43.0).  Long columns in wide tiles (768 x 4864 x 3328 71.3 and 77.9,
+//     128 x 6016 x 2048 40.8 and 43.3) and long work (896 x 16384 x 2432 162 and 168) stay apart.
+// Of the 328 forks 109 are joined, four of them to their loss (6 % at most); the joined ones gain 6 % in the mean.
 int igemm_grads_launch(const int8_t* A, const int8_t* Ut, const EpiParams& ex, const int8_t* Gt, const int8_t* Zt, const EpiParams& ew,
-                       int M, int N, int K, int* status, cudaStream_t st, bool* did) {
+                       int M, int N, int K, bool fork, int* status, cudaStream_t st, bool* did) {
   *did = false;
   const int sms = dev_sm_count();
   if (sms <= 0) return DET_ERR_CUDA;
-  double work[2] = {};
-  if (igemm_pick(EPI_DX, M, K, N, 0, &work[0]) == 512 || igemm_pick(EPI_DW, N, K, M, 0, &work[1]) == 512) return DET_OK;
+  const IgPlan px = igemm_pick(EPI_DX, M, K, N, 0), pw = igemm_pick(EPI_DW, N, K, M, 0);
+  if (px.bn == 512 || pw.bn == 512) return DET_OK;
   int bn = 0, lead = 0, grid = 0;
   bool w_first = false;
   double best = 0.0;
@@ -654,7 +668,10 @@ int igemm_grads_launch(const int8_t* A, const int8_t* Ut, const EpiParams& ex, c
     const double t = (tiles[f] / g) * each[f] + part + ((left + g - 1) / g) * each[1 - f] + tail;
     if (!bn || t < best) { bn = c.bn; best = t; lead = l; grid = g; w_first = f; }
   }
-  if (best > work[0] + work[1] + 5.5 || work[0] + work[1] > 50.0 || (long long)M * (K / 64) > 16ll * 16384) return DET_OK;
+  const double work = px.work + pw.work;
+  if (fork ? best > behind_each_other(px, pw, sms) - ((size_t)M * (K / 64) <= SUM_CHUNK ? 5.0 : 9.0) || (bn == 256 && K >= 2048) || work > 70.0
+           : best > work + 5.5)
+    return DET_OK;
   IgProduct x = {}, w = {};
   if (!make_map(&x.a, A, M, N, 128) || !make_map(&x.b, Ut, K, N, bn) || !make_map(&w.a, Gt, N, M, 128) || !make_map(&w.b, Zt, K, M, bn))
     return DET_ERR_CUDA;

@@ -86,9 +86,10 @@ int dev_sm_count();                                                 // SMs of th
 int igemm_launch(int epi, const int8_t* A, const int8_t* B, int I, int J, int K, const EpiParams& ep, int* status,
                  cudaStream_t st, int force_one_cta = 0, int fill = 0);
 
-// dX [M,K] = A [M,N] . (Ut [K,N])^T and dW [N,K] = Gt [N,M] . (Zt [K,M])^T in one launch; *did: whether the sizes are for that
+// dX [M,K] = A [M,N] . (Ut [K,N])^T and dW [N,K] = Gt [N,M] . (Zt [K,M])^T in one launch; *did: whether the sizes are for that (fork: they would
+// go to two streams otherwise)
 int igemm_grads_launch(const int8_t* A, const int8_t* Ut, const EpiParams& ex, const int8_t* Gt, const int8_t* Zt, const EpiParams& ew,
-                       int M, int N, int K, int* status, cudaStream_t st, bool* did);
+                       int M, int N, int K, bool fork, int* status, cudaStream_t st, bool* did);
 
 // Sliced (arithmetic version 2) contractions: out = round(I 2^(Ea + Eb - 280)) from the int8 slices of both operands,
 // Z problems per launch (lmhead_v2.cu).

@@ -698,10 +698,10 @@ extern "C" int det_linear_bwd(const det_bf16* dY, const det_bf16* X, const int8_
   // 256 -> 2944, backward: 26.8 against 25.1 us, 25.7 in one launch).  Large ones are persistent grids whose blocks leave as their tiles
   // run out; the weight gradient, on an auxiliary stream, moves onto the SMs that the last partial round of the input
   // gradient leaves idle, and the sum does not wait for it.
-  bool both;
-  int rc = igemm_grads_launch(Aq, qWt_bwd, ex, GqT, ZqT, ew, M, N, K, status_dev, st, &both);
-  if (rc != DET_OK) return rc;
   const bool small = (long long)(M / 128 + N / 128) * (K / 128) <= dev_sm_count();
+  bool both;
+  int rc = igemm_grads_launch(Aq, qWt_bwd, ex, GqT, ZqT, ew, M, N, K, !small, status_dev, st, &both);
+  if (rc != DET_OK) return rc;
   if (!both && small) {
     rc = igemm_launch(EPI_DX, Aq, qWt_bwd, M, K, N, ex, status_dev, st);
     if (rc == DET_OK) rc = igemm_launch(EPI_DW, GqT, ZqT, N, K, M, ew, status_dev, st, 0, 1);
