@@ -220,8 +220,8 @@ __global__ void __launch_bounds__(PV_THREADS, 1)
     for (int c = 0; c < 16; ++c) o[c] = make_float2(0.0f, 0.0f);
     // o = o * alpha + u of block t, once its product is there
     auto collect = [&](int t) -> bool {
-      bool ok = mbar_wait(&bar_p, (uint32_t)t & 1u, abort_flag, status) && mbar_wait(&bar_mma, (uint32_t)t & 1u, abort_flag, status);
-      if (!__all_sync(0xffffffffu, ok)) return false;   // the TMEM load below is warp-collective
+      // the TMEM load below is warp-collective
+      if (!mbar_wait_warp(&bar_p, (uint32_t)t & 1u, abort_flag, status) || !mbar_wait_warp(&bar_mma, (uint32_t)t & 1u, abort_flag, status)) return false;
       tc_fence_after();
       const float2 al = same2(alpha_s[t & 1][orow]), cs = same2(cs_s[t & 3]);
 #pragma unroll
@@ -251,7 +251,8 @@ __global__ void __launch_bounds__(PV_THREADS, 1)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
       for (int sl = 0; sl < 8; sl += PV_HS) {
-        if (!mbar_wait(&bar_full[slot], par, abort_flag, status)) { ok = false; break; }
+        ok = mbar_wait_warp(&bar_full[slot], par, abort_flag, status);
+        if (!ok) break;
         const bool tiny = tiny_q != 0 || *reinterpret_cast<const uint32_t*>(tiny_s[slot]) != 0;
 #pragma unroll 1
         for (int sub = 0; sub < PV_HS; ++sub) {
@@ -263,7 +264,6 @@ __global__ void __launch_bounds__(PV_THREADS, 1)
         if (lane == 0) mbar_arrive(&bar_empty[slot]);
         if (++slot == PV_SLOTS) { slot = 0; par ^= 1u; }
       }
-      ok = __all_sync(0xffffffffu, ok);
       if (ok && t > 0) ok = collect(t - 1);
       if (!ok) break;
       const float sum = softmax_block(acc, j0 + 8 * tx, q0 + lrow, q0 + wrow + ROW_OF_LANE(lane), j0 + PK - 1, W, diag, edge, lane,

@@ -308,7 +308,7 @@ __device__ __forceinline__ void ig_body(const CUtensorMap& tmA, const CUtensorMa
       const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
       int i0, j0;
       tile_origin(tile, TWO && job ? tiles_i[1] : tiles_i[0], tiles_j, BN, i0, j0);
-      if (!mbar_wait(&bar_tfull[acc], acc_phase, abort_flag, status)) { ok = false; break; }
+      if (!mbar_wait_warp(&bar_tfull[acc], acc_phase, abort_flag, status)) { ok = false; break; }   // the loads below are the warp's
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + part * CW);
       if (!TWO || !job) epi_row<CW, EPI>(ep, taddr, i0 + q * 32 + lane, J, j0 + part * CW, cscale, inv_s, sx, stage);
@@ -467,7 +467,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
       int i0, j0;
       if (tiles_j <= tiles_i) { j0 = (tile % tiles_j) * BN2; i0 = (tile / tiles_j) * 256; }
       else { i0 = (tile % tiles_i) * 256; j0 = (tile / tiles_i) * BN2; }
-      if (!mbar_wait(&bar_tfull[acc], acc_phase, abort_flag, status)) { ok = false; break; }
+      if (!mbar_wait_warp(&bar_tfull[acc], acc_phase, abort_flag, status)) { ok = false; break; }   // the loads below are the warp's
       tc_fence_after();
       epi_row<BN2 / 2, EPI>(ep, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN2 + half * (BN2 / 2)),
                             i0 + (int)rank * 128 + q * 32 + lane, J, j0 + half * (BN2 / 2), cscale, inv_s, sx, stage);
