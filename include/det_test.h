@@ -37,6 +37,14 @@ int det_test_wait_warp(int* gone_on, long long limit_cycles, void* stream);
 int det_test_lmhead_tile(int which, int tile, const void* A, const det_bf16* B, int M, int V, int K, void* out, int first_chunk,
                          void* stream);
 
+/* det_attn_fwd_q with a form of the caller's choice: rows per CTA 128, 64 or 32, or 33 for 32 rows with two groups of warps; the result does not
+ * depend on it. */
+int det_test_attn_fwd(int rows, const det_bf16* q, const det_bf16* k, const det_bf16* v, int ld, int B, int H, int Hkv, int S, int window,
+                      det_bf16* out, int ld_out, float* lse, const float* s_q, int8_t* qout, void* stream);
+
+/* The form that det_attn_fwd takes on this device for that many heads (of all sequences together); 0 for sizes that it refuses. */
+int det_test_attn_rows(int heads, int S, int window);
+
 #ifdef __cplusplus
 }
 #endif

@@ -67,7 +67,8 @@ _SIGNATURES = {
     "det_tensor_hash_ws_bytes": "zz", "det_tensor_hash_async": "ipzppzp", "det_tensor_hash": "ipzppzp",
     "det_tensor_hash_batch_ws_bytes": "zpi", "det_tensor_hash_batch": "ippippzp", "det_test_prim": "iipppzp",
     "det_residual_rmsnorm_fwd": "ipppiifpppppp", "det_rmsnorm_bwd_residual": "ippppiippppzp", "det_test_igemm_tn": "ippiiipipp", "det_test_lmhead_tile": "iiippiiipip",
-    "det_test_wait_timeout": "iplp", "det_test_wait_warp": "iplp",
+    "det_test_wait_timeout": "iplp", "det_test_wait_warp": "iplp", "det_test_attn_fwd": "iipppiiiiiipipppp",
+    "det_test_attn_rows": "iiii",
 }
 
 # The entry points that csrc/binding.cpp calls directly: what it makes of each Python argument (letters as above; w: a workspace tensor or None,
@@ -383,6 +384,15 @@ def det_lmhead_bwd(dlogits, H, W, M, V, K, dH, dW, first_chunk):
 
 def det_test_lmhead_tile(which, tile, A, B, M, V, K, out, first_chunk=1):
     _check("det_test_lmhead_tile", load().det_test_lmhead_tile(which, tile, _ptr(A), _ptr(B), M, V, K, _ptr(out), first_chunk, _stream()))
+
+
+def det_test_attn_fwd(rows, q, k, v, ld, B, H, S, out, ld_out, lse, s_q, qout, Hkv=None, window=0):
+    _check("det_test_attn_fwd", load().det_test_attn_fwd(rows, _ptr(q), _ptr(k), _ptr(v), ld, B, H, H if Hkv is None else Hkv, S, window,
+                                                         _ptr(out), ld_out, _ptr(lse), _ptr(s_q), _ptr(qout), _stream()))
+
+
+def det_test_attn_rows(heads, S, window=0):
+    return load().det_test_attn_rows(heads, S, window)
 
 
 # ---- gradient accumulation, AdamW, hash ---------------------------------------------------------------------------

@@ -907,15 +907,15 @@ static int attn_rows(int heads, int S, int window) {
   return best;
 }
 
-static int attn_fwd_impl(const det_bf16* q, const det_bf16* k, const det_bf16* v, int ld, int B, int H, int Hkv, int S,
-                         int window, det_bf16* out, int ld_out, float* lse, const float* s_q, int8_t* qout, void* stream) {
+static int attn_fwd_impl(const det_bf16* q, const det_bf16* k, const det_bf16* v, int ld, int B, int H, int Hkv, int S, int window,
+                         det_bf16* out, int ld_out, float* lse, const float* s_q, int8_t* qout, void* stream, int rows = 0) {
   if (!q || !k || !v || !out || !lse || B <= 0 || H <= 0 || Hkv <= 0 || S <= 0 || window < 0) return DET_ERR_ARG;
   if (qout && (!s_q || (((uintptr_t)qout) & 3u))) return qout && !s_q ? DET_ERR_ARG : DET_ERR_ALIGN;
   if (S % 64 || ld % 8 || ld_out % 8 || ld < H * DH || ld_out < H * DH || H % Hkv || window % 128) return DET_ERR_SHAPE;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out)) return DET_ERR_ALIGN;
   if (window >= S) window = 0;                     // no row has a key that far behind it
   int rc;
-  switch (attn_rows(B * H, S, window)) {
+  switch (rows ? rows : attn_rows(B * H, S, window)) {
     case 128: rc = attn_fwd_run<AfTall>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, (cudaStream_t)stream); break;
     case 64: rc = attn_fwd_run<AfHalf>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, (cudaStream_t)stream); break;
     case 33: rc = attn_fwd_run<AfPair>(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, (cudaStream_t)stream); break;
@@ -934,6 +934,14 @@ extern "C" int det_attn_fwd_q(const det_bf16* q, const det_bf16* k, const det_bf
                               int window, det_bf16* out, int ld_out, float* lse, const float* s_q, int8_t* qout, void* stream) {
   if (!s_q || !qout) return DET_ERR_ARG;
   return attn_fwd_impl(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, stream);
+}
+extern "C" int det_test_attn_fwd(int rows, const det_bf16* q, const det_bf16* k, const det_bf16* v, int ld, int B, int H, int Hkv, int S,
+                                 int window, det_bf16* out, int ld_out, float* lse, const float* s_q, int8_t* qout, void* stream) {
+  if (!s_q || !qout || (rows != 128 && rows != 64 && rows != 32 && rows != 33)) return DET_ERR_ARG;
+  return attn_fwd_impl(q, k, v, ld, B, H, Hkv, S, window, out, ld_out, lse, s_q, qout, stream, rows);
+}
+extern "C" int det_test_attn_rows(int heads, int S, int window) {
+  return heads > 0 && S > 0 && window >= 0 && window % 128 == 0 ? attn_rows(heads, S, window >= S ? 0 : window) : 0;
 }
 
 // workspace: bf16(P) and bf16(dS), [B*H, S, S] each, and Delta f32 [B*H, S]

@@ -208,8 +208,8 @@ def test_lmhead_v2_non_finite_warp(det, M, V, K):
     assert_same_bits(got[~bad], want[~bad], "version-2 logits")
 
 
-# attention at head and row counts where the rows per CTA change (32, 64, 128 rows), S off the 128 grid, windows that start
-# and end inside a block, grouped heads (one accumulator over the whole group)
+# attention with the form that the rule gives to the heads and rows (test_attention_forward_every_form runs each), S off the 128 grid, windows
+# that start and end inside a block, grouped heads (one accumulator over the whole group)
 @pytest.mark.parametrize("B,H,Hkv,S,W", [(1, 2, 2, 576, 0), (1, 40, 40, 320, 0), (2, 80, 80, 192, 0), (1, 3, 3, 704, 256),
                                          (1, 60, 60, 448, 128), (3, 64, 64, 320, 128), (1, 8, 2, 384, 0), (1, 6, 1, 448, 128)])
 @pytest.mark.parametrize("fixq", [False, True])
@@ -236,6 +236,86 @@ def test_attention_row_blocks(det, B, H, Hkv, S, W, fixq):
     got = host(dqkv, np.uint16)
     for name, lo, hi in (("dq", 0, HD), ("dk", HD, HD + KD), ("dv", HD + KD, ld)):
         assert_same_bits(got[:, lo:hi], want[:, lo:hi], name)
+
+
+def _underflow(qkv, B, H, Hkv, S):
+    """Values below 2^-63 whose products with factors that are not, subnormal, are what a sum shows that does not flush them.  In q and k: the
+    first row of every head is seen by the first query alone, whose logsumexp is the logit itself, here 2^-116 and fifteen products of about
+    2^-127; they lie in the 16 dimensions kvh mod 8.  In v: of dimension 10 + b all is zero but 16 keys of key block b, one 2^-115 and
+    fifteen of 2^-125 .. 2^-126, which the weights bring below.  Zeros count as large, so a slab of 16 is the only one of its kind in a head."""
+    rng = np.random.default_rng(S + H)
+    HD, KD = H * 128, Hkv * 128
+    x = synth.from_bf16(qkv).reshape(B, S, H + 2 * Hkv, 128).copy()
+    q, k, v = x[:, :, :H], x[:, :, H:H + Hkv], x[:, :, H + Hkv:]
+    for h in range(H):
+        d = 16 * (h // (H // Hkv) % 8)
+        q[:, 0, h] = 0
+        q[:, 0, h, d:d + 16] = F(2.0 ** -62) * (1 + rng.integers(0, 4, 16) / 8)
+        q[:, 0, h, d] = F(2.0 ** -60)
+    for h in range(Hkv):
+        d = 16 * (h % 8)
+        k[:, 0, h, d:d + 16] = F(2.0 ** -65)
+        k[:, 0, h, d] = F(2.0 ** -56)
+        for b in range(S // 128 if S > 128 else 1):
+            at = 128 * b + 16 * ((h + b) % min(8, S // 16))
+            v[:, :, h, 10 + b] = 0
+            v[:, at:at + 16, h, 10 + b] = F(2.0 ** -126) * (1 + rng.integers(0, 8, 16) / 8)
+            v[:, at, h, 10 + b] = F(2.0 ** -115)
+    return synth.to_bf16(x.reshape(B * S, HD + 2 * KD))
+
+
+# every form of the forward (rows per CTA; 33: 32 rows and two groups) at sizes of one row block up to several, off the 128 grid, grouped heads,
+# windows that begin inside a block, one to three key blocks long; ordinary, saturated and underflowing inputs
+@pytest.mark.parametrize("rows", [128, 64, 32, 33])
+@pytest.mark.parametrize("B,H,Hkv,S,W", [(1, 8, 8, 64, 0), (1, 16, 8, 448, 0), (2, 8, 8, 640, 0), (1, 8, 8, 448, 128), (1, 16, 8, 704, 256), (2, 8, 8, 576, 384)])
+@pytest.mark.parametrize("kind", ["plain", "saturated", "underflow"])
+def test_attention_forward_every_form(det, rows, B, H, Hkv, S, W, kind):
+    HD, KD = H * 128, Hkv * 128
+    ld = HD + 2 * KD
+    qkv = synth.normal_bf16((B * S, ld), 1.0, seed=S + W, tid=1)
+    if kind == "saturated":
+        qkv[:, :HD] = synth.to_bf16(synth.from_bf16(qkv[:, :HD]) * F(40.0))          # logits of order +-400
+    elif kind == "underflow":
+        qkv = _underflow(qkv, B, H, Hkv, S)
+    d = dev(qkv)
+    q = d.data_ptr()
+    s_q = np.array([0.02], F)
+    out, lse, codes = empty((B * S, HD), np.uint16), empty((B, H, S), F), empty((B * S, HD), np.int8)
+    det.det_test_attn_fwd(rows, q, q + 2 * HD, q + 2 * (HD + KD), ld, B, H, S, out, HD, lse, dev(s_q), codes, Hkv=Hkv, window=W)
+    _sync()
+    oout, olse = oracle.attn_fwd(qkv, B, H, S, Hkv=Hkv, window=W)
+    if kind == "underflow":
+        assert (olse[:, :, 0] != 0).all() and (np.abs(olse[:, :, 0]) < 2.0 ** -110).all()
+    assert_same_bits(host(lse), olse, "lse")
+    assert_same_bits(host(out, np.uint16), oout, "out")
+    assert_same_bits(host(codes).reshape(-1), np.asarray(oracle.lsq_quantize(oout, s_q, False)).reshape(-1).view(np.int8), "codes")
+
+
+# the same products in the logits of the form with int8 P.V
+@pytest.mark.parametrize("B,H,Hkv,S,W", [(1, 8, 8, 192, 0), (1, 16, 8, 448, 128)])
+def test_int8_pv_underflow(det, B, H, Hkv, S, W):
+    import torch
+    HD, KD = H * 128, Hkv * 128
+    ld = HD + 2 * KD
+    qkv = _underflow(synth.normal_bf16((B * S, ld), 1.0, seed=S, tid=1), B, H, Hkv, S)
+    d = dev(qkv)
+    q = d.data_ptr()
+    out, lse, status = empty((B * S, HD), np.uint16), empty((B, H, S), F), torch.zeros(1, dtype=torch.int32, device="cuda")
+    det.det_attn_fwd_int8pv(q, q + 2 * HD, q + 2 * (HD + KD), ld, B, H, S, out, HD, lse, status, Hkv=Hkv, window=W)
+    _sync()
+    assert int(status.item()) == 0
+    oout, olse = oracle.attn_fwd(qkv, B, H, S, Hkv=Hkv, window=W, int8_pv=True)
+    assert (olse[:, :, 0] != 0).all() and (np.abs(olse[:, :, 0]) < 2.0 ** -110).all()
+    assert_same_bits(host(lse), olse, "lse")
+    assert_same_bits(host(out, np.uint16), oout, "out")
+
+
+# which form the forward takes, where it has been measured on this device's SMs: four windows shorter than the sequence, one that is not
+@pytest.mark.parametrize("heads,S,W,rows", [(16, 2048, 128, 128), (16, 4096, 512, 64), (8, 512, 256, 33), (32, 512, 128, 128), (8, 512, 512, 33)])
+def test_attention_forward_form(det, heads, S, W, rows):
+    if det.det_device_sm_count() != 148:
+        pytest.skip("measured on 148 SMs")
+    assert det.det_test_attn_rows(heads, S, W) == rows
 
 
 # the backward on either side of the number of blocks (seven quarters of the SMs) from which warps of their own form P and dS: heads of two
