@@ -338,6 +338,68 @@ def test_attention_backward_epilogue_warps(det, per_head, S, W, more):
     assert_same_bits(host(d, np.uint16), oracle.attn_bwd(dout, qkv, oout, olse, B, H, S, window=W), "gradients")
 
 
+def _scores(q, k, v, g, out, lse):
+    """P and dS of one head for every pair, as bf16, in the arithmetic of the primitives; all arguments binary32."""
+    op, scale, S = oracle.prim, np.full((len(q), len(q)), 0.08838834764831845, F), len(q)
+    s, dp = np.zeros((S, S), F), np.zeros((S, S), F)
+    for c in range(128):
+        s = op("add", s, op("mul", np.broadcast_to(q[:, c, None], (S, S)), np.broadcast_to(k[None, :, c], (S, S))))
+        dp = op("add", dp, op("mul", np.broadcast_to(g[:, c, None], (S, S)), np.broadcast_to(v[None, :, c], (S, S))))
+    t = op("mul", g, out)
+    while t.shape[1] > 1:
+        t = op("add", t[:, 0::2], t[:, 1::2])
+    p = op("exp", op("sub", op("mul", s, scale), np.broadcast_to(lse[:, None], (S, S))))
+    return synth.to_bf16(p), synth.to_bf16(op("mul", op("mul", p, op("sub", dp, np.broadcast_to(t, (S, S)))), scale))
+
+
+# the three forms of the kernel that forms P and dS (few blocks; up to seven quarters of the SMs; epilogue warps) on the inputs that their branches are
+# for: a logsumexp that is not the row's own (positive arguments of the exponential), weights that vanish, non-finite values, and products of
+# dO and v that underflow, all of them in one slab of 16 dimensions, in which v alone is below 2^-63 (heads take turns through the eight).
+# P and dS themselves, of the pairs that are visible, from the workspace: nine heads
+@pytest.mark.parametrize("form", ["few", "lone", "tall"])
+@pytest.mark.parametrize("per_head,S,W", [(3, 256, 0), (5, 320, 128)])
+@pytest.mark.parametrize("kind", ["logsumexp", "saturated", "non-finite", "underflow"])
+def test_attention_backward_scores(det, form, per_head, S, W, kind):
+    B, H = 1, 8 if form == "few" else 7 * det.det_device_sm_count() // 4 // per_head + (form == "tall")
+    HD = H * 128
+    rng = np.random.default_rng(S + H)
+    x = synth.from_bf16(synth.normal_bf16((S, 3 * HD), 1.0, seed=H, tid=1)).reshape(S, 3, H, 128).copy()
+    g = synth.from_bf16(synth.normal_bf16((S, HD), 0.1, seed=H, tid=2)).reshape(S, H, 128).copy()
+    if kind == "saturated":
+        x[:, 0] *= F(40.0)
+    elif kind == "non-finite":                                     # in three heads of every eight, at both ends of the sequence and inside
+        x[S - 1, 0, 1::8, 5], x[3, 1, 4::8, 70], x[130, 2, 6::8, 127] = np.nan, np.inf, -np.inf
+    elif kind == "underflow":
+        x[:, 2], g[:] = 0, 0
+        for h in range(H):
+            d = 16 * (h % 8)
+            x[:, 2, h, d:d + 16] = F(2.0 ** -65) * (1 + rng.integers(0, 4, (S, 16)) / 8)
+            x[:, 2, h, d] = rng.choice(np.array([-1, 1], F), S) * F(2.0 ** -56)
+            g[:, h, d:d + 16] = F(2.0 ** -62) * (1 + rng.integers(0, 4, (S, 16)) / 8)
+            g[:, h, d] = F(2.0 ** -60)
+    qkv, dout = synth.to_bf16(x.reshape(S, 3 * HD)), synth.to_bf16(g.reshape(S, HD))
+    x, g = synth.from_bf16(qkv).reshape(S, 3, H, 128), synth.from_bf16(dout).reshape(S, H, 128)
+    out, lse = oracle.attn_fwd(qkv, B, H, S, window=W)
+    if kind == "logsumexp":
+        lse -= rng.choice(np.array([0.0, 0.75, 3.0, -2.0], F), lse.shape)
+    d_in, d, scratch = dev(qkv), empty((S, 3 * HD), np.uint16), ws(det.det_attn_bwd_ws_bytes(B, H, S))
+    q, o = d_in.data_ptr(), d.data_ptr()
+    det.det_attn_bwd(dev(dout), q, q + 2 * HD, q + 4 * HD, dev(out), dev(lse), 3 * HD, HD, B, H, S, o, o + 2 * HD, o + 4 * HD, 3 * HD, scratch, window=W)
+    _sync()
+    raw, n = host(scratch), H * S * S * 2
+    got = [raw[at:at + n].view(np.uint16).reshape(H, S, S) for at in (0, -(-n // 256) * 256)]
+    i, j = np.indices((S, S))
+    vis = (j <= i) & ((W == 0) | (j > i - W))
+    o = synth.from_bf16(out).reshape(S, H, 128)
+    for h in [8 * (r * (H // 8) // 8) + r for r in range(8)] + [H - 1]:
+        for name, a, b in zip(("P", "dS"), got, _scores(x[:, 0, h], x[:, 1, h], x[:, 2, h], g[:, h], o[:, h], lse[0, h])):
+            a, b = a[h][vis], b[vis]
+            nan = np.isnan(synth.from_bf16(b))
+            assert np.array_equal(np.isnan(synth.from_bf16(a)), nan) and (kind == "non-finite" or not nan.any())
+            assert_same_bits(a[~nan], b[~nan], "%s of head %d" % (name, h))
+            assert kind == "non-finite" or np.count_nonzero(synth.from_bf16(b)) > S
+
+
 # the backward's blocks in equal runs, in runs with short ones at the end, and by whole query blocks: heads of one call against the
 # same heads in calls of their own
 @pytest.mark.parametrize("B,H,S", [(1, 3, 1344), (1, 18, 2048), (4, 16, 2048)])
