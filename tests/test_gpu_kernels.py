@@ -552,6 +552,33 @@ def test_linear_gradients_together(det, M, N, K, hb):
     assert_same_bits(host(gs), ods, "ds_x")
 
 
+# the same in one launch with more tiles than SMs, so that a CTA passes from a tile of one product to one of the other: each product first, all three
+# widths, CTAs that take two and three tiles of the second product while others are at the first, first products of one and of two tiles a CTA.
+# prep: launches of the operand preparation, without the rotation and with it (two passes for few tiles, two times two for many)
+@pytest.mark.parametrize("M,N,K,hb,prep", [(128, 128, 4992, 128, 2), (4224, 1920, 256, 0, 5), (7296, 2304, 256, 0, 5), (128, 3840, 640, 128, 2),
+                                           (6528, 128, 768, 0, 5), (128, 4224, 1280, 0, 5), (6144, 128, 1024, 0, 5), (512, 3072, 1792, 0, 5)])
+def test_linear_gradients_together_many_tiles(det, M, N, K, hb, prep):
+    import torch
+    X, W = synth.normal_bf16((M, K), 1.0, seed=N, tid=1), synth.normal_bf16((N, K), 0.02, seed=N, tid=2)
+    dY = synth.normal_bf16((M, N), 0.01, seed=N, tid=3)
+    sw, sx = oracle.lsq_weight_scale(W), oracle.lsq_act_scale_init(X)
+    odX, odW, ods = oracle.linear_bwd(dY, X, W, sx, sw, hb=hb)
+    dX_, dW_, s_w, s_x = dev(X), dev(W), dev(sw), dev(sx)
+    qW, qWt, s_u = empty((N, K), np.int8), empty((K, N), np.int8), empty((1,), F)
+    det.det_lsq_quantize_weight(dW_, s_w, N, K, hb, qW, qWt, s_u, ws(det.det_lsq_quantize_weight_ws_bytes(N, K)))
+    Y, qX, status = empty((M, N), np.uint16), empty((M, K), np.int8), torch.zeros(1, dtype=torch.int32, device="cuda")
+    det.det_linear_fwd(dX_, qW, s_x, s_w, M, N, K, Y, qX, status)
+    gX, gW, gs = empty((M, K), np.uint16), empty((N, K), F), empty((1,), F)
+    before = det.det_launch_count()
+    det.det_linear_bwd(dev(dY), dX_, qX, dW_, qWt, s_x, s_w, s_u, M, N, K, hb, gX, gW, gs, ws(det.det_linear_bwd_ws_bytes(M, N, K)), status)
+    assert det.det_launch_count() - before == prep + 1 + (1 if M * K // 64 <= 16384 else 2)      # the products in one, the sum of the step gradient
+    _sync()
+    assert int(status.item()) == 0
+    assert_same_bits(host(gX, np.uint16), odX, "dX")
+    assert_same_bits(host(gW), odW, "dW")
+    assert_same_bits(host(gs), ods, "ds_x")
+
+
 # the norms with the residual stream beside them: rows off the block of eight, D off the leaf of 256, with and without codes
 @pytest.mark.parametrize("rows,D,q", [(1, 8, True), (13, 1000, False), (300, 2048, True), (64, 384, True), (21, 256, True), (22, 512, False),
                                       (23, 1024, True), (9, 1032, True), (515, 200, False)])
