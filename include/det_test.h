@@ -37,6 +37,9 @@ int det_test_wait_warp(int* gone_on, long long limit_cycles, void* stream);
 int det_test_lmhead_tile(int which, int tile, const void* A, const det_bf16* B, int M, int V, int K, void* out, int first_chunk,
                          void* stream);
 
+/* The tile (numbers as above) that det_lmhead_fwd takes on this device; -1 for sizes that it refuses. */
+int det_test_lmhead_pick(int M, int V, int K);
+
 /* det_attn_fwd_q with a form of the caller's choice: rows per CTA 128, 64 or 32, or 33 for 32 rows with two groups of warps; the result does not
  * depend on it. */
 int det_test_attn_fwd(int rows, const det_bf16* q, const det_bf16* k, const det_bf16* v, int ld, int B, int H, int Hkv, int S, int window,

@@ -68,7 +68,7 @@ _SIGNATURES = {
     "det_tensor_hash_batch_ws_bytes": "zpi", "det_tensor_hash_batch": "ippippzp", "det_test_prim": "iipppzp",
     "det_residual_rmsnorm_fwd": "ipppiifpppppp", "det_rmsnorm_bwd_residual": "ippppiippppzp", "det_test_igemm_tn": "ippiiipipp", "det_test_lmhead_tile": "iiippiiipip",
     "det_test_wait_timeout": "iplp", "det_test_wait_warp": "iplp", "det_test_attn_fwd": "iipppiiiiiipipppp",
-    "det_test_attn_rows": "iiii",
+    "det_test_attn_rows": "iiii", "det_test_lmhead_pick": "iiii",
 }
 
 # The entry points that csrc/binding.cpp calls directly: what it makes of each Python argument (letters as above; w: a workspace tensor or None,
@@ -393,6 +393,10 @@ def det_test_attn_fwd(rows, q, k, v, ld, B, H, S, out, ld_out, lse, s_q, qout, H
 
 def det_test_attn_rows(heads, S, window=0):
     return load().det_test_attn_rows(heads, S, window)
+
+
+def det_test_lmhead_pick(M, V, K):
+    return load().det_test_lmhead_pick(M, V, K)
 
 
 # ---- gradient accumulation, AdamW, hash ---------------------------------------------------------------------------

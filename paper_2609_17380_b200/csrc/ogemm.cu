@@ -67,3 +67,8 @@ extern "C" int det_test_lmhead_tile(int which, int tile, const void* A, const de
   DET_CHECK_LAUNCH();
   return DET_OK;
 }
+
+extern "C" int det_test_lmhead_pick(int M, int V, int K) {
+  if (M <= 0 || V <= 0 || K <= 0 || K % 16 || V % 4) return -1;
+  return og_pick(OG_ROW_RATES, plain_args(nullptr, nullptr, nullptr, M, V, K, K, K, V, 0), 1, 1, 0, 0.0);
+}

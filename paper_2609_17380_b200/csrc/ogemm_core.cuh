@@ -283,6 +283,10 @@ struct OgTile {
 typedef OgTile<128, 256, 16, 2, 2, 1, 1, 216, 72, 2> OgWide;
 typedef OgTile<128, 128, 16, 4, 2, 1, 2, 208, 48, 3, true> OgSquare;
 typedef OgTile<64, 128, 8, 2, 2, 2, 2, 0, 0, 4> OgHalf;
+// Both operands CONTIG: the two halves of a row's 32 bytes of a slab are two producer warps' and meet in the first-level cache, of which two
+// rings of four slabs a slot leave 28 KiB beside them, three 92 KiB.  64 x 27184 x 1680 (W comes from memory): 201 us with four, 162 with three;
+// 2048 x 8064 x 2048 1355 and 1366; one CTA on each SM, 2048 steps, 112 and 116 (strided operands, read in whole rows, lose 5 % with three).
+typedef OgTile<64, 128, 8, 2, 2, 2, 2, 0, 0, 3> OgHalfRows;
 typedef OgTile<32, 64, 4, 2, 2, 4, 4, 0, 0, 4, true> OgSmall;
 typedef OgTile<64, 128, 8, 2, 2, 1, 2, 0, 0, 2, false, 0> OgFix;       // with 64 KiB of 64-bit accumulators beside the ring
 constexpr size_t OG_FIX_BYTES = (size_t)64 * 128 * 8;
@@ -506,15 +510,20 @@ static int ogemm_run(const OgemmArgs& p, int batches, cudaStream_t st) {
 // of the larger bounds is taken.
 struct OgRate { int tm, tn; float alone, full; };     // cycles per step of a CTA alone on its SM; multiply-adds per cycle and SM of a full one
 constexpr OgRate OG_RATES[4] = {{128, 256, 302.0f, 108.5f}, {128, 128, 165.0f, 107.0f}, {64, 128, 93.0f, 98.0f}, {32, 64, 56.0f, 76.0f}};
+// Both operands CONTIG (the head's forward): staging turns both, which costs the small tiles most.  Measured as above 290, 161, 100, 53 cycles and 111, 109,
+// 89, 59; the rates here, within 2 % but for the last one (its grids seldom fill an SM's four places), take a tile 0.2 % slower than the
+// best one in the mean over 464 shapes (8 .. 2400 x 320 .. 51200 x 128 .. 2560), the measured ones 0.5 %, those of strided operands 1.3 % and up to 29 %
+// (640 x 2048 x 2048 32 x 64 tiles, 217 us, for 128 x 128, 169; 304 x 37424 x 1408 754 and 639).
+constexpr OgRate OG_ROW_RATES[4] = {{128, 256, 290.0f, 109.0f}, {128, 128, 161.0f, 110.0f}, {64, 128, 100.0f, 90.0f}, {32, 64, 53.0f, 64.0f}};
 // share: how many such contractions run side by side; beside: SM-cycles of other work that is queued to fill the SMs that a small
 // grid leaves idle (the head's two gradients at 384 tokens: 96 CTAs of 64 x 128 and the weight gradient on the other SMs,
 // head and loss forward and backward 4.34 ms; 384 CTAs of 32 x 64 on all of them and the weight gradient behind, 5.27 ms)
-static int og_pick(const OgemmArgs& p, int batches, int share, int widest, double beside) {
+static int og_pick(const OgRate (&rates)[4], const OgemmArgs& p, int batches, int share, int widest, double beside) {
   const int sms = dev_sm_count() > 0 ? dev_sm_count() : 1;
   int best = widest;
   double best_t = 0.0;
   for (int c = widest; c < 4; ++c) {
-    const OgRate r = OG_RATES[c];
+    const OgRate r = rates[c];
     const double ni = (p.I + r.tm - 1) / r.tm, nj = (p.J + r.tn - 1) / r.tn;
     const double tiles = ni * nj * batches;
     double longest, total;           // steps of the contraction: of one tile, and summed over the tiles
@@ -544,19 +553,22 @@ static int og_pick(const OgemmArgs& p, int batches, int share, int widest, doubl
 }
 template <int WIDEST> struct OgFirst { typedef OgWide T; };
 template <> struct OgFirst<1> { typedef OgSquare T; };
+template <int AMODE, int BMODE> struct OgHalfOf { typedef OgHalf T; };
+template <> struct OgHalfOf<CONTIG, CONTIG> { typedef OgHalfRows T; };
 // WIDEST: 0, or 1 where the output has no 256 columns (the head dimension of the attention contractions is 128)
 template <int AMODE, int BMODE, bool AF32, bool OUT_BF16, int WIDEST>
 static int ogemm_tile(int tile, const OgemmArgs& p, int batches, cudaStream_t st) {
   switch (tile) {
     case 0: return ogemm_run<AMODE, BMODE, AF32, OUT_BF16, typename OgFirst<WIDEST>::T>(p, batches, st);
     case 1: return ogemm_run<AMODE, BMODE, AF32, OUT_BF16, OgSquare>(p, batches, st);
-    case 2: return ogemm_run<AMODE, BMODE, AF32, OUT_BF16, OgHalf>(p, batches, st);
+    case 2: return ogemm_run<AMODE, BMODE, AF32, OUT_BF16, typename OgHalfOf<AMODE, BMODE>::T>(p, batches, st);
     default: return ogemm_run<AMODE, BMODE, AF32, OUT_BF16, OgSmall>(p, batches, st);
   }
 }
 template <int AMODE, int BMODE, bool AF32, bool OUT_BF16, int WIDEST>
 static int ogemm_launch(const OgemmArgs& p, int batches, int share, cudaStream_t st, double beside = 0.0) {
-  return ogemm_tile<AMODE, BMODE, AF32, OUT_BF16, WIDEST>(og_pick(p, batches, share, WIDEST, beside), p, batches, st);
+  const OgRate(&rates)[4] = AMODE == CONTIG && BMODE == CONTIG ? OG_ROW_RATES : OG_RATES;
+  return ogemm_tile<AMODE, BMODE, AF32, OUT_BF16, WIDEST>(og_pick(rates, p, batches, share, WIDEST, beside), p, batches, st);
 }
 
 }  // namespace det

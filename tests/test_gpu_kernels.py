@@ -115,6 +115,14 @@ def test_lmhead_slots_of_slabs(det, tile, C):
         assert_same_bits(host(dW), oracle.lmhead_bwd(gm, Hm, synth.normal_bf16((32, 16), 0.05, seed=M, tid=6))[1], "dW")
 
 
+# the tile that the head's forward takes at sizes where the rates of strided operands would choose a slower one
+@pytest.mark.parametrize("M,V,K,tile", [(640, 2048, 640, 1), (640, 2048, 2048, 1), (832, 16384, 2048, 1), (304, 37424, 1408, 0), (88, 14128, 496, 1), (384, 2048, 2048, 2)])
+def test_lmhead_forward_tile(det, M, V, K, tile):
+    if det.det_device_sm_count() != 148:
+        pytest.skip("measured on 148 SMs")
+    assert det.det_test_lmhead_pick(M, V, K) == tile
+
+
 # version-2 gradients where a row of logits is long enough for eight warps (4096 values), and one step below; a token gradient of 36
 # tiles and 16 steps (two CTAs a tile, bf16 results), one of 80 (pairs, bf16 results); the 1B shape's vocabulary, an odd number of row
 # tiles for the weight gradient
