@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS) k_ogemm(const OgemmArgs p)
 #pragma unroll
       for (int d = 0; d < PF; ++d) {
         if (s0 + d >= nslab) return;
-        const int sub = HS == 1 ? 0 : (s0 + d) % HS;
+        const int sub = (s0 + d) % HS;
         if (sub == 0) {
           if (!mbar_wait(&bar_empty[slot], par, abort_flag, nullptr)) return;   // the consumers have left this slot
           least = ~0u;
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(T::THREADS, T::CPS) k_ogemm(const OgemmArgs p)
         if (tiny) slab_mac<false, TM, TN, CT>(As[at], Bs[at], ty, tx, acc);
         else if constexpr (CT == 16) slabs_ordered<false, TM, TN, CT>(As[at], Bs[at], 1, ty, tx, acc);
         else slab_mac<true, TM, TN, CT>(As[at], Bs[at], ty, tx, acc);
-        if (HS == 1 || sub == HS - 1 || s == nslab - 1) break;
+        if (sub == HS - 1 || s == nslab - 1) break;
         ++s;
       }
     }
