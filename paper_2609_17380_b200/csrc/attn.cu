@@ -420,7 +420,9 @@ __global__ void __launch_bounds__(256) k_attn_delta(const uint16_t* __restrict__
 // into step and left it idle during their epilogues, a latency-bound 12.5 of 52 thousand cycles a key block; now one multiplies on
 // while the exponentials fill the issue slots it leaves: 16 heads x 2048 0.453 -> 0.406 ms; the whole windowed attention (16 x 4096, forward and
 // backward) 1.380 -> 1.348 ms, two sequences of 8 x 1088 0.478 -> 0.460.  A fourth slot (1.381) and slots of two slabs (1.372) leave less of the
-// memory to the first-level cache and were slower.
+// memory to the first-level cache and were slower.  158 bytes of the consumers' 184 and the producers' 56 registers' work are spilled, half by
+// either (none by the epilogue: without its arithmetic as many, without the staging 84, without the multiply loops none); with 216 and 72 and
+// no epilogue warps it is 48.
 // Without EPI a consumer thread works on its own sums, which is the shorter way where a CTA has a key block or two.
 // Nothing is carried from one key block to the next, so the blocks of all heads are numbered (head, query block, key block) and
 // every CTA of a resident grid takes an equal run of them; where a run enters another query block the consumers stage its rows.

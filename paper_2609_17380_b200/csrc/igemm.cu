@@ -339,7 +339,8 @@ __global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
   ig_body<BN, EPI, -1>(tmA, tmB, ep, I, J, K, status, fill, nullptr, 0);
   if (fill) grid_fill_end();
 }
-// both gradient products of a linear layer, dX [M, K] over N and dW [N, K] over M, `p` before `s`
+// both gradient products of a linear layer, dX [M, K] over N and dW [N, K] over M, `p` before `s`; two epilogues in one kernel spill 28, 48 and 88 bytes
+// a thread with 64, 128 and 256 columns
 template <int BN, bool W_FIRST>
 __global__ void __launch_bounds__(IgTile<BN>::THREADS, 1)
     k_igemm_grads(const __grid_constant__ IgProduct p, const __grid_constant__ IgProduct s, int J, int* status, int lead) {

@@ -24,7 +24,7 @@ enum { CONTIG = 0, STRIDED = 1 };
 // lane rounded on its own).
 //
 // The 8 x 16 and 8 x 4 tiles (FUSED) fetch the next step's operands before they multiply the current one's and keep that order
-// (volatile): 302 instead of 306 cycles per step of the 128 x 256 tile; other orders of the 64 multiply-adds (rows outermost, zigzag,
+// (volatile): 302 instead of 306 cycles per step of the 128 x 256 tile, then (295 now); other orders of the 64 multiply-adds (rows outermost, zigzag,
 // 2 x 2 blocks) took 302 to 326, a copy of A with every value doubled 365, and bf16 words in shared memory that the consumers unpack
 // 335 to 383.  Counters say why: a packed multiply-add holds the issue port of its scheduler for two cycles, and twice the
 // multiply-adds plus everything else comes to 98 % of the cycles, so each further instruction costs its cycle.
@@ -40,7 +40,7 @@ __device__ __forceinline__ void ffma2_ordered(float a, float2 b, float2& c) {
 }
 // CARRY: the last step of a slab fetches the first operands of the next one, n slabs in all; else one slab.  One warp per scheduler
 // sees the latency of those loads (128 x 128 tiles alone on their SMs 171 -> 165 cycles per step, 32 x 64 56 -> 52), two hide it for each other
-// (128 x 256: 302 -> 308), and the 8 x 8 loop is best left to the compiler (64 x 128 alone: 91 -> 99).
+// (128 x 256: 2 % slower), and the 8 x 8 loop is best left to the compiler (64 x 128 alone: 91 -> 99).
 template <bool CARRY, int TM, int TN, int CT, int LA, int LB>
 __device__ __forceinline__ void slabs_ordered(const float (*As)[LA], const float (*Bs)[LB], int n, int ty, int tx, float2 (&acc)[8][CT / 2]) {
   const float *pa = &As[0][ty * 4], *pb = &Bs[0][tx * 4];
@@ -137,7 +137,7 @@ __device__ __forceinline__ bool least_tiny(uint32_t m) { return (m & 0xffffu) < 
 // last one repeat it: their results are not stored.
 // Every instruction here takes an issue cycle from the consumers of its scheduler (see slabs_ordered).  Running pointers instead of
 // addresses and bounds per load, the two-instruction test and the paired stores took the instructions beside the multiply-adds
-// from 0.30 to 0.25 per multiply-add (LM head forward, 128 x 256 tiles: 308 -> 302 cycles per step; weight gradient 310 -> 302).
+// from 0.30 to 0.25 per multiply-add (128 x 256 tiles: 2 % faster in the LM head's forward, 2.6 % in the weight gradient).
 template <int MODE, bool F32IN, int ROWS>
 struct OgSide {
   static constexpr int EPW = F32IN ? 4 : 8, ESZ = F32IN ? 4 : 2;          // CONTIG: contraction indices of a 16-byte word
@@ -264,9 +264,9 @@ enum { OG_LEAD = 1, OG_FILL = 2, OG_BACK = 4 };
 // registers, CPS CTAs per SM; RC / RP: registers of a consumer / producer thread after the hand-over (0: none); PAD: floats behind
 // each row of a slab (four instead of none are worth 2 % in every tile; with the 64-bit totals there is no room for them).
 // A hand-over costs a consumer some 35 instructions and, with one warp per scheduler, their latency; over HS slabs it is paid once.
-// Cycles per step of a CTA alone on its SM / multiply-adds per cycle and SM of a full GPU, by slabs per slot: 64 x 128 tiles 1: 103,
-// 97; 2: 97, 99; 4: 92, 102.  32 x 64 tiles 1: 67, 67; 2: 60, 76; 4: 52, 77.  128 x 128 tiles 1: 173, 97; 2: 170, 98; 3: 165, 99.  128 x 256
-// tiles 1 and 2: 302, 108.5; 4 in two slots 308, 105.
+// 64 x 128 tiles by slabs per slot, two slots: token gradient of 384 x 8064 x 1024 2: 394, 3: 394, 4: 373 us; weight gradient of 1024 x 4096 x
+// 1024 189, 188, 182.  Smaller chains gain most (32 x 64 tiles of one CTA on an SM 22 % from one slab to four, 128 x 128 5 % to three), the
+// 128 x 256 tiles nothing.
 template <int TM_, int TN_, int CT_, int LY_, int ST_, int PF_, int CPS_, int RC_, int RP_, int HS_, bool CARRY_ = false, int PAD_ = 4>
 struct OgTile {
   static constexpr int TM = TM_, TN = TN_, CT = CT_, LY = LY_, ST = ST_, PF = PF_, CPS = CPS_, RC = RC_, RP = RP_, HS = HS_;
@@ -277,9 +277,14 @@ struct OgTile {
   // what the block is launched with: 65536 registers over CPS blocks, in steps of eight a thread
   static_assert(RC == 0 || CONS * RC + OG_PROD * RP <= (65536 / (CPS * THREADS) / 8 * 8) * THREADS, "register hand-over exceeds the block's allocation");
 };
-// Measured at 2048 contraction steps on full GPUs (multiply-adds per cycle and SM, 128 is the pipe): 108.5, 107, 98, 76; one CTA
-// on each SM: 302, 165, 93, 56 cycles per step.  Some 20 to 40 cycles of every step are not multiply-adds whatever the tile, so
-// a smaller tile shortens a chain but never reaches the rate of a larger one.
+// Measured at 1965 MHz: cycles per step of one CTA on each SM, from 2048 and 6144 steps, and multiply-adds per cycle and SM (128 is the pipe) of
+// grids of eight full rounds of 2048 steps, start and stores included.  128 x 256, 128 x 128, 64 x 128, 32 x 64 tiles:
+//   head forward     290, 161, 100, 53;  111, 109, 89, 59
+//   token gradient   295, 158,  86, 54;  109, 106, 97, 67
+//   weight gradient  290, 153,  92, 53;  111, 112, 99, 77
+// (128 x 128 spills up to 16 bytes a thread, 64 x 128 and 32 x 64 16 to 32, the head forward's 64 x 128 64 stored and 108 loaded.)
+// Some 20 to 40 cycles of every step are not multiply-adds whatever the tile, so a smaller tile shortens a chain but never reaches the rate of a
+// larger one.
 typedef OgTile<128, 256, 16, 2, 2, 1, 1, 216, 72, 2> OgWide;
 typedef OgTile<128, 128, 16, 4, 2, 1, 2, 208, 48, 3, true> OgSquare;
 typedef OgTile<64, 128, 8, 2, 2, 2, 2, 0, 0, 4> OgHalf;
@@ -509,11 +514,13 @@ static int ogemm_run(const OgemmArgs& p, int batches, cudaStream_t st) {
 // which falls with the tile (more operand loads per multiply).  Both are measured figures; the tile with the smaller
 // of the larger bounds is taken.
 struct OgRate { int tm, tn; float alone, full; };     // cycles per step of a CTA alone on its SM; multiply-adds per cycle and SM of a full one
+// Strided operands (the gradients, and attention's contractions with them), of the order of both gradients' figures above: the weight gradient takes a
+// tile 2.1 % from its best one in the mean over 264 shapes, with its own figures 2.0 %.
 constexpr OgRate OG_RATES[4] = {{128, 256, 302.0f, 108.5f}, {128, 128, 165.0f, 107.0f}, {64, 128, 93.0f, 98.0f}, {32, 64, 56.0f, 76.0f}};
-// Both operands CONTIG (the head's forward): staging turns both, which costs the small tiles most.  Measured as above 290, 161, 100, 53 cycles and 111, 109,
-// 89, 59; the rates here, within 2 % but for the last one (its grids seldom fill an SM's four places), take a tile 0.2 % slower than the
-// best one in the mean over 464 shapes (8 .. 2400 x 320 .. 51200 x 128 .. 2560), the measured ones 0.5 %, those of strided operands 1.3 % and up to 29 %
-// (640 x 2048 x 2048 32 x 64 tiles, 217 us, for 128 x 128, 169; 304 x 37424 x 1408 754 and 639).
+// Both operands CONTIG (the head's forward): staging turns both, which costs the small tiles most.  Within 2 % of the figures above but for the
+// last one (its grids seldom fill an SM's four places), these take a tile 0.2 % slower than the best one in the mean over 464 shapes (8 .. 2400 x
+// 320 .. 51200 x 128 .. 2560), the figures above 0.5 %, OG_RATES 1.3 % and up to 29 % (640 x 2048 x 2048: 32 x 64 tiles, 217 us, for 128 x 128, 169;
+// 304 x 37424 x 1408 754 and 639).
 constexpr OgRate OG_ROW_RATES[4] = {{128, 256, 290.0f, 109.0f}, {128, 128, 161.0f, 110.0f}, {64, 128, 100.0f, 90.0f}, {32, 64, 53.0f, 64.0f}};
 // share: how many such contractions run side by side; beside: SM-cycles of other work that is queued to fill the SMs that a small
 // grid leaves idle (the head's two gradients at 384 tokens: 96 CTAs of 64 x 128 and the weight gradient on the other SMs,
