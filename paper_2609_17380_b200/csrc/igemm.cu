@@ -299,16 +299,18 @@ __device__ __forceinline__ void ig_body(const CUtensorMap& tmA, const CUtensorMa
     const int q = warp & 3, part = (warp - 2) >> 2;  // TMEM lane quarter this warp may read; its share of the columns
     uint8_t* stage = smem + STAGES * STAGE_BYTES + (warp - 2) * 4096;  // this warp's 32 x 128-byte staging tile
     int job, tile = walk.before();
-    bool ok = true;
     float cscale, inv_s, sx, cscale2 = 1.0f, inv_s2 = 1.0f, sx2 = 1.0f;
     epi_scalars<EPI>(ep, cscale, inv_s, sx);
     if constexpr (TWO) epi_scalars<EPI2>(second->ep, cscale2, inv_s2, sx2);
-    for (int it = 0; ok && walk.tile(it, job, tile); ++it) {
+    // A wait that ran out is passed over and the loop runs to its end: a tile's loads and stores are the warp's, and lanes that have given up must
+    // not leave the others in them (later waits see the abort flag after a few polls; the output is undefined then).  A vote of the warp instead
+    // costs up to 2 % where the epilogue bounds (forward of 1792 x 14336 x 256 20.1 and 20.5 us).
+    for (int it = 0; walk.tile(it, job, tile); ++it) {
       const int acc = it & 1;
       const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
       int i0, j0;
       tile_origin(tile, TWO && job ? tiles_i[1] : tiles_i[0], tiles_j, BN, i0, j0);
-      if (!mbar_wait_warp(&bar_tfull[acc], acc_phase, abort_flag, status)) { ok = false; break; }   // the loads below are the warp's
+      mbar_wait(&bar_tfull[acc], acc_phase, abort_flag, status);
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + part * CW);
       if (!TWO || !job) epi_row<CW, EPI>(ep, taddr, i0 + q * 32 + lane, J, j0 + part * CW, cscale, inv_s, sx, stage);
@@ -458,17 +460,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     const int q = warp & 3, half = (warp - 2) >> 2;
     uint8_t* stage = smem + STAGES2 * STAGE_BYTES + (warp - 2) * 4096;  // this warp's 32 x 128-byte staging tile
     int it = 0;
-    bool ok = true;
     float cscale, inv_s, sx;
     epi_scalars<EPI>(ep, cscale, inv_s, sx);
     const uint32_t tempty_leader0 = mapa_u32(smem_u32(&bar_tempty[0]), 0), tempty_leader1 = mapa_u32(smem_u32(&bar_tempty[1]), 0);
-    for (int tile = cluster_id; tile < num_tiles && ok; tile += nclusters, ++it) {
+    for (int tile = cluster_id; tile < num_tiles; tile += nclusters, ++it) {
       const int acc = it & 1;
       const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
       int i0, j0;
       if (tiles_j <= tiles_i) { j0 = (tile % tiles_j) * BN2; i0 = (tile / tiles_j) * 256; }
       else { i0 = (tile % tiles_i) * 256; j0 = (tile / tiles_i) * BN2; }
-      if (!mbar_wait_warp(&bar_tfull[acc], acc_phase, abort_flag, status)) { ok = false; break; }   // the loads below are the warp's
+      mbar_wait(&bar_tfull[acc], acc_phase, abort_flag, status);   // passed over when it ran out, as in the one-CTA kernel
       tc_fence_after();
       epi_row<BN2 / 2, EPI>(ep, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN2 + half * (BN2 / 2)),
                             i0 + (int)rank * 128 + q * 32 + lane, J, j0 + half * (BN2 / 2), cscale, inv_s, sx, stage);
